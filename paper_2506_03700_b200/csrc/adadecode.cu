@@ -146,13 +146,15 @@ struct ada_session {
     float inv_temp = 1.0f;
     int steps_per_launch = 256;
     unsigned long long wait_ns = st::WAIT_NS_DEFAULT;
-    // dense prompt pass (tcgen05 GEMMs over blocks of up to 128 positions)
-    bool dense_ok = false, dense_on = false;   // available for this session / in use by the prefill that is running
-    int cur_rows = 0;                          // rows of the pass being issued
-    __nv_bfloat16 *pf_hi = nullptr, *pf_lo = nullptr;   // [128][max K]: high and low parts of a GEMM's input
+    // dense prompt pass (tcgen05 GEMMs over blocks of up to dg::PF_ROWS positions)
+    bool dense_ok = false;                     // available for this session
+    int pf_pairs = 0;                          // CTA pairs of this device
+    unsigned pf_epoch = 0;                     // dense products launched so far (tags published partial sums)
+    float *pf_resid = nullptr, *pf_cs = nullptr, *pf_part = nullptr;
+    __nv_bfloat16 *pf_x = nullptr, *pf_u = nullptr;   // high and low parts of a product's input: model width; queries, attention result / FFN activations
+    unsigned *pf_flag = nullptr;
     int *pf_err = nullptr;
-    float *pf_part = nullptr;                  // shares of depth-split products: [splits][128][N]
-    size_t pf_part_bytes = 0;
+    std::vector<CUtensorMap> pf_maps;          // [L][7]: wq, wk, wv, wo, w_gate, w_up, w_down
     bool prefill_dense = true;                 // ada_debug_set_prefill
     int64_t launches = 0, syncs = 0, layer_passes = 0;
     // per-class profiling
@@ -177,16 +179,18 @@ namespace {
 // Scratch layout (all offsets 256-byte aligned).
 struct Layout {
     size_t st, rt, fill, tokens, page_table, head_res, resid, xn, qkv, q, attn_out, gu, hact, rope_cs, attn_part,
-        head_part, logit_stage, head_log, t_out, pf_hi, pf_lo, pf_err, pf_part, maps, mm, exit_at, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
+        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_err, pf_flag, pf_part, maps, mm, exit_at, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
         grid_ctr, pub, err, q_stage, qinfo, uniforms, total;
 };
 
 bool model_fits_persistent(const ada_config &g);
-constexpr size_t kDenseSplitMax = 4;   // shares of a depth-split dense product (O and down projections)
-// rows a layer pass may carry: the decode rows of all sequences, or a 128-position block of a dense prompt pass
+// rows a layer pass of the per-operation path may carry: the decode rows of all sequences, or a block of prompt positions
 int rows_alloc_for(const ada_config &g, int batch, int max_early) {
-    return std::max(batch * (max_early + 1), model_fits_persistent(g) ? dg::BM : 32);
+    return std::max(batch * (max_early + 1), model_fits_persistent(g) ? 64 : 32);
 }
+// positions of one block of a dense prompt pass: a prompt is cut alike whatever the session's length limit
+int pf_rows_for(int max_seq) { return std::min(dg::PF_ROWS, (int)align_up((size_t)max_seq, dg::BM)); }
+constexpr int kGemmMaxPairs = 80;   // CTA pairs the exchange area of cut tiles is laid out for
 
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
@@ -219,12 +223,15 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
     L.logit_stage = take(sizeof(float) * (size_t)R * g.vocab);
     L.head_log = take(sizeof(float) * 4 * kHeadLogCap);
     L.t_out = take(sizeof(float) * (size_t)R * g.d_model);
-    if (model_fits_persistent(g)) {   // dense prompt pass: a GEMM's input as two bf16 matrices [128][K]
-        const size_t kmax = (size_t)std::max(std::max(g.d_model, g.n_q_heads * g.head_dim), g.d_ff);
-        L.pf_hi = take(sizeof(__nv_bfloat16) * dg::BM * kmax);
-        L.pf_lo = take(sizeof(__nv_bfloat16) * dg::BM * kmax);
+    if (model_fits_persistent(g)) {   // dense prompt pass: residual and the two bf16 parts of every product's input
+        const size_t P = pf_rows_for(max_seq);
+        L.pf_resid = take(sizeof(float) * P * g.d_model);
+        L.pf_x = take(sizeof(__nv_bfloat16) * 2 * P * g.d_model);
+        L.pf_u = take(sizeof(__nv_bfloat16) * P * std::max(4 * (size_t)qd, 2 * (size_t)g.d_ff));
+        L.pf_cs = take(sizeof(float) * P * g.head_dim);
         L.pf_err = take(256);
-        L.pf_part = take(kDenseSplitMax * sizeof(float) * dg::BM * (size_t)g.d_model);
+        L.pf_flag = take(sizeof(unsigned) * 2 * kGemmMaxPairs * dg::GEPI_WARPS);
+        L.pf_part = take(dg::GPART_CTA * 2 * kGemmMaxPairs);
     }
     // persistent-kernel buffers (bf16 models)
     if (g.dtype == ADA_DTYPE_BF16) {
@@ -305,105 +312,113 @@ void prof_collect(ada_session *S) {
 
 // ---- typed launch helpers --------------------------------------------------------------------
 
-// ---- dense prompt pass: one decoder layer over a block of up to 128 prompt rows (rows 0 .. cur_rows - 1) -------
+// ---- dense prompt pass: one decoder layer over a block of up to dg::PF_ROWS prompt positions --------------------
 
-// One tcgen05 GEMM over the input last split into S->pf_hi / pf_lo (depth K): Y = or += X W^T.  Products with few
-// tiles are split in depth over several CTAs per tile (shares added in a fixed order by k_dense_reduce).
-int dense_gemm(ada_session *S, int cls, bool add, const void *W, int N, int K, float *Y, int ldy) {
-    Prof pf(S, cls, (double)N * K * 2);
-    CUtensorMap mhi, mlo, mw;
-    int rc;
-    if ((rc = make_map_2d(&mhi, S->pf_hi, dg::BM, K, dg::BM)) || (rc = make_map_2d(&mlo, S->pf_lo, dg::BM, K, dg::BM)) ||
-        (rc = make_map_2d(&mw, W, N, K, dg::BN)))
-        return rc;
-    const int tiles = (N + dg::BN - 1) / dg::BN, nkb = K / dg::BK;
-    int splits = 1;
-    while (tiles * splits < 96 && splits * 2 <= nkb / 8 && (size_t)(splits * 2) * dg::BM * N * sizeof(float) <= S->pf_part_bytes && N % 4 == 0) splits *= 2;
-    if (splits == 1) {
-        if (add) dg::k_dense_gemm<1><<<tiles, dg::DTHREADS, dg::DSMEM_BYTES, S->stream>>>(mhi, mlo, mw, Y, ldy, S->cur_rows, N, K, 0, S->pf_err);
-        else dg::k_dense_gemm<0><<<tiles, dg::DTHREADS, dg::DSMEM_BYTES, S->stream>>>(mhi, mlo, mw, Y, ldy, S->cur_rows, N, K, 0, S->pf_err);
-        CK(cudaGetLastError());
-        S->launches++;
-    } else {
-        const size_t stride = (size_t)dg::BM * N;
-        dg::k_dense_gemm<0><<<dim3(tiles, splits), dg::DTHREADS, dg::DSMEM_BYTES, S->stream>>>(mhi, mlo, mw, S->pf_part, N, S->cur_rows, N, K, stride, S->pf_err);
-        CK(cudaGetLastError());
-        dg::k_dense_reduce<<<dim3((N / 4 + 255) / 256, S->cur_rows), 256, 0, S->stream>>>(S->pf_part, stride, splits, Y, ldy, S->cur_rows, N, add ? 1 : 0);
-        CK(cudaGetLastError());
-        S->launches += 2;
+// How a product of `nt` tile columns and depth K over `rows` positions is divided over at most `pairs` CTA pairs.  More
+// tiles than pairs: whole waves, then one wave's worth of tiles and the remainder cut by chunks so that all pairs end
+// together (cutting the remainder alone would cut a tile into more pieces, each of which costs an exchange).  Fewer:
+// all tiles cut over the number of pairs that minimises chunks of the busiest pair (8192 tensor-core cycles each) plus
+// the reading of a tile's other pieces by its last pair (128 KB per CTA, measured at some 3300 cycles).
+dg::GemmPlan plan_dense(int rows, int nt, int K, int pairs) {
+    dg::GemmPlan g{};
+    g.mt = (rows + dg::TM - 1) / dg::TM;
+    g.tiles = g.mt * nt;
+    g.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
+    if (g.tiles >= pairs) {
+        g.pairs = pairs;
+        if (g.tiles % pairs) { g.sk_tiles = g.tiles % pairs + pairs; g.sk_pairs = pairs; }
+        return g;
     }
-    return ADA_OK;
+    const int units = g.tiles * g.chunks;
+    double best = 0;
+    for (int p = g.tiles; p <= std::min(pairs, units); ++p) {
+        const int per = units / p;
+        const int pieces = p == g.tiles ? 0 : (g.chunks + per - 1) / per;
+        const double cost = 8192.0 * ((units + p - 1) / p) + 3300.0 * pieces * std::min(1.0, rows / (double)dg::BM) + (pieces ? 3000.0 : 0.0);
+        if (!g.pairs || cost < best) { best = cost; g.pairs = p; }
+    }
+    g.sk_tiles = g.tiles;
+    g.sk_pairs = g.pairs;
+    return g;
 }
 
-int run_layer_dense(ada_session *S, int layer, int rows) {
+template <int EPI, int HD>
+int launch_dense(cudaStream_t stream, const CUtensorMap &xh, const CUtensorMap &xl, const CUtensorMap &w0, const CUtensorMap &w1,
+                 const CUtensorMap &w2, const Ctx &c, const dg::GemmArgs &a) {
+    dg::k_dense_gemm<EPI, HD><<<2 * a.plan.pairs, dg::GTHREADS, dg::DSMEM_BYTES, stream>>>(xh, xl, w0, w1, w2, c, a);
+    CK(cudaGetLastError());
+    return ADA_OK;
+}
+template <int EPI, int HD> cudaError_t prepare_dense() {
+    return cudaFuncSetAttribute(dg::k_dense_gemm<EPI, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES);
+}
+
+// Tensor maps of the inputs of a block's products (they end at the block's last row: rows behind it read as zero).
+struct PfMaps { CUtensorMap xh, xl, oh, ol, hh, hl; };
+
+int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int pos0, int rows) {
     const ada_model *m = S->m;
     const ada_config &g = m->cfg;
     const LayerW &w = m->layers[layer];
-    const int d = g.d_model, hd = g.head_dim, qd = g.n_q_heads * hd, kvd = g.n_kv_heads * hd, qkv_rows = S->c.qkv_rows;
+    const int d = g.d_model, hd = g.head_dim, qd = g.n_q_heads * hd, kvd = g.n_kv_heads * hd, group = g.n_q_heads / g.n_kv_heads;
+    const CUtensorMap *wm = &S->pf_maps[7 * (size_t)layer];
+    const size_t P = pf_rows_for(S->max_seq);
+    __nv_bfloat16 *xh = S->pf_x, *xl = xh + P * d, *qh = S->pf_u, *ql = qh + P * qd, *oh = ql + P * qd, *ol = oh + P * qd, *hh = S->pf_u, *hl = hh + P * g.d_ff;
     typedef __nv_bfloat16 T;
     int rc;
+    if (group != 1 && group != 2 && group != 4) return ADA_EUNSUPPORTED;
+    dg::GemmArgs a{};
+    a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err;
     S->layer_passes++;
-    {
+    S->launches += 7;
+    auto norm = [&](const void *gain) {
         Prof pf(S, 1, 0.0);
-        dg::k_norm_split_rows<<<dg::BM, 256, 0, S->stream>>>(S->c.resid, rows, d, (const T *)w.attn_norm, g.rms_eps, S->pf_hi, S->pf_lo);
-    }
+        dg::k_norm_split_rows<<<rows, 256, 0, S->stream>>>(S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl);
+    };
+    norm(w.attn_norm);
     CK(cudaGetLastError());
-    S->launches++;
-    if ((const T *)w.wk == (const T *)w.wq + (size_t)qd * d && (const T *)w.wv == (const T *)w.wk + (size_t)kvd * d) {
-        if ((rc = dense_gemm(S, 2, false, w.wq, qkv_rows, d, S->c.qkv, qkv_rows))) return rc;
-    } else {
-        if ((rc = dense_gemm(S, 2, false, w.wq, qd, d, S->c.qkv, qkv_rows))) return rc;
-        if ((rc = dense_gemm(S, 2, false, w.wk, kvd, d, S->c.qkv + qd, qkv_rows))) return rc;
-        if ((rc = dense_gemm(S, 2, false, w.wv, kvd, d, S->c.qkv + qd + kvd, qkv_rows))) return rc;
-    }
     {
-        Prof pf(S, 3, 0.0);
-        k_rope_kv<T><<<rows, 128, 0, S->stream>>>(S->c, layer);
+        Prof pf(S, 2, (double)(qd + 2 * kvd) * d * 2);
+        a.nw[0] = qd; a.nw[1] = a.nw[2] = kvd;
+        a.nt[0] = (qd + dg::TN - 1) / dg::TN; a.nt[1] = a.nt[2] = (kvd + dg::TN - 1) / dg::TN;
+        a.K = d; a.hi = qh; a.lo = ql; a.epoch = ++S->pf_epoch;
+        a.plan = plan_dense(rows, a.nt[0] + a.nt[1] + a.nt[2], d, S->pf_pairs);
+        rc = hd == 128 ? launch_dense<dg::EPI_QKV, 128>(S->stream, pm.xh, pm.xl, wm[0], wm[1], wm[2], S->c, a)
+                       : launch_dense<dg::EPI_QKV, 64>(S->stream, pm.xh, pm.xl, wm[0], wm[1], wm[2], S->c, a);
+        if (rc) return rc;
     }
-    CK(cudaGetLastError());
-    S->launches++;
     {
         Prof pf(S, 4, 0.0);
-        const int group = g.n_q_heads / g.n_kv_heads;
-        if (group != 1 && group != 2 && group != 4) return ADA_EUNSUPPORTED;
         const dim3 grid((rows + 64 / group - 1) / (64 / group), g.n_kv_heads);   // four warps of 16 / group positions each
-#define PF_ATTN(H, G) dg::k_pf_attn_mma<H, G><<<grid, 128, 0, S->stream>>>(S->c, layer, rows)
+#define PF_ATTN(H, G) dg::k_pf_attn_mma<H, G><<<grid, 128, 0, S->stream>>>(S->c, layer, rows, seq, pos0, qh, ql, oh, ol)
         if (hd == 128) { if (group == 4) PF_ATTN(128, 4); else if (group == 2) PF_ATTN(128, 2); else PF_ATTN(128, 1); }
-        else if (hd == 64) { if (group == 4) PF_ATTN(64, 4); else if (group == 2) PF_ATTN(64, 2); else PF_ATTN(64, 1); }
-        else return ADA_EUNSUPPORTED;
+        else { if (group == 4) PF_ATTN(64, 4); else if (group == 2) PF_ATTN(64, 2); else PF_ATTN(64, 1); }
 #undef PF_ATTN
     }
     CK(cudaGetLastError());
-    S->launches++;
+    a.nt[0] = (d + dg::TN - 1) / dg::TN;
+    a.nt[1] = a.nt[2] = 0;
+    a.Y = S->pf_resid; a.ldy = d;
     {
-        Prof pf(S, 11, 0.0);
-        dg::k_split_rows<<<dg::BM, 256, 0, S->stream>>>(S->c.attn_out, qd, rows, qd, S->pf_hi, S->pf_lo);
+        Prof pf(S, 5, (double)d * qd * 2);
+        a.nw[0] = d; a.K = qd; a.epoch = ++S->pf_epoch;
+        a.plan = plan_dense(rows, a.nt[0], qd, S->pf_pairs);
+        if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.oh, pm.ol, wm[3], wm[3], wm[3], S->c, a))) return rc;
     }
-    CK(cudaGetLastError());
-    if ((rc = dense_gemm(S, 5, true, w.wo, d, qd, S->c.resid, d))) return rc;
-    {
-        Prof pf(S, 1, 0.0);
-        dg::k_norm_split_rows<<<dg::BM, 256, 0, S->stream>>>(S->c.resid, rows, d, (const T *)w.ffn_norm, g.rms_eps, S->pf_hi, S->pf_lo);
-    }
-    CK(cudaGetLastError());
-    if ((const T *)w.w_up == (const T *)w.w_gate + (size_t)g.d_ff * d) {
-        if ((rc = dense_gemm(S, 6, false, w.w_gate, 2 * g.d_ff, d, S->c.gu, 2 * g.d_ff))) return rc;
-    } else {
-        if ((rc = dense_gemm(S, 6, false, w.w_gate, g.d_ff, d, S->c.gu, 2 * g.d_ff))) return rc;
-        if ((rc = dense_gemm(S, 6, false, w.w_up, g.d_ff, d, S->c.gu + g.d_ff, 2 * g.d_ff))) return rc;
-    }
-    {
-        Prof pf(S, 7, 0.0);
-        k_swiglu<<<dim3((g.d_ff + 255) / 256, rows), 256, 0, S->stream>>>(S->c, layer);
-    }
+    norm(w.ffn_norm);
     CK(cudaGetLastError());
     {
-        Prof pf(S, 11, 0.0);
-        dg::k_split_rows<<<dg::BM, 256, 0, S->stream>>>(S->c.hact, g.d_ff, rows, g.d_ff, S->pf_hi, S->pf_lo);
+        Prof pf(S, 6, (double)2 * g.d_ff * d * 2);
+        a.nw[0] = a.nw[1] = g.d_ff; a.K = d; a.hi = hh; a.lo = hl; a.epoch = ++S->pf_epoch;
+        a.plan = plan_dense(rows, (g.d_ff + dg::BNH - 1) / dg::BNH, d, S->pf_pairs);
+        if ((rc = launch_dense<dg::EPI_SWIGLU, 0>(S->stream, pm.xh, pm.xl, wm[4], wm[5], wm[5], S->c, a))) return rc;
     }
-    CK(cudaGetLastError());
-    S->launches += 4;
-    if ((rc = dense_gemm(S, 8, true, w.w_down, d, g.d_ff, S->c.resid, d))) return rc;
+    {
+        Prof pf(S, 8, (double)d * g.d_ff * 2);
+        a.nw[0] = d; a.K = g.d_ff; a.epoch = ++S->pf_epoch;
+        a.plan = plan_dense(rows, a.nt[0], g.d_ff, S->pf_pairs);
+        if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.hh, pm.hl, wm[6], wm[6], wm[6], S->c, a))) return rc;
+    }
     return ADA_OK;
 }
 
@@ -535,7 +550,6 @@ int run_head_t(ada_session *S, int layer1, int sel, int rows) {
 }
 
 int run_layer(ada_session *S, int layer, int rows) {
-    if (S->dense_on) return run_layer_dense(S, layer, rows);
     return S->m->cfg.dtype == ADA_DTYPE_BF16 ? run_layer_t<__nv_bfloat16>(S, layer, rows) : run_layer_t<float>(S, layer, rows);
 }
 int run_head(ada_session *S, int layer1, int sel, int rows) {
@@ -562,6 +576,43 @@ int capture_rows(ada_session *S, int row0) {
     k_capture_advance<<<1, 32, 0, S->stream>>>(S->c);
     CK(cudaGetLastError());
     S->launches += 2;
+    return ADA_OK;
+}
+
+// Prompt pass over dense blocks: equal blocks of at most dg::PF_ROWS positions, then the LM head on the last position.
+int prefill_dense(ada_session *S, int seq, int n_prompt) {
+    const ada_model *m = S->m;
+    const ada_config &g = m->cfg;
+    const int d = g.d_model, qd = g.n_q_heads * g.head_dim;
+    const size_t P = pf_rows_for(S->max_seq);
+    __nv_bfloat16 *oh = S->pf_u + 2 * P * qd, *hh = S->pf_u;
+    const int blocks = (n_prompt + (int)P - 1) / (int)P;
+    int rc;
+    CK(cudaMemsetAsync(S->pf_err, 0, sizeof(int), S->stream));
+    for (int i = 0; i < blocks; ++i) {
+        const int p0 = (int)((long long)n_prompt * i / blocks), n = (int)((long long)n_prompt * (i + 1) / blocks) - p0;
+        PfMaps pm;
+        if ((rc = make_map_2d(&pm.xh, S->pf_x, n, d, dg::BM)) || (rc = make_map_2d(&pm.xl, S->pf_x + P * d, n, d, dg::BM)) ||
+            (rc = make_map_2d(&pm.oh, oh, n, qd, dg::BM)) || (rc = make_map_2d(&pm.ol, oh + P * qd, n, qd, dg::BM)) ||
+            (rc = make_map_2d(&pm.hh, hh, n, g.d_ff, dg::BM)) || (rc = make_map_2d(&pm.hl, hh + P * g.d_ff, n, g.d_ff, dg::BM)))
+            return rc;
+        dg::k_pf_embed<<<n, 256, 0, S->stream>>>(S->c, (const __nv_bfloat16 *)m->tok_embed, g.rope_base, seq, p0, S->pf_resid, S->pf_cs);
+        CK(cudaGetLastError());
+        S->launches++;
+        for (int l = 0; l < g.n_layers; ++l) if ((rc = run_layer_dense(S, pm, l, seq, p0, n))) return rc;
+        if (i + 1 == blocks) dg::k_pf_last<<<1, 1024, 0, S->stream>>>(S->c, S->pf_resid, n - 1, seq, n_prompt - 1);
+        CK(cudaGetLastError());
+    }
+    if ((rc = run_head(S, 0, SEL_LAST, 1))) return rc;
+    k_prefill_end<<<1, 32, 0, S->stream>>>(S->c, seq, n_prompt, 1, n_prompt);
+    CK(cudaGetLastError());
+    if (seq == 0 && (rc = capture_rows(S, 0))) return rc;
+    CK(cudaMemcpyAsync(S->pinned, S->pf_err, sizeof(int), cudaMemcpyDeviceToHost, S->stream));
+    CK(cudaStreamSynchronize(S->stream));
+    if (S->pinned[0] != 0) {
+        g_cuda_err = "dense prompt pass: a bounded device-side wait expired";
+        return ADA_ETIMEOUT;
+    }
     return ADA_OK;
 }
 
@@ -1193,15 +1244,31 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
         int dev = 0, major = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-        if (major == 10 &&
-            cudaFuncSetAttribute(dg::k_dense_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES) == cudaSuccess &&
-            cudaFuncSetAttribute(dg::k_dense_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES) == cudaSuccess) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (major == 10 && sms >= 2 && prepare_dense<dg::EPI_QKV, 64>() == cudaSuccess && prepare_dense<dg::EPI_QKV, 128>() == cudaSuccess &&
+            prepare_dense<dg::EPI_ADD, 0>() == cudaSuccess && prepare_dense<dg::EPI_SWIGLU, 0>() == cudaSuccess) {
             S->dense_ok = true;
-            S->pf_hi = (__nv_bfloat16 *)(b + lay.pf_hi);
-            S->pf_lo = (__nv_bfloat16 *)(b + lay.pf_lo);
+            S->pf_pairs = std::min(sms / 2, kGemmMaxPairs);
+            S->pf_resid = (float *)(b + lay.pf_resid);
+            S->pf_x = (__nv_bfloat16 *)(b + lay.pf_x);
+            S->pf_u = (__nv_bfloat16 *)(b + lay.pf_u);
+            S->pf_cs = (float *)(b + lay.pf_cs);
             S->pf_err = (int *)(b + lay.pf_err);
+            S->pf_flag = (unsigned *)(b + lay.pf_flag);
             S->pf_part = (float *)(b + lay.pf_part);
-            S->pf_part_bytes = kDenseSplitMax * sizeof(float) * dg::BM * (size_t)g.d_model;
+            const int d = g.d_model, qd = g.n_q_heads * g.head_dim, kvd = g.n_kv_heads * g.head_dim;
+            S->pf_maps.assign(7 * (size_t)g.n_layers, CUtensorMap());
+            for (int l = 0; l < g.n_layers; ++l) {
+                const LayerW &w = m->layers[l];
+                CUtensorMap *wm = &S->pf_maps[7 * (size_t)l];
+                int rc;
+                if ((rc = make_map_2d(wm + 0, w.wq, qd, d, dg::BNH)) || (rc = make_map_2d(wm + 1, w.wk, kvd, d, dg::BNH)) ||
+                    (rc = make_map_2d(wm + 2, w.wv, kvd, d, dg::BNH)) || (rc = make_map_2d(wm + 3, w.wo, d, qd, dg::BNH)) ||
+                    (rc = make_map_2d(wm + 4, w.w_gate, g.d_ff, d, dg::BNH)) || (rc = make_map_2d(wm + 5, w.w_up, g.d_ff, d, dg::BNH)) ||
+                    (rc = make_map_2d(wm + 6, w.w_down, d, g.d_ff, dg::BNH)))
+                    return fail(rc);
+            }
         } else cudaGetLastError();
     }
     // free list: pages are handed out from the back, in a scrambled order so that the page-table
@@ -1260,8 +1327,7 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         int32_t zero = 0;
         CK(cudaMemcpyAsync(&S->c.st->capture_n, &zero, sizeof(int32_t), cudaMemcpyHostToDevice, S->stream));
     }
-    // Prompts of some length take the dense pass: blocks of 128 positions, every weight matrix streamed once per block
-    // through the tcgen05 GEMM, the other operations by the per-operation kernels.
+    // Prompts of some length take the dense pass: blocks of up to dg::PF_ROWS positions through the tcgen05 products.
     const bool dense = S->dense_ok && S->prefill_dense && n_prompt >= 32;
     if (!dense && S->mega && S->path == 1) {
         // prompt passes of eight positions through the persistent kernel
@@ -1274,17 +1340,18 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         S->h_reported[seq] = 0;
         return ADA_OK;
     }
-    const int chunk = dense ? dg::BM : std::min(std::min(S->rows_alloc, kMaxRows), 64);
-    if (dense) CK(cudaMemsetAsync(S->pf_err, 0, sizeof(int), S->stream));
-    struct DenseScope {   // dense_on only while this prefill issues its passes
-        ada_session *S;
-        ~DenseScope() { S->dense_on = false; }
-    } scope{S};
-    S->dense_on = dense;
+    if (dense) {
+        if ((rc = prefill_dense(S, seq, n_prompt))) return rc;
+        S->prefilled[seq] = 1;
+        S->h_prompt[seq] = n_prompt;
+        S->h_len[seq] = n_prompt + 1;
+        S->h_reported[seq] = 0;
+        return ADA_OK;
+    }
+    const int chunk = std::min(std::min(S->rows_alloc, kMaxRows), 64);
     for (int p0 = 0; p0 < n_prompt; p0 += chunk) {
         const int n = std::min(chunk, n_prompt - p0);
         const int last = p0 + n == n_prompt;
-        S->cur_rows = n;
         if (g.dtype == ADA_DTYPE_BF16)
             k_prefill_begin<__nv_bfloat16><<<1, 256, 0, S->stream>>>(S->c, (const __nv_bfloat16 *)m->tok_embed, g.rope_base, seq, p0, n);
         else
@@ -1295,14 +1362,6 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         k_prefill_end<<<1, 32, 0, S->stream>>>(S->c, seq, p0 + n, last, n_prompt);
         CK(cudaGetLastError());
         if (last && seq == 0 && (rc = capture_rows(S, n - 1))) return rc;
-    }
-    if (dense) {
-        CK(cudaMemcpyAsync(S->pinned, S->pf_err, sizeof(int), cudaMemcpyDeviceToHost, S->stream));
-        CK(cudaStreamSynchronize(S->stream));
-        if (S->pinned[0] != 0) {
-            g_cuda_err = "dense prompt pass: a bounded device-side wait expired";
-            return ADA_ETIMEOUT;
-        }
     }
     CK(cudaStreamSynchronize(S->stream));
     S->prefilled[seq] = 1;
@@ -1560,18 +1619,22 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     __nv_bfloat16 *hi = (__nv_bfloat16 *)work_dev, *lo = hi + (size_t)dg::BM * K;
     int *err = (int *)(lo + (size_t)dg::BM * K);
     CUtensorMap mhi, mlo, mw;
-    int rc;
-    if ((rc = make_map_2d(&mhi, hi, dg::BM, K, dg::BM)) || (rc = make_map_2d(&mlo, lo, dg::BM, K, dg::BM)) || (rc = make_map_2d(&mw, W_dev, N, K, dg::BN)))
+    int rc, sms = 0;
+    if ((rc = make_map_2d(&mhi, hi, rows, K, dg::BM)) || (rc = make_map_2d(&mlo, lo, rows, K, dg::BM)) || (rc = make_map_2d(&mw, W_dev, N, K, dg::BNH)))
         return rc;
-    CK(cudaFuncSetAttribute(dg::k_dense_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES));
-    CK(cudaFuncSetAttribute(dg::k_dense_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES));
+    CK((prepare_dense<dg::EPI_STORE, 0>()));
+    CK((prepare_dense<dg::EPI_ADD, 0>()));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaMemsetAsync(err, 0, sizeof(int), stream));
-    dg::k_split_rows<<<dg::BM, 256, 0, stream>>>(X_dev, K, rows, K, hi, lo);
+    dg::k_split_rows<<<rows, 256, 0, stream>>>(X_dev, K, rows, K, hi, lo);
     CK(cudaGetLastError());
-    const int grid = (N + dg::BN - 1) / dg::BN;
-    if (accumulate) dg::k_dense_gemm<1><<<grid, dg::DTHREADS, dg::DSMEM_BYTES, stream>>>(mhi, mlo, mw, Y_dev, ldy, rows, N, K, 0, err);
-    else dg::k_dense_gemm<0><<<grid, dg::DTHREADS, dg::DSMEM_BYTES, stream>>>(mhi, mlo, mw, Y_dev, ldy, rows, N, K, 0, err);
-    CK(cudaGetLastError());
+    dg::GemmArgs a{};
+    a.rows = rows; a.K = K; a.nw[0] = N; a.nt[0] = (N + dg::TN - 1) / dg::TN; a.Y = Y_dev; a.ldy = ldy; a.err = err;
+    a.plan.mt = 1; a.plan.tiles = a.nt[0]; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;   // whole tiles: no exchange area needed
+    a.plan.pairs = std::max(1, std::min(a.plan.tiles, sms / 2));
+    const Ctx none{};
+    rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, mw, none, a);
+    if (rc) return rc;
     int herr = 0;
     CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));

@@ -1,0 +1,81 @@
+"""The dense prompt pass at the edges of its tiles, blocks and work division, against the prompt pass through the
+decode kernel (eight positions at a time)."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from paper_2506_03700_b200 import binding, synth
+
+
+def _model(head_dim, n_q, n_kv, d_model=256, d_ff=704, layers=2):
+    cfg = synth.small_config(dtype="bf16", n_layers=layers, d_model=d_model, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=head_dim,
+                             d_ff=d_ff, vocab=1024, sigma=0.06, resid_scale=0.8, exit_layers=(1,))
+    return cfg, binding.Model(cfg, synth.make_weights(cfg, device="cuda"))
+
+
+def _compare(cfg, gm, n, page_tokens=64):
+    prompt = synth.make_prompt(cfg, n=n).numpy()
+    out = []
+    for dense in (True, False):
+        S = binding.Session(gm, 1, n + 40, page_tokens if dense else 64, 0)
+        S.capture_logits(4)
+        S.set_prefill(dense)
+        S.prefill(prompt)
+        pos = sorted({p for p in (0, 1, 31, 63, 64, 127, 128, 129, 255, 256, n // 2, n - 2, n - 1) if 0 <= p < n})
+        kv = np.stack([S.read_kv(w, l, p) for l in range(cfg.n_layers) for p in pos for w in (0, 1)])
+        out.append((S.state(), kv, S.captured_logits().cpu().numpy()))
+    (sd, kd, ld), (sc, kc, lc) = out
+    assert sd[0] == sc[0] == n + 1 and np.array_equal(sd[1], sc[1])
+    # Both sides hold fp32 sums of the same bf16 products; they differ where a sum's last bits decide the cache's bf16
+    # rounding (one step is at most 2^-7 of a value, i.e. below 2^-8 of the largest of a row twice its size), and by what
+    # such steps move in the layer above.
+    assert np.abs(kd - kc).max() <= 2.0 ** -7 * np.abs(kc).max() * 1.5
+    assert np.linalg.norm(kd - kc) <= 1e-3 * np.linalg.norm(kc)
+    assert np.linalg.norm(ld[0] - lc[0]) <= 5e-3 * np.linalg.norm(lc[0])
+
+
+@pytest.mark.parametrize("n", [32, 63, 128, 129, 256, 257, 513])
+def test_tile_edges(n):
+    _compare(*_model(64, 4, 2), n)
+
+
+@pytest.mark.parametrize("hd,nq,nkv,d,dff", [(128, 4, 1, 512, 1088), (128, 3, 3, 320, 64), (64, 5, 5, 64, 192), (64, 12, 3, 1152, 2624)])
+def test_shapes_of_the_fused_epilogues(hd, nq, nkv, d, dff):
+    """Widths that are no multiples of a tile, of a head pair or of an accumulator chunk."""
+    _compare(*_model(hd, nq, nkv, d, dff), 150)
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 4100])
+def test_block_edges(n):
+    _compare(*_model(64, 4, 1), n)
+
+
+@pytest.mark.parametrize("page_tokens", [16, 32, 128, 256])
+def test_page_sizes(page_tokens):
+    _compare(*_model(128, 2, 1), 300, page_tokens)
+
+
+def test_separate_and_fused_tensors_give_the_same_cache():
+    """q, k, v and gate, up lent as separate tensors go through the same tiles as slices of one."""
+    cfg, gm = _model(64, 4, 2)
+    w = synth.make_weights(cfg, device="cuda")
+    qd, kvd = cfg.n_q_heads * cfg.head_dim, cfg.n_kv_heads * cfg.head_dim
+    sep = {}
+    for k, t in w.items():
+        p = k.rsplit(".", 1)[0] + "."
+        if k.endswith("wqkv"):
+            for name, a, b in (("wq", 0, qd), ("wk", qd, qd + kvd), ("wv", qd + kvd, qd + 2 * kvd)):
+                sep[p + name] = t[a:b].clone()
+        elif k.endswith("w_gate_up"):
+            sep[p + "w_gate"], sep[p + "w_up"] = t[:cfg.d_ff].clone(), t[cfg.d_ff:].clone()
+        else:
+            sep[k] = t
+    prompt = synth.make_prompt(cfg, n=200).numpy()
+    rows = []
+    for m in (gm, binding.Model(cfg, sep)):
+        S = binding.Session(m, 1, 256, 64, 0)
+        S.prefill(prompt)
+        rows.append(np.stack([S.read_kv(wh, l, p) for wh in (0, 1) for l in range(cfg.n_layers) for p in (0, 100, 199)]))
+    assert np.array_equal(rows[0], rows[1])
