@@ -50,7 +50,8 @@ struct Pub {                   // what CTA 0 publishes at a control point
     unsigned seq;
     int action;
     StepDesc d;
-    int pad[8];
+    int cap_keep, cap_at, cap_row0;   // logit capture (test hook): rows to copy, where to, first row of the staging buffer
+    int pad[5];
 };
 
 struct MegaLayer {
@@ -798,22 +799,19 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         }
         if (action == ACT_NEWSTEP || action == ACT_CONTINUE) pub->d = nd;
         pub->action = action;
+        pub->cap_keep = 0;
+        if (kind == CTRL_TOP && c.capture && verified) {
+            const int at = st->capture_n, keep = min(st->keep_rows, st->capture_cap - at);
+            pub->cap_keep = max(keep, 0);
+            pub->cap_at = at;
+            pub->cap_row0 = st->keep_row0;
+            if (keep > 0) st->capture_n = at + keep;
+        }
         sm->bcast[0] = action;
-        sm->bcast[3] = verified;
     }
     bar_consumers();
     const int action = sm->bcast[0];
-    // (c) logits of the verified rows (test hook), then the embedding of the next newest token
-    if (kind == CTRL_TOP && c.capture && sm->bcast[3]) {
-        const int keep = st->keep_rows, at = st->capture_n;
-        for (int j = 0; j < keep && at + j < st->capture_cap; ++j) {
-            const float *src = c.logit_stage + (size_t)(st->keep_row0 + j) * c.vocab;
-            float *dst = c.capture + (size_t)(at + j) * c.vocab;
-            for (int i = tid; i < c.vocab; i += CONS_THREADS) dst[i] = __ldcg(src + i);
-        }
-        bar_consumers();
-        if (tid == 0) st->capture_n = min(st->capture_cap, at + keep);
-    }
+    // (c) the embedding of the next newest token
     if (action == ACT_NEWSTEP) {
         const StepDesc &nd = pub->d;
         const __nv_bfloat16 *g0 = M.layer[0].attn_norm;
@@ -905,10 +903,38 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
         }
         if (threadIdx.x == 0) {
             grid_wait(S, &pub->seq, pub_no);
-            sm->bcast[1] = fetch();
+            const bool cap = kind == CTRL_TOP && A.c.capture && !aborted(S);
+            const int cap_keep = cap ? *(volatile const int *)&pub->cap_keep : 0, cap_at = cap ? *(volatile const int *)&pub->cap_at : 0,
+                      cap_row0 = cap ? *(volatile const int *)&pub->cap_row0 : 0;
+            sm->bcast[1] = fetch();   // also checks that the record was still the expected one after it had been read
+            sm->bcast[5] = aborted(S) ? 0 : cap_keep;
+            sm->bcast[6] = cap_at;
+            sm->bcast[7] = cap_row0;
         }
         bar_consumers();
         action = sm->bcast[1];
+        // Logits of the verified rows (test hook): every CTA copies its share.  (CTA 0 alone took 80 us for a row of 128256
+        // logits, with the whole GPU waiting; shared out it is one round trip to L2.)
+        if (kind == CTRL_TOP && A.c.capture) {
+            const int keep = sm->bcast[5], V = A.c.vocab;
+            for (int j = 0; j < keep; ++j) {
+                const float *src = A.c.logit_stage + (size_t)(sm->bcast[7] + j) * V;
+                float *dst = A.c.capture + (size_t)(sm->bcast[6] + j) * V;
+                for (int i0 = blockIdx.x * CONS_THREADS + threadIdx.x; i0 < V; i0 += 4 * gridDim.x * CONS_THREADS) {
+                    float v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = i0 + u * gridDim.x * CONS_THREADS;
+                        v[u] = i < V ? __ldcg(src + i) : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = i0 + u * gridDim.x * CONS_THREADS;
+                        if (i < V) dst[i] = v[u];
+                    }
+                }
+            }
+        }
     } else {
         grid_wait(S, &pub->seq, pub_no);
         action = fetch();
