@@ -72,9 +72,8 @@ int make_weight_map(CUtensorMap *out, const void *W, int N, int K) {
     return ADA_OK;
 }
 
-// Tensor map of a row-major bf16 matrix [rows][K] for the dense GEMM of the prompt pass: dimensions (K, rows),
-// box (64, box_rows), 128-byte swizzle, zero fill outside.
-int make_map_2d(CUtensorMap *out, const void *base, int rows, int K, int box_rows) {
+// Tensor map of bf16 data: dims innermost first, strides in bytes of dims 1.., zero fill outside.
+int make_map(CUtensorMap *out, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, bool swizzle) {
     typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -89,19 +88,37 @@ int make_map_2d(CUtensorMap *out, const void *base, int rows, int K, int box_row
         }
         encode = (EncodeFn)fn;
     }
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void *>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        g_cuda_err = "cuTensorMapEncodeTiled failed with CUresult " + std::to_string((int)r);
+        return ADA_ECUDA;
+    }
+    return ADA_OK;
+}
+// A row-major matrix [rows][K] as the dense products read it: box (64, box_rows), 128-byte swizzle.
+int make_map_2d(CUtensorMap *out, const void *base, int rows, int K, int box_rows) {
     if (K % 64 || rows < 1 || (uintptr_t)base % 16) return ADA_EUNSUPPORTED;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
     const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult r = encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        g_cuda_err = "cuTensorMapEncodeTiled (2-D) failed with CUresult " + std::to_string((int)r);
-        return ADA_ECUDA;
-    }
-    return ADA_OK;
+    return make_map(out, base, 2, dims, strides, box, true);
+}
+// Queries [rows][heads][hd] of the prompt attention: box of 128 (position, q head of one group) rows x 64 features.
+int make_map_q(CUtensorMap *out, const void *base, int rows, int heads, int hd, int group) {
+    const cuuint64_t dims[3] = {(cuuint64_t)hd, (cuuint64_t)heads, (cuuint64_t)rows};
+    const cuuint64_t strides[2] = {(cuuint64_t)hd * 2, (cuuint64_t)heads * hd * 2};
+    const cuuint32_t box[3] = {64, (cuuint32_t)group, (cuuint32_t)(dg::AT_Q / group)};
+    return make_map(out, base, 3, dims, strides, box, true);
+}
+// The page pool as rows of hd elements: box of box_rows positions x 64 features, copied as stored.
+int make_map_kv(CUtensorMap *out, const void *base, size_t rows, int hd, int box_rows) {
+    const cuuint64_t dims[2] = {(cuuint64_t)hd, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)hd * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    return make_map(out, base, 2, dims, strides, box, false);
 }
 
 }  // namespace
@@ -155,6 +172,8 @@ struct ada_session {
     unsigned *pf_flag = nullptr;
     int *pf_err = nullptr;
     std::vector<CUtensorMap> pf_maps;          // [L][7]: wq, wk, wv, wo, w_gate, w_up, w_down
+    CUtensorMap pf_kv;                         // the page pool
+    int pf_kv_box = 0;                         // positions one copy of it covers
     bool prefill_dense = true;                 // ada_debug_set_prefill
     int64_t launches = 0, syncs = 0, layer_passes = 0;
     // per-class profiling
@@ -354,7 +373,19 @@ template <int EPI, int HD> cudaError_t prepare_dense() {
 }
 
 // Tensor maps of the inputs of a block's products (they end at the block's last row: rows behind it read as zero).
-struct PfMaps { CUtensorMap xh, xl, oh, ol, hh, hl; };
+struct PfMaps { CUtensorMap xh, xl, qh, ql, oh, ol, hh, hl; };
+
+template <int HD, int GROUP>
+int launch_attn_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int pos0, int rows, __nv_bfloat16 *oh, __nv_bfloat16 *ol) {
+    const int per = 2 * dg::AT_Q / GROUP, grid = (rows + per - 1) / per * S->c.nkv;
+    dg::k_pf_attn<HD, GROUP><<<grid, dg::AT_THREADS, dg::at_smem_bytes<HD>(), S->stream>>>(pm.qh, pm.ql, S->pf_kv, S->c, layer, rows, seq, pos0,
+                                                                                          S->pf_kv_box, oh, ol, S->pf_err);
+    CK(cudaGetLastError());
+    return ADA_OK;
+}
+template <int HD, int GROUP> cudaError_t prepare_attn() {
+    return cudaFuncSetAttribute(dg::k_pf_attn<HD, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::at_smem_bytes<HD>());
+}
 
 int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int pos0, int rows) {
     const ada_model *m = S->m;
@@ -366,7 +397,6 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     __nv_bfloat16 *xh = S->pf_x, *xl = xh + P * d, *qh = S->pf_u, *ql = qh + P * qd, *oh = ql + P * qd, *ol = oh + P * qd, *hh = S->pf_u, *hl = hh + P * g.d_ff;
     typedef __nv_bfloat16 T;
     int rc;
-    if (group != 1 && group != 2 && group != 4) return ADA_EUNSUPPORTED;
     dg::GemmArgs a{};
     a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err;
     S->layer_passes++;
@@ -389,13 +419,12 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     }
     {
         Prof pf(S, 4, 0.0);
-        const dim3 grid((rows + 64 / group - 1) / (64 / group), g.n_kv_heads);   // four warps of 16 / group positions each
-#define PF_ATTN(H, G) dg::k_pf_attn_mma<H, G><<<grid, 128, 0, S->stream>>>(S->c, layer, rows, seq, pos0, qh, ql, oh, ol)
-        if (hd == 128) { if (group == 4) PF_ATTN(128, 4); else if (group == 2) PF_ATTN(128, 2); else PF_ATTN(128, 1); }
-        else { if (group == 4) PF_ATTN(64, 4); else if (group == 2) PF_ATTN(64, 2); else PF_ATTN(64, 1); }
-#undef PF_ATTN
+        if (hd == 128) rc = group == 4 ? launch_attn_dense<128, 4>(S, pm, layer, seq, pos0, rows, oh, ol)
+                          : group == 2 ? launch_attn_dense<128, 2>(S, pm, layer, seq, pos0, rows, oh, ol) : launch_attn_dense<128, 1>(S, pm, layer, seq, pos0, rows, oh, ol);
+        else rc = group == 4 ? launch_attn_dense<64, 4>(S, pm, layer, seq, pos0, rows, oh, ol)
+                : group == 2 ? launch_attn_dense<64, 2>(S, pm, layer, seq, pos0, rows, oh, ol) : launch_attn_dense<64, 1>(S, pm, layer, seq, pos0, rows, oh, ol);
+        if (rc) return rc;
     }
-    CK(cudaGetLastError());
     a.nt[0] = (d + dg::TN - 1) / dg::TN;
     a.nt[1] = a.nt[2] = 0;
     a.Y = S->pf_resid; a.ldy = d;
@@ -592,7 +621,10 @@ int prefill_dense(ada_session *S, int seq, int n_prompt) {
     for (int i = 0; i < blocks; ++i) {
         const int p0 = (int)((long long)n_prompt * i / blocks), n = (int)((long long)n_prompt * (i + 1) / blocks) - p0;
         PfMaps pm;
-        if ((rc = make_map_2d(&pm.xh, S->pf_x, n, d, dg::BM)) || (rc = make_map_2d(&pm.xl, S->pf_x + P * d, n, d, dg::BM)) ||
+        const int group = g.n_q_heads / g.n_kv_heads;
+        if (group != 1 && group != 2 && group != 4) return ADA_EUNSUPPORTED;
+        if ((rc = make_map_q(&pm.qh, S->pf_u, n, g.n_q_heads, g.head_dim, group)) || (rc = make_map_q(&pm.ql, S->pf_u + P * qd, n, g.n_q_heads, g.head_dim, group)) ||
+            (rc = make_map_2d(&pm.xh, S->pf_x, n, d, dg::BM)) || (rc = make_map_2d(&pm.xl, S->pf_x + P * d, n, d, dg::BM)) ||
             (rc = make_map_2d(&pm.oh, oh, n, qd, dg::BM)) || (rc = make_map_2d(&pm.ol, oh + P * qd, n, qd, dg::BM)) ||
             (rc = make_map_2d(&pm.hh, hh, n, g.d_ff, dg::BM)) || (rc = make_map_2d(&pm.hl, hh + P * g.d_ff, n, g.d_ff, dg::BM)))
             return rc;
@@ -1247,7 +1279,9 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (major == 10 && sms >= 2 && prepare_dense<dg::EPI_QKV, 64>() == cudaSuccess && prepare_dense<dg::EPI_QKV, 128>() == cudaSuccess &&
-            prepare_dense<dg::EPI_ADD, 0>() == cudaSuccess && prepare_dense<dg::EPI_SWIGLU, 0>() == cudaSuccess) {
+            prepare_dense<dg::EPI_ADD, 0>() == cudaSuccess && prepare_dense<dg::EPI_SWIGLU, 0>() == cudaSuccess && prepare_attn<64, 1>() == cudaSuccess &&
+            prepare_attn<64, 2>() == cudaSuccess && prepare_attn<64, 4>() == cudaSuccess && prepare_attn<128, 1>() == cudaSuccess &&
+            prepare_attn<128, 2>() == cudaSuccess && prepare_attn<128, 4>() == cudaSuccess) {
             S->dense_ok = true;
             S->pf_pairs = std::min(sms / 2, kGemmMaxPairs);
             S->pf_resid = (float *)(b + lay.pf_resid);
@@ -1258,6 +1292,11 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
             S->pf_flag = (unsigned *)(b + lay.pf_flag);
             S->pf_part = (float *)(b + lay.pf_part);
             const int d = g.d_model, qd = g.n_q_heads * g.head_dim, kvd = g.n_kv_heads * g.head_dim;
+            S->pf_kv_box = std::min(page_tokens, 64);
+            {
+                const int rc = make_map_kv(&S->pf_kv, kv_pool_dev, (size_t)n_pages * g.n_layers * 2 * g.n_kv_heads * page_tokens, g.head_dim, S->pf_kv_box);
+                if (rc) return fail(rc);
+            }
             S->pf_maps.assign(7 * (size_t)g.n_layers, CUtensorMap());
             for (int l = 0; l < g.n_layers; ++l) {
                 const LayerW &w = m->layers[l];

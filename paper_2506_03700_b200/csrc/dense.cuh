@@ -115,16 +115,49 @@ __device__ __forceinline__ void umma_commit_pair(unsigned long long *bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(s32(bar)), "h"((uint16_t)3)
                  : "memory");
 }
-// 32 consecutive fp32 columns of this warp's 32 tensor-memory lanes.
+// 32 consecutive fp32 columns of this warp's 32 tensor-memory lanes, waited for (in one statement: the registers are not
+// to be touched before the wait).
 __device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t addr) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
                    "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
                    "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
                    "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                 : "r"(addr));
+                 : "r"(addr)
+                 : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld128(uint32_t (&v)[128], uint32_t addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x128.b32 {"
+                 "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
+                 "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
+                 "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63, "
+                 "%64, %65, %66, %67, %68, %69, %70, %71, %72, %73, %74, %75, %76, %77, %78, %79, "
+                 "%80, %81, %82, %83, %84, %85, %86, %87, %88, %89, %90, %91, %92, %93, %94, %95, "
+                 "%96, %97, %98, %99, %100, %101, %102, %103, %104, %105, %106, %107, %108, %109, %110, %111, "
+                 "%112, %113, %114, %115, %116, %117, %118, %119, %120, %121, %122, %123, %124, %125, %126, %127"
+                 "}, [%128];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+                   "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+                   "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31]),
+                   "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]), "=r"(v[38]), "=r"(v[39]),
+                   "=r"(v[40]), "=r"(v[41]), "=r"(v[42]), "=r"(v[43]), "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]),
+                   "=r"(v[48]), "=r"(v[49]), "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]), "=r"(v[55]),
+                   "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]), "=r"(v[61]), "=r"(v[62]), "=r"(v[63]),
+                   "=r"(v[64]), "=r"(v[65]), "=r"(v[66]), "=r"(v[67]), "=r"(v[68]), "=r"(v[69]), "=r"(v[70]), "=r"(v[71]),
+                   "=r"(v[72]), "=r"(v[73]), "=r"(v[74]), "=r"(v[75]), "=r"(v[76]), "=r"(v[77]), "=r"(v[78]), "=r"(v[79]),
+                   "=r"(v[80]), "=r"(v[81]), "=r"(v[82]), "=r"(v[83]), "=r"(v[84]), "=r"(v[85]), "=r"(v[86]), "=r"(v[87]),
+                   "=r"(v[88]), "=r"(v[89]), "=r"(v[90]), "=r"(v[91]), "=r"(v[92]), "=r"(v[93]), "=r"(v[94]), "=r"(v[95]),
+                   "=r"(v[96]), "=r"(v[97]), "=r"(v[98]), "=r"(v[99]), "=r"(v[100]), "=r"(v[101]), "=r"(v[102]), "=r"(v[103]),
+                   "=r"(v[104]), "=r"(v[105]), "=r"(v[106]), "=r"(v[107]), "=r"(v[108]), "=r"(v[109]), "=r"(v[110]), "=r"(v[111]),
+                   "=r"(v[112]), "=r"(v[113]), "=r"(v[114]), "=r"(v[115]), "=r"(v[116]), "=r"(v[117]), "=r"(v[118]), "=r"(v[119]),
+                   "=r"(v[120]), "=r"(v[121]), "=r"(v[122]), "=r"(v[123]), "=r"(v[124]), "=r"(v[125]), "=r"(v[126]), "=r"(v[127])
+                 : "r"(addr)
+                 : "memory");
+}
 
 // 16-byte load from L2 that the compiler keeps in program order (register pressure stays what the source says).
 __device__ __forceinline__ float4 ld_cg_inorder(const float4 *p) {
@@ -453,7 +486,6 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                         uint32_t v[32];
                         const int col = EPI == EPI_SWIGLU ? (j >> 1) * BNH + h * 64 + (j & 1) * 32 : h * 128 + j * 32;
                         tmem_ld32(v, t_lane + (uint32_t)(b * TN + col));
-                        tmem_ld_wait();
 #pragma unroll
                         for (int e = 0; e < 32; ++e) acc[32 * j + e] += __uint_as_float(v[e]);
 #pragma unroll
@@ -612,149 +644,335 @@ __global__ void k_split_rows(const float *__restrict__ X, int ldx, int rows, int
     }
 }
 
-// Causal attention of a block of prompt rows on the tensor cores (mma.sync m16n8k16, bf16 cache).  One warp owns
-// one 16-row query tile: 16 / GROUP consecutive prompt positions x the GROUP q heads of one kv head; a block of
-// four warps shares the K and V rows of 64 cache positions at a time, copied into shared memory exactly as the
-// cache stores them (16-byte chunks xor-swizzled by position: conflict-free for ldmatrix).  Queries are rotated
-// already, scaled and split into bf16 high / low parts (epi_qkv), the probabilities are split in registers, so nothing but the cache itself is rounded to bf16.  Online softmax in position order; the context
-// is not split, the result goes straight to the next product's
-// input, split into high and low parts.
+// ---------------------------------------------------------------- causal attention of a block of prompt positions
+//
+// Work item = one kv head x 256 query rows: two tiles of 128 rows, a row being one (position, q head of the kv head's
+// group) pair, so that the q heads of a group share every K and V tile.  K and V tiles of 128 positions come from the
+// cache pages by TMA exactly as they are stored: the cache's own 16-byte-chunk swizzle is the 128-byte swizzle of the
+// tensor core's operand layouts (K: K-major; V: MN-major), so nothing is rearranged.  Per tile and key tile
+//     S = Q.lo K^T + Q.hi K^T  (tensor memory, 128 columns)  ->  softmax, one thread per row  ->
+//     P as bf16 high and low parts over the columns of S  ->  O += P V  (A operand from tensor memory).
+// The two tiles take turns: the tensor core works on one while the 128 threads of the other compute its softmax.
+// Online softmax with a lazy reference: O is rescaled only when a row's maximum has grown by more than 2^8 since its
+// reference was set (the reference cancels in the end), so most key tiles touch O in the tensor core only.
+//
+// What bounds it: the tensor core, 4 x 128 x 128 x HD multiply-adds per tile and key tile (high and low parts of Q and
+// of P), 2048 cycles at HD = 128; the softmax of a tile takes about 1500 cycles of its warps and hides behind the other
+// tile.  Key tiles of 128 because an S of 64 columns would read Q from shared memory twice as often as its bandwidth
+// (128 B per cycle) allows.  Rows are independent of each other, so positions past the prompt only waste work.
+constexpr int AT_Q = 128, AT_K = 128, AT_THREADS = 384;
+constexpr int AT_REGS_ISSUE = 56, AT_REGS_SOFT = 224;   // (56 + 224 + 224) x 128 = 168 x 384
+template <int HD> struct AtSmem {   // must start on a 1024-byte boundary
+    static constexpr int HALF = AT_Q * 128;             // 128 rows x 64 features
+    static constexpr int KV = HD / 64 * AT_K * 128;     // one K or V tile
+    static constexpr int SLOTS = HD == 128 ? 3 : 6;
+    alignas(1024) unsigned char q[2][2][HD / 64][HALF];  // [tile][high | low][64-feature group]
+    alignas(1024) unsigned char kv[SLOTS][KV];           // ring of K and V tiles in turn
+    alignas(8) unsigned long long q_full[2], kv_full[SLOTS], kv_empty[SLOTS], s_full[2], p_full[2], o_full[2], tail;
+    uint32_t tmem_base;
+    int abort;
+};
+template <int HD> constexpr size_t at_smem_bytes() { return sizeof(AtSmem<HD>) + 1024; }
+static_assert(at_smem_bytes<128>() <= 232448, "exceeds the 227 KB of shared memory a block may use");
+
+// Descriptor of V [128 positions][64 features] x groups as the MN-major B operand: 64-feature groups AT_K x 128 bytes
+// apart (leading byte offset), groups of eight positions 1024 bytes apart (stride byte offset), 128-byte swizzle.
+__device__ __forceinline__ unsigned long long smem_desc_mn(uint32_t saddr) {
+    return (unsigned long long)((saddr >> 4) & 0x3fffu) | ((unsigned long long)(AT_K * 128 / 16) << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void umma_ss(uint32_t d, unsigned long long a, unsigned long long b, uint32_t id, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b),
+                 "r"(id), "r"(accumulate)
+                 : "memory");
+}
+__device__ __forceinline__ void umma_ts(uint32_t d, uint32_t a, unsigned long long b, uint32_t id, uint32_t accumulate) {   // A from tensor memory
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d), "r"(a), "l"(b),
+                 "r"(id), "r"(accumulate)
+                 : "memory");
+}
+__device__ __forceinline__ void umma_commit(unsigned long long *bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(bar)) : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t addr, const uint32_t *v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(addr),
+                 "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+                   "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
+                   "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
+                   "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t *v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(addr),
+                 "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+                   "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void tma_tile_2d(void *dst, const CUtensorMap *map, int c0, int c1, unsigned long long *bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(s32(dst)), "l"(map),
+                 "r"(c0), "r"(c1), "r"(s32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void tma_tile_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2, unsigned long long *bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(s32(dst)),
+                 "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(s32(bar))
+                 : "memory");
+}
+
+// mapQhi / mapQlo: 3-D maps over the queries [rows][q heads][HD] (box 64 x GROUP x 128 / GROUP, 128-byte swizzle, rows past
+// the block read as zero).  mapKV: 2-D map over the page pool as rows of HD elements (box 64 x kv_box rows, no swizzle).
+// Grid: (256-row items of the block) x kv heads, the items with the longest context first.
 template <int HD, int GROUP>
-__global__ void __launch_bounds__(128) k_pf_attn_mma(Ctx c, int layer, int rows, int seq, int pos0, const __nv_bfloat16 *__restrict__ qhi,
-                                                     const __nv_bfloat16 *__restrict__ qlo, __nv_bfloat16 *__restrict__ ohi, __nv_bfloat16 *__restrict__ olo) {
-    constexpr int KSQ = HD / 16, NT = HD / 8, PPW = 16 / GROUP, TILE = 64;
-    __shared__ __align__(128) unsigned char sK[TILE * HD * 2], sV[TILE * HD * 2];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, kvh = blockIdx.y;
-    const int r_blk = blockIdx.x * 4 * PPW, r_w = r_blk + warp * PPW;   // first row of the block / of this warp
-    const int pos_blk_max = pos0 + min(r_blk + 4 * PPW, rows) - 1;
-    const __nv_bfloat16 *pool = reinterpret_cast<const __nv_bfloat16 *>(c.kv_pool);
-    // ---- this lane's parts of the query fragments: rows lane/4 and lane/4 + 8 of the tile
-    int lim[2];
-    uint32_t ah[KSQ][4], al[KSQ][4];
+__global__ void __launch_bounds__(AT_THREADS, 1)
+k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CUtensorMap mapQlo, const __grid_constant__ CUtensorMap mapKV,
+          const __grid_constant__ Ctx c, int layer, int rows, int seq, int pos0, int kv_box, __nv_bfloat16 *__restrict__ ohi,
+          __nv_bfloat16 *__restrict__ olo, int *err) {
+    typedef AtSmem<HD> Sm;
+    constexpr int PT = AT_Q / GROUP, SLOTS = Sm::SLOTS, HG = HD / 64;
+    extern __shared__ unsigned char dsm_raw[];
+    Sm *sm = reinterpret_cast<Sm *>(dsm_raw + ((1024u - (s32(dsm_raw) & 1023u)) & 1023u));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int kvh = blockIdx.x % c.nkv, item = gridDim.x / c.nkv - 1 - blockIdx.x / c.nkv;
+    const int r0 = item * 2 * PT;                                  // first row (position within the block) of the item
+    const int last = pos0 + min(r0 + 2 * PT, rows) - 1;            // last position any row of the item sees
+    int n_kt[2];                                                   // key tiles of the two query tiles (0: the tile has no rows)
 #pragma unroll
-    for (int rh = 0; rh < 2; ++rh) {
-        const int row = (lane >> 2) + 8 * rh, r = r_w + row / GROUP, g = row % GROUP;
-        const bool live = r < rows;
-        lim[rh] = live ? pos0 + r : -1;
-        const size_t o = ((size_t)min(r, rows - 1) * c.nq + kvh * GROUP + g) * HD;
-#pragma unroll
-        for (int ks = 0; ks < KSQ; ++ks)
-#pragma unroll
-            for (int kh = 0; kh < 2; ++kh) {
-                const int j = ks * 16 + kh * 8 + 2 * (lane & 3);
-                ah[ks][rh + 2 * kh] = live ? *reinterpret_cast<const uint32_t *>(qhi + o + j) : 0u;
-                al[ks][rh + 2 * kh] = live ? *reinterpret_cast<const uint32_t *>(qlo + o + j) : 0u;
-            }
+    for (int t = 0; t < 2; ++t) n_kt[t] = r0 + t * PT < rows ? (pos0 + min(r0 + (t + 1) * PT, rows) - 1) / AT_K + 1 : 0;
+    const int n = max(n_kt[0], n_kt[1]);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sm->q_full[i], 1); mbar_init(&sm->s_full[i], 1); mbar_init(&sm->p_full[i], 4); mbar_init(&sm->o_full[i], 1);
+        }
+        for (int i = 0; i < SLOTS; ++i) { mbar_init(&sm->kv_full[i], 1); mbar_init(&sm->kv_empty[i], 1); }
+        mbar_init(&sm->tail, 1);
+        sm->abort = 0;
+        fence_mbar_init();
+        fence_proxy_async();
     }
-    const int lim_w = r_w < rows ? pos0 + min(r_w + PPW, rows) - 1 : -1;   // last position any row of this warp sees (the same in every lane)
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-    float o[NT][4];
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) o[nt][i] = 0.f;
-    for (int t0 = 0; t0 <= pos_blk_max; t0 += TILE) {
-        __syncthreads();   // the previous tile has been used
-        for (int i = threadIdx.x; i < TILE * (HD / 8); i += 128) {
-            const int t = i / (HD / 8), ch = i - t * (HD / 8), p = t0 + t;
-            uint4 kq = make_uint4(0, 0, 0, 0), vq = kq;
-            if (p <= pos_blk_max) {
-                kq = *reinterpret_cast<const uint4 *>(pool + kv_index(c, seq, layer, 0, kvh, p) + ch * 8);
-                vq = *reinterpret_cast<const uint4 *>(pool + kv_index(c, seq, layer, 1, kvh, p) + ch * 8);
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&sm->tmem_base)), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *(volatile uint32_t *)&sm->tmem_base;   // columns: S of the tiles at 0 and 128, O at 256 and 384
+
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AT_REGS_ISSUE));
+        if (warp == 0) {
+            const int32_t *table = c.page_table + (size_t)seq * c.max_pages;
+            const int last_page = last >> c.page_shift;
+            if (lane == 0)
+                for (int t = 0; t < 2; ++t) {
+                    if (n_kt[t] == 0) continue;
+                    mbar_expect_tx(&sm->q_full[t], 2u * HG * Sm::HALF);
+                    for (int g = 0; g < HG; ++g) {
+                        tma_tile_3d(sm->q[t][0][g], &mapQhi, g * 64, kvh * GROUP, r0 + t * PT, &sm->q_full[t]);
+                        tma_tile_3d(sm->q[t][1][g], &mapQlo, g * 64, kvh * GROUP, r0 + t * PT, &sm->q_full[t]);
+                    }
+                }
+            bool ok = true;
+            for (int it = 0; ok && it < 2 * n; ++it) {   // K of key tile 0, V of key tile 0, K of key tile 1, ...
+                const int st = it % SLOTS, j = it >> 1, which = it & 1;
+                ok = dwait(sm, err, &sm->kv_empty[st], ((it / SLOTS) & 1) ^ 1);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                // V rows of positions the item does not see are multiplied by zero probabilities; they may hold anything (another
+                // sequence's rows, or none), so they are cleared before the tensor core reads them
+                const bool tail = which == 1 && (j + 1) * AT_K - 1 > last;
+                unsigned long long *bar = tail ? &sm->tail : &sm->kv_full[st];
+                if (lane == 0) {
+                    mbar_expect_tx(bar, (uint32_t)Sm::KV);
+                    for (int r = 0; r < AT_K; r += kv_box) {
+                        const int p = j * AT_K + r, page = table[min(p >> c.page_shift, last_page)];
+                        const int row = (int)(((((long long)page * c.L + layer) * 2 + which) * c.nkv + kvh) * c.page_tokens) + (p & (c.page_tokens - 1));
+                        for (int g = 0; g < HG; ++g) tma_tile_2d(sm->kv[st] + g * (AT_K * 128) + r * 128, &mapKV, g * 64, row, bar);
+                    }
+                }
+                __syncwarp();
+                if (tail) {   // at most once: the last tile
+                    ok = dwait(sm, err, &sm->tail, 0);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const int from = last + 1 - j * AT_K;   // first cleared row
+                    for (int g = 0; g < HG; ++g)
+                        for (int i = from * 8 + lane; i < AT_K * 8; i += 32)
+                            *reinterpret_cast<uint4 *>(sm->kv[st] + g * (AT_K * 128) + i * 16) = make_uint4(0, 0, 0, 0);
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sm->kv_full[st]);
+                }
             }
-            *reinterpret_cast<uint4 *>(sK + (size_t)t * HD * 2 + ch * 16) = kq;
-            *reinterpret_cast<uint4 *>(sV + (size_t)t * HD * 2 + ch * 16) = vq;
+        } else if (warp == 1 && lane == 0) {
+            constexpr uint32_t ID_S = Idesc<AT_Q, AT_K>::v, ID_O = Idesc<AT_Q, HD>::v | (1u << 16);   // bit 16: B is MN-major
+            bool ok = true;
+            auto issue_s = [&](int t, int st) {
+                const uint32_t d = tmem + (uint32_t)(t * AT_K);
+                uint32_t add = 0;
+#pragma unroll 1
+                for (int i = 2 * HG - 1; i >= 0; --i) {   // low parts first: the small products are added up before the large ones
+                    const int part = i / HG, g = i % HG;
+                    const unsigned long long qd = smem_desc(s32(sm->q[t][part][g])), kd = smem_desc(s32(sm->kv[st] + g * (AT_K * 128)));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        umma_ss(d, qd + 2 * k, kd + 2 * k, ID_S, add);
+                        add = 1u;
+                    }
+                }
+                umma_commit(&sm->s_full[t]);
+            };
+            if (n > 0) ok = dwait(sm, err, &sm->kv_full[0], 0);
+            tc_fence_after();
+            for (int t = 0; ok && t < 2; ++t) {
+                if (n_kt[t] == 0) continue;
+                ok = dwait(sm, err, &sm->q_full[t], 0);
+                if (!ok) break;
+                tc_fence_after();
+                issue_s(t, 0);
+            }
+            if (ok) umma_commit(&sm->kv_empty[0]);
+            for (int j = 0; ok && j < n; ++j) {
+                const int iv = 2 * j + 1, ik = 2 * j + 2, sv = iv % SLOTS, sk = ik % SLOTS;
+                ok = dwait(sm, err, &sm->kv_full[sv], (iv / SLOTS) & 1);
+                if (!ok) break;
+                tc_fence_after();
+                bool have_k = false;
+                for (int t = 0; ok && t < 2; ++t) {
+                    if (j >= n_kt[t]) continue;
+                    ok = dwait(sm, err, &sm->p_full[t], j & 1);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d = tmem + 256u + (uint32_t)(t * 128), pa = tmem + (uint32_t)(t * AT_K);
+                    uint32_t add = j > 0 ? 1u : 0u;
+#pragma unroll 1
+                    for (int i = 3; i >= 0; --i) {   // P.lo, then P.hi, half of the positions at a time
+                        const unsigned long long vd = smem_desc_mn(s32(sm->kv[sv])) + 512 * (i & 1);
+                        const uint32_t pi = pa + (uint32_t)(32 * i);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {   // sixteen positions: two groups of eight rows of V, eight columns of P
+                            umma_ts(d, pi + (uint32_t)(8 * k), vd + 128 * k, ID_O, add);
+                            add = 1u;
+                        }
+                    }
+                    if (t == 1 || n_kt[1] <= j) umma_commit(&sm->kv_empty[sv]);
+                    if (j + 1 < n_kt[t]) {
+                        if (!have_k) {
+                            ok = dwait(sm, err, &sm->kv_full[sk], (ik / SLOTS) & 1);
+                            if (!ok) break;
+                            tc_fence_after();
+                            have_k = true;
+                        }
+                        issue_s(t, sk);
+                    } else umma_commit(&sm->o_full[t]);
+                }
+                if (ok && j + 1 < n) umma_commit(&sm->kv_empty[sk]);
+            }
         }
-        __syncthreads();
-        for (int sl = 0; sl < TILE / 16; ++sl) {
-            const int p0 = t0 + 16 * sl;
-            if (p0 > lim_w) break;   // nothing further in this tile is visible to this warp (uniform per warp)
-            // ---- scores of the 16 positions p0 .. p0 + 15
-            float sh[2][4], sl_[2][4];
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(AT_REGS_SOFT));
+        const int t = (warp - 4) >> 2, q = warp & 3, row = q * 32 + lane;
+        const int r = r0 + t * PT + row / GROUP, pos = pos0 + r;             // row of the block, its position
+        const int pos_min = pos0 + r0 + t * PT;                              // smallest position of the tile
+        const uint32_t t_s = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * AT_K), t_o = tmem + ((uint32_t)(q * 32) << 16) + 256u + (uint32_t)(t * 128);
+        constexpr float LOG2E = 1.4426950408889634f;
+        float ref = 0.f, l = 0.f;   // ref: reference exponent (log2 units) the row's P, O and l are relative to
+        bool ok = true;
+        for (int j = 0; ok && j < n_kt[t]; ++j) {
+            ok = dwait(sm, err, &sm->s_full[t], j & 1);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            uint32_t s[128];
+            tmem_ld128(s, t_s);
+            if ((j + 1) * AT_K - 1 > pos_min) {   // some row of the tile does not see all of these positions
+                const int lim = pos - j * AT_K;
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+                for (int e = 0; e < 128; ++e) s[e] = e <= lim ? s[e] : 0xff800000u;
+            }
+            float mx[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) { sh[nt][i] = 0.f; sl_[nt][i] = 0.f; }
-            const int id = lane >> 3;
-            {
-                const int pl = 16 * sl + (lane & 7) + 8 * (id >> 1);
-                const unsigned char *krow = sK + pl * (HD * 2);
+            for (int e = 0; e < 4; ++e) mx[e] = __uint_as_float(s[e]);
 #pragma unroll
-                for (int ks = 0; ks < KSQ; ++ks) {
-                    uint32_t kf[4];
-                    ldmatrix_x4(kf, krow + ((((2 * ks) | (id & 1)) ^ (pl & 7)) << 4));
-                    mma16816(sh[0], ah[ks], kf[0], kf[1]);
-                    mma16816(sh[1], ah[ks], kf[2], kf[3]);
-                    mma16816(sl_[0], al[ks], kf[0], kf[1]);
-                    mma16816(sl_[1], al[ks], kf[2], kf[3]);
+            for (int e = 4; e < 128; ++e) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(s[e]));
+            const float m2 = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * LOG2E;
+            if (j == 0) ref = m2;
+            else if (__any_sync(0xffffffffu, m2 > ref + 8.f)) {
+                // the previous key tile's O is complete (its products were issued before those of this S)
+                const float nr = m2 > ref + 8.f ? m2 : ref, f = ex2(ref - nr);
+                ref = nr;
+                l *= f;
+#pragma unroll 1
+                for (int b = 0; b < HD / 32; ++b) {
+                    uint32_t v[32];
+                    tmem_ld32(v, t_o + 32 * b);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * f);
+                    tmem_st32(t_o + 32 * b, v);
                 }
             }
-            float s[2][4];
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int b = 0; b < 4; ++b) {   // 32 probabilities -> 16 words of high parts and 16 of low parts
+                uint32_t h[16], lo[16];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int pos = p0 + 8 * nt + 2 * (lane & 3) + (i & 1);
-                    s[nt][i] = pos <= lim[i >> 1] ? sh[nt][i] + sl_[nt][i] : -INFINITY;
+                for (int e = 0; e < 16; ++e) {
+                    const float p0 = ex2(fmaf(__uint_as_float(s[32 * b + 2 * e]), LOG2E, -ref)), p1 = ex2(fmaf(__uint_as_float(s[32 * b + 2 * e + 1]), LOG2E, -ref));
+                    sum[2 * (e & 1)] += p0;
+                    sum[2 * (e & 1) + 1] += p1;
+                    split2(p0, p1, h[e], lo[e]);
                 }
-            // ---- online softmax
-            uint32_t ph[4], plo[4];
-#pragma unroll
-            for (int rh = 0; rh < 2; ++rh) {
-                float mx = fmaxf(fmaxf(s[0][2 * rh], s[0][2 * rh + 1]), fmaxf(s[1][2 * rh], s[1][2 * rh + 1]));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                const float mn = fmaxf(m_run[rh], mx);
-                float corr = 1.f, p[4] = {0.f, 0.f, 0.f, 0.f};
-                if (mn != -INFINITY) {
-                    corr = __expf(m_run[rh] - mn);
-                    p[0] = __expf(s[0][2 * rh] - mn); p[1] = __expf(s[0][2 * rh + 1] - mn);
-                    p[2] = __expf(s[1][2 * rh] - mn); p[3] = __expf(s[1][2 * rh + 1] - mn);
-                }
-                m_run[rh] = mn;
-                l_run[rh] = l_run[rh] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) { o[nt][2 * rh] *= corr; o[nt][2 * rh + 1] *= corr; }
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(p[0], p[1]), h1 = __floats2bfloat162_rn(p[2], p[3]);
-                const __nv_bfloat162 l0 = __floats2bfloat162_rn(p[0] - __low2float(h0), p[1] - __high2float(h0));
-                const __nv_bfloat162 l1 = __floats2bfloat162_rn(p[2] - __low2float(h1), p[3] - __high2float(h1));
-                ph[rh] = *reinterpret_cast<const uint32_t *>(&h0);
-                ph[2 + rh] = *reinterpret_cast<const uint32_t *>(&h1);
-                plo[rh] = *reinterpret_cast<const uint32_t *>(&l0);
-                plo[2 + rh] = *reinterpret_cast<const uint32_t *>(&l1);
+                tmem_st16(t_s + 16 * b, h);
+                tmem_st16(t_s + 64 + 16 * b, lo);
             }
-            // ---- o += P V
-            {
-                const int pl = 16 * sl + (lane & 7) + 8 * (id & 1);
-                const unsigned char *vrow = sV + pl * (HD * 2);
+            l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm->p_full[t]);
+        }
+        if (ok && n_kt[t] > 0) {
+            ok = dwait(sm, err, &sm->o_full[t], 0);
+            ok = __all_sync(0xffffffffu, ok);
+            tc_fence_after();
+            if (ok) {
+                const float inv = 1.0f / l;
+                const size_t o = ((size_t)r * c.nq + kvh * GROUP + row % GROUP) * HD;
+#pragma unroll 1
+                for (int b = 0; b < HD / 32; ++b) {
+                    uint32_t v[32];
+                    tmem_ld32(v, t_o + 32 * b);
+                    if (r < rows)
 #pragma unroll
-                for (int np = 0; np < NT / 2; ++np) {
-                    uint32_t vf[4];
-                    ldmatrix_x4_trans(vf, vrow + ((((2 * np) | (id >> 1)) ^ (pl & 7)) << 4));
-                    mma16816(o[2 * np], ph, vf[0], vf[1]);
-                    mma16816(o[2 * np + 1], ph, vf[2], vf[3]);
-                    mma16816(o[2 * np], plo, vf[0], vf[1]);
-                    mma16816(o[2 * np + 1], plo, vf[2], vf[3]);
+                        for (int e = 0; e < 32; e += 8) {
+                            uint4 h, w;
+                            split2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv, h.x, w.x);
+                            split2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv, h.y, w.y);
+                            split2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv, h.z, w.z);
+                            split2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv, h.w, w.w);
+                            *reinterpret_cast<uint4 *>(ohi + o + 32 * b + e) = h;
+                            *reinterpret_cast<uint4 *>(olo + o + 32 * b + e) = w;
+                        }
                 }
             }
         }
     }
-#pragma unroll
-    for (int rh = 0; rh < 2; ++rh) {
-        l_run[rh] += __shfl_xor_sync(0xffffffffu, l_run[rh], 1);
-        l_run[rh] += __shfl_xor_sync(0xffffffffu, l_run[rh], 2);
-        const int row = (lane >> 2) + 8 * rh, r = r_w + row / GROUP, g = row % GROUP;
-        if (r < rows) {
-            const size_t o_at = ((size_t)r * c.nq + kvh * GROUP + g) * HD;
-            const float inv = 1.0f / l_run[rh];
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                uint32_t h, l;
-                split2(o[nt][2 * rh] * inv, o[nt][2 * rh + 1] * inv, h, l);
-                *reinterpret_cast<uint32_t *>(ohi + o_at + nt * 8 + 2 * (lane & 3)) = h;
-                *reinterpret_cast<uint32_t *>(olo + o_at + nt * 8 + 2 * (lane & 3)) = l;
-            }
-        }
+    if (*(volatile int *)&sm->abort) {   // copies already issued may still be landing: give them time before the block's memory goes
+        const unsigned long long t0 = gtime();
+        while (gtime() - t0 < 200000ull) __nanosleep(1000);
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }
 }
 
