@@ -361,12 +361,24 @@ dg::GemmPlan plan_dense(int rows, int nt, int K, int pairs) {
     return g;
 }
 
+// Launch of a kernel that may start while the one before it in the stream drains (it calls dg::pdl_wait()).
+template <typename... P, typename... V>
+int launch_overlapped(cudaStream_t stream, void (*kernel)(P...), int grid, int threads, size_t smem, V &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, kernel, std::forward<V>(args)...));
+    return ADA_OK;
+}
+
 template <int EPI, int HD>
 int launch_dense(cudaStream_t stream, const CUtensorMap &xh, const CUtensorMap &xl, const CUtensorMap &w0, const CUtensorMap &w1,
                  const CUtensorMap &w2, const Ctx &c, const dg::GemmArgs &a) {
-    dg::k_dense_gemm<EPI, HD><<<2 * a.plan.pairs, dg::GTHREADS, dg::DSMEM_BYTES, stream>>>(xh, xl, w0, w1, w2, c, a);
-    CK(cudaGetLastError());
-    return ADA_OK;
+    return launch_overlapped(stream, dg::k_dense_gemm<EPI, HD>, 2 * a.plan.pairs, dg::GTHREADS, dg::DSMEM_BYTES, xh, xl, w0, w1, w2, c, a);
 }
 template <int EPI, int HD> cudaError_t prepare_dense() {
     return cudaFuncSetAttribute(dg::k_dense_gemm<EPI, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES);
@@ -378,10 +390,8 @@ struct PfMaps { CUtensorMap xh, xl, qh, ql, oh, ol, hh, hl; };
 template <int HD, int GROUP>
 int launch_attn_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int pos0, int rows, __nv_bfloat16 *oh, __nv_bfloat16 *ol) {
     const int per = 2 * dg::AT_Q / GROUP, grid = (rows + per - 1) / per * S->c.nkv;
-    dg::k_pf_attn<HD, GROUP><<<grid, dg::AT_THREADS, dg::at_smem_bytes<HD>(), S->stream>>>(pm.qh, pm.ql, S->pf_kv, S->c, layer, rows, seq, pos0,
-                                                                                          S->pf_kv_box, oh, ol, S->pf_err);
-    CK(cudaGetLastError());
-    return ADA_OK;
+    return launch_overlapped(S->stream, dg::k_pf_attn<HD, GROUP>, grid, dg::AT_THREADS, dg::at_smem_bytes<HD>(), pm.qh, pm.ql, S->pf_kv, S->c, layer, rows,
+                             seq, pos0, S->pf_kv_box, oh, ol, S->pf_err);
 }
 template <int HD, int GROUP> cudaError_t prepare_attn() {
     return cudaFuncSetAttribute(dg::k_pf_attn<HD, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::at_smem_bytes<HD>());
@@ -403,10 +413,9 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     S->launches += 7;
     auto norm = [&](const void *gain) {
         Prof pf(S, 1, 0.0);
-        dg::k_norm_split_rows<<<rows, 256, 0, S->stream>>>(S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl);
+        return launch_overlapped(S->stream, dg::k_norm_split_rows, rows, 256, 0, S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl);
     };
-    norm(w.attn_norm);
-    CK(cudaGetLastError());
+    if ((rc = norm(w.attn_norm))) return rc;
     {
         Prof pf(S, 2, (double)(qd + 2 * kvd) * d * 2);
         a.nw[0] = qd; a.nw[1] = a.nw[2] = kvd;
@@ -434,8 +443,7 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
         a.plan = plan_dense(rows, a.nt[0], qd, S->pf_pairs);
         if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.oh, pm.ol, wm[3], wm[3], wm[3], S->c, a))) return rc;
     }
-    norm(w.ffn_norm);
-    CK(cudaGetLastError());
+    if ((rc = norm(w.ffn_norm))) return rc;
     {
         Prof pf(S, 6, (double)2 * g.d_ff * d * 2);
         a.nw[0] = a.nw[1] = g.d_ff; a.K = d; a.hi = hh; a.lo = hl; a.epoch = ++S->pf_epoch;

@@ -66,6 +66,13 @@ constexpr size_t DSMEM_BYTES = sizeof(DSmem) + 1024;
 static_assert(STAGE_BYTES % 1024 == 0 && A_BYTES % 1024 == 0, "operand tiles must start on 1024-byte boundaries");
 static_assert(DSMEM_BYTES <= 232448, "exceeds the 227 KB of shared memory a block may use");
 
+// Programmatic dependent launch: the kernels of a layer follow one another in the stream, each allowed to start (launch,
+// barriers, tensor memory, first weight tiles) while the one before it drains.  Nothing that an earlier kernel writes, and
+// nothing that an earlier kernel may still read, is touched before pdl_wait(), which returns when all of them are complete.
+// Every CTA passes pdl_wait(), so "the kernel before me is complete" carries over to all kernels before it.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -372,6 +379,7 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const int pair = blockIdx.x >> 1, nkb = a.K / BK;
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int i = 0; i < STAGES; ++i) { mbar_init(&sm->full[i], 1); mbar_init(&sm->empty[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&sm->acc_full[i], 1); mbar_init(&sm->acc_empty[i], 2 * GEPI_WARPS); }
@@ -393,36 +401,55 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GREGS_ISSUE));
         if (warp == 0 && lane == 0) {
+            const uint32_t m_row = rank * BM;
+            auto weights = [&](int tn, const CUtensorMap *&mw) -> int {   // map and first row of this CTA's half of the tile's weight rows
+                mw = &mapW0;
+                if (EPI == EPI_SWIGLU) {
+                    if (rank) mw = &mapW1;
+                    return tn * BNH;
+                }
+                int t = tn;
+                if (EPI == EPI_QKV && t >= a.nt[0]) {
+                    t -= a.nt[0];
+                    mw = &mapW1;
+                    if (t >= a.nt[1]) { t -= a.nt[1]; mw = &mapW2; }
+                }
+                return t * TN + (int)rank * BNH;
+            };
+            auto load_w = [&](int st, const CUtensorMap *mw, int kb, int n0) {
+                if (rank == 0) mbar_expect_tx(&sm->full[st], 2u * STAGE_BYTES);   // both CTAs' tiles complete on the first CTA's barrier
+                tma_load_2d_pair(sm->stage[st] + 2 * A_BYTES, mw, kb * BK, n0, map_to_cta(&sm->full[st], 0));
+            };
+            // the weights of the first stages do not depend on earlier kernels
+            int ahead = 0;
+            {
+                Sched sch(a.plan, pair);
+                Seg s;
+                if (sch.next(s)) {
+                    const CUtensorMap *mw;
+                    const int n0 = weights(s.tile / a.plan.mt, mw), kb0 = s.c0 * CK, kb1 = min(s.c1 * CK, nkb);
+                    for (; ahead < STAGES && kb0 + ahead < kb1; ++ahead) load_w(ahead, mw, kb0 + ahead, n0);
+                }
+            }
+            pdl_wait();
             Sched sch(a.plan, pair);
             Seg s;
             int it = 0;
             bool ok = true;
             while (ok && sch.next(s)) {
-                const int tm = s.tile % a.plan.mt, tn = s.tile / a.plan.mt, m0 = tm * TM + (int)rank * BM;
-                const CUtensorMap *mw = &mapW0;
-                int n0;
-                if (EPI == EPI_SWIGLU) {
-                    n0 = tn * BNH;
-                    if (rank) mw = &mapW1;
-                } else {
-                    int t = tn;
-                    if (EPI == EPI_QKV && t >= a.nt[0]) {
-                        t -= a.nt[0];
-                        mw = &mapW1;
-                        if (t >= a.nt[1]) { t -= a.nt[1]; mw = &mapW2; }
-                    }
-                    n0 = t * TN + (int)rank * BNH;
-                }
-                const int kb1 = min(s.c1 * CK, nkb);
+                const int tm = s.tile % a.plan.mt, m0 = tm * TM + (int)m_row;
+                const CUtensorMap *mw;
+                const int n0 = weights(s.tile / a.plan.mt, mw), kb1 = min(s.c1 * CK, nkb);
                 for (int kb = s.c0 * CK; kb < kb1; ++kb, ++it) {
                     const int st = it % STAGES;
-                    ok = dwait(sm, a.err, &sm->empty[st], ((it / STAGES) & 1) ^ 1);
-                    if (!ok) break;
-                    if (rank == 0) mbar_expect_tx(&sm->full[st], 2u * STAGE_BYTES);   // both CTAs' tiles complete on the first CTA's barrier
+                    if (it >= ahead) {
+                        ok = dwait(sm, a.err, &sm->empty[st], ((it / STAGES) & 1) ^ 1);
+                        if (!ok) break;
+                        load_w(st, mw, kb, n0);
+                    }
                     const uint32_t bar = map_to_cta(&sm->full[st], 0);
                     tma_load_2d_pair(sm->stage[st], &mapXhi, kb * BK, m0, bar);
                     tma_load_2d_pair(sm->stage[st] + A_BYTES, &mapXlo, kb * BK, m0, bar);
-                    tma_load_2d_pair(sm->stage[st] + 2 * A_BYTES, mw, kb * BK, n0, bar);
                 }
             }
         }
@@ -463,6 +490,7 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
         // epilogue: warp w may read the 32 lanes 32 (w % 4) .. of the tensor memory; lane = position within the CTA's 128
         const int q = warp & 3, h = (warp - 4) >> 2, ew = warp - 4;
         const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
+        pdl_wait();
         Sched sch(a.plan, pair);
         Seg s;
         int ch = 0;
@@ -528,12 +556,12 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                     if (!ok) break;
                     const float4 *in = reinterpret_cast<const float4 *>(reinterpret_cast<const unsigned char *>(a.part) + (size_t)cta * GPART_CTA + ew * GPART_WARP) + lane;
 #pragma unroll
-                    for (int j0 = 0; j0 < 32; j0 += 8) {   // eight loads in flight: more would not fit beside the sums
-                        float4 r[8];
+                    for (int j0 = 0; j0 < 32; j0 += 16) {   // sixteen loads in flight: more would not fit beside the sums
+                        float4 r[16];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) r[j] = ld_cg_inorder(in + 32 * (j0 + j));
+                        for (int j = 0; j < 16; ++j) r[j] = ld_cg_inorder(in + 32 * (j0 + j));
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
+                        for (int j = 0; j < 16; ++j) {
                             const int e = 4 * (j0 + j);
                             acc[e] += r[j].x; acc[e + 1] += r[j].y; acc[e + 2] += r[j].z; acc[e + 3] += r[j].w;
                         }
@@ -608,6 +636,8 @@ __global__ void __launch_bounds__(256) k_norm_split_rows(const float *__restrict
                                                          float eps, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
     const int r = blockIdx.x;
     __shared__ float red[8];
+    pdl_trigger();
+    pdl_wait();
     const float4 *x = reinterpret_cast<const float4 *>(X + (size_t)r * K);
     float ss = 0.f;
     for (int i = threadIdx.x; i < K / 4; i += 256) {
@@ -744,6 +774,7 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
 #pragma unroll
     for (int t = 0; t < 2; ++t) n_kt[t] = r0 + t * PT < rows ? (pos0 + min(r0 + (t + 1) * PT, rows) - 1) / AT_K + 1 : 0;
     const int n = max(n_kt[0], n_kt[1]);
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sm->q_full[i], 1); mbar_init(&sm->s_full[i], 1); mbar_init(&sm->p_full[i], 4); mbar_init(&sm->o_full[i], 1);
@@ -767,6 +798,7 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AT_REGS_ISSUE));
         if (warp == 0) {
+            pdl_wait();
             const int32_t *table = c.page_table + (size_t)seq * c.max_pages;
             const int last_page = last >> c.page_shift;
             if (lane == 0)
@@ -882,6 +914,7 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
         const int pos_min = pos0 + r0 + t * PT;                              // smallest position of the tile
         const uint32_t t_s = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * AT_K), t_o = tmem + ((uint32_t)(q * 32) << 16) + 256u + (uint32_t)(t * 128);
         constexpr float LOG2E = 1.4426950408889634f;
+        pdl_wait();
         float ref = 0.f, l = 0.f;   // ref: reference exponent (log2 units) the row's P, O and l are relative to
         bool ok = true;
         for (int j = 0; ok && j < n_kt[t]; ++j) {
