@@ -20,6 +20,12 @@ namespace {
 
 thread_local std::string g_cuda_err;
 
+// a launch helper that already reports its own error
+#define CKL(expr)                     \
+    do {                              \
+        const int rc__ = (expr);      \
+        if (rc__ != ADA_OK) return rc__; \
+    } while (0)
 #define CK(expr)                                                                                    \
     do {                                                                                            \
         cudaError_t e__ = (expr);                                                                   \
@@ -209,6 +215,7 @@ int rows_alloc_for(const ada_config &g, int batch, int max_early) {
 }
 // positions of one block of a dense prompt pass: a prompt is cut alike whatever the session's length limit
 int pf_rows_for(int max_seq) { return std::min(dg::PF_ROWS, (int)align_up((size_t)max_seq, dg::BM)); }
+constexpr int kDenseMin = 17;       // prompt tokens from which the dense pass is taken
 constexpr int kGemmMaxPairs = 80;   // CTA pairs the exchange area of cut tiles is laid out for
 
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
@@ -331,6 +338,20 @@ void prof_collect(ada_session *S) {
 
 // ---- typed launch helpers --------------------------------------------------------------------
 
+// Launch of a kernel that may start while the one before it in the stream drains (it calls pdl_wait()).
+template <typename... P, typename... V>
+int launch_overlapped(cudaStream_t stream, void (*kernel)(P...), dim3 grid, int threads, size_t smem, V &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, kernel, std::forward<V>(args)...));
+    return ADA_OK;
+}
+
 // ---- dense prompt pass: one decoder layer over a block of up to dg::PF_ROWS prompt positions --------------------
 
 // How a product of `nt` tile columns and depth K over `rows` positions is divided over at most `pairs` CTA pairs.  More
@@ -359,20 +380,6 @@ dg::GemmPlan plan_dense(int rows, int nt, int K, int pairs) {
     g.sk_tiles = g.tiles;
     g.sk_pairs = g.pairs;
     return g;
-}
-
-// Launch of a kernel that may start while the one before it in the stream drains (it calls dg::pdl_wait()).
-template <typename... P, typename... V>
-int launch_overlapped(cudaStream_t stream, void (*kernel)(P...), int grid, int threads, size_t smem, V &&...args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    CK(cudaLaunchKernelEx(&cfg, kernel, std::forward<V>(args)...));
-    return ADA_OK;
 }
 
 template <int EPI, int HD>
@@ -464,9 +471,9 @@ int launch_gemv(ada_session *S, int cls, int epi, const void *W, int N, int K, c
     Prof pf(S, cls, (double)N * K * sizeof(T));
     int blocks = std::min((N + 7) / 8, 148 * 4);
     if (epi == 0)
-        k_gemv<T, 0><<<blocks, 256, 0, S->stream>>>(S->c, (const T *)W, N, K, X, ldx, Y, ldy, sel);
+        CKL(launch_overlapped(S->stream, k_gemv<T, 0>, blocks, 256, 0, S->c, (const T *)W, N, K, X, ldx, Y, ldy, sel));
     else
-        k_gemv<T, 1><<<blocks, 256, 0, S->stream>>>(S->c, (const T *)W, N, K, X, ldx, Y, ldy, sel);
+        CKL(launch_overlapped(S->stream, k_gemv<T, 1>, blocks, 256, 0, S->c, (const T *)W, N, K, X, ldx, Y, ldy, sel));
     S->launches++;
     CK(cudaGetLastError());
     return ADA_OK;
@@ -478,17 +485,17 @@ int launch_attn(ada_session *S, int layer, int rows) {
     Prof pf(S, 4, 0.0);
     dim3 grid(S->n_chunks, g.n_q_heads, rows);
     switch (g.head_dim / 32) {
-        case 1: k_attn_partial<T, 1><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        case 2: k_attn_partial<T, 2><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        case 3: k_attn_partial<T, 3><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        case 4: k_attn_partial<T, 4><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        case 5: k_attn_partial<T, 5><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        case 6: k_attn_partial<T, 6><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        case 7: k_attn_partial<T, 7><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
-        default: k_attn_partial<T, 8><<<grid, 32, 0, S->stream>>>(S->c, layer); break;
+        case 1: CKL(launch_overlapped(S->stream, k_attn_partial<T, 1>, grid, 32, 0, S->c, layer)); break;
+        case 2: CKL(launch_overlapped(S->stream, k_attn_partial<T, 2>, grid, 32, 0, S->c, layer)); break;
+        case 3: CKL(launch_overlapped(S->stream, k_attn_partial<T, 3>, grid, 32, 0, S->c, layer)); break;
+        case 4: CKL(launch_overlapped(S->stream, k_attn_partial<T, 4>, grid, 32, 0, S->c, layer)); break;
+        case 5: CKL(launch_overlapped(S->stream, k_attn_partial<T, 5>, grid, 32, 0, S->c, layer)); break;
+        case 6: CKL(launch_overlapped(S->stream, k_attn_partial<T, 6>, grid, 32, 0, S->c, layer)); break;
+        case 7: CKL(launch_overlapped(S->stream, k_attn_partial<T, 7>, grid, 32, 0, S->c, layer)); break;
+        default: CKL(launch_overlapped(S->stream, k_attn_partial<T, 8>, grid, 32, 0, S->c, layer)); break;
     }
     CK(cudaGetLastError());
-    k_attn_combine<<<dim3(g.n_q_heads, rows), 64, 0, S->stream>>>(S->c, layer);
+    CKL(launch_overlapped(S->stream, k_attn_combine, dim3(g.n_q_heads, rows), 64, 0, S->c, layer));
     CK(cudaGetLastError());
     S->launches += 2;
     return ADA_OK;
@@ -506,7 +513,7 @@ int run_layer_t(ada_session *S, int layer, int rows) {
     S->layer_passes++;
     {
         Prof pf(S, 1, 0.0);
-        k_rmsnorm<T><<<rows, 256, 0, S->stream>>>(S->c, (const T *)w.attn_norm, layer, S->c.xn, ldx);
+        CKL(launch_overlapped(S->stream, k_rmsnorm<T>, rows, 256, 0, S->c, (const T *)w.attn_norm, layer, S->c.xn, ldx));
     }
     CK(cudaGetLastError());
     S->launches++;
@@ -523,7 +530,7 @@ int run_layer_t(ada_session *S, int layer, int rows) {
     }
     {
         Prof pf(S, 3, 0.0);
-        k_rope_kv<T><<<rows, 128, 0, S->stream>>>(S->c, layer);
+        CKL(launch_overlapped(S->stream, k_rope_kv<T>, rows, 128, 0, S->c, layer));
     }
     CK(cudaGetLastError());
     S->launches++;
@@ -531,7 +538,7 @@ int run_layer_t(ada_session *S, int layer, int rows) {
     if ((rc = launch_gemv<T>(S, 5, 1, w.wo, d, qd, S->c.attn_out, qd, S->c.resid, d, layer))) return rc;
     {
         Prof pf(S, 1, 0.0);
-        k_rmsnorm<T><<<rows, 256, 0, S->stream>>>(S->c, (const T *)w.ffn_norm, layer, S->c.xn, ldx);
+        CKL(launch_overlapped(S->stream, k_rmsnorm<T>, rows, 256, 0, S->c, (const T *)w.ffn_norm, layer, S->c.xn, ldx));
     }
     CK(cudaGetLastError());
     S->launches++;
@@ -543,7 +550,7 @@ int run_layer_t(ada_session *S, int layer, int rows) {
     }
     {
         Prof pf(S, 7, 0.0);
-        k_swiglu<<<dim3((g.d_ff + 255) / 256, rows), 256, 0, S->stream>>>(S->c, layer);
+        CKL(launch_overlapped(S->stream, k_swiglu, dim3((g.d_ff + 255) / 256, rows), 256, 0, S->c, layer));
     }
     CK(cudaGetLastError());
     S->launches++;
@@ -561,7 +568,7 @@ int run_head_t(ada_session *S, int layer1, int sel, int rows) {
     int rc;
     {
         Prof pf(S, 1, 0.0);
-        k_rmsnorm<T><<<rows, 256, 0, S->stream>>>(S->c, (const T *)m->final_norm, sel, S->c.xn, d);
+        CKL(launch_overlapped(S->stream, k_rmsnorm<T>, rows, 256, 0, S->c, (const T *)m->final_norm, sel, S->c.xn, d));
     }
     CK(cudaGetLastError());
     S->launches++;
@@ -577,9 +584,9 @@ int run_head_t(ada_session *S, int layer1, int sel, int rows) {
     const int store = (layer1 == 0 && S->capture_dev) ? 1 : 0;
     {
         Prof pf(S, 9, (double)g.vocab * d * sizeof(T));
-        k_head_partial<T><<<S->head_blocks, 256, 0, S->stream>>>(S->c, (const T *)m->lm_head, x, d, scale, sel, store);
+        CKL(launch_overlapped(S->stream, k_head_partial<T>, S->head_blocks, 256, 0, S->c, (const T *)m->lm_head, x, d, scale, sel, store));
         CK(cudaGetLastError());
-        k_head_final<<<rows, 32, 0, S->stream>>>(S->c, S->head_blocks, sel);
+        CKL(launch_overlapped(S->stream, k_head_final, rows, 32, 0, S->c, S->head_blocks, sel));
     }
     CK(cudaGetLastError());
     S->launches += 2;
@@ -597,9 +604,9 @@ int step_begin(ada_session *S) {
     const ada_model *m = S->m;
     Prof pf(S, 0, 0.0);
     if (m->cfg.dtype == ADA_DTYPE_BF16)
-        k_step_begin<__nv_bfloat16><<<1, 256, 0, S->stream>>>(S->c, (const __nv_bfloat16 *)m->tok_embed, m->cfg.rope_base);
+        CKL(launch_overlapped(S->stream, k_step_begin<__nv_bfloat16>, 1, 256, 0, S->c, (const __nv_bfloat16 *)m->tok_embed, m->cfg.rope_base));
     else
-        k_step_begin<float><<<1, 256, 0, S->stream>>>(S->c, (const float *)m->tok_embed, m->cfg.rope_base);
+        CKL(launch_overlapped(S->stream, k_step_begin<float>, 1, 256, 0, S->c, (const float *)m->tok_embed, m->cfg.rope_base));
     CK(cudaGetLastError());
     S->launches++;
     return ADA_OK;
@@ -608,9 +615,9 @@ int step_begin(ada_session *S) {
 int capture_rows(ada_session *S, int row0) {
     if (!S->capture_dev) return ADA_OK;
     Prof pf(S, 11, 0.0);
-    k_capture<<<64, 256, 0, S->stream>>>(S->c, row0);
+    CKL(launch_overlapped(S->stream, k_capture, 64, 256, 0, S->c, row0));
     CK(cudaGetLastError());
-    k_capture_advance<<<1, 32, 0, S->stream>>>(S->c);
+    CKL(launch_overlapped(S->stream, k_capture_advance, 1, 32, 0, S->c));
     CK(cudaGetLastError());
     S->launches += 2;
     return ADA_OK;
@@ -928,7 +935,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
             if ((rc = run_head(S, 0, SEL_FINAL, rows))) return rc;
             {
                 Prof pf(S, 0, 0.0);
-                k_verify<<<1, 32, 0, S->stream>>>(S->c);
+                CKL(launch_overlapped(S->stream, k_verify, 1, 32, 0, S->c));
             }
             CK(cudaGetLastError());
             S->launches++;
@@ -950,7 +957,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
                     if ((rc = run_head(S, l + 1, SEL_HEAD, rows))) return rc;
                     {
                         Prof pf(S, 0, 0.0);
-                        k_exit_control<<<1, 32, 0, S->stream>>>(S->c, l + 1);
+                        CKL(launch_overlapped(S->stream, k_exit_control, 1, 32, 0, S->c, l + 1));
                     }
                     CK(cudaGetLastError());
                     S->launches++;
@@ -963,7 +970,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
                 if ((rc = run_head(S, 0, SEL_FINAL, rows))) return rc;
                 {
                     Prof pf(S, 0, 0.0);
-                    k_verify<<<1, 32, 0, S->stream>>>(S->c);
+                    CKL(launch_overlapped(S->stream, k_verify, 1, 32, 0, S->c));
                 }
                 CK(cudaGetLastError());
                 S->launches++;
@@ -1374,8 +1381,10 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         int32_t zero = 0;
         CK(cudaMemcpyAsync(&S->c.st->capture_n, &zero, sizeof(int32_t), cudaMemcpyHostToDevice, S->stream));
     }
-    // Prompts of some length take the dense pass: blocks of up to dg::PF_ROWS positions through the tcgen05 products.
-    const bool dense = S->dense_ok && S->prefill_dense && n_prompt >= 32;
+    // Prompts of some length take the dense pass: blocks of up to dg::PF_ROWS positions through the tcgen05 products.  The
+    // decode path takes eight positions a pass; measured, 16 / 17 prompt tokens: 1B 1.99 / 2.82 against 2.21 ms dense, 8B 6.8 /
+    // 9.8 against 7.3, 13B 10.7 / 15.9 against 11.1: three passes cost more than the dense one, two less.
+    const bool dense = S->dense_ok && S->prefill_dense && n_prompt >= kDenseMin;
     if (!dense && S->mega && S->path == 1) {
         // prompt passes of eight positions through the persistent kernel
         mg::k_prefill_arm<<<1, 32, 0, S->stream>>>(S->c, seq, n_prompt);

@@ -66,13 +66,6 @@ constexpr size_t DSMEM_BYTES = sizeof(DSmem) + 1024;
 static_assert(STAGE_BYTES % 1024 == 0 && A_BYTES % 1024 == 0, "operand tiles must start on 1024-byte boundaries");
 static_assert(DSMEM_BYTES <= 232448, "exceeds the 227 KB of shared memory a block may use");
 
-// Programmatic dependent launch: the kernels of a layer follow one another in the stream, each allowed to start (launch,
-// barriers, tensor memory, first weight tiles) while the one before it drains.  Nothing that an earlier kernel writes, and
-// nothing that an earlier kernel may still read, is touched before pdl_wait(), which returns when all of them are complete.
-// Every CTA passes pdl_wait(), so "the kernel before me is complete" carries over to all kernels before it.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -632,12 +625,11 @@ __global__ void k_pf_last(Ctx c, const float *__restrict__ resid, int row, int s
 
 // RMSNorm and split in one pass: x = resid[r] / sqrt(mean(resid[r]^2) + eps) * g -> high and low parts.  One CTA
 // (256 threads) per row, four elements per access; K a multiple of 64.
-__global__ void __launch_bounds__(256) k_norm_split_rows(const float *__restrict__ X, int K, const __nv_bfloat16 *__restrict__ gain,
-                                                         float eps, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+__global__ void __launch_bounds__(256) k_norm_split_rows(const float *X, int K, const __nv_bfloat16 *__restrict__ gain,
+                                                         float eps, __nv_bfloat16 *hi, __nv_bfloat16 *lo) {
     const int r = blockIdx.x;
     __shared__ float red[8];
-    pdl_trigger();
-    pdl_wait();
+    pdl_begin();
     const float4 *x = reinterpret_cast<const float4 *>(X + (size_t)r * K);
     float ss = 0.f;
     for (int i = threadIdx.x; i < K / 4; i += 256) {
@@ -760,8 +752,8 @@ __device__ __forceinline__ void tma_tile_3d(void *dst, const CUtensorMap *map, i
 template <int HD, int GROUP>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CUtensorMap mapQlo, const __grid_constant__ CUtensorMap mapKV,
-          const __grid_constant__ Ctx c, int layer, int rows, int seq, int pos0, int kv_box, __nv_bfloat16 *__restrict__ ohi,
-          __nv_bfloat16 *__restrict__ olo, int *err) {
+          const __grid_constant__ Ctx c, int layer, int rows, int seq, int pos0, int kv_box, __nv_bfloat16 *ohi,
+          __nv_bfloat16 *olo, int *err) {
     typedef AtSmem<HD> Sm;
     constexpr int PT = AT_Q / GROUP, SLOTS = Sm::SLOTS, HG = HD / 64;
     extern __shared__ unsigned char dsm_raw[];

@@ -46,9 +46,20 @@ struct Ctx {
 
 // ------------------------------------------------------------------ small helpers
 
+// Programmatic dependent launch: kernels that follow one another in the stream, each allowed to start (launch, and whatever
+// it can set up by itself) while the one before it drains.  Nothing that an earlier kernel writes, and nothing that an
+// earlier kernel may still read, is touched before pdl_wait(), which returns when all of them are complete.  Every CTA
+// passes pdl_wait(), so "the kernel before me is complete" carries over to all kernels before it.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() { pdl_trigger(); pdl_wait(); }
+
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {
     static constexpr int E = 4;
+    static __device__ __forceinline__ void unpack(const uint4 &v, float (&o)[4]) {
+        o[0] = __uint_as_float(v.x); o[1] = __uint_as_float(v.y); o[2] = __uint_as_float(v.z); o[3] = __uint_as_float(v.w);
+    }
     static __device__ __forceinline__ void load_stream(const float *p, float (&o)[4]) {
         float4 v = __ldcs(reinterpret_cast<const float4 *>(p));
         o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
@@ -159,6 +170,7 @@ __device__ void embed_row(const Ctx &c, const T *embed, float rope_base, int r, 
 // tokens and t_i with the layer at which each resumes (P[l] (+) t_i for every l at once).
 template <typename T>
 __global__ void k_step_begin(Ctx c, const T *embed, float rope_base) {
+    pdl_begin();
     DevState *st = c.st;
     RowTable *rt = c.rt;
     if (threadIdx.x == 0) {
@@ -229,6 +241,7 @@ __global__ void k_prefill_end(Ctx c, int seq, int pos_end, int last, int n_promp
 // out[r] = resid[r] / sqrt(mean(resid[r]^2) + eps) * g, one block per row.
 template <typename T>
 __global__ void __launch_bounds__(256) k_rmsnorm(Ctx c, const T *gain, int sel, float *out, int ldo) {
+    pdl_begin();
     int r = blockIdx.x;
     if (!selected(c, r, sel)) return;
     const float *x = c.resid + (size_t)r * c.d;
@@ -252,8 +265,9 @@ __global__ void __launch_bounds__(256) k_rmsnorm(Ctx c, const T *gain, int sel, 
 // then a shuffle tree), so a row's result does not depend on the other rows.
 // EPI 0: store to Y.  EPI 1: Y[r][n] += result (residual add; each (r, n) has one writer).
 template <typename T, int EPI>
-__global__ void __launch_bounds__(256) k_gemv(Ctx c, const T *__restrict__ W, int N, int K, const float *__restrict__ X,
-                                              int ldx, float *__restrict__ Y, int ldy, int sel) {
+__global__ void __launch_bounds__(256) k_gemv(Ctx c, const T *__restrict__ W, int N, int K, const float *X,
+                                              int ldx, float *Y, int ldy, int sel) {
+    pdl_begin();
     __shared__ int rows[kMaxRows];
     __shared__ int nr_sh;
     const int nr = build_row_list(c, sel, rows, &nr_sh);
@@ -316,6 +330,7 @@ __global__ void __launch_bounds__(256) k_gemv(Ctx c, const T *__restrict__ W, in
 // position (Algorithm 1: "update KV cache at layer l").  One block per row.
 template <typename T>
 __global__ void k_rope_kv(Ctx c, int layer) {
+    pdl_begin();
     int r = blockIdx.x;
     if (!selected(c, r, layer)) return;
     const int half = c.hd / 2, seq = c.rt->seq[r], pos = c.rt->pos[r];
@@ -353,6 +368,7 @@ __global__ void k_rope_kv(Ctx c, int layer) {
 // do not depend on the context length or on other rows.  One warp per block; lane holds hd/32 dims.
 template <typename T, int EPL>
 __global__ void __launch_bounds__(32) k_attn_partial(Ctx c, int layer) {
+    pdl_begin();
     const int r = blockIdx.z;
     if (!selected(c, r, layer)) return;
     const int pos = c.rt->pos[r], seq = c.rt->seq[r];
@@ -366,22 +382,43 @@ __global__ void __launch_bounds__(32) k_attn_partial(Ctx c, int layer) {
 #pragma unroll
     for (int e = 0; e < EPL; ++e) { qv[e] = c.q[((size_t)r * c.nq + h) * c.hd + lane * EPL + e]; acc[e] = 0.f; }
     float m = -INFINITY, l = 0.f;
-    for (int t = t0; t <= t1; ++t) {
-        const T *kp = pool + kv_index(c, seq, layer, 0, kvh, t);
-        const T *vp = pool + kv_index(c, seq, layer, 1, kvh, t);
-        float dot = 0.f, vv[EPL];
+    // Eight positions (of one cache page) at a time: their loads, dot products and exponentials are independent; one after
+    // the other each position was a chain of two loads, a shuffle tree and an exponential (some 200 ns a position).
+    for (int t8 = t0; t8 <= t1; t8 += 8) {
+        const T *kp = pool + kv_index(c, seq, layer, 0, kvh, t8), *vp = pool + kv_index(c, seq, layer, 1, kvh, t8);
+        float sc[8], vv[8][EPL];
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) {
-            const int j = kv_swz(c, lane * EPL + e, t);
-            dot = fmaf(qv[e], to_f<T>(kp[j]), dot);
-            vv[e] = to_f<T>(vp[j]);
+        for (int u = 0; u < 8; ++u) {
+            const bool in = t8 + u <= t1;
+            sc[u] = 0.f;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) {
+                const int j = u * c.hd + kv_swz(c, lane * EPL + e, t8 + u);
+                sc[u] = in ? fmaf(qv[e], to_f<T>(kp[j]), sc[u]) : 0.f;
+                vv[u][e] = in ? to_f<T>(vp[j]) : 0.f;
+            }
         }
-        float sc = warp_sum(dot) * scale;
-        float mn = fmaxf(m, sc);
-        float corr = expf(m - mn), p = expf(sc - mn);
-        l = l * corr + p;
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) acc[e] = acc[e] * corr + p * vv[e];
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sc[u] += __shfl_xor_sync(0xffffffffu, sc[u], o);
+        float mn = m;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            sc[u] = t8 + u <= t1 ? sc[u] * scale : -INFINITY;
+            mn = fmaxf(mn, sc[u]);
+        }
+        const float corr = expf(m - mn);
+        l *= corr;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[e] *= corr;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float p = expf(sc[u] - mn);
+            l += p;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) acc[e] = fmaf(p, vv[u][e], acc[e]);
+        }
         m = mn;
     }
     float *out = c.attn_part + (((size_t)r * c.nq + h) * c.n_chunks + chunk) * (c.hd + 2);
@@ -392,6 +429,7 @@ __global__ void __launch_bounds__(32) k_attn_partial(Ctx c, int layer) {
 
 // Merge the chunk partials of one (row, head) in ascending chunk order; write attn_out.
 __global__ void k_attn_combine(Ctx c, int layer) {
+    pdl_begin();
     const int r = blockIdx.y, h = blockIdx.x;
     if (!selected(c, r, layer)) return;
     const int nch = c.rt->pos[r] / kAttnChunk + 1;
@@ -411,6 +449,7 @@ __global__ void k_attn_combine(Ctx c, int layer) {
 // ------------------------------------------------------------------ SwiGLU
 
 __global__ void k_swiglu(Ctx c, int layer) {
+    pdl_begin();
     const int r = blockIdx.y;
     if (!selected(c, r, layer)) return;
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -435,8 +474,9 @@ __device__ __forceinline__ Msa msa_merge(Msa a, Msa b) {
 // Logits z[r][v] = scale * E[v] . x[r] for the selected rows, reduced on the fly to per-block
 // (max, sum exp(z - max), argmax); logits go to memory only when logit_stage is set (tests).
 template <typename T>
-__global__ void __launch_bounds__(256) k_head_partial(Ctx c, const T *__restrict__ E, const float *__restrict__ X, int ldx,
+__global__ void __launch_bounds__(256) k_head_partial(Ctx c, const T *__restrict__ E, const float *X, int ldx,
                                                       float scale, int sel, int store_logits) {
+    pdl_begin();
     __shared__ int rows[kMaxRows];
     __shared__ int nr_sh;
     __shared__ Msa red[8][8];
@@ -452,6 +492,47 @@ __global__ void __launch_bounds__(256) k_head_partial(Ctx c, const T *__restrict
         Msa run[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) { run[j].m = -INFINITY; run[j].s = 0.f; run[j].i = INT_MAX; }
+        if (cnt == 1) {
+            // One row (every prompt's head, and plain decoding): four vocabulary entries at a time, eight 16-byte loads in flight
+            // per lane and each piece of x read once for the four.  Per entry the order of the sum is that of the general loop.
+            const float *x = X + (size_t)rows[g0] * ldx;
+            for (int n0 = warp; n0 < N; n0 += 4 * nwarps) {
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int c0 = lane; c0 < nch; c0 += 64) {
+                    uint4 w[2][4];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int n = n0 + q * nwarps, cc = c0 + 32 * u;
+                            w[u][q] = n < N && cc < nch ? __ldcs(reinterpret_cast<const uint4 *>(E + (size_t)n * K) + cc) : make_uint4(0, 0, 0, 0);
+                        }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int cc = c0 + 32 * u;
+                        if (cc >= nch) continue;
+                        float xv[EV];
+                        load_x<EV>(x + (size_t)cc * EV, xv);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            float wv[EV];
+                            Vec16<T>::unpack(w[u][q], wv);
+#pragma unroll
+                            for (int e = 0; e < EV; ++e) acc[q] = fmaf(wv[e], xv[e], acc[q]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int n = n0 + q * nwarps;
+                    if (n >= N) break;
+                    const float z = warp_sum(acc[q]) * scale;
+                    if (store_logits && lane == 0) c.logit_stage[(size_t)rows[g0] * N + n] = z;
+                    Msa one; one.m = z; one.s = 1.f; one.i = n;
+                    run[0] = msa_merge(run[0], one);
+                }
+            }
+        } else
         for (int n = warp; n < N; n += nwarps) {
             const T *wrow = E + (size_t)n * K;
             float acc[8];
@@ -508,6 +589,7 @@ __global__ void __launch_bounds__(256) k_head_partial(Ctx c, const T *__restrict
 // l + 32, ..., then the lanes are folded by a butterfly; the order depends on the number of blocks alone.  (One thread
 // merging the 592 blocks one after the other was a chain of as many dependent loads: 300 us on a cold L2, 130 us warm.)
 __global__ void k_head_final(Ctx c, int n_blocks, int sel) {
+    pdl_begin();
     const int r = blockIdx.x, lane = threadIdx.x;
     if (!selected(c, r, sel)) return;
     Msa a; a.m = -INFINITY; a.s = 0.f; a.i = INT_MAX;
@@ -548,6 +630,7 @@ __device__ __forceinline__ void mark_idle(const Ctx &c, int s) {
 // sequence (tentatively), the newest token stays in flight at depth e, and the sequence stops
 // climbing for this step.
 __global__ void k_exit_control(Ctx c, int e) {
+    pdl_begin();
     DevState *st = c.st;
     if (threadIdx.x == 0) {
         int nclimb = 0;
@@ -594,6 +677,7 @@ __global__ void k_exit_control(Ctx c, int e) {
 // base+j+1.  First mismatch: the token is replaced by a_j, the sequence is cut after it and every
 // layer's fill level drops to its position.  No mismatch: a_last is appended.
 __global__ void k_verify(Ctx c) {
+    pdl_begin();
     DevState *st = c.st;
     if (threadIdx.x != 0) return;
     int ndone = 0;
@@ -654,6 +738,7 @@ __global__ void k_verify(Ctx c) {
 
 // Copy the kept rows' staged final logits of sequence 0 into the capture buffer.
 __global__ void k_capture(Ctx c, int row0) {
+    pdl_begin();
     DevState *st = c.st;
     const int keep = st->keep_rows, at = st->capture_n;
     for (int j = 0; j < keep; ++j) {
@@ -664,6 +749,7 @@ __global__ void k_capture(Ctx c, int row0) {
     }
 }
 __global__ void k_capture_advance(Ctx c) {
+    pdl_begin();
     if (threadIdx.x == 0 && blockIdx.x == 0) c.st->capture_n += c.st->keep_rows;
 }
 
