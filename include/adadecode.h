@@ -140,7 +140,7 @@ void ada_session_destroy(ada_session *s);
 int ada_session_reset(ada_session *s, int32_t seq);
 
 /* KV cache <- LM(x) (first line of Algorithm 1): runs the n_prompt tokens of sequence `seq`
- * through all layers (prompts of 17 tokens or more in dense blocks of up to 2048 positions, see ada_debug_set_prefill).  The first generated token (full-depth argmax at the last prompt token)
+ * through all layers (prompts of 9 tokens or more in dense blocks of up to 2048 positions, see ada_debug_set_prefill).  The first generated token (full-depth argmax at the last prompt token)
  * becomes the sequence's pending token.  ADA_ECAPACITY if pages or max_seq_len do not suffice. */
 int ada_prefill(ada_session *s, int32_t seq, const int32_t *prompt_host, int32_t n_prompt);
 
@@ -219,7 +219,7 @@ int ada_debug_profile_read(ada_session *s, double *ms_out, int64_t *launches_out
  * ada_stats.path reports the path a decode call ran on. */
 int ada_debug_set_path(ada_session *s, int32_t path);
 int ada_debug_get_path(ada_session *s, int32_t *path_out);
-/* How ada_prefill runs prompts of 17 tokens or more.  1 (the default wherever it is available: bf16 models of
+/* How ada_prefill runs prompts of 9 tokens or more.  1 (the default wherever it is available: bf16 models of
  * the shapes the persistent kernel takes, on sm_100): the dense pass, equal blocks of at most 2048 positions, every
  * weight matrix streamed once per block through a tcgen05 GEMM with its accumulators in tensor memory.  0: through
  * the decode path itself (passes of eight positions in the persistent kernel, or one kernel per operation).

@@ -177,7 +177,7 @@ struct ada_session {
     __nv_bfloat16 *pf_x = nullptr, *pf_u = nullptr;   // high and low parts of a product's input: model width; queries, attention result / FFN activations
     unsigned *pf_flag = nullptr;
     int *pf_err = nullptr;
-    std::vector<CUtensorMap> pf_maps;          // [L][7]: wq, wk, wv, wo, w_gate, w_up, w_down
+    std::vector<CUtensorMap> pf_maps;          // [L][5]: wqkv (reordered copy), wo, w_gate, w_up, w_down
     CUtensorMap pf_kv;                         // the page pool
     int pf_kv_box = 0;                         // positions one copy of it covers
     bool prefill_dense = true;                 // ada_debug_set_prefill
@@ -214,8 +214,8 @@ int rows_alloc_for(const ada_config &g, int batch, int max_early) {
     return std::max(batch * (max_early + 1), model_fits_persistent(g) ? 64 : 32);
 }
 // positions of one block of a dense prompt pass: a prompt is cut alike whatever the session's length limit
-int pf_rows_for(int max_seq) { return std::min(dg::PF_ROWS, (int)align_up((size_t)max_seq, dg::BM)); }
-constexpr int kDenseMin = 17;       // prompt tokens from which the dense pass is taken
+int pf_rows_for(int max_seq) { return std::min(dg::PF_ROWS, (int)align_up((size_t)max_seq, 128)); }
+constexpr int kDenseMin = 9;        // prompt tokens from which the dense pass is taken
 constexpr int kGemmMaxPairs = 80;   // CTA pairs the exchange area of cut tiles is laid out for
 
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
@@ -354,15 +354,23 @@ int launch_overlapped(cudaStream_t stream, void (*kernel)(P...), dim3 grid, int 
 
 // ---- dense prompt pass: one decoder layer over a block of up to dg::PF_ROWS prompt positions --------------------
 
-// How a product of `nt` tile columns and depth K over `rows` positions is divided over at most `pairs` CTA pairs.  More
-// tiles than pairs: whole waves, then one wave's worth of tiles and the remainder cut by chunks so that all pairs end
-// together (cutting the remainder alone would cut a tile into more pieces, each of which costs an exchange).  Fewer:
-// all tiles cut over the number of pairs that minimises chunks of the busiest pair (8192 tensor-core cycles each) plus
-// the reading of a tile's other pieces by its last pair (128 KB per CTA, measured at some 3300 cycles).
-dg::GemmPlan plan_dense(int rows, int nt, int K, int pairs) {
+// Positions per tile of a product over `rows` positions: equal tiles, in steps of 32.
+int position_tile(int rows) {
+    const int mt = (rows + dg::NT_MAX - 1) / dg::NT_MAX, per = (rows + mt - 1) / mt;
+    return (per + 31) / 32 * 32;
+}
+
+// How a product of N weight rows (`per_tile` of them to a tile) and depth K over `rows` positions is divided over at most
+// `pairs` CTA pairs.  More tiles than pairs: whole waves, then one wave's worth of tiles and the remainder cut by
+// chunks so that all pairs end together (cutting the remainder alone would cut a tile into more pieces, each of which
+// costs an exchange).  Fewer: all tiles cut over the number of pairs that minimises, in cycles, the chunks of the busiest
+// pair (8192 of the tensor core at full width; not below the 5600 that a chunk's weights take to arrive at a pair's share
+// of HBM bandwidth) plus the exchange of the pieces (3300 cycles per further piece of full width, 3000 to begin with).
+dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
     dg::GemmPlan g{};
-    g.mt = (rows + dg::TM - 1) / dg::TM;
-    g.tiles = g.mt * nt;
+    g.nt = position_tile(rows);
+    g.mt = (rows + g.nt - 1) / g.nt;
+    g.tiles = g.mt * ((N + per_tile - 1) / per_tile);
     g.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
     if (g.tiles >= pairs) {
         g.pairs = pairs;
@@ -370,11 +378,12 @@ dg::GemmPlan plan_dense(int rows, int nt, int K, int pairs) {
         return g;
     }
     const int units = g.tiles * g.chunks;
+    const double width = (double)g.nt / dg::NT_MAX, chunk = std::max(8192.0 * width, 5600.0);
     double best = 0;
     for (int p = g.tiles; p <= std::min(pairs, units); ++p) {
         const int per = units / p;
         const int pieces = p == g.tiles ? 0 : (g.chunks + per - 1) / per;
-        const double cost = 8192.0 * ((units + p - 1) / p) + 3300.0 * pieces * std::min(1.0, rows / (double)dg::BM) + (pieces ? 3000.0 : 0.0);
+        const double cost = chunk * ((units + p - 1) / p) + 3300.0 * pieces * width + (pieces ? 3000.0 : 0.0);
         if (!g.pairs || cost < best) { best = cost; g.pairs = p; }
     }
     g.sk_tiles = g.tiles;
@@ -383,15 +392,16 @@ dg::GemmPlan plan_dense(int rows, int nt, int K, int pairs) {
 }
 
 template <int EPI, int HD>
-int launch_dense(cudaStream_t stream, const CUtensorMap &xh, const CUtensorMap &xl, const CUtensorMap &w0, const CUtensorMap &w1,
-                 const CUtensorMap &w2, const Ctx &c, const dg::GemmArgs &a) {
-    return launch_overlapped(stream, dg::k_dense_gemm<EPI, HD>, 2 * a.plan.pairs, dg::GTHREADS, dg::DSMEM_BYTES, xh, xl, w0, w1, w2, c, a);
+int launch_dense(cudaStream_t stream, const CUtensorMap &xh, const CUtensorMap &xl, const CUtensorMap &w0, const CUtensorMap &w1, const Ctx &c,
+                 const dg::GemmArgs &a) {
+    return launch_overlapped(stream, dg::k_dense_gemm<EPI, HD>, 2 * a.plan.pairs, dg::GTHREADS, dg::DSMEM_BYTES, xh, xl, w0, w1, c, a);
 }
 template <int EPI, int HD> cudaError_t prepare_dense() {
     return cudaFuncSetAttribute(dg::k_dense_gemm<EPI, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::DSMEM_BYTES);
 }
 
-// Tensor maps of the inputs of a block's products (they end at the block's last row: rows behind it read as zero).
+// Tensor maps of the inputs of a block's products (they end at the block's last row: rows behind it read as zero): high and
+// low parts of the normalised residual, the queries, the attention result, the FFN activations.
 struct PfMaps { CUtensorMap xh, xl, qh, ql, oh, ol, hh, hl; };
 
 template <int HD, int GROUP>
@@ -408,29 +418,32 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     const ada_model *m = S->m;
     const ada_config &g = m->cfg;
     const LayerW &w = m->layers[layer];
-    const int d = g.d_model, hd = g.head_dim, qd = g.n_q_heads * hd, kvd = g.n_kv_heads * hd, group = g.n_q_heads / g.n_kv_heads;
-    const CUtensorMap *wm = &S->pf_maps[7 * (size_t)layer];
+    const int d = g.d_model, hd = g.head_dim, qd = g.n_q_heads * hd, group = g.n_q_heads / g.n_kv_heads, qkv = S->c.qkv_rows;
+    const CUtensorMap *wm = &S->pf_maps[5 * (size_t)layer];
     const size_t P = pf_rows_for(S->max_seq);
     __nv_bfloat16 *xh = S->pf_x, *xl = xh + P * d, *qh = S->pf_u, *ql = qh + P * qd, *oh = ql + P * qd, *ol = oh + P * qd, *hh = S->pf_u, *hl = hh + P * g.d_ff;
     typedef __nv_bfloat16 T;
     int rc;
     dg::GemmArgs a{};
     a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err;
+    a.Y = S->pf_resid; a.ldy = d;
     S->layer_passes++;
     S->launches += 7;
     auto norm = [&](const void *gain) {
         Prof pf(S, 1, 0.0);
         return launch_overlapped(S->stream, dg::k_norm_split_rows, rows, 256, 0, S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl);
     };
+    auto shape = [&](int N, int per_tile, int K) {
+        a.N = N; a.K = K; a.epoch = ++S->pf_epoch;
+        a.plan = plan_dense(rows, N, per_tile, K, S->pf_pairs);
+    };
     if ((rc = norm(w.attn_norm))) return rc;
     {
-        Prof pf(S, 2, (double)(qd + 2 * kvd) * d * 2);
-        a.nw[0] = qd; a.nw[1] = a.nw[2] = kvd;
-        a.nt[0] = (qd + dg::TN - 1) / dg::TN; a.nt[1] = a.nt[2] = (kvd + dg::TN - 1) / dg::TN;
-        a.K = d; a.hi = qh; a.lo = ql; a.epoch = ++S->pf_epoch;
-        a.plan = plan_dense(rows, a.nt[0] + a.nt[1] + a.nt[2], d, S->pf_pairs);
-        rc = hd == 128 ? launch_dense<dg::EPI_QKV, 128>(S->stream, pm.xh, pm.xl, wm[0], wm[1], wm[2], S->c, a)
-                       : launch_dense<dg::EPI_QKV, 64>(S->stream, pm.xh, pm.xl, wm[0], wm[1], wm[2], S->c, a);
+        Prof pf(S, 2, (double)qkv * d * 2);
+        shape(qkv, dg::TW, d);
+        a.hi = qh; a.lo = ql;
+        rc = hd == 128 ? launch_dense<dg::EPI_QKV, 128>(S->stream, pm.xh, pm.xl, wm[0], wm[0], S->c, a)
+                       : launch_dense<dg::EPI_QKV, 64>(S->stream, pm.xh, pm.xl, wm[0], wm[0], S->c, a);
         if (rc) return rc;
     }
     {
@@ -441,27 +454,22 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
                 : group == 2 ? launch_attn_dense<64, 2>(S, pm, layer, seq, pos0, rows, oh, ol) : launch_attn_dense<64, 1>(S, pm, layer, seq, pos0, rows, oh, ol);
         if (rc) return rc;
     }
-    a.nt[0] = (d + dg::TN - 1) / dg::TN;
-    a.nt[1] = a.nt[2] = 0;
-    a.Y = S->pf_resid; a.ldy = d;
     {
         Prof pf(S, 5, (double)d * qd * 2);
-        a.nw[0] = d; a.K = qd; a.epoch = ++S->pf_epoch;
-        a.plan = plan_dense(rows, a.nt[0], qd, S->pf_pairs);
-        if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.oh, pm.ol, wm[3], wm[3], wm[3], S->c, a))) return rc;
+        shape(d, dg::TW, qd);
+        if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.oh, pm.ol, wm[1], wm[1], S->c, a))) return rc;
     }
     if ((rc = norm(w.ffn_norm))) return rc;
     {
         Prof pf(S, 6, (double)2 * g.d_ff * d * 2);
-        a.nw[0] = a.nw[1] = g.d_ff; a.K = d; a.hi = hh; a.lo = hl; a.epoch = ++S->pf_epoch;
-        a.plan = plan_dense(rows, (g.d_ff + dg::BNH - 1) / dg::BNH, d, S->pf_pairs);
-        if ((rc = launch_dense<dg::EPI_SWIGLU, 0>(S->stream, pm.xh, pm.xl, wm[4], wm[5], wm[5], S->c, a))) return rc;
+        shape(g.d_ff, dg::BW, d);
+        a.hi = hh; a.lo = hl;
+        if ((rc = launch_dense<dg::EPI_SWIGLU, 0>(S->stream, pm.xh, pm.xl, wm[2], wm[3], S->c, a))) return rc;
     }
     {
         Prof pf(S, 8, (double)d * g.d_ff * 2);
-        a.nw[0] = d; a.K = g.d_ff; a.epoch = ++S->pf_epoch;
-        a.plan = plan_dense(rows, a.nt[0], g.d_ff, S->pf_pairs);
-        if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.hh, pm.hl, wm[6], wm[6], wm[6], S->c, a))) return rc;
+        shape(d, dg::TW, g.d_ff);
+        if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.hh, pm.hl, wm[4], wm[4], S->c, a))) return rc;
     }
     return ADA_OK;
 }
@@ -638,10 +646,12 @@ int prefill_dense(ada_session *S, int seq, int n_prompt) {
         PfMaps pm;
         const int group = g.n_q_heads / g.n_kv_heads;
         if (group != 1 && group != 2 && group != 4) return ADA_EUNSUPPORTED;
+        // a product's position tiles are the same for every layer; one box is what one CTA of a pair holds of a tile
+        const int bx = position_tile(n) / 2;
         if ((rc = make_map_q(&pm.qh, S->pf_u, n, g.n_q_heads, g.head_dim, group)) || (rc = make_map_q(&pm.ql, S->pf_u + P * qd, n, g.n_q_heads, g.head_dim, group)) ||
-            (rc = make_map_2d(&pm.xh, S->pf_x, n, d, dg::BM)) || (rc = make_map_2d(&pm.xl, S->pf_x + P * d, n, d, dg::BM)) ||
-            (rc = make_map_2d(&pm.oh, oh, n, qd, dg::BM)) || (rc = make_map_2d(&pm.ol, oh + P * qd, n, qd, dg::BM)) ||
-            (rc = make_map_2d(&pm.hh, hh, n, g.d_ff, dg::BM)) || (rc = make_map_2d(&pm.hl, hh + P * g.d_ff, n, g.d_ff, dg::BM)))
+            (rc = make_map_2d(&pm.xh, S->pf_x, n, d, bx)) || (rc = make_map_2d(&pm.xl, S->pf_x + P * d, n, d, bx)) ||
+            (rc = make_map_2d(&pm.oh, oh, n, qd, bx)) || (rc = make_map_2d(&pm.ol, oh + P * qd, n, qd, bx)) ||
+            (rc = make_map_2d(&pm.hh, hh, n, g.d_ff, bx)) || (rc = make_map_2d(&pm.hl, hh + P * g.d_ff, n, g.d_ff, bx)))
             return rc;
         dg::k_pf_embed<<<n, 256, 0, S->stream>>>(S->c, (const __nv_bfloat16 *)m->tok_embed, g.rope_base, seq, p0, S->pf_resid, S->pf_cs);
         CK(cudaGetLastError());
@@ -1306,21 +1316,17 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
             S->pf_err = (int *)(b + lay.pf_err);
             S->pf_flag = (unsigned *)(b + lay.pf_flag);
             S->pf_part = (float *)(b + lay.pf_part);
-            const int d = g.d_model, qd = g.n_q_heads * g.head_dim, kvd = g.n_kv_heads * g.head_dim;
+            const int d = g.d_model, qd = g.n_q_heads * g.head_dim;
             S->pf_kv_box = std::min(page_tokens, 64);
-            {
-                const int rc = make_map_kv(&S->pf_kv, kv_pool_dev, (size_t)n_pages * g.n_layers * 2 * g.n_kv_heads * page_tokens, g.head_dim, S->pf_kv_box);
-                if (rc) return fail(rc);
-            }
-            S->pf_maps.assign(7 * (size_t)g.n_layers, CUtensorMap());
+            int rc = make_map_kv(&S->pf_kv, kv_pool_dev, (size_t)n_pages * g.n_layers * 2 * g.n_kv_heads * page_tokens, g.head_dim, S->pf_kv_box);
+            if (rc) return fail(rc);
+            S->pf_maps.assign(5 * (size_t)g.n_layers, CUtensorMap());
             for (int l = 0; l < g.n_layers; ++l) {
                 const LayerW &w = m->layers[l];
-                CUtensorMap *wm = &S->pf_maps[7 * (size_t)l];
-                int rc;
-                if ((rc = make_map_2d(wm + 0, w.wq, qd, d, dg::BNH)) || (rc = make_map_2d(wm + 1, w.wk, kvd, d, dg::BNH)) ||
-                    (rc = make_map_2d(wm + 2, w.wv, kvd, d, dg::BNH)) || (rc = make_map_2d(wm + 3, w.wo, d, qd, dg::BNH)) ||
-                    (rc = make_map_2d(wm + 4, w.w_gate, g.d_ff, d, dg::BNH)) || (rc = make_map_2d(wm + 5, w.w_up, g.d_ff, d, dg::BNH)) ||
-                    (rc = make_map_2d(wm + 6, w.w_down, d, g.d_ff, dg::BNH)))
+                CUtensorMap *wm = &S->pf_maps[5 * (size_t)l];
+                if ((rc = make_map_2d(wm + 0, w.wqkv_perm, c.qkv_rows, d, dg::BW)) || (rc = make_map_2d(wm + 1, w.wo, d, qd, dg::BW)) ||
+                    (rc = make_map_2d(wm + 2, w.w_gate, g.d_ff, d, 16)) || (rc = make_map_2d(wm + 3, w.w_up, g.d_ff, d, 16)) ||
+                    (rc = make_map_2d(wm + 4, w.w_down, d, g.d_ff, dg::BW)))
                     return fail(rc);
             }
         } else cudaGetLastError();
@@ -1382,8 +1388,8 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         CK(cudaMemcpyAsync(&S->c.st->capture_n, &zero, sizeof(int32_t), cudaMemcpyHostToDevice, S->stream));
     }
     // Prompts of some length take the dense pass: blocks of up to dg::PF_ROWS positions through the tcgen05 products.  The
-    // decode path takes eight positions a pass; measured, 16 / 17 prompt tokens: 1B 1.99 / 2.82 against 2.21 ms dense, 8B 6.8 /
-    // 9.8 against 7.3, 13B 10.7 / 15.9 against 11.1: three passes cost more than the dense one, two less.
+    // decode path takes eight positions a pass; measured, one / two passes against the dense pass: 1B 1.06 / 1.96 against
+    // 1.69 ms, 8B 3.5 / 6.8 against 5.4, 13B 5.4 / 10.7 against 8.0.
     const bool dense = S->dense_ok && S->prefill_dense && n_prompt >= kDenseMin;
     if (!dense && S->mega && S->path == 1) {
         // prompt passes of eight positions through the persistent kernel
@@ -1657,14 +1663,16 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     return herr ? ADA_ETIMEOUT : ADA_OK;
 }
 
+constexpr int kDenseDebugRows = 128;   // most rows of ada_debug_dense_gemm
+
 size_t ada_debug_dense_gemm_work_bytes(int32_t K) {
     if (K < 64) return 0;
-    return 2 * (size_t)dg::BM * K * sizeof(__nv_bfloat16) + 256;
+    return 2 * (size_t)kDenseDebugRows * K * sizeof(__nv_bfloat16) + 256;
 }
 
 int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X_dev, int32_t rows, float *Y_dev, int32_t ldy,
                          int32_t accumulate, void *work_dev, size_t work_bytes, void *cuda_stream) {
-    if (!W_dev || !X_dev || !Y_dev || !work_dev || N < 1 || K < 64 || K % 64 || rows < 1 || rows > dg::BM || ldy < N) return ADA_EINVAL;
+    if (!W_dev || !X_dev || !Y_dev || !work_dev || N < 1 || K < 64 || K % 64 || rows < 1 || rows > kDenseDebugRows || ldy < N) return ADA_EINVAL;
     if ((uintptr_t)W_dev % 16 || (uintptr_t)work_dev % 256 || (uintptr_t)Y_dev % 16 || ldy % 4) return ADA_EINVAL;
     if (work_bytes < ada_debug_dense_gemm_work_bytes(K)) return ADA_ECAPACITY;
     int dev = 0, major = 0;
@@ -1672,11 +1680,12 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
     if (major != 10) return ADA_EUNSUPPORTED;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    __nv_bfloat16 *hi = (__nv_bfloat16 *)work_dev, *lo = hi + (size_t)dg::BM * K;
-    int *err = (int *)(lo + (size_t)dg::BM * K);
+    __nv_bfloat16 *hi = (__nv_bfloat16 *)work_dev, *lo = hi + (size_t)kDenseDebugRows * K;
+    int *err = (int *)(lo + (size_t)kDenseDebugRows * K);
     CUtensorMap mhi, mlo, mw;
     int rc, sms = 0;
-    if ((rc = make_map_2d(&mhi, hi, rows, K, dg::BM)) || (rc = make_map_2d(&mlo, lo, rows, K, dg::BM)) || (rc = make_map_2d(&mw, W_dev, N, K, dg::BNH)))
+    const int nt = position_tile(rows);
+    if ((rc = make_map_2d(&mhi, hi, rows, K, nt / 2)) || (rc = make_map_2d(&mlo, lo, rows, K, nt / 2)) || (rc = make_map_2d(&mw, W_dev, N, K, dg::BW)))
         return rc;
     CK((prepare_dense<dg::EPI_STORE, 0>()));
     CK((prepare_dense<dg::EPI_ADD, 0>()));
@@ -1685,11 +1694,11 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     dg::k_split_rows<<<rows, 256, 0, stream>>>(X_dev, K, rows, K, hi, lo);
     CK(cudaGetLastError());
     dg::GemmArgs a{};
-    a.rows = rows; a.K = K; a.nw[0] = N; a.nt[0] = (N + dg::TN - 1) / dg::TN; a.Y = Y_dev; a.ldy = ldy; a.err = err;
-    a.plan.mt = 1; a.plan.tiles = a.nt[0]; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;   // whole tiles: no exchange area needed
-    a.plan.pairs = std::max(1, std::min(a.plan.tiles, sms / 2));
+    a.rows = rows; a.N = N; a.K = K; a.Y = Y_dev; a.ldy = ldy; a.err = err;
+    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = (N + dg::TW - 1) / dg::TW; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
+    a.plan.pairs = std::max(1, std::min(a.plan.tiles, sms / 2));   // whole tiles: no exchange area needed
     const Ctx none{};
-    rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, mw, none, a);
+    rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, none, a);
     if (rc) return rc;
     int herr = 0;
     CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream));

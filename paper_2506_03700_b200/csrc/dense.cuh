@@ -7,11 +7,14 @@
 // X arrives as two bf16 matrices, a high part and a low part (x = hi + lo, as everywhere in this library: fp32
 // activations lose nothing), both multiplied into the same fp32 accumulator: 4 m n k floating-point operations.
 //
-// What bounds it.  From about 128 positions up the tensor cores (the weights of a block are fetched once from
-// HBM and then from L2).  A pair of CTAs computes a tile of 256 positions x 256 weight rows: each CTA holds its
-// own 128 positions (hi and lo) and half of the weight rows, so a k block of 64 costs a CTA 48 KB of shared-memory
-// fill per 1024 tensor-core cycles.  One CTA per tile of 128 x 128 (the previous form) needed 48 KB per 512
-// cycles and 2.7 times the L2 traffic per weight byte, and was bound by that.
+// What bounds it.  Below about 128 positions the weights' way from HBM, above it the tensor cores and the L2 cache
+// together: the gate / up product of a 1024-position block keeps the tensor pipe 82 % busy while 10.9 TB/s move from L2 to
+// the SMs (ncu).  The weights are the 256-row operand of a pair of CTAs, the positions the other one, 32 to 256 wide in
+// steps of 32: a block is cut into equal position tiles, so that little is multiplied for padding (777 positions: 4 tiles
+// of 224; with positions as the 256-row operand a prompt of 45 positions cost as much as one of 256).  At full width a
+// k block of 64 costs a CTA 48 KB of shared-memory fill per 1024 tensor-core cycles; one CTA per tile of 128 x 128 needed
+// 48 KB per 512 cycles and 2.7 times the L2 traffic per weight byte.  Two accumulators of 128 positions (gate and up side
+// by side) were 15 % slower than one of 256: at that width the operands' way out of shared memory is the bound.
 //
 // Accumulation.  The tensor core adds into its fp32 accumulator with truncation, so the error of one accumulator
 // grows with the products added to it (1e-3 absolute at K = 14336 with sums of size 10).  A product is therefore cut
@@ -39,31 +42,33 @@ using namespace st;
 
 constexpr int PF_ROWS = 2048;  // prompt positions of one block: 32 layers of launches and ragged waves are paid once per
                                // block; activations of a block stay below the size of the L2 cache per product
-constexpr int BM = 128;        // positions one CTA of a pair holds (UMMA M = 256 over the pair)
-constexpr int BNH = 128;       // weight rows one CTA of a pair holds (UMMA N = 256)
-constexpr int TM = 2 * BM, TN = 2 * BNH;
+constexpr int BW = 128;        // weight rows one CTA of a pair holds (UMMA M = 256 over the pair)
+constexpr int TW = 2 * BW;
+constexpr int NT_MAX = 256;    // positions per tile, at most
 constexpr int BK = 64;         // k elements per stage: one 128-byte swizzle row
 constexpr int CK = 8;          // k blocks per accumulator chunk
-constexpr int STAGES = 4;
-constexpr int GEPI_WARPS = 8;  // epilogue warps: lane quadrant (warp % 4) x half of the tile's columns
+constexpr int MAX_STAGES = 12;
+constexpr int GEPI_WARPS = 8;  // epilogue warps: lane quadrant (warp % 4) x half of the tile's positions
 constexpr int GTHREADS = 128 + 32 * GEPI_WARPS;
 // The register file is divided per warpgroup at launch (168 a thread); the epilogue warps hold 128 sums each and take
-// what the first warpgroup (TMA, MMA, two idle warps) gives back: (56 + 224 + 224) x 128 = 168 x 384.
+// what the first warpgroup (TMA, MMA, two idle warps) gives back: (40 + 232 + 232) x 128 = 168 x 384.
 constexpr int GREGS_ISSUE = 40, GREGS_EPI = 232;
-constexpr int A_BYTES = BM * BK * 2, B_BYTES = BNH * BK * 2, STAGE_BYTES = 2 * A_BYTES + B_BYTES;
+constexpr int W_BYTES = BW * BK * 2;
+constexpr int RING_BYTES = 196608;
 constexpr int TMEM_COLS = 512; // two accumulator buffers of 256 fp32 columns
 constexpr unsigned long long DENSE_WAIT_NS = 2000000000ull;
 constexpr size_t GPART_WARP = 128 * 32 * sizeof(float);           // partial sums of one epilogue warp
 constexpr size_t GPART_CTA = GEPI_WARPS * GPART_WARP;
 
 struct DSmem {   // must start on a 1024-byte boundary (swizzle pattern)
-    alignas(1024) unsigned char stage[STAGES][STAGE_BYTES];   // [X.hi 128 x 64 | X.lo 128 x 64 | W 128 x 64], rows of 128 B
-    alignas(8) unsigned long long full[STAGES], empty[STAGES], acc_full[2], acc_empty[2];
+    // stages of [W 128 x 64 (SwiGLU: 16 rows of gate, 16 of up, ...) | X.hi NT / 2 x 64 | X.lo NT / 2 x 64], rows of 128 B: as many as fit
+    alignas(1024) unsigned char ring[RING_BYTES];
+    alignas(8) unsigned long long full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2];
+    alignas(16) float stash[GEPI_WARPS][32][32];   // per epilogue warp: 32 positions x its 32 weight rows
     uint32_t tmem_base;
     int abort;
 };
 constexpr size_t DSMEM_BYTES = sizeof(DSmem) + 1024;
-static_assert(STAGE_BYTES % 1024 == 0 && A_BYTES % 1024 == 0, "operand tiles must start on 1024-byte boundaries");
 static_assert(DSMEM_BYTES <= 232448, "exceeds the 227 KB of shared memory a block may use");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -102,12 +107,12 @@ __device__ __forceinline__ unsigned long long smem_desc(uint32_t saddr) {
 // both K-major (bits 15, 16 = 0), N / 8 in bits 17-22, M / 16 in bits 24-28.
 template <int M, int N> struct Idesc { static constexpr uint32_t v = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24); };
 
-__device__ __forceinline__ void umma_pair(uint32_t d_tmem, unsigned long long adesc, unsigned long long bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_pair(uint32_t d_tmem, unsigned long long adesc, unsigned long long bdesc, uint32_t id, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(Idesc<TM, TN>::v), "r"(accumulate)
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(id), "r"(accumulate)
         : "memory");
 }
 // The barrier at this offset of both CTAs is arrived on once every MMA issued so far by this thread has completed.
@@ -124,6 +129,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t addr) {
                    "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
                    "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
                    "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                  : "r"(addr)
                  : "memory");
 }
@@ -187,7 +200,7 @@ template <typename SM> __device__ __forceinline__ bool dwait(SM *sm, int *err, u
 // Division of one product's tiles over the CTA pairs (chosen on the host, plan_dense).  Tiles are numbered with the
 // position tile fastest, so that the pairs at work at one time share weight rows.  The last sk_tiles tiles are divided
 // by chunks over sk_pairs pairs, the others are dealt out whole.
-struct GemmPlan { int mt, tiles, chunks, pairs, sk_tiles, sk_pairs; };
+struct GemmPlan { int nt, mt, tiles, chunks, pairs, sk_tiles, sk_pairs; };   // nt positions per tile, mt position tiles
 
 struct Seg { int tile, c0, c1; };   // chunks [c0, c1) of a tile
 struct Sched {
@@ -255,10 +268,9 @@ struct Sched {
 constexpr int EPI_STORE = 0, EPI_ADD = 1, EPI_QKV = 2, EPI_SWIGLU = 3;
 struct GemmArgs {
     GemmPlan plan;
-    int rows, K;
-    int nw[3], nt[3];             // weight rows and tile columns of the up to three matrices (QKV: q, k, v; SwiGLU: gate, up)
+    int rows, N, K;               // positions, weight rows (SwiGLU: of one of the two matrices), depth
     float *Y; int ldy;            // STORE, ADD
-    __nv_bfloat16 *hi, *lo;       // QKV: scaled queries [rows][nw[0]]; SwiGLU: activations [rows][nw[0]]
+    __nv_bfloat16 *hi, *lo;       // QKV: scaled queries [rows][q features]; SwiGLU: activations [rows][N]
     const float *cs;              // QKV: cos, sin [rows][hd / 2][2]
     int layer, seq, pos0;         // QKV: rows are positions pos0 .. of sequence seq
     float *part;                  // partial sums of tiles cut between pairs
@@ -275,106 +287,138 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
-// Y[m][n] = or += acc (columns [n, n + 128) of row m; ldy a multiple of 4, N arbitrary).
-template <bool ADD> __device__ __forceinline__ void epi_rows(const float (&acc)[128], float *__restrict__ y, int left) {
+// Epilogues.  A lane holds one weight row and acc[j] its value for position m0 + j.  Thirty-two positions at a time go through
+// shared memory (x[position][weight row of the warp]), from where they are written in whole sectors.  What a round needs
+// from memory is loaded before anything is stored: the compiler cannot move a load over a store that might alias, and one
+// round trip to L2 per position made the QKV epilogue 40 us long.
+template <class Body> __device__ __forceinline__ void epi_rounds(const float (&acc)[128], float (*x)[32], int lane, int left, Body &&body) {
+#pragma unroll 1
+    for (int g = 0; 32 * g < left; ++g) {
+        __syncwarp();
 #pragma unroll
-    for (int j = 0; j < 128; j += 4) {
-        if (j + 4 <= left) {
-            float4 o = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
-            float4 *p = reinterpret_cast<float4 *>(y + j);
-            if (ADD) { const float4 r = *p; o.x += r.x; o.y += r.y; o.z += r.z; o.w += r.w; }
-            *p = o;
-        } else {
+        for (int k = 0; k < 4; ++k)
+            if (g == k) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (j + e < left) y[j + e] = (ADD ? y[j + e] : 0.f) + acc[j + e];
+                for (int j = 0; j < 32; ++j) x[j][lane] = acc[32 * k + j];
+            }
+        __syncwarp();
+        body(32 * g, min(32, left - 32 * g));
+    }
+}
+
+// Y[m][n] = or += x: four neighbouring n per lane, four positions per access.  N arbitrary, ldy a multiple of 4.
+template <bool ADD> __device__ __forceinline__ void epi_rows(const float (*x)[32], float *y, int ldy, int n_left, int lane, int left) {
+    const int n = 4 * (lane & 7);
+    y += n;
+    if (n + 4 <= n_left) {
+float4 r[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int j = 4 * i + (lane >> 3);
+            r[i] = *reinterpret_cast<const float4 *>(&x[j][n]);
+            if (ADD && j < left) {
+                const float4 o = *reinterpret_cast<const float4 *>(y + (size_t)j * ldy);
+                r[i].x += o.x; r[i].y += o.y; r[i].z += o.z; r[i].w += o.w;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int j = 4 * i + (lane >> 3);
+            if (j < left) *reinterpret_cast<float4 *>(y + (size_t)j * ldy) = r[i];
+        }
+    } else {
+        for (int j = lane >> 3; j < left; j += 4)
+            for (int e = 0; n + e < n_left; ++e) y[(size_t)j * ldy + e] = x[j][n + e] + (ADD ? y[(size_t)j * ldy + e] : 0.f);
+    }
+}
+
+// q, k and v: the weight rows come reordered (see k_repack_qkv), so that rows r and r + 8 of 16 are the partners of a rotation.
+// q and k are rotated, q is scaled and split into bf16 high and low parts, k and v go to the cache rows of the positions
+// (16-byte chunks xor-swizzled, see kv_swz).  n_w: first weight row of the warp; all 32 belong to one head.  A lane
+// computes one pair of partners for every second position and, with its neighbour, writes two neighbouring features.
+template <int HD> __device__ __forceinline__ void epi_qkv(const Ctx &c, const GemmArgs &a, const float (*x)[32], int n_w, int lane, int m0, int left) {
+    const int qd = c.nq * HD, kvd = c.nkv * HD;
+    const int which = n_w < qd ? 0 : n_w < qd + kvd ? 1 : 2;
+    const int nr = n_w - (which == 0 ? 0 : which == 1 ? qd : qd + kvd), head = nr / HD, r0 = nr % HD;   // first row within the head
+    const int l = lane & 15, row = (l >> 3) * 16 + (l & 7);          // the pair is rows `row` and `row` + 8 of the warp's 32
+    const bool odd = lane & 1;
+    const int jj = r0 / 2 + l;                                        // frequency of the pair
+    // features this lane writes: of the rotation's lower half (even lanes) or upper half (odd lanes); v rows are in order
+    const int fe = which < 2 ? (jj & ~1) + (odd ? HD / 2 : 0) : r0 + (row & ~1) + (odd ? 8 : 0);
+    const float scale = which == 0 ? rsqrtf((float)HD) : 1.f;
+    const int32_t *table = c.page_table + (size_t)a.seq * c.max_pages;
+    __nv_bfloat16 *pool = reinterpret_cast<__nv_bfloat16 *>(c.kv_pool);
+    float2 cs[16];
+    int page[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int m = m0 + min(2 * i + (lane >> 4), left - 1);
+        if (which < 2) cs[i] = *reinterpret_cast<const float2 *>(a.cs + ((size_t)m * (HD / 2) + jj) * 2);
+        if (which > 0) page[i] = table[(a.pos0 + m) >> c.page_shift];
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int jm = 2 * i + (lane >> 4), m = m0 + jm;
+        float y0 = x[jm][row], y1 = x[jm][row + 8];
+        if (which < 2) {   // the same in every lane
+            const float z0 = y0 * cs[i].x - y1 * cs[i].y, z1 = y1 * cs[i].x + y0 * cs[i].y;
+            y0 = z0 * scale; y1 = z1 * scale;
+        }
+        const float got = __shfl_xor_sync(0xffffffffu, odd ? y0 : y1, 1);
+        const float v0 = odd ? got : y0, v1 = odd ? y1 : got;
+        if (jm < left) {
+            if (which == 0) {
+                uint32_t h, w;
+                split2(v0, v1, h, w);
+                const size_t o = (size_t)m * qd + head * HD + fe;
+                *reinterpret_cast<uint32_t *>(a.hi + o) = h;
+                *reinterpret_cast<uint32_t *>(a.lo + o) = w;
+            } else {
+                const int pos = a.pos0 + m, t = pos & (c.page_tokens - 1);
+                const size_t base = ((((size_t)page[i] * c.L + a.layer) * 2 + (which - 1)) * c.nkv + head) * ((size_t)c.page_tokens * HD) + (size_t)t * HD;
+                *reinterpret_cast<__nv_bfloat162 *>(pool + base + ((((fe >> 3) ^ (pos & c.kv_swz)) << 3) | (fe & 7))) = __floats2bfloat162_rn(v0, v1);
+            }
         }
     }
 }
 
-// One row's q, k or v features [n, n + 128) of its matrix: q and k are rotated, q is scaled and split into bf16 high and
-// low parts, k and v go to the cache row of the position (16-byte chunks xor-swizzled, see kv_swz).
-template <int HD> __device__ __forceinline__ void epi_qkv(const Ctx &c, const GemmArgs &a, float (&acc)[128], int which, int n, int m) {
-    const int pos = a.pos0 + m;
+// SwiGLU: rows 0 .. 15 are the gate values of sixteen features, rows 16 .. 31 their up values; a lane takes two neighbouring
+// features of every fourth position.  The activations are split into bf16 high and low parts.
+__device__ __forceinline__ void epi_swiglu(const float (*x)[32], __nv_bfloat16 *hi, __nv_bfloat16 *lo, int ld, int lane, int left) {
+    const int n = 2 * (lane & 7);
+    uint32_t h[8], l[8];
 #pragma unroll
-    for (int h = 0; h < 128 / HD; ++h) {
-        if (n + h * HD >= a.nw[which]) break;
-        const int head = n / HD + h;
-        if (which < 2) {
-            const float *cs = a.cs + (size_t)m * HD;
+    for (int i = 0; i < 8; ++i) {
+        const int j = 4 * i + (lane >> 3);
+        const float2 g = *reinterpret_cast<const float2 *>(&x[j][n]), u = *reinterpret_cast<const float2 *>(&x[j][16 + n]);
+        split2(g.x / (1.0f + expf(-g.x)) * u.x, g.y / (1.0f + expf(-g.y)) * u.y, h[i], l[i]);
+    }
 #pragma unroll
-            for (int i = 0; i < HD / 2; i += 2) {
-                const float4 t = *reinterpret_cast<const float4 *>(cs + 2 * i);
-                float &x0 = acc[h * HD + i], &x1 = acc[h * HD + i + HD / 2], &y0 = acc[h * HD + i + 1], &y1 = acc[h * HD + i + 1 + HD / 2];
-                const float a0 = x0 * t.x - x1 * t.y, a1 = x1 * t.x + x0 * t.y, b0 = y0 * t.z - y1 * t.w, b1 = y1 * t.z + y0 * t.w;
-                x0 = a0; x1 = a1; y0 = b0; y1 = b1;
-            }
-        }
-        if (which == 0) {
-            const float scale = rsqrtf((float)HD);
-            const size_t o = (size_t)m * a.nw[0] + head * HD;
-#pragma unroll
-            for (int j = 0; j < HD; j += 8) {
-                uint4 hi, lo;
-                const float *v = acc + h * HD + j;
-                split2(v[0] * scale, v[1] * scale, hi.x, lo.x);
-                split2(v[2] * scale, v[3] * scale, hi.y, lo.y);
-                split2(v[4] * scale, v[5] * scale, hi.z, lo.z);
-                split2(v[6] * scale, v[7] * scale, hi.w, lo.w);
-                *reinterpret_cast<uint4 *>(a.hi + o + j) = hi;
-                *reinterpret_cast<uint4 *>(a.lo + o + j) = lo;
-            }
-        } else {
-            __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(c.kv_pool) + kv_index(c, a.seq, a.layer, which - 1, head, pos);
-#pragma unroll
-            for (int j = 0; j < HD; j += 8) {
-                uint4 o;
-                const float *v = acc + h * HD + j;
-                __nv_bfloat162 b[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) b[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-                o = *reinterpret_cast<const uint4 *>(b);
-                *reinterpret_cast<uint4 *>(dst + (((j >> 3) ^ (pos & c.kv_swz)) << 3)) = o;
-            }
+    for (int i = 0; i < 8; ++i) {
+        const int j = 4 * i + (lane >> 3);
+        if (j < left) {
+            *reinterpret_cast<uint32_t *>(hi + (size_t)j * ld + n) = h[i];
+            *reinterpret_cast<uint32_t *>(lo + (size_t)j * ld + n) = l[i];
         }
     }
 }
 
-// 64 gate and 64 up features of one row -> SwiGLU activation, split into bf16 high and low parts.
-__device__ __forceinline__ void epi_swiglu(const float (&acc)[128], __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
-#pragma unroll
-    for (int j = 0; j < 64; j += 8) {
-        float s[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float g = acc[j + e];
-            s[e] = g / (1.0f + expf(-g)) * acc[64 + j + e];
-        }
-        uint4 h, l;
-        split2(s[0], s[1], h.x, l.x);
-        split2(s[2], s[3], h.y, l.y);
-        split2(s[4], s[5], h.z, l.z);
-        split2(s[6], s[7], h.w, l.w);
-        *reinterpret_cast<uint4 *>(hi + j) = h;
-        *reinterpret_cast<uint4 *>(lo + j) = l;
-    }
-}
-
-// mapXhi / mapXlo: 2-D maps over the bf16 matrices [rows][K] (box 64 x 128); mapW0..2: over the weight matrices [N][K]
-// (box 64 x 128); all 128-byte swizzled, zero fill outside.  K a multiple of 64.  Grid: 2 x plan.pairs CTAs.
+// mapXhi / mapXlo: 2-D maps over the bf16 matrices [rows][K] (box 64 x plan.nt / 2); mapW0, mapW1: over the weight matrices
+// [N][K] (box 64 x 128; SwiGLU: gate and up, box 64 x 16); all 128-byte swizzled, zero fill outside.  K a multiple of 64.
+// Grid: 2 x plan.pairs CTAs.
 template <int EPI, int HD>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GTHREADS, 1)
 k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__ CUtensorMap mapXlo, const __grid_constant__ CUtensorMap mapW0,
-             const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ CUtensorMap mapW2, const __grid_constant__ Ctx c,
-             const __grid_constant__ GemmArgs a) {
+             const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ Ctx c, const __grid_constant__ GemmArgs a) {
     extern __shared__ unsigned char dsm_raw[];
     DSmem *sm = reinterpret_cast<DSmem *>(dsm_raw + ((1024u - (s32(dsm_raw) & 1023u)) & 1023u));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
-    const int pair = blockIdx.x >> 1, nkb = a.K / BK;
+    const int pair = blockIdx.x >> 1, nkb = a.K / BK, nt = a.plan.nt;
+    const int x_bytes = nt / 2 * BK * 2, stage_bytes = W_BYTES + 2 * x_bytes, stages = min(MAX_STAGES, RING_BYTES / stage_bytes);
     pdl_trigger();
     if (threadIdx.x == 0) {
-        for (int i = 0; i < STAGES; ++i) { mbar_init(&sm->full[i], 1); mbar_init(&sm->empty[i], 1); }
+        for (int i = 0; i < MAX_STAGES; ++i) { mbar_init(&sm->full[i], 1); mbar_init(&sm->empty[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&sm->acc_full[i], 1); mbar_init(&sm->acc_empty[i], 2 * GEPI_WARPS); }
         sm->abort = 0;
         fence_mbar_init();
@@ -394,24 +438,17 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(GREGS_ISSUE));
         if (warp == 0 && lane == 0) {
-            const uint32_t m_row = rank * BM;
-            auto weights = [&](int tn, const CUtensorMap *&mw) -> int {   // map and first row of this CTA's half of the tile's weight rows
-                mw = &mapW0;
-                if (EPI == EPI_SWIGLU) {
-                    if (rank) mw = &mapW1;
-                    return tn * BNH;
-                }
-                int t = tn;
-                if (EPI == EPI_QKV && t >= a.nt[0]) {
-                    t -= a.nt[0];
-                    mw = &mapW1;
-                    if (t >= a.nt[1]) { t -= a.nt[1]; mw = &mapW2; }
-                }
-                return t * TN + (int)rank * BNH;
-            };
-            auto load_w = [&](int st, const CUtensorMap *mw, int kb, int n0) {
-                if (rank == 0) mbar_expect_tx(&sm->full[st], 2u * STAGE_BYTES);   // both CTAs' tiles complete on the first CTA's barrier
-                tma_load_2d_pair(sm->stage[st] + 2 * A_BYTES, mw, kb * BK, n0, map_to_cta(&sm->full[st], 0));
+            auto load_w = [&](int st, int kb, int tn) {
+                if (rank == 0) mbar_expect_tx(&sm->full[st], 2u * (uint32_t)stage_bytes);   // both CTAs' tiles complete on the first CTA's barrier
+                const uint32_t bar = map_to_cta(&sm->full[st], 0);
+                unsigned char *dst = sm->ring + st * stage_bytes;
+                if (EPI == EPI_SWIGLU) {   // sixteen gate rows, the same rows of up, ...: one warp's lanes hold both
+                    for (int i = 0; i < 4; ++i) {
+                        const int f = tn * BW + (int)rank * 64 + 16 * i;
+                        tma_load_2d_pair(dst + i * 4096, &mapW0, kb * BK, f, bar);
+                        tma_load_2d_pair(dst + i * 4096 + 2048, &mapW1, kb * BK, f, bar);
+                    }
+                } else tma_load_2d_pair(dst, &mapW0, kb * BK, tn * TW + (int)rank * BW, bar);
             };
             // the weights of the first stages do not depend on earlier kernels
             int ahead = 0;
@@ -419,37 +456,38 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                 Sched sch(a.plan, pair);
                 Seg s;
                 if (sch.next(s)) {
-                    const CUtensorMap *mw;
-                    const int n0 = weights(s.tile / a.plan.mt, mw), kb0 = s.c0 * CK, kb1 = min(s.c1 * CK, nkb);
-                    for (; ahead < STAGES && kb0 + ahead < kb1; ++ahead) load_w(ahead, mw, kb0 + ahead, n0);
+                    const int kb0 = s.c0 * CK, kb1 = min(s.c1 * CK, nkb);
+                    for (; ahead < stages && kb0 + ahead < kb1; ++ahead) load_w(ahead, kb0 + ahead, s.tile / a.plan.mt);
                 }
             }
             pdl_wait();
             Sched sch(a.plan, pair);
             Seg s;
-            int it = 0;
+            int it = 0, st = 0;
+            uint32_t ph = 1;
             bool ok = true;
             while (ok && sch.next(s)) {
-                const int tm = s.tile % a.plan.mt, m0 = tm * TM + (int)m_row;
-                const CUtensorMap *mw;
-                const int n0 = weights(s.tile / a.plan.mt, mw), kb1 = min(s.c1 * CK, nkb);
+                const int tm = s.tile % a.plan.mt, tn = s.tile / a.plan.mt, x0 = tm * nt + (int)rank * (nt / 2), kb1 = min(s.c1 * CK, nkb);
                 for (int kb = s.c0 * CK; kb < kb1; ++kb, ++it) {
-                    const int st = it % STAGES;
                     if (it >= ahead) {
-                        ok = dwait(sm, a.err, &sm->empty[st], ((it / STAGES) & 1) ^ 1);
+                        ok = dwait(sm, a.err, &sm->empty[st], ph);
                         if (!ok) break;
-                        load_w(st, mw, kb, n0);
+                        load_w(st, kb, tn);
                     }
                     const uint32_t bar = map_to_cta(&sm->full[st], 0);
-                    tma_load_2d_pair(sm->stage[st], &mapXhi, kb * BK, m0, bar);
-                    tma_load_2d_pair(sm->stage[st] + A_BYTES, &mapXlo, kb * BK, m0, bar);
+                    unsigned char *dst = sm->ring + st * stage_bytes + W_BYTES;
+                    tma_load_2d_pair(dst, &mapXhi, kb * BK, x0, bar);
+                    tma_load_2d_pair(dst + x_bytes, &mapXlo, kb * BK, x0, bar);
+                    if (++st == stages) { st = 0; ph ^= 1; }
                 }
             }
         }
         if (warp == 1 && lane == 0 && rank == 0) {
+            const uint32_t id = Idesc<TW, 0>::v | ((uint32_t)(nt >> 3) << 17);
             Sched sch(a.plan, pair);
             Seg s;
-            int it = 0, ch = 0;
+            int ch = 0, st = 0;
+            uint32_t ph = 0;
             bool ok = true;
             while (ok && sch.next(s)) {
                 for (int cc = s.c0; ok && cc < s.c1; ++cc, ++ch) {
@@ -457,22 +495,22 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                     ok = dwait(sm, a.err, &sm->acc_empty[b], ((ch >> 1) & 1) ^ 1);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t acc = tmem + (uint32_t)(b * TN);
                     uint32_t add = 0;
-                    for (int kb = cc * CK; kb < kb1; ++kb, ++it) {
-                        const int st = it % STAGES;
-                        ok = dwait(sm, a.err, &sm->full[st], (it / STAGES) & 1);
+                    for (int kb = cc * CK; kb < kb1; ++kb) {
+                        ok = dwait(sm, a.err, &sm->full[st], ph);
                         if (!ok) break;
                         tc_fence_after();
-                        const unsigned long long ahi = smem_desc(s32(sm->stage[st])), alo = smem_desc(s32(sm->stage[st] + A_BYTES)),
-                                                 w = smem_desc(s32(sm->stage[st] + 2 * A_BYTES));
+                        const uint32_t base = s32(sm->ring + st * stage_bytes);
+                        const unsigned long long w = smem_desc(base), xh = smem_desc(base + W_BYTES), xl = smem_desc(base + W_BYTES + x_bytes);
+                        const uint32_t acc = tmem + (uint32_t)(b * 256);
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {   // 32 bytes further along the swizzled row per K = 16 step
-                            umma_pair(acc, ahi + 2 * k, w + 2 * k, add);
-                            umma_pair(acc, alo + 2 * k, w + 2 * k, 1u);
-                            add = 1u;
+                            umma_pair(acc, w + 2 * k, xh + 2 * k, id, k == 0 ? add : 1u);
+                            umma_pair(acc, w + 2 * k, xl + 2 * k, id, 1u);
                         }
+                        add = 1u;
                         umma_commit_pair(&sm->empty[st]);   // the stage is free in both CTAs once these MMAs have read it
+                        if (++st == stages) { st = 0; ph ^= 1; }
                     }
                     umma_commit_pair(&sm->acc_full[b]);
                 }
@@ -480,9 +518,9 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GREGS_EPI));
-        // epilogue: warp w may read the 32 lanes 32 (w % 4) .. of the tensor memory; lane = position within the CTA's 128
-        const int q = warp & 3, h = (warp - 4) >> 2, ew = warp - 4;
-        const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
+        // epilogue: warp w may read the 32 lanes 32 (w % 4) .. of the tensor memory; lane = weight row within the CTA's 128
+        const int q = warp & 3, h = (warp - 4) >> 2, ew = warp - 4, nh = nt / 2;
+        const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * nh);
         pdl_wait();
         Sched sch(a.plan, pair);
         Seg s;
@@ -490,8 +528,10 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
         bool ok = true;
         while (ok && sch.next(s)) {
             const int tm = s.tile % a.plan.mt, tn = s.tile / a.plan.mt;
-            const int mw = tm * TM + (int)rank * BM + q * 32, m = mw + lane;   // first row of the warp, row of the lane
-            const bool live = mw < a.rows;                                     // the same in every lane, and in the same warp of every pair
+            // first position; first weight row (SwiGLU: feature) of the warp
+            const int m0 = tm * nt + h * nh, n_w = EPI == EPI_SWIGLU ? tn * BW + (int)rank * 64 + q * 16 : tn * TW + (int)rank * BW + q * 32;
+            const int left = min(nh, a.rows - m0);
+            const bool live = left > 0 && n_w < a.N;   // the same in every lane, and in the same warp of every pair
             float acc[128];
 #pragma unroll
             for (int j = 0; j < 128; ++j) acc[j] = 0.f;
@@ -503,15 +543,15 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                 tc_fence_after();
                 if (live) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint32_t v[32];
-                        const int col = EPI == EPI_SWIGLU ? (j >> 1) * BNH + h * 64 + (j & 1) * 32 : h * 128 + j * 32;
-                        tmem_ld32(v, t_lane + (uint32_t)(b * TN + col));
+                    for (int g = 0; g < 8; ++g)
+                        if (16 * g < nh) {
+                            uint32_t v[16];
+                            tmem_ld16(v, t_lane + (uint32_t)(b * 256 + 16 * g));
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) acc[32 * j + e] += __uint_as_float(v[e]);
+                            for (int e = 0; e < 16; ++e) acc[16 * g + e] += __uint_as_float(v[e]);
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) asm volatile("" : "+f"(acc[32 * j + e]));
-                    }
+                            for (int e = 0; e < 16; ++e) asm volatile("" : "+f"(acc[16 * g + e]));
+                        }
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -521,7 +561,8 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
             if (s.c1 < a.plan.chunks) {   // another pair finishes this tile
                 float4 *o = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a.part) + (size_t)(2 * pair + (int)rank) * GPART_CTA + ew * GPART_WARP) + lane;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) __stcg(o + 32 * j, make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]));
+                for (int j = 0; j < 32; ++j)
+                    if (4 * j < nh) __stcg(o + 32 * j, make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]));
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.flag + (2 * pair + (int)rank) * GEPI_WARPS + ew), "r"(a.epoch) : "memory");
@@ -552,7 +593,9 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                     for (int j0 = 0; j0 < 32; j0 += 16) {   // sixteen loads in flight: more would not fit beside the sums
                         float4 r[16];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) r[j] = ld_cg_inorder(in + 32 * (j0 + j));
+                        for (int j = 0; j < 16; ++j)
+                            if (4 * (j0 + j) < nh) r[j] = ld_cg_inorder(in + 32 * (j0 + j));
+                            else r[j] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             const int e = 4 * (j0 + j);
@@ -562,22 +605,13 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                 }
                 if (!ok) continue;
             }
-            if (m >= a.rows) continue;
-            if constexpr (EPI == EPI_STORE || EPI == EPI_ADD) {
-                const int n = tn * TN + h * 128;
-                if (n < a.nw[0]) epi_rows<EPI == EPI_ADD>(acc, a.Y + (size_t)m * a.ldy + n, a.nw[0] - n);
-            } else if constexpr (EPI == EPI_QKV) {
-                int t = tn, which = 0;
-                if (t >= a.nt[0]) {
-                    t -= a.nt[0];
-                    which = 1;
-                    if (t >= a.nt[1]) { t -= a.nt[1]; which = 2; }
-                }
-                epi_qkv<HD>(c, a, acc, which, t * TN + h * 128, m);
-            } else {
-                const int n = tn * BNH + h * 64;
-                if (n < a.nw[0]) epi_swiglu(acc, a.hi + (size_t)m * a.nw[0] + n, a.lo + (size_t)m * a.nw[0] + n);
-            }
+            float(*x)[32] = sm->stash[ew];
+            epi_rounds(acc, x, lane, left, [&](int j0, int cnt) {
+                const int m = m0 + j0;
+                if constexpr (EPI == EPI_STORE || EPI == EPI_ADD) epi_rows<EPI == EPI_ADD>(x, a.Y + (size_t)m * a.ldy + n_w, a.ldy, a.N - n_w, lane, cnt);
+                else if constexpr (EPI == EPI_QKV) epi_qkv<HD>(c, a, x, n_w, lane, m, cnt);
+                else epi_swiglu(x, a.hi + (size_t)m * a.N + n_w, a.lo + (size_t)m * a.N + n_w, a.N, lane, cnt);   // N is a multiple of 64: the warp's features are all there
+            });
         }
     }
     if (*(volatile int *)&sm->abort) {   // copies already issued may still be landing: give them time before the block's memory goes

@@ -36,7 +36,7 @@ def _compare(cfg, gm, n, page_tokens=64):
     assert np.linalg.norm(ld[0] - lc[0]) <= 5e-3 * np.linalg.norm(lc[0])
 
 
-@pytest.mark.parametrize("n", [32, 63, 128, 129, 256, 257, 513])
+@pytest.mark.parametrize("n", [9, 31, 32, 33, 64, 65, 128, 129, 256, 257, 513, 800])
 def test_tile_edges(n):
     _compare(*_model(64, 4, 2), n)
 
