@@ -205,7 +205,7 @@ namespace {
 struct Layout {
     size_t st, rt, fill, tokens, page_table, head_res, resid, xn, qkv, q, attn_out, gu, hact, rope_cs, attn_part,
         head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_err, pf_flag, pf_part, maps, mm, exit_at, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
-        grid_ctr, pub, err, q_stage, qinfo, uniforms, total;
+        grid_ctr, pub, err, attn_tag, q_stage, qinfo, uniforms, total;
 };
 
 bool model_fits_persistent(const ada_config &g);
@@ -221,6 +221,11 @@ constexpr int kGemmMaxPairs = 80;   // CTA pairs the exchange area of cut tiles 
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
 constexpr int kPartMaxGrid = 256;
+
+// chunk partials of the decode attention as tagged words (see attn_consume_single)
+size_t attn_tag_bytes(const ada_config &g, int n_chunks) {
+    return sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)n_chunks * (g.head_dim + 2);
+}
 
 Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, int head_blocks) {
     Layout L{};
@@ -279,6 +284,7 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.grid_ctr = take(256);
         L.pub = take(sizeof(mg::Pub) * 2);
         L.err = take(256);
+        L.attn_tag = take(attn_tag_bytes(g, n_chunks));
         // sampled decoding: the logits and normalisers of the intermediate head that drew each token in flight, and the
         // random numbers of every sequence position
         L.q_stage = take(sizeof(float) * (size_t)batch * st::MAX_COLS * g.vocab);
@@ -802,6 +808,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     a.attn_part = S->c.attn_part;
     a.head_part = S->c.head_part;
     a.attn_cnt = (unsigned *)(b + lay.attn_cnt);
+    a.attn_tag = (unsigned long long *)(b + lay.attn_tag);
     a.rope_freq = (const double *)(b + lay.rope_freq);
     a.part = S->grid <= kPartMaxGrid ? (unsigned long long *)(b + lay.part) : nullptr;
     a.grid_ctr = (unsigned *)(b + lay.grid_ctr);
@@ -876,6 +883,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             CK(cudaMemsetAsync(a.grid_ctr, 0, sizeof(unsigned), S->stream));
             CK(cudaMemsetAsync(a.pub, 0, sizeof(mg::Pub) * 2, S->stream));
             if (a.part) CK(cudaMemsetAsync(a.part, 0, kPartBytesPerCta * (size_t)S->grid, S->stream));
+            CK(cudaMemsetAsync(a.attn_tag, 0, attn_tag_bytes(g, S->n_chunks), S->stream));   // phase numbers start over with every launch
             void *params[] = {(void *)&a};
             CK(cudaLaunchCooperativeKernel(kern, dim3(S->grid), dim3(st::THREADS), params, st::SMEM_BYTES, S->stream));
             S->launches++;

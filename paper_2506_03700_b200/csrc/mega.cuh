@@ -83,6 +83,7 @@ struct MegaArgs {
     const double *rope_freq;   // [hd/2]: base^(-2i/hd), computed once on the host
     unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
     unsigned *attn_cnt;        // [nkv]
+    unsigned long long *attn_tag;   // [8][nq][n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume_single); zeroed before each launch
     unsigned *grid_ctr;
     Pub *pub;                  // [2]
     int *err;
@@ -951,8 +952,12 @@ template <int HD> struct AttnSmem {
     union {
         uint32_t qfrag[2][HD / 16][32][8];   // A fragments of the rotated, scaled queries: hi a0..a3, lo a0..a3
         float o[2][2][16][HD];               // merge buffers [query tile][source]
+        float oq[4][16][HD];                 // one tile in use: [position quarter]
     };
-    float ml[2][2][2][16];                   // [query tile][source][max | sum][row]
+    union {
+        float ml[2][2][2][16];               // [query tile][source][max | sum][row]
+        float mlq[4][2][16];                 // [position quarter][max | sum][row]
+    };
 };
 static_assert(sizeof(AttnSmem<128>) <= SCRATCH_BYTES, "attention buffers exceed the consumers' scratch");
 
@@ -1125,6 +1130,18 @@ __device__ __forceinline__ void attn_produce_single(const MegaArgs &A, const Sha
     }
 }
 
+// Two partial softmaxes (max, sum, unnormalised output) become one: (m, l) takes over (mb, lb); an output is a o + b ob.  The
+// operations are written out (no contraction left to the compiler): two places that merge the same pair get the same bits.
+__device__ __forceinline__ float merge_value(float oa, float a, float ob, float b) { return __fmaf_rn(oa, a, __fmul_rn(ob, b)); }
+__device__ __forceinline__ void merge_weights(float &m, float &l, float mb, float lb, float &a, float &b) {
+    const float mn = fmaxf(m, mb);
+    a = 1.f;
+    b = 0.f;
+    if (mn != -INFINITY) { a = __expf(m - mn); b = __expf(mb - mn); }
+    m = mn;
+    l = merge_value(l, a, lb, b);
+}
+
 // Merge (max, sum, unnormalised output) of another warp, read from shared memory, into this warp's.
 template <int NT, int HD>
 __device__ __forceinline__ void attn_merge_from(float (&o)[NT][4], float (&m_run)[2], float (&l_run)[2], const float (*so)[HD],
@@ -1132,17 +1149,13 @@ __device__ __forceinline__ void attn_merge_from(float (&o)[NT][4], float (&m_run
 #pragma unroll
     for (int rh = 0; rh < 2; ++rh) {
         const int row = (lane >> 2) + 8 * rh;
-        const float ms = sml[0][row], ls = sml[1][row];
-        const float mn = fmaxf(m_run[rh], ms);
-        float a = 1.f, b = 0.f;
-        if (mn != -INFINITY) { a = __expf(m_run[rh] - mn); b = __expf(ms - mn); }
-        m_run[rh] = mn;
-        l_run[rh] = l_run[rh] * a + ls * b;
+        float a, b;
+        merge_weights(m_run[rh], l_run[rh], sml[0][row], sml[1][row], a, b);
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {   // columns rotated by 8 (row % 8): conflict-free 8-byte accesses
             const float2 v = *reinterpret_cast<const float2 *>(&so[row][(nt * 8 + 2 * (lane & 3) + 8 * (row & 7)) & (HD - 1)]);
-            o[nt][2 * rh] = o[nt][2 * rh] * a + v.x * b;
-            o[nt][2 * rh + 1] = o[nt][2 * rh + 1] * a + v.y * b;
+            o[nt][2 * rh] = merge_value(o[nt][2 * rh], a, v.x, b);
+            o[nt][2 * rh + 1] = merge_value(o[nt][2 * rh + 1], a, v.y, b);
         }
     }
 }
@@ -1176,103 +1189,72 @@ __device__ __forceinline__ int div_group(int x, int group) {
     return group == 4 ? x >> 2 : group == 2 ? x >> 1 : group == 1 ? x : (x * 43) >> 7;
 }
 
+// Query tiles in use (bit t: some (column, q head) pair of the columns mk lies in rows [16 t, 16 t + 16)).
+__device__ __forceinline__ bool tile_in_use(unsigned mk, int t, int group) {
+    const int lo = div_group(16 * t, group), hi = div_group(16 * t + 15, group);
+    return (mk & ((2u << hi) - (1u << lo)) & 0xffu) != 0;
+}
+__device__ __forceinline__ void st_tagged2(unsigned long long *p, float a, float b, unsigned tag) {   // two tagged words; 16-byte aligned
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | __float_as_uint(a)), "l"(t | __float_as_uint(b)) : "memory");
+}
+__device__ __forceinline__ bool ld_tagged2(const unsigned long long *p, float &a, float &b, unsigned tag) {
+    unsigned long long x, y;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(p) : "memory");
+    a = __uint_as_float((unsigned)x);
+    b = __uint_as_float((unsigned)y);
+    return (unsigned)(x >> 32) == tag && (unsigned)(y >> 32) == tag;
+}
+
 // The same for a phase in which no CTA owns more than one item (contexts up to about 128 positions x CTAs / kv heads:
-// the common case of short and medium contexts): one item, its two query tiles on the two warp groups, merged by
-// whichever CTA completes a head last.  Kept as a path of its own: the general form below, with its rounds of two
-// items, costs this case 2-4 % of the step.
+// the common case of short and medium contexts): one item, its two query tiles on the two warp groups.  Kept as a path of
+// its own: the general form below, with its rounds of two items, costs this case 2-4 % of the step.
+//
+// The phase is a chain of latencies (1 us of arithmetic, 1 us of traffic, 11-14 us measured), so its exchanges are kept short:
+//   * with one query tile in use (plain decoding, few columns) the four position quarters meet once in shared memory and
+//     every thread merges elements of its own, in place of two levels of warp-to-warp merges with four barriers;
+//   * the chunk partials travel as 8-byte words that carry the phase number beside the value: whoever sees the tag sees the
+//     value, so no fence, counter and second look stand between writing and reading them (3.1-3.8 us before);
+//   * each of a head's chunk CTAs merges its share of the head's outputs, so a CTA reads as much as it wrote, in one
+//     round trip, however many chunks there are.  Who merges does not change what is computed.
 template <int HD>
-__device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, Rings &r) {
+__device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, unsigned tag, Rings &r) {
     const Ctx &c = A.c;
     Smem *sm = S.sm;
     AttnSmem<HD> *as = reinterpret_cast<AttnSmem<HD> *>(sm->scratch);
     constexpr int KSQ = HD / 16, NT = HD / 8;
-    constexpr int ATT_STRIDE = HD + 4;                     // floats per chunk partial: output, max, sum, padding (16-byte rows)
+    constexpr int TS = HD + 2;                             // tagged words per chunk partial: output, max, sum
     constexpr int QV = 2 * KSQ * 64 / CONS_THREADS;        // 16-byte pieces of a kv head's query fragments per thread
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x, G = gridDim.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x;
     const int group = c.group;
     const int n_items = attn_items(A, d, mask);
     const int mt = warp >> 2, qr = warp & 3;
     (void)layer;
-    // Merge of the chunk partials of one kv head into the O-projection's input (by a whole CTA).
-    auto merge_chunks = [&](int kvh, unsigned mk) {   // mk: the active columns of the work item's sequence
-        // Four features of one (column, q head) per thread and pass; the chunk partials are folded in
-        // ascending order, eight at a time with all their loads in flight, by the usual running-max rule.
-        const int nqc = MAX_COLS * group;
-        for (int idx = tid; idx < nqc * (HD / 4); idx += CONS_THREADS) {
-            const int qcol = idx / (HD / 4), dim = (idx - qcol * (HD / 4)) * 4, cc = div_group(qcol, group), g = qcol - cc * group;
-            if (!((mk >> cc) & 1u)) continue;
-            const int h = kvh * group + g;
-            const int nch = d.pos[cc] / ATT_CHUNK + 1;
-            const float *part = A.attn_part + (((size_t)cc * c.nq + h) * c.n_chunks) * ATT_STRIDE;
-            float Mx = -INFINITY, den = 0.f;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int k0 = 0; k0 < nch; k0 += 8) {
-                float2 ml[8];
-                float4 ov[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const bool ok = k0 + u < nch;
-                    const float *pk = part + (size_t)(k0 + u) * ATT_STRIDE;
-                    ml[u] = ok ? __ldcg(reinterpret_cast<const float2 *>(pk + HD)) : make_float2(-INFINITY, 0.f);
-                    ov[u] = ok ? __ldcg(reinterpret_cast<const float4 *>(pk + dim)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                float Mn = Mx;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) Mn = fmaxf(Mn, ml[u].x);
-                if (Mn == -INFINITY) continue;
-                const float sc = Mx == -INFINITY ? 0.f : __expf(Mx - Mn);
-                den *= sc; acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (ml[u].x != -INFINITY) {
-                        const float w = __expf(ml[u].x - Mn);
-                        den += ml[u].y * w;
-                        acc.x += ov[u].x * w; acc.y += ov[u].y * w; acc.z += ov[u].z * w; acc.w += ov[u].w * w;
-                    }
-                }
-                Mx = Mn;
-            }
-            xfrag_store(A.XO, h * HD + dim, cc, acc.x / den);
-            xfrag_store(A.XO, h * HD + dim + 1, cc, acc.y / den);
-            xfrag_store(A.XO, h * HD + dim + 2, cc, acc.z / den);
-            xfrag_store(A.XO, h * HD + dim + 3, cc, acc.w / den);
-        }
-    };
-    // With at most one work item per CTA the CTA that completes a head last merges it at once; with more,
-    // designated CTAs do (see below).  Who merges does not change what is computed.
-    const bool last_arriver_merges = true;   // at most one item per CTA (the caller's condition)
-    for (int item = cta; item < n_items; item += G) {
+    for (int item = cta; item < n_items; item += n_items) {   // at most one (the caller's condition)
         int ks_, kvh, j, nchunk;
         attn_item(A, d, mask, item, ks_, kvh, j, nchunk);
         const unsigned mk = mask & seq_cols(A, ks_);   // the item's sequence: its columns only
         const int p_base = j * ATT_CHUNK;
         const int nsb = min(ATT_CHUNK / ATT_PAGE, (d.seq_pmax[ks_] - p_base) / ATT_PAGE + 1);
-        // ---- the kv head's query fragments: one round trip to L2, then shared memory
-        {
-            const uint4 *src = reinterpret_cast<const uint4 *>(A.qfrag) + (size_t)kvh * (2 * KSQ * 64);
-            uint4 v[QV];
-#pragma unroll
-            for (int u = 0; u < QV; ++u) v[u] = __ldcg(src + tid + u * CONS_THREADS);
-            bar_consumers();   // the previous item is done with the shared buffers
-#pragma unroll
-            for (int u = 0; u < QV; ++u) reinterpret_cast<uint4 *>(&as->qfrag[0][0][0][0])[tid + u * CONS_THREADS] = v[u];
-        }
-        bar_consumers();
-        if (tid == 0) trace(S, EV_ATT, 2);   // queries ready
-        // ---- per-warp online softmax state: rows (lane/4) and (lane/4)+8 of query tile mt
+        const bool one_tile = !tile_in_use(mk, 1, group), tile_used = tile_in_use(mk, mt, group);
+        // per-warp online softmax state: rows (lane/4) and (lane/4)+8 of query tile mt
         int lim[2];
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {
             const int qcol = mt * 16 + (lane >> 2) + rh * 8, cc = div_group(qcol, group);
             lim[rh] = (cc < MAX_COLS && ((mk >> cc) & 1u)) ? d.pos[cc] : -1;
         }
-        // a query tile none of whose 16 (column, q head) pairs is in use does no arithmetic (uniform per warp)
-        bool tile_used = false;
+        // ---- the kv head's query fragments: one round trip to L2, then shared memory
+        {
+            const uint4 *src = reinterpret_cast<const uint4 *>(A.qfrag) + (size_t)kvh * (2 * KSQ * 64);
+            uint4 v[QV];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int cc = div_group(mt * 16 + q, group);
-            tile_used = tile_used || (cc < MAX_COLS && ((mk >> cc) & 1u));
+            for (int u = 0; u < QV; ++u) v[u] = __ldcg(src + tid + u * CONS_THREADS);
+#pragma unroll
+            for (int u = 0; u < QV; ++u) reinterpret_cast<uint4 *>(&as->qfrag[0][0][0][0])[tid + u * CONS_THREADS] = v[u];
         }
+        bar_consumers();
+        if (tid == 0) trace(S, EV_ATT, 2);   // queries ready
         float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
         float o[NT][4];
 #pragma unroll
@@ -1389,46 +1371,113 @@ __device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Sha
         }
         if (tid == 0) trace(S, EV_ATT, 5);   // sub-blocks done
         bar_consumers();   // every warp is done with the query fragments, whose space the merge reuses
-        // (a query tile without a query in use skips the merge: its warps only keep the barriers)
-        if ((qr & 1) && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
-        bar_consumers();
-        if (!(qr & 1) && tile_used) attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
-        bar_consumers();
-        if (qr == 2 && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
-        bar_consumers();
-        if (qr == 0) {
-            if (tile_used) attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
-            // ---- chunk partial (unnormalised output, max, sum) of every valid (column, q head)
+        auto words = [&](int cc, int h, int chunk) { return A.attn_tag + (((size_t)cc * c.nq + h) * c.n_chunks + chunk) * TS; };
+        if (one_tile) {
+            if (mt == 0) attn_merge_to<NT, HD>(o, m_run, l_run, as->oq[qr], as->mlq[qr], lane);
+            bar_consumers();
+            // two features per thread and pass: (quarter 0 + quarter 1) + (quarter 2 + quarter 3), like the warps below
+            for (int idx = tid; idx < 16 * (HD / 2); idx += CONS_THREADS) {
+                const int row = idx / (HD / 2), dim = (idx % (HD / 2)) * 2, cc = div_group(row, group), g = row - cc * group;
+                if (cc >= MAX_COLS || !((mk >> cc) & 1u) || d.pos[cc] < p_base) continue;
+                float m[4], l[4];
+                float2 v[4];
 #pragma unroll
-            for (int rh = 0; rh < 2; ++rh) {
-                const int qcol = mt * 16 + (lane >> 2) + 8 * rh, cc = div_group(qcol, group), g = qcol - cc * group;
-                if (cc < MAX_COLS && ((mk >> cc) & 1u) && d.pos[cc] >= p_base) {
-                    float *out = A.attn_part + (((size_t)cc * c.nq + kvh * group + g) * c.n_chunks + j) * ATT_STRIDE;
+                for (int q = 0; q < 4; ++q) {
+                    m[q] = as->mlq[q][0][row];
+                    l[q] = as->mlq[q][1][row];
+                    v[q] = *reinterpret_cast<const float2 *>(&as->oq[q][row][(dim + 8 * (row & 7)) & (HD - 1)]);
+                }
+                float a, b;
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt)
-                        *reinterpret_cast<float2 *>(out + nt * 8 + 2 * (lane & 3)) = make_float2(o[nt][2 * rh], o[nt][2 * rh + 1]);
-                    if ((lane & 3) == 0) *reinterpret_cast<float2 *>(out + HD) = make_float2(m_run[rh], l_run[rh]);
+                for (int q = 0; q < 4; q += 2) {
+                    merge_weights(m[q], l[q], m[q + 1], l[q + 1], a, b);
+                    v[q].x = merge_value(v[q].x, a, v[q + 1].x, b);
+                    v[q].y = merge_value(v[q].y, a, v[q + 1].y, b);
+                }
+                merge_weights(m[0], l[0], m[2], l[2], a, b);
+                unsigned long long *out = words(cc, kvh * group + g, j);
+                st_tagged2(out + dim, merge_value(v[0].x, a, v[2].x, b), merge_value(v[0].y, a, v[2].y, b), tag);
+                if (dim == 0) st_tagged2(out + HD, m[0], l[0], tag);
+            }
+        } else {
+            // merge the four position quarters of each query tile: (q0 + q1) and (q2 + q3), then the two halves
+            // (a query tile without a query in use skips the merge: its warps only keep the barriers)
+            if ((qr & 1) && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
+            bar_consumers();
+            if (!(qr & 1) && tile_used) attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
+            bar_consumers();
+            if (qr == 2 && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
+            bar_consumers();
+            if (qr == 0 && tile_used) {
+                attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
+                // ---- chunk partial (unnormalised output, max, sum) of every valid (column, q head)
+#pragma unroll
+                for (int rh = 0; rh < 2; ++rh) {
+                    const int qcol = mt * 16 + (lane >> 2) + 8 * rh, cc = div_group(qcol, group), g = qcol - cc * group;
+                    if (cc < MAX_COLS && ((mk >> cc) & 1u) && d.pos[cc] >= p_base) {
+                        unsigned long long *out = words(cc, kvh * group + g, j);
+#pragma unroll
+                        for (int nt = 0; nt < NT; ++nt) st_tagged2(out + nt * 8 + 2 * (lane & 3), o[nt][2 * rh], o[nt][2 * rh + 1], tag);
+                        if ((lane & 3) == 0) st_tagged2(out + HD, m_run[rh], l_run[rh], tag);
+                    }
                 }
             }
         }
-        // ---- this item's partials are complete: count it (a release that returns nothing, so nobody waits for it)
         if (tid == 0) trace(S, EV_ITEM, item);
-        bar_consumers();
-        if (last_arriver_merges) {
-            if (tid == 0) {   // release this block's partials and acquire the others' in one step
-                unsigned old;
-                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(A.attn_cnt + ks_ * c.nkv + kvh) : "memory");
-                sm->bcast[2] = (int)old;
+        // ---- this CTA's share of the head's outputs: two features of one (column, q head) per thread and pass; the chunk
+        // partials are folded in ascending order, eight at a time with all their loads in flight, by the running-max rule
+        const int units = __popc(mk) * group * (HD / 2), u1 = units * (j + 1) / nchunk;
+        for (int u = units * j / nchunk + tid; u < u1; u += CONS_THREADS) {
+            const int row = u / (HD / 2), dim = (u % (HD / 2)) * 2, nth = div_group(row, group), g = row - nth * group;
+            int cc = 0;   // the nth active column
+#pragma unroll
+            for (int q = 0; q < MAX_COLS; ++q)
+                if (((mk >> q) & 1u) && __popc(mk & ((1u << q) - 1u)) == nth) cc = q;
+            const int h = kvh * group + g, nch = d.pos[cc] / ATT_CHUNK + 1;
+            const unsigned long long *part = words(cc, h, 0);
+            float Mx = -INFINITY, den = 0.f, ax = 0.f, ay = 0.f;
+            for (int k0 = 0; k0 < nch; k0 += 8) {
+                float ml[8], ll[8], ox[8], oy[8];
+                unsigned long long t0 = 0;
+                for (uint32_t it = 0;; ++it) {
+                    bool ok = true;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        ml[q] = -INFINITY; ll[q] = 0.f; ox[q] = 0.f; oy[q] = 0.f;
+                        if (k0 + q < nch) {
+                            const bool a = ld_tagged2(part + (size_t)(k0 + q) * TS + HD, ml[q], ll[q], tag);
+                            const bool b = ld_tagged2(part + (size_t)(k0 + q) * TS + dim, ox[q], oy[q], tag);
+                            ok = ok && a && b;
+                        }
+                    }
+                    if (ok) break;
+                    if ((it & 15u) == 15u || S.wait_ns < SHORT_LIMIT_NS) {   // bounded like every other wait on another CTA
+                        if (aborted(S)) break;
+                        if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; break; }
+                        const unsigned long long t = gtime();
+                        if (t0 == 0) t0 = t;
+                        else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_GRID); break; }
+                    }
+                }
+                float Mn = Mx;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) Mn = fmaxf(Mn, ml[q]);
+                if (Mn == -INFINITY) continue;
+                const float sc = Mx == -INFINITY ? 0.f : __expf(Mx - Mn);
+                den = __fmul_rn(den, sc); ax = __fmul_rn(ax, sc); ay = __fmul_rn(ay, sc);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (ml[q] != -INFINITY) {
+                        const float w = __expf(ml[q] - Mn);
+                        den = __fmaf_rn(ll[q], w, den);
+                        ax = __fmaf_rn(ox[q], w, ax);
+                        ay = __fmaf_rn(oy[q], w, ay);
+                    }
+                Mx = Mn;
             }
-            bar_consumers();
-            if (sm->bcast[2] == nchunk - 1) {
-                merge_chunks(kvh, mk);
-                if (tid == 0) { A.attn_cnt[ks_ * c.nkv + kvh] = 0u; trace(S, EV_COMBINE, kvh); }
-            }
-        } else if (tid == 0) {
-            __threadfence();
-            red_release_add(A.attn_cnt + ks_ * c.nkv + kvh, 1u);
+            xfrag_store2(A.XO, h * HD + dim, cc, ax / den, ay / den);
         }
+        if (tid == 0) trace(S, EV_COMBINE, kvh);
     }
 }
 
@@ -1473,13 +1522,13 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
                 for (int u = 0; u < 8; ++u) Mn = fmaxf(Mn, ml[u].x);
                 if (Mn == -INFINITY) continue;
                 const float sc = Mx == -INFINITY ? 0.f : __expf(Mx - Mn);
-                den *= sc; acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
+                den = __fmul_rn(den, sc); acc.x = __fmul_rn(acc.x, sc); acc.y = __fmul_rn(acc.y, sc); acc.z = __fmul_rn(acc.z, sc); acc.w = __fmul_rn(acc.w, sc);
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     if (ml[u].x != -INFINITY) {
                         const float w = __expf(ml[u].x - Mn);
-                        den += ml[u].y * w;
-                        acc.x += ov[u].x * w; acc.y += ov[u].y * w; acc.z += ov[u].z * w; acc.w += ov[u].w * w;
+                        den = __fmaf_rn(ml[u].y, w, den);
+                        acc.x = __fmaf_rn(ov[u].x, w, acc.x); acc.y = __fmaf_rn(ov[u].y, w, acc.y); acc.z = __fmaf_rn(ov[u].z, w, acc.z); acc.w = __fmaf_rn(ov[u].w, w, acc.w);
                     }
                 }
                 Mx = Mn;
@@ -1731,11 +1780,11 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
 
 // ---------------------------------------------------------------- the walker
 
-template <int ROLE, int PAIR, class Epi>
-__device__ __forceinline__ void gemm_phase(const Shared &S, const Gemm &g, Rings &r, uint64_t pol, Epi &&epi) {
+template <int ROLE, int PAIR, class Ready, class Epi>
+__device__ __forceinline__ void gemm_phase(const Shared &S, const Gemm &g, Rings &r, uint64_t pol, Ready &&ready, Epi &&epi) {
     const int cta = blockIdx.x, G = gridDim.x;
     if (ROLE == 0) gemm_produce_w(S, g, cta, G, r, pol);
-    else if (ROLE == 1) gemm_produce_x(S, g, cta, G, r, pol);
+    else if (ROLE == 1) gemm_produce_x(S, g, cta, G, r, pol, NoHook(), ready);
     else gemm_consume<PAIR>(S, g, cta, G, r, epi);
 }
 
@@ -1802,7 +1851,6 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
     // head over E* with the fused (max, sum exp, argmax) reduction; X = final-normed residual (or T output)
     auto head_phase = [&](const __nv_bfloat16 *X, const float *ssq, float scale, unsigned cols, bool inter) {
         Gemm g; g.W = M.lm_head; g.X = reinterpret_cast<const uint4 *>(X); g.N = c.vocab; g.K = d_model; g.pair = 1; g.half = 0; g.ctas = n_head; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(cols);
-        x_ready();
         const unsigned vseq = bar_no + 1;
         if (ROLE == 2) {
             Msa run[2];
@@ -1868,9 +1916,9 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 o[0] = a.m; o[1] = a.s; o[2] = __int_as_float(a.i);
             }
         } else if (ROLE == 1) {
-            gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { if (ssq) rstd_produce(sm, ssq, ntd, d_model, c.eps, vseq); });
+            gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { if (ssq) rstd_produce(sm, ssq, ntd, d_model, c.eps, vseq); }, x_ready);
         } else {
-            gemm_phase<ROLE, 1>(S, g, r, pol, NoEpi());
+            gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
         }
         phase_barrier(9);
     };
@@ -1893,7 +1941,6 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
             // are then rows r and r + 8 of one tile, which one thread holds for its two columns.
             {
                 Gemm g; g.W = ly.wqkv; g.X = reinterpret_cast<const uint4 *>(A.XA); g.N = c.qkv_rows; g.K = d_model; g.pair = 1; g.half = 0; g.ctas = n_qkv; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(mask);
-                x_ready();
                 const unsigned vseq = bar_no + 1;
                 if (ROLE == 2) {
                     constexpr int HALF = HD / 2, KSQ = HD / 16;
@@ -1963,8 +2010,8 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                             }
                         }
                     });
-                } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_a, ntd, d_model, c.eps, vseq); });
-                else gemm_phase<ROLE, 1>(S, g, r, pol, NoEpi());
+                } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_a, ntd, d_model, c.eps, vseq); }, x_ready);
+                else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
                 phase_barrier(2);
             }
             // ---- attention (work items that hold no row of this pass are fetched before the QKV phase has ended)
@@ -1973,14 +2020,13 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 else attn_produce(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
             }
             if (ROLE == 2) {
-                if (attn_items(A, d, mask) <= G) attn_consume_single<HD>(A, S, d, l, mask, r);
+                if (attn_items(A, d, mask) <= G) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
                 else attn_consume<HD>(A, S, d, l, mask, r);
             }
             phase_barrier(4);
             // ---- O projection + residual; prepares the FFN input
             {
                 Gemm g; g.W = ly.wo; g.X = reinterpret_cast<const uint4 *>(A.XO); g.N = d_model; g.K = qd; g.pair = 1; g.half = 0; g.ctas = n_d; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(mask);
-                x_ready();
                 if (ROLE == 2) {
                     const __nv_bfloat16 *gain = ly.ffn_norm;
                     uint32_t *stash = stash_of(sm);
@@ -2015,7 +2061,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                             if (lane < 4 && ((mask >> (c0 + q)) & 1u)) A.ssq_b[(size_t)tile * MAX_COLS + c0 + q] = sq[q];
                         }
                     });
-                } else gemm_phase<ROLE, 1>(S, g, r, pol, NoEpi());
+                } else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
                 phase_barrier(5);
             }
             // ---- gate / up + SwiGLU
@@ -2024,7 +2070,6 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 // the one GEMM of the layer where the unit-balanced split pays (measured: it shortens gate-up by 1.4 us,
                 // but lengthens down, QKV and O, whose tile groups are k-split among the warps)
                 g.part = A.part; g.phase_id = bar_no + 1; g.columns(mask);
-                x_ready();
                 const unsigned vseq = bar_no + 1;
                 if (ROLE == 2) {
                     const int c0 = 2 * (lane & 3);
@@ -2042,14 +2087,13 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                             }
                         }
                     });
-                } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_b, ntd, d_model, c.eps, vseq); });
-                else gemm_phase<ROLE, 2>(S, g, r, pol, NoEpi());
+                } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_b, ntd, d_model, c.eps, vseq); }, x_ready);
+                else gemm_phase<ROLE, 2>(S, g, r, pol, x_ready, NoEpi());
                 phase_barrier(6);
             }
             // ---- down projection + residual; prepares the next layer's (and the head's) input
             {
                 Gemm g; g.W = ly.wdown; g.X = reinterpret_cast<const uint4 *>(A.XH); g.N = d_model; g.K = c.dff; g.pair = 1; g.half = 0; g.ctas = n_d; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(mask);
-                x_ready();
                 if (ROLE == 2) {
                     const __nv_bfloat16 *gain_next = l + 1 < L ? M.layer[l + 1].attn_norm : nullptr;
                     const bool want_f = l + 1 == L || A.exit_at[l + 1] != 0;
@@ -2091,7 +2135,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                             if (lane < 4 && ((mask >> (c0 + q)) & 1u)) A.ssq_a[(size_t)tile * MAX_COLS + c0 + q] = sq[q];
                         }
                     });
-                } else gemm_phase<ROLE, 1>(S, g, r, pol, NoEpi());
+                } else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
                 phase_barrier(8);
             }
             // ---- intermediate head (Section 2.1) and the early-prediction rule (Eq. 1)
@@ -2100,7 +2144,6 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 const MegaLayer &hl = M.layer[l + 1];
                 if (hl.wT) {
                     Gemm g; g.W = hl.wT; g.X = reinterpret_cast<const uint4 *>(A.XF); g.N = d_model; g.K = d_model; g.pair = 1; g.half = 0; g.ctas = n_d; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(hcols);
-                    x_ready();
                     const unsigned vseq = bar_no + 1;
                     if (ROLE == 2) {
                         const int c0 = 2 * (lane & 3);
@@ -2114,8 +2157,8 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                                 xfrag_store(A.XT, n, cc, acc[0][i] * ((i & 1) ? r1 : r0));
                             }
                         });
-                    } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_a, ntd, d_model, c.eps, vseq); });
-                    else gemm_phase<ROLE, 1>(S, g, r, pol, NoEpi());
+                    } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_a, ntd, d_model, c.eps, vseq); }, x_ready);
+                    else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
                     phase_barrier(10);
                     head_phase(A.XT, nullptr, hl.head_scale, hcols, true);
                 } else {

@@ -286,6 +286,13 @@ __device__ __forceinline__ void xfrag_store(__nv_bfloat16 *X, int k, int col, fl
     X[i] = hi;
     X[i + 4] = lo;
 }
+// two neighbouring elements k (even), k + 1
+__device__ __forceinline__ void xfrag_store2(__nv_bfloat16 *X, int k, int col, float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    const size_t i = xfrag_index(k, col);
+    *reinterpret_cast<__nv_bfloat162 *>(X + i) = h;
+    *reinterpret_cast<__nv_bfloat162 *>(X + i + 4) = __floats2bfloat162_rn(a - __low2float(h), b - __high2float(h));
+}
 __host__ __device__ inline size_t xfrag_bytes(int K) { return (size_t)((K + KC - 1) / KC) * X_STAGE; }
 
 // ---------------------------------------------------------------- GEMM phase
@@ -446,8 +453,10 @@ __device__ __forceinline__ void gemm_produce_w(const Shared &S, const Gemm &g, i
 // Activation producer warp: one stage per (tile group, k chunk).
 // `after_first` runs once, after the first stage has been issued: work of the phase that is not
 // needed before the epilogues (the normalisation factors) and must not delay the first copy.
-template <class Hook>
-__device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, int cta, int G, Rings &r, uint64_t pol, Hook &&after_first) {
+// `ready` runs once, immediately before the first copy: it waits until the input is complete (the division of the work is
+// worked out before that wait, not after it).
+template <class Hook, class Ready>
+__device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, int cta, int G, Rings &r, uint64_t pol, Hook &&after_first, Ready &&ready) {
     Smem *sm = S.sm;
     const int lane = threadIdx.x & 31;
     const Plan pl = make_plan(g, cta, G);
@@ -460,6 +469,7 @@ __device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, i
             const int nc = min(XC, nch - kc);
             const int slot = r.xi % NX;
             mbar_wait(S, &sm->x_empty[slot], ((r.xi / NX) & 1) ^ 1);
+            if (!hooked) ready();
             if (lane == 0 && !aborted(S)) {
                 const uint32_t bytes = (uint32_t)g.ncp * 4096u;
                 mbar_expect_tx(&sm->x_full[slot], bytes * nc);
@@ -471,13 +481,13 @@ __device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, i
             if (!hooked) { after_first(); hooked = true; }
         }
     }
-    if (!hooked) after_first();
+    if (!hooked) { ready(); after_first(); }
 }
 struct NoHook {
     __device__ __forceinline__ void operator()() const {}
 };
 __device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, int cta, int G, Rings &r, uint64_t pol) {
-    gemm_produce_x(S, g, cta, G, r, pol, NoHook());
+    gemm_produce_x(S, g, cta, G, r, pol, NoHook(), NoHook());
 }
 
 // The k-steps ks_id + KS_ j (j < 32 / KS_) of one full weight stage: fragment loads run PF steps
