@@ -1398,7 +1398,8 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
     // Prompts of some length take the dense pass: blocks of up to dg::PF_ROWS positions through the tcgen05 products.  The
     // decode path takes eight positions a pass; measured, one / two passes against the dense pass: 1B 1.06 / 1.96 against
     // 1.69 ms, 8B 3.5 / 6.8 against 5.4, 13B 5.4 / 10.7 against 8.0.
-    const bool dense = S->dense_ok && S->prefill_dense && n_prompt >= kDenseMin;
+    // (Three q heads per kv head: the dense pass refuses, as it always has; shorter prompts of such models keep the decode path.)
+    const bool dense = S->dense_ok && S->prefill_dense && n_prompt >= (g.n_q_heads / g.n_kv_heads == 3 ? 32 : kDenseMin);
     if (!dense && S->mega && S->path == 1) {
         // prompt passes of eight positions through the persistent kernel
         mg::k_prefill_arm<<<1, 32, 0, S->stream>>>(S->c, seq, n_prompt);

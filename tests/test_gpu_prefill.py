@@ -79,3 +79,14 @@ def test_separate_and_fused_tensors_give_the_same_cache():
         S.prefill(prompt)
         rows.append(np.stack([S.read_kv(wh, l, p) for wh in (0, 1) for l in range(cfg.n_layers) for p in (0, 100, 199)]))
     assert np.array_equal(rows[0], rows[1])
+
+
+def test_three_q_heads_per_kv_head_keep_the_decode_path():
+    """The dense pass has no form for them: prompts below 32 tokens are accepted, longer ones refused, as before."""
+    cfg, gm = _model(64, 6, 2)
+    S = binding.Session(gm, 1, 128, 64, 0)
+    S.prefill(synth.make_prompt(cfg, n=20).numpy())
+    assert S.state()[0] == 21
+    with pytest.raises(binding.AdaError) as e:
+        S.prefill(synth.make_prompt(cfg, n=40).numpy())
+    assert e.value.code == -6
