@@ -33,6 +33,7 @@ EXPORTS = [
     "ada_debug_profile", "ada_debug_profile_read", "ada_debug_gemm", "ada_debug_gemm_plan", "ada_debug_gemm_work_bytes", "ada_debug_get_path", "ada_debug_set_launch_steps", "ada_debug_trace", "ada_gemm_noalloc",
     "ada_model_arena_bytes", "ada_model_set_arena", "ada_debug_set_wait_limit", "ada_debug_set_prefill",
     "ada_debug_dense_gemm", "ada_debug_dense_gemm_work_bytes", "ada_sampling_decode",
+    "ada_debug_dense_plan",
 ]
 
 
@@ -97,6 +98,7 @@ def load() -> C.CDLL:
         L.ada_debug_dense_gemm_work_bytes.restype = sz
         L.ada_debug_dense_gemm_work_bytes.argtypes = [i32]
         L.ada_debug_dense_gemm.argtypes = [vp, i32, i32, vp, i32, vp, i32, i32, vp, sz, vp]
+        L.ada_debug_dense_plan.argtypes = [i32, i32, i32, i32, i32, i32, C.POINTER(i32), vp, i32, C.POINTER(i32)]
         L.ada_model_destroy.argtypes = [vp]
         L.ada_model_destroy.restype = None
         L.ada_session_scratch_bytes.restype = sz
@@ -143,6 +145,14 @@ def debug_gemm_plan(N: int, K: int, mode: int, grid: int, cta: int, split: bool 
     _ck(load().ada_debug_gemm_plan(N, K, mode, grid, cta, 1 if split else 0, out), "ada_debug_gemm_plan")
     keys = ("split", "t0", "t1", "n", "ta", "tb", "s0_own_k0", "s0_pub_k1", "sl_k1")
     return dict(zip(keys, list(out)))
+
+
+def debug_dense_plan(rows: int, N: int, per_tile: int, K: int, pairs: int, pair: int):
+    """ada_debug_dense_plan: (plan, segments (tile, first chunk, end chunk) of pair `pair`) of a dense product (host only, no GPU)."""
+    plan, n = (C.c_int32 * 6)(), C.c_int32(0)
+    segs = np.zeros((4096, 3), dtype=np.int32)
+    _ck(load().ada_debug_dense_plan(rows, N, per_tile, K, pairs, pair, plan, segs.ctypes.data, len(segs), C.byref(n)), "ada_debug_dense_plan")
+    return dict(zip(("nt", "mt", "tiles", "chunks", "groups", "pairs"), list(plan))), segs[:n.value].tolist()
 
 
 def debug_gemm(W, X, mode: int = 0, repeat: int = 1):

@@ -216,7 +216,7 @@ int rows_alloc_for(const ada_config &g, int batch, int max_early) {
 // positions of one block of a dense prompt pass: a prompt is cut alike whatever the session's length limit
 int pf_rows_for(int max_seq) { return std::min(dg::PF_ROWS, (int)align_up((size_t)max_seq, 128)); }
 constexpr int kDenseMin = 9;        // prompt tokens from which the dense pass is taken
-constexpr int kGemmMaxPairs = 80;   // CTA pairs the exchange area of cut tiles is laid out for
+constexpr int kGemmMaxPairs = 76;   // CTA pairs the exchange area of cut tiles is laid out for
 
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
@@ -366,33 +366,58 @@ int position_tile(int rows) {
     return (per + 31) / 32 * 32;
 }
 
+// What a division of the shared tiles by whole groups over p pairs costs: chunks of the busiest pair, pieces of the tile cut
+// into most.  False: some pair would hold two groups or more from the middle of a tile (see the kernel: it publishes one).
+bool cut_by_groups(const dg::GemmPlan &g, int p, int *chunks_max, int *pieces_max) {
+    *chunks_max = *pieces_max = 0;
+    int pieces = 0;
+    for (int i = 0; i < p; ++i) {
+        int u = (int)((long long)g.sk_tiles * g.groups * i / p), n = 0;
+        const int end = (int)((long long)g.sk_tiles * g.groups * (i + 1) / p);
+        while (u < end) {
+            const int a = u % g.groups, b = std::min(g.groups, a + end - u);
+            if (a > 0 && b < g.groups && b - a > 1) return false;
+            pieces = a == 0 ? 1 : pieces + 1;
+            *pieces_max = std::max(*pieces_max, pieces);
+            n += dg::group_begin(g, b) - dg::group_begin(g, a);
+            u += b - a;
+        }
+        *chunks_max = std::max(*chunks_max, n);
+    }
+    return true;
+}
+
 // How a product of N weight rows (`per_tile` of them to a tile) and depth K over `rows` positions is divided over at most
-// `pairs` CTA pairs.  More tiles than pairs: whole waves, then one wave's worth of tiles and the remainder cut by
-// chunks so that all pairs end together (cutting the remainder alone would cut a tile into more pieces, each of which
-// costs an exchange).  Fewer: all tiles cut over the number of pairs that minimises, in cycles, the chunks of the busiest
-// pair (8192 of the tensor core at full width; not below the 5600 that a chunk's weights take to arrive at a pair's share
-// of HBM bandwidth) plus the exchange of the pieces (3300 cycles per further piece of full width, 3000 to begin with).
+// `pairs` CTA pairs.  The number of groups of a tile's depth does not depend on `rows` (the order of the sums follows from
+// it): as many as the pairs that one position tile leaves for each of its tiles.  More tiles than pairs: whole waves, then
+// one wave's worth of tiles and the remainder cut by chunks so that all pairs end together (cutting the remainder alone would
+// cut a tile into more pieces, each of which costs an exchange).  Fewer: all tiles cut by groups over the number of pairs
+// that minimises, in cycles, the chunks of the busiest pair (8192 of the tensor core at full width; not below the 5600 that
+// a chunk's weights take to arrive at a pair's share of HBM bandwidth) plus the exchange of the pieces (3300 cycles per
+// further piece of full width, 3000 to begin with).
 dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
     dg::GemmPlan g{};
+    const int across = (N + per_tile - 1) / per_tile;
     g.nt = position_tile(rows);
     g.mt = (rows + g.nt - 1) / g.nt;
-    g.tiles = g.mt * ((N + per_tile - 1) / per_tile);
+    g.tiles = g.mt * across;
     g.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
+    g.groups = std::max(1, std::min({pairs / across, g.chunks, dg::MAX_GROUPS}));
     if (g.tiles >= pairs) {
         g.pairs = pairs;
         if (g.tiles % pairs) { g.sk_tiles = g.tiles % pairs + pairs; g.sk_pairs = pairs; }
         return g;
     }
-    const int units = g.tiles * g.chunks;
+    g.sk_tiles = g.tiles;
+    g.by_group = 1;
     const double width = (double)g.nt / dg::NT_MAX, chunk = std::max(8192.0 * width, 5600.0);
     double best = 0;
-    for (int p = g.tiles; p <= std::min(pairs, units); ++p) {
-        const int per = units / p;
-        const int pieces = p == g.tiles ? 0 : (g.chunks + per - 1) / per;
-        const double cost = chunk * ((units + p - 1) / p) + 3300.0 * pieces * width + (pieces ? 3000.0 : 0.0);
+    for (int p = g.tiles; p <= std::min(pairs, g.tiles * g.groups); ++p) {
+        int most, pieces;
+        if (!cut_by_groups(g, p, &most, &pieces)) continue;
+        const double cost = chunk * most + (pieces > 1 ? 3300.0 * pieces * width + 3000.0 : 0.0);
         if (!g.pairs || cost < best) { best = cost; g.pairs = p; }
     }
-    g.sk_tiles = g.tiles;
     g.sk_pairs = g.pairs;
     return g;
 }
@@ -408,7 +433,8 @@ template <int EPI, int HD> cudaError_t prepare_dense() {
 
 // Tensor maps of the inputs of a block's products (they end at the block's last row: rows behind it read as zero): high and
 // low parts of the normalised residual, the queries, the attention result, the FFN activations.
-struct PfMaps { CUtensorMap xh, xl, qh, ql, oh, ol, hh, hl; };
+// Also how each of the products is divided.
+struct PfMaps { CUtensorMap xh, xl, qh, ql, oh, ol, hh, hl; dg::GemmPlan qkv, o, gate_up, down; };
 
 template <int HD, int GROUP>
 int launch_attn_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int pos0, int rows, __nv_bfloat16 *oh, __nv_bfloat16 *ol) {
@@ -439,14 +465,11 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
         Prof pf(S, 1, 0.0);
         return launch_overlapped(S->stream, dg::k_norm_split_rows, rows, 256, 0, S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl);
     };
-    auto shape = [&](int N, int per_tile, int K) {
-        a.N = N; a.K = K; a.epoch = ++S->pf_epoch;
-        a.plan = plan_dense(rows, N, per_tile, K, S->pf_pairs);
-    };
+    auto shape = [&](int N, int K, const dg::GemmPlan &plan) { a.N = N; a.K = K; a.epoch = ++S->pf_epoch; a.plan = plan; };
     if ((rc = norm(w.attn_norm))) return rc;
     {
         Prof pf(S, 2, (double)qkv * d * 2);
-        shape(qkv, dg::TW, d);
+        shape(qkv, d, pm.qkv);
         a.hi = qh; a.lo = ql;
         rc = hd == 128 ? launch_dense<dg::EPI_QKV, 128>(S->stream, pm.xh, pm.xl, wm[0], wm[0], S->c, a)
                        : launch_dense<dg::EPI_QKV, 64>(S->stream, pm.xh, pm.xl, wm[0], wm[0], S->c, a);
@@ -462,19 +485,19 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     }
     {
         Prof pf(S, 5, (double)d * qd * 2);
-        shape(d, dg::TW, qd);
+        shape(d, qd, pm.o);
         if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.oh, pm.ol, wm[1], wm[1], S->c, a))) return rc;
     }
     if ((rc = norm(w.ffn_norm))) return rc;
     {
         Prof pf(S, 6, (double)2 * g.d_ff * d * 2);
-        shape(g.d_ff, dg::BW, d);
+        shape(g.d_ff, d, pm.gate_up);
         a.hi = hh; a.lo = hl;
         if ((rc = launch_dense<dg::EPI_SWIGLU, 0>(S->stream, pm.xh, pm.xl, wm[2], wm[3], S->c, a))) return rc;
     }
     {
         Prof pf(S, 8, (double)d * g.d_ff * 2);
-        shape(d, dg::TW, g.d_ff);
+        shape(d, g.d_ff, pm.down);
         if ((rc = launch_dense<dg::EPI_ADD, 0>(S->stream, pm.hh, pm.hl, wm[4], wm[4], S->c, a))) return rc;
     }
     return ADA_OK;
@@ -652,6 +675,10 @@ int prefill_dense(ada_session *S, int seq, int n_prompt) {
         PfMaps pm;
         const int group = g.n_q_heads / g.n_kv_heads;
         if (group != 1 && group != 2 && group != 4) return ADA_EUNSUPPORTED;
+        pm.qkv = plan_dense(n, S->c.qkv_rows, dg::TW, d, S->pf_pairs);
+        pm.o = plan_dense(n, d, dg::TW, qd, S->pf_pairs);
+        pm.gate_up = plan_dense(n, g.d_ff, dg::BW, d, S->pf_pairs);
+        pm.down = plan_dense(n, d, dg::TW, g.d_ff, S->pf_pairs);
         // a product's position tiles are the same for every layer; one box is what one CTA of a pair holds of a tile
         const int bx = position_tile(n) / 2;
         if ((rc = make_map_q(&pm.qh, S->pf_u, n, g.n_q_heads, g.head_dim, group)) || (rc = make_map_q(&pm.ql, S->pf_u + P * qd, n, g.n_q_heads, g.head_dim, group)) ||
@@ -1672,6 +1699,24 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     return herr ? ADA_ETIMEOUT : ADA_OK;
 }
 
+int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan6,
+                         int32_t *segs_host, int32_t max_segs, int32_t *n_segs) {
+    if (!plan6 || !segs_host || !n_segs || max_segs < 1 || rows < 1 || rows > dg::PF_ROWS || N < 1 || K < 64 || K % 64) return ADA_EINVAL;
+    if ((per_tile != dg::TW && per_tile != dg::BW) || pairs < 1 || pairs > kGemmMaxPairs || pair < 0 || pair >= pairs) return ADA_EINVAL;
+    const dg::GemmPlan g = plan_dense(rows, N, per_tile, K, pairs);
+    const int32_t v[6] = {g.nt, g.mt, g.tiles, g.chunks, g.groups, g.pairs};
+    memcpy(plan6, v, sizeof(v));
+    *n_segs = 0;
+    if (pair >= g.pairs) return ADA_OK;
+    dg::Sched sch(g, pair);
+    for (dg::Seg s; sch.next(s); ++*n_segs) {
+        if (*n_segs == max_segs) return ADA_ECAPACITY;
+        int32_t *o = segs_host + 3 * *n_segs;
+        o[0] = s.tile; o[1] = s.c0; o[2] = s.c1;
+    }
+    return ADA_OK;
+}
+
 constexpr int kDenseDebugRows = 128;   // most rows of ada_debug_dense_gemm
 
 size_t ada_debug_dense_gemm_work_bytes(int32_t K) {
@@ -1704,7 +1749,7 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     CK(cudaGetLastError());
     dg::GemmArgs a{};
     a.rows = rows; a.N = N; a.K = K; a.Y = Y_dev; a.ldy = ldy; a.err = err;
-    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = (N + dg::TW - 1) / dg::TW; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
+    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = (N + dg::TW - 1) / dg::TW; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK; a.plan.groups = 1;
     a.plan.pairs = std::max(1, std::min(a.plan.tiles, sms / 2));   // whole tiles: no exchange area needed
     const Ctx none{};
     rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, none, a);

@@ -21,11 +21,22 @@
 // into chunks of 512 k; a chunk accumulates in one of two 256-column tensor-memory buffers while the epilogue warps
 // add the other one, already complete, to fp32 registers (round to nearest).  Each buffer sees 64 additions.
 //
-// Work division.  Tiles in excess of whole waves over the CTA pairs are divided by chunks, not by tiles
-// ("stream-K"): every pair gets the same number of chunks (+- 1).  A tile cut between pairs is summed by the pair
-// that holds its last chunk, in a fixed order; the others publish their partial sums first thing in the kernel, and
-// a pair only ever waits for pairs with a lower number, so no assumption about co-residency is made.  With whole
-// tiles a 1024-position block of the 8B shape would fill 83 % of its waves, a 500-position one 60 %.
+// Order of the sums.  It is a function of N, K and the device alone, so that the cache rows of a prompt's prefix have the
+// same bits whatever follows the prefix.  The chunks of a tile form 1 to 4 groups (group_begin; as many as one position
+// tile has pairs to spare for, so that short prompts can use them side by side).  A group is summed from zero in the order
+// of its chunks, the groups are then added in their order: ((g0 + g1) + g2) + g3.  A pair that holds several groups of a
+// tile keeps the running total in scratch while it sums the next group (there are registers for one set of sums); that
+// traffic runs under the tensor core's next chunk.
+//
+// Work division.  A tile may be cut between pairs (GemmPlan, plan_dense):
+//   * with more tiles than pairs, tiles in excess of whole waves are divided by chunks ("stream-K"), every pair getting the
+//     same number (+- 1), at least a tile's worth.  A tile then has at most two pieces, and the pair with the second one
+//     goes on from the total and the unfinished group of the first;
+//   * with fewer, between groups only.  Every piece starts its group from zero; the pair that holds the last group adds
+//     the other pairs' sums before its own.
+// What another pair waits for is computed first thing in the kernel, and a pair only ever waits for pairs with a lower
+// number, so no assumption about co-residency is made.  With whole tiles a 1024-position block of the 8B shape would fill
+// 83 % of its waves, a 500-position one 60 %.
 //
 // Roles of a CTA: warp 0 issues the TMA loads, warp 1 allocates the tensor memory and (in the first CTA of the pair)
 // issues the MMAs, warps 4..11 read the accumulators and run the epilogue.  Every wait is bounded; on expiry an
@@ -57,8 +68,12 @@ constexpr int W_BYTES = BW * BK * 2;
 constexpr int RING_BYTES = 196608;
 constexpr int TMEM_COLS = 512; // two accumulator buffers of 256 fp32 columns
 constexpr unsigned long long DENSE_WAIT_NS = 2000000000ull;
-constexpr size_t GPART_WARP = 128 * 32 * sizeof(float);           // partial sums of one epilogue warp
-constexpr size_t GPART_CTA = GEPI_WARPS * GPART_WARP;
+constexpr int MAX_GROUPS = 4;
+constexpr size_t GPART_WARP = 128 * 32 * sizeof(float);           // sums of one epilogue warp
+constexpr size_t GPART_SLOT = GEPI_WARPS * GPART_WARP;
+// per CTA: what it publishes (the total of whole groups; the unfinished group), and the running total of a tile it keeps
+constexpr int SLOT_TOTAL = 0, SLOT_GROUP = 1, SLOT_OWN = 2;
+constexpr size_t GPART_CTA = 3 * GPART_SLOT;
 
 struct DSmem {   // must start on a 1024-byte boundary (swizzle pattern)
     // stages of [W 128 x 64 (SwiGLU: 16 rows of gate, 16 of up, ...) | X.hi NT / 2 x 64 | X.lo NT / 2 x 64], rows of 128 B: as many as fit
@@ -199,15 +214,21 @@ template <typename SM> __device__ __forceinline__ bool dwait(SM *sm, int *err, u
 
 // Division of one product's tiles over the CTA pairs (chosen on the host, plan_dense).  Tiles are numbered with the
 // position tile fastest, so that the pairs at work at one time share weight rows.  The last sk_tiles tiles are divided
-// by chunks over sk_pairs pairs, the others are dealt out whole.
-struct GemmPlan { int nt, mt, tiles, chunks, pairs, sk_tiles, sk_pairs; };   // nt positions per tile, mt position tiles
+// over sk_pairs pairs, by chunks or (by_group) by whole groups, the others are dealt out whole.
+struct GemmPlan { int nt, mt, tiles, chunks, groups, pairs, sk_tiles, sk_pairs, by_group; };   // nt positions per tile, mt position tiles
+__host__ __device__ __forceinline__ int group_begin(const GemmPlan &g, int i) { return i * g.chunks / g.groups; }   // first chunk of group i
 
 struct Seg { int tile, c0, c1; };   // chunks [c0, c1) of a tile
 struct Sched {
     GemmPlan g;
     int pair, t_last, t_first, u_end, u_beg, i, phase;   // phase 0: last shared tile, 1: the whole ones between, 2: whole tiles, 3: first shared tile, 4: end
-    __device__ __forceinline__ int unit(int p) const { return (int)((long long)g.sk_tiles * g.chunks * p / g.sk_pairs); }
-    __device__ __forceinline__ Sched(const GemmPlan &g_, int pair_) : g(g_), pair(pair_), t_last(0), t_first(0), u_end(0), u_beg(0), i(0), phase(2) {
+    // first chunk of pair p's share, counted over the shared tiles
+    __host__ __device__ __forceinline__ int unit(int p) const {
+        if (!g.by_group) return (int)((long long)g.sk_tiles * g.chunks * p / g.sk_pairs);
+        const int u = (int)((long long)g.sk_tiles * g.groups * p / g.sk_pairs), t = u / g.groups;
+        return t * g.chunks + group_begin(g, u - t * g.groups);
+    }
+    __host__ __device__ __forceinline__ Sched(const GemmPlan &g_, int pair_) : g(g_), pair(pair_), t_last(0), t_first(0), u_end(0), u_beg(0), i(0), phase(2) {
         if (g.sk_tiles > 0 && pair < g.sk_pairs) {
             u_beg = unit(pair);
             u_end = unit(pair + 1);
@@ -220,7 +241,7 @@ struct Sched {
         if (phase == 2) i = pair;
     }
     // Pieces another pair waits for come first, the piece that waits for others comes last.
-    __device__ __forceinline__ bool next(Seg &s) {
+    __host__ __device__ __forceinline__ bool next(Seg &s) {
         const int base = g.tiles - g.sk_tiles;
         if (phase == 0) {
             phase = 1;
@@ -273,8 +294,8 @@ struct GemmArgs {
     __nv_bfloat16 *hi, *lo;       // QKV: scaled queries [rows][q features]; SwiGLU: activations [rows][N]
     const float *cs;              // QKV: cos, sin [rows][hd / 2][2]
     int layer, seq, pos0;         // QKV: rows are positions pos0 .. of sequence seq
-    float *part;                  // partial sums of tiles cut between pairs
-    unsigned *flag;               // [CTA][epilogue warp]: launch number of the partial sums published last
+    float *part;                  // [CTA][slot]: sums of tiles cut between pairs, running totals (null: one group, nothing cut)
+    unsigned *flag;               // [CTA][epilogue warp]: launch number of the sums published last
     unsigned epoch;
     int *err;
 };
@@ -305,6 +326,39 @@ template <class Body> __device__ __forceinline__ void epi_rounds(const float (&a
         body(32 * g, min(32, left - 32 * g));
     }
 }
+
+// One set of sums of an epilogue warp in scratch: 16 bytes of every lane side by side.
+__device__ __forceinline__ void sums_store(const float (&acc)[128], float4 *o, int nh) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+        if (4 * j < nh) __stcg(o + 32 * j, make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]));
+}
+// acc = ((src[0] + src[1]) + src[2]) + acc over N sources, W 16-byte loads of each in flight (more would not fit beside the sums).
+template <int N, int W> __device__ __forceinline__ void sums_add_n(float (&acc)[128], const float4 *const (&src)[MAX_GROUPS - 1], int nh) {
+#pragma unroll
+    for (int j0 = 0; j0 < 32; j0 += W) {
+        if (4 * j0 >= nh) break;
+        float4 r[N][W];
+#pragma unroll
+        for (int s = 0; s < N; ++s)
+#pragma unroll
+            for (int j = 0; j < W; ++j) r[s][j] = 4 * (j0 + j) < nh ? ld_cg_inorder(src[s] + 32 * (j0 + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const int e = 4 * (j0 + j);
+            float4 t = r[0][j];
+#pragma unroll
+            for (int s = 1; s < N; ++s) { t.x += r[s][j].x; t.y += r[s][j].y; t.z += r[s][j].z; t.w += r[s][j].w; }
+            acc[e] += t.x; acc[e + 1] += t.y; acc[e + 2] += t.z; acc[e + 3] += t.w;
+        }
+    }
+}
+__device__ __forceinline__ void sums_add(float (&acc)[128], const float4 *const (&src)[MAX_GROUPS - 1], int n, int nh) {
+    if (n == 1) sums_add_n<1, 16>(acc, src, nh);
+    else if (n == 2) sums_add_n<2, 8>(acc, src, nh);
+    else sums_add_n<3, 4>(acc, src, nh);
+}
+static_assert(MAX_GROUPS == 4, "sums_add takes up to three sources");
 
 // Y[m][n] = or += x: four neighbouring n per lane, four positions per access.  N arbitrary, ldy a multiple of 4.
 template <bool ADD> __device__ __forceinline__ void epi_rows(const float (*x)[32], float *y, int ldy, int n_left, int lane, int left) {
@@ -401,6 +455,26 @@ __device__ __forceinline__ void epi_swiglu(const float (*x)[32], __nv_bfloat16 *
             *reinterpret_cast<uint32_t *>(lo + (size_t)j * ld + n) = l[i];
         }
     }
+}
+
+// Waits until the epilogue warp ew of a CTA has published its sums of this launch (whole warp).
+template <typename SM> __device__ __forceinline__ bool flag_wait(SM *sm, const GemmArgs &a, int cta, int ew) {
+    const unsigned *f = a.flag + cta * GEPI_WARPS + ew;
+    const unsigned long long t0 = gtime();
+    bool ok = true;
+    for (;;) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+        if (v == a.epoch) break;
+        if (*(volatile int *)&sm->abort) { ok = false; break; }
+        if (gtime() - t0 > DENSE_WAIT_NS) {
+            atomicCAS(a.err, 0, ERR_TIMEOUT_MBAR);
+            *(volatile int *)&sm->abort = 1;
+            ok = false;
+            break;
+        }
+    }
+    return __all_sync(0xffffffffu, ok);
 }
 
 // mapXhi / mapXlo: 2-D maps over the bf16 matrices [rows][K] (box 64 x plan.nt / 2); mapW0, mapW1: over the weight matrices
@@ -535,7 +609,26 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
             float acc[128];
 #pragma unroll
             for (int j = 0; j < 128; ++j) acc[j] = 0.f;
-            for (int cc = s.c0; cc < s.c1; ++cc, ++ch) {
+            const int chunks = a.plan.chunks, first = s.c0, end = s.c1;
+            const bool last = end == chunks;                 // this pair finishes the tile
+            const bool middle = first > 0 && !last;          // one group, published by itself
+            int grp = 0;
+            while (group_begin(a.plan, grp + 1) <= first) ++grp;
+            int grp_end = group_begin(a.plan, grp + 1);
+            bool own_total = false;                          // the total of the groups before this one is in this CTA's scratch
+            auto slot = [&](int cta, int which) {
+                return reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a.part) + (size_t)cta * GPART_CTA + which * GPART_SLOT + ew * GPART_WARP) + lane;
+            };
+            const int cta = 2 * pair + (int)rank;
+            const float4 *src[MAX_GROUPS - 1] = {nullptr, nullptr, nullptr};
+            if (live && first > group_begin(a.plan, grp)) {  // the group was begun by the pair before this one
+                ok = flag_wait(sm, a, cta - 2, ew);
+                if (ok) {
+                    src[0] = slot(cta - 2, SLOT_GROUP);
+                    sums_add(acc, src, 1, nh);
+                }
+            }
+            for (int cc = first; ok && cc < end; ++cc, ++ch) {
                 const int b = ch & 1;
                 ok = dwait(sm, a.err, &sm->acc_full[b], (ch >> 1) & 1);
                 ok = __all_sync(0xffffffffu, ok);
@@ -556,54 +649,42 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(map_to_cta(&sm->acc_empty[b], 0));
+                if (cc + 1 < grp_end) continue;
+                // a group is complete
+                if (live && grp > 0 && !middle) {   // add it to the total of those before it
+                    int n = 1;
+                    if (own_total) src[0] = slot(cta, last ? SLOT_OWN : SLOT_TOTAL);
+                    else {                          // other pairs': the tile's pieces in their order
+                        const int u0 = (s.tile - (a.plan.tiles - a.plan.sk_tiles)) * chunks;
+                        int p0 = pair - 1;
+                        while (p0 > 0 && sch.unit(p0) > u0) --p0;
+                        n = pair - p0;
+#pragma unroll
+                        for (int i = 0; i < MAX_GROUPS - 1; ++i)
+                            if (ok && i < n) {
+                                ok = flag_wait(sm, a, 2 * (p0 + i) + (int)rank, ew);
+                                src[i] = slot(2 * (p0 + i) + (int)rank, SLOT_TOTAL);
+                            }
+                        if (!ok) break;
+                    }
+                    sums_add(acc, src, n, nh);
+                }
+                ++grp;
+                grp_end = group_begin(a.plan, grp + 1);
+                if (live && cc + 1 < end) {
+                    sums_store(acc, slot(cta, last ? SLOT_OWN : SLOT_TOTAL), nh);
+                    own_total = true;
+#pragma unroll
+                    for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+                }
             }
             if (!ok || !live) continue;
-            if (s.c1 < a.plan.chunks) {   // another pair finishes this tile
-                float4 *o = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a.part) + (size_t)(2 * pair + (int)rank) * GPART_CTA + ew * GPART_WARP) + lane;
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (4 * j < nh) __stcg(o + 32 * j, make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]));
+            if (!last) {   // another pair finishes this tile
+                sums_store(acc, slot(cta, end == group_begin(a.plan, grp) ? SLOT_TOTAL : SLOT_GROUP), nh);
                 __threadfence();
                 __syncwarp();
-                if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.flag + (2 * pair + (int)rank) * GEPI_WARPS + ew), "r"(a.epoch) : "memory");
+                if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.flag + cta * GEPI_WARPS + ew), "r"(a.epoch) : "memory");
                 continue;
-            }
-            if (s.c0 > 0) {   // add what the pairs before this one computed of the tile: nearest first
-                const int u0 = (s.tile - (a.plan.tiles - a.plan.sk_tiles)) * a.plan.chunks;
-                for (int p = pair - 1; ok && p >= 0 && sch.unit(p + 1) > u0; --p) {
-                    const int cta = 2 * p + (int)rank;
-                    const unsigned *f = a.flag + cta * GEPI_WARPS + ew;
-                    unsigned v;
-                    const unsigned long long t0 = gtime();
-                    for (;;) {
-                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-                        if (v == a.epoch) break;
-                        if (*(volatile int *)&sm->abort) { ok = false; break; }
-                        if (gtime() - t0 > DENSE_WAIT_NS) {
-                            atomicCAS(a.err, 0, ERR_TIMEOUT_MBAR);
-                            *(volatile int *)&sm->abort = 1;
-                            ok = false;
-                            break;
-                        }
-                    }
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                    const float4 *in = reinterpret_cast<const float4 *>(reinterpret_cast<const unsigned char *>(a.part) + (size_t)cta * GPART_CTA + ew * GPART_WARP) + lane;
-#pragma unroll
-                    for (int j0 = 0; j0 < 32; j0 += 16) {   // sixteen loads in flight: more would not fit beside the sums
-                        float4 r[16];
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (4 * (j0 + j) < nh) r[j] = ld_cg_inorder(in + 32 * (j0 + j));
-                            else r[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int e = 4 * (j0 + j);
-                            acc[e] += r[j].x; acc[e + 1] += r[j].y; acc[e + 2] += r[j].z; acc[e + 3] += r[j].w;
-                        }
-                    }
-                }
-                if (!ok) continue;
             }
             float(*x)[32] = sm->stash[ew];
             epi_rounds(acc, x, lane, left, [&](int j0, int cnt) {

@@ -90,3 +90,24 @@ def test_three_q_heads_per_kv_head_keep_the_decode_path():
     with pytest.raises(binding.AdaError) as e:
         S.prefill(synth.make_prompt(cfg, n=40).numpy())
     assert e.value.code == -6
+
+
+def _rows(S, cfg, positions):
+    return np.stack([S.read_kv(w, l, p) for l in range(cfg.n_layers) for p in positions for w in (0, 1)])
+
+
+@pytest.mark.parametrize("hd,nq,nkv,d,dff", [(64, 16, 4, 1024, 3072), (128, 16, 16, 2048, 5504)])
+def test_a_prefix_leaves_the_same_cache_bits_whatever_follows_it(hd, nq, nkv, d, dff):
+    """The order of every sum is that of the shapes, not of the prompt's length: prompts that start alike leave the same K
+    and V rows for what they share, whichever tiles, pieces and blocks the products were divided into."""
+    cfg, gm = _model(hd, nq, nkv, d, dff, layers=3)
+    prompt = synth.make_prompt(cfg, n=4200).numpy()
+    S = binding.Session(gm, 1, 4300, 64, 0)
+    seen = {}
+    for n in (9, 33, 70, 140, 257, 300, 520, 777, 1024, 1500, 2048, 2049, 4200):
+        S.prefill(prompt[:n])
+        for p in (0, 5, 8, 32, 60, 69, 128, 139, 256, 299, 500, 519, 776, 1023, 1400, 2047, 2048):
+            if p < n:
+                rows = _rows(S, cfg, [p])
+                first = seen.setdefault(p, (n, rows))
+                assert np.array_equal(first[1], rows), (p, first[0], n)
