@@ -216,7 +216,6 @@ int rows_alloc_for(const ada_config &g, int batch, int max_early) {
 // positions of one block of a dense prompt pass: a prompt is cut alike whatever the session's length limit
 int pf_rows_for(int max_seq) { return std::min(dg::PF_ROWS, (int)align_up((size_t)max_seq, 128)); }
 constexpr int kDenseMin = 9;        // prompt tokens from which the dense pass is taken
-constexpr int kGemmMaxPairs = 76;   // CTA pairs the exchange area of cut tiles is laid out for
 
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
@@ -261,8 +260,8 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.pf_u = take(sizeof(__nv_bfloat16) * P * std::max(4 * (size_t)qd, 2 * (size_t)g.d_ff));
         L.pf_cs = take(sizeof(float) * P * g.head_dim);
         L.pf_err = take(256);
-        L.pf_flag = take(sizeof(unsigned) * 2 * kGemmMaxPairs * dg::GEPI_WARPS);
-        L.pf_part = take(dg::GPART_CTA * 2 * kGemmMaxPairs);
+        L.pf_flag = take(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS);
+        L.pf_part = take(dg::GPART_CTA * 2 * dg::MAX_PAIRS);
     }
     // persistent-kernel buffers (bf16 models)
     if (g.dtype == ADA_DTYPE_BF16) {
@@ -366,20 +365,20 @@ int position_tile(int rows) {
     return (per + 31) / 32 * 32;
 }
 
-// What a division of the shared tiles by whole groups over p pairs costs: chunks of the busiest pair, pieces of the tile cut
-// into most.  False: some pair would hold two groups or more from the middle of a tile (see the kernel: it publishes one).
+// What a division of the tiles by whole groups over p pairs costs: chunks of the busiest pair, pieces of the tile cut into
+// most.  False: some pair would hold two groups or more from the middle of a tile (see the kernel: it publishes one).
 bool cut_by_groups(const dg::GemmPlan &g, int p, int *chunks_max, int *pieces_max) {
     *chunks_max = *pieces_max = 0;
     int pieces = 0;
     for (int i = 0; i < p; ++i) {
-        int u = (int)((long long)g.sk_tiles * g.groups * i / p), n = 0;
-        const int end = (int)((long long)g.sk_tiles * g.groups * (i + 1) / p);
+        int u = (int)((long long)g.tiles * g.groups * i / p), n = 0;
+        const int end = (int)((long long)g.tiles * g.groups * (i + 1) / p);
         while (u < end) {
             const int a = u % g.groups, b = std::min(g.groups, a + end - u);
             if (a > 0 && b < g.groups && b - a > 1) return false;
             pieces = a == 0 ? 1 : pieces + 1;
             *pieces_max = std::max(*pieces_max, pieces);
-            n += dg::group_begin(g, b) - dg::group_begin(g, a);
+            n += g.group[b] - g.group[a];
             u += b - a;
         }
         *chunks_max = std::max(*chunks_max, n);
@@ -403,13 +402,17 @@ dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
     g.tiles = g.mt * across;
     g.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
     g.groups = std::max(1, std::min({pairs / across, g.chunks, dg::MAX_GROUPS}));
+    for (int i = 0; i < dg::MAX_GROUPS + 2; ++i) g.group[i] = std::min(g.chunks, i * g.chunks / g.groups);
     if (g.tiles >= pairs) {
         g.pairs = pairs;
-        if (g.tiles % pairs) { g.sk_tiles = g.tiles % pairs + pairs; g.sk_pairs = pairs; }
+        const int shared = g.tiles % pairs ? g.tiles % pairs + pairs : 0;
+        g.whole = g.tiles - shared;
+        for (int p = 0; p <= pairs; ++p) {
+            const int u = (int)((long long)shared * g.chunks * p / pairs);
+            g.start[p] = u / g.chunks << 16 | u % g.chunks;
+        }
         return g;
     }
-    g.sk_tiles = g.tiles;
-    g.by_group = 1;
     const double width = (double)g.nt / dg::NT_MAX, chunk = std::max(8192.0 * width, 5600.0);
     double best = 0;
     for (int p = g.tiles; p <= std::min(pairs, g.tiles * g.groups); ++p) {
@@ -418,7 +421,10 @@ dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
         const double cost = chunk * most + (pieces > 1 ? 3300.0 * pieces * width + 3000.0 : 0.0);
         if (!g.pairs || cost < best) { best = cost; g.pairs = p; }
     }
-    g.sk_pairs = g.pairs;
+    for (int p = 0; p <= g.pairs; ++p) {
+        const int u = (int)((long long)g.tiles * g.groups * p / g.pairs);
+        g.start[p] = u / g.groups << 16 | g.group[u % g.groups];
+    }
     return g;
 }
 
@@ -1343,7 +1349,7 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
             prepare_attn<64, 2>() == cudaSuccess && prepare_attn<64, 4>() == cudaSuccess && prepare_attn<128, 1>() == cudaSuccess &&
             prepare_attn<128, 2>() == cudaSuccess && prepare_attn<128, 4>() == cudaSuccess) {
             S->dense_ok = true;
-            S->pf_pairs = std::min(sms / 2, kGemmMaxPairs);
+            S->pf_pairs = std::min(sms / 2, dg::MAX_PAIRS);
             S->pf_resid = (float *)(b + lay.pf_resid);
             S->pf_x = (__nv_bfloat16 *)(b + lay.pf_x);
             S->pf_u = (__nv_bfloat16 *)(b + lay.pf_u);
@@ -1702,7 +1708,7 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
 int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan6,
                          int32_t *segs_host, int32_t max_segs, int32_t *n_segs) {
     if (!plan6 || !segs_host || !n_segs || max_segs < 1 || rows < 1 || rows > dg::PF_ROWS || N < 1 || K < 64 || K % 64) return ADA_EINVAL;
-    if ((per_tile != dg::TW && per_tile != dg::BW) || pairs < 1 || pairs > kGemmMaxPairs || pair < 0 || pair >= pairs) return ADA_EINVAL;
+    if ((per_tile != dg::TW && per_tile != dg::BW) || pairs < 1 || pairs > dg::MAX_PAIRS || pair < 0 || pair >= pairs) return ADA_EINVAL;
     const dg::GemmPlan g = plan_dense(rows, N, per_tile, K, pairs);
     const int32_t v[6] = {g.nt, g.mt, g.tiles, g.chunks, g.groups, g.pairs};
     memcpy(plan6, v, sizeof(v));
@@ -1749,8 +1755,9 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     CK(cudaGetLastError());
     dg::GemmArgs a{};
     a.rows = rows; a.N = N; a.K = K; a.Y = Y_dev; a.ldy = ldy; a.err = err;
-    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = (N + dg::TW - 1) / dg::TW; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK; a.plan.groups = 1;
-    a.plan.pairs = std::max(1, std::min(a.plan.tiles, sms / 2));   // whole tiles: no exchange area needed
+    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = a.plan.whole = (N + dg::TW - 1) / dg::TW; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK; a.plan.groups = 1;
+    a.plan.pairs = std::max(1, std::min({a.plan.tiles, sms / 2, dg::MAX_PAIRS}));   // whole tiles: no exchange area needed
+    for (int i = 1; i < dg::MAX_GROUPS + 2; ++i) a.plan.group[i] = a.plan.chunks;
     const Ctx none{};
     rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, none, a);
     if (rc) return rc;

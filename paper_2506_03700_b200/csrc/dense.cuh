@@ -22,7 +22,7 @@
 // add the other one, already complete, to fp32 registers (round to nearest).  Each buffer sees 64 additions.
 //
 // Order of the sums.  It is a function of N, K and the device alone, so that the cache rows of a prompt's prefix have the
-// same bits whatever follows the prefix.  The chunks of a tile form 1 to 4 groups (group_begin; as many as one position
+// same bits whatever follows the prefix.  The chunks of a tile form 1 to 4 groups (as many as one position
 // tile has pairs to spare for, so that short prompts can use them side by side).  A group is summed from zero in the order
 // of its chunks, the groups are then added in their order: ((g0 + g1) + g2) + g3.  A pair that holds several groups of a
 // tile keeps the running total in scratch while it sums the next group (there are registers for one set of sums); that
@@ -212,50 +212,48 @@ template <typename SM> __device__ __forceinline__ bool dwait(SM *sm, int *err, u
     }
 }
 
-// Division of one product's tiles over the CTA pairs (chosen on the host, plan_dense).  Tiles are numbered with the
-// position tile fastest, so that the pairs at work at one time share weight rows.  The last sk_tiles tiles are divided
-// over sk_pairs pairs, by chunks or (by_group) by whole groups, the others are dealt out whole.
-struct GemmPlan { int nt, mt, tiles, chunks, groups, pairs, sk_tiles, sk_pairs, by_group; };   // nt positions per tile, mt position tiles
-__host__ __device__ __forceinline__ int group_begin(const GemmPlan &g, int i) { return i * g.chunks / g.groups; }   // first chunk of group i
+// Division of one product's tiles over the CTA pairs (worked out on the host, plan_dense, down to every pair's share: a
+// division on the device is cold code in front of a kernel's first load).  Tiles are numbered with the position tile fastest,
+// so that the pairs at work at one time share weight rows.  The tiles from `whole` on are divided over the pairs, by chunks or
+// by groups: pair p holds (tile - whole) << 16 | chunk from start[p] to start[p + 1]; the tiles before are dealt out whole.
+constexpr int MAX_PAIRS = 76;
+struct GemmPlan {
+    int nt, mt, chunks, groups, pairs;       // positions per tile, position tiles, chunks and groups of a tile
+    int tiles, whole;
+    int group[MAX_GROUPS + 2];               // first chunk of each group; `chunks` for the last group's end and behind
+    int start[MAX_PAIRS + 1];
+};
 
 struct Seg { int tile, c0, c1; };   // chunks [c0, c1) of a tile
 struct Sched {
-    GemmPlan g;
-    int pair, t_last, t_first, u_end, u_beg, i, phase;   // phase 0: last shared tile, 1: the whole ones between, 2: whole tiles, 3: first shared tile, 4: end
-    // first chunk of pair p's share, counted over the shared tiles
-    __host__ __device__ __forceinline__ int unit(int p) const {
-        if (!g.by_group) return (int)((long long)g.sk_tiles * g.chunks * p / g.sk_pairs);
-        const int u = (int)((long long)g.sk_tiles * g.groups * p / g.sk_pairs), t = u / g.groups;
-        return t * g.chunks + group_begin(g, u - t * g.groups);
-    }
-    __host__ __device__ __forceinline__ Sched(const GemmPlan &g_, int pair_) : g(g_), pair(pair_), t_last(0), t_first(0), u_end(0), u_beg(0), i(0), phase(2) {
-        if (g.sk_tiles > 0 && pair < g.sk_pairs) {
-            u_beg = unit(pair);
-            u_end = unit(pair + 1);
-            if (u_end > u_beg) {
-                t_first = u_beg / g.chunks;
-                t_last = (u_end - 1) / g.chunks;
-                phase = 0;
-            }
+    const GemmPlan &g;
+    int pair, t_first, c_first, t_last, c_last, i, phase;   // phase 0: last shared tile, 1: the whole ones between, 2: whole tiles, 3: first shared tile, 4: end
+    __host__ __device__ __forceinline__ Sched(const GemmPlan &g_, int pair_) : g(g_), pair(pair_), t_first(0), c_first(0), t_last(0), c_last(0), i(pair_), phase(2) {
+        const int beg = g.start[pair], end = g.start[pair + 1];
+        if (end > beg) {
+            t_first = beg >> 16;
+            c_first = beg & 0xffff;
+            c_last = end & 0xffff;
+            t_last = (end >> 16) - (c_last == 0);
+            if (c_last == 0) c_last = g.chunks;
+            phase = 0;
         }
-        if (phase == 2) i = pair;
     }
     // Pieces another pair waits for come first, the piece that waits for others comes last.
     __host__ __device__ __forceinline__ bool next(Seg &s) {
-        const int base = g.tiles - g.sk_tiles;
         if (phase == 0) {
             phase = 1;
             i = t_last - 1;
-            if (t_last != t_first || u_end < (t_last + 1) * g.chunks) {
-                s.tile = base + t_last;
-                s.c0 = t_last == t_first ? u_beg - t_last * g.chunks : 0;
-                s.c1 = u_end - t_last * g.chunks;
+            if (t_last != t_first || c_last < g.chunks) {
+                s.tile = g.whole + t_last;
+                s.c0 = t_last == t_first ? c_first : 0;
+                s.c1 = c_last;
                 return true;
             }
         }
         if (phase == 1) {
             if (i > t_first) {
-                s.tile = base + i--;
+                s.tile = g.whole + i--;
                 s.c0 = 0;
                 s.c1 = g.chunks;
                 return true;
@@ -264,7 +262,7 @@ struct Sched {
             i = pair;
         }
         if (phase == 2) {
-            if (i < base) {
+            if (i < g.whole) {
                 s.tile = i;
                 s.c0 = 0;
                 s.c1 = g.chunks;
@@ -275,9 +273,9 @@ struct Sched {
         }
         if (phase == 3) {
             phase = 4;
-            if (u_end > u_beg && (t_first != t_last || u_end == (t_last + 1) * g.chunks)) {
-                s.tile = base + t_first;
-                s.c0 = u_beg - t_first * g.chunks;
+            if (g.start[pair + 1] > g.start[pair] && (t_first != t_last || c_last == g.chunks)) {
+                s.tile = g.whole + t_first;
+                s.c0 = c_first;
                 s.c1 = g.chunks;
                 return true;
             }
@@ -333,32 +331,21 @@ __device__ __forceinline__ void sums_store(const float (&acc)[128], float4 *o, i
     for (int j = 0; j < 32; ++j)
         if (4 * j < nh) __stcg(o + 32 * j, make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]));
 }
-// acc = ((src[0] + src[1]) + src[2]) + acc over N sources, W 16-byte loads of each in flight (more would not fit beside the sums).
-template <int N, int W> __device__ __forceinline__ void sums_add_n(float (&acc)[128], const float4 *const (&src)[MAX_GROUPS - 1], int nh) {
+// acc += what sums_store left: sixteen loads in flight, more would not fit beside the sums.
+__device__ __forceinline__ void sums_add(float (&acc)[128], const float4 *src, int nh) {
 #pragma unroll
-    for (int j0 = 0; j0 < 32; j0 += W) {
+    for (int j0 = 0; j0 < 32; j0 += 16) {
         if (4 * j0 >= nh) break;
-        float4 r[N][W];
+        float4 r[16];
 #pragma unroll
-        for (int s = 0; s < N; ++s)
+        for (int j = 0; j < 16; ++j) r[j] = 4 * (j0 + j) < nh ? ld_cg_inorder(src + 32 * (j0 + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < W; ++j) r[s][j] = 4 * (j0 + j) < nh ? ld_cg_inorder(src[s] + 32 * (j0 + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
+        for (int j = 0; j < 16; ++j) {
             const int e = 4 * (j0 + j);
-            float4 t = r[0][j];
-#pragma unroll
-            for (int s = 1; s < N; ++s) { t.x += r[s][j].x; t.y += r[s][j].y; t.z += r[s][j].z; t.w += r[s][j].w; }
-            acc[e] += t.x; acc[e + 1] += t.y; acc[e + 2] += t.z; acc[e + 3] += t.w;
+            acc[e] += r[j].x; acc[e + 1] += r[j].y; acc[e + 2] += r[j].z; acc[e + 3] += r[j].w;
         }
     }
 }
-__device__ __forceinline__ void sums_add(float (&acc)[128], const float4 *const (&src)[MAX_GROUPS - 1], int n, int nh) {
-    if (n == 1) sums_add_n<1, 16>(acc, src, nh);
-    else if (n == 2) sums_add_n<2, 8>(acc, src, nh);
-    else sums_add_n<3, 4>(acc, src, nh);
-}
-static_assert(MAX_GROUPS == 4, "sums_add takes up to three sources");
 
 // Y[m][n] = or += x: four neighbouring n per lane, four positions per access.  N arbitrary, ldy a multiple of 4.
 template <bool ADD> __device__ __forceinline__ void epi_rows(const float (*x)[32], float *y, int ldy, int n_left, int lane, int left) {
@@ -609,78 +596,101 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
             float acc[128];
 #pragma unroll
             for (int j = 0; j < 128; ++j) acc[j] = 0.f;
-            const int chunks = a.plan.chunks, first = s.c0, end = s.c1;
+            const int chunks = a.plan.chunks, end = s.c1;
             const bool last = end == chunks;                 // this pair finishes the tile
-            const bool middle = first > 0 && !last;          // one group, published by itself
-            int grp = 0;
-            while (group_begin(a.plan, grp + 1) <= first) ++grp;
-            int grp_end = group_begin(a.plan, grp + 1);
-            bool own_total = false;                          // the total of the groups before this one is in this CTA's scratch
-            auto slot = [&](int cta, int which) {
-                return reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a.part) + (size_t)cta * GPART_CTA + which * GPART_SLOT + ew * GPART_WARP) + lane;
-            };
+            const bool middle = s.c0 > 0 && !last;           // one group, published by itself
             const int cta = 2 * pair + (int)rank;
-            const float4 *src[MAX_GROUPS - 1] = {nullptr, nullptr, nullptr};
-            if (live && first > group_begin(a.plan, grp)) {  // the group was begun by the pair before this one
-                ok = flag_wait(sm, a, cta - 2, ew);
-                if (ok) {
-                    src[0] = slot(cta - 2, SLOT_GROUP);
-                    sums_add(acc, src, 1, nh);
-                }
+            auto slot = [&](int at, int which) {
+                return reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a.part) + (size_t)at * GPART_CTA + which * GPART_SLOT + ew * GPART_WARP) + lane;
+            };
+            int cc = s.c0, grp = 0;
+            while (a.plan.group[grp + 1] <= cc) ++grp;
+            // Steps of a segment, each in one place of the code (the instruction cache is what a second copy of 128 additions
+            // costs: 6 us per launch): add sums from scratch, store the sums and go on from zero, multiply to the end of the
+            // group or of the segment.
+            const int own_slot = last ? SLOT_OWN : SLOT_TOTAL;
+            int add_from = 0, add_n = 0, add_slot = SLOT_TOTAL;   // sums to add: add_slot of add_n CTAs from add_from on, every second one
+            float4 *store_to = nullptr;
+            bool own_total = false;                          // the total of the groups before this one is in this CTA's scratch
+            bool group_done = false, publish = false;
+            if (live && cc > a.plan.group[grp]) {     // the pair before this one began the group
+                add_from = cta - 2;
+                add_n = 1;
+                add_slot = SLOT_GROUP;
             }
-            for (int cc = first; ok && cc < end; ++cc, ++ch) {
-                const int b = ch & 1;
-                ok = dwait(sm, a.err, &sm->acc_full[b], (ch >> 1) & 1);
-                ok = __all_sync(0xffffffffu, ok);
+            while (ok) {
+                for (; add_n > 0; --add_n, add_from += 2) {
+                    if (add_from != cta && !(ok = flag_wait(sm, a, add_from, ew))) break;
+                    sums_add(acc, slot(add_from, add_from == cta ? own_slot : add_slot), nh);
+                }
                 if (!ok) break;
-                tc_fence_after();
-                if (live) {
-#pragma unroll
-                    for (int g = 0; g < 8; ++g)
-                        if (16 * g < nh) {
-                            uint32_t v[16];
-                            tmem_ld16(v, t_lane + (uint32_t)(b * 256 + 16 * g));
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) acc[16 * g + e] += __uint_as_float(v[e]);
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) asm volatile("" : "+f"(acc[16 * g + e]));
-                        }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_at(map_to_cta(&sm->acc_empty[b], 0));
-                if (cc + 1 < grp_end) continue;
-                // a group is complete
-                if (live && grp > 0 && !middle) {   // add it to the total of those before it
-                    int n = 1;
-                    if (own_total) src[0] = slot(cta, last ? SLOT_OWN : SLOT_TOTAL);
-                    else {                          // other pairs': the tile's pieces in their order
-                        const int u0 = (s.tile - (a.plan.tiles - a.plan.sk_tiles)) * chunks;
-                        int p0 = pair - 1;
-                        while (p0 > 0 && sch.unit(p0) > u0) --p0;
-                        n = pair - p0;
-#pragma unroll
-                        for (int i = 0; i < MAX_GROUPS - 1; ++i)
-                            if (ok && i < n) {
-                                ok = flag_wait(sm, a, 2 * (p0 + i) + (int)rank, ew);
-                                src[i] = slot(2 * (p0 + i) + (int)rank, SLOT_TOTAL);
-                            }
-                        if (!ok) break;
-                    }
-                    sums_add(acc, src, n, nh);
-                }
-                ++grp;
-                grp_end = group_begin(a.plan, grp + 1);
-                if (live && cc + 1 < end) {
-                    sums_store(acc, slot(cta, last ? SLOT_OWN : SLOT_TOTAL), nh);
-                    own_total = true;
+                if (store_to) {
+                    sums_store(acc, store_to, nh);
+                    if (publish) break;
+                    store_to = nullptr;
 #pragma unroll
                     for (int j = 0; j < 128; ++j) acc[j] = 0.f;
+                    if (group_done) {   // these were set aside: first the other pairs' in their order, then they themselves
+                        add_n = (cta - add_from) / 2 + 1;
+                        continue;
+                    }
+                }
+                if (group_done) {
+                    group_done = false;
+                    ++grp;
+                    if (cc == end && last) break;
+                    if (live) {
+                        store_to = slot(cta, own_slot);
+                        publish = cc == end;
+                        own_total = true;
+                        continue;
+                    }
+                    if (cc == end) break;
+                }
+                const int grp_end = a.plan.group[grp + 1], stop = min(end, grp_end);
+                for (; cc < stop; ++cc, ++ch) {
+                    const int b = ch & 1;
+                    ok = dwait(sm, a.err, &sm->acc_full[b], (ch >> 1) & 1);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (live) {
+#pragma unroll
+                        for (int g = 0; g < 8; ++g)
+                            if (16 * g < nh) {
+                                uint32_t v[16];
+                                tmem_ld16(v, t_lane + (uint32_t)(b * 256 + 16 * g));
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) acc[16 * g + e] += __uint_as_float(v[e]);
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) asm volatile("" : "+f"(acc[16 * g + e]));
+                            }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_at(map_to_cta(&sm->acc_empty[b], 0));
+                }
+                if (!ok) break;
+                if (stop < grp_end) {             // the next pair goes on with this group
+                    if (!live) break;
+                    store_to = slot(cta, SLOT_GROUP);
+                    publish = true;
+                    continue;
+                }
+                group_done = true;
+                if (!live || grp == 0 || middle) continue;
+                if (own_total) { add_from = cta; add_n = 1; }
+                else {                            // other pairs hold the groups before this one
+                    int p0 = pair - 1;
+                    while (p0 > 0 && a.plan.start[p0] > (s.tile - a.plan.whole) << 16) --p0;
+                    add_from = 2 * p0 + (int)rank;
+                    add_slot = SLOT_TOTAL;
+                    if (p0 == pair - 1) add_n = 1;
+                    else store_to = slot(cta, own_slot);
                 }
             }
             if (!ok || !live) continue;
             if (!last) {   // another pair finishes this tile
-                sums_store(acc, slot(cta, end == group_begin(a.plan, grp) ? SLOT_TOTAL : SLOT_GROUP), nh);
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.flag + cta * GEPI_WARPS + ew), "r"(a.epoch) : "memory");
