@@ -280,12 +280,12 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
                          int32_t accumulate, void *work_dev, size_t work_bytes, void *cuda_stream);
 
 /* Host-only: how the dense GEMM divides a product of `rows` positions with N weight rows (per_tile of them to a tile: 256;
- * 128 where gate and up are multiplied side by side) and depth K over `pairs` pairs of CTAs.  plan6 (host) receives
- * {positions per tile, position tiles, tiles, 512-deep chunks of a tile, groups of chunks, pairs in use}; group i of a tile
- * starts at chunk i * chunks / groups (rounded down), and the number of groups does not depend on `rows`.  segs_host
+ * 128 where gate and up are multiplied side by side) and depth K over `pairs` pairs of CTAs.  plan7 (host) receives
+ * {positions per tile, position tiles, tiles, 64-wide k blocks of a chunk, chunks of a tile, groups of chunks, pairs in use};
+ * group i of a tile starts at chunk i * chunks / groups (rounded down).  Chunks and groups do not depend on `rows`.  segs_host
  * [max_segs][3] receives the work of pair `pair` in its order: (tile, first chunk, end chunk), *n_segs how many there are.
  * No GPU is touched.  ADA_EINVAL on bad arguments, ADA_ECAPACITY if max_segs does not suffice. */
-int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan6,
+int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan7,
                          int32_t *segs_host, int32_t max_segs, int32_t *n_segs);
 
 /* The same streaming GEMM as ada_debug_gemm (modes, shapes and layouts as described there, one

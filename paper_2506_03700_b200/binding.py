@@ -149,10 +149,10 @@ def debug_gemm_plan(N: int, K: int, mode: int, grid: int, cta: int, split: bool 
 
 def debug_dense_plan(rows: int, N: int, per_tile: int, K: int, pairs: int, pair: int):
     """ada_debug_dense_plan: (plan, segments (tile, first chunk, end chunk) of pair `pair`) of a dense product (host only, no GPU)."""
-    plan, n = (C.c_int32 * 6)(), C.c_int32(0)
+    plan, n = (C.c_int32 * 7)(), C.c_int32(0)
     segs = np.zeros((4096, 3), dtype=np.int32)
     _ck(load().ada_debug_dense_plan(rows, N, per_tile, K, pairs, pair, plan, segs.ctypes.data, len(segs), C.byref(n)), "ada_debug_dense_plan")
-    return dict(zip(("nt", "mt", "tiles", "chunks", "groups", "pairs"), list(plan))), segs[:n.value].tolist()
+    return dict(zip(("nt", "mt", "tiles", "ck", "chunks", "groups", "pairs"), list(plan))), segs[:n.value].tolist()
 
 
 def debug_gemm(W, X, mode: int = 0, repeat: int = 1):

@@ -386,13 +386,18 @@ bool cut_by_groups(const dg::GemmPlan &g, int p, int *chunks_max, int *pieces_ma
     return true;
 }
 
+// k blocks of a chunk: an eighth of the depth, 256 to 512 k.  Where the depth itself is small (2048: the 1B shape) the sums of
+// 512 k would show beside the split of the activations, and the shorter chunks cost nothing (its prompts wait for launches
+// and exchanges; 64 to 300 tokens: no difference measured).
+int chunk_blocks(int K) { return std::min(8, std::max(4, K / dg::BK / 8)); }
+
 // How a product of N weight rows (`per_tile` of them to a tile) and depth K over `rows` positions is divided over at most
 // `pairs` CTA pairs.  The number of groups of a tile's depth does not depend on `rows` (the order of the sums follows from
 // it): as many as the pairs that one position tile leaves for each of its tiles.  More tiles than pairs: whole waves, then
 // one wave's worth of tiles and the remainder cut by chunks so that all pairs end together (cutting the remainder alone would
 // cut a tile into more pieces, each of which costs an exchange).  Fewer: all tiles cut by groups over the number of pairs
-// that minimises, in cycles, the chunks of the busiest pair (8192 of the tensor core at full width; not below the 5600 that
-// a chunk's weights take to arrive at a pair's share of HBM bandwidth) plus the exchange of the pieces (3300 cycles per
+// that minimises, in cycles, the chunks of the busiest pair (per eight k blocks 8192 of the tensor core at full width; not
+// below the 5600 that their weights take to arrive at a pair's share of HBM bandwidth) plus the exchange of the pieces (3300 cycles per
 // further piece of full width, 3000 to begin with).
 dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
     dg::GemmPlan g{};
@@ -400,7 +405,8 @@ dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
     g.nt = position_tile(rows);
     g.mt = (rows + g.nt - 1) / g.nt;
     g.tiles = g.mt * across;
-    g.chunks = (K / dg::BK + dg::CK - 1) / dg::CK;
+    g.ck = chunk_blocks(K);
+    g.chunks = (K / dg::BK + g.ck - 1) / g.ck;
     g.groups = std::max(1, std::min({pairs / across, g.chunks, dg::MAX_GROUPS}));
     for (int i = 0; i < dg::MAX_GROUPS + 2; ++i) g.group[i] = std::min(g.chunks, i * g.chunks / g.groups);
     if (g.tiles >= pairs) {
@@ -413,7 +419,7 @@ dg::GemmPlan plan_dense(int rows, int N, int per_tile, int K, int pairs) {
         }
         return g;
     }
-    const double width = (double)g.nt / dg::NT_MAX, chunk = std::max(8192.0 * width, 5600.0);
+    const double width = (double)g.nt / dg::NT_MAX, chunk = std::max(8192.0 * width, 5600.0) * g.ck / 8;
     double best = 0;
     for (int p = g.tiles; p <= std::min(pairs, g.tiles * g.groups); ++p) {
         int most, pieces;
@@ -1705,13 +1711,13 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     return herr ? ADA_ETIMEOUT : ADA_OK;
 }
 
-int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan6,
+int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan7,
                          int32_t *segs_host, int32_t max_segs, int32_t *n_segs) {
-    if (!plan6 || !segs_host || !n_segs || max_segs < 1 || rows < 1 || rows > dg::PF_ROWS || N < 1 || K < 64 || K % 64) return ADA_EINVAL;
+    if (!plan7 || !segs_host || !n_segs || max_segs < 1 || rows < 1 || rows > dg::PF_ROWS || N < 1 || K < 64 || K % 64) return ADA_EINVAL;
     if ((per_tile != dg::TW && per_tile != dg::BW) || pairs < 1 || pairs > dg::MAX_PAIRS || pair < 0 || pair >= pairs) return ADA_EINVAL;
     const dg::GemmPlan g = plan_dense(rows, N, per_tile, K, pairs);
-    const int32_t v[6] = {g.nt, g.mt, g.tiles, g.chunks, g.groups, g.pairs};
-    memcpy(plan6, v, sizeof(v));
+    const int32_t v[7] = {g.nt, g.mt, g.tiles, g.ck, g.chunks, g.groups, g.pairs};
+    memcpy(plan7, v, sizeof(v));
     *n_segs = 0;
     if (pair >= g.pairs) return ADA_OK;
     dg::Sched sch(g, pair);
@@ -1755,7 +1761,9 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     CK(cudaGetLastError());
     dg::GemmArgs a{};
     a.rows = rows; a.N = N; a.K = K; a.Y = Y_dev; a.ldy = ldy; a.err = err;
-    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = a.plan.whole = (N + dg::TW - 1) / dg::TW; a.plan.chunks = (K / dg::BK + dg::CK - 1) / dg::CK; a.plan.groups = 1;
+    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = a.plan.whole = (N + dg::TW - 1) / dg::TW; a.plan.groups = 1;
+    a.plan.ck = chunk_blocks(K);
+    a.plan.chunks = (K / dg::BK + a.plan.ck - 1) / a.plan.ck;
     a.plan.pairs = std::max(1, std::min({a.plan.tiles, sms / 2, dg::MAX_PAIRS}));   // whole tiles: no exchange area needed
     for (int i = 1; i < dg::MAX_GROUPS + 2; ++i) a.plan.group[i] = a.plan.chunks;
     const Ctx none{};

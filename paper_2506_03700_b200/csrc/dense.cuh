@@ -16,10 +16,12 @@
 // 48 KB per 512 cycles and 2.7 times the L2 traffic per weight byte.  Two accumulators of 128 positions (gate and up side
 // by side) were 15 % slower than one of 256: at that width the operands' way out of shared memory is the bound.
 //
-// Accumulation.  The tensor core adds into its fp32 accumulator with truncation, so the error of one accumulator
-// grows with the products added to it (1e-3 absolute at K = 14336 with sums of size 10).  A product is therefore cut
-// into chunks of 512 k; a chunk accumulates in one of two 256-column tensor-memory buffers while the epilogue warps
-// add the other one, already complete, to fp32 registers (round to nearest).  Each buffer sees 64 additions.
+// Accumulation.  The tensor core adds into its fp32 accumulator with truncation, so an accumulator falls short by
+// 1.5e-8 of the sum per addition (1e-3 absolute at K = 14336 with sums of size 10).  A product is therefore cut into chunks
+// of 512 k, shallow ones of 256 (chunk_blocks); a chunk accumulates in one of two 256-column tensor-memory buffers while the
+// epilogue warps add the other one, already complete, to fp32 registers (round to nearest).  Error of the sums alone, 2-norm:
+// 1.10e-6 with chunks of 512, 0.56e-6 of 256, 0.30e-6 of 128; the split of the activations is 2.45e-6.  Chunks of 256 (128)
+// everywhere cost a 777-token prompt of the 8B shape 4 % (22 %): the epilogue then holds up the tensor core.
 //
 // Order of the sums.  It is a function of N, K and the device alone, so that the cache rows of a prompt's prefix have the
 // same bits whatever follows the prefix.  The chunks of a tile form 1 to 4 groups (as many as one position
@@ -57,7 +59,6 @@ constexpr int BW = 128;        // weight rows one CTA of a pair holds (UMMA M = 
 constexpr int TW = 2 * BW;
 constexpr int NT_MAX = 256;    // positions per tile, at most
 constexpr int BK = 64;         // k elements per stage: one 128-byte swizzle row
-constexpr int CK = 8;          // k blocks per accumulator chunk
 constexpr int MAX_STAGES = 12;
 constexpr int GEPI_WARPS = 8;  // epilogue warps: lane quadrant (warp % 4) x half of the tile's positions
 constexpr int GTHREADS = 128 + 32 * GEPI_WARPS;
@@ -218,7 +219,7 @@ template <typename SM> __device__ __forceinline__ bool dwait(SM *sm, int *err, u
 // by groups: pair p holds (tile - whole) << 16 | chunk from start[p] to start[p + 1]; the tiles before are dealt out whole.
 constexpr int MAX_PAIRS = 76;
 struct GemmPlan {
-    int nt, mt, chunks, groups, pairs;       // positions per tile, position tiles, chunks and groups of a tile
+    int nt, mt, ck, chunks, groups, pairs;   // positions per tile, position tiles; k blocks of a chunk, chunks and groups of a tile
     int tiles, whole;
     int group[MAX_GROUPS + 2];               // first chunk of each group; `chunks` for the last group's end and behind
     int start[MAX_PAIRS + 1];
@@ -475,7 +476,7 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
     DSmem *sm = reinterpret_cast<DSmem *>(dsm_raw + ((1024u - (s32(dsm_raw) & 1023u)) & 1023u));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
-    const int pair = blockIdx.x >> 1, nkb = a.K / BK, nt = a.plan.nt;
+    const int pair = blockIdx.x >> 1, nkb = a.K / BK, nt = a.plan.nt, ck = a.plan.ck;
     const int x_bytes = nt / 2 * BK * 2, stage_bytes = W_BYTES + 2 * x_bytes, stages = min(MAX_STAGES, RING_BYTES / stage_bytes);
     pdl_trigger();
     if (threadIdx.x == 0) {
@@ -517,7 +518,7 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                 Sched sch(a.plan, pair);
                 Seg s;
                 if (sch.next(s)) {
-                    const int kb0 = s.c0 * CK, kb1 = min(s.c1 * CK, nkb);
+                    const int kb0 = s.c0 * ck, kb1 = min(s.c1 * ck, nkb);
                     for (; ahead < stages && kb0 + ahead < kb1; ++ahead) load_w(ahead, kb0 + ahead, s.tile / a.plan.mt);
                 }
             }
@@ -528,8 +529,8 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
             uint32_t ph = 1;
             bool ok = true;
             while (ok && sch.next(s)) {
-                const int tm = s.tile % a.plan.mt, tn = s.tile / a.plan.mt, x0 = tm * nt + (int)rank * (nt / 2), kb1 = min(s.c1 * CK, nkb);
-                for (int kb = s.c0 * CK; kb < kb1; ++kb, ++it) {
+                const int tm = s.tile % a.plan.mt, tn = s.tile / a.plan.mt, x0 = tm * nt + (int)rank * (nt / 2), kb1 = min(s.c1 * ck, nkb);
+                for (int kb = s.c0 * ck; kb < kb1; ++kb, ++it) {
                     if (it >= ahead) {
                         ok = dwait(sm, a.err, &sm->empty[st], ph);
                         if (!ok) break;
@@ -552,12 +553,12 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
             bool ok = true;
             while (ok && sch.next(s)) {
                 for (int cc = s.c0; ok && cc < s.c1; ++cc, ++ch) {
-                    const int b = ch & 1, kb1 = min((cc + 1) * CK, nkb);
+                    const int b = ch & 1, kb1 = min((cc + 1) * ck, nkb);
                     ok = dwait(sm, a.err, &sm->acc_empty[b], ((ch >> 1) & 1) ^ 1);
                     if (!ok) break;
                     tc_fence_after();
                     uint32_t add = 0;
-                    for (int kb = cc * CK; kb < kb1; ++kb) {
+                    for (int kb = cc * ck; kb < kb1; ++kb) {
                         ok = dwait(sm, a.err, &sm->full[st], ph);
                         if (!ok) break;
                         tc_fence_after();

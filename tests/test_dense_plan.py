@@ -74,6 +74,7 @@ def check(rows, N, per_tile, K, pairs):
     assert 32 <= plan["nt"] <= 256 and plan["nt"] % 32 == 0 and plan["nt"] * plan["mt"] >= rows
     assert plan["tiles"] == plan["mt"] * -(-N // per_tile) and 1 <= plan["pairs"] <= pairs
     assert len(set(sums.values())) == 1
+    assert plan["ck"] == min(8, max(4, K // 512)) and plan["chunks"] == -(-(K // 64) // plan["ck"])
     return plan["groups"], sums[0]
 
 

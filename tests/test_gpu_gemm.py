@@ -73,3 +73,20 @@ def test_dense_gemm_matches_float64(N, K, rows):
     Y2 = torch.ones_like(Y)
     binding.debug_dense_gemm(W, X, Y2)
     assert np.abs(Y2.double().cpu().numpy() - (ref + 1.0)).max() <= 2e-5 * max(1.0, np.abs(ref).max())
+
+
+# deepest accumulator: an eighth of the depth, 256 to 512
+@pytest.mark.parametrize("N,K,rows,depth", [(3072, 2048, 100, 256), (2048, 2048, 21, 256), (16384, 2048, 128, 256), (5120, 3008, 64, 320),
+                                            (4096, 4096, 77, 512), (4096, 14336, 9, 512)])
+def test_sums_of_the_dense_gemm(N, K, rows, depth):
+    """The error that the sums add to that of the operand's split.  The tensor core truncates after every addition of sixteen
+    products, twice per sixteen k (high and low parts): half a unit in the last place on average, 0.36 * 2^-23 of a partial sum
+    that is two thirds of the final one, i.e. 2.9e-8 of the result per addition at most, half of it where the digits are
+    spread evenly; 1e-7 for the fp32 additions of the accumulators."""
+    W = synth.normal_tensor(9, 11, (N, K), 0.05, torch.bfloat16, "cuda")
+    X = synth.normal_tensor(9, 12, (rows, K), 1.0, torch.float32, "cuda")
+    hi = X.bfloat16()
+    lo = (X - hi.float()).bfloat16()
+    ref = (hi.double() + lo.double()) @ W.double().T
+    err = (binding.debug_dense_gemm(W, X).double() - ref).norm() / ref.norm()
+    assert err <= 1.6e-8 * (2 * depth / 16) + 1e-7, err
