@@ -173,7 +173,7 @@ struct ada_session {
     bool dense_ok = false;                     // available for this session
     int pf_pairs = 0;                          // CTA pairs of this device
     unsigned pf_epoch = 0;                     // dense products launched so far (tags published partial sums)
-    float *pf_resid = nullptr, *pf_cs = nullptr, *pf_part = nullptr;
+    float *pf_resid = nullptr, *pf_cs = nullptr, *pf_rstd = nullptr, *pf_part = nullptr;
     __nv_bfloat16 *pf_x = nullptr, *pf_u = nullptr;   // high and low parts of a product's input: model width; queries, attention result / FFN activations
     unsigned *pf_flag = nullptr;
     int *pf_err = nullptr;
@@ -204,7 +204,7 @@ namespace {
 // Scratch layout (all offsets 256-byte aligned).
 struct Layout {
     size_t st, rt, fill, tokens, page_table, head_res, resid, xn, qkv, q, attn_out, gu, hact, rope_cs, attn_part,
-        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_err, pf_flag, pf_part, maps, mm, exit_at, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
+        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, maps, mm, exit_at, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
         grid_ctr, pub, err, attn_tag, q_stage, qinfo, uniforms, total;
 };
 
@@ -259,6 +259,7 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.pf_x = take(sizeof(__nv_bfloat16) * 2 * P * g.d_model);
         L.pf_u = take(sizeof(__nv_bfloat16) * P * std::max(4 * (size_t)qd, 2 * (size_t)g.d_ff));
         L.pf_cs = take(sizeof(float) * P * g.head_dim);
+        L.pf_rstd = take(sizeof(float) * P);
         L.pf_err = take(256);
         L.pf_flag = take(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS);
         L.pf_part = take(dg::GPART_CTA * 2 * dg::MAX_PAIRS);
@@ -469,13 +470,13 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     typedef __nv_bfloat16 T;
     int rc;
     dg::GemmArgs a{};
-    a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err;
+    a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.rstd = S->pf_rstd; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err;
     a.Y = S->pf_resid; a.ldy = d;
     S->layer_passes++;
     S->launches += 7;
     auto norm = [&](const void *gain) {
         Prof pf(S, 1, 0.0);
-        return launch_overlapped(S->stream, dg::k_norm_split_rows, rows, 256, 0, S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl);
+        return launch_overlapped(S->stream, dg::k_norm_split_rows, rows, 256, 0, S->pf_resid, d, (const T *)gain, g.rms_eps, xh, xl, S->pf_rstd);
     };
     auto shape = [&](int N, int K, const dg::GemmPlan &plan) { a.N = N; a.K = K; a.epoch = ++S->pf_epoch; a.plan = plan; };
     if ((rc = norm(w.attn_norm))) return rc;
@@ -1360,6 +1361,7 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
             S->pf_x = (__nv_bfloat16 *)(b + lay.pf_x);
             S->pf_u = (__nv_bfloat16 *)(b + lay.pf_u);
             S->pf_cs = (float *)(b + lay.pf_cs);
+            S->pf_rstd = (float *)(b + lay.pf_rstd);
             S->pf_err = (int *)(b + lay.pf_err);
             S->pf_flag = (unsigned *)(b + lay.pf_flag);
             S->pf_part = (float *)(b + lay.pf_part);

@@ -292,6 +292,7 @@ struct GemmArgs {
     float *Y; int ldy;            // STORE, ADD
     __nv_bfloat16 *hi, *lo;       // QKV: scaled queries [rows][q features]; SwiGLU: activations [rows][N]
     const float *cs;              // QKV: cos, sin [rows][hd / 2][2]
+    const float *rstd;            // QKV, SwiGLU: 1 / rms of the rows, applied to the products
     int layer, seq, pos0;         // QKV: rows are positions pos0 .. of sequence seq
     float *part;                  // [CTA][slot]: sums of tiles cut between pairs, running totals (null: one group, nothing cut)
     unsigned *flag;               // [CTA][epilogue warp]: launch number of the sums published last
@@ -374,7 +375,8 @@ float4 r[8];
     }
 }
 
-// q, k and v: the weight rows come reordered (see k_repack_qkv), so that rows r and r + 8 of 16 are the partners of a rotation.
+// q, k and v: the products are those of the rows before normalisation (k_norm_split_rows) and take its factor here.
+// The weight rows come reordered (see k_repack_qkv), so that rows r and r + 8 of 16 are the partners of a rotation.
 // q and k are rotated, q is scaled and split into bf16 high and low parts, k and v go to the cache rows of the positions
 // (16-byte chunks xor-swizzled, see kv_swz).  n_w: first weight row of the warp; all 32 belong to one head.  A lane
 // computes one pair of partners for every second position and, with its neighbour, writes two neighbouring features.
@@ -391,17 +393,19 @@ template <int HD> __device__ __forceinline__ void epi_qkv(const Ctx &c, const Ge
     const int32_t *table = c.page_table + (size_t)a.seq * c.max_pages;
     __nv_bfloat16 *pool = reinterpret_cast<__nv_bfloat16 *>(c.kv_pool);
     float2 cs[16];
+    float rstd[16];
     int page[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int m = m0 + min(2 * i + (lane >> 4), left - 1);
+        rstd[i] = a.rstd[m];
         if (which < 2) cs[i] = *reinterpret_cast<const float2 *>(a.cs + ((size_t)m * (HD / 2) + jj) * 2);
         if (which > 0) page[i] = table[(a.pos0 + m) >> c.page_shift];
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const int jm = 2 * i + (lane >> 4), m = m0 + jm;
-        float y0 = x[jm][row], y1 = x[jm][row + 8];
+        float y0 = x[jm][row] * rstd[i], y1 = x[jm][row + 8] * rstd[i];
         if (which < 2) {   // the same in every lane
             const float z0 = y0 * cs[i].x - y1 * cs[i].y, z1 = y1 * cs[i].x + y0 * cs[i].y;
             y0 = z0 * scale; y1 = z1 * scale;
@@ -426,13 +430,17 @@ template <int HD> __device__ __forceinline__ void epi_qkv(const Ctx &c, const Ge
 
 // SwiGLU: rows 0 .. 15 are the gate values of sixteen features, rows 16 .. 31 their up values; a lane takes two neighbouring
 // features of every fourth position.  The activations are split into bf16 high and low parts.
-__device__ __forceinline__ void epi_swiglu(const float (*x)[32], __nv_bfloat16 *hi, __nv_bfloat16 *lo, int ld, int lane, int left) {
+__device__ __forceinline__ void epi_swiglu(const float (*x)[32], const float *rstd, __nv_bfloat16 *hi, __nv_bfloat16 *lo, int ld, int lane, int left) {
     const int n = 2 * (lane & 7);
     uint32_t h[8], l[8];
+    float rs[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) rs[i] = rstd[min(4 * i + (lane >> 3), left - 1)];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int j = 4 * i + (lane >> 3);
-        const float2 g = *reinterpret_cast<const float2 *>(&x[j][n]), u = *reinterpret_cast<const float2 *>(&x[j][16 + n]);
+        float2 g = *reinterpret_cast<const float2 *>(&x[j][n]), u = *reinterpret_cast<const float2 *>(&x[j][16 + n]);
+        g.x *= rs[i]; g.y *= rs[i]; u.x *= rs[i]; u.y *= rs[i];
         split2(g.x / (1.0f + expf(-g.x)) * u.x, g.y / (1.0f + expf(-g.y)) * u.y, h[i], l[i]);
     }
 #pragma unroll
@@ -702,7 +710,7 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
                 const int m = m0 + j0;
                 if constexpr (EPI == EPI_STORE || EPI == EPI_ADD) epi_rows<EPI == EPI_ADD>(x, a.Y + (size_t)m * a.ldy + n_w, a.ldy, a.N - n_w, lane, cnt);
                 else if constexpr (EPI == EPI_QKV) epi_qkv<HD>(c, a, x, n_w, lane, m, cnt);
-                else epi_swiglu(x, a.hi + (size_t)m * a.N + n_w, a.lo + (size_t)m * a.N + n_w, a.N, lane, cnt);   // N is a multiple of 64: the warp's features are all there
+                else epi_swiglu(x, a.rstd + m, a.hi + (size_t)m * a.N + n_w, a.lo + (size_t)m * a.N + n_w, a.N, lane, cnt);   // N is a multiple of 64: the warp's features are all there
             });
         }
     }
@@ -749,10 +757,12 @@ __global__ void k_pf_last(Ctx c, const float *__restrict__ resid, int row, int s
     }
 }
 
-// RMSNorm and split in one pass: x = resid[r] / sqrt(mean(resid[r]^2) + eps) * g -> high and low parts.  One CTA
-// (256 threads) per row, four elements per access; K a multiple of 64.
+// RMSNorm and split in one pass: x = resid[r] * g -> high and low parts, rstd[r] = 1 / sqrt(mean(resid[r]^2) + eps), which the
+// epilogue of the product applies.  (The factor before the split would cost the first layer the exactness of its split: bf16
+// embeddings have no low part, their products with the factor have one, and five times as many rounded K and V differed.)
+// One CTA (256 threads) per row, four elements per access; K a multiple of 64.
 __global__ void __launch_bounds__(256) k_norm_split_rows(const float *X, int K, const __nv_bfloat16 *__restrict__ gain,
-                                                         float eps, __nv_bfloat16 *hi, __nv_bfloat16 *lo) {
+                                                         float eps, __nv_bfloat16 *hi, __nv_bfloat16 *lo, float *rstd) {
     const int r = blockIdx.x;
     __shared__ float red[8];
     pdl_begin();
@@ -768,13 +778,13 @@ __global__ void __launch_bounds__(256) k_norm_split_rows(const float *X, int K, 
     float tot = 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) tot += red[w];
-    const float rstd = 1.0f / sqrtf(tot / K + eps);
+    if (threadIdx.x == 0) rstd[r] = 1.0f / sqrtf(tot / K + eps);
     for (int i = threadIdx.x; i < K / 4; i += 256) {
         const float4 v = x[i];
         const uint2 gq = reinterpret_cast<const uint2 *>(gain)[i];
         uint2 h, l;
-        split2(v.x * rstd * __uint_as_float(gq.x << 16), v.y * rstd * __uint_as_float(gq.x & 0xffff0000u), h.x, l.x);
-        split2(v.z * rstd * __uint_as_float(gq.y << 16), v.w * rstd * __uint_as_float(gq.y & 0xffff0000u), h.y, l.y);
+        split2(v.x * __uint_as_float(gq.x << 16), v.y * __uint_as_float(gq.x & 0xffff0000u), h.x, l.x);
+        split2(v.z * __uint_as_float(gq.y << 16), v.w * __uint_as_float(gq.y & 0xffff0000u), h.y, l.y);
         reinterpret_cast<uint2 *>(hi + (size_t)r * K)[i] = h;
         reinterpret_cast<uint2 *>(lo + (size_t)r * K)[i] = l;
     }

@@ -3,6 +3,7 @@ decode kernel (eight positions at a time)."""
 
 import numpy as np
 import pytest
+import torch
 
 pytestmark = pytest.mark.gpu
 
@@ -111,3 +112,27 @@ def test_a_prefix_leaves_the_same_cache_bits_whatever_follows_it(hd, nq, nkv, d,
                 rows = _rows(S, cfg, [p])
                 first = seen.setdefault(p, (n, rows))
                 assert np.array_equal(first[1], rows), (p, first[0], n)
+
+
+@pytest.mark.parametrize("hd,nq,nkv,d", [(64, 16, 4, 1024), (128, 16, 16, 2048)])
+@pytest.mark.parametrize("n", [9, 31, 100])
+def test_first_layer_rounds_what_the_embeddings_give(hd, nq, nkv, d, n):
+    """The first layer's input is bf16: its products can be as exact as their sums, whether eight positions or the whole prompt
+    are multiplied at once.  A K or V differs from the rounded float64 one where an error e of the sums straddles a rounding
+    boundary, i.e. with probability e / ulp: below 1.2e-6 / 2^-8 = 3e-4 (values near zero have wider errors relative to them
+    than the sums' 2-norm says: twice that).  A normalised row would be split with an error of 2.5e-6 instead: 3e-3 measured."""
+    cfg, gm = _model(hd, nq, nkv, d, 1024, layers=1)
+    w = synth.make_weights(cfg, device="cuda")
+    prompt = synth.make_prompt(cfg, n=n)
+    S = binding.Session(gm, 1, n + 8, 64, 0)
+    S.prefill(prompt.numpy())
+    x = w["tok_embed"][prompt.long().cuda()].double()
+    qkv = (x / torch.sqrt((x * x).mean(-1, keepdim=True) + np.float32(cfg.rms_eps).item())) @ w["layers.0.wqkv"].double().T
+    k, v = qkv[:, nq * hd:].view(n, 2, nkv, hd).unbind(1)
+    angle = torch.arange(n, dtype=torch.float64, device="cuda")[:, None] * cfg.rope_base ** (-2.0 * torch.arange(hd // 2, dtype=torch.float64, device="cuda") / hd)
+    co, si = angle.cos()[:, None], angle.sin()[:, None]
+    a, b = k[..., :hd // 2], k[..., hd // 2:]
+    k = torch.cat([a * co - b * si, b * co + a * si], -1)
+    want = torch.stack([k, v], 1).float().bfloat16().float().cpu().numpy().reshape(n, 2, nkv * hd)
+    got = _rows(S, cfg, range(n)).reshape(n, 2, nkv * hd)
+    assert np.mean(got != want) <= 6e-4
