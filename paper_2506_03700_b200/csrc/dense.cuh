@@ -818,6 +818,12 @@ __global__ void k_split_rows(const float *__restrict__ X, int ldx, int rows, int
 // of P), 2048 cycles at HD = 128; the softmax of a tile takes about 1500 cycles of its warps and hides behind the other
 // tile.  Key tiles of 128 because an S of 64 columns would read Q from shared memory twice as often as its bandwidth
 // (128 B per cycle) allows.  Rows are independent of each other, so positions past the prompt only waste work.
+//
+// A masked position has probability zero, which hides everything but a V that is not finite.  So the V tiles that some row
+// of the item must not see whole are gone over before the tensor core reads them: rows behind the item's last position
+// are cleared (they hold another sequence's rows, or none), and a value that is not finite becomes zero, its feature
+// remembered with the position: the rows that do see it get NaN in the end, which is what p * V would have left of them.
+// One warp, 0.3 us per tile, for the one to three key tiles at the diagonal.
 constexpr int AT_Q = 128, AT_K = 128, AT_THREADS = 384;
 constexpr int AT_REGS_ISSUE = 56, AT_REGS_SOFT = 224;   // (56 + 224 + 224) x 128 = 168 x 384
 template <int HD> struct AtSmem {   // must start on a 1024-byte boundary
@@ -826,7 +832,9 @@ template <int HD> struct AtSmem {   // must start on a 1024-byte boundary
     static constexpr int SLOTS = HD == 128 ? 3 : 6;
     alignas(1024) unsigned char q[2][2][HD / 64][HALF];  // [tile][high | low][64-feature group]
     alignas(1024) unsigned char kv[SLOTS][KV];           // ring of K and V tiles in turn
-    alignas(8) unsigned long long q_full[2], kv_full[SLOTS], kv_empty[SLOTS], s_full[2], p_full[2], o_full[2], tail;
+    alignas(8) unsigned long long q_full[2], kv_full[SLOTS], kv_empty[SLOTS], s_full[2], p_full[2], o_full[2], diag;
+    int bad[HD];                                         // per feature: first position of a causally cut key tile whose V is not finite
+    int any_bad;
     uint32_t tmem_base;
     int abort;
 };
@@ -882,6 +890,27 @@ __device__ __forceinline__ void tma_tile_3d(void *dst, const CUtensorMap *map, i
                  : "memory");
 }
 
+// Takes the values that are not finite out of the first `seen` rows of a V tile (positions from p0 on); see above.  Rare, and out
+// of line for that reason.  Chunk c of row r is stored at c ^ (r % 8).
+template <int HD> __device__ __noinline__ void pf_attn_take_out(AtSmem<HD> *sm, unsigned char *tile, int p0, int seen, int lane) {
+    if (*(volatile int *)&sm->any_bad == 0)
+        for (int f = lane; f < HD; f += 32) sm->bad[f] = INT_MAX;
+    __syncwarp();
+    for (int g = 0; g < HD / 64; ++g)
+        for (int i = lane; i < seen * 8; i += 32) {
+            __nv_bfloat16 *x = reinterpret_cast<__nv_bfloat16 *>(tile + g * (AT_K * 128) + i * 16);
+            const int row = i >> 3, f = g * 64 + ((i ^ row) & 7) * 8;
+            for (int e = 0; e < 8; ++e)
+                if (!isfinite(__bfloat162float(x[e]))) {
+                    atomicMin(&sm->bad[f + e], p0 + row);
+                    x[e] = __float2bfloat16_rn(0.f);
+                }
+        }
+    __syncwarp();
+    if (lane == 0) *(volatile int *)&sm->any_bad = 1;
+    __syncwarp();
+}
+
 // mapQhi / mapQlo: 3-D maps over the queries [rows][q heads][HD] (box 64 x GROUP x 128 / GROUP, 128-byte swizzle, rows past
 // the block read as zero).  mapKV: 2-D map over the page pool as rows of HD elements (box 64 x kv_box rows, no swizzle).
 // Grid: (256-row items of the block) x kv heads, the items with the longest context first.
@@ -908,7 +937,8 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
             mbar_init(&sm->q_full[i], 1); mbar_init(&sm->s_full[i], 1); mbar_init(&sm->p_full[i], 4); mbar_init(&sm->o_full[i], 1);
         }
         for (int i = 0; i < SLOTS; ++i) { mbar_init(&sm->kv_full[i], 1); mbar_init(&sm->kv_empty[i], 1); }
-        mbar_init(&sm->tail, 1);
+        mbar_init(&sm->diag, 1);
+        sm->any_bad = 0;
         sm->abort = 0;
         fence_mbar_init();
         fence_proxy_async();
@@ -939,15 +969,14 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
                     }
                 }
             bool ok = true;
+            int n_cut = 0;
             for (int it = 0; ok && it < 2 * n; ++it) {   // K of key tile 0, V of key tile 0, K of key tile 1, ...
                 const int st = it % SLOTS, j = it >> 1, which = it & 1;
                 ok = dwait(sm, err, &sm->kv_empty[st], ((it / SLOTS) & 1) ^ 1);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                // V rows of positions the item does not see are multiplied by zero probabilities; they may hold anything (another
-                // sequence's rows, or none), so they are cleared before the tensor core reads them
-                const bool tail = which == 1 && (j + 1) * AT_K - 1 > last;
-                unsigned long long *bar = tail ? &sm->tail : &sm->kv_full[st];
+                const bool cut = which == 1 && (j + 1) * AT_K - 1 > pos0 + r0;   // some row of the item does not see the whole tile
+                unsigned long long *bar = cut ? &sm->diag : &sm->kv_full[st];
                 if (lane == 0) {
                     mbar_expect_tx(bar, (uint32_t)Sm::KV);
                     for (int r = 0; r < AT_K; r += kv_box) {
@@ -957,14 +986,25 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
                     }
                 }
                 __syncwarp();
-                if (tail) {   // at most once: the last tile
-                    ok = dwait(sm, err, &sm->tail, 0);
+                if (cut) {
+                    ok = dwait(sm, err, &sm->diag, n_cut & 1);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
-                    const int from = last + 1 - j * AT_K;   // first cleared row
-                    for (int g = 0; g < HG; ++g)
-                        for (int i = from * 8 + lane; i < AT_K * 8; i += 32)
-                            *reinterpret_cast<uint4 *>(sm->kv[st] + g * (AT_K * 128) + i * 16) = make_uint4(0, 0, 0, 0);
+                    ++n_cut;
+                    const int seen = min(AT_K, last + 1 - j * AT_K);   // rows of the tile that the item sees
+                    uint32_t found = 0;
+                    for (int g = 0; g < HG; ++g) {
+                        uint4 *v = reinterpret_cast<uint4 *>(sm->kv[st] + g * (AT_K * 128));
+                        int i = lane;
+#pragma unroll 8
+                        for (; i < seen * 8; i += 32) {   // exponent bits all set: adding one to them carries into the sign bit
+                            const uint4 x = v[i];
+                            found |= ((x.x & 0x7f807f80u) + 0x00800080u) | ((x.y & 0x7f807f80u) + 0x00800080u) |
+                                     ((x.z & 0x7f807f80u) + 0x00800080u) | ((x.w & 0x7f807f80u) + 0x00800080u);
+                        }
+                        for (; i < AT_K * 8; i += 32) v[i] = make_uint4(0, 0, 0, 0);
+                    }
+                    if (__any_sync(0xffffffffu, (found & 0x80008000u) != 0)) pf_attn_take_out<HD>(sm, sm->kv[st], j * AT_K, seen, lane);
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&sm->kv_full[st]);
@@ -1104,11 +1144,15 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
             tc_fence_after();
             if (ok) {
                 const float inv = 1.0f / l;
+                const bool any_bad = *(volatile int *)&sm->any_bad != 0;
                 const size_t o = ((size_t)r * c.nq + kvh * GROUP + row % GROUP) * HD;
 #pragma unroll 1
                 for (int b = 0; b < HD / 32; ++b) {
                     uint32_t v[32];
                     tmem_ld32(v, t_o + 32 * b);
+                    if (any_bad)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = pos >= *(volatile int *)&sm->bad[32 * b + e] ? 0x7fc00000u : v[e];
                     if (r < rows)
 #pragma unroll
                         for (int e = 0; e < 32; e += 8) {

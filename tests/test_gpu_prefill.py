@@ -136,3 +136,36 @@ def test_first_layer_rounds_what_the_embeddings_give(hd, nq, nkv, d, n):
     want = torch.stack([k, v], 1).float().bfloat16().float().cpu().numpy().reshape(n, 2, nkv * hd)
     got = _rows(S, cfg, range(n)).reshape(n, 2, nkv * hd)
     assert np.mean(got != want) <= 6e-4
+
+
+@pytest.mark.parametrize("hd,nq,nkv", [(64, 4, 1), (128, 4, 2), (128, 2, 2)])
+@pytest.mark.parametrize("bad", ["nan", "infinity", "one value"])
+@pytest.mark.parametrize("n,at", [(40, 20), (129, 127), (200, 128), (700, 513), (2100, 1060)])
+def test_a_token_that_is_not_finite_leaves_the_positions_before_it_alone(hd, nq, nkv, bad, n, at):
+    """Causality with values that no multiplication by zero can hide: the positions before such a token keep, bit for bit, the
+    cache rows that they have without it; what follows is not finite.  "one value": a single feature of the token's value row
+    of one head overflows, everything else about the token is finite."""
+    cfg, _ = _model(hd, nq, nkv)
+    w = synth.make_weights(cfg, device="cuda")
+    w["tok_embed"][:, 3] = 0.0
+    prompt = synth.make_prompt(cfg, n=n).numpy()
+    token = next(t for t in range(cfg.vocab) if t not in prompt)
+    prompt[at] = token
+    w["tok_embed"][token, 3] = 0.5
+    rows = []
+    for broken in (False, True):
+        if broken and bad == "one value":
+            w["layers.0.wqkv"][(cfg.n_q_heads + cfg.n_kv_heads) * hd + 5, 3] = 3e38
+        elif broken:
+            w["tok_embed"][token, 3] = float("nan") if bad == "nan" else float("inf")
+        S = binding.Session(binding.Model(cfg, w), 1, n + 8, 64, 0)
+        S.prefill(prompt)
+        rows.append((_rows(S, cfg, range(max(0, at - 200), at)), _rows(S, cfg, [at]), _rows(S, cfg, [n - 1])))
+    (good, good_own, good_after), (before, own, after) = rows
+    assert np.isfinite(good).all() and np.isfinite(good_own).all() and np.isfinite(good_after).all()
+    assert np.array_equal(good, before)
+    assert np.array_equal(good_after[:2], after[:2]) and np.isnan(after[2:]).all()   # layer 0 sees the token itself only, the next one all
+    if bad == "one value":
+        assert np.array_equal(good_own[0], own[0]) and np.flatnonzero(~np.isfinite(own[1])).tolist() == [5]
+    else:
+        assert np.isnan(own).all()
