@@ -221,9 +221,11 @@ constexpr int kDenseMin = 9;        // prompt tokens from which the dense pass i
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
 constexpr int kPartMaxGrid = 256;
 
-// chunk partials of the decode attention as tagged words (see attn_consume_single)
+// chunk partials of the decode attention as tagged words (see attn_consume_single): the chunks that a phase with at most
+// ONE_ITEM_MAX work items, i.e. (kv head, chunk) pairs, can have; longer contexts exchange theirs through attn_part
+int attn_tag_chunks(const ada_config &g, int n_chunks) { return std::min(n_chunks, std::max(1, mg::ONE_ITEM_MAX / g.n_kv_heads)); }
 size_t attn_tag_bytes(const ada_config &g, int n_chunks) {
-    return sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)n_chunks * (g.head_dim + 2);
+    return sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)attn_tag_chunks(g, n_chunks) * (g.head_dim + 2);
 }
 
 Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, int head_blocks) {
@@ -849,6 +851,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     a.head_part = S->c.head_part;
     a.attn_cnt = (unsigned *)(b + lay.attn_cnt);
     a.attn_tag = (unsigned long long *)(b + lay.attn_tag);
+    a.tag_chunks = attn_tag_chunks(g, S->n_chunks);
     a.rope_freq = (const double *)(b + lay.rope_freq);
     a.part = S->grid <= kPartMaxGrid ? (unsigned long long *)(b + lay.part) : nullptr;
     a.grid_ctr = (unsigned *)(b + lay.grid_ctr);

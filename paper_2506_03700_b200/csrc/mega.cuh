@@ -30,6 +30,7 @@ using namespace st;
 constexpr int ACT_CONTINUE = 1, ACT_NEWSTEP = 2, ACT_STOP = 3;
 constexpr int CTRL_START = 0, CTRL_HEAD = 1, CTRL_TOP = 2;
 constexpr int ATT_PAGE = 64;          // cache positions per attention sub-block (= KV page size on this path)
+constexpr int ONE_ITEM_MAX = 256;     // most attention work items of a phase that gives every CTA at most one (attn_consume_single)
 constexpr int ATT_CHUNK = kAttnChunk; // positions per attention work item (fixed: anchored at position 0)
 constexpr int ERR_BAD_STATE = 3;
 
@@ -83,7 +84,8 @@ struct MegaArgs {
     const double *rope_freq;   // [hd/2]: base^(-2i/hd), computed once on the host
     unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
     unsigned *attn_cnt;        // [nkv]
-    unsigned long long *attn_tag;   // [8][nq][n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume_single); zeroed before each launch
+    unsigned long long *attn_tag;   // [8][nq][tag_chunks][hd + 2]: chunk partials as tagged words (see attn_consume_single); zeroed before each launch
+    int tag_chunks;            // chunks of a sequence they are laid out for: no more occur with ONE_ITEM_MAX work items in all
     unsigned *grid_ctr;
     Pub *pub;                  // [2]
     int *err;
@@ -1371,7 +1373,7 @@ __device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Sha
         }
         if (tid == 0) trace(S, EV_ATT, 5);   // sub-blocks done
         bar_consumers();   // every warp is done with the query fragments, whose space the merge reuses
-        auto words = [&](int cc, int h, int chunk) { return A.attn_tag + (((size_t)cc * c.nq + h) * c.n_chunks + chunk) * TS; };
+        auto words = [&](int cc, int h, int chunk) { return A.attn_tag + (((size_t)cc * c.nq + h) * A.tag_chunks + chunk) * TS; };
         if (one_tile) {
             if (mt == 0) attn_merge_to<NT, HD>(o, m_run, l_run, as->oq[qr], as->mlq[qr], lane);
             bar_consumers();
@@ -2015,12 +2017,13 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 phase_barrier(2);
             }
             // ---- attention (work items that hold no row of this pass are fetched before the QKV phase has ended)
+            const bool one_item = ROLE != 0 && attn_items(A, d, mask) <= min(G, ONE_ITEM_MAX);
             if (ROLE == 1) {
-                if (attn_items(A, d, mask) <= G) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
+                if (one_item) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
                 else attn_produce(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
             }
             if (ROLE == 2) {
-                if (attn_items(A, d, mask) <= G) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
+                if (one_item) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
                 else attn_consume<HD>(A, S, d, l, mask, r);
             }
             phase_barrier(4);

@@ -45,3 +45,19 @@ def test_host_side_argument_checks_need_no_gpu():
     assert lib.ada_session_scratch_bytes(h, 1, 256, 5) > 0
     assert lib.ada_kv_page_bytes(h, 64) == 4 * 2 * 4 * 64 * 64 * 4
     lib.ada_model_destroy(h)
+
+
+def test_session_scratch_does_not_pay_for_chunk_partials_that_cannot_occur():
+    """The tagged partials of the one-item attention path are laid out for the chunks that 256 work items can have (32 of 128
+    positions with eight kv heads), whatever the session's length: from there on a position costs its share of the other
+    buffers only (attention partials: 8 columns x 32 heads x 132 floats per 128 positions)."""
+    lib = binding.load()
+    h = ctypes.c_void_p()
+    cfg = binding.Config(32, 4096, 32, 8, 128, 14336, 128256, 1, 0, 500000.0, 1e-5)
+    assert lib.ada_model_create(ctypes.byref(cfg), ctypes.byref(h)) == 0
+    size = lambda n: lib.ada_session_scratch_bytes(h, 1, n, 5)
+    rows = 64
+    per_chunk = rows * 32 * (128 + 4) * 4 + 128 * 64     # partials of every row the per-operation path may carry; tokens, tables, random numbers
+    assert size(131072) - size(65536) <= 512 * per_chunk
+    assert size(8192) - size(4096) <= 32 * per_chunk
+    lib.ada_model_destroy(h)
