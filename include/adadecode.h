@@ -279,6 +279,13 @@ size_t ada_debug_dense_gemm_work_bytes(int32_t K);
 int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X_dev, int32_t rows, float *Y_dev, int32_t ldy,
                          int32_t accumulate, void *work_dev, size_t work_bytes, void *cuda_stream);
 
+/* The same product as the prompt pass runs it: up to 2048 rows, divided over `pairs` pairs of CTAs (0: all of the device's) as
+ * ada_debug_dense_plan says, cut tiles and running totals included.  work_dev: device scratch of
+ * ada_debug_dense_product_work_bytes(rows, K) bytes, 256-byte aligned; the rest as for ada_debug_dense_gemm. */
+size_t ada_debug_dense_product_work_bytes(int32_t rows, int32_t K);
+int ada_debug_dense_product(const void *W_dev, int32_t N, int32_t K, const float *X_dev, int32_t rows, int32_t pairs, float *Y_dev,
+                            int32_t ldy, int32_t accumulate, void *work_dev, size_t work_bytes, void *cuda_stream);
+
 /* Host-only: how the dense GEMM divides a product of `rows` positions with N weight rows (per_tile of them to a tile: 256;
  * 128 where gate and up are multiplied side by side) and depth K over `pairs` pairs of CTAs.  plan7 (host) receives
  * {positions per tile, position tiles, tiles, 64-wide k blocks of a chunk, chunks of a tile, groups of chunks, pairs in use};

@@ -33,7 +33,7 @@ EXPORTS = [
     "ada_debug_profile", "ada_debug_profile_read", "ada_debug_gemm", "ada_debug_gemm_plan", "ada_debug_gemm_work_bytes", "ada_debug_get_path", "ada_debug_set_launch_steps", "ada_debug_trace", "ada_gemm_noalloc",
     "ada_model_arena_bytes", "ada_model_set_arena", "ada_debug_set_wait_limit", "ada_debug_set_prefill",
     "ada_debug_dense_gemm", "ada_debug_dense_gemm_work_bytes", "ada_sampling_decode",
-    "ada_debug_dense_plan",
+    "ada_debug_dense_plan", "ada_debug_dense_product", "ada_debug_dense_product_work_bytes",
 ]
 
 
@@ -98,6 +98,9 @@ def load() -> C.CDLL:
         L.ada_debug_dense_gemm_work_bytes.restype = sz
         L.ada_debug_dense_gemm_work_bytes.argtypes = [i32]
         L.ada_debug_dense_gemm.argtypes = [vp, i32, i32, vp, i32, vp, i32, i32, vp, sz, vp]
+        L.ada_debug_dense_product_work_bytes.restype = sz
+        L.ada_debug_dense_product_work_bytes.argtypes = [i32, i32]
+        L.ada_debug_dense_product.argtypes = [vp, i32, i32, vp, i32, i32, vp, i32, i32, vp, sz, vp]
         L.ada_debug_dense_plan.argtypes = [i32, i32, i32, i32, i32, i32, C.POINTER(i32), vp, i32, C.POINTER(i32)]
         L.ada_model_destroy.argtypes = [vp]
         L.ada_model_destroy.restype = None
@@ -192,6 +195,24 @@ def debug_dense_gemm(W, X, Y=None):
     off = (-work.data_ptr()) % 256
     _ck(lib.ada_debug_dense_gemm(W.data_ptr(), N, K, X.data_ptr(), rows, Y.data_ptr(), Y.shape[1], 1 if acc else 0,
                                  work.data_ptr() + off, wb, torch.cuda.current_stream().cuda_stream), "ada_debug_dense_gemm")
+    return Y
+
+
+def debug_dense_product(W, X, Y=None, pairs: int = 0):
+    """ada_debug_dense_product: the dense GEMM over up to 2048 rows, divided over `pairs` pairs of CTAs (0: all) as the prompt
+    pass divides it.  W bf16 [N, K] (cuda), X fp32 [rows, K] (cuda); returns Y fp32 [rows, N], or Y += with Y given."""
+    import torch
+    lib = load()
+    (N, K), rows, acc = W.shape, X.shape[0], Y is not None
+    assert W.is_cuda and W.dtype == torch.bfloat16 and W.is_contiguous()
+    assert X.is_cuda and X.dtype == torch.float32 and X.is_contiguous() and X.shape[1] == K
+    if Y is None:
+        Y = torch.full((rows, N), float("nan"), dtype=torch.float32, device="cuda")
+    wb = lib.ada_debug_dense_product_work_bytes(rows, K)
+    work = torch.empty(wb + 256, dtype=torch.uint8, device="cuda")
+    off = (-work.data_ptr()) % 256
+    _ck(lib.ada_debug_dense_product(W.data_ptr(), N, K, X.data_ptr(), rows, pairs, Y.data_ptr(), Y.shape[1], 1 if acc else 0,
+                                    work.data_ptr() + off, wb, torch.cuda.current_stream().cuda_stream), "ada_debug_dense_product")
     return Y
 
 

@@ -455,7 +455,7 @@ template <int HD, int GROUP>
 int launch_attn_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int pos0, int rows, __nv_bfloat16 *oh, __nv_bfloat16 *ol) {
     const int per = 2 * dg::AT_Q / GROUP, grid = (rows + per - 1) / per * S->c.nkv;
     return launch_overlapped(S->stream, dg::k_pf_attn<HD, GROUP>, grid, dg::AT_THREADS, dg::at_smem_bytes<HD>(), pm.qh, pm.ql, S->pf_kv, S->c, layer, rows,
-                             seq, pos0, S->pf_kv_box, oh, ol, S->pf_err);
+                             seq, pos0, S->pf_kv_box, oh, ol, S->pf_err, S->wait_ns);
 }
 template <int HD, int GROUP> cudaError_t prepare_attn() {
     return cudaFuncSetAttribute(dg::k_pf_attn<HD, GROUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dg::at_smem_bytes<HD>());
@@ -472,7 +472,7 @@ int run_layer_dense(ada_session *S, const PfMaps &pm, int layer, int seq, int po
     typedef __nv_bfloat16 T;
     int rc;
     dg::GemmArgs a{};
-    a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.rstd = S->pf_rstd; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err;
+    a.rows = rows; a.layer = layer; a.seq = seq; a.pos0 = pos0; a.cs = S->pf_cs; a.rstd = S->pf_rstd; a.part = S->pf_part; a.flag = S->pf_flag; a.err = S->pf_err; a.wait_ns = S->wait_ns;
     a.Y = S->pf_resid; a.ldy = d;
     S->layer_passes++;
     S->launches += 7;
@@ -1734,11 +1734,51 @@ int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, i
     return ADA_OK;
 }
 
+namespace {
+
+// Y = or += X W^T with the given plan over the device scratch `work`: high and low parts of X, error word, published launch
+// numbers, exchange area (the last two only where the plan cuts tiles or keeps totals).
+size_t dense_work_bytes(int rows, int K, bool exchange) {
+    return align_up(2 * (size_t)rows * K * sizeof(__nv_bfloat16), 256) + 256 +
+           (exchange ? align_up(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS, 256) + dg::GPART_CTA * 2 * dg::MAX_PAIRS : 0);
+}
+int run_dense_product(const void *W, int N, int K, const float *X, int rows, const dg::GemmPlan &plan, float *Y, int ldy, bool accumulate,
+                      void *work, bool exchange, cudaStream_t stream) {
+    __nv_bfloat16 *hi = (__nv_bfloat16 *)work, *lo = hi + (size_t)rows * K;
+    char *rest = (char *)work + align_up(2 * (size_t)rows * K * sizeof(__nv_bfloat16), 256);
+    CUtensorMap mhi, mlo, mw;
+    int rc;
+    if ((rc = make_map_2d(&mhi, hi, rows, K, plan.nt / 2)) || (rc = make_map_2d(&mlo, lo, rows, K, plan.nt / 2)) || (rc = make_map_2d(&mw, W, N, K, dg::BW)))
+        return rc;
+    CK((prepare_dense<dg::EPI_STORE, 0>()));
+    CK((prepare_dense<dg::EPI_ADD, 0>()));
+    dg::GemmArgs a{};
+    a.plan = plan; a.rows = rows; a.N = N; a.K = K; a.Y = Y; a.ldy = ldy; a.err = (int *)rest; a.wait_ns = st::WAIT_NS_DEFAULT;
+    CK(cudaMemsetAsync(a.err, 0, sizeof(int), stream));
+    if (exchange) {
+        a.flag = (unsigned *)(rest + 256);
+        a.part = (float *)(rest + 256 + align_up(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS, 256));
+        a.epoch = 1;
+        CK(cudaMemsetAsync(a.flag, 0, sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS, stream));
+    }
+    dg::k_split_rows<<<rows, 256, 0, stream>>>(X, K, K, hi, lo);
+    CK(cudaGetLastError());
+    const Ctx none{};
+    rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, none, a);
+    if (rc) return rc;
+    int herr = 0;
+    CK(cudaMemcpyAsync(&herr, a.err, sizeof(int), cudaMemcpyDeviceToHost, stream));
+    CK(cudaStreamSynchronize(stream));
+    return herr ? ADA_ETIMEOUT : ADA_OK;
+}
+
+}  // namespace
+
 constexpr int kDenseDebugRows = 128;   // most rows of ada_debug_dense_gemm
 
 size_t ada_debug_dense_gemm_work_bytes(int32_t K) {
     if (K < 64) return 0;
-    return 2 * (size_t)kDenseDebugRows * K * sizeof(__nv_bfloat16) + 256;
+    return dense_work_bytes(kDenseDebugRows, K, false);
 }
 
 int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X_dev, int32_t rows, float *Y_dev, int32_t ldy,
@@ -1746,38 +1786,39 @@ int ada_debug_dense_gemm(const void *W_dev, int32_t N, int32_t K, const float *X
     if (!W_dev || !X_dev || !Y_dev || !work_dev || N < 1 || K < 64 || K % 64 || rows < 1 || rows > kDenseDebugRows || ldy < N) return ADA_EINVAL;
     if ((uintptr_t)W_dev % 16 || (uintptr_t)work_dev % 256 || (uintptr_t)Y_dev % 16 || ldy % 4) return ADA_EINVAL;
     if (work_bytes < ada_debug_dense_gemm_work_bytes(K)) return ADA_ECAPACITY;
-    int dev = 0, major = 0;
+    int dev = 0, major = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
     if (major != 10) return ADA_EUNSUPPORTED;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    __nv_bfloat16 *hi = (__nv_bfloat16 *)work_dev, *lo = hi + (size_t)kDenseDebugRows * K;
-    int *err = (int *)(lo + (size_t)kDenseDebugRows * K);
-    CUtensorMap mhi, mlo, mw;
-    int rc, sms = 0;
-    const int nt = position_tile(rows);
-    if ((rc = make_map_2d(&mhi, hi, rows, K, nt / 2)) || (rc = make_map_2d(&mlo, lo, rows, K, nt / 2)) || (rc = make_map_2d(&mw, W_dev, N, K, dg::BW)))
-        return rc;
-    CK((prepare_dense<dg::EPI_STORE, 0>()));
-    CK((prepare_dense<dg::EPI_ADD, 0>()));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    CK(cudaMemsetAsync(err, 0, sizeof(int), stream));
-    dg::k_split_rows<<<rows, 256, 0, stream>>>(X_dev, K, rows, K, hi, lo);
-    CK(cudaGetLastError());
-    dg::GemmArgs a{};
-    a.rows = rows; a.N = N; a.K = K; a.Y = Y_dev; a.ldy = ldy; a.err = err;
-    a.plan.nt = nt; a.plan.mt = 1; a.plan.tiles = a.plan.whole = (N + dg::TW - 1) / dg::TW; a.plan.groups = 1;
-    a.plan.ck = chunk_blocks(K);
-    a.plan.chunks = (K / dg::BK + a.plan.ck - 1) / a.plan.ck;
-    a.plan.pairs = std::max(1, std::min({a.plan.tiles, sms / 2, dg::MAX_PAIRS}));   // whole tiles: no exchange area needed
-    for (int i = 1; i < dg::MAX_GROUPS + 2; ++i) a.plan.group[i] = a.plan.chunks;
-    const Ctx none{};
-    rc = accumulate ? launch_dense<dg::EPI_ADD, 0>(stream, mhi, mlo, mw, mw, none, a) : launch_dense<dg::EPI_STORE, 0>(stream, mhi, mlo, mw, mw, none, a);
-    if (rc) return rc;
-    int herr = 0;
-    CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    CK(cudaStreamSynchronize(stream));
-    return herr ? ADA_ETIMEOUT : ADA_OK;
+    dg::GemmPlan plan{};   // whole tiles, one group: no exchange area needed
+    plan.nt = position_tile(rows); plan.mt = 1; plan.tiles = plan.whole = (N + dg::TW - 1) / dg::TW; plan.groups = 1;
+    plan.ck = chunk_blocks(K);
+    plan.chunks = (K / dg::BK + plan.ck - 1) / plan.ck;
+    plan.pairs = std::max(1, std::min({plan.tiles, sms / 2, dg::MAX_PAIRS}));
+    for (int i = 1; i < dg::MAX_GROUPS + 2; ++i) plan.group[i] = plan.chunks;
+    return run_dense_product(W_dev, N, K, X_dev, rows, plan, Y_dev, ldy, accumulate != 0, work_dev, false, (cudaStream_t)cuda_stream);
+}
+
+size_t ada_debug_dense_product_work_bytes(int32_t rows, int32_t K) {
+    if (rows < 1 || rows > dg::PF_ROWS || K < 64) return 0;
+    return dense_work_bytes(rows, K, true);
+}
+
+int ada_debug_dense_product(const void *W_dev, int32_t N, int32_t K, const float *X_dev, int32_t rows, int32_t pairs, float *Y_dev,
+                            int32_t ldy, int32_t accumulate, void *work_dev, size_t work_bytes, void *cuda_stream) {
+    if (!W_dev || !X_dev || !Y_dev || !work_dev || N < 1 || K < 64 || K % 64 || rows < 1 || rows > dg::PF_ROWS || ldy < N || pairs < 0) return ADA_EINVAL;
+    if ((uintptr_t)W_dev % 16 || (uintptr_t)work_dev % 256 || (uintptr_t)Y_dev % 16 || ldy % 4) return ADA_EINVAL;
+    if (work_bytes < ada_debug_dense_product_work_bytes(rows, K)) return ADA_ECAPACITY;
+    int dev = 0, major = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+    if (major != 10) return ADA_EUNSUPPORTED;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int most = std::min(sms / 2, dg::MAX_PAIRS);
+    if (pairs > most) return ADA_EINVAL;
+    return run_dense_product(W_dev, N, K, X_dev, rows, plan_dense(rows, N, dg::TW, K, pairs ? pairs : most), Y_dev, ldy, accumulate != 0, work_dev, true,
+                             (cudaStream_t)cuda_stream);
 }
 
 // ---- streaming GEMM without caller scratch ---------------------------------------------------------

@@ -68,7 +68,6 @@ constexpr int GREGS_ISSUE = 40, GREGS_EPI = 232;
 constexpr int W_BYTES = BW * BK * 2;
 constexpr int RING_BYTES = 196608;
 constexpr int TMEM_COLS = 512; // two accumulator buffers of 256 fp32 columns
-constexpr unsigned long long DENSE_WAIT_NS = 2000000000ull;
 constexpr int MAX_GROUPS = 4;
 constexpr size_t GPART_WARP = 128 * 32 * sizeof(float);           // sums of one epilogue warp
 constexpr size_t GPART_SLOT = GEPI_WARPS * GPART_WARP;
@@ -81,6 +80,7 @@ struct DSmem {   // must start on a 1024-byte boundary (swizzle pattern)
     alignas(1024) unsigned char ring[RING_BYTES];
     alignas(8) unsigned long long full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2];
     alignas(16) float stash[GEPI_WARPS][32][32];   // per epilogue warp: 32 positions x its 32 weight rows
+    unsigned long long wait_ns;
     uint32_t tmem_base;
     int abort;
 };
@@ -200,11 +200,11 @@ template <typename SM> __device__ __forceinline__ bool dwait(SM *sm, int *err, u
     unsigned long long t0 = 0;
     for (uint32_t it = 0;; ++it) {
         if (mbar_try(bar, parity)) return true;
-        if ((it & 255u) == 0) {
+        if ((it & 255u) == 0 || sm->wait_ns < SHORT_LIMIT_NS) {
             if (*(volatile int *)&sm->abort) return false;
             const unsigned long long t = gtime();
             if (t0 == 0) t0 = t;
-            else if (t - t0 > DENSE_WAIT_NS) {
+            else if (t - t0 > sm->wait_ns) {
                 atomicCAS(err, 0, ERR_TIMEOUT_MBAR);
                 *(volatile int *)&sm->abort = 1;
                 return false;
@@ -298,6 +298,7 @@ struct GemmArgs {
     unsigned *flag;               // [CTA][epilogue warp]: launch number of the sums published last
     unsigned epoch;
     int *err;
+    unsigned long long wait_ns;   // limit of every wait
 };
 
 // a pair of fp32 values as bf16 high parts and low parts
@@ -463,7 +464,7 @@ template <typename SM> __device__ __forceinline__ bool flag_wait(SM *sm, const G
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
         if (v == a.epoch) break;
         if (*(volatile int *)&sm->abort) { ok = false; break; }
-        if (gtime() - t0 > DENSE_WAIT_NS) {
+        if (gtime() - t0 > a.wait_ns) {
             atomicCAS(a.err, 0, ERR_TIMEOUT_MBAR);
             *(volatile int *)&sm->abort = 1;
             ok = false;
@@ -491,6 +492,7 @@ k_dense_gemm(const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__
         for (int i = 0; i < MAX_STAGES; ++i) { mbar_init(&sm->full[i], 1); mbar_init(&sm->empty[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&sm->acc_full[i], 1); mbar_init(&sm->acc_empty[i], 2 * GEPI_WARPS); }
         sm->abort = 0;
+        sm->wait_ns = a.wait_ns;
         fence_mbar_init();
         fence_proxy_async();
     }
@@ -790,12 +792,12 @@ __global__ void __launch_bounds__(256) k_norm_split_rows(const float *X, int K, 
     }
 }
 
-// fp32 rows X[r][ldx] (r < rows) -> the two bf16 matrices [128][K] the dense GEMM reads: high part and low part
-// (x = hi + lo); rows >= `rows` are zero.  One block per row.
-__global__ void k_split_rows(const float *__restrict__ X, int ldx, int rows, int K, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+// fp32 rows X[r][ldx] -> the two bf16 matrices [rows][K] the dense GEMM reads: high part and low part (x = hi + lo).  One
+// block per row.
+__global__ void k_split_rows(const float *__restrict__ X, int ldx, int K, __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
     const int r = blockIdx.x;
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const float v = r < rows ? X[(size_t)r * ldx + k] : 0.f;
+        const float v = X[(size_t)r * ldx + k];
         const __nv_bfloat16 h = __float2bfloat16_rn(v);
         hi[(size_t)r * K + k] = h;
         lo[(size_t)r * K + k] = __float2bfloat16_rn(v - __bfloat162float(h));
@@ -835,6 +837,7 @@ template <int HD> struct AtSmem {   // must start on a 1024-byte boundary
     alignas(8) unsigned long long q_full[2], kv_full[SLOTS], kv_empty[SLOTS], s_full[2], p_full[2], o_full[2], diag;
     int bad[HD];                                         // per feature: first position of a causally cut key tile whose V is not finite
     int any_bad;
+    unsigned long long wait_ns;
     uint32_t tmem_base;
     int abort;
 };
@@ -918,7 +921,7 @@ template <int HD, int GROUP>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CUtensorMap mapQlo, const __grid_constant__ CUtensorMap mapKV,
           const __grid_constant__ Ctx c, int layer, int rows, int seq, int pos0, int kv_box, __nv_bfloat16 *ohi,
-          __nv_bfloat16 *olo, int *err) {
+          __nv_bfloat16 *olo, int *err, unsigned long long wait_ns) {
     typedef AtSmem<HD> Sm;
     constexpr int PT = AT_Q / GROUP, SLOTS = Sm::SLOTS, HG = HD / 64;
     extern __shared__ unsigned char dsm_raw[];
@@ -940,6 +943,7 @@ k_pf_attn(const __grid_constant__ CUtensorMap mapQhi, const __grid_constant__ CU
         mbar_init(&sm->diag, 1);
         sm->any_bad = 0;
         sm->abort = 0;
+        sm->wait_ns = wait_ns;
         fence_mbar_init();
         fence_proxy_async();
     }

@@ -90,3 +90,33 @@ def test_sums_of_the_dense_gemm(N, K, rows, depth):
     ref = (hi.double() + lo.double()) @ W.double().T
     err = (binding.debug_dense_gemm(W, X).double() - ref).norm() / ref.norm()
     assert err <= 1.6e-8 * (2 * depth / 16) + 1e-7, err
+
+
+def _product(N, K, rows, pairs=0, seed=9):
+    W = synth.normal_tensor(seed, 11, (N, K), 0.05, torch.bfloat16, "cuda")
+    X = synth.normal_tensor(seed, 12, (rows, K), 1.0, torch.float32, "cuda")
+    return W, X, binding.debug_dense_product(W, X, pairs=pairs)
+
+
+# tiles of 256 weight rows x one position tile against `pairs` pairs of CTAs: one short of a wave, a wave, one more, two waves and one
+# more; several position tiles; depths that are no multiple of a chunk or leave a last group shorter
+@pytest.mark.parametrize("N,K,rows,pairs", [
+    (73 * 256, 1088, 100, 74), (74 * 256, 1088, 64, 74), (75 * 256, 1088, 33, 74), (149 * 256, 576, 40, 74),
+    (4 * 256, 3008, 100, 5), (5 * 256, 3008, 100, 5), (6 * 256, 3008, 256, 5), (11 * 256, 3008, 256, 5), (3 * 256 - 60, 5504, 300, 7),
+    (4096, 14336, 777, 74), (6144, 4096, 2048, 74), (2048, 8192, 513, 74), (256, 14336, 257, 74), (64, 64, 2048, 74), (300, 192, 1, 74)])
+def test_divided_products_match_float64(N, K, rows, pairs):
+    W, X, Y = _product(N, K, rows, pairs)
+    ref = X.double() @ W.double().T
+    assert torch.isfinite(Y).all()
+    # the split of X leaves 2^-17 of an element at most, 2.5e-6 of a result in the 2-norm; the sums 1.1e-6 (test_sums_of_the_dense_gemm)
+    assert (Y.double() - ref).norm() <= 3e-6 * ref.norm()
+    assert (Y.double() - ref).abs().max() <= 2e-5 * max(1.0, ref.abs().max())
+    Y2 = binding.debug_dense_product(W, X, torch.ones_like(Y), pairs=pairs)
+    assert (Y2.double() - (ref + 1.0)).abs().max() <= 2e-5 * max(1.0, ref.abs().max())
+
+
+@pytest.mark.parametrize("N,K", [(2048, 8192), (4096, 3008), (19 * 256, 5504)])
+def test_rows_of_a_divided_product_do_not_depend_on_how_many_there_are(N, K):
+    W, X, Y = _product(N, K, 2048)
+    for rows in (32, 97, 256, 260, 600, 1111):
+        assert torch.equal(binding.debug_dense_product(W, X[:rows].contiguous()), Y[:rows]), rows

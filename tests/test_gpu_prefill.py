@@ -169,3 +169,25 @@ def test_a_token_that_is_not_finite_leaves_the_positions_before_it_alone(hd, nq,
         assert np.array_equal(good_own[0], own[0]) and np.flatnonzero(~np.isfinite(own[1])).tolist() == [5]
     else:
         assert np.isnan(own).all()
+
+
+@pytest.mark.parametrize("hd,nq,nkv", [(64, 4, 2), (128, 2, 2)])
+def test_a_wait_that_runs_out_ends_the_prompt_pass_with_a_timeout_and_the_session_recovers(hd, nq, nkv):
+    """The dense pass's waits end at the session's limit like the decode kernel's: set far below what a copy takes, the call
+    returns ADA_ETIMEOUT, and with the usual limit the same session gives what a fresh one gives."""
+    cfg, gm = _model(hd, nq, nkv)
+    prompt = synth.make_prompt(cfg, n=300).numpy()
+    F = binding.Session(gm, 1, 400, 64, 0)
+    F.prefill(prompt)
+    S = binding.Session(gm, 1, 400, 64, 0)
+    S.set_wait_limit(20)                  # nanoseconds
+    with pytest.raises(binding.AdaError) as e:
+        S.prefill(prompt)
+    assert e.value.code == -5
+    torch.cuda.synchronize()              # the context is intact
+    S.set_wait_limit(2_000_000_000)
+    S.reset()
+    S.prefill(prompt)
+    positions = (0, 127, 128, 299)
+    assert np.array_equal(_rows(S, cfg, positions), _rows(F, cfg, positions))
+    assert np.array_equal(S.plain_decode(4), F.plain_decode(4))
