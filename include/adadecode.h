@@ -213,8 +213,8 @@ int ada_debug_profile_read(ada_session *s, double *ms_out, int64_t *launches_out
  * or 128, at most 4 q heads per kv head, d_model / n_q_heads*head_dim / d_ff multiples of 64); it is
  * the default wherever a session qualifies; a session that qualifies but cannot be set up fails in
  * ada_session_create instead of taking the other path).  0 = one kernel per operation on CUDA cores
- * (any dtype, any batch; sequences of a batch share every layer pass).  On path 1 the sequences of a batch are
- * decoded one after another, each streaming the weights for itself.  ADA_EUNSUPPORTED if path 1 is asked of a
+ * (any dtype, any batch; sequences of a batch share every layer pass).  On path 1 the sequences of a batch share
+ * a launch, and its weight stream, as far as eight token columns go (max_early + 1 each).  ADA_EUNSUPPORTED if path 1 is asked of a
  * session that does not qualify.
  * ada_stats.path reports the path a decode call ran on. */
 int ada_debug_set_path(ada_session *s, int32_t path);
@@ -228,9 +228,9 @@ int ada_debug_set_prefill(ada_session *s, int32_t dense);
 /* Steps of Algorithm 1 one launch of the persistent kernel may start before it returns to the host
  * (default 256; the host relaunches until the call is complete). */
 int ada_debug_set_launch_steps(ada_session *s, int32_t steps);
-/* Every wait inside the persistent kernel (on a shared-memory barrier, on the grid-wide counter, on
- * another CTA's partial sums) gives up after `ns` nanoseconds (default 2 s): the kernel then sets an
- * error word, lets every other wait fall through, ends, and the decode call returns ADA_ETIMEOUT.
+/* Every wait inside the persistent kernel and the dense prompt pass (on a shared-memory barrier, on the grid-wide counter,
+ * on another CTA's partial sums) gives up after `ns` nanoseconds (default 2 s): the kernel then sets an
+ * error word, lets every other wait fall through, ends, and the decode or prefill call returns ADA_ETIMEOUT.
  * The sequence state is undefined after that; ada_session_reset + ada_prefill make the session
  * usable again.  A limit shorter than a grid-wide wait normally lasts (a few microseconds) makes the
  * next decode call time out: that is how the give-up path is tested. */

@@ -339,7 +339,7 @@ def test_a_wait_that_runs_out_ends_the_call_with_a_timeout_and_the_session_recov
 
 @pytest.mark.parametrize("mk,n_prompt", [(gqa, 200), (hd128, 131), (mha, 77)])
 def test_dense_prompt_pass_matches_the_pass_through_the_decode_path_and_the_oracle(mk, n_prompt):
-    """KV cache <- LM(x): prompts of 32 tokens or more run in blocks of 128 positions through the tcgen05
+    """KV cache <- LM(x): prompts of 9 tokens or more run in blocks of up to 2048 positions through the tcgen05
     GEMMs.  The cache it leaves and the first token agree with the prompt pass through the decode kernel
     (eight positions at a time) within the cache's bf16 rounding, and decoding on from it matches the oracle."""
     cfg = mk()
