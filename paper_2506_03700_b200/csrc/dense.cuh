@@ -8,13 +8,12 @@
 // activations lose nothing), both multiplied into the same fp32 accumulator: 4 m n k floating-point operations.
 //
 // What bounds it.  Below about 128 positions the weights' way from HBM, above it the tensor cores and the L2 cache
-// together: the gate / up product of a 1024-position block keeps the tensor pipe 82 % busy while 10.9 TB/s move from L2 to
-// the SMs (ncu).  The weights are the 256-row operand of a pair of CTAs, the positions the other one, 32 to 256 wide in
+// together: the gate / up product of a 1024-position block of the 8B shape keeps the tensor pipe 79 % busy while 8.7 TB/s
+// move from L2 to the SMs (profiles/k_dense_gemm_8b_1024_ncu.md).  The weights are the 256-row operand of a pair of CTAs, the positions the other one, 32 to 256 wide in
 // steps of 32: a block is cut into equal position tiles, so that little is multiplied for padding (777 positions: 4 tiles
 // of 224; with positions as the 256-row operand a prompt of 45 positions cost as much as one of 256).  At full width a
 // k block of 64 costs a CTA 48 KB of shared-memory fill per 1024 tensor-core cycles; one CTA per tile of 128 x 128 needed
-// 48 KB per 512 cycles and 2.7 times the L2 traffic per weight byte.  Two accumulators of 128 positions (gate and up side
-// by side) were 15 % slower than one of 256: at that width the operands' way out of shared memory is the bound.
+// 48 KB per 512 cycles and 2.7 times the L2 traffic per weight byte.
 //
 // Accumulation.  The tensor core adds into its fp32 accumulator with truncation, so an accumulator falls short by
 // 1.5e-8 of the sum per addition (1e-3 absolute at K = 14336 with sums of size 10).  A product is therefore cut into chunks
@@ -355,7 +354,7 @@ template <bool ADD> __device__ __forceinline__ void epi_rows(const float (*x)[32
     const int n = 4 * (lane & 7);
     y += n;
     if (n + 4 <= n_left) {
-float4 r[8];
+        float4 r[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = 4 * i + (lane >> 3);
