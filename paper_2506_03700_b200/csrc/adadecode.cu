@@ -45,40 +45,8 @@ struct LayerW {
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Tensor map of a row-major bf16 weight matrix [N][K] for the streaming GEMM: dimensions (64
-// elements, N rows, K/64 groups), box (64, 16, 8), 128-byte swizzle, zero fill outside.  The
-// driver entry point is looked up at run time, so the library loads without libcuda.
-int make_weight_map(CUtensorMap *out, const void *W, int N, int K) {
-    typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                 const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static EncodeFn encode = nullptr;
-    if (!encode) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult qr;
-        cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qr);
-        if (e != cudaSuccess || qr != cudaDriverEntryPointSuccess || !fn) {
-            g_cuda_err = std::string("cuTensorMapEncodeTiled is not available: ") + cudaGetErrorString(e);
-            return ADA_ECUDA;
-        }
-        encode = (EncodeFn)fn;
-    }
-    if (K % 64 || N < 1 || (uintptr_t)W % 16) return ADA_EUNSUPPORTED;
-    const cuuint64_t dims[3] = {64, (cuuint64_t)N, (cuuint64_t)(K / 64)};
-    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, 128};
-    const cuuint32_t box[3] = {64, (cuuint32_t)st::TILE_N, (cuuint32_t)st::KG};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(W), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        g_cuda_err = "cuTensorMapEncodeTiled failed with CUresult " + std::to_string((int)r);
-        return ADA_ECUDA;
-    }
-    return ADA_OK;
-}
-
-// Tensor map of bf16 data: dims innermost first, strides in bytes of dims 1.., zero fill outside.
+// Tensor map of bf16 data: dims innermost first, strides in bytes of dims 1.., zero fill outside.  The driver entry point is
+// looked up at run time, so the library loads without libcuda.
 int make_map(CUtensorMap *out, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, bool swizzle) {
     typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -103,6 +71,15 @@ int make_map(CUtensorMap *out, const void *base, int rank, const cuuint64_t *dim
         return ADA_ECUDA;
     }
     return ADA_OK;
+}
+// A row-major weight matrix [N][K] as the streaming GEMM reads it: dimensions (64 elements, N rows, K / 64 groups), box
+// (64, 16, 8), 128-byte swizzle.
+int make_weight_map(CUtensorMap *out, const void *W, int N, int K) {
+    if (K % 64 || N < 1 || (uintptr_t)W % 16) return ADA_EUNSUPPORTED;
+    const cuuint64_t dims[3] = {64, (cuuint64_t)N, (cuuint64_t)(K / 64)};
+    const cuuint64_t strides[2] = {(cuuint64_t)K * 2, 128};
+    const cuuint32_t box[3] = {64, (cuuint32_t)st::TILE_N, (cuuint32_t)st::KG};
+    return make_map(out, W, 3, dims, strides, box, true);
 }
 // A row-major matrix [rows][K] as the dense products read it: box (64, box_rows), 128-byte swizzle.
 int make_map_2d(CUtensorMap *out, const void *base, int rows, int K, int box_rows) {
@@ -252,7 +229,9 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
     L.rope_cs = take(sizeof(float) * (size_t)R * g.head_dim);
     L.attn_part = take(sizeof(float) * (size_t)R * g.n_q_heads * n_chunks * (g.head_dim + 2));
     L.head_part = take(sizeof(float) * (size_t)head_blocks * kMaxRows * 4);
-    L.logit_stage = take(sizeof(float) * (size_t)R * g.vocab);
+    // staged logits; a prompt's products exchange sums in the same memory (a head's logits are read within its own step)
+    const size_t exchange = model_fits_persistent(g) ? dg::GPART_CTA * 2 * dg::MAX_PAIRS : 0;
+    L.logit_stage = L.pf_part = take(std::max(sizeof(float) * (size_t)R * g.vocab, exchange));
     L.head_log = take(sizeof(float) * 4 * kHeadLogCap);
     L.t_out = take(sizeof(float) * (size_t)R * g.d_model);
     if (model_fits_persistent(g)) {   // dense prompt pass: residual and the two bf16 parts of every product's input
@@ -264,7 +243,6 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.pf_rstd = take(sizeof(float) * P);
         L.pf_err = take(256);
         L.pf_flag = take(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS);
-        L.pf_part = take(dg::GPART_CTA * 2 * dg::MAX_PAIRS);
     }
     // persistent-kernel buffers (bf16 models)
     if (g.dtype == ADA_DTYPE_BF16) {
@@ -852,6 +830,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     a.attn_cnt = (unsigned *)(b + lay.attn_cnt);
     a.attn_tag = (unsigned long long *)(b + lay.attn_tag);
     a.tag_chunks = attn_tag_chunks(g, S->n_chunks);
+    a.one_item_max = std::min(S->grid, mg::ONE_ITEM_MAX);
     a.rope_freq = (const double *)(b + lay.rope_freq);
     a.part = S->grid <= kPartMaxGrid ? (unsigned long long *)(b + lay.part) : nullptr;
     a.grid_ctr = (unsigned *)(b + lay.grid_ctr);

@@ -85,6 +85,7 @@ struct MegaArgs {
     unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
     unsigned *attn_cnt;        // [nkv]
     unsigned long long *attn_tag;   // [8][nq][tag_chunks][hd + 2]: chunk partials as tagged words (see attn_consume_single); zeroed before each launch
+    int one_item_max;          // min(grid, ONE_ITEM_MAX)
     int tag_chunks;            // chunks of a sequence they are laid out for: no more occur with ONE_ITEM_MAX work items in all
     unsigned *grid_ctr;
     Pub *pub;                  // [2]
@@ -2017,13 +2018,12 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 phase_barrier(2);
             }
             // ---- attention (work items that hold no row of this pass are fetched before the QKV phase has ended)
-            const bool one_item = ROLE != 0 && attn_items(A, d, mask) <= min(G, ONE_ITEM_MAX);
             if (ROLE == 1) {
-                if (one_item) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
+                if (attn_items(A, d, mask) <= A.one_item_max) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
                 else attn_produce(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
             }
             if (ROLE == 2) {
-                if (one_item) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
+                if (attn_items(A, d, mask) <= A.one_item_max) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
                 else attn_consume<HD>(A, S, d, l, mask, r);
             }
             phase_barrier(4);
