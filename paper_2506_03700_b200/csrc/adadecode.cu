@@ -140,8 +140,6 @@ struct ada_session {
     int grid = 0;
     mg::MegaArgs margs;
     CUtensorMap *maps_dev = nullptr;      // [6 L + 2]: wqkv, wo, wgu, wup, wdown per layer, lm_head, then T per 1-based layer
-    mg::MegaModel *mm_dev = nullptr;
-    int *exit_at_dev = nullptr;
     bool sampling = false;   // the call in progress draws its tokens (ada_sampling_decode)
     float inv_temp = 1.0f;
     int steps_per_launch = 256;
@@ -173,7 +171,6 @@ struct ada_session {
     int32_t *head_log_n_out = nullptr;
     std::vector<uint8_t> tape;
     std::vector<CUtensorMap> maps_host;
-    std::unique_ptr<mg::MegaModel> mm_host;
 };
 
 namespace {
@@ -181,7 +178,7 @@ namespace {
 // Scratch layout (all offsets 256-byte aligned).
 struct Layout {
     size_t st, rt, fill, tokens, page_table, head_res, resid, xn, qkv, q, attn_out, gu, hact, rope_cs, attn_part,
-        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, maps, mm, exit_at, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
+        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, maps, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
         grid_ctr, pub, err, attn_tag, q_stage, qinfo, uniforms, total;
 };
 
@@ -247,8 +244,6 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
     // persistent-kernel buffers (bf16 models)
     if (g.dtype == ADA_DTYPE_BF16) {
         L.maps = take(sizeof(CUtensorMap) * (6 * (size_t)g.n_layers + 2));
-        L.mm = take(sizeof(mg::MegaModel));
-        L.exit_at = take(sizeof(int) * (g.n_layers + 1));
         L.xa = take(st::xfrag_bytes(g.d_model));
         L.xb = take(st::xfrag_bytes(g.d_model));
         L.xf = take(st::xfrag_bytes(g.d_model));
@@ -782,45 +777,35 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     const int L = g.n_layers;
     char *b = (char *)S->scratch;
     S->maps_dev = (CUtensorMap *)(b + lay.maps);
-    S->mm_dev = (mg::MegaModel *)(b + lay.mm);
-    S->exit_at_dev = (int *)(b + lay.exit_at);
-    S->maps_host.assign(6 * (size_t)L + 2, CUtensorMap());
-    S->mm_host.reset(new mg::MegaModel());
-    mg::MegaModel &M = *S->mm_host;
+    S->maps_host.assign((mg::MAPS_PER_LAYER + 1) * (size_t)L + 2, CUtensorMap());
+    mg::MegaModel &M = S->margs.m;
     memset(&M, 0, sizeof(M));
     int rc;
     for (int l = 0; l < L; ++l) {
         const LayerW &w = m->layers[l];
+        CUtensorMap *wm = &S->maps_host[mg::MAPS_PER_LAYER * (size_t)l];
         const bool gu_fused = (const __nv_bfloat16 *)w.w_up == (const __nv_bfloat16 *)w.w_gate + (size_t)g.d_ff * g.d_model;
         if (!w.wqkv_perm) return ADA_ESTATE;
-        if ((rc = make_weight_map(&S->maps_host[5 * l + 0], w.wqkv_perm, S->c.qkv_rows, g.d_model))) return rc;
-        if ((rc = make_weight_map(&S->maps_host[5 * l + 1], w.wo, g.d_model, qd))) return rc;
-        if ((rc = make_weight_map(&S->maps_host[5 * l + 2], w.w_gate, gu_fused ? 2 * g.d_ff : g.d_ff, g.d_model))) return rc;
-        if (!gu_fused && (rc = make_weight_map(&S->maps_host[5 * l + 3], w.w_up, g.d_ff, g.d_model))) return rc;
-        if ((rc = make_weight_map(&S->maps_host[5 * l + 4], w.w_down, g.d_model, g.d_ff))) return rc;
-        M.layer[l].wqkv = S->maps_dev + 5 * l + 0;
-        M.layer[l].wo = S->maps_dev + 5 * l + 1;
-        M.layer[l].wgu = S->maps_dev + 5 * l + 2;
-        M.layer[l].wup = gu_fused ? nullptr : S->maps_dev + 5 * l + 3;
-        M.layer[l].wdown = S->maps_dev + 5 * l + 4;
-        M.layer[l].attn_norm = (const __nv_bfloat16 *)w.attn_norm;
-        M.layer[l].ffn_norm = (const __nv_bfloat16 *)w.ffn_norm;
+        if ((rc = make_weight_map(wm + 0, w.wqkv_perm, S->c.qkv_rows, g.d_model))) return rc;
+        if ((rc = make_weight_map(wm + 1, w.wo, g.d_model, qd))) return rc;
+        if ((rc = make_weight_map(wm + 2, w.w_gate, gu_fused ? 2 * g.d_ff : g.d_ff, g.d_model))) return rc;
+        if (!gu_fused && (rc = make_weight_map(wm + 3, w.w_up, g.d_ff, g.d_model))) return rc;
+        if ((rc = make_weight_map(wm + 4, w.w_down, g.d_model, g.d_ff))) return rc;
+        M.gu_two[l] = !gu_fused;
+        M.attn_norm[l] = (const __nv_bfloat16 *)w.attn_norm;
+        M.ffn_norm[l] = (const __nv_bfloat16 *)w.ffn_norm;
     }
-    if ((rc = make_weight_map(&S->maps_host[5 * L], m->lm_head, g.vocab, g.d_model))) return rc;
-    M.lm_head = S->maps_dev + 5 * L;
+    if ((rc = make_weight_map(&S->maps_host[mg::MAPS_PER_LAYER * (size_t)L], m->lm_head, g.vocab, g.d_model))) return rc;
+    M.maps = S->maps_dev;
     M.tok_embed = (const __nv_bfloat16 *)m->tok_embed;
     M.final_norm = (const __nv_bfloat16 *)m->final_norm;
-    M.rope_base = g.rope_base;
     CK(cudaMemcpyAsync(S->maps_dev, S->maps_host.data(), sizeof(CUtensorMap) * S->maps_host.size(), cudaMemcpyHostToDevice, S->stream));
-    CK(cudaMemcpyAsync(S->mm_dev, &M, sizeof(M), cudaMemcpyHostToDevice, S->stream));
     std::vector<double> freq(g.head_dim / 2);
     for (int i = 0; i < g.head_dim / 2; ++i) freq[i] = pow((double)g.rope_base, -2.0 * i / g.head_dim);
     CK(cudaMemcpyAsync(b + lay.rope_freq, freq.data(), sizeof(double) * freq.size(), cudaMemcpyHostToDevice, S->stream));
     CK(cudaStreamSynchronize(S->stream));
     mg::MegaArgs &a = S->margs;
     a.c = S->c;
-    a.mm = S->mm_dev;
-    a.exit_at = S->exit_at_dev;
     a.XA = (__nv_bfloat16 *)(b + lay.xa); a.XB = (__nv_bfloat16 *)(b + lay.xb); a.XO = (__nv_bfloat16 *)(b + lay.xo);
     a.XH = (__nv_bfloat16 *)(b + lay.xh); a.XF = (__nv_bfloat16 *)(b + lay.xf); a.XT = (__nv_bfloat16 *)(b + lay.xt);
     a.ssq_a = (float *)(b + lay.ssq_a); a.ssq_b = (float *)(b + lay.ssq_b);
@@ -862,31 +847,26 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
     const ada_model *m = S->m;
     const ada_config &g = m->cfg;
     const int L = g.n_layers;
-    std::vector<int> ex(L + 1, 0);
-    mg::MegaModel &M = *S->mm_host;
+    mg::MegaModel &M = S->margs.m;
+    memset(M.exit_at, 0, sizeof(M.exit_at));
     if (!plain) {
         for (int i = 0; i < n_exit; ++i) {
             const int e = exit_layers[i];
-            ex[e] = 1 + i;
-            M.layer[e].has_head = 1;
-            M.layer[e].head_scale = m->head_scale[e];
-            M.layer[e].wT = nullptr;
+            M.exit_at[e] = (unsigned char)(1 + i);
+            M.head_scale[e] = m->head_scale[e];
+            M.has_T[e] = m->head_T[e] != nullptr;
             if (m->head_T[e]) {
-                CUtensorMap &tm = S->maps_host[5 * (size_t)L + 1 + e];
+                const size_t at = mg::MAPS_PER_LAYER * (size_t)L + 1 + e;
+                CUtensorMap &tm = S->maps_host[at];
                 int rc = make_weight_map(&tm, m->head_T[e], g.d_model, g.d_model);
                 if (rc) return rc;
-                CK(cudaMemcpyAsync(S->maps_dev + 5 * L + 1 + e, &tm, sizeof(tm), cudaMemcpyHostToDevice, S->stream));
-                M.layer[e].wT = S->maps_dev + 5 * L + 1 + e;
+                CK(cudaMemcpyAsync(S->maps_dev + at, &tm, sizeof(tm), cudaMemcpyHostToDevice, S->stream));
             }
-            CK(cudaMemcpyAsync(&S->mm_dev->layer[e], &M.layer[e], sizeof(mg::MegaLayer), cudaMemcpyHostToDevice, S->stream));
         }
     }
-    CK(cudaMemcpyAsync(S->exit_at_dev, ex.data(), sizeof(int) * (L + 1), cudaMemcpyHostToDevice, S->stream));
     // a call that ended on a device-side error may have left the error word and the attention counters set
     CK(cudaMemsetAsync(S->margs.err, 0, sizeof(int), S->stream));
     CK(cudaMemsetAsync(S->margs.attn_cnt, 0, sizeof(unsigned) * g.n_kv_heads * st::MAX_COLS, S->stream));
-    CK(cudaStreamSynchronize(S->stream));   // ex and the maps live on the host until copied
-    S->syncs++;
     const void *kern = persistent_kernel_for(g.head_dim);
     const int per_launch = together ? std::max(1, st::MAX_COLS / S->slots) : 1;
     for (int sq = seq_begin; sq < seq_end; sq += per_launch) {
@@ -1636,10 +1616,7 @@ int ada_debug_gemm_plan(int32_t N, int32_t K, int32_t mode, int32_t grid, int32_
     if (!out9 || N < 1 || K < 64 || K % 64 || mode < 0 || mode > 1 || grid < 1 || cta < 0 || cta >= grid) return ADA_EINVAL;
     if (mode == 1 && (N % 2 || (N / 2) % 16)) return ADA_EINVAL;
     st::Gemm g;
-    memset(&g, 0, sizeof(g));
-    g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0; g.ctas = grid;
-    static unsigned long long dummy;
-    g.part = split ? &dummy : nullptr;   // only tested for null by the plan
+    g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0; g.split = split != 0;
     const st::Plan p = st::make_plan(g, cta, grid);
     const int32_t v[9] = {p.split, p.t0, p.t1, p.n, p.ta, p.tb, p.s0_own_k0, p.s0_pub_k1, p.sl_k1};
     memcpy(out9, v, sizeof(v));
@@ -1671,7 +1648,7 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     CK(cudaMemsetAsync(err, 0, sizeof(int), stream));
     CK(cudaMemcpyAsync(dmap, &hmap, sizeof(hmap), cudaMemcpyHostToDevice, stream));
     CK(cudaStreamSynchronize(stream));   // hmap lives on this stack frame
-    k_xfrag_pack<<<(K + 255) / 256, 256, 0, stream>>>(X_dev, K, cols, (__nv_bfloat16 *)work_dev);
+    k_xfrag_pack<<<(K + st::KC - 1) / st::KC * 2, st::KC / 2, 0, stream>>>(X_dev, K, cols, (__nv_bfloat16 *)work_dev);
     CK(cudaGetLastError());
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
@@ -1842,7 +1819,7 @@ int ada_gemm_noalloc(const void *W_dev, int32_t N, int32_t K, int32_t mode, cons
     CK(cudaMemsetAsync(err, 0, sizeof(int), stream));   // the one word that must start at zero
     CK(cudaMemcpyAsync(dmap, &hmap, sizeof(hmap), cudaMemcpyHostToDevice, stream));
     CK(cudaStreamSynchronize(stream));   // hmap lives on this stack frame
-    k_xfrag_pack<<<(K + 255) / 256, 256, 0, stream>>>(X_dev, K, cols, (__nv_bfloat16 *)base);
+    k_xfrag_pack<<<(K + st::KC - 1) / st::KC * 2, st::KC / 2, 0, stream>>>(X_dev, K, cols, (__nv_bfloat16 *)base);
     CK(cudaGetLastError());
     k_gemm_probe<<<sms_of_device[dev], st::THREADS, st::SMEM_BYTES, stream>>>(dmap, N, K, mode, (const uint4 *)base, Y_dev, ldy, cols, 1, err, nullptr);
     CK(cudaGetLastError());

@@ -6,11 +6,11 @@
 
 namespace ada {
 
-// fp32 activations X[cols][K] -> fragment layout (high/low bf16 split).
+// fp32 activations X[cols][K] -> fragment layout (high/low bf16 split), the last block padded with zeros.
 __global__ void k_xfrag_pack(const float *__restrict__ X, int K, int cols, __nv_bfloat16 *__restrict__ out) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    for (int c = 0; c < st::MAX_COLS; ++c) st::xfrag_store(out, k, c, c < cols ? X[(size_t)c * K + k] : 0.f);
+    if (k >= (K + st::KC - 1) / st::KC * st::KC) return;
+    for (int c = 0; c < st::MAX_COLS; ++c) st::xfrag_store(out, k, c, c < cols && k < K ? X[(size_t)c * K + k] : 0.f);
 }
 
 // mode 0: Y[col][n] = sum_k W[n][k] X[col][k]                       (N rows)
@@ -23,42 +23,30 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
     st::smem_init(sm);
     __syncthreads();
     st::Shared S{sm, err, st::Trace{nullptr, nullptr, 0}, 0, st::WAIT_NS_DEFAULT};
-    st::Gemm g;
-    g.W = W; g.X = X; g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0;
-    g.ctas = st::balanced_ctas(g.tiles(), gridDim.x);
-    g.cp0 = 0; g.ncp = (cols + 1) / 2;
-    // tiles split between CTAs need a grid-wide meeting between products: only for a single product
-    g.part = repeat == 1 ? part : nullptr; g.phase_id = 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cta = blockIdx.x, G = gridDim.x;
-    st::Rings r{0, 0};
+    st::Gemm g;
+    g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0;
+    // tiles split between CTAs need a grid-wide meeting between products: only for a single product
+    g.split = repeat == 1 && part != nullptr;
+    const st::Plan pl = st::make_plan(g, cta, G);
+    const st::Cols cols_used((1u << cols) - 1u);
+    st::Rings r;
     if (warp == st::CONS_WARPS) {
         const uint64_t pol = st::policy_evict_first();
-        for (int it = 0; it < repeat; ++it) st::gemm_produce_w(S, g, cta, G, r, pol);
+        for (int it = 0; it < repeat; ++it) st::gemm_produce_w(S, pl, W, nullptr, r, pol);
     } else if (warp == st::CONS_WARPS + 1) {
         const uint64_t pol = st::policy_evict_last();
-        for (int it = 0; it < repeat; ++it) st::gemm_produce_x(S, g, cta, G, r, pol);
+        for (int it = 0; it < repeat; ++it) st::gemm_produce_x(S, pl, X, cols_used, r, pol, st::NoHook(), st::NoHook());
     } else {
-        for (int it = 0; it < repeat; ++it) {
-            if (mode == 0) {
-                st::gemm_consume<1>(S, g, cta, G, r, [&](int tile, float (&d)[1][4]) {
+        for (int it = 0; it < repeat; ++it)
+            st::gemm_consume(S, pl, cols_used, part, 1u, cta, r, st::NoPre(), [&](int tile, float (&d0)[4], float (&d1)[4]) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
-                        if (n < N && c < cols) Y[(size_t)c * ldy + n] = d[0][i];
-                    }
-                });
-            } else {
-                st::gemm_consume<2>(S, g, cta, G, r, [&](int tile, float (&d)[2][4]) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
-                        const float gv = d[0][i], u = d[1][i];
-                        if (n < g.half && c < cols) Y[(size_t)c * ldy + n] = gv / (1.0f + expf(-gv)) * u;
-                    }
-                });
-            }
-        }
+                for (int i = 0; i < 4; ++i) {
+                    const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
+                    if (n < (mode == 0 ? N : g.half) && c < cols) Y[(size_t)c * ldy + n] = mode == 0 ? d0[i] : d0[i] / (1.0f + expf(-d0[i])) * d1[i];
+                }
+            });
     }
     st::settle_on_abort(S);
 }

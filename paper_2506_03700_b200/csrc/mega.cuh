@@ -55,27 +55,25 @@ struct Pub {                   // what CTA 0 publishes at a control point
     int pad[5];
 };
 
-struct MegaLayer {
-    // wqkv: the fused q | k | v matrix with the rows of every q and k head reordered for the rotation (see the QKV phase);
-    // wgu: gate stacked over up, or the gate matrix alone when wup is set (the two lent as separate tensors)
-    const CUtensorMap *wqkv, *wo, *wgu, *wup, *wdown, *wT;
-    const __nv_bfloat16 *attn_norm, *ffn_norm;
-    float head_scale;
-    int has_head;
-};
-
+// What the phases need to know of the model.  It travels as a kernel argument: the constant bank answers at once, where a
+// pointer read from global memory was a round trip to L2 in front of the loads that depend on it (the L1 copy does not
+// survive the acquire of a grid barrier).
 struct MegaModel {
-    const CUtensorMap *lm_head;
+    // per layer: wqkv (the fused q | k | v matrix with the rows of every q and k head reordered for the rotation, see the QKV
+    // phase), wo, wgu (gate stacked over up, or gate alone where gu_two is set), wup, wdown; then the LM head; then T per 1-based layer
+    const CUtensorMap *maps;
     const __nv_bfloat16 *tok_embed, *final_norm;
-    float rope_base;
-    int pad;
-    MegaLayer layer[ADA_MAX_LAYERS + 1];   // [l] for 0-based layer l; head fields of 1-based layer e live in layer[e]
+    const __nv_bfloat16 *attn_norm[ADA_MAX_LAYERS], *ffn_norm[ADA_MAX_LAYERS];
+    float head_scale[ADA_MAX_LAYERS + 1];        // by 1-based layer
+    unsigned char exit_at[ADA_MAX_LAYERS + 1];   // 1 + the index of 1-based layer e among the call's exit layers if the call consults its head, else 0
+    unsigned char has_T[ADA_MAX_LAYERS + 1];     // that head has a transformation of its own
+    unsigned char gu_two[ADA_MAX_LAYERS];        // gate and up are separate tensors
 };
+enum { MAPS_PER_LAYER = 5 };
 
 struct MegaArgs {
     Ctx c;
-    const MegaModel *mm;
-    const int *exit_at;        // [L + 1]: 1 + the index of 1-based layer e among the call's exit layers if the call consults its head, else 0
+    MegaModel m;
     __nv_bfloat16 *XA, *XB, *XO, *XH, *XF, *XT;   // GEMM inputs in fragment layout (see stream.cuh)
     float *ssq_a, *ssq_b;      // [d/16][8] partial sums of squares of the residual (per 16-feature tile, per column)
     uint32_t *qfrag;           // [nkv][2][hd/16][32][8]: rotated, scaled queries as tensor-core A fragments (bf16 high parts, then low parts)
@@ -142,17 +140,20 @@ __device__ __forceinline__ void rstd_produce(Smem *sm, const float *ssq, int nti
     if (lane == 0) *(volatile unsigned *)&sm->vec_seq = seq;
 }
 
-// Grid barrier as seen by the consumers of a CTA.
-__device__ __forceinline__ void barrier_consumers(const Shared &S, unsigned *ctr, unsigned &bar_no, int G, int cls) {
+// The end of a phase as seen by the consumers of a CTA: they report it to the grid and go on.  Whoever needs what the other
+// CTAs wrote waits for the counter: the activation producer before it fetches a product's input, the consumers themselves
+// (consumers_meet) where they read other CTAs' results directly.  Consumers of a product wait for its first input stage only,
+// and set up its epilogue's operands while the grid is still meeting.
+__device__ __forceinline__ void consumers_arrive(const Shared &S, unsigned *ctr, int cls) {
     if (threadIdx.x == 0) trace(S, EV_EPI_END, cls);
     bar_consumers();
-    ++bar_no;
     if (threadIdx.x == 0) {
         grid_arrive(ctr);
         trace(S, EV_ARRIVE, cls);
-        grid_wait(S, ctr, bar_no * (unsigned)G);
-        trace(S, EV_PHASE_BEGIN, cls);
     }
+}
+__device__ __forceinline__ void consumers_meet(const Shared &S, const unsigned *ctr, unsigned target) {
+    if (threadIdx.x == 0) grid_wait(S, ctr, target);
     bar_consumers();
 }
 
@@ -567,7 +568,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                                           int &steps_started) {
     const Ctx &c = A.c;
     DevState *st = c.st;
-    const MegaModel &M = *A.mm;
+    const MegaModel &M = A.m;
     const int tid = threadIdx.x, G = gridDim.x;
     const int nseq = A.nseq, seq0 = A.seq0, cps = c.slots, L = c.L;   // cps: token columns per sequence
     Pub *pub = A.pub + (pub_no & 1);
@@ -603,7 +604,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     // (a') sampled decoding replaces the tokens and probabilities the bookkeeping below works with
     if (A.sampling && kind != CTRL_START && !(kind == CTRL_TOP && st->pf_end > 0)) {
         SampleArgs sa{A.uniforms, A.q_stage, A.qinfo, c.logit_stage, c.head_res, st, c.vocab, c.max_seq, cps, L, seq0, nseq,
-                      kind == CTRL_HEAD ? A.exit_at[e] - 1 : 0, A.head_part, G};
+                      kind == CTRL_HEAD ? (int)M.exit_at[e] - 1 : 0, A.head_part, G};
         sample_stage(sa, sm, kind == CTRL_HEAD, &dprev, head_cols);
     }
     // (b) bookkeeping, one thread.  Every scalar it may need is read up front (the loads overlap);
@@ -818,7 +819,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     // (c) the embedding of the next newest token
     if (action == ACT_NEWSTEP) {
         const StepDesc &nd = pub->d;
-        const __nv_bfloat16 *g0 = M.layer[0].attn_norm;
+        const __nv_bfloat16 *g0 = M.attn_norm[0];
         const int half = c.hd / 2;
         for (int col = 0; col < MAX_COLS; ++col) {
             if (!((nd.fresh >> col) & 1)) continue;
@@ -1076,15 +1077,15 @@ __device__ __forceinline__ void attn_produce(const MegaArgs &A, const Shared &S,
                     if (!it[g].have || sb >= it[g].nsb) continue;
                     const int32_t *pages = c.page_table + (size_t)(A.seq0 + it[g].k) * c.max_pages;
                     const int page = pages[(it[g].p_base + sb * ATT_PAGE) >> c.page_shift];
-                    const int slot = r.xi % NX;
-                    mbar_wait(S, &sm->x_empty[slot], ((r.xi / NX) & 1) ^ 1);
+                    const uint32_t slot = r.xs;
+                    mbar_wait(S, &sm->x_empty[slot], r.xp ^ 1);
                     if (lane == 0 && !aborted(S)) {
                         const size_t blk = ((((size_t)page * c.L + layer) * 2 + which) * c.nkv + it[g].kvh) * ((size_t)ATT_PAGE * c.hd);
                         mbar_expect_tx(&sm->x_full[slot], bytes);
                         bulk_g2s(sm->x[slot], pool + blk, bytes, &sm->x_full[slot], pol);
                         trace(S, EV_ATT, 9 + 16 * (2 * sb + which));
                     }
-                    ++r.xi;
+                    r.next_x();
                 }
     }
 }
@@ -1119,15 +1120,15 @@ __device__ __forceinline__ void attn_produce_single(const MegaArgs &A, const Sha
         for (int sb = 0; sb < nsb; ++sb) {
             const int page = pages[(p_base + sb * ATT_PAGE) >> c.page_shift];
             for (int which = 0; which < 2; ++which) {
-                const int slot = r.xi % NX;
-                mbar_wait(S, &sm->x_empty[slot], ((r.xi / NX) & 1) ^ 1);
+                const uint32_t slot = r.xs;
+                mbar_wait(S, &sm->x_empty[slot], r.xp ^ 1);
                 if (lane == 0 && !aborted(S)) {
                     const size_t blk = ((((size_t)page * c.L + layer) * 2 + which) * c.nkv + kvh) * ((size_t)ATT_PAGE * c.hd);
                     mbar_expect_tx(&sm->x_full[slot], bytes);
                     bulk_g2s(sm->x[slot], pool + blk, bytes, &sm->x_full[slot], pol);
                     trace(S, EV_ATT, 9 + 16 * (2 * sb + which));
                 }
-                ++r.xi;
+                r.next_x();
             }
         }
     }
@@ -1268,8 +1269,8 @@ __device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Sha
             const int p0 = p_base + sb * ATT_PAGE;
             float s[2][4];
             {   // ---- K block
-                const int slot = r.xi % NX;
-                mbar_wait(S, &sm->x_full[slot], (r.xi / NX) & 1);
+                const uint32_t slot = r.xs;
+                mbar_wait(S, &sm->x_full[slot], r.xp);
                 if (tid == 0) trace(S, EV_ATT, 3 + 16 * sb);   // K block landed
                 const unsigned char *kb = sm->x[slot];
                 float sh[2][4], sl[2][4];
@@ -1310,7 +1311,7 @@ __device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Sha
                     }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                ++r.xi;
+                r.next_x();
             }
             // ---- online softmax over this warp's 16 positions
             uint32_t ph[4], plo[4];
@@ -1338,8 +1339,8 @@ __device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Sha
                 plo[2 + rh] = pack_bf16(p[2] - __low2float(h1), p[3] - __high2float(h1));
             }
             {   // ---- V block
-                const int slot = r.xi % NX;
-                mbar_wait(S, &sm->x_full[slot], (r.xi / NX) & 1);
+                const uint32_t slot = r.xs;
+                mbar_wait(S, &sm->x_full[slot], r.xp);
                 if (tid == 0) trace(S, EV_ATT, 4 + 16 * sb);   // V block landed
                 const unsigned char *vb = sm->x[slot];
                 const int id = lane >> 3;
@@ -1362,7 +1363,7 @@ __device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Sha
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                ++r.xi;
+                r.next_x();
             }
         }
         // ---- row sums over the quad, then merge the four position quarters of each query tile:
@@ -1603,8 +1604,8 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
 #pragma unroll 1
             for (int g = 0; g < per_round; ++g) {   // ---- K block(s)
                 if (!itg[g].have || sb >= itg[g].nsb) continue;
-                const int slot = r.xi % NX;
-                mbar_wait(S, &sm->x_full[slot], (r.xi / NX) & 1);
+                const uint32_t slot = r.xs;
+                mbar_wait(S, &sm->x_full[slot], r.xp);
                 if (tid == 0) trace(S, EV_ATT, 3 + 16 * sb);   // K block landed
                 if (!dual || g == mt) {
                     const unsigned char *kb = sm->x[slot];
@@ -1647,7 +1648,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                ++r.xi;
+                r.next_x();
             }
             // ---- online softmax over this warp's 16 positions
             uint32_t ph[4] = {0u, 0u, 0u, 0u}, plo[4] = {0u, 0u, 0u, 0u};
@@ -1679,8 +1680,8 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
 #pragma unroll 1
             for (int g = 0; g < per_round; ++g) {   // ---- V block(s)
                 if (!itg[g].have || sb >= itg[g].nsb) continue;
-                const int slot = r.xi % NX;
-                mbar_wait(S, &sm->x_full[slot], (r.xi / NX) & 1);
+                const uint32_t slot = r.xs;
+                mbar_wait(S, &sm->x_full[slot], r.xp);
                 if (tid == 0) trace(S, EV_ATT, 4 + 16 * sb);   // V block landed
                 if (!dual || g == mt) {
                     const unsigned char *vb = sm->x[slot];
@@ -1705,7 +1706,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                ++r.xi;
+                r.next_x();
             }
         }
         // ---- row sums over the quad, then merge the four position quarters of each warp group:
@@ -1783,33 +1784,259 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
 
 // ---------------------------------------------------------------- the walker
 
-template <int ROLE, int PAIR, class Ready, class Epi>
-__device__ __forceinline__ void gemm_phase(const Shared &S, const Gemm &g, Rings &r, uint64_t pol, Ready &&ready, Epi &&epi) {
-    const int cta = blockIdx.x, G = gridDim.x;
-    if (ROLE == 0) gemm_produce_w(S, g, cta, G, r, pol);
-    else if (ROLE == 1) gemm_produce_x(S, g, cta, G, r, pol, NoHook(), ready);
-    else gemm_consume<PAIR>(S, g, cta, G, r, epi);
+// Phases of a step.  The first six are products; their plans are worked out once per launch (Smem::plan).
+enum { PH_QKV = 0, PH_O, PH_GU, PH_DOWN, PH_T, PH_HEAD, PH_PRODUCTS, PH_ATTN = PH_PRODUCTS };
+__device__ __forceinline__ int prof_class(int ph) {   // class of ada_debug_profile that the phase's time is booked to
+    return ph == PH_QKV ? 2 : ph == PH_ATTN ? 4 : ph == PH_O ? 5 : ph == PH_GU ? 6 : ph == PH_DOWN ? 8 : ph == PH_T ? 10 : 9;
+}
+// The one product of the layer where the unit-balanced split pays is gate / up (measured: it shortens it by 1.4 us, but
+// lengthens down, QKV and O, whose tile groups are k-split among the warps).
+__device__ __forceinline__ Gemm phase_gemm(const MegaArgs &A, int ph) {
+    const Ctx &c = A.c;
+    Gemm g;
+    g.N = ph == PH_QKV ? c.qkv_rows : ph == PH_GU ? 2 * c.dff : ph == PH_HEAD ? c.vocab : c.d;
+    g.K = ph == PH_O ? c.nq * c.hd : ph == PH_DOWN ? c.dff : c.d;
+    g.pair = ph == PH_GU ? 2 : 1;
+    g.half = ph == PH_GU ? c.dff : 0;
+    g.split = ph == PH_GU && A.part != nullptr;
+    return g;
 }
 
-struct NoEpi {
-    template <class T> __device__ __forceinline__ void operator()(int, T &) const {}
+// Epilogues of the products: consumer warps, see gemm_consume.  lane / 4 (+ 8) is the row of the tile, 2 (lane % 4) + {0, 1} the columns.
+template <int HD> struct Epilogue {
+    const MegaArgs &A;
+    const Shared &S;
+    const StepDesc &d;
+    int ph, l;               // phase, 0-based layer
+    unsigned mask;           // columns of the product
+    unsigned vseq;           // phase number whose normalisation factors vec[] has to hold
+    bool scaled;             // the product's result is multiplied by them
+    float scale;             // head: scale of the logits
+    bool inter;              // head: an intermediate one
+    bool next_in, final_in;  // down product: prepares the next layer's input, a head's input
+
+    static constexpr int HALF = HD / 2, KSQ = HD / 16;
+
+    // operands fetched while the weights stream
+    __device__ __forceinline__ void pre(int tile) const {
+        const Ctx &c = A.c;
+        const int lane = threadIdx.x & 31, rq = lane >> 2, c0 = 2 * (lane & 3), n0 = tile * 16;
+        uint32_t *stash = stash_of(S.sm);
+        if (ph == PH_QKV) {   // rotary factors and cache pages of this lane's two columns
+            const int qd = c.nq * HD, kvd = c.nkv * HD;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int cc = c0 + q;
+                if (!((mask >> cc) & 1u)) continue;
+                if (n0 < qd + kvd) {
+                    const float *cs = c.rope_cs + ((size_t)cc * HALF + ((n0 & (HD - 1)) >> 1) + rq) * 2;
+                    cp_async4(stash + (2 * q) * 32, cs);
+                    cp_async4(stash + (2 * q + 1) * 32, cs + 1);
+                }
+                if (n0 >= qd) cp_async4(stash + (4 + q) * 32, c.page_table + (size_t)(A.seq0 + (A.nseq == 1 ? 0 : cc / c.slots)) * c.max_pages + (d.pos[cc] >> c.page_shift));
+            }
+        } else if (ph == PH_O || ph == PH_DOWN) {   // residual and gains
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int n = n0 + rq + (i >> 1) * 8, cc = c0 + (i & 1);
+                if ((mask >> cc) & 1u) cp_async4(stash + i * 32, c.resid + (size_t)cc * c.d + n);
+            }
+            const __nv_bfloat16 *g1 = ph == PH_O ? A.m.ffn_norm[l] : A.m.attn_norm[next_in ? l + 1 : l];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int n2 = (n0 + rq + h * 8) & ~1;
+                cp_async4(stash + (4 + h) * 32, g1 + n2);
+                if (final_in) cp_async4(stash + (6 + h) * 32, A.m.final_norm + n2);
+            }
+        }
+    }
+    __device__ __forceinline__ void qkv(int tile, float (&acc)[4], float r0, float r1) const {
+        const Ctx &c = A.c;
+        const int lane = threadIdx.x & 31, rq = lane >> 2, c0 = 2 * (lane & 3), n0 = tile * 16;
+        const int qd = c.nq * HD, kvd = c.nkv * HD, group = c.group;
+        const float qscale = rsqrtf((float)HD);
+        uint32_t *stash = stash_of(S.sm);
+        __nv_bfloat16 *pool = reinterpret_cast<__nv_bfloat16 *>(c.kv_pool);
+        if (n0 >= c.qkv_rows) return;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int cc = c0 + q;
+            if (!((mask >> cc) & 1u)) continue;
+            const float rs = q ? r1 : r0;
+            const float x0 = acc[q] * rs, x1 = acc[2 + q] * rs;   // rows rq and rq + 8 of the tile
+            if (n0 < qd + kvd) {
+                const float co = __uint_as_float(stash[(2 * q) * 32]), si = __uint_as_float(stash[(2 * q + 1) * 32]);
+                const int j = ((n0 & (HD - 1)) >> 1) + rq;   // feature j pairs with j + hd/2
+                const float y0 = x0 * co - x1 * si, y1 = x1 * co + x0 * si;
+                if (n0 < qd) {
+                    const int h = n0 / HD, kvh = div_group(h, group), qcol = cc * group + (h - kvh * group);
+                    const int row = qcol & 15, m = qcol >> 4;
+                    __nv_bfloat16 *f0 = reinterpret_cast<__nv_bfloat16 *>(A.qfrag + (((size_t)kvh * 2 + m) * KSQ) * 256);
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {
+                        const int dim = j + hh * HALF;
+                        const float y = (hh ? y1 : y0) * qscale;
+                        const int ks = dim >> 4, kk = dim & 15;
+                        const int ln = (row & 7) * 4 + ((kk & 7) >> 1), reg = (row >> 3) + 2 * (kk >> 3);
+                        const __nv_bfloat16 hi = __float2bfloat16_rn(y);
+                        const __nv_bfloat16 lo = __float2bfloat16_rn(y - __bfloat162float(hi));
+                        __nv_bfloat16 *f = f0 + ((size_t)ks * 32 + ln) * 16;
+                        f[reg * 2 + (kk & 1)] = hi;
+                        f[8 + reg * 2 + (kk & 1)] = lo;
+                    }
+                } else {
+                    const int kvh = (n0 - qd) / HD, pos = d.pos[cc], t = pos & (ATT_PAGE - 1);
+                    const size_t blk = ((((size_t)stash[(4 + q) * 32] * c.L + l) * 2 + 0) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)t * HD;
+                    pool[blk + ((((j >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(y0);
+                    pool[blk + (((((j + HALF) >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(y1);
+                }
+            } else {
+                const int nv = n0 - qd - kvd, kvh = nv / HD, j = (nv & (HD - 1)) + rq, pos = d.pos[cc], t = pos & (ATT_PAGE - 1);
+                const size_t blk = ((((size_t)stash[(4 + q) * 32] * c.L + l) * 2 + 1) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)t * HD;
+                pool[blk + ((((j >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(x0);
+                pool[blk + (((((j + 8) >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(x1);
+            }
+        }
+    }
+    // O and down: residual add, inputs of the products that follow, partial sums of squares
+    __device__ __forceinline__ void residual(int tile, float (&acc)[4]) const {
+        const Ctx &c = A.c;
+        const int lane = threadIdx.x & 31, c0 = 2 * (lane & 3);
+        const uint32_t *stash = stash_of(S.sm);
+        __nv_bfloat16 *X1 = ph == PH_O ? A.XB : A.XA;
+        float *ssq = ph == PH_O ? A.ssq_b : A.ssq_a;
+        float sq[2] = {0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
+            if ((mask >> cc) & 1u) {
+                const float v = __uint_as_float(stash[i * 32]) + acc[i];
+                c.resid[(size_t)cc * c.d + n] = v;
+                if (next_in) xfrag_store(X1, n, cc, v * bf16_of_word(stash[(4 + (i >> 1)) * 32], n));
+                if (final_in) xfrag_store(A.XF, n, cc, v * bf16_of_word(stash[(6 + (i >> 1)) * 32], n));
+                sq[i & 1] += v * v;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 4);
+            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 8);
+            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 16);
+            if (lane < 4 && ((mask >> (c0 + q)) & 1u)) ssq[(size_t)tile * MAX_COLS + c0 + q] = sq[q];
+        }
+    }
+    __device__ __forceinline__ void operator()(int tile, float (&a0)[4], float (&a1)[4]) const {
+        const Ctx &c = A.c;
+        const int lane = threadIdx.x & 31, c0 = 2 * (lane & 3);
+        float r0 = 1.f, r1 = 1.f;
+        if (scaled) { vec_wait(S, vseq); r0 = S.sm->vec[c0]; r1 = S.sm->vec[c0 + 1]; }
+        if (ph == PH_GU) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
+                if ((mask >> cc) & 1u) {
+                    const float rs = (i & 1) ? r1 : r0;
+                    const float gv = a0[i] * rs, u = a1[i] * rs;
+                    xfrag_store(A.XH, n, cc, gv / (1.0f + expf(-gv)) * u);
+                }
+            }
+        } else if (ph == PH_HEAD) {
+            // running (max, sum exp, argmax) of this lane's two columns, kept in its stash words; sampled decoding: logits over
+            // the temperature, which are kept, the final head's by column, an intermediate head's by the position of its row
+            // (the verification of the token drawn from them needs them again)
+            uint32_t *stash = stash_of(S.sm);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int col = c0 + q;
+                const float f = (q ? r1 : r0) * scale;
+                float *zrow = nullptr;
+                if ((mask >> col) & 1u) {
+                    if (A.sampling && inter) zrow = A.q_stage + ((size_t)(A.seq0 + (A.nseq == 1 ? 0 : col / c.slots)) * MAX_COLS + (d.pos[col] & 7)) * c.vocab;
+                    else if (A.sampling || A.store_logits) zrow = c.logit_stage + (size_t)col * c.vocab;
+                }
+                Msa run;
+                run.m = __uint_as_float(stash[(3 * q) * 32]); run.s = __uint_as_float(stash[(3 * q + 1) * 32]); run.i = (int)stash[(3 * q + 2) * 32];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int n = tile * 16 + (lane >> 2) + h * 8;
+                    if (n < c.vocab) {
+                        const float z = a0[q + 2 * h] * f;
+                        if (zrow) zrow[n] = z;
+                        Msa one; one.m = z; one.s = 1.f; one.i = n;
+                        run = msa_merge(run, one);
+                    }
+                }
+                stash[(3 * q) * 32] = __float_as_uint(run.m); stash[(3 * q + 1) * 32] = __float_as_uint(run.s); stash[(3 * q + 2) * 32] = (uint32_t)run.i;
+            }
+        } else if (ph == PH_T) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
+                xfrag_store(A.XT, n, cc, a0[i] * ((i & 1) ? r1 : r0));
+            }
+        } else {
+            cp_async_wait_all();
+            if (ph == PH_QKV) qkv(tile, a0, r0, r1);
+            else residual(tile, a0);
+        }
+    }
+    __device__ __forceinline__ void head_begin() const {
+        uint32_t *stash = stash_of(S.sm);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) { stash[(3 * q) * 32] = __float_as_uint(-INFINITY); stash[(3 * q + 1) * 32] = 0u; stash[(3 * q + 2) * 32] = (uint32_t)INT_MAX; }
+    }
+    // the CTA's (max, sum exp, argmax) per column: lanes sharing lane%4 hold the same columns; they are folded, then the warps, in a fixed order
+    __device__ __forceinline__ void head_end() const {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c0 = 2 * (lane & 3);
+        const uint32_t *stash = stash_of(S.sm);
+        float *wp = reinterpret_cast<float *>(S.sm->scratch);   // [warp][col][4]
+        bar_consumers();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            Msa run;
+            run.m = __uint_as_float(stash[(3 * q) * 32]); run.s = __uint_as_float(stash[(3 * q + 1) * 32]); run.i = (int)stash[(3 * q + 2) * 32];
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {
+                Msa o;
+                o.m = __shfl_xor_sync(0xffffffffu, run.m, off);
+                o.s = __shfl_xor_sync(0xffffffffu, run.s, off);
+                o.i = __shfl_xor_sync(0xffffffffu, run.i, off);
+                run = msa_merge(run, o);
+            }
+            if (lane < 4) {
+                float *o = wp + ((size_t)warp * MAX_COLS + c0 + q) * 4;
+                o[0] = run.m; o[1] = run.s; o[2] = __int_as_float(run.i);
+            }
+        }
+        bar_consumers();
+        if (threadIdx.x < MAX_COLS) {
+            Msa a; a.m = -INFINITY; a.s = 0.f; a.i = INT_MAX;
+            for (int w = 0; w < CONS_WARPS; ++w) {
+                const float *o = wp + ((size_t)w * MAX_COLS + threadIdx.x) * 4;
+                Msa x; x.m = o[0]; x.s = o[1]; x.i = __float_as_int(o[2]);
+                a = msa_merge(a, x);
+            }
+            float *o = A.head_part + ((size_t)blockIdx.x * MAX_COLS + threadIdx.x) * 4;
+            o[0] = a.m; o[1] = a.s; o[2] = __int_as_float(a.i);
+        }
+    }
 };
 
 // ROLE 0: weight producer warp, 1: activation / KV producer warp, 2: consumer warps.
+//
+// A step is a sequence of phases; every role walks it with one loop whose body holds each piece of code once (one product, one
+// attention, one control point) and takes from the phase number what differs.
 template <int ROLE, int HD>
 __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
     const Ctx &c = A.c;
-    const MegaModel &M = *A.mm;
+    const MegaModel &M = A.m;
     Smem *sm = S.sm;
-    const int G = gridDim.x, lane = threadIdx.x & 31;
-    const int L = c.L, d_model = c.d, qd = c.nq * c.hd, ntd = d_model / 16;
+    const int G = gridDim.x;
+    const int L = c.L, d_model = c.d, ntd = d_model / 16;
     const uint64_t pol = ROLE == 0 ? policy_evict_first() : policy_evict_last();
-    Rings r{0, 0};
-    unsigned bar_no = 0, pub_no = 0;
+    Rings r;
+    unsigned bar_no = 0, pub_no = 0;   // phases and control points behind this role
     int steps_started = 0;
-    // CTAs that share the tiles of each kind of GEMM (the rest idle through that phase)
-    const int n_qkv = balanced_ctas((c.qkv_rows + 15) / 16, G), n_d = balanced_ctas(ntd, G), n_gu = balanced_ctas(c.dff / 16, G),
-              n_head = balanced_ctas((c.vocab + 15) / 16, G);
     // The step descriptor lives in shared memory, one copy per role (the roles pass a control point at
     // different times): indexed by a run-time column it would otherwise sit in local memory, whose
     // cached lines do not survive the acquire of a grid barrier -- every first touch after a barrier
@@ -1822,361 +2049,114 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
     }
     if (ROLE == 2) bar_consumers(); else __syncwarp();
 
-    // barrier between phases, per role; CTA 0 books the time since the previous one to the phase's class
     unsigned long long t_last = gtime();
-    auto phase_barrier = [&](int cls) {
-        if (ROLE == 2) {
-            barrier_consumers(S, A.grid_ctr, bar_no, G, cls);
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                const unsigned long long t = gtime();
-                // reductions, not read-modify-write: thread 0 of CTA 0 must not wait for a load from L2 at every barrier
-                atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_ns[cls]), t - t_last);
-                atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_count[cls]), 1ull);
-                t_last = t;
-            }
-        } else ++bar_no;
-    };
-    auto book_control = [&]() {
+    auto book = [&](int cls) {   // CTA 0 books the time since the last event to a class
         if (ROLE == 2 && blockIdx.x == 0 && threadIdx.x == 0) {
             const unsigned long long t = gtime();
-            atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_ns[0]), t - t_last);
-            atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_count[0]), 1ull);
+            // reductions, not read-modify-write: thread 0 of CTA 0 must not wait for a load from L2 at every phase
+            atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_ns[cls]), t - t_last);
+            atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_count[cls]), 1ull);
             t_last = t;
         }
     };
-    // the activation producer must not fetch a phase's input before the phase that wrote it is complete
-    auto x_ready = [&]() {
-        if (ROLE == 1) {
-            grid_wait(S, A.grid_ctr, bar_no * (unsigned)G);
-            fence_proxy_async();
-        }
-    };
-    // head over E* with the fused (max, sum exp, argmax) reduction; X = final-normed residual (or T output)
-    auto head_phase = [&](const __nv_bfloat16 *X, const float *ssq, float scale, unsigned cols, bool inter) {
-        Gemm g; g.W = M.lm_head; g.X = reinterpret_cast<const uint4 *>(X); g.N = c.vocab; g.K = d_model; g.pair = 1; g.half = 0; g.ctas = n_head; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(cols);
-        const unsigned vseq = bar_no + 1;
-        if (ROLE == 2) {
-            Msa run[2];
-            run[0].m = run[1].m = -INFINITY; run[0].s = run[1].s = 0.f; run[0].i = run[1].i = INT_MAX;
-            const int c0 = 2 * (lane & 3);
-            // sampled decoding: logits over the temperature; they are kept, the final head's by column, an intermediate
-            // head's by the position of its row (the verification of the token drawn from them needs them again)
-            if (A.sampling) scale *= A.inv_temp;
-            float *zrow[2] = {nullptr, nullptr};
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int col = c0 + q;
-                if (!((cols >> col) & 1u)) continue;
-                if (A.sampling && inter) zrow[q] = A.q_stage + ((size_t)(A.seq0 + (A.nseq == 1 ? 0 : col / c.slots)) * MAX_COLS + (d.pos[col] & 7)) * c.vocab;
-                else if (A.sampling || A.store_logits) zrow[q] = c.logit_stage + (size_t)col * c.vocab;
-            }
-            float r0 = scale, r1 = scale;
-            bool have_r = ssq == nullptr;
-            gemm_consume<1>(S, g, blockIdx.x, G, r, [&](int tile, float (&acc)[1][4]) {
-                if (!have_r) { vec_wait(S, vseq); r0 = sm->vec[c0] * scale; r1 = sm->vec[c0 + 1] * scale; have_r = true; }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8;
-                    if (n < c.vocab) {
-                        const float z = acc[0][i] * ((i & 1) ? r1 : r0);
-                        if (zrow[i & 1]) zrow[i & 1][n] = z;
-                        Msa one; one.m = z; one.s = 1.f; one.i = n;
-                        run[i & 1] = msa_merge(run[i & 1], one);
-                    }
-                }
-            });
-            // lanes sharing lane%4 hold the same columns: fold them, then the warps, in a fixed order
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-#pragma unroll
-                for (int off = 4; off < 32; off <<= 1) {
-                    Msa o;
-                    o.m = __shfl_xor_sync(0xffffffffu, run[q].m, off);
-                    o.s = __shfl_xor_sync(0xffffffffu, run[q].s, off);
-                    o.i = __shfl_xor_sync(0xffffffffu, run[q].i, off);
-                    run[q] = msa_merge(run[q], o);
-                }
-            }
-            const int warp = threadIdx.x >> 5;
-            float *wp = reinterpret_cast<float *>(sm->scratch);   // [warp][col][4]
-            bar_consumers();
-            if (lane < 4) {
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    float *o = wp + ((size_t)warp * MAX_COLS + c0 + q) * 4;
-                    o[0] = run[q].m; o[1] = run[q].s; o[2] = __int_as_float(run[q].i);
-                }
-            }
-            bar_consumers();
-            if (threadIdx.x < MAX_COLS) {
-                Msa a; a.m = -INFINITY; a.s = 0.f; a.i = INT_MAX;
-                for (int w = 0; w < CONS_WARPS; ++w) {
-                    const float *o = wp + ((size_t)w * MAX_COLS + threadIdx.x) * 4;
-                    Msa x; x.m = o[0]; x.s = o[1]; x.i = __float_as_int(o[2]);
-                    a = msa_merge(a, x);
-                }
-                float *o = A.head_part + ((size_t)blockIdx.x * MAX_COLS + threadIdx.x) * 4;
-                o[0] = a.m; o[1] = a.s; o[2] = __int_as_float(a.i);
-            }
-        } else if (ROLE == 1) {
-            gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { if (ssq) rstd_produce(sm, ssq, ntd, d_model, c.eps, vseq); }, x_ready);
-        } else {
-            gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
-        }
-        phase_barrier(9);
-    };
 
-    int action = control_point<ROLE>(A, S, CTRL_START, 0, pub_no, d, steps_started);
-    book_control();
-    int step_i = 0;
-    while (action == ACT_NEWSTEP) {
-        bool restart = false;
-        S.tr_on = step_i >= A.trace_step0 && step_i < A.trace_step1;
-        ++step_i;
-        for (int l = 0; l < L; ++l) {
-            const MegaLayer &ly = M.layer[l];
-            const unsigned mask = active_mask(d, l);
-            // ---- QKV, finished in the epilogue: q rotated, scaled and stored as tensor-core fragments for the
-            // attention phase; k rotated, v as it is, both rounded to bf16 and written straight into their cache
-            // rows (Algorithm 1: "update KV cache at layer l by processing all tokens in P[l] in parallel").
-            // The rows of every q and k head come reordered so that a 16-row tile holds the features
-            // [8 t, 8 t + 8) and [hd/2 + 8 t, hd/2 + 8 t + 8): the two partners (i, i + hd/2) of a rotation
-            // are then rows r and r + 8 of one tile, which one thread holds for its two columns.
-            {
-                Gemm g; g.W = ly.wqkv; g.X = reinterpret_cast<const uint4 *>(A.XA); g.N = c.qkv_rows; g.K = d_model; g.pair = 1; g.half = 0; g.ctas = n_qkv; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(mask);
-                const unsigned vseq = bar_no + 1;
+    int ctl = CTRL_START, e = 0;   // the control point ahead; 1-based layer of its head
+    int step_i = 0, l = 0, ph = PH_QKV;
+#pragma unroll 1
+    for (;;) {
+        if (ROLE == 2 && blockIdx.x == 0) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);   // CTA 0 reads every CTA's head partials
+        const int action = control_point<ROLE>(A, S, ctl, e, pub_no, d, steps_started);
+        book(0);
+        if (action == ACT_NEWSTEP) {
+            l = 0;
+            S.tr_on = step_i >= A.trace_step0 && step_i < A.trace_step1;
+            ++step_i;
+        } else if (action == ACT_CONTINUE) {
+            l = e;   // exit layers are below the last one
+        } else {
+            return;
+        }
+        ph = PH_QKV;
+        // ---- the phases up to the next control point
+#pragma unroll 1
+        for (;;) {
+            const bool final_head = ph == PH_HEAD && l == L;   // heads: l counts the layers that are complete
+            const bool inter = (ph == PH_HEAD || ph == PH_T) && !final_head;
+            const unsigned mask = active_mask(d, final_head ? L - 1 : inter ? l - 1 : l);
+            const unsigned cmask = inter ? (unsigned)d.head_mask & mask : mask;
+            if (ph == PH_ATTN) {
+                // work items that hold no row of this pass are fetched before the QKV phase has ended
+                const bool single = attn_items(A, d, mask) <= A.one_item_max;
+                if (ROLE == 1) {
+                    if (single) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
+                    else attn_produce(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
+                }
                 if (ROLE == 2) {
-                    constexpr int HALF = HD / 2, KSQ = HD / 16;
-                    const int c0 = 2 * (lane & 3), rq = lane >> 2;
-                    const int kvd = c.nkv * HD, group = c.group;
-                    const float qscale = rsqrtf((float)HD);
-                    float r0 = 0.f, r1 = 0.f;
-                    bool have_r = false;
-                    uint32_t *stash = stash_of(sm);
-                    __nv_bfloat16 *pool = reinterpret_cast<__nv_bfloat16 *>(c.kv_pool);
-                    gemm_consume<1>(S, g, blockIdx.x, G, r, [&](int tile) {
-                        // rotary factors and cache pages of this lane's two columns, fetched while the weights stream
-                        const int n0 = tile * 16;
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int cc = c0 + q;
-                            if (!((mask >> cc) & 1u)) continue;
-                            if (n0 < qd + kvd) {
-                                const float *cs = c.rope_cs + ((size_t)cc * HALF + ((n0 & (HD - 1)) >> 1) + rq) * 2;
-                                cp_async4(stash + (2 * q) * 32, cs);
-                                cp_async4(stash + (2 * q + 1) * 32, cs + 1);
-                            }
-                            if (n0 >= qd) cp_async4(stash + (4 + q) * 32, c.page_table + (size_t)(A.seq0 + (A.nseq == 1 ? 0 : cc / c.slots)) * c.max_pages + (d.pos[cc] >> c.page_shift));
-                        }
-                    }, [&](int tile, float (&acc)[1][4]) {
-                        if (!have_r) { vec_wait(S, vseq); r0 = sm->vec[c0]; r1 = sm->vec[c0 + 1]; have_r = true; }
-                        cp_async_wait_all();
-                        const int n0 = tile * 16;
-                        if (n0 >= c.qkv_rows) return;
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int cc = c0 + q;
-                            if (!((mask >> cc) & 1u)) continue;
-                            const float rs = q ? r1 : r0;
-                            const float x0 = acc[0][q] * rs, x1 = acc[0][2 + q] * rs;   // rows rq and rq + 8 of the tile
-                            if (n0 < qd + kvd) {
-                                const float co = __uint_as_float(stash[(2 * q) * 32]), si = __uint_as_float(stash[(2 * q + 1) * 32]);
-                                const int j = ((n0 & (HD - 1)) >> 1) + rq;   // feature j pairs with j + hd/2
-                                float y0 = x0 * co - x1 * si, y1 = x1 * co + x0 * si;
-                                if (n0 < qd) {
-                                    const int h = n0 / HD, kvh = div_group(h, group), qcol = cc * group + (h - kvh * group);
-                                    const int row = qcol & 15, m = qcol >> 4;
-                                    __nv_bfloat16 *f0 = reinterpret_cast<__nv_bfloat16 *>(A.qfrag + (((size_t)kvh * 2 + m) * KSQ) * 256);
-#pragma unroll
-                                    for (int hh = 0; hh < 2; ++hh) {
-                                        const int dim = j + hh * HALF;
-                                        const float y = (hh ? y1 : y0) * qscale;
-                                        const int ks = dim >> 4, kk = dim & 15;
-                                        const int ln = (row & 7) * 4 + ((kk & 7) >> 1), reg = (row >> 3) + 2 * (kk >> 3);
-                                        const __nv_bfloat16 hi = __float2bfloat16_rn(y);
-                                        const __nv_bfloat16 lo = __float2bfloat16_rn(y - __bfloat162float(hi));
-                                        __nv_bfloat16 *f = f0 + ((size_t)ks * 32 + ln) * 16;
-                                        f[reg * 2 + (kk & 1)] = hi;
-                                        f[8 + reg * 2 + (kk & 1)] = lo;
-                                    }
-                                } else {
-                                    const int kvh = (n0 - qd) / HD, pos = d.pos[cc], t = pos & (ATT_PAGE - 1);
-                                    const size_t blk = ((((size_t)stash[(4 + q) * 32] * c.L + l) * 2 + 0) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)t * HD;
-                                    pool[blk + ((((j >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(y0);
-                                    pool[blk + (((((j + HALF) >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(y1);
-                                }
-                            } else {
-                                const int nv = n0 - qd - kvd, kvh = nv / HD, j = (nv & (HD - 1)) + rq, pos = d.pos[cc], t = pos & (ATT_PAGE - 1);
-                                const size_t blk = ((((size_t)stash[(4 + q) * 32] * c.L + l) * 2 + 1) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)t * HD;
-                                pool[blk + ((((j >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(x0);
-                                pool[blk + (((((j + 8) >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(x1);
-                            }
-                        }
-                    });
-                } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_a, ntd, d_model, c.eps, vseq); }, x_ready);
-                else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
-                phase_barrier(2);
-            }
-            // ---- attention (work items that hold no row of this pass are fetched before the QKV phase has ended)
-            if (ROLE == 1) {
-                if (attn_items(A, d, mask) <= A.one_item_max) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
-                else attn_produce(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
+                    consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
+                    if (single) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
+                    else attn_consume<HD>(A, S, d, l, mask, r);
+                }
+            } else {
+                // ---- a product.  QKV is finished in its epilogue: q rotated, scaled and stored as tensor-core fragments for the
+                // attention phase; k rotated, v as it is, both rounded to bf16 and written straight into their cache
+                // rows (Algorithm 1: "update KV cache at layer l by processing all tokens in P[l] in parallel").
+                // The rows of every q and k head come reordered so that a 16-row tile holds the features
+                // [8 t, 8 t + 8) and [hd/2 + 8 t, hd/2 + 8 t + 8): the two partners (i, i + hd/2) of a rotation
+                // are then rows r and r + 8 of one tile, which one thread holds for its two columns.
+                const Plan &pl = sm->plan[ph];
+                const bool with_T = inter && M.has_T[l];
+                const unsigned vseq = bar_no + 1;
+                // the product's result is multiplied by the normalisation factors of its input's rows
+                const bool scaled = ph == PH_QKV || ph == PH_GU || ph == PH_T || (ph == PH_HEAD && !with_T);
+                if (ROLE == 0) {
+                    const CUtensorMap *W = M.maps + (ph == PH_HEAD ? MAPS_PER_LAYER * L : ph == PH_T ? MAPS_PER_LAYER * L + 1 + l
+                                                     : MAPS_PER_LAYER * l + (ph == PH_QKV ? 0 : ph == PH_O ? 1 : ph == PH_GU ? 2 : 4));
+                    gemm_produce_w(S, pl, W, ph == PH_GU && M.gu_two[l] ? W + 1 : nullptr, r, pol);
+                }
+                if (ROLE == 1) {
+                    const __nv_bfloat16 *X = ph == PH_QKV ? A.XA : ph == PH_O ? A.XO : ph == PH_GU ? A.XB : ph == PH_DOWN ? A.XH : ph == PH_HEAD && with_T ? A.XT : A.XF;
+                    gemm_produce_x(S, pl, reinterpret_cast<const uint4 *>(X), Cols(cmask), r, pol,
+                                   [&]() { if (scaled) rstd_produce(sm, ph == PH_GU ? A.ssq_b : A.ssq_a, ntd, d_model, c.eps, vseq); },
+                                   [&]() {   // the input must not be fetched before the phase that wrote it is complete
+                                       grid_wait(S, A.grid_ctr, bar_no * (unsigned)G);
+                                       fence_proxy_async();
+                                       if ((threadIdx.x & 31) == 0) trace(S, EV_PHASE_BEGIN, prof_class(ph));
+                                   });
+                }
+                if (ROLE == 2) {
+                    const Epilogue<HD> epi{A, S, d, ph, l, cmask, vseq, scaled,
+                                           final_head ? (A.sampling ? A.inv_temp : 1.0f) : inter ? M.head_scale[l] * (A.sampling ? A.inv_temp : 1.0f) : 1.0f, inter,
+                                           ph == PH_O || l + 1 < L, ph == PH_DOWN && (l + 1 == L || M.exit_at[l + 1] != 0)};
+                    // (an idle CTA must not report a phase before the one in front of it is complete: the counter would run ahead)
+                    if (Groups(pl).left <= 0) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
+                    if (ph == PH_HEAD) epi.head_begin();
+                    gemm_consume(S, pl, Cols(cmask), A.part, vseq, blockIdx.x, r, [&](int tile) { epi.pre(tile); }, epi);
+                    if (ph == PH_HEAD) epi.head_end();
+                }
             }
             if (ROLE == 2) {
-                if (attn_items(A, d, mask) <= A.one_item_max) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
-                else attn_consume<HD>(A, S, d, l, mask, r);
+                consumers_arrive(S, A.grid_ctr, prof_class(ph));
+                book(prof_class(ph));
             }
-            phase_barrier(4);
-            // ---- O projection + residual; prepares the FFN input
-            {
-                Gemm g; g.W = ly.wo; g.X = reinterpret_cast<const uint4 *>(A.XO); g.N = d_model; g.K = qd; g.pair = 1; g.half = 0; g.ctas = n_d; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(mask);
-                if (ROLE == 2) {
-                    const __nv_bfloat16 *gain = ly.ffn_norm;
-                    uint32_t *stash = stash_of(sm);
-                    gemm_consume<1>(S, g, blockIdx.x, G, r, [&](int tile) {   // residual and gain are fetched while the weights stream
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = 2 * (lane & 3) + (i & 1);
-                            if ((mask >> cc) & 1u) cp_async4(stash + i * 32, c.resid + (size_t)cc * d_model + n);
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) cp_async4(stash + (4 + h) * 32, gain + ((tile * 16 + (lane >> 2) + h * 8) & ~1));
-                    }, [&](int tile, float (&acc)[1][4]) {
-                        const int c0 = 2 * (lane & 3);
-                        float sq[2] = {0.f, 0.f};
-                        cp_async_wait_all();
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-                            if ((mask >> cc) & 1u) {
-                                float *rp = c.resid + (size_t)cc * d_model + n;
-                                const float v = __uint_as_float(stash[i * 32]) + acc[0][i];
-                                *rp = v;
-                                xfrag_store(A.XB, n, cc, v * bf16_of_word(stash[(4 + (i >> 1)) * 32], n));
-                                sq[i & 1] += v * v;
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 4);
-                            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 8);
-                            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 16);
-                            if (lane < 4 && ((mask >> (c0 + q)) & 1u)) A.ssq_b[(size_t)tile * MAX_COLS + c0 + q] = sq[q];
-                        }
-                    });
-                } else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
-                phase_barrier(5);
+            ++bar_no;
+            // ---- what comes next
+            if (ph == PH_HEAD) {
+                ctl = final_head ? CTRL_TOP : CTRL_HEAD;
+                e = l;
+                break;
             }
-            // ---- gate / up + SwiGLU
-            {
-                Gemm g; g.W = ly.wgu; g.W2 = ly.wup; g.X = reinterpret_cast<const uint4 *>(A.XB); g.N = 2 * c.dff; g.K = d_model; g.pair = 2; g.half = c.dff; g.ctas = n_gu;
-                // the one GEMM of the layer where the unit-balanced split pays (measured: it shortens gate-up by 1.4 us,
-                // but lengthens down, QKV and O, whose tile groups are k-split among the warps)
-                g.part = A.part; g.phase_id = bar_no + 1; g.columns(mask);
-                const unsigned vseq = bar_no + 1;
-                if (ROLE == 2) {
-                    const int c0 = 2 * (lane & 3);
-                    float r0 = 0.f, r1 = 0.f;
-                    bool have_r = false;
-                    gemm_consume<2>(S, g, blockIdx.x, G, r, [&](int tile, float (&acc)[2][4]) {
-                        if (!have_r) { vec_wait(S, vseq); r0 = sm->vec[c0]; r1 = sm->vec[c0 + 1]; have_r = true; }
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-                            if ((mask >> cc) & 1u) {
-                                const float rs = (i & 1) ? r1 : r0;
-                                const float gv = acc[0][i] * rs, u = acc[1][i] * rs;
-                                xfrag_store(A.XH, n, cc, gv / (1.0f + expf(-gv)) * u);
-                            }
-                        }
-                    });
-                } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_b, ntd, d_model, c.eps, vseq); }, x_ready);
-                else gemm_phase<ROLE, 2>(S, g, r, pol, x_ready, NoEpi());
-                phase_barrier(6);
+            if (ph == PH_QKV) ph = PH_ATTN;
+            else if (ph == PH_ATTN) ph = PH_O;
+            else if (ph == PH_O) ph = PH_GU;
+            else if (ph == PH_GU) ph = PH_DOWN;
+            else if (ph == PH_T) ph = PH_HEAD;
+            else {   // a layer is complete: an intermediate head (Section 2.1) and the early-prediction rule (Eq. 1), the next layer, or the final head
+                ++l;
+                if (l < L && M.exit_at[l] != 0 && ((unsigned)d.head_mask & mask) != 0) ph = M.has_T[l] ? PH_T : PH_HEAD;   // newest tokens that reached it and may exit early
+                else if (l < L) ph = PH_QKV;
+                else if (d.run_final) ph = PH_HEAD;   // final head for every column, then verification (Eq. 2 at temperature zero) in the control point
+                else { ctl = CTRL_TOP; e = 0; break; }
             }
-            // ---- down projection + residual; prepares the next layer's (and the head's) input
-            {
-                Gemm g; g.W = ly.wdown; g.X = reinterpret_cast<const uint4 *>(A.XH); g.N = d_model; g.K = c.dff; g.pair = 1; g.half = 0; g.ctas = n_d; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(mask);
-                if (ROLE == 2) {
-                    const __nv_bfloat16 *gain_next = l + 1 < L ? M.layer[l + 1].attn_norm : nullptr;
-                    const bool want_f = l + 1 == L || A.exit_at[l + 1] != 0;
-                    const __nv_bfloat16 *gain_f = M.final_norm;
-                    uint32_t *stash = stash_of(sm);
-                    gemm_consume<1>(S, g, blockIdx.x, G, r, [&](int tile) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = 2 * (lane & 3) + (i & 1);
-                            if ((mask >> cc) & 1u) cp_async4(stash + i * 32, c.resid + (size_t)cc * d_model + n);
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int n2 = (tile * 16 + (lane >> 2) + h * 8) & ~1;
-                            if (gain_next) cp_async4(stash + (4 + h) * 32, gain_next + n2);
-                            if (want_f) cp_async4(stash + (6 + h) * 32, gain_f + n2);
-                        }
-                    }, [&](int tile, float (&acc)[1][4]) {
-                        const int c0 = 2 * (lane & 3);
-                        float sq[2] = {0.f, 0.f};
-                        cp_async_wait_all();
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-                            if ((mask >> cc) & 1u) {
-                                float *rp = c.resid + (size_t)cc * d_model + n;
-                                const float v = __uint_as_float(stash[i * 32]) + acc[0][i];
-                                *rp = v;
-                                if (gain_next) xfrag_store(A.XA, n, cc, v * bf16_of_word(stash[(4 + (i >> 1)) * 32], n));
-                                if (want_f) xfrag_store(A.XF, n, cc, v * bf16_of_word(stash[(6 + (i >> 1)) * 32], n));
-                                sq[i & 1] += v * v;
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 4);
-                            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 8);
-                            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 16);
-                            if (lane < 4 && ((mask >> (c0 + q)) & 1u)) A.ssq_a[(size_t)tile * MAX_COLS + c0 + q] = sq[q];
-                        }
-                    });
-                } else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
-                phase_barrier(8);
-            }
-            // ---- intermediate head (Section 2.1) and the early-prediction rule (Eq. 1)
-            const unsigned hcols = (unsigned)d.head_mask & mask;   // newest tokens that reached this layer and may exit early
-            if (l + 1 < L && A.exit_at[l + 1] != 0 && hcols != 0) {
-                const MegaLayer &hl = M.layer[l + 1];
-                if (hl.wT) {
-                    Gemm g; g.W = hl.wT; g.X = reinterpret_cast<const uint4 *>(A.XF); g.N = d_model; g.K = d_model; g.pair = 1; g.half = 0; g.ctas = n_d; g.part = nullptr; g.phase_id = bar_no + 1; g.columns(hcols);
-                    const unsigned vseq = bar_no + 1;
-                    if (ROLE == 2) {
-                        const int c0 = 2 * (lane & 3);
-                        float r0 = 0.f, r1 = 0.f;
-                        bool have_r = false;
-                        gemm_consume<1>(S, g, blockIdx.x, G, r, [&](int tile, float (&acc)[1][4]) {
-                            if (!have_r) { vec_wait(S, vseq); r0 = sm->vec[c0]; r1 = sm->vec[c0 + 1]; have_r = true; }
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-                                xfrag_store(A.XT, n, cc, acc[0][i] * ((i & 1) ? r1 : r0));
-                            }
-                        });
-                    } else if (ROLE == 1) gemm_produce_x(S, g, blockIdx.x, G, r, pol, [&]() { rstd_produce(sm, A.ssq_a, ntd, d_model, c.eps, vseq); }, x_ready);
-                    else gemm_phase<ROLE, 1>(S, g, r, pol, x_ready, NoEpi());
-                    phase_barrier(10);
-                    head_phase(A.XT, nullptr, hl.head_scale, hcols, true);
-                } else {
-                    head_phase(A.XF, A.ssq_a, hl.head_scale, hcols, true);
-                }
-                action = control_point<ROLE>(A, S, CTRL_HEAD, l + 1, pub_no, d, steps_started);
-                book_control();
-                if (action != ACT_CONTINUE) { restart = true; break; }
-            }
-        }
-        if (!restart) {
-            // ---- final head for every column, then verification (Eq. 2 at temperature zero) in the control point
-            if (d.run_final) head_phase(A.XF, A.ssq_a, 1.0f, active_mask(d, L - 1), false);
-            action = control_point<ROLE>(A, S, CTRL_TOP, 0, pub_no, d, steps_started);
-            book_control();
         }
     }
 }
@@ -2223,6 +2203,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_decode_persistent(const __grid_c
     extern __shared__ unsigned char smem_raw[];
     Smem *sm = smem_base(smem_raw);
     smem_init(sm);
+    if (threadIdx.x >= 32 && threadIdx.x < 32 + PH_PRODUCTS) {
+        const int ph = threadIdx.x - 32;
+        sm->plan[ph] = make_plan(phase_gemm(A, ph), blockIdx.x, gridDim.x);
+    }
     __syncthreads();
     Shared S{sm, A.err, A.trace, 0, A.wait_ns};
     const int warp = threadIdx.x >> 5;

@@ -51,17 +51,107 @@ constexpr int ERR_TIMEOUT_MBAR = 1, ERR_TIMEOUT_GRID = 2;
 constexpr unsigned long long WAIT_NS_DEFAULT = 2000000000ull;   // a single wait gives up after two seconds unless told otherwise
 constexpr unsigned long long SHORT_LIMIT_NS = 1000000ull;       // a limit below this is checked at every poll, not every 64th or 128th
 
+// ---------------------------------------------------------------- GEMM shapes and their division
+
+// One GEMM as seen by the whole grid: Y[n][col] = sum_k W[n][k] X[k][col].
+//   pair == 1: N rows, tiles of 16 rows (the last may be ragged).
+//   pair == 2: W holds two stacked matrices of `half` rows each (gate over up), or they are two tensors; a tile is rows
+//              [16 t, 16 t + 16) of both, and the epilogue sees both accumulators.
+// The weights are described by a rank-3 tensor map over the row-major [N][K] matrix, dimensions
+// (64 elements, N rows, K/64 groups) with strides (2 B, 2K B, 128 B) and box (64, 16, 8): one box
+// is a stage.  Rows past N and k groups past K read as zeros.  K must be a multiple of 64.
+struct Gemm {
+    int N, K, pair, half;
+    int split;   // tiles may be cut between two CTAs (needs an exchange area; see Plan)
+    __host__ __device__ __forceinline__ int tiles() const { return pair == 2 ? half / TILE_N : (N + TILE_N - 1) / TILE_N; }
+};
+
+__host__ __device__ __forceinline__ void cta_tile_range(int T, int cta, int G, int &t0, int &t1) {
+    if (cta >= G) { t0 = t1 = 0; return; }
+    t0 = (int)((long long)T * cta / G);
+    t1 = (int)((long long)T * (cta + 1) / G);
+}
+// ---------------------------------------------------------------- unit-balanced split of a GEMM
+// With whole tiles some CTAs stream one tile more than the others (7 against 6 in the 8B gate-up
+// GEMM) and the phase lasts as long as they do.  When g.split is set the work is instead measured in
+// units of (tile, k chunk): CTA c takes the units [U c / C, U (c + 1) / C) of the tile-major order,
+// so every CTA streams the same number of stages (+- one).  A tile cut by a CTA boundary is
+// computed in two parts.  The CTA with its chunks from 0 (the head part, [0, kb)) meets them early
+// in its k loop and publishes its partial sums as soon as they are complete; the CTA with the later
+// chunks (the tail part, [ka, nch)) finishes them at the end of its loop, adds the published part
+// (own + published, the published k-splits in index order: the sum does not depend on timing) and
+// runs the epilogue.  All tiles of a CTA, partial ones included, form one group that shares every
+// activation chunk; when the head part ends before the tail part begins they take turns in slot 0.
+// GEMMs with fewer units per CTA than chunks per tile, or more tiles per CTA than consumer warps,
+// keep whole tiles.  The plan is a function of the GEMM's shape and the grid only.
+struct Plan {
+    int pair, half, nch;   // of the GEMM; nch = k chunks
+    int split;       // 0: whole tiles [t0, t1) in groups of CONS_WARPS
+    int t0, t1;
+    // split: one group of n slots; slot s holds tile ta + s, except that
+    int n, ta, tb;
+    int s0_own_k0;   //   slot 0 multiplies its own tile from chunk s0_own_k0 on (0: a whole tile),
+    int s0_pub_k1;   //   and before that the chunks below s0_pub_k1 of tile tb, to publish (0: none);
+    int sl_k1;       //   the last slot (if not slot 0) multiplies chunks below sl_k1 only, to publish (nch: a whole tile)
+    int ksp;         // split with a tail part: k-splits in which the CTA before publishes its head part
+};
+// the k-splits of a group of ng slots
+__host__ __device__ __forceinline__ int group_ks(int ng) {
+    int TS = 1;
+    while (TS < ng) TS <<= 1;
+    return CONS_WARPS / TS;
+}
+__host__ __device__ inline Plan make_plan(const Gemm &g, int cta, int C, bool with_ksp = true) {
+    Plan p;
+    p.pair = g.pair;
+    p.half = g.half;
+    p.split = 0;
+    p.t0 = p.t1 = p.n = p.ta = p.tb = p.s0_own_k0 = p.s0_pub_k1 = p.ksp = 0;
+    const int T = g.tiles(), nch = (g.K + KC - 1) / KC;
+    p.nch = p.sl_k1 = nch;
+    if (cta < 0 || cta >= C) return p;
+    // 32-bit arithmetic throughout (a 64-bit division costs hundreds of cycles); GEMMs whose unit
+    // count times the CTA count does not fit keep whole tiles
+    const unsigned U = (unsigned)T * (unsigned)nch;
+    const bool fits = (unsigned long long)T * nch * (unsigned)(C + 1) < 0x7fffffffull;
+    const unsigned L = (U + C - 1) / C;      // most units of one CTA; a run of L units touches <= (L + nch - 2) / nch + 1 tiles
+    if (!g.split || !fits || U / C < (unsigned)nch || (L + nch - 2) / nch + 1 > (unsigned)CONS_WARPS) {
+        cta_tile_range(T, cta, C, p.t0, p.t1);
+        return p;
+    }
+    p.split = 1;
+    const unsigned u0 = U * (unsigned)cta / C, u1 = U * (unsigned)(cta + 1) / C;
+    p.ta = (int)(u0 / nch);
+    p.tb = (int)((u1 - 1) / nch);
+    const int ka = (int)(u0 - p.ta * nch), kb = (int)((u1 - 1) - p.tb * nch) + 1;
+    const bool has_tail = ka > 0, has_head = kb < nch;
+    const bool shared = has_tail && has_head && kb <= ka;
+    p.s0_own_k0 = ka;
+    p.n = p.tb - p.ta + 1;
+    if (shared) { p.s0_pub_k1 = kb; p.n -= 1; }
+    else if (has_head) p.sl_k1 = kb;
+    if (ka > 0 && with_ksp) p.ksp = group_ks(make_plan(g, cta - 1, C, false).n);
+    return p;
+}
+// the tile slot s of a split plan multiplies at chunk kc (-1: none)
+__host__ __device__ __forceinline__ int plan_tile(const Plan &p, int s, int kc) {
+    if (s == 0) return kc < p.s0_pub_k1 ? p.tb : (kc >= p.s0_own_k0 ? p.ta : -1);
+    if (s == p.n - 1 && kc >= p.sl_k1) return -1;
+    return p.ta + s;
+}
+
 struct Smem {                                    // must start on a 1024-byte boundary (swizzle pattern)
     alignas(1024) unsigned char w[NW][W_STAGE];
     alignas(128) unsigned char x[NX][X_STAGE];
     alignas(16) unsigned char scratch[SCRATCH_BYTES];
-    alignas(16) float vec[64];                    // per-column scalars (rstd, ...)
+    alignas(16) float vec[MAX_COLS];                   // per-column scalars (rstd, ...)
     alignas(8) unsigned long long w_full[NW], w_empty[NW], x_full[NX], x_empty[NX];
     alignas(16) int desc[3][32];                  // per-role copy of the step descriptor (persistent decode kernel)
     int abort;
     int bcast[8];
     unsigned trace_n;
     unsigned vec_seq;                             // phase for which vec[] holds the normalisation factors (see vec_wait)
+    Plan plan[6];                                 // this CTA's share of every product of the program
 };
 
 // ---------------------------------------------------------------- PTX wrappers
@@ -297,110 +387,34 @@ __host__ __device__ inline size_t xfrag_bytes(int K) { return (size_t)((K + KC -
 
 // ---------------------------------------------------------------- GEMM phase
 
-// One GEMM as seen by the whole grid: Y[n][col] = sum_k W[n][k] X[k][col].
-//   pair == 1: N rows, tiles of 16 rows (the last may be ragged).
-//   pair == 2: W holds two stacked matrices of `half` rows each (gate over up); a tile is rows
-//              [16 t, 16 t + 16) of both, and the epilogue sees both accumulators.
-// The weights are described by a rank-3 tensor map over the row-major [N][K] matrix, dimensions
-// (64 elements, N rows, K/64 groups) with strides (2 B, 2K B, 128 B) and box (64, 16, 8): one box
-// is a stage.  Rows past N and k groups past K read as zeros.  K must be a multiple of 64.
-struct Gemm {
-    const CUtensorMap *W;
-    const CUtensorMap *W2 = nullptr;   // pair == 2 only: map of the second matrix when the two are separate tensors (null: stacked in W)
-    const uint4 *X;
-    int N, K, pair, half;
-    int ctas;   // CTAs 0 .. ctas-1 share the tiles (see balanced_ctas); 0 = the whole grid
-    // Exchange area for tiles split between two CTAs (null: whole tiles only): [grid][CONS_WARPS][8][32]
-    // words of 8 bytes, each a partial sum (low half) tagged with the phase that wrote it (high half).
-    // A word is written and read by one 8-byte access, so a reader that sees the tag sees the sum:
-    // no fence is needed on either side (a fence in the middle of the stream stalls the publishing
-    // warp, and with it the whole ring, for microseconds).  phase_id is unique per GEMM of a launch
-    // and never 0; the area is zeroed before each launch.
-    unsigned long long *part;
-    unsigned phase_id;
-    int cp0, ncp;   // column pairs cp0 .. cp0+ncp-1 of the activations are fetched
-    __device__ __forceinline__ void columns(unsigned mask) {   // the pairs spanning the columns set in `mask`
-        if (mask == 0) { cp0 = 0; ncp = 1; return; }
-        cp0 = (__ffs(mask) - 1) >> 1;
-        ncp = ((31 - __clz(mask)) >> 1) - cp0 + 1;
+// The activation columns a pass fetches: column pairs cp0 .. cp0 + ncp - 1.
+struct Cols {
+    int cp0, ncp;
+    __device__ __forceinline__ explicit Cols(unsigned mask) {   // the pairs spanning the columns set in `mask`
+        cp0 = mask ? (__ffs(mask) - 1) >> 1 : 0;
+        ncp = mask ? ((31 - __clz(mask)) >> 1) - cp0 + 1 : 1;
     }
     // k chunks whose activations share one 16 KB stage: 4 for one column pair, 2 for two, else 1.  (The
     // ring holds three stages; with one chunk per stage a CTA that owns two weight tiles would wait
     // for an activation copy every 96 KB of weights.)
-    __device__ __forceinline__ int xchunks() const { return ncp == 1 ? 4 : ncp == 2 ? 2 : 1; }
-    __host__ __device__ __forceinline__ int tiles() const { return pair == 2 ? half / TILE_N : (N + TILE_N - 1) / TILE_N; }
+    __device__ __forceinline__ int chunks() const { return ncp == 1 ? 4 : ncp == 2 ? 2 : 1; }
+    // Up to four columns: one multiply-add takes their high parts as token columns 0..3 and their low parts as 4..7.
+    __device__ __forceinline__ bool packed() const { return ncp <= 2; }
 };
 
-struct Rings { uint32_t wi, xi; };   // stage counters of one role (slot = i % N, parity = (i / N) & 1)
-
-__host__ __device__ __forceinline__ void cta_tile_range(int T, int cta, int G, int &t0, int &t1) {
-    if (cta >= G) { t0 = t1 = 0; return; }
-    t0 = (int)((long long)T * cta / G);
-    t1 = (int)((long long)T * (cta + 1) / G);
-}
-// ---------------------------------------------------------------- unit-balanced split of a GEMM
-// With whole tiles some CTAs stream one tile more than the others (7 against 6 in the 8B gate-up
-// GEMM) and the phase lasts as long as they do.  When g.part is set the work is instead measured in
-// units of (tile, k chunk): CTA c takes the units [U c / C, U (c + 1) / C) of the tile-major order,
-// so every CTA streams the same number of stages (+- one).  A tile cut by a CTA boundary is
-// computed in two parts.  The CTA with its chunks from 0 (the head part, [0, kb)) meets them early
-// in its k loop and publishes its partial sums as soon as they are complete; the CTA with the later
-// chunks (the tail part, [ka, nch)) finishes them at the end of its loop, adds the published part
-// (own + published, the published k-splits in index order: the sum does not depend on timing) and
-// runs the epilogue.  All tiles of a CTA, partial ones included, form one group that shares every
-// activation chunk; when the head part ends before the tail part begins they take turns in slot 0.
-// GEMMs with fewer units per CTA than chunks per tile, or more tiles per CTA than consumer warps,
-// keep whole tiles.  The plan is a function of the GEMM's shape and the grid only.
-struct Plan {
-    int split;       // 0: whole tiles [t0, t1) in groups of CONS_WARPS
-    int t0, t1;
-    // split: one group of n slots; slot s holds tile ta + s, except that
-    int n, ta, tb;
-    int s0_own_k0;   //   slot 0 multiplies its own tile from chunk s0_own_k0 on (0: a whole tile),
-    int s0_pub_k1;   //   and before that the chunks below s0_pub_k1 of tile tb, to publish (0: none);
-    int sl_k1;       //   the last slot (if not slot 0) multiplies chunks below sl_k1 only, to publish (nch: a whole tile)
+struct Rings {   // position of one role in the two rings: slot and parity of the next stage
+    uint32_t ws = 0, wp = 0, xs = 0, xp = 0;
+    __device__ __forceinline__ void next_w() { if (++ws == NW) { ws = 0; wp ^= 1; } }
+    __device__ __forceinline__ void next_x() { if (++xs == NX) { xs = 0; xp ^= 1; } }
 };
-__host__ __device__ __forceinline__ Plan make_plan(const Gemm &g, int cta, int G) {
-    Plan p;
-    p.split = 0;
-    p.t0 = p.t1 = p.n = p.ta = p.tb = p.s0_own_k0 = p.s0_pub_k1 = 0;
-    const int C = g.ctas > 0 ? g.ctas : G, T = g.tiles(), nch = (g.K + KC - 1) / KC;
-    p.sl_k1 = nch;
-    if (cta < 0 || cta >= C) return p;
-    // 32-bit arithmetic throughout (a 64-bit division costs hundreds of cycles); GEMMs whose unit
-    // count times the CTA count does not fit keep whole tiles
-    const unsigned U = (unsigned)T * (unsigned)nch;
-    const bool fits = (unsigned long long)T * nch * (unsigned)(C + 1) < 0x7fffffffull;
-    const unsigned L = (U + C - 1) / C;      // most units of one CTA; a run of L units touches <= (L + nch - 2) / nch + 1 tiles
-    if (!g.part || !fits || U / C < (unsigned)nch || (L + nch - 2) / nch + 1 > (unsigned)CONS_WARPS) {
-        cta_tile_range(T, cta, C, p.t0, p.t1);
-        return p;
-    }
-    p.split = 1;
-    const unsigned u0 = U * (unsigned)cta / C, u1 = U * (unsigned)(cta + 1) / C;
-    p.ta = (int)(u0 / nch);
-    p.tb = (int)((u1 - 1) / nch);
-    const int ka = (int)(u0 - p.ta * nch), kb = (int)((u1 - 1) - p.tb * nch) + 1;
-    const bool has_tail = ka > 0, has_head = kb < nch;
-    const bool shared = has_tail && has_head && kb <= ka;
-    p.s0_own_k0 = ka;
-    p.n = p.tb - p.ta + 1;
-    if (shared) { p.s0_pub_k1 = kb; p.n -= 1; }
-    else if (has_head) p.sl_k1 = kb;
-    return p;
-}
-// the tile slot s of a split plan multiplies at chunk kc (-1: none)
-__host__ __device__ __forceinline__ int plan_tile(const Plan &p, int s, int kc) {
-    if (s == 0) return kc < p.s0_pub_k1 ? p.tb : (kc >= p.s0_own_k0 ? p.ta : -1);
-    if (s == p.n - 1 && kc >= p.sl_k1) return -1;
-    return p.ta + s;
-}
-// the k-splits of a group of ng slots
-__host__ __device__ __forceinline__ int group_ks(int ng) {
-    int TS = 1;
-    while (TS < ng) TS <<= 1;
-    return CONS_WARPS / TS;
-}
+
+// A plan as a sequence of groups of at most CONS_WARPS slots: a split plan is one group.
+struct Groups {
+    int g0, left;
+    __device__ __forceinline__ explicit Groups(const Plan &p) : g0(p.split ? p.ta : p.t0), left(p.split ? p.n : p.t1 - p.t0) {}
+    __device__ __forceinline__ int slots() const { return min(left, CONS_WARPS); }
+    __device__ __forceinline__ void next() { g0 += CONS_WARPS; left -= CONS_WARPS; }
+};
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -410,110 +424,120 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
     return v;
 }
 
-// How many CTAs share the tiles of a GEMM: all of them.  (With its consumers attached one SM
-// sustains about 45 GB/s through the ring, roughly its fair share of HBM with all 148 SMs
-// streaming; giving equal tile counts to fewer CTAs was measured and lost more than the uneven
-// split costs.)
-__host__ __device__ inline int balanced_ctas(int T, int G) { (void)T; return G; }
-
-// Weight producer warp: streams this CTA's tiles of the GEMM through the weight ring.
-__device__ __forceinline__ void gemm_produce_w(const Shared &S, const Gemm &g, int cta, int G, Rings &r, uint64_t pol) {
+// Weight producer warp: streams this CTA's tiles of the GEMM through the weight ring.  W2: map of the second matrix of a
+// pair where the two are separate tensors (null: stacked in W).
+__device__ __forceinline__ void gemm_produce_w(const Shared &S, const Plan &pl, const CUtensorMap *W, const CUtensorMap *W2, Rings &r, uint64_t pol) {
     Smem *sm = S.sm;
     const int lane = threadIdx.x & 31;
-    const Plan pl = make_plan(g, cta, G);
-    const int nch = (g.K + KC - 1) / KC;
+    const int nch = pl.nch, pair = pl.pair;
     if (lane == 0) trace(S, EV_WP_BEGIN, 0);
-    auto stage = [&](int tile, int p, int kc) {
-        const int slot = r.wi % NW;
-        mbar_wait(S, &sm->w_empty[slot], ((r.wi / NW) & 1) ^ 1);
-        if (lane == 0 && !aborted(S)) {
-            mbar_expect_tx(&sm->w_full[slot], (uint32_t)W_STAGE);
-            tma_load_3d(sm->w[slot], (p && g.W2) ? g.W2 : g.W, 0, tile * TILE_N + ((p && !g.W2) ? g.half : 0), kc * KG, &sm->w_full[slot], pol);
-        }
-        ++r.wi;
-    };
-    if (pl.split) {
+#pragma unroll 1
+    for (Groups g(pl); g.left > 0; g.next()) {
+        const int ng = g.slots();
+#pragma unroll 1
         for (int kc = 0; kc < nch; ++kc)
-            for (int s = 0; s < pl.n; ++s) {
-                const int tile = plan_tile(pl, s, kc);
+#pragma unroll 1
+            for (int s = 0; s < ng; ++s) {
+                const int tile = pl.split ? plan_tile(pl, s, kc) : g.g0 + s;
                 if (tile < 0) continue;
-                for (int p = 0; p < g.pair; ++p) stage(tile, p, kc);
+#pragma unroll 1
+                for (int p = 0; p < pair; ++p) {
+                    mbar_wait(S, &sm->w_empty[r.ws], r.wp ^ 1);
+                    if (lane == 0 && !aborted(S)) {
+                        mbar_expect_tx(&sm->w_full[r.ws], (uint32_t)W_STAGE);
+                        tma_load_3d(sm->w[r.ws], (p && W2) ? W2 : W, 0, tile * TILE_N + ((p && !W2) ? pl.half : 0), kc * KG, &sm->w_full[r.ws], pol);
+                    }
+                    r.next_w();
+                }
             }
-    } else {
-        for (int g0 = pl.t0; g0 < pl.t1; g0 += CONS_WARPS) {
-            const int ng = min(CONS_WARPS, pl.t1 - g0);
-            for (int kc = 0; kc < nch; ++kc)
-                for (int s = 0; s < ng; ++s)
-                    for (int p = 0; p < g.pair; ++p) stage(g0 + s, p, kc);
-        }
     }
     if (lane == 0) trace(S, EV_WP_END, 0);
 }
 
-// Activation producer warp: one stage per (tile group, k chunk).
+// Activation producer warp: one stage per (tile group, k chunks).
 // `after_first` runs once, after the first stage has been issued: work of the phase that is not
 // needed before the epilogues (the normalisation factors) and must not delay the first copy.
-// `ready` runs once, immediately before the first copy: it waits until the input is complete (the division of the work is
-// worked out before that wait, not after it).
+// `ready` runs once, immediately before the first copy: it waits until the input is complete.
 template <class Hook, class Ready>
-__device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, int cta, int G, Rings &r, uint64_t pol, Hook &&after_first, Ready &&ready) {
+__device__ __forceinline__ void gemm_produce_x(const Shared &S, const Plan &pl, const uint4 *X, const Cols &cols, Rings &r, uint64_t pol, Hook &&after_first,
+                                               Ready &&ready) {
     Smem *sm = S.sm;
     const int lane = threadIdx.x & 31;
-    const Plan pl = make_plan(g, cta, G);
-    const int nch = (g.K + KC - 1) / KC;
-    const int XC = g.xchunks();
-    const int ngroups = pl.split ? (pl.n > 0 ? 1 : 0) : (pl.t1 - pl.t0 + CONS_WARPS - 1) / CONS_WARPS;
-    bool hooked = false;
-    for (int gi = 0; gi < ngroups; ++gi) {
+    const int nch = pl.nch, XC = cols.chunks();
+    const uint32_t bytes = (uint32_t)cols.ncp * 4096u;
+    const unsigned char *src = reinterpret_cast<const unsigned char *>(X) + cols.cp0 * 4096;
+    // as many rounds as the plan has groups; a CTA without any still passes `ready` and the hook
+    Groups g(pl);
+    bool first = true;
+#pragma unroll 1
+    do {
+#pragma unroll 1
         for (int kc = 0; kc < nch; kc += XC) {
-            const int nc = min(XC, nch - kc);
-            const int slot = r.xi % NX;
-            mbar_wait(S, &sm->x_empty[slot], ((r.xi / NX) & 1) ^ 1);
-            if (!hooked) ready();
-            if (lane == 0 && !aborted(S)) {
-                const uint32_t bytes = (uint32_t)g.ncp * 4096u;
-                mbar_expect_tx(&sm->x_full[slot], bytes * nc);
-                for (int q = 0; q < nc; ++q)   // chunk kc+q: column pairs cp0.. at [q][pair - cp0] of the stage
-                    bulk_g2s(sm->x[slot] + q * bytes, reinterpret_cast<const unsigned char *>(g.X) + (size_t)(kc + q) * X_STAGE + g.cp0 * 4096,
-                             bytes, &sm->x_full[slot], pol);
+            const bool some = g.left > 0;
+            if (some) mbar_wait(S, &sm->x_empty[r.xs], r.xp ^ 1);
+            if (first) ready();
+            if (some) {
+                const int nc = min(XC, nch - kc);
+                if (lane == 0 && !aborted(S)) {
+                    mbar_expect_tx(&sm->x_full[r.xs], bytes * nc);
+                    for (int q = 0; q < nc; ++q)   // chunk kc+q: column pairs cp0.. at [q][pair - cp0] of the stage
+                        bulk_g2s(sm->x[r.xs] + q * bytes, src + (size_t)(kc + q) * X_STAGE, bytes, &sm->x_full[r.xs], pol);
+                }
+                r.next_x();
             }
-            ++r.xi;
-            if (!hooked) { after_first(); hooked = true; }
+            if (first) { after_first(); first = false; }
+            if (!some) break;
         }
-    }
-    if (!hooked) { ready(); after_first(); }
+        g.next();
+    } while (g.left > 0);
 }
 struct NoHook {
     __device__ __forceinline__ void operator()() const {}
 };
-__device__ __forceinline__ void gemm_produce_x(const Shared &S, const Gemm &g, int cta, int G, Rings &r, uint64_t pol) {
-    gemm_produce_x(S, g, cta, G, r, pol, NoHook(), NoHook());
-}
 
-// The k-steps ks_id + KS_ j (j < 32 / KS_) of one full weight stage: fragment loads run PF steps
-// ahead of the multiply-adds that use them.  Even j accumulate into acc[0] (high parts) and acc[2]
-// (low parts), odd j into acc[1] and acc[3]: four independent accumulation chains.
-template <int KS_>
-__device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned char *ws, const uint4 *xs, int ks_id, int a_hi, int a_sw) {
-    constexpr int NJ = KSTEPS / KS_;
-    constexpr int PF = NJ < 4 ? NJ : 4;
+// The 32 k-steps of one weight stage: fragment loads run four steps ahead of the multiply-adds that use them.
+// Even k-steps accumulate into acc[0] (high parts) and acc[2] (low parts), odd ones into acc[1] and acc[3]: four independent
+// accumulation chains.
+__device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+    constexpr int PF = 4;
     uint32_t a[PF][4];
     uint4 b[PF];
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
-        const int ks = ks_id + KS_ * j;
-        ldmatrix_x4(a[j], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
-        b[j] = xs[ks * 8];
+        ldmatrix_x4(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
+        b[j] = *reinterpret_cast<const uint4 *>(xs + j * 128);
     }
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
+    for (int j = 0; j < KSTEPS; ++j) {
         const int cur = j % PF;
         mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
         mma16816(acc[(j & 1) + 2], a[cur], b[cur].z, b[cur].w);
-        if (j + PF < NJ) {
-            const int ks = ks_id + KS_ * (j + PF);
+        if (j + PF < KSTEPS) {
+            const int ks = j + PF;
             ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
-            b[cur] = xs[ks * 8];
+            b[cur] = *reinterpret_cast<const uint4 *>(xs + ks * 128);
+        }
+    }
+}
+// The same for up to four columns: their high parts are token columns 0..3 of one multiply-add, their low parts 4..7.
+// Half the multiply-adds and half the shared-memory reads; every sum has the order it has above.
+__device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+    constexpr int PF = 4;
+    uint32_t a[PF][4];
+    uint2 b[PF];
+#pragma unroll
+    for (int j = 0; j < PF; ++j) {
+        ldmatrix_x4(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
+        b[j] = *reinterpret_cast<const uint2 *>(xs + j * 128);
+    }
+#pragma unroll
+    for (int j = 0; j < KSTEPS; ++j) {
+        const int cur = j % PF;
+        mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
+        if (j + PF < KSTEPS) {
+            const int ks = j + PF;
+            ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
+            b[cur] = *reinterpret_cast<const uint2 *>(xs + ks * 128);
         }
     }
 }
@@ -521,118 +545,127 @@ __device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned ch
 // Consumer warps.  Within a group of up to eight tiles the warps are arranged as TS tile slots x
 // KS k-splits (TS * KS = 8, TS the smallest power of two holding the group); a warp multiplies
 // the stages of its slot whose k chunk is ks_id (mod KS).  The k-splits of a tile are summed in a
-// fixed order through shared memory, then `epi(tile, acc)` runs in the slot's first warp with
-//   acc[p][i]: fragment element i of matrix p: rows lane/4 (i<2) or lane/4+8, columns 2(lane%4)+(i&1).
+// fixed order through shared memory, then `epi(tile, d0, d1)` runs in the slot's first warp with
+//   dp[i]: fragment element i of matrix p: rows lane/4 (i<2) or lane/4+8, columns 2(lane%4)+(i&1).
 // The arrangement depends only on the tile partition, never on which token columns are in use.
 // `pre(tile)` runs in the same warp before the group's first stage (a place to start loads the epilogue will need).
-template <int PAIR, class Pre, class Epi>
-__device__ __forceinline__ void gemm_consume(const Shared &S, const Gemm &g, int cta, int G, Rings &r, Pre &&pre, Epi &&epi) {
+//
+// One body for every product of a program (the caller loops over its phases and branches on the phase in `pre` and `epi`): with
+// a copy of it per product and role the persistent kernel was 790 KB of code, more than the instruction caches hold, and every
+// phase began and ended with instruction fetches from L2 on its critical path.
+// k steps past K multiply zeros (the tensor map fills weights with them, the activation blocks are padded with them).
+template <class Pre, class Epi>
+__device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, const Cols &cols, unsigned long long *part, unsigned phase_id, int cta, Rings &r,
+                                             Pre &&pre, Epi &&epi) {
     Smem *sm = S.sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nch = (g.K + KC - 1) / KC, XC = g.xchunks();
-    bool first_group = true;
+    const int nch = pl.nch, pair = pl.pair, XC = cols.chunks();
+    const bool packed = cols.packed();
+    const int s0_own_k0 = pl.s0_own_k0, s0_pub_k1 = pl.s0_pub_k1, sl_k1 = pl.sl_k1;
     // ldmatrix source of this lane inside a stage: row (lane%8) + 8 ((lane/8)%2), 16-byte chunk lane/16 of the k-step
     const int a_row = (lane & 7) + ((lane >> 3) & 1) * 8;
     const int a_off = a_row * 128, a_hi = lane >> 4, a_sw = a_row & 7;
-    // One group of ng tile slots; slot s holds tile g0 + s.  Whole tiles: s0_own_k0 = s0_pub_k1 = 0,
-    // sl_k1 = nch.  The group of a split plan: see Plan; ksp = k-splits of the CTA before (0: no tail part).
-    auto group = [&](int g0, int ng, int s0_own_k0, int s0_pub_k1, int sl_k1, int ksp, bool last_group) {
+    // this lane's column pair, if it was fetched (else any fetched pair: its column is not in use), and its 16 (8) bytes
+    const int xpair = packed ? min((lane >> 3) & 1, cols.ncp - 1) : min(max((lane >> 3) - cols.cp0, 0), cols.ncp - 1);
+    const int x_off = xpair * 4096 + (lane & 7) * 16 + (packed ? (lane >> 4) * 8 : 0);
+    bool first = true;
+#pragma unroll 1
+    for (Groups g(pl); g.left > 0; g.next()) {
+        const int ng = g.slots();
         int TS = 1;
         while (TS < ng) TS <<= 1;
         const int KS = CONS_WARPS / TS;
-        const int slot_id = warp % TS, ks_id = warp / TS;
+        const int slot_id = warp & (TS - 1), ks_id = warp / TS;
         const bool mine = slot_id < ng;
         const bool pub_only = slot_id > 0 && slot_id == ng - 1 && sl_k1 < nch;
         // this warp's slot: chunks below my_pub_k1 go to the published part, chunks from my_own_k0 to its own tile
         const int my_pub_k1 = !mine ? 0 : slot_id == 0 ? s0_pub_k1 : pub_only ? sl_k1 : 0;
         const int my_own_k0 = (!mine || pub_only) ? nch : slot_id == 0 ? s0_own_k0 : 0;
-        const int own_tile = (mine && !pub_only) ? g0 + slot_id : -1;
+        const int own_tile = (mine && !pub_only) ? g.g0 + slot_id : -1;
         const bool tail = own_tile >= 0 && my_own_k0 > 0;   // the head part of this tile comes from CTA cta - 1
         if (ks_id == 0 && own_tile >= 0) pre(own_tile);
-        float acc[PAIR][4][4];   // [matrix][even/odd step x hi/lo][fragment]
+        float acc0[4][4], acc1[4][4];   // [even/odd step x hi/lo][fragment] of the one or two matrices
 #pragma unroll
-        for (int p = 0; p < PAIR; ++p)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+            for (int i = 0; i < 4; ++i) acc0[q][i] = acc1[q][i] = 0.f;
+        // fold the partial accumulators in a fixed order: (even.hi + odd.hi) + (even.lo + odd.lo)
+        float d0[4], d1[4];
+        auto fold = [&](float (&d)[4], float (&acc)[4][4]) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[p][q][i] = 0.f;
+            for (int i = 0; i < 4; ++i) {
+                float hi = acc[0][i] + acc[1][i];
+                if (packed) {   // the low parts' sums are two lanes on; then to the lanes the columns belong to
+                    hi += __shfl_xor_sync(0xffffffffu, hi, 2);
+                    d[i] = __shfl_sync(0xffffffffu, hi, (lane & ~3) | ((lane - cols.cp0) & 1));
+                } else {
+                    d[i] = hi + (acc[2][i] + acc[3][i]);
+                }
+            }
+        };
+#pragma unroll 1
         for (int kc = 0; kc < nch; ++kc) {
-            const int ksteps = min(KC, g.K - kc * KC) >> 4;
-            const int xslot = r.xi % NX;
-            if (kc % XC == 0) mbar_wait(S, &sm->x_full[xslot], (r.xi / NX) & 1);
-            if (threadIdx.x == 0 && kc == 0 && first_group) trace(S, EV_X0, 0);
-            // this lane's column pair, if it was fetched (else any fetched pair: its column is not in use)
-            const int xp = min(max((lane >> 3) - g.cp0, 0), g.ncp - 1);
-            const uint4 *xs = reinterpret_cast<const uint4 *>(sm->x[xslot]) + ((kc % XC) * g.ncp + xp) * 256 + (lane & 7);
+            if (kc % XC == 0) mbar_wait(S, &sm->x_full[r.xs], r.xp);
+            if (threadIdx.x == 0 && first) trace(S, EV_X0, 0);
+            first = false;
+            const unsigned char *xs = sm->x[r.xs] + (kc % XC) * cols.ncp * 4096 + x_off;
             // the k-splits of a slot take whole stages in turn, counted from the first chunk of the part
             // (chunk kc belongs to split (kc - first) mod KS): a warp then multiplies all 32 k-steps of
             // a stage, which amortises the per-stage waiting and set-up (splitting every stage among
             // the warps streamed 20-30 % slower)
             const int kbase = kc < my_pub_k1 ? 0 : my_own_k0;
             const bool my_turn = mine && ((kc - kbase) & (KS - 1)) == ks_id;
+#pragma unroll 1
             for (int s = 0; s < ng; ++s) {
                 if (s == 0 ? (kc >= s0_pub_k1 && kc < s0_own_k0) : (s == ng - 1 && kc >= sl_k1)) continue;   // no stage: outside the parts
-#pragma unroll
-                for (int p = 0; p < PAIR; ++p) {
-                    const int wslot = r.wi % NW;
+#pragma unroll 1
+                for (int p = 0; p < pair; ++p) {
                     // Every warp waits for and releases every stage in order, although only its owner
                     // uses it.  An mbarrier tells phases apart by one parity bit: a warp that ran ahead
                     // of, or fell behind, the others by a ring would mistake one phase of a slot for
                     // another (releasing stages by their owners alone was tried: a lagging warp then
                     // waits for a refill that needs its own release).  With all eight arrivals per
                     // stage no warp is ever more than one ring away from any other.
-                    mbar_wait(S, &sm->w_full[wslot], (r.wi / NW) & 1);
+                    mbar_wait(S, &sm->w_full[r.ws], r.wp);
                     if (s == slot_id && my_turn) {
-                        if (threadIdx.x == 0 && kc == 0 && first_group && p == 0) trace(S, EV_W0, 0);
-                        const unsigned char *ws = sm->w[wslot] + a_off;
-                        if (ksteps == KSTEPS) {   // full chunk: software-pipelined, fully unrolled
-                            stage_full<1>(acc[p], ws, xs, 0, a_hi, a_sw);
-                        } else {                  // short last chunk of K
-                            int par = 0;
-                            for (int ks = 0; ks < ksteps; ++ks) {
-                                uint32_t a[4];
-                                ldmatrix_x4(a, ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
-                                const uint4 b = xs[ks * 8];
-                                if (par == 0) { mma16816(acc[p][0], a, b.x, b.y); mma16816(acc[p][2], a, b.z, b.w); }
-                                else { mma16816(acc[p][1], a, b.x, b.y); mma16816(acc[p][3], a, b.z, b.w); }
-                                par ^= 1;
-                            }
+                        const unsigned char *ws = sm->w[r.ws] + a_off;
+                        if (packed) {
+                            if (p == 0) stage_packed(acc0, ws, xs, a_hi, a_sw);
+                            else stage_packed(acc1, ws, xs, a_hi, a_sw);
+                        } else {
+                            if (p == 0) stage_full(acc0, ws, xs, a_hi, a_sw);
+                            else stage_full(acc1, ws, xs, a_hi, a_sw);
                         }
                     }
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
-                    ++r.wi;
+                    if (lane == 0) mbar_arrive(&sm->w_empty[r.ws]);
+                    r.next_w();
                 }
             }
             if (kc % XC == XC - 1 || kc == nch - 1) {
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&sm->x_empty[xslot]);
-                ++r.xi;
+                if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
+                r.next_x();
             }
             if (kc + 1 == my_pub_k1) {
                 // The head part of a split tile is complete: every k-split warp publishes its own sums
                 // (no meeting inside the CTA in the middle of the stream) and starts over for the tail
                 // part that may follow in this slot.
-                unsigned long long *pb = g.part + (size_t)(cta * CONS_WARPS + ks_id) * 256;
+                unsigned long long *pb = part + (size_t)(cta * CONS_WARPS + ks_id) * 256;
+                fold(d0, acc0);
+                fold(d1, acc1);
 #pragma unroll
-                for (int p = 0; p < PAIR; ++p)
+                for (int i = 0; i < 4; ++i) {
+                    st_relaxed_u64(pb + i * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d0[i]));
+                    if (pair == 2) st_relaxed_u64(pb + (4 + i) * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d1[i]));
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float v = (acc[p][0][i] + acc[p][1][i]) + (acc[p][2][i] + acc[p][3][i]);
-                        st_relaxed_u64(pb + (p * 4 + i) * 32 + lane, ((unsigned long long)g.phase_id << 32) | __float_as_uint(v));
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) acc[p][q][i] = 0.f;
-                    }
+                    for (int q = 0; q < 4; ++q) acc0[q][i] = acc1[q][i] = 0.f;
+                }
             }
         }
-        if (threadIdx.x == 0 && last_group) trace(S, EV_MAIN_END, 0);
-        first_group = false;
-        // fold the four partial accumulators in a fixed order: (even.hi + odd.hi) + (even.lo + odd.lo)
-        float d[PAIR][4];
-#pragma unroll
-        for (int p = 0; p < PAIR; ++p)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) d[p][i] = (acc[p][0][i] + acc[p][1][i]) + (acc[p][2][i] + acc[p][3][i]);
+        if (threadIdx.x == 0 && g.left <= CONS_WARPS) trace(S, EV_MAIN_END, 0);
+        fold(d0, acc0);
+        fold(d1, acc1);
         // The head part published by CTA cta - 1, in ksp k-splits: this slot's k-split warp j fetches
         // the published splits j, j + KS, ... (all at once: one round trip) and adds them to its own
         // sums in index order; the fixed-order reduction below then covers both parts.
@@ -640,27 +673,27 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Gemm &g, int
             unsigned long long t0 = 0;
             for (uint32_t it = 0;; ++it) {
                 bool ok = true;
-                float add[PAIR][4];
+                float add[2][4];
 #pragma unroll
-                for (int p = 0; p < PAIR; ++p)
+                for (int p = 0; p < 2; ++p)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) add[p][i] = 0.f;
-                for (int q = ks_id; q < ksp; q += KS) {
-                    const unsigned long long *pb = g.part + (size_t)((cta - 1) * CONS_WARPS + q) * 256;
+                for (int q = ks_id; q < pl.ksp; q += KS) {
+                    const unsigned long long *pb = part + (size_t)((cta - 1) * CONS_WARPS + q) * 256;
 #pragma unroll
-                    for (int p = 0; p < PAIR; ++p)
+                    for (int p = 0; p < 2; ++p) {
+                        if (p >= pair) break;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
                             const unsigned long long v = ld_relaxed_u64(pb + (p * 4 + i) * 32 + lane);
-                            ok = ok && (unsigned)(v >> 32) == g.phase_id;
+                            ok = ok && (unsigned)(v >> 32) == phase_id;
                             add[p][i] += __uint_as_float((unsigned)v);
                         }
+                    }
                 }
                 if (__all_sync(0xffffffffu, ok)) {
 #pragma unroll
-                    for (int p = 0; p < PAIR; ++p)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) d[p][i] += add[p][i];
+                    for (int i = 0; i < 4; ++i) { d0[i] += add[0][i]; d1[i] += add[1][i]; }
                     break;
                 }
                 if ((it & 15u) == 15u || S.wait_ns < SHORT_LIMIT_NS) {   // bounded like every other wait on another CTA
@@ -674,34 +707,26 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Gemm &g, int
             }
         }
         if (KS > 1) {
-            float *red = reinterpret_cast<float *>(sm->scratch) + (size_t)warp * (PAIR * 128);
+            float *red = reinterpret_cast<float *>(sm->scratch) + (size_t)warp * (pair * 128);
 #pragma unroll
-            for (int p = 0; p < PAIR; ++p)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) red[(p * 4 + i) * 32 + lane] = d[p][i];
+            for (int i = 0; i < 4; ++i) {
+                red[i * 32 + lane] = d0[i];
+                if (pair == 2) red[(4 + i) * 32 + lane] = d1[i];
+            }
             bar_consumers();
             if (ks_id == 0) {
                 for (int q = 1; q < KS; ++q) {
-                    const float *o = reinterpret_cast<const float *>(sm->scratch) + (size_t)(q * TS + slot_id) * (PAIR * 128);
+                    const float *o = reinterpret_cast<const float *>(sm->scratch) + (size_t)(q * TS + slot_id) * (pair * 128);
 #pragma unroll
-                    for (int p = 0; p < PAIR; ++p)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) d[p][i] += o[(p * 4 + i) * 32 + lane];
+                    for (int i = 0; i < 4; ++i) {
+                        d0[i] += o[i * 32 + lane];
+                        if (pair == 2) d1[i] += o[(4 + i) * 32 + lane];
+                    }
                 }
             }
         }
-        if (ks_id == 0 && own_tile >= 0) epi(own_tile, d);
+        if (ks_id == 0 && own_tile >= 0) epi(own_tile, d0, d1);
         if (KS > 1) bar_consumers();
-    };
-    {
-        const Plan pl = make_plan(g, cta, G);
-        if (pl.split) {
-            const int ksp = pl.s0_own_k0 > 0 ? group_ks(make_plan(g, cta - 1, G).n) : 0;
-            if (pl.n > 0) group(pl.ta, pl.n, pl.s0_own_k0, pl.s0_pub_k1, pl.sl_k1, ksp, true);
-        } else {
-            for (int g0 = pl.t0; g0 < pl.t1; g0 += CONS_WARPS)
-                group(g0, min(CONS_WARPS, pl.t1 - g0), 0, 0, nch, 0, g0 + CONS_WARPS >= pl.t1);
-        }
     }
 }
 
@@ -717,10 +742,6 @@ __device__ __forceinline__ Smem *smem_base(unsigned char *raw) {
 struct NoPre {
     __device__ __forceinline__ void operator()(int) const {}
 };
-template <int PAIR, class Epi>
-__device__ __forceinline__ void gemm_consume(const Shared &S, const Gemm &g, int cta, int G, Rings &r, Epi &&epi) {
-    gemm_consume<PAIR>(S, g, cta, G, r, NoPre(), epi);
-}
 
 // Shared-memory set-up by the whole block (call once, followed by __syncthreads()).
 __device__ __forceinline__ void smem_init(Smem *sm) {
