@@ -768,8 +768,10 @@ int setup_persistent(ada_session *S, const Layout &lay) {
         return ADA_EUNSUPPORTED;
     }
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES));
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, st::THREADS, st::SMEM_BYTES));
-    if (nb < 1) {
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, mg::MEGA_THREADS, st::SMEM_BYTES));
+    cudaFuncAttributes fa;
+    CK(cudaFuncGetAttributes(&fa, kern));
+    if (nb < 1 || fa.numRegs * mg::MEGA_THREADS < mg::MEGA_REGS) {   // (a warp group waits for registers that the block was not launched with)
         g_cuda_err = "the persistent decode kernel does not fit on one multiprocessor of this device";
         return ADA_EUNSUPPORTED;
     }
@@ -887,7 +889,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             if (a.part) CK(cudaMemsetAsync(a.part, 0, kPartBytesPerCta * (size_t)S->grid, S->stream));
             CK(cudaMemsetAsync(a.attn_tag, 0, attn_tag_bytes(g, S->n_chunks), S->stream));   // phase numbers start over with every launch
             void *params[] = {(void *)&a};
-            CK(cudaLaunchCooperativeKernel(kern, dim3(S->grid), dim3(st::THREADS), params, st::SMEM_BYTES, S->stream));
+            CK(cudaLaunchCooperativeKernel(kern, dim3(S->grid), dim3(mg::MEGA_THREADS), params, st::SMEM_BYTES, S->stream));
             S->launches++;
             CK(cudaMemcpyAsync(S->pinned, &S->c.st->n_climbing, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, S->stream));
             CK(cudaMemcpyAsync(S->pinned + 2, a.err, sizeof(int32_t), cudaMemcpyDeviceToHost, S->stream));

@@ -13,6 +13,16 @@ __global__ void k_xfrag_pack(const float *__restrict__ X, int K, int cols, __nv_
     for (int c = 0; c < st::MAX_COLS; ++c) st::xfrag_store(out, k, c, c < cols && k < K ? X[(size_t)c * K + k] : 0.f);
 }
 
+struct ProbeEpilogue {
+    float *Y;
+    int ldy, mode, rows;
+    __device__ __forceinline__ void pre(int, int, int, int) const {}
+    __device__ __forceinline__ void operator()(int, bool act, int tile, int row, int col, float d0, float d1) const {
+        const int n = tile * 16 + row;
+        if (act && n < rows) Y[(size_t)col * ldy + n] = mode == 0 ? d0 : d0 / (1.0f + expf(-d0)) * d1;
+    }
+};
+
 // mode 0: Y[col][n] = sum_k W[n][k] X[col][k]                       (N rows)
 // mode 1: Y[col][n] = silu(g) * u, g = W[n].X, u = W[half + n].X     (half = N/2 rows of each)
 __global__ void __launch_bounds__(st::THREADS, 1)
@@ -23,7 +33,7 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
     st::smem_init(sm);
     __syncthreads();
     st::Shared S{sm, err, st::Trace{nullptr, nullptr, 0}, 0, st::WAIT_NS_DEFAULT};
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     const int cta = blockIdx.x, G = gridDim.x;
     st::Gemm g;
     g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0;
@@ -39,14 +49,11 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
         const uint64_t pol = st::policy_evict_last();
         for (int it = 0; it < repeat; ++it) st::gemm_produce_x(S, pl, X, cols_used, r, pol, st::NoHook(), st::NoHook());
     } else {
-        for (int it = 0; it < repeat; ++it)
-            st::gemm_consume(S, pl, cols_used, part, 1u, cta, r, st::NoPre(), [&](int tile, float (&d0)[4], float (&d1)[4]) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, c = 2 * (lane & 3) + (i & 1);
-                    if (n < (mode == 0 ? N : g.half) && c < cols) Y[(size_t)c * ldy + n] = mode == 0 ? d0[i] : d0[i] / (1.0f + expf(-d0[i])) * d1[i];
-                }
-            });
+        const ProbeEpilogue epi{Y, ldy, mode, mode == 0 ? N : g.half};
+        for (int it = 0; it < repeat; ++it) {
+            st::gemm_consume(S, pl, cols_used, (1u << cols) - 1u, part, 1u, cta, r, epi);
+            st::bar_consumers();   // the exchange area is free for the next product
+        }
     }
     st::settle_on_abort(S);
 }

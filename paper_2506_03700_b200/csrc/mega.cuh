@@ -1802,13 +1802,12 @@ __device__ __forceinline__ Gemm phase_gemm(const MegaArgs &A, int ph) {
     return g;
 }
 
-// Epilogues of the products: consumer warps, see gemm_consume.  lane / 4 (+ 8) is the row of the tile, 2 (lane % 4) + {0, 1} the columns.
+// Epilogues of the products: consumer warps, one element (row of the tile, column) per thread and pass; see gemm_consume.
 template <int HD> struct Epilogue {
     const MegaArgs &A;
     const Shared &S;
     const StepDesc &d;
     int ph, l;               // phase, 0-based layer
-    unsigned mask;           // columns of the product
     unsigned vseq;           // phase number whose normalisation factors vec[] has to hold
     bool scaled;             // the product's result is multiplied by them
     float scale;             // head: scale of the logits
@@ -1816,203 +1815,135 @@ template <int HD> struct Epilogue {
     bool next_in, final_in;  // down product: prepares the next layer's input, a head's input
 
     static constexpr int HALF = HD / 2, KSQ = HD / 16;
+    __device__ __forceinline__ int seq_of(int col) const { return A.seq0 + (A.nseq == 1 ? 0 : col / A.c.slots); }
 
     // operands fetched while the weights stream
-    __device__ __forceinline__ void pre(int tile) const {
+    __device__ __forceinline__ void pre(int ps, int tile, int row, int col) const {
         const Ctx &c = A.c;
-        const int lane = threadIdx.x & 31, rq = lane >> 2, c0 = 2 * (lane & 3), n0 = tile * 16;
-        uint32_t *stash = stash_of(S.sm);
-        if (ph == PH_QKV) {   // rotary factors and cache pages of this lane's two columns
+        const int n0 = tile * 16, n = n0 + row;
+        uint32_t *stash = stash_of(S.sm, ps);
+        if (ph == PH_QKV) {   // rotary factors, cache page
             const int qd = c.nq * HD, kvd = c.nkv * HD;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int cc = c0 + q;
-                if (!((mask >> cc) & 1u)) continue;
-                if (n0 < qd + kvd) {
-                    const float *cs = c.rope_cs + ((size_t)cc * HALF + ((n0 & (HD - 1)) >> 1) + rq) * 2;
-                    cp_async4(stash + (2 * q) * 32, cs);
-                    cp_async4(stash + (2 * q + 1) * 32, cs + 1);
-                }
-                if (n0 >= qd) cp_async4(stash + (4 + q) * 32, c.page_table + (size_t)(A.seq0 + (A.nseq == 1 ? 0 : cc / c.slots)) * c.max_pages + (d.pos[cc] >> c.page_shift));
-            }
-        } else if (ph == PH_O || ph == PH_DOWN) {   // residual and gains
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = n0 + rq + (i >> 1) * 8, cc = c0 + (i & 1);
-                if ((mask >> cc) & 1u) cp_async4(stash + i * 32, c.resid + (size_t)cc * c.d + n);
-            }
-            const __nv_bfloat16 *g1 = ph == PH_O ? A.m.ffn_norm[l] : A.m.attn_norm[next_in ? l + 1 : l];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int n2 = (n0 + rq + h * 8) & ~1;
-                cp_async4(stash + (4 + h) * 32, g1 + n2);
-                if (final_in) cp_async4(stash + (6 + h) * 32, A.m.final_norm + n2);
-            }
-        }
-    }
-    __device__ __forceinline__ void qkv(int tile, float (&acc)[4], float r0, float r1) const {
-        const Ctx &c = A.c;
-        const int lane = threadIdx.x & 31, rq = lane >> 2, c0 = 2 * (lane & 3), n0 = tile * 16;
-        const int qd = c.nq * HD, kvd = c.nkv * HD, group = c.group;
-        const float qscale = rsqrtf((float)HD);
-        uint32_t *stash = stash_of(S.sm);
-        __nv_bfloat16 *pool = reinterpret_cast<__nv_bfloat16 *>(c.kv_pool);
-        if (n0 >= c.qkv_rows) return;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int cc = c0 + q;
-            if (!((mask >> cc) & 1u)) continue;
-            const float rs = q ? r1 : r0;
-            const float x0 = acc[q] * rs, x1 = acc[2 + q] * rs;   // rows rq and rq + 8 of the tile
             if (n0 < qd + kvd) {
-                const float co = __uint_as_float(stash[(2 * q) * 32]), si = __uint_as_float(stash[(2 * q + 1) * 32]);
-                const int j = ((n0 & (HD - 1)) >> 1) + rq;   // feature j pairs with j + hd/2
-                const float y0 = x0 * co - x1 * si, y1 = x1 * co + x0 * si;
-                if (n0 < qd) {
-                    const int h = n0 / HD, kvh = div_group(h, group), qcol = cc * group + (h - kvh * group);
-                    const int row = qcol & 15, m = qcol >> 4;
-                    __nv_bfloat16 *f0 = reinterpret_cast<__nv_bfloat16 *>(A.qfrag + (((size_t)kvh * 2 + m) * KSQ) * 256);
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        const int dim = j + hh * HALF;
-                        const float y = (hh ? y1 : y0) * qscale;
-                        const int ks = dim >> 4, kk = dim & 15;
-                        const int ln = (row & 7) * 4 + ((kk & 7) >> 1), reg = (row >> 3) + 2 * (kk >> 3);
-                        const __nv_bfloat16 hi = __float2bfloat16_rn(y);
-                        const __nv_bfloat16 lo = __float2bfloat16_rn(y - __bfloat162float(hi));
-                        __nv_bfloat16 *f = f0 + ((size_t)ks * 32 + ln) * 16;
-                        f[reg * 2 + (kk & 1)] = hi;
-                        f[8 + reg * 2 + (kk & 1)] = lo;
-                    }
-                } else {
-                    const int kvh = (n0 - qd) / HD, pos = d.pos[cc], t = pos & (ATT_PAGE - 1);
-                    const size_t blk = ((((size_t)stash[(4 + q) * 32] * c.L + l) * 2 + 0) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)t * HD;
-                    pool[blk + ((((j >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(y0);
-                    pool[blk + (((((j + HALF) >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(y1);
-                }
-            } else {
-                const int nv = n0 - qd - kvd, kvh = nv / HD, j = (nv & (HD - 1)) + rq, pos = d.pos[cc], t = pos & (ATT_PAGE - 1);
-                const size_t blk = ((((size_t)stash[(4 + q) * 32] * c.L + l) * 2 + 1) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)t * HD;
-                pool[blk + ((((j >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(x0);
-                pool[blk + (((((j + 8) >> 3) ^ (pos & 7)) << 3) | (j & 7))] = __float2bfloat16_rn(x1);
+                const float *cs = c.rope_cs + ((size_t)col * HALF + ((n0 & (HD - 1)) >> 1) + (row & 7)) * 2;
+                cp_async4(stash, cs);
+                cp_async4(stash + CONS_THREADS, cs + 1);
             }
+            if (n0 >= qd) cp_async4(stash + 2 * CONS_THREADS, c.page_table + (size_t)seq_of(col) * c.max_pages + (d.pos[col] >> c.page_shift));
+        } else if (ph == PH_O || ph == PH_DOWN) {   // residual and gains
+            cp_async4(stash, c.resid + (size_t)col * c.d + n);
+            if (next_in) cp_async4(stash + CONS_THREADS, (ph == PH_O ? A.m.ffn_norm[l] : A.m.attn_norm[l + 1]) + (n & ~1));
+            if (final_in) cp_async4(stash + 2 * CONS_THREADS, A.m.final_norm + (n & ~1));
         }
     }
-    // O and down: residual add, inputs of the products that follow, partial sums of squares
-    __device__ __forceinline__ void residual(int tile, float (&acc)[4]) const {
+    __device__ __forceinline__ void operator()(int ps, bool act, int tile, int row, int col, float a0, float a1) const {
         const Ctx &c = A.c;
-        const int lane = threadIdx.x & 31, c0 = 2 * (lane & 3);
-        const uint32_t *stash = stash_of(S.sm);
-        __nv_bfloat16 *X1 = ph == PH_O ? A.XB : A.XA;
-        float *ssq = ph == PH_O ? A.ssq_b : A.ssq_a;
-        float sq[2] = {0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-            if ((mask >> cc) & 1u) {
-                const float v = __uint_as_float(stash[i * 32]) + acc[i];
-                c.resid[(size_t)cc * c.d + n] = v;
-                if (next_in) xfrag_store(X1, n, cc, v * bf16_of_word(stash[(4 + (i >> 1)) * 32], n));
-                if (final_in) xfrag_store(A.XF, n, cc, v * bf16_of_word(stash[(6 + (i >> 1)) * 32], n));
-                sq[i & 1] += v * v;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 4);
-            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 8);
-            sq[q] += __shfl_xor_sync(0xffffffffu, sq[q], 16);
-            if (lane < 4 && ((mask >> (c0 + q)) & 1u)) ssq[(size_t)tile * MAX_COLS + c0 + q] = sq[q];
-        }
-    }
-    __device__ __forceinline__ void operator()(int tile, float (&a0)[4], float (&a1)[4]) const {
-        const Ctx &c = A.c;
-        const int lane = threadIdx.x & 31, c0 = 2 * (lane & 3);
-        float r0 = 1.f, r1 = 1.f;
-        if (scaled) { vec_wait(S, vseq); r0 = S.sm->vec[c0]; r1 = S.sm->vec[c0 + 1]; }
+        const int n0 = tile * 16, n = n0 + row;
+        uint32_t *stash = stash_of(S.sm, ps);
+        float rs = 1.f;
+        if (scaled) { vec_wait(S, vseq); rs = S.sm->vec[col]; }
+        a0 *= rs;
         if (ph == PH_GU) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-                if ((mask >> cc) & 1u) {
-                    const float rs = (i & 1) ? r1 : r0;
-                    const float gv = a0[i] * rs, u = a1[i] * rs;
-                    xfrag_store(A.XH, n, cc, gv / (1.0f + expf(-gv)) * u);
-                }
-            }
+            a1 *= rs;
+            if (act) xfrag_store(A.XH, n, col, a0 / (1.0f + expf(-a0)) * a1);
         } else if (ph == PH_HEAD) {
-            // running (max, sum exp, argmax) of this lane's two columns, kept in its stash words; sampled decoding: logits over
+            // running (max, sum exp, argmax) of this thread's rows, kept in its stash words; sampled decoding: logits over
             // the temperature, which are kept, the final head's by column, an intermediate head's by the position of its row
             // (the verification of the token drawn from them needs them again)
-            uint32_t *stash = stash_of(S.sm);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int col = c0 + q;
-                const float f = (q ? r1 : r0) * scale;
-                float *zrow = nullptr;
-                if ((mask >> col) & 1u) {
-                    if (A.sampling && inter) zrow = A.q_stage + ((size_t)(A.seq0 + (A.nseq == 1 ? 0 : col / c.slots)) * MAX_COLS + (d.pos[col] & 7)) * c.vocab;
-                    else if (A.sampling || A.store_logits) zrow = c.logit_stage + (size_t)col * c.vocab;
-                }
-                Msa run;
-                run.m = __uint_as_float(stash[(3 * q) * 32]); run.s = __uint_as_float(stash[(3 * q + 1) * 32]); run.i = (int)stash[(3 * q + 2) * 32];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int n = tile * 16 + (lane >> 2) + h * 8;
-                    if (n < c.vocab) {
-                        const float z = a0[q + 2 * h] * f;
-                        if (zrow) zrow[n] = z;
-                        Msa one; one.m = z; one.s = 1.f; one.i = n;
-                        run = msa_merge(run, one);
-                    }
-                }
-                stash[(3 * q) * 32] = __float_as_uint(run.m); stash[(3 * q + 1) * 32] = __float_as_uint(run.s); stash[(3 * q + 2) * 32] = (uint32_t)run.i;
+            if (act && n < c.vocab) {
+                const float z = a0 * scale;
+                if (A.sampling && inter) A.q_stage[((size_t)seq_of(col) * MAX_COLS + (d.pos[col] & 7)) * c.vocab + n] = z;
+                else if (A.sampling || A.store_logits) c.logit_stage[(size_t)col * c.vocab + n] = z;
+                Msa run, one;
+                run.m = __uint_as_float(stash[0]); run.s = __uint_as_float(stash[CONS_THREADS]); run.i = (int)stash[2 * CONS_THREADS];
+                one.m = z; one.s = 1.f; one.i = n;
+                run = msa_merge(run, one);
+                stash[0] = __float_as_uint(run.m); stash[CONS_THREADS] = __float_as_uint(run.s); stash[2 * CONS_THREADS] = (uint32_t)run.i;
             }
         } else if (ph == PH_T) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = tile * 16 + (lane >> 2) + (i >> 1) * 8, cc = c0 + (i & 1);
-                xfrag_store(A.XT, n, cc, a0[i] * ((i & 1) ? r1 : r0));
-            }
-        } else {
+            if (act) xfrag_store(A.XT, n, col, a0);
+        } else if (ph == PH_QKV) {
             cp_async_wait_all();
-            if (ph == PH_QKV) qkv(tile, a0, r0, r1);
-            else residual(tile, a0);
+            const float other = __shfl_xor_sync(0xffffffffu, a0, 8);   // the partner of a rotation
+            const int qd = c.nq * HD, kvd = c.nkv * HD;
+            if (!act || n0 >= c.qkv_rows) return;
+            if (n0 < qd + kvd) {
+                const float co = __uint_as_float(stash[0]), si = __uint_as_float(stash[CONS_THREADS]);
+                const int dim = ((n0 & (HD - 1)) >> 1) + (row & 7) + (row >> 3) * HALF;   // rows r and r + 8 hold features j and j + hd/2
+                const float y = a0 * co + (row < 8 ? -other : other) * si;
+                if (n0 < qd) {
+                    const int h = n0 / HD, kvh = div_group(h, c.group), qcol = col * c.group + (h - kvh * c.group);
+                    const int qrow = qcol & 15, m = qcol >> 4, ks = dim >> 4, kk = dim & 15;
+                    const int ln = (qrow & 7) * 4 + ((kk & 7) >> 1), reg = (qrow >> 3) + 2 * (kk >> 3);
+                    const float yq = y * rsqrtf((float)HD);
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(yq);
+                    __nv_bfloat16 *f = reinterpret_cast<__nv_bfloat16 *>(A.qfrag) + ((((size_t)kvh * 2 + m) * KSQ + ks) * 32 + ln) * 16 + reg * 2 + (kk & 1);
+                    f[0] = hi;
+                    f[8] = __float2bfloat16_rn(yq - __bfloat162float(hi));
+                } else {
+                    cache_row(stash[2 * CONS_THREADS], 0, (n0 - qd) / HD, d.pos[col], dim, y);
+                }
+            } else {
+                const int nv = n - qd - kvd;
+                cache_row(stash[2 * CONS_THREADS], 1, nv / HD, d.pos[col], nv & (HD - 1), a0);
+            }
+        } else {   // O and down: residual add, inputs of the products that follow, partial sums of squares
+            cp_async_wait_all();
+            const float v = act ? __uint_as_float(stash[0]) + a0 : 0.f;
+            float sq = v * v;
+            sq += __shfl_xor_sync(0xffffffffu, sq, 8);
+            sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+            sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+            sq += __shfl_xor_sync(0xffffffffu, sq, 4);
+            if (!act) return;
+            c.resid[(size_t)col * c.d + n] = v;
+            if (next_in) xfrag_store(ph == PH_O ? A.XB : A.XA, n, col, v * bf16_of_word(stash[CONS_THREADS], n));
+            if (final_in) xfrag_store(A.XF, n, col, v * bf16_of_word(stash[2 * CONS_THREADS], n));
+            if (row == 0) (ph == PH_O ? A.ssq_b : A.ssq_a)[(size_t)tile * MAX_COLS + col] = sq;
         }
     }
-    __device__ __forceinline__ void head_begin() const {
-        uint32_t *stash = stash_of(S.sm);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) { stash[(3 * q) * 32] = __float_as_uint(-INFINITY); stash[(3 * q + 1) * 32] = 0u; stash[(3 * q + 2) * 32] = (uint32_t)INT_MAX; }
+    __device__ __forceinline__ void cache_row(uint32_t page, int which, int kvh, int pos, int dim, float v) const {   // one element of a K or V row
+        const Ctx &c = A.c;
+        const size_t blk = ((((size_t)page * c.L + l) * 2 + which) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)(pos & (ATT_PAGE - 1)) * HD;
+        reinterpret_cast<__nv_bfloat16 *>(c.kv_pool)[blk + ((((dim >> 3) ^ (pos & 7)) << 3) | (dim & 7))] = __float2bfloat16_rn(v);
     }
-    // the CTA's (max, sum exp, argmax) per column: lanes sharing lane%4 hold the same columns; they are folded, then the warps, in a fixed order
-    __device__ __forceinline__ void head_end() const {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c0 = 2 * (lane & 3);
-        const uint32_t *stash = stash_of(S.sm);
-        float *wp = reinterpret_cast<float *>(S.sm->scratch);   // [warp][col][4]
+    __device__ __forceinline__ void head_begin() const {
+#pragma unroll 1
+        for (int ps = 0; ps < STASH_PASSES; ++ps) {
+            uint32_t *stash = stash_of(S.sm, ps);
+            stash[0] = __float_as_uint(-INFINITY); stash[CONS_THREADS] = 0u; stash[2 * CONS_THREADS] = (uint32_t)INT_MAX;
+        }
+    }
+    // The CTA's (max, sum exp, argmax) of every column in use: the rows of a half-warp by a butterfly, then the column's
+    // half-warps (tile slots, see gemm_consume) in ascending order.
+    __device__ __forceinline__ void head_end(const Plan &pl, unsigned mask) const {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        float *wp = reinterpret_cast<float *>(S.sm->scratch);   // [half-warp of all passes][4]
         bar_consumers();
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
+#pragma unroll 1
+        for (int ps = 0; ps < STASH_PASSES; ++ps) {
+            const uint32_t *stash = stash_of(S.sm, ps);
             Msa run;
-            run.m = __uint_as_float(stash[(3 * q) * 32]); run.s = __uint_as_float(stash[(3 * q + 1) * 32]); run.i = (int)stash[(3 * q + 2) * 32];
+            run.m = __uint_as_float(stash[0]); run.s = __uint_as_float(stash[CONS_THREADS]); run.i = (int)stash[2 * CONS_THREADS];
 #pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
+            for (int off = 1; off < 16; off <<= 1) {
                 Msa o;
                 o.m = __shfl_xor_sync(0xffffffffu, run.m, off);
                 o.s = __shfl_xor_sync(0xffffffffu, run.s, off);
                 o.i = __shfl_xor_sync(0xffffffffu, run.i, off);
                 run = msa_merge(run, o);
             }
-            if (lane < 4) {
-                float *o = wp + ((size_t)warp * MAX_COLS + c0 + q) * 4;
+            if ((lane & 15) == 0) {
+                float *o = wp + (16 * ps + 2 * warp + (lane >> 4)) * 4;
                 o[0] = run.m; o[1] = run.s; o[2] = __int_as_float(run.i);
             }
         }
         bar_consumers();
-        if (threadIdx.x < MAX_COLS) {
+        if (threadIdx.x < MAX_COLS && ((mask >> threadIdx.x) & 1u)) {
+            const int sh = element_shift(Groups(pl).left), ci = __popc(mask & ((1u << threadIdx.x) - 1u));
             Msa a; a.m = -INFINITY; a.s = 0.f; a.i = INT_MAX;
-            for (int w = 0; w < CONS_WARPS; ++w) {
-                const float *o = wp + ((size_t)w * MAX_COLS + threadIdx.x) * 4;
+            for (int w = 0; w < 1 << sh; ++w) {
+                const float *o = wp + ((ci << sh) + w) * 4;
                 Msa x; x.m = o[0]; x.s = o[1]; x.i = __float_as_int(o[2]);
                 a = msa_merge(a, x);
             }
@@ -2103,7 +2034,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 // The rows of every q and k head come reordered so that a 16-row tile holds the features
                 // [8 t, 8 t + 8) and [hd/2 + 8 t, hd/2 + 8 t + 8): the two partners (i, i + hd/2) of a rotation
                 // are then rows r and r + 8 of one tile, which one thread holds for its two columns.
-                const Plan &pl = sm->plan[ph];
+                const Plan pl = sm->plan[ph];
                 const bool with_T = inter && M.has_T[l];
                 const unsigned vseq = bar_no + 1;
                 // the product's result is multiplied by the normalisation factors of its input's rows
@@ -2124,14 +2055,14 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                                    });
                 }
                 if (ROLE == 2) {
-                    const Epilogue<HD> epi{A, S, d, ph, l, cmask, vseq, scaled,
+                    const Epilogue<HD> epi{A, S, d, ph, l, vseq, scaled,
                                            final_head ? (A.sampling ? A.inv_temp : 1.0f) : inter ? M.head_scale[l] * (A.sampling ? A.inv_temp : 1.0f) : 1.0f, inter,
                                            ph == PH_O || l + 1 < L, ph == PH_DOWN && (l + 1 == L || M.exit_at[l + 1] != 0)};
                     // (an idle CTA must not report a phase before the one in front of it is complete: the counter would run ahead)
                     if (Groups(pl).left <= 0) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
                     if (ph == PH_HEAD) epi.head_begin();
-                    gemm_consume(S, pl, Cols(cmask), A.part, vseq, blockIdx.x, r, [&](int tile) { epi.pre(tile); }, epi);
-                    if (ph == PH_HEAD) epi.head_end();
+                    gemm_consume(S, pl, Cols(cmask), cmask, A.part, vseq, blockIdx.x, r, epi);
+                    if (ph == PH_HEAD) epi.head_end(pl, cmask);
                 }
             }
             if (ROLE == 2) {
@@ -2198,8 +2129,15 @@ __global__ void k_prefill_arm(Ctx c, int seq, int n_prompt) {
     for (int l = 0; l < c.L; ++l) c.fill[(size_t)seq * c.L + l] = 0;
 }
 
+// Warps 0-7 consume, warp 8 produces weights, warp 9 activations and K / V blocks; warps 10 and 11 only complete the producers'
+// warp group, which hands registers to the consumers.  (At 168 registers a thread -- three warps on a quarter of the SM --
+// the consumers kept loop variables in local memory, whose L1 lines do not survive the acquires of the grid barrier.)
+constexpr int MEGA_THREADS = CONS_THREADS + 128;
+constexpr int REGS_CONSUME = 216, REGS_PRODUCE = 72;
+constexpr int MEGA_REGS = CONS_THREADS * REGS_CONSUME + 128 * REGS_PRODUCE;   // the block must have been launched with as many
+
 template <int HD>
-__global__ void __launch_bounds__(THREADS, 1) k_decode_persistent(const __grid_constant__ MegaArgs A) {
+__global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __grid_constant__ MegaArgs A) {
     extern __shared__ unsigned char smem_raw[];
     Smem *sm = smem_base(smem_raw);
     smem_init(sm);
@@ -2210,9 +2148,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_decode_persistent(const __grid_c
     __syncthreads();
     Shared S{sm, A.err, A.trace, 0, A.wait_ns};
     const int warp = threadIdx.x >> 5;
-    if (warp == CONS_WARPS) run<0, HD>(A, S);
-    else if (warp == CONS_WARPS + 1) run<1, HD>(A, S);
-    else run<2, HD>(A, S);
+    if (warp < CONS_WARPS) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_CONSUME));
+        run<2, HD>(A, S);
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PRODUCE));
+        if (warp == CONS_WARPS) run<0, HD>(A, S);
+        else if (warp == CONS_WARPS + 1) run<1, HD>(A, S);
+    }
     settle_on_abort(S);
 }
 

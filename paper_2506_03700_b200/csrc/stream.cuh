@@ -151,6 +151,7 @@ struct Smem {                                    // must start on a 1024-byte bo
     int bcast[8];
     unsigned trace_n;
     unsigned vec_seq;                             // phase for which vec[] holds the normalisation factors (see vec_wait)
+    unsigned w_issued;                            // weight stages issued so far (see w_wait)
     Plan plan[6];                                 // this CTA's share of every product of the program
 };
 
@@ -299,15 +300,15 @@ __device__ __forceinline__ void mbar_wait(const Shared &S, unsigned long long *b
     }
 }
 
-// Epilogue operands are fetched while the weights stream, by 4-byte asynchronous copies into a
-// per-warp corner of the scratch area (word k of lane l at [k][l]) rather than into registers: a
+// Epilogue operands are fetched while the weights stream, by 4-byte asynchronous copies into words of
+// the scratch area that belong to one thread each (word k of pass p at [p][k][thread]) rather than into registers: a
 // value held in a register across the main loop ties up the register file, and wherever the
-// compiler has to move it the warp first waits for the load.  Each lane reads back only its own
-// words, after cp_async_wait_all().  The k-split reduction uses the first 8 KB of the scratch area.
-constexpr int STASH_OFFSET = 8192, STASH_WORDS = 8;
-static_assert(STASH_OFFSET + CONS_WARPS * STASH_WORDS * 32 * 4 <= SCRATCH_BYTES, "stash exceeds the scratch area");
-__device__ __forceinline__ uint32_t *stash_of(Smem *sm) {
-    return reinterpret_cast<uint32_t *>(sm->scratch + STASH_OFFSET) + (threadIdx.x >> 5) * (STASH_WORDS * 32) + (threadIdx.x & 31);
+// compiler has to move it the warp first waits for the load.  Each thread reads back only its own
+// words, after cp_async_wait_all().  The exchange of partial sums uses the first 8 KB of the scratch area.
+constexpr int STASH_OFFSET = RED_BYTES, STASH_WORDS = 3, STASH_PASSES = 4;   // passes: 8 tiles x 8 columns of 16 rows by 256 threads
+static_assert(STASH_OFFSET + STASH_PASSES * STASH_WORDS * CONS_THREADS * 4 <= SCRATCH_BYTES, "stash exceeds the scratch area");
+__device__ __forceinline__ uint32_t *stash_of(Smem *sm, int pass) {
+    return reinterpret_cast<uint32_t *>(sm->scratch + STASH_OFFSET) + pass * (STASH_WORDS * CONS_THREADS) + threadIdx.x;
 }
 __device__ __forceinline__ void cp_async4(uint32_t *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s32(dst)), "l"(src) : "memory");
@@ -335,8 +336,9 @@ __device__ __forceinline__ void vec_wait(const Shared &S, unsigned seq) {
 // Grid barrier on a monotonically increasing counter: arrive once per CTA, wait for `target`.
 __device__ __forceinline__ void grid_arrive(unsigned *ctr) {
     // the release of the reduction orders this thread's earlier writes, and through the block-level
-    // barrier before it those of the whole CTA; a separate fence before it only adds its latency
-    fence_proxy_async();
+    // barrier before it those of the whole CTA; a separate fence before it only adds its latency.  What bulk copies read of
+    // them is ordered by the proxy fence that every reader passes between its acquire and its first copy (one here as well
+    // cost 0.2 us a phase).
     red_release_add(ctr, 1u);
 }
 __device__ __forceinline__ void grid_wait(const Shared &S, const unsigned *ctr, unsigned target) {
@@ -397,14 +399,13 @@ struct Cols {
     // k chunks whose activations share one 16 KB stage: 4 for one column pair, 2 for two, else 1.  (The
     // ring holds three stages; with one chunk per stage a CTA that owns two weight tiles would wait
     // for an activation copy every 96 KB of weights.)
-    __device__ __forceinline__ int chunks() const { return ncp == 1 ? 4 : ncp == 2 ? 2 : 1; }
+    __device__ __forceinline__ int chunks() const { return ncp == 1 ? 4 : ncp == 2 ? 2 : 1; }   // a power of two
     // Up to four columns: one multiply-add takes their high parts as token columns 0..3 and their low parts as 4..7.
     __device__ __forceinline__ bool packed() const { return ncp <= 2; }
 };
 
-struct Rings {   // position of one role in the two rings: slot and parity of the next stage
-    uint32_t ws = 0, wp = 0, xs = 0, xp = 0;
-    __device__ __forceinline__ void next_w() { if (++ws == NW) { ws = 0; wp ^= 1; } }
+struct Rings {   // position of one role in the two rings: number of the next weight stage; slot and parity of the next activation stage
+    uint32_t w = 0, xs = 0, xp = 0;
     __device__ __forceinline__ void next_x() { if (++xs == NX) { xs = 0; xp ^= 1; } }
 };
 
@@ -415,6 +416,9 @@ struct Groups {
     __device__ __forceinline__ int slots() const { return min(left, CONS_WARPS); }
     __device__ __forceinline__ void next() { g0 += CONS_WARPS; left -= CONS_WARPS; }
 };
+// Tile slots over which gemm_consume spreads the elements of a group: log2 (eight where a plan has several groups, so that every
+// group is spread alike).
+__device__ __forceinline__ int element_shift(int slots) { return slots > CONS_WARPS ? 3 : slots > 1 ? 32 - __clz(slots - 1) : 0; }
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -422,6 +426,43 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
+}
+
+// Stages of a group of ng slots in front of chunk kc (in units of the plan's one or two matrices).
+__device__ __forceinline__ int stages_before(const Plan &p, int ng, int kc) {
+    const int gap = max(0, min(kc, p.s0_own_k0) - p.s0_pub_k1);            // chunks below kc at which slot 0 has none
+    const int end = ng > 1 ? max(0, kc - p.sl_k1) : 0;                     // chunks below kc at which the last slot has none any more
+    return kc * ng - gap - end;
+}
+
+// A weight stage is used, waited for and released by one warp only.  An mbarrier tells phases apart by one parity bit: a warp that
+// looks at a slot two fills ahead would take the fill before for its own.  So the producer publishes how many stages it has
+// issued: once stage i is among them, the fill before it in the same slot has been released, and the parity is unambiguous.
+// (With all eight warps waiting for and releasing every stage each of them walked the whole stream, and a slot was free again
+// only when the slowest of them, busy multiplying, had come by.)
+__device__ __forceinline__ void w_issued_set(Smem *sm, uint32_t n) { asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(s32(&sm->w_issued)), "r"(n) : "memory"); }
+__device__ __forceinline__ uint32_t w_issued_get(Smem *sm) {
+    uint32_t n;
+    asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(n) : "r"(s32(&sm->w_issued)) : "memory");
+    return n;
+}
+// Wait until stage i has landed; `known`: stages this warp knows to be issued.
+__device__ __forceinline__ void w_wait(const Shared &S, uint32_t i, uint32_t &known) {
+    if ((int)(known - i) <= 0) {
+        unsigned long long t0 = 0;
+        for (uint32_t it = 0;; ++it) {
+            known = w_issued_get(S.sm);
+            if ((int)(known - i) > 0) break;
+            if ((it & 127u) == 127u || S.wait_ns < SHORT_LIMIT_NS) {
+                if (aborted(S)) return;
+                if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; return; }
+                const unsigned long long t = gtime();
+                if (t0 == 0) t0 = t;
+                else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_MBAR); return; }
+            }
+        }
+    }
+    mbar_wait(S, &S.sm->w_full[i % NW], (i / NW) & 1);
 }
 
 // Weight producer warp: streams this CTA's tiles of the GEMM through the weight ring.  W2: map of the second matrix of a
@@ -442,12 +483,16 @@ __device__ __forceinline__ void gemm_produce_w(const Shared &S, const Plan &pl, 
                 if (tile < 0) continue;
 #pragma unroll 1
                 for (int p = 0; p < pair; ++p) {
-                    mbar_wait(S, &sm->w_empty[r.ws], r.wp ^ 1);
-                    if (lane == 0 && !aborted(S)) {
-                        mbar_expect_tx(&sm->w_full[r.ws], (uint32_t)W_STAGE);
-                        tma_load_3d(sm->w[r.ws], (p && W2) ? W2 : W, 0, tile * TILE_N + ((p && !W2) ? pl.half : 0), kc * KG, &sm->w_full[r.ws], pol);
+                    const uint32_t ws = r.w % NW;
+                    mbar_wait(S, &sm->w_empty[ws], ((r.w / NW) & 1) ^ 1);
+                    ++r.w;
+                    if (lane == 0) {
+                        if (!aborted(S)) {
+                            mbar_expect_tx(&sm->w_full[ws], (uint32_t)W_STAGE);
+                            tma_load_3d(sm->w[ws], (p && W2) ? W2 : W, 0, tile * TILE_N + ((p && !W2) ? pl.half : 0), kc * KG, &sm->w_full[ws], pol);
+                        }
+                        w_issued_set(sm, r.w);
                     }
-                    r.next_w();
                 }
             }
     }
@@ -496,9 +541,9 @@ struct NoHook {
 };
 
 // The 32 k-steps of one weight stage: fragment loads run four steps ahead of the multiply-adds that use them.
-// Even k-steps accumulate into acc[0] (high parts) and acc[2] (low parts), odd ones into acc[1] and acc[3]: four independent
-// accumulation chains.
-__device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+// K-step j accumulates into chain j % 4: acc[j % 4] (high parts) and acc[4 + j % 4] (low parts).  A chain's multiply-adds wait
+// for one another; with two chains a stage was sixteen of them in a row (0.4 us).
+__device__ __forceinline__ void stage_full(float (&acc)[8][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
     constexpr int PF = 4;
     uint32_t a[PF][4];
     uint4 b[PF];
@@ -510,8 +555,8 @@ __device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned ch
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
         const int cur = j % PF;
-        mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
-        mma16816(acc[(j & 1) + 2], a[cur], b[cur].z, b[cur].w);
+        mma16816(acc[j & 3], a[cur], b[cur].x, b[cur].y);
+        mma16816(acc[(j & 3) + 4], a[cur], b[cur].z, b[cur].w);
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
             ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
@@ -521,7 +566,7 @@ __device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned ch
 }
 // The same for up to four columns: their high parts are token columns 0..3 of one multiply-add, their low parts 4..7.
 // Half the multiply-adds and half the shared-memory reads; every sum has the order it has above.
-__device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+__device__ __forceinline__ void stage_packed(float (&acc)[8][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
     constexpr int PF = 4;
     uint32_t a[PF][4];
     uint2 b[PF];
@@ -533,7 +578,7 @@ __device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned 
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
         const int cur = j % PF;
-        mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
+        mma16816(acc[j & 3], a[cur], b[cur].x, b[cur].y);
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
             ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
@@ -544,19 +589,23 @@ __device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned 
 
 // Consumer warps.  Within a group of up to eight tiles the warps are arranged as TS tile slots x
 // KS k-splits (TS * KS = 8, TS the smallest power of two holding the group); a warp multiplies
-// the stages of its slot whose k chunk is ks_id (mod KS).  The k-splits of a tile are summed in a
-// fixed order through shared memory, then `epi(tile, d0, d1)` runs in the slot's first warp with
-//   dp[i]: fragment element i of matrix p: rows lane/4 (i<2) or lane/4+8, columns 2(lane%4)+(i&1).
-// The arrangement depends only on the tile partition, never on which token columns are in use.
-// `pre(tile)` runs in the same warp before the group's first stage (a place to start loads the epilogue will need).
+// the stages of its slot whose k chunk is ks_id (mod KS).  The arrangement depends only on the tile partition, never on which
+// token columns are in use.
+//
+// All warps' sums then meet in shared memory and every thread finishes elements of its own: half-warp u takes (tile slot
+// u mod E, the (u / E)-th column in use; E: element_shift), lane % 16 the row, in passes of sixteen half-warps; it adds the k-splits in index
+// order and calls `epi(pass, active, tile, row, column, d0, d1)` (the whole warp calls it together).  One warp per tile finishing
+// four elements a thread, the k-splits one after the other, was a chain of 1.6 us at the end of every phase.
+// `epi.pre(pass, tile, row, column)` runs in the same thread before the group's first stage: a place to start loads the epilogue will
+// need.
 //
 // One body for every product of a program (the caller loops over its phases and branches on the phase in `pre` and `epi`): with
 // a copy of it per product and role the persistent kernel was 790 KB of code, more than the instruction caches hold, and every
 // phase began and ended with instruction fetches from L2 on its critical path.
 // k steps past K multiply zeros (the tensor map fills weights with them, the activation blocks are padded with them).
-template <class Pre, class Epi>
-__device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, const Cols &cols, unsigned long long *part, unsigned phase_id, int cta, Rings &r,
-                                             Pre &&pre, Epi &&epi) {
+template <class Epi>
+__device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, const Cols &cols, unsigned mask, unsigned long long *part, unsigned phase_id, int cta,
+                                             Rings &r, const Epi &epi) {
     Smem *sm = S.sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = pl.nch, pair = pl.pair, XC = cols.chunks();
@@ -568,14 +617,16 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
     // this lane's column pair, if it was fetched (else any fetched pair: its column is not in use), and its 16 (8) bytes
     const int xpair = packed ? min((lane >> 3) & 1, cols.ncp - 1) : min(max((lane >> 3) - cols.cp0, 0), cols.ncp - 1);
     const int x_off = xpair * 4096 + (lane & 7) * 16 + (packed ? (lane >> 4) * 8 : 0);
+    const int nact = __popc(mask), row = lane & 15;
+    uint32_t known = r.w;
     bool first = true;
+    const int esh = element_shift(Groups(pl).left), eslots = 1 << esh;
+    const int n_pass = ((nact << esh) + 15) >> 4;
 #pragma unroll 1
     for (Groups g(pl); g.left > 0; g.next()) {
-        const int ng = g.slots();
-        int TS = 1;
-        while (TS < ng) TS <<= 1;
-        const int KS = CONS_WARPS / TS;
-        const int slot_id = warp & (TS - 1), ks_id = warp / TS;
+        const int ng = g.slots(), lts = 32 - __clz(ng - 1);   // (clz(0) = 32)
+        const int TS = 1 << lts, KS = CONS_WARPS >> lts;
+        const int slot_id = warp & (TS - 1), ks_id = warp >> lts;
         const bool mine = slot_id < ng;
         const bool pub_only = slot_id > 0 && slot_id == ng - 1 && sl_k1 < nch;
         // this warp's slot: chunks below my_pub_k1 go to the published part, chunks from my_own_k0 to its own tile
@@ -583,66 +634,65 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
         const int my_own_k0 = (!mine || pub_only) ? nch : slot_id == 0 ? s0_own_k0 : 0;
         const int own_tile = (mine && !pub_only) ? g.g0 + slot_id : -1;
         const bool tail = own_tile >= 0 && my_own_k0 > 0;   // the head part of this tile comes from CTA cta - 1
-        if (ks_id == 0 && own_tile >= 0) pre(own_tile);
-        float acc0[4][4], acc1[4][4];   // [even/odd step x hi/lo][fragment] of the one or two matrices
+        // this thread's elements: columns by pass, four bits each
+        unsigned my_cols = 0;
+#pragma unroll 1
+        for (int ps = 0; ps < n_pass; ++ps) {
+            const int u = 16 * ps + 2 * warp + (lane >> 4), slot = u & (eslots - 1);
+            int ci = u >> esh;
+            unsigned m = mask;
+            for (; ci > 0 && m; --ci) m &= m - 1;
+            const bool act = m != 0 && slot < ng && !(slot > 0 && slot == ng - 1 && sl_k1 < nch);
+            my_cols |= (act ? (unsigned)__ffs(m) - 1u : 15u) << (4 * ps);
+            if (act) epi.pre(ps, g.g0 + slot, row, __ffs(m) - 1);
+        }
+        float acc0[8][4], acc1[8][4];   // [hi/lo x chain][fragment] of the one or two matrices
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 8; ++q)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc0[q][i] = acc1[q][i] = 0.f;
-        // fold the partial accumulators in a fixed order: (even.hi + odd.hi) + (even.lo + odd.lo)
+        // fold the partial accumulators in a fixed order: the chains of the high parts, those of the low parts, both.
+        // Four columns or fewer: the result of column pair cp0 + j stands in the lanes with lane % 4 = j, else of pair j.
         float d0[4], d1[4];
-        auto fold = [&](float (&d)[4], float (&acc)[4][4]) {
+        auto fold = [&](float (&d)[4], float (&acc)[8][4]) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                float hi = acc[0][i] + acc[1][i];
-                if (packed) {   // the low parts' sums are two lanes on; then to the lanes the columns belong to
-                    hi += __shfl_xor_sync(0xffffffffu, hi, 2);
-                    d[i] = __shfl_sync(0xffffffffu, hi, (lane & ~3) | ((lane - cols.cp0) & 1));
-                } else {
-                    d[i] = hi + (acc[2][i] + acc[3][i]);
-                }
+                const float hi = (acc[0][i] + acc[1][i]) + (acc[2][i] + acc[3][i]);
+                d[i] = hi + (packed ? __shfl_xor_sync(0xffffffffu, hi, 2) : (acc[4][i] + acc[5][i]) + (acc[6][i] + acc[7][i]));
             }
         };
 #pragma unroll 1
         for (int kc = 0; kc < nch; ++kc) {
-            if (kc % XC == 0) mbar_wait(S, &sm->x_full[r.xs], r.xp);
+            if ((kc & (XC - 1)) == 0) mbar_wait(S, &sm->x_full[r.xs], r.xp);
             if (threadIdx.x == 0 && first) trace(S, EV_X0, 0);
             first = false;
-            const unsigned char *xs = sm->x[r.xs] + (kc % XC) * cols.ncp * 4096 + x_off;
             // the k-splits of a slot take whole stages in turn, counted from the first chunk of the part
             // (chunk kc belongs to split (kc - first) mod KS): a warp then multiplies all 32 k-steps of
             // a stage, which amortises the per-stage waiting and set-up (splitting every stage among
             // the warps streamed 20-30 % slower)
+            const bool here = kc < my_pub_k1 || kc >= my_own_k0;   // this slot has a stage at chunk kc
             const int kbase = kc < my_pub_k1 ? 0 : my_own_k0;
-            const bool my_turn = mine && ((kc - kbase) & (KS - 1)) == ks_id;
+            if (here && ((kc - kbase) & (KS - 1)) == ks_id) {
+                const unsigned char *xs = sm->x[r.xs] + (kc & (XC - 1)) * cols.ncp * 4096 + x_off;
+                const bool gap0 = slot_id > 0 && kc >= s0_pub_k1 && kc < s0_own_k0;   // slot 0 has none here
+                uint32_t i = r.w + (uint32_t)((stages_before(pl, ng, kc) + slot_id - gap0) * pair);
 #pragma unroll 1
-            for (int s = 0; s < ng; ++s) {
-                if (s == 0 ? (kc >= s0_pub_k1 && kc < s0_own_k0) : (s == ng - 1 && kc >= sl_k1)) continue;   // no stage: outside the parts
-#pragma unroll 1
-                for (int p = 0; p < pair; ++p) {
-                    // Every warp waits for and releases every stage in order, although only its owner
-                    // uses it.  An mbarrier tells phases apart by one parity bit: a warp that ran ahead
-                    // of, or fell behind, the others by a ring would mistake one phase of a slot for
-                    // another (releasing stages by their owners alone was tried: a lagging warp then
-                    // waits for a refill that needs its own release).  With all eight arrivals per
-                    // stage no warp is ever more than one ring away from any other.
-                    mbar_wait(S, &sm->w_full[r.ws], r.wp);
-                    if (s == slot_id && my_turn) {
-                        const unsigned char *ws = sm->w[r.ws] + a_off;
-                        if (packed) {
-                            if (p == 0) stage_packed(acc0, ws, xs, a_hi, a_sw);
-                            else stage_packed(acc1, ws, xs, a_hi, a_sw);
-                        } else {
-                            if (p == 0) stage_full(acc0, ws, xs, a_hi, a_sw);
-                            else stage_full(acc1, ws, xs, a_hi, a_sw);
-                        }
+                for (int p = 0; p < pair; ++p, ++i) {
+                    w_wait(S, i, known);
+                    const uint32_t wslot = i % NW;
+                    const unsigned char *ws = sm->w[wslot] + a_off;
+                    if (packed) {
+                        if (p == 0) stage_packed(acc0, ws, xs, a_hi, a_sw);
+                        else stage_packed(acc1, ws, xs, a_hi, a_sw);
+                    } else {
+                        if (p == 0) stage_full(acc0, ws, xs, a_hi, a_sw);
+                        else stage_full(acc1, ws, xs, a_hi, a_sw);
                     }
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm->w_empty[r.ws]);
-                    r.next_w();
+                    if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
                 }
             }
-            if (kc % XC == XC - 1 || kc == nch - 1) {
+            if ((kc & (XC - 1)) == XC - 1 || kc == nch - 1) {   // activation stages are shared: every warp waits for and releases each of them
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
                 r.next_x();
@@ -653,19 +703,20 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 // part that may follow in this slot.
                 unsigned long long *pb = part + (size_t)(cta * CONS_WARPS + ks_id) * 256;
                 fold(d0, acc0);
-                fold(d1, acc1);
+                if (pair == 2) fold(d1, acc1);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     st_relaxed_u64(pb + i * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d0[i]));
                     if (pair == 2) st_relaxed_u64(pb + (4 + i) * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d1[i]));
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) acc0[q][i] = acc1[q][i] = 0.f;
+                    for (int q = 0; q < 8; ++q) acc0[q][i] = acc1[q][i] = 0.f;
                 }
             }
         }
+        r.w += (uint32_t)(stages_before(pl, ng, nch) * pair);
         if (threadIdx.x == 0 && g.left <= CONS_WARPS) trace(S, EV_MAIN_END, 0);
         fold(d0, acc0);
-        fold(d1, acc1);
+        if (pair == 2) fold(d1, acc1);
         // The head part published by CTA cta - 1, in ksp k-splits: this slot's k-split warp j fetches
         // the published splits j, j + KS, ... (all at once: one round trip) and adds them to its own
         // sums in index order; the fixed-order reduction below then covers both parts.
@@ -706,27 +757,33 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 __nanosleep(64);
             }
         }
-        if (KS > 1) {
-            float *red = reinterpret_cast<float *>(sm->scratch) + (size_t)warp * (pair * 128);
+        float *red = reinterpret_cast<float *>(sm->scratch);   // [matrix][warp][fragment element][lane]
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                red[i * 32 + lane] = d0[i];
-                if (pair == 2) red[(4 + i) * 32 + lane] = d1[i];
-            }
-            bar_consumers();
-            if (ks_id == 0) {
-                for (int q = 1; q < KS; ++q) {
-                    const float *o = reinterpret_cast<const float *>(sm->scratch) + (size_t)(q * TS + slot_id) * (pair * 128);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        d0[i] += o[i * 32 + lane];
-                        if (pair == 2) d1[i] += o[(4 + i) * 32 + lane];
-                    }
-                }
-            }
+        for (int i = 0; i < 4; ++i) {
+            red[(warp * 4 + i) * 32 + lane] = d0[i];
+            if (pair == 2) red[((CONS_WARPS + warp) * 4 + i) * 32 + lane] = d1[i];
         }
-        if (ks_id == 0 && own_tile >= 0) epi(own_tile, d0, d1);
-        if (KS > 1) bar_consumers();
+        bar_consumers();
+#pragma unroll 1
+        for (int ps = 0; ps < n_pass; ++ps) {
+            const int slot = (16 * ps + 2 * warp + (lane >> 4)) & (eslots - 1), cn = (my_cols >> (4 * ps)) & 15;
+            const bool act = cn < MAX_COLS;
+            const int col = act ? cn : 0;
+            // element (row, column) of a warp's sums: fragment element 2 (row / 8) + column % 2 of lane 4 (row % 8) + column pair
+            const float *o = red + (((slot & (TS - 1)) * 4 + 2 * (row >> 3) + (col & 1)) * 32 + ((row & 7) << 2) + ((col >> 1) - (packed && act ? cols.cp0 : 0)));
+            float v0[CONS_WARPS], v1[CONS_WARPS];
+#pragma unroll
+            for (int q = 0; q < CONS_WARPS; ++q) {
+                v0[q] = q < KS ? o[(q << lts) * 128] : 0.f;
+                v1[q] = q < KS && pair == 2 ? o[(CONS_WARPS + (q << lts)) * 128] : 0.f;
+            }
+            float e0 = v0[0], e1 = v1[0];
+#pragma unroll
+            for (int q = 1; q < CONS_WARPS; ++q)
+                if (q < KS) { e0 += v0[q]; e1 += v1[q]; }
+            epi(ps, act, g.g0 + slot, row, col, e0, e1);
+        }
+        if (g.left > CONS_WARPS) bar_consumers();   // the next group writes the exchange area again (after the last one the caller meets)
     }
 }
 
@@ -739,18 +796,15 @@ __device__ __forceinline__ Smem *smem_base(unsigned char *raw) {
     return reinterpret_cast<Smem *>(raw + ((1024u - (a & 1023u)) & 1023u));
 }
 
-struct NoPre {
-    __device__ __forceinline__ void operator()(int) const {}
-};
-
 // Shared-memory set-up by the whole block (call once, followed by __syncthreads()).
 __device__ __forceinline__ void smem_init(Smem *sm) {
     if (threadIdx.x == 0) {
-        for (int i = 0; i < NW; ++i) { mbar_init(&sm->w_full[i], 1); mbar_init(&sm->w_empty[i], CONS_WARPS); }
+        for (int i = 0; i < NW; ++i) { mbar_init(&sm->w_full[i], 1); mbar_init(&sm->w_empty[i], 1); }
         for (int i = 0; i < NX; ++i) { mbar_init(&sm->x_full[i], 1); mbar_init(&sm->x_empty[i], CONS_WARPS); }
         sm->abort = 0;
         sm->trace_n = 0;
         sm->vec_seq = 0;
+        sm->w_issued = 0;
         fence_mbar_init();
         fence_proxy_async();
     }
