@@ -12,6 +12,7 @@
 #include "kernels.cuh"
 #include "gemm_probe.cuh"
 #include "mega.cuh"
+#include "resident.cuh"
 #include "dense.cuh"
 
 using namespace ada;
@@ -142,6 +143,11 @@ struct ada_session {
     CUtensorMap *maps_dev = nullptr;      // [6 L + 2]: wqkv, wo, wgu, wup, wdown per layer, lm_head, then T per 1-based layer
     bool sampling = false;   // the call in progress draws its tokens (ada_sampling_decode)
     float inv_temp = 1.0f;
+    // fp32 models whose rows fit: whole calls in one launch (resident.cuh)
+    bool resident = false;
+    size_t res_smem = 0, res_words = 0;      // shared memory of a CTA; bytes of the exchanged words
+    int res_grid = 0;
+    rs::Args rargs;
     int steps_per_launch = 256;
     unsigned long long wait_ns = st::WAIT_NS_DEFAULT;
     // dense prompt pass (tcgen05 GEMMs over blocks of up to dg::PF_ROWS positions)
@@ -178,7 +184,7 @@ namespace {
 // Scratch layout (all offsets 256-byte aligned).
 struct Layout {
     size_t st, rt, fill, tokens, page_table, head_res, resid, xn, qkv, q, attn_out, gu, hact, rope_cs, attn_part,
-        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, maps, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
+        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, res, res_err, maps, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
         grid_ctr, pub, err, attn_tag, q_stage, qinfo, uniforms, total;
 };
 
@@ -200,6 +206,20 @@ constexpr int kPartMaxGrid = 256;
 int attn_tag_chunks(const ada_config &g, int n_chunks) { return std::min(n_chunks, std::max(1, mg::ONE_ITEM_MAX / g.n_kv_heads)); }
 size_t attn_tag_bytes(const ada_config &g, int n_chunks) {
     return sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)attn_tag_chunks(g, n_chunks) * (g.head_dim + 2);
+}
+
+// Whether an fp32 model's calls can run in one launch (resident.cuh): most rows of its passes, or 0.  The bounds are those of the
+// kernel's tables; that the rows fit the shared memory is asked of the device when the session is created.
+int resident_rows(const ada_config &g, int batch, int max_early) {
+    if (g.dtype != ADA_DTYPE_FP32 || g.n_layers >= rs::MAX_L || (g.head_dim != 32 && g.head_dim != 64 && g.head_dim != 128)) return 0;
+    const int R = rows_alloc_for(g, batch, max_early);
+    return max_early + 1 <= rs::MAX_SLOTS && R <= rs::MAX_R ? R : 0;
+}
+constexpr int kResidentMaxGrid = 256;
+// exchanged words: layer input, FFN input, T output, q | k | v, attention partials, FFN activations, head partials
+size_t resident_words(const ada_config &g, int R, int n_chunks) {
+    const size_t qkv = (size_t)(g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim, part = (size_t)g.n_q_heads * n_chunks * (g.head_dim + 2);
+    return (size_t)R * (3 * (size_t)g.d_model + qkv + part + g.d_ff) + 4 * (size_t)R * kResidentMaxGrid;
 }
 
 Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, int head_blocks) {
@@ -240,6 +260,10 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.pf_rstd = take(sizeof(float) * P);
         L.pf_err = take(256);
         L.pf_flag = take(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS);
+    }
+    if (resident_rows(g, batch, max_early) > 0) {
+        L.res = take(resident_words(g, R, n_chunks) * sizeof(rs::u64));
+        L.res_err = take(256);
     }
     // persistent-kernel buffers (bf16 models)
     if (g.dtype == ADA_DTYPE_BF16) {
@@ -840,6 +864,112 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     return ADA_OK;
 }
 
+const void *resident_kernel(int hd) {
+    return hd == 32 ? (const void *)rs::k_decode_resident<1> : hd == 64 ? (const void *)rs::k_decode_resident<2> : (const void *)rs::k_decode_resident<4>;
+}
+// Set up the one-launch path of an fp32 session where it is open to it; other fp32 sessions run one kernel per operation.
+int setup_resident(ada_session *S, const Layout &lay) {
+    const ada_model *m = S->m;
+    const ada_config &g = m->cfg;
+    S->resident = false;
+    int R = resident_rows(g, S->batch, S->max_early);
+    if (R == 0) return ADA_OK;
+    // embeddings and gains are read eight bytes at a time, weight rows sixteen (as the per-operation kernels do)
+    auto aligned = [](const void *p, size_t a) { return (uintptr_t)p % a == 0; };
+    bool ok = aligned(m->tok_embed, 8) && aligned(m->final_norm, 8);
+    for (const LayerW &w : m->layers) ok = ok && aligned(w.attn_norm, 8) && aligned(w.ffn_norm, 8);
+    if (!ok) return ADA_OK;
+    const int qd = g.n_q_heads * g.head_dim, ku = std::max(std::max(g.d_model, qd), g.d_ff);
+    int ring = 2;
+    while (ring < S->slots + 1) ring *= 2;
+    int dev = 0, sms = 0, coop = 0, smem = 0, nb = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    CK(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // a prompt pass takes fewer rows where that is what fits (a row is d_model + ku floats of shared memory)
+    const int need = std::max(S->batch * S->slots, 8);
+    for (;; R -= 8) {
+        if (R < need) R = need;
+        S->res_smem = rs::shm_bytes(R, g.d_model, ku, g.head_dim, std::max(R, S->batch * ring), S->batch, g.n_layers);
+        if (S->res_smem <= (size_t)smem) break;
+        if (R == need) return ADA_OK;
+    }
+    if (!coop) return ADA_OK;
+    const void *kern = resident_kernel(g.head_dim);
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, rs::THREADS, S->res_smem));
+    if (nb < 1) return ADA_OK;
+    S->res_grid = std::min(sms, kResidentMaxGrid);
+    rs::Args &a = S->rargs;
+    memset(&a, 0, sizeof(a));
+    a.tok_embed = (const float *)m->tok_embed;
+    a.lm_head = (const float *)m->lm_head;
+    a.final_norm = (const float *)m->final_norm;
+    for (int l = 0; l < g.n_layers; ++l) {
+        const LayerW &w = m->layers[l];
+        a.layer[l] = {(const float *)w.attn_norm, (const float *)w.ffn_norm, (const float *)w.wq, (const float *)w.wk, (const float *)w.wv,
+                      (const float *)w.wo, (const float *)w.w_gate, (const float *)w.w_up, (const float *)w.w_down};
+    }
+    a.rope_base = g.rope_base;
+    a.batch = S->batch;
+    a.R = R;
+    a.ku = ku;
+    a.cs_ring = ring;
+    a.pf_rows = std::min(R, rs::TOK_RING);
+    S->res_words = resident_words(g, R, S->n_chunks) * sizeof(rs::u64);
+    rs::u64 *w = (rs::u64 *)((char *)S->scratch + lay.res);
+    auto take = [&](size_t n) { rs::u64 *at = w; w += n; return at; };
+    a.XA = take((size_t)R * g.d_model);
+    a.XB = take((size_t)R * g.d_model);
+    a.TT = take((size_t)R * g.d_model);
+    a.QT = take((size_t)R * S->c.qkv_rows);
+    a.PT = take((size_t)R * g.n_q_heads * S->n_chunks * (g.head_dim + 2));
+    a.HT = take((size_t)R * g.d_ff);
+    a.HP = take(4 * (size_t)R * kResidentMaxGrid);
+    a.err = (int *)((char *)S->scratch + lay.res_err);
+    S->resident = true;
+    return ADA_OK;
+}
+
+// One launch: the prompt of sequence pf_seq (pf_n tokens), or, with pf_n = 0, a whole decode call.
+int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layers, int n_exit, float gamma, int max_early, int eos_id, int tape_n, int n_tokens) {
+    const ada_model *m = S->m;
+    rs::Args &a = S->rargs;
+    a.c = S->c;   // capture pointers may have changed
+    memset(a.exit_at, 0, sizeof(a.exit_at));
+    for (int i = 0; i < n_exit; ++i) {
+        const int e = exit_layers[i];
+        a.exit_at[e] = 1;
+        a.head_scale[e] = m->head_scale[e];
+        a.head_T[e] = (const float *)m->head_T[e];
+    }
+    a.gamma = gamma;
+    a.max_early = max_early;
+    a.eos_id = eos_id;
+    a.tape_n = tape_n;
+    a.capture_cap = S->capture_cap;
+    a.store_logits = S->capture_dev ? 1 : 0;
+    a.prof = S->prof ? 1 : 0;
+    a.pf_seq = pf_seq;
+    a.pf_n = pf_n;
+    a.max_steps = (long long)(n_tokens + 2) * (max_early + 2) * 4 + 16;
+    a.wait_ns = S->wait_ns;
+    CK(cudaMemsetAsync(a.XA, 0, S->res_words, S->stream));   // phase numbers start over with every launch
+    CK(cudaMemsetAsync(a.err, 0, sizeof(int), S->stream));
+    void *params[] = {(void *)&a};
+    CK(cudaLaunchCooperativeKernel(resident_kernel(m->cfg.head_dim), dim3(S->res_grid), dim3(rs::THREADS), params, S->res_smem, S->stream));
+    S->launches++;
+    CK(cudaMemcpyAsync(S->pinned, a.err, sizeof(int), cudaMemcpyDeviceToHost, S->stream));
+    CK(cudaStreamSynchronize(S->stream));
+    S->syncs++;
+    if (S->pinned[0] != 0) {
+        g_cuda_err = "fp32 decode kernel: device-side error " + std::to_string(S->pinned[0]);
+        return ADA_ETIMEOUT;
+    }
+    return ADA_OK;
+}
+
 // Run the persistent kernel until the call's token targets are met.
 // The kernel holds eight token columns.  A sequence needs max_early + 1 of them, so a launch decodes
 // min(8 / (max_early + 1), batch) sequences together (one weight stream for all of them, lock-step: every step runs
@@ -949,6 +1079,8 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
     const bool plain = (n_exit == 0 || max_early == 0);
     if (S->mega && S->path == 1) {
         if ((rc = run_persistent(S, exit_layers, n_exit, plain, 0, S->batch, true))) return rc;
+    } else if (S->resident) {
+        if ((rc = run_resident(S, 0, 0, exit_layers, plain ? 0 : n_exit, gamma, max_early, eos_id, tape_n, n_tokens))) return rc;
     } else if (plain) {
         // every step is one token through all layers; the step count is known, no read-back needed
         for (int it = 0; it < max_steps_plain; ++it) {
@@ -1305,6 +1437,7 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
 #undef CKS
     {
         int rc = setup_persistent(S, lay);
+        if (!rc) rc = setup_resident(S, lay);
         if (rc) return fail(rc);
     }
     // dense prompt pass: bf16 models of the shapes above on a device with fifth-generation tensor cores
@@ -1418,6 +1551,14 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
     }
     if (dense) {
         if ((rc = prefill_dense(S, seq, n_prompt))) return rc;
+        S->prefilled[seq] = 1;
+        S->h_prompt[seq] = n_prompt;
+        S->h_len[seq] = n_prompt + 1;
+        S->h_reported[seq] = 0;
+        return ADA_OK;
+    }
+    if (S->resident) {
+        if ((rc = run_resident(S, seq, n_prompt, nullptr, 0, 2.0f, 0, -1, 0, 0))) return rc;
         S->prefilled[seq] = 1;
         S->h_prompt[seq] = n_prompt;
         S->h_len[seq] = n_prompt + 1;

@@ -1,0 +1,58 @@
+"""fp32 decoding in one launch (csrc/resident.cuh) against the per-operation kernels, which take the sessions that do not
+qualify for it: here one with room for sixteen early tokens."""
+
+import numpy as np
+import pytest
+
+from paper_2506_03700_b200 import binding, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def decode(gm, cfg, prompts, n, early, max_early, mode):
+    S = binding.Session(gm, len(prompts), max(len(p) for p in prompts) + n + 8, 16, max_early)
+    S.capture_logits(n)
+    for i, p in enumerate(prompts):
+        S.prefill(p, seq=i)
+    if mode == "plain":
+        out = S.plain_decode(n)
+    else:
+        if mode == "tape":   # exits against the heads' own decisions, so that tokens are rejected and the cache rolled back
+            S.set_exit_tape([1, 1, 0, 1, 2, 1, 1, 1, 0, 0, 1] * 6)
+        out = S.adaptive_decode(n, 0.3, cfg.exit_layers, early)
+    return out, S.captured_logits().cpu().numpy().astype(np.float64)
+
+
+# (q heads, kv heads, head_dim, width, d_ff, vocabulary): one and several 16-byte pieces per lane, ragged ones, rows of 768
+# elements and more (the weights of a row in several pieces; prompt passes of fewer rows), an odd vocabulary
+SHAPES = [(4, 4, 64, 256, 688, 2048), (6, 2, 32, 192, 328, 1001), (2, 1, 128, 256, 800, 515), (4, 1, 32, 1032, 136, 300)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("lens,early,mode", [((1,), 5, "plain"), ((31,), 5, "adaptive"), ((33,), 1, "tape"), ((127,), 5, "tape"),
+                                              ((130, 5, 64), 3, "adaptive"), ((40, 9, 17, 32, 1, 3, 8, 2), 5, "tape")])
+def test_one_launch_equals_the_per_operation_path(shape, lens, early, mode):
+    nq, nkv, hd, d, dff, vocab = shape
+    cfg = synth.small_config(n_layers=4, d_model=d, n_q_heads=nq, n_kv_heads=nkv, head_dim=hd, d_ff=dff, vocab=vocab, sigma=0.08,
+                             resid_scale=0.5, exit_layers=(1, 3))
+    w = synth.make_weights(cfg, device="cuda", norm_gain_jitter=0.2)
+    gm = binding.Model(cfg, w)
+    gm.set_exit_head(1, synth.make_head_transform(cfg, 1, device="cuda", noise=0.1), 4.0)
+    gm.set_exit_head(3, None, 4.0)
+    prompts = [synth.make_prompt(cfg, n=k, seq=i).numpy() for i, k in enumerate(lens)]
+    n = 20
+    out, lg = decode(gm, cfg, prompts, n, early, 5, mode)
+    ref, lr = decode(gm, cfg, prompts, n, early, 15 if len(lens) == 8 else 16, mode)
+    assert lg.shape == lr.shape
+    # The same fp32 products summed in another order.  Rounding of a sum of up to 1032 products: 6e-8 x sqrt(1032) = 2e-6 of its
+    # size; some 28 products one after the other: 1e-5; both sides and the largest of 6000 logits (four standard deviations):
+    # 6e-5 of the logits' spread.  Asserted: the bound that fp32 logits are held to against the oracle.
+    tol = 1e-4 * lr.std()
+    top = np.sort(lr, axis=-1)
+    clear = (top[:, -1] - top[:, -2]) > 2 * tol
+    stop = int(np.argmin(clear)) if not clear.all() else n
+    assert stop > 3, "the synthetic logits leave nothing to compare"
+    assert np.abs(lg[:stop] - lr[:stop]).max() <= tol
+    assert np.array_equal(out[0][:stop], ref[0][:stop])
+    for s in range(1, len(lens)):   # the other sequences' logits are not kept: their tokens
+        assert np.array_equal(out[s], ref[s])
