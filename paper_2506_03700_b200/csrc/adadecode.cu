@@ -184,8 +184,8 @@ namespace {
 // Scratch layout (all offsets 256-byte aligned).
 struct Layout {
     size_t st, rt, fill, tokens, page_table, head_res, resid, xn, qkv, q, attn_out, gu, hact, rope_cs, attn_part,
-        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, res, res_err, maps, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, attn_cnt, rope_freq, part,
-        grid_ctr, pub, err, attn_tag, q_stage, qinfo, uniforms, total;
+        head_part, logit_stage, head_log, t_out, pf_resid, pf_x, pf_u, pf_cs, pf_rstd, pf_err, pf_flag, pf_part, res, res_err, maps, xa, xb, xo, xh, xf, xt, ssq_a, ssq_b, qfrag, rope_freq, part,
+        grid_ctr, pub, err, q_stage, qinfo, uniforms, total;
 };
 
 bool model_fits_persistent(const ada_config &g);
@@ -201,11 +201,10 @@ constexpr int kDenseMin = 9;        // prompt tokens from which the dense pass i
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
 constexpr int kPartMaxGrid = 256;
 
-// chunk partials of the decode attention as tagged words (see attn_consume_single): the chunks that a phase with at most
-// ONE_ITEM_MAX work items, i.e. (kv head, chunk) pairs, can have; longer contexts exchange theirs through attn_part
-int attn_tag_chunks(const ada_config &g, int n_chunks) { return std::min(n_chunks, std::max(1, mg::ONE_ITEM_MAX / g.n_kv_heads)); }
+// Chunk partials of the decode attention: as floats for the per-operation kernels, as tagged words (see attn_consume) for the
+// persistent kernel, in the same memory (a session uses one path at a time, and the words are cleared before each launch).
 size_t attn_tag_bytes(const ada_config &g, int n_chunks) {
-    return sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)attn_tag_chunks(g, n_chunks) * (g.head_dim + 2);
+    return model_fits_persistent(g) ? sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)n_chunks * (g.head_dim + 2) : 0;
 }
 
 // Whether an fp32 model's calls can run in one launch (resident.cuh): most rows of its passes, or 0.  The bounds are those of the
@@ -244,7 +243,7 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
     L.gu = take(sizeof(float) * (size_t)R * 2 * g.d_ff);
     L.hact = take(sizeof(float) * (size_t)R * g.d_ff);
     L.rope_cs = take(sizeof(float) * (size_t)R * g.head_dim);
-    L.attn_part = take(sizeof(float) * (size_t)R * g.n_q_heads * n_chunks * (g.head_dim + 2));
+    L.attn_part = take(std::max(sizeof(float) * (size_t)R * g.n_q_heads * n_chunks * (g.head_dim + 2), attn_tag_bytes(g, n_chunks)));
     L.head_part = take(sizeof(float) * (size_t)head_blocks * kMaxRows * 4);
     // staged logits; a prompt's products exchange sums in the same memory (a head's logits are read within its own step)
     const size_t exchange = model_fits_persistent(g) ? dg::GPART_CTA * 2 * dg::MAX_PAIRS : 0;
@@ -276,14 +275,12 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.xh = take(st::xfrag_bytes(g.d_ff));
         L.ssq_a = take(sizeof(float) * (size_t)((g.d_model + 15) / 16) * st::MAX_COLS);
         L.ssq_b = take(sizeof(float) * (size_t)((g.d_model + 15) / 16) * st::MAX_COLS);
-        L.qfrag = take((size_t)g.n_kv_heads * 2 * (g.head_dim / 16) * 1024);
-        L.attn_cnt = take(sizeof(unsigned) * g.n_kv_heads * st::MAX_COLS);   // per (sequence of a launch, kv head)
+        L.qfrag = take((size_t)st::MAX_COLS * g.n_kv_heads * 2 * (g.head_dim / 16) * 1024);   // two tiles per (sequence of a launch, kv head)
         L.rope_freq = take(sizeof(double) * (g.head_dim / 2));
         L.part = take(kPartBytesPerCta * kPartMaxGrid);
         L.grid_ctr = take(256);
         L.pub = take(sizeof(mg::Pub) * 2);
         L.err = take(256);
-        L.attn_tag = take(attn_tag_bytes(g, n_chunks));
         // sampled decoding: the logits and normalisers of the intermediate head that drew each token in flight, and the
         // random numbers of every sequence position
         L.q_stage = take(sizeof(float) * (size_t)batch * st::MAX_COLS * g.vocab);
@@ -836,12 +833,8 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     a.XH = (__nv_bfloat16 *)(b + lay.xh); a.XF = (__nv_bfloat16 *)(b + lay.xf); a.XT = (__nv_bfloat16 *)(b + lay.xt);
     a.ssq_a = (float *)(b + lay.ssq_a); a.ssq_b = (float *)(b + lay.ssq_b);
     a.qfrag = (uint32_t *)(b + lay.qfrag);
-    a.attn_part = S->c.attn_part;
     a.head_part = S->c.head_part;
-    a.attn_cnt = (unsigned *)(b + lay.attn_cnt);
-    a.attn_tag = (unsigned long long *)(b + lay.attn_tag);
-    a.tag_chunks = attn_tag_chunks(g, S->n_chunks);
-    a.one_item_max = std::min(S->grid, mg::ONE_ITEM_MAX);
+    a.attn_tag = (unsigned long long *)S->c.attn_part;
     a.rope_freq = (const double *)(b + lay.rope_freq);
     a.part = S->grid <= kPartMaxGrid ? (unsigned long long *)(b + lay.part) : nullptr;
     a.grid_ctr = (unsigned *)(b + lay.grid_ctr);
@@ -996,9 +989,8 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             }
         }
     }
-    // a call that ended on a device-side error may have left the error word and the attention counters set
+    // a call that ended on a device-side error has left the error word set
     CK(cudaMemsetAsync(S->margs.err, 0, sizeof(int), S->stream));
-    CK(cudaMemsetAsync(S->margs.attn_cnt, 0, sizeof(unsigned) * g.n_kv_heads * st::MAX_COLS, S->stream));
     const void *kern = persistent_kernel_for(g.head_dim);
     const int per_launch = together ? std::max(1, st::MAX_COLS / S->slots) : 1;
     for (int sq = seq_begin; sq < seq_end; sq += per_launch) {

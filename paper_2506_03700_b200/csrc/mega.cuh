@@ -30,7 +30,6 @@ using namespace st;
 constexpr int ACT_CONTINUE = 1, ACT_NEWSTEP = 2, ACT_STOP = 3;
 constexpr int CTRL_START = 0, CTRL_HEAD = 1, CTRL_TOP = 2;
 constexpr int ATT_PAGE = 64;          // cache positions per attention sub-block (= KV page size on this path)
-constexpr int ONE_ITEM_MAX = 256;     // most attention work items of a phase that gives every CTA at most one (attn_consume_single)
 constexpr int ATT_CHUNK = kAttnChunk; // positions per attention work item (fixed: anchored at position 0)
 constexpr int ERR_BAD_STATE = 3;
 
@@ -76,21 +75,18 @@ struct MegaArgs {
     MegaModel m;
     __nv_bfloat16 *XA, *XB, *XO, *XH, *XF, *XT;   // GEMM inputs in fragment layout (see stream.cuh)
     float *ssq_a, *ssq_b;      // [d/16][8] partial sums of squares of the residual (per 16-feature tile, per column)
-    uint32_t *qfrag;           // [nkv][2][hd/16][32][8]: rotated, scaled queries as tensor-core A fragments (bf16 high parts, then low parts)
-    float *attn_part;          // [8 * nq][n_chunks][hd + 4]
+    uint32_t *qfrag;           // [sequence][nkv][2][hd/16][32][8]: rotated, scaled queries as tensor-core A fragments (bf16 high parts, then low parts)
     float *head_part;          // [grid][8][4]
     const double *rope_freq;   // [hd/2]: base^(-2i/hd), computed once on the host
     unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
-    unsigned *attn_cnt;        // [nkv]
-    unsigned long long *attn_tag;   // [8][nq][tag_chunks][hd + 2]: chunk partials as tagged words (see attn_consume_single); zeroed before each launch
-    int one_item_max;          // min(grid, ONE_ITEM_MAX)
-    int tag_chunks;            // chunks of a sequence they are laid out for: no more occur with ONE_ITEM_MAX work items in all
+    unsigned long long *attn_tag;   // [8][nq][n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume); zeroed before each launch
     unsigned *grid_ctr;
     Pub *pub;                  // [2]
     int *err;
     int step_budget;           // steps this launch may start
-    int seq0, nseq;            // the launch decodes sequences seq0 .. seq0 + nseq - 1 of the session together: sequence k of them owns the
-                               // token columns [k slots, (k + 1) slots), slots = max_early + 1, nseq slots <= 8; they share every weight stream
+    int seq0, nseq;            // the launch decodes sequences seq0 .. seq0 + nseq - 1 of the session together, nseq slots <= 8 (slots = max_early + 1):
+                               // slot j of sequence k of them is token column j nseq + k (neighbouring columns are then of equal age, and a
+                               // pass that carries the newest tokens only fetches few column pairs); they share every weight stream
     unsigned long long wait_ns;   // a single device-side wait gives up after this long
     int store_logits;
     // Sampled decoding (Eq. 1 with a drawn token, Eq. 2 with its acceptance test and the resampling): off = greedy
@@ -513,7 +509,7 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
     if (after_head) {
         for (int col = 0; col < MAX_COLS; ++col) {
             if (!((head_cols >> col) & 1u)) continue;
-            const int s = a.seq0 + (a.nseq == 1 ? 0 : col / cps), pos = dprev->pos[col], slot = s * MAX_COLS + (pos & 7);
+            const int s = a.seq0 + (a.nseq == 1 ? 0 : col % a.nseq), pos = dprev->pos[col], slot = s * MAX_COLS + (pos & 7);
             float total, wt;
             const int tok = block_draw_head(sm, a.q_stage + (size_t)slot * V, hr_s[col].zmax, a.head_part, col, a.G, V, unif(s, pos + 1, 3 + a.exit_idx), total, wt);
             if (tid == 0) {
@@ -525,11 +521,11 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
         }
     } else {
         for (int k = 0; k < a.nseq; ++k) {
-            const int s = a.seq0 + k, ln = a.st->len[s], bs = a.st->base[s], nrow = ln - bs, c0 = k * cps;
-            if (nrow < 1 || nrow > cps || dprev->first_layer[c0 + nrow - 1] > a.L - 1) continue;
+            const int s = a.seq0 + k, ln = a.st->len[s], bs = a.st->base[s], nrow = ln - bs;
+            if (nrow < 1 || nrow > cps || dprev->first_layer[(nrow - 1) * a.nseq + k] > a.L - 1) continue;
             bool rejected = false;
             for (int r = 0; r + 1 < nrow && !rejected; ++r) {
-                const int col = c0 + r, pos_t = bs + r + 1, t = min(max(tok_s[col], 0), V - 1), slot = s * MAX_COLS + ((bs + r) & 7);
+                const int col = r * a.nseq + k, pos_t = bs + r + 1, t = min(max(tok_s[col], 0), V - 1), slot = s * MAX_COLS + ((bs + r) & 7);
                 const float *zs = a.logit_stage + (size_t)col * V;
                 const float4 qi = a.qinfo[slot];
                 const float ps = __expf(__ldcg(zs + t) - hr_s[col].zmax) / hr_s[col].sumexp;
@@ -548,7 +544,7 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
                 if (tid == 0) hr_s[col].token = max(tok, 0);
             }
             if (!rejected) {
-                const int col = c0 + nrow - 1;
+                const int col = (nrow - 1) * a.nseq + k;
                 float total, wt;
                 const int tok = block_draw_head(sm, a.logit_stage + (size_t)col * V, hr_s[col].zmax, a.head_part, col, a.G, V, unif(s, ln, 0), total, wt);
                 if (tid == 0) hr_s[col].token = max(tok, 0);
@@ -581,10 +577,10 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     static_assert(ADA_MAX_LAYERS * MAX_COLS * sizeof(int) <= 8192, "fill levels of a launch's sequences must fit the scratch corner");
     for (int i = tid; i < nseq * L; i += CONS_THREADS) fill_s[i] = c.fill[(size_t)seq0 * L + i];
     if (tid >= CONS_THREADS - MAX_COLS) {
-        const int j = tid - (CONS_THREADS - MAX_COLS), k = j / cps;
+        const int j = tid - (CONS_THREADS - MAX_COLS), k = j % nseq;
         int v = -1;
-        if (k < nseq) {
-            const int at = st->base[seq0 + k] + (j - k * cps) + 1;
+        if (j / nseq < cps) {
+            const int at = st->base[seq0 + k] + j / nseq + 1;
             if (at < c.max_seq) v = c.tokens[(size_t)(seq0 + k) * c.max_seq + at];
         }
         tok_s[j] = v;
@@ -634,7 +630,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
             unsigned still = 0;   // sequences that go on climbing in this step
             int n_steps_seen = 0;
             for (int k = 0; k < nseq; ++k) {
-                const int s = seq0 + k, col = k * cps + (len[k] - 1 - base[k]);
+                const int s = seq0 + k, col = (len[k] - 1 - base[k]) * nseq + k;
                 if (col < 0 || col >= MAX_COLS || dprev.first_layer[col] > e - 1) continue;   // not in this step any more
                 if (!((head_cols >> col) & 1u)) { still |= 1u << k; continue; }                // climbing, but may not exit early
                 const HeadResult hr = hr_s[col];
@@ -665,8 +661,10 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                 bump(&st->st.exits_at_layer[e], 1);
                 bump(&st->st.steps, 1);
                 ++n_steps_seen;
-                for (int j = 0; j < cps; ++j) nd.first_layer[k * cps + j] = INT_MAX;   // the sequence sits out the rest of the step
-                nd.head_mask &= ~(((1 << cps) - 1) << (k * cps));
+                for (int j = k; j < MAX_COLS; j += nseq) {   // the sequence sits out the rest of the step
+                    nd.first_layer[j] = INT_MAX;
+                    nd.head_mask &= ~(1 << j);
+                }
             }
             if (tape_i != st->tape_i) st->tape_i = tape_i;
             if (hl_n != hl_n0) st->head_log_n = hl_n;
@@ -697,19 +695,19 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         // ---- verification (Eq. 2 at temperature zero) of every sequence whose newest token reached the last layer
         if (action != ACT_STOP && kind == CTRL_TOP && !prefilling) {
             for (int k = 0; k < nseq; ++k) {
-                const int s = seq0 + k, nrow = len[k] - base[k], c0 = k * cps;
-                if (nrow < 1 || nrow > cps || dprev.first_layer[c0 + nrow - 1] > L - 1) continue;   // left the step at an exit layer, or idle
+                const int s = seq0 + k, nrow = len[k] - base[k];
+                if (nrow < 1 || nrow > cps || dprev.first_layer[(nrow - 1) * nseq + k] > L - 1) continue;   // left the step at an exit layer, or idle
                 int32_t *tok = c.tokens + (size_t)s * c.max_seq;
                 long long rl = 0;
                 for (int l = 0; l < L; ++l) rl += len[k] - fill_s[k * L + l];
                 bump(&st->st.row_layers, rl);
                 int bad = -1;
                 for (int j = 0; j + 1 < nrow; ++j)
-                    if (hr_s[c0 + j].token != tok_s[c0 + j]) { bad = j; break; }
+                    if (hr_s[j * nseq + k].token != tok_s[j * nseq + k]) { bad = j; break; }
                 int new_base, keep;
                 if (bad < 0) {
                     bump(&st->st.accepted, nrow - 1);
-                    tok[len[k]] = min(max(hr_s[c0 + nrow - 1].token, 0), c.vocab - 1);
+                    tok[len[k]] = min(max(hr_s[(nrow - 1) * nseq + k].token, 0), c.vocab - 1);
                     new_base = len[k];
                     keep = nrow;
                 } else {
@@ -717,7 +715,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                     bump(&st->st.rejected, 1);
                     bump(&st->st.discarded, nrow - 2 - bad);
                     new_base = base[k] + bad + 1;
-                    tok[new_base] = min(max(hr_s[c0 + bad].token, 0), c.vocab - 1);
+                    tok[new_base] = min(max(hr_s[bad * nseq + k].token, 0), c.vocab - 1);
                     keep = bad + 1;
                 }
                 // Algorithm 1 runs "while t_i != [EOS]": the verified tokens of this step (positions base + 1 .. new_base,
@@ -726,7 +724,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                 int tgt = target[k];
                 if (eos0 >= 0) {
                     for (int j = 0; j < keep; ++j)
-                        if (min(max(hr_s[c0 + j].token, 0), c.vocab - 1) == eos0) {
+                        if (min(max(hr_s[j * nseq + k].token, 0), c.vocab - 1) == eos0) {
                             if (base[k] + j + 2 <= tgt) { tgt = base[k] + j + 2; st->eos_hit[s] = 1; }
                             break;
                         }
@@ -779,8 +777,8 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
             } else {
                 for (int k = 0; k < nseq; ++k) {
                     if (done[k]) continue;   // a sequence that has reached its target idles while the others go on
-                    const int nrow = len[k] - base[k], c0 = k * cps;
-                    if (nrow < 1 || nrow > cps || c0 + nrow > MAX_COLS || len[k] > c.max_seq || base[k] < 0) {
+                    const int nrow = len[k] - base[k];
+                    if (nrow < 1 || nrow > cps || nrow * nseq > MAX_COLS || len[k] > c.max_seq || base[k] < 0) {
                         atomicCAS(A.err, 0, ERR_BAD_STATE);
                         action = ACT_STOP;
                         break;
@@ -789,10 +787,10 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                         const int pos = base[k] + j;
                         int fl = 0;
                         for (int l = 0; l < L; ++l) fl += fill_s[k * L + l] > pos;
-                        nd.first_layer[c0 + j] = fl;
-                        nd.pos[c0 + j] = pos;
+                        nd.first_layer[j * nseq + k] = fl;
+                        nd.pos[j * nseq + k] = pos;
                     }
-                    const int cn = c0 + nrow - 1;
+                    const int cn = (nrow - 1) * nseq + k;
                     nd.n_cols += nrow;
                     nd.newest_mask |= 1 << cn;
                     nd.fresh |= 1 << cn;
@@ -824,7 +822,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         for (int col = 0; col < MAX_COLS; ++col) {
             if (!((nd.fresh >> col) & 1)) continue;
             const int pos = nd.pos[col];
-            const int tokid = min(max(c.tokens[(size_t)(seq0 + (nseq == 1 ? 0 : col / cps)) * c.max_seq + pos], 0), c.vocab - 1);
+            const int tokid = min(max(c.tokens[(size_t)(seq0 + (nseq == 1 ? 0 : col % nseq)) * c.max_seq + pos], 0), c.vocab - 1);
             const __nv_bfloat16 *erow = M.tok_embed + (size_t)tokid * c.d;
             for (int n0 = 0; n0 < c.d; n0 += 8 * CONS_THREADS) {   // eight loads of the embedding row and of the gain in flight per thread
                 float v[8], gn[8];
@@ -923,7 +921,7 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
         if (kind == CTRL_TOP && A.c.capture) {
             const int keep = sm->bcast[5], V = A.c.vocab;
             for (int j = 0; j < keep; ++j) {
-                const float *src = A.c.logit_stage + (size_t)(sm->bcast[7] + j) * V;
+                const float *src = A.c.logit_stage + (size_t)(sm->bcast[7] + j * A.nseq) * V;   // sequence 0's columns
                 float *dst = A.c.capture + (size_t)(sm->bcast[6] + j) * V;
                 for (int i0 = blockIdx.x * CONS_THREADS + threadIdx.x; i0 < V; i0 += 4 * gridDim.x * CONS_THREADS) {
                     float v[4];
@@ -950,18 +948,10 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
 
 // ---------------------------------------------------------------- attention phase
 
-// Shared memory of the attention phase, carved from the consumers' scratch.  The query fragments
-// are dead once the last score tile of an item is computed; the merge buffers reuse their space.
+// Shared memory of the attention phase: the consumers' scratch.
 template <int HD> struct AttnSmem {
-    union {
-        uint32_t qfrag[2][HD / 16][32][8];   // A fragments of the rotated, scaled queries: hi a0..a3, lo a0..a3
-        float o[2][2][16][HD];               // merge buffers [query tile][source]
-        float oq[4][16][HD];                 // one tile in use: [position quarter]
-    };
-    union {
-        float ml[2][2][2][16];               // [query tile][source][max | sum][row]
-        float mlq[4][2][16];                 // [position quarter][max | sum][row]
-    };
+    float o[CONS_WARPS][8][HD];      // unnormalised outputs of eight query rows by warp, columns rotated by 8 (row % 8)
+    float mx[CONS_WARPS][16], l[CONS_WARPS][16];   // row maxima and sums by warp
 };
 static_assert(sizeof(AttnSmem<128>) <= SCRATCH_BYTES, "attention buffers exceed the consumers' scratch");
 
@@ -969,235 +959,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t *>(&v);
 }
-
-// Attention work items of a launch that holds several sequences: sequence k of the launch (token columns
-// [k cps, (k + 1) cps); all eight in a prompt pass, which holds one sequence) contributes n_kv_heads x its
-// own number of 128-position chunks, and an item works on that sequence's columns and cache pages only.
-__device__ __forceinline__ unsigned seq_cols(const MegaArgs &A, int k) {
-    return A.nseq == 1 ? 0xffu : (((1u << A.c.slots) - 1u) << (k * A.c.slots));
-}
-__device__ __forceinline__ int seq_chunks(const MegaArgs &A, const StepDesc &d, unsigned mask, int k) {
-    return ((mask & seq_cols(A, k)) != 0 && d.seq_pmax[k] >= 0) ? d.seq_pmax[k] / ATT_CHUNK + 1 : 0;
-}
-__device__ __forceinline__ int attn_items(const MegaArgs &A, const StepDesc &d, unsigned mask) {
-    int n = 0;
-    for (int k = 0; k < A.nseq; ++k) n += A.c.nkv * seq_chunks(A, d, mask, k);
-    return n;
-}
-// item -> (sequence of the launch, kv head, chunk); nchunk = the sequence's chunk count
-__device__ __forceinline__ void attn_item(const MegaArgs &A, const StepDesc &d, unsigned mask, int item, int &k, int &kvh, int &j, int &nchunk) {
-    k = 0;
-    nchunk = seq_chunks(A, d, mask, 0);
-    while (k + 1 < A.nseq && item >= A.c.nkv * nchunk) {
-        item -= A.c.nkv * nchunk;
-        ++k;
-        nchunk = seq_chunks(A, d, mask, k);
-    }
-    nchunk = max(nchunk, 1);
-    kvh = min(item / nchunk, A.c.nkv - 1);
-    j = item - kvh * nchunk;
-}
-
-// Query tiles (16 (column, q head) pairs each) that hold a pair of the columns mk: bit t = tile t.
-__device__ __forceinline__ unsigned seq_tiles(const MegaArgs &A, unsigned mk) {
-    unsigned t = 0;
-#pragma unroll
-    for (int cc = 0; cc < MAX_COLS; ++cc)
-        if ((mk >> cc) & 1u) t |= (1u << ((cc * A.c.group) >> 4)) | (1u << ((cc * A.c.group + A.c.group - 1) >> 4));
-    return t & 3u;
-}
-// The consumers are two groups of four warps.  Where an item's queries span both tiles, group t works on tile t
-// of the same item.  Where every sequence's queries fit one tile (plain decoding; few columns; one q head per kv
-// head) the second group would idle: the groups then take DIFFERENT items, two per round, which halves the rounds
-// of a CTA that owns several items.  Which warps compute an item never changes what is computed.
-__device__ __forceinline__ bool attn_dual(const MegaArgs &A, unsigned mask) {
-    bool dual = true;
-    for (int k = 0; k < A.nseq; ++k) {
-        const unsigned t = seq_tiles(A, mask & seq_cols(A, k));
-        dual = dual && t != 3u;
-    }
-    return dual;
-}
-// One item of a round as every role sees it.
-struct AttnItem {
-    int k, kvh, j, nchunk, nsb, p_base, qt;   // sequence of the launch, kv head, chunk, the sequence's chunks, 64-position sub-blocks, first position, query tile
-    unsigned mk;                              // the sequence's active columns
-    bool have;
-};
-__device__ __forceinline__ AttnItem attn_item_of(const MegaArgs &A, const StepDesc &d, unsigned mask, int item, int n_items, bool dual, int grp) {
-    AttnItem it;
-    it.have = item < n_items;
-    it.k = it.kvh = it.j = it.nsb = it.p_base = it.qt = 0; it.nchunk = 1; it.mk = 0;
-    if (!it.have) return it;
-    attn_item(A, d, mask, item, it.k, it.kvh, it.j, it.nchunk);
-    it.mk = mask & seq_cols(A, it.k);
-    it.p_base = it.j * ATT_CHUNK;
-    it.nsb = min(ATT_CHUNK / ATT_PAGE, (d.seq_pmax[it.k] - it.p_base) / ATT_PAGE + 1);
-    it.qt = dual ? ((seq_tiles(A, it.mk) & 1u) ? 0 : 1) : grp;
-    return it;
-}
-
-// K/V producer: for every work item of this CTA, the K and V page blocks of its sub-blocks, in the order the
-// consumers walk them: per round (one item, or two in the dual arrangement) sub-block by sub-block, K of every
-// item of the round, then V.  The K and V rows of the tokens of this pass were written into the cache by the QKV
-// epilogues of other CTAs; an item whose positions include such a row is fetched only once the grid has passed
-// the barrier that ends the QKV phase (`bar_target`).  Every other item reads rows of earlier passes only and is
-// fetched as soon as ring slots are free, i.e. while the QKV product is still streaming.
-__device__ __forceinline__ void attn_produce(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, unsigned bar_target,
-                                             Rings &r, uint64_t pol) {
-    const Ctx &c = A.c;
-    Smem *sm = S.sm;
-    const int lane = threadIdx.x & 31, cta = blockIdx.x, G = gridDim.x;
-    const int n_items = attn_items(A, d, mask);
-    const bool dual = attn_dual(A, mask);
-    const int per_round = dual ? 2 : 1;
-    const uint32_t bytes = (uint32_t)(ATT_PAGE * c.hd * 2);
-    const __nv_bfloat16 *pool = reinterpret_cast<const __nv_bfloat16 *>(c.kv_pool);
-    bool synced = false;
-    if (lane == 0) trace(S, EV_ATT, 8);
-    for (int it0 = cta; it0 < n_items; it0 += G * per_round) {
-        AttnItem it[2];
-        it[0] = attn_item_of(A, d, mask, it0, n_items, dual, 0);
-        it[1] = attn_item_of(A, d, mask, dual ? it0 + G : n_items, n_items, dual, 1);
-        bool has_new = false;
-#pragma unroll
-        for (int g = 0; g < 2; ++g)
-#pragma unroll
-            for (int cc = 0; cc < MAX_COLS; ++cc)
-                has_new = has_new || (it[g].have && ((it[g].mk >> cc) & 1u) && d.pos[cc] >= it[g].p_base && d.pos[cc] < it[g].p_base + ATT_CHUNK);
-        if (has_new && !synced) {
-            grid_wait(S, A.grid_ctr, bar_target);
-            fence_proxy_async();
-            synced = true;
-        }
-        const int nsb = max(it[0].nsb, it[1].nsb);
-        for (int sb = 0; sb < nsb; ++sb)
-            for (int which = 0; which < 2; ++which)
-                for (int g = 0; g < per_round; ++g) {
-                    if (!it[g].have || sb >= it[g].nsb) continue;
-                    const int32_t *pages = c.page_table + (size_t)(A.seq0 + it[g].k) * c.max_pages;
-                    const int page = pages[(it[g].p_base + sb * ATT_PAGE) >> c.page_shift];
-                    const uint32_t slot = r.xs;
-                    mbar_wait(S, &sm->x_empty[slot], r.xp ^ 1);
-                    if (lane == 0 && !aborted(S)) {
-                        const size_t blk = ((((size_t)page * c.L + layer) * 2 + which) * c.nkv + it[g].kvh) * ((size_t)ATT_PAGE * c.hd);
-                        mbar_expect_tx(&sm->x_full[slot], bytes);
-                        bulk_g2s(sm->x[slot], pool + blk, bytes, &sm->x_full[slot], pol);
-                        trace(S, EV_ATT, 9 + 16 * (2 * sb + which));
-                    }
-                    r.next_x();
-                }
-    }
-}
-
-// The producer of a phase in which no CTA owns more than one item (see attn_consume_single).
-__device__ __forceinline__ void attn_produce_single(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, unsigned bar_target,
-                                             Rings &r, uint64_t pol) {
-    const Ctx &c = A.c;
-    Smem *sm = S.sm;
-    const int lane = threadIdx.x & 31, cta = blockIdx.x, G = gridDim.x;
-    const int n_items = attn_items(A, d, mask);
-    const uint32_t bytes = (uint32_t)(ATT_PAGE * c.hd * 2);
-    const __nv_bfloat16 *pool = reinterpret_cast<const __nv_bfloat16 *>(c.kv_pool);
-    bool synced = false;
-    if (lane == 0) trace(S, EV_ATT, 8);
-    for (int item = cta; item < n_items; item += G) {
-        int k, kvh, j, nchunk;
-        attn_item(A, d, mask, item, k, kvh, j, nchunk);
-        const unsigned mk = mask & seq_cols(A, k);
-        const int32_t *pages = c.page_table + (size_t)(A.seq0 + k) * c.max_pages;
-        const int p_base = j * ATT_CHUNK;
-        const int nsb = min(ATT_CHUNK / ATT_PAGE, (d.seq_pmax[k] - p_base) / ATT_PAGE + 1);
-        bool has_new = false;
-#pragma unroll
-        for (int cc = 0; cc < MAX_COLS; ++cc)
-            has_new = has_new || (((mk >> cc) & 1u) && d.pos[cc] >= p_base && d.pos[cc] < p_base + ATT_CHUNK);
-        if (has_new && !synced) {
-            grid_wait(S, A.grid_ctr, bar_target);
-            fence_proxy_async();
-            synced = true;
-        }
-        for (int sb = 0; sb < nsb; ++sb) {
-            const int page = pages[(p_base + sb * ATT_PAGE) >> c.page_shift];
-            for (int which = 0; which < 2; ++which) {
-                const uint32_t slot = r.xs;
-                mbar_wait(S, &sm->x_empty[slot], r.xp ^ 1);
-                if (lane == 0 && !aborted(S)) {
-                    const size_t blk = ((((size_t)page * c.L + layer) * 2 + which) * c.nkv + kvh) * ((size_t)ATT_PAGE * c.hd);
-                    mbar_expect_tx(&sm->x_full[slot], bytes);
-                    bulk_g2s(sm->x[slot], pool + blk, bytes, &sm->x_full[slot], pol);
-                    trace(S, EV_ATT, 9 + 16 * (2 * sb + which));
-                }
-                r.next_x();
-            }
-        }
-    }
-}
-
-// Two partial softmaxes (max, sum, unnormalised output) become one: (m, l) takes over (mb, lb); an output is a o + b ob.  The
-// operations are written out (no contraction left to the compiler): two places that merge the same pair get the same bits.
-__device__ __forceinline__ float merge_value(float oa, float a, float ob, float b) { return __fmaf_rn(oa, a, __fmul_rn(ob, b)); }
-__device__ __forceinline__ void merge_weights(float &m, float &l, float mb, float lb, float &a, float &b) {
-    const float mn = fmaxf(m, mb);
-    a = 1.f;
-    b = 0.f;
-    if (mn != -INFINITY) { a = __expf(m - mn); b = __expf(mb - mn); }
-    m = mn;
-    l = merge_value(l, a, lb, b);
-}
-
-// Merge (max, sum, unnormalised output) of another warp, read from shared memory, into this warp's.
-template <int NT, int HD>
-__device__ __forceinline__ void attn_merge_from(float (&o)[NT][4], float (&m_run)[2], float (&l_run)[2], const float (*so)[HD],
-                                                const float (*sml)[16], int lane) {
-#pragma unroll
-    for (int rh = 0; rh < 2; ++rh) {
-        const int row = (lane >> 2) + 8 * rh;
-        float a, b;
-        merge_weights(m_run[rh], l_run[rh], sml[0][row], sml[1][row], a, b);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {   // columns rotated by 8 (row % 8): conflict-free 8-byte accesses
-            const float2 v = *reinterpret_cast<const float2 *>(&so[row][(nt * 8 + 2 * (lane & 3) + 8 * (row & 7)) & (HD - 1)]);
-            o[nt][2 * rh] = merge_value(o[nt][2 * rh], a, v.x, b);
-            o[nt][2 * rh + 1] = merge_value(o[nt][2 * rh + 1], a, v.y, b);
-        }
-    }
-}
-template <int NT, int HD>
-__device__ __forceinline__ void attn_merge_to(const float (&o)[NT][4], const float (&m_run)[2], const float (&l_run)[2], float (*so)[HD],
-                                              float (*sml)[16], int lane) {
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int rh = 0; rh < 2; ++rh) {
-            const int row = (lane >> 2) + 8 * rh;
-            *reinterpret_cast<float2 *>(&so[row][(nt * 8 + 2 * (lane & 3) + 8 * (row & 7)) & (HD - 1)]) = make_float2(o[nt][2 * rh], o[nt][2 * rh + 1]);
-        }
-    if ((lane & 3) == 0) {
-#pragma unroll
-        for (int rh = 0; rh < 2; ++rh) {
-            sml[0][(lane >> 2) + 8 * rh] = m_run[rh];
-            sml[1][(lane >> 2) + 8 * rh] = l_run[rh];
-        }
-    }
-}
-
-// Consumers: causal attention of every active column over the cache, which by now holds the rows
-// of this pass too (the QKV epilogue wrote them).  Work item = (kv head, 128-position chunk).
-// Within a 64-position sub-block warp (mt, qr) handles query tile mt (16 of the up to 32 (column,
-// q head) pairs of the kv head) and positions [16 qr, 16 qr + 16).  The queries arrive rotated,
-// scaled and split into bf16 high / low parts, laid out as the tensor-core A fragments.
 // x / group for the q heads per kv head the persistent path admits (1..4) and x < 128, without the
 // general integer division (some thirty of those sat on the critical path of every attention item)
 __device__ __forceinline__ int div_group(int x, int group) {
     return group == 4 ? x >> 2 : group == 2 ? x >> 1 : group == 1 ? x : (x * 43) >> 7;
 }
-
-// Query tiles in use (bit t: some (column, q head) pair of the columns mk lies in rows [16 t, 16 t + 16)).
-__device__ __forceinline__ bool tile_in_use(unsigned mk, int t, int group) {
-    const int lo = div_group(16 * t, group), hi = div_group(16 * t + 15, group);
-    return (mk & ((2u << hi) - (1u << lo)) & 0xffu) != 0;
-}
+__device__ __forceinline__ void st_tagged(unsigned long long *p, float v, unsigned tag) { st_relaxed_u64(p, ((unsigned long long)tag << 32) | __float_as_uint(v)); }
 __device__ __forceinline__ void st_tagged2(unsigned long long *p, float a, float b, unsigned tag) {   // two tagged words; 16-byte aligned
     const unsigned long long t = (unsigned long long)tag << 32;
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | __float_as_uint(a)), "l"(t | __float_as_uint(b)) : "memory");
@@ -1210,576 +977,415 @@ __device__ __forceinline__ bool ld_tagged2(const unsigned long long *p, float &a
     return (unsigned)(x >> 32) == tag && (unsigned)(y >> 32) == tag;
 }
 
-// The same for a phase in which no CTA owns more than one item (contexts up to about 128 positions x CTAs / kv heads:
-// the common case of short and medium contexts): one item, its two query tiles on the two warp groups.  Kept as a path of
-// its own: the general form below, with its rounds of two items, costs this case 2-4 % of the step.
+// The active columns of the launch's k-th sequence as slots (bit j: column j nseq + k), and its 128-position chunks in this step.
+__device__ __forceinline__ unsigned seq_slots(const MegaArgs &A, unsigned mask, int k) {
+    if (A.nseq == 1) return mask;
+    unsigned m = 0;
+    for (int j = 0, col = k; col < MAX_COLS; ++j, col += A.nseq) m |= ((mask >> col) & 1u) << j;
+    return m;
+}
+__device__ __forceinline__ int seq_chunks(const MegaArgs &A, const StepDesc &d, unsigned mask, int k) {
+    return (d.seq_pmax[k] >= 0 && seq_slots(A, mask, k) != 0) ? d.seq_pmax[k] / ATT_CHUNK + 1 : 0;
+}
+
+// A work item: (sequence of the launch, kv head, 128-position chunk anchored at position 0).
+struct AttnItem {
+    int k, kvh, j, nsb, p_base;   // sequence, kv head, chunk, 64-position sub-blocks, first position
+    unsigned slots;               // the sequence's active slots
+    unsigned tiles;               // query tiles in use: row slot group + head of the sequence's (token, q head) pairs, sixteen to a tile
+    bool has_new;                 // holds positions of this pass, whose cache rows this step's QKV phase writes
+};
+// The items of one CTA in the order in which every role walks them: cta, cta + G, ...; those with rows of this pass last, since
+// their cache rows are there only when the QKV phase is complete.
+struct AttnWalk {
+    int pass, at, n;
+    __device__ __forceinline__ AttnWalk(const MegaArgs &A, const StepDesc &d, unsigned mask) : pass(0), at(blockIdx.x), n(0) {
+        for (int k = 0; k < A.nseq; ++k) n += A.c.nkv * seq_chunks(A, d, mask, k);
+    }
+    __device__ __forceinline__ bool next(const MegaArgs &A, const StepDesc &d, unsigned mask, AttnItem &it) {
+#pragma unroll 1
+        for (; pass < 2; ++pass, at = blockIdx.x)
+#pragma unroll 1
+            for (; at < n;) {
+                int i = at, nchunk = seq_chunks(A, d, mask, 0);
+                it.k = 0;
+                while (it.k + 1 < A.nseq && i >= A.c.nkv * nchunk) {
+                    i -= A.c.nkv * nchunk;
+                    nchunk = seq_chunks(A, d, mask, ++it.k);
+                }
+                nchunk = max(nchunk, 1);
+                it.kvh = min(i / nchunk, A.c.nkv - 1);
+                it.j = i - it.kvh * nchunk;
+                it.slots = seq_slots(A, mask, it.k);
+                it.p_base = it.j * ATT_CHUNK;
+                it.has_new = d.pos[(__ffs(it.slots) - 1) * A.nseq + it.k] < it.p_base + ATT_CHUNK;   // the lowest position of the pass
+                at += gridDim.x;
+                if ((int)it.has_new != pass) continue;
+                it.nsb = min(ATT_CHUNK / ATT_PAGE, (d.seq_pmax[it.k] - it.p_base) / ATT_PAGE + 1);
+                const int lo = (__ffs(it.slots) - 1) * A.c.group, hi = (32 - __clz(it.slots)) * A.c.group - 1;   // first and last row in use
+                it.tiles = (lo < 16 ? 1u : 0u) | (hi >= 16 ? 2u : 0u);
+                return true;
+            }
+        return false;
+    }
+};
+
+// K and V blocks (64 positions of one kv head, one cache page's share) travel through the weight ring, in line between the QKV
+// and the O product's weights: per item K of its sub-blocks, then V.  Nine blocks are in flight per CTA instead of the three that
+// the activation ring held, and O's weights follow without a gap.
+// The rows of the tokens of this pass are written by the QKV epilogues of other CTAs: an item that holds one is fetched once the
+// grid has passed the barrier that ends the QKV phase (`bar_target`), every other as soon as the ring has room.
+__device__ __forceinline__ void attn_produce_kv(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, unsigned bar_target,
+                                                Rings &r, uint64_t pol) {
+    const Ctx &c = A.c;
+    Smem *sm = S.sm;
+    const int lane = threadIdx.x & 31;
+    const uint32_t bytes = (uint32_t)(ATT_PAGE * c.hd * 2);
+    const __nv_bfloat16 *pool = reinterpret_cast<const __nv_bfloat16 *>(c.kv_pool);
+    AttnWalk w(A, d, mask);
+    AttnItem it;
+    bool synced = false;
+#pragma unroll 1
+    while (w.next(A, d, mask, it)) {
+        if (it.has_new && !synced) {
+            grid_wait(S, A.grid_ctr, bar_target);
+            fence_proxy_async();
+            synced = true;
+        }
+        const int32_t *pages = c.page_table + (size_t)(A.seq0 + it.k) * c.max_pages + (it.p_base >> c.page_shift);
+#pragma unroll 1
+        for (int b = 0; b < 2 * it.nsb; ++b) {
+            const int which = b >= it.nsb, page = pages[which ? b - it.nsb : b];
+            const uint32_t ws = r.w % NW;
+            mbar_wait(S, &sm->w_empty[ws], ((r.w / NW) & 1) ^ 1);
+            ++r.w;
+            if (lane == 0) {
+                if (!aborted(S)) {
+                    const size_t blk = ((((size_t)page * c.L + layer) * 2 + which) * c.nkv + it.kvh) * ((size_t)ATT_PAGE * c.hd);
+                    mbar_expect_tx(&sm->w_full[ws], bytes);
+                    bulk_g2s(sm->w[ws], pool + blk, bytes, &sm->w_full[ws], pol);
+                }
+                w_issued_set(sm, r.w);
+            }
+        }
+    }
+}
+// The items' query fragments come through the activation ring, one stage per item: the tiles in use, 64 hd bytes each.
+__device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &S, const StepDesc &d, unsigned mask, unsigned bar_target, Rings &r, uint64_t pol) {
+    const Ctx &c = A.c;
+    Smem *sm = S.sm;
+    const uint32_t tile_bytes = (uint32_t)c.hd * 64;
+    AttnWalk w(A, d, mask);
+    AttnItem it;
+    bool synced = false;
+#pragma unroll 1
+    while (w.next(A, d, mask, it)) {
+        mbar_wait(S, &sm->x_empty[r.xs], r.xp ^ 1);
+        if (!synced) {
+            grid_wait(S, A.grid_ctr, bar_target);
+            fence_proxy_async();
+            synced = true;
+        }
+        if ((threadIdx.x & 31) == 0 && !aborted(S)) {
+            const unsigned char *src = reinterpret_cast<const unsigned char *>(A.qfrag) + (size_t)(it.k * c.nkv + it.kvh) * 2 * tile_bytes + (it.tiles == 2u ? tile_bytes : 0u);
+            const uint32_t bytes = it.tiles == 3u ? 2 * tile_bytes : tile_bytes;
+            mbar_expect_tx(&sm->x_full[r.xs], bytes);
+            bulk_g2s(sm->x[r.xs], src, bytes, &sm->x_full[r.xs], pol);
+        }
+        r.next_x();
+    }
+}
+
+// Consumers: causal attention of every active column over the cache, which by now holds the rows of this pass too (the QKV
+// epilogue wrote them).  The queries arrive rotated, scaled and split into bf16 high / low parts, laid out as tensor-core A
+// fragments.
 //
-// The phase is a chain of latencies (1 us of arithmetic, 1 us of traffic, 11-14 us measured), so its exchanges are kept short:
-//   * with one query tile in use (plain decoding, few columns) the four position quarters meet once in shared memory and
-//     every thread merges elements of its own, in place of two levels of warp-to-warp merges with four barriers;
-//   * the chunk partials travel as 8-byte words that carry the phase number beside the value: whoever sees the tag sees the
-//     value, so no fence, counter and second look stand between writing and reading them (3.1-3.8 us before);
-//   * each of a head's chunk CTAs merges its share of the head's outputs, so a CTA reads as much as it wrote, in one
-//     round trip, however many chunks there are.  Who merges does not change what is computed.
+// An item's 128 positions are eight slices of sixteen.  Where its queries fit one tile of sixteen rows (plain decoding, few tokens
+// in flight) each warp takes a slice; where they span two, warp (tile, quarter) takes slices quarter and quarter + 4 of that tile.
+// Either way a row's numbers are formed alike: the maximum over the chunk first (exchanged through shared memory), weights
+// exp(score - maximum), one product per slice, slices s and s + 4 added, then (0 + 1) + (2 + 3).  So a token's attention does not
+// depend on which other tokens ride along.  (Running maxima per warp over two sub-blocks left half of the warps idle in the
+// one-tile case and cost two more meetings.)
+//
+// The chunk partials travel as 8-byte words that carry the phase number beside the value: whoever sees the tag sees the
+// value, so no fence, counter and second look stand between writing and reading them; all CTAs share the merging (a range of
+// the launch's (token, q head, feature pair)s each), in one round trip per eight chunks.  Who merges does not change what is computed.
 template <int HD>
-__device__ __forceinline__ void attn_consume_single(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, unsigned tag, Rings &r) {
+__device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S, const StepDesc &d, unsigned mask, unsigned tag, Rings &r) {
     const Ctx &c = A.c;
     Smem *sm = S.sm;
     AttnSmem<HD> *as = reinterpret_cast<AttnSmem<HD> *>(sm->scratch);
     constexpr int KSQ = HD / 16, NT = HD / 8;
     constexpr int TS = HD + 2;                             // tagged words per chunk partial: output, max, sum
-    constexpr int QV = 2 * KSQ * 64 / CONS_THREADS;        // 16-byte pieces of a kv head's query fragments per thread
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x;
-    const int group = c.group;
-    const int n_items = attn_items(A, d, mask);
-    const int mt = warp >> 2, qr = warp & 3;
-    (void)layer;
-    for (int item = cta; item < n_items; item += n_items) {   // at most one (the caller's condition)
-        int ks_, kvh, j, nchunk;
-        attn_item(A, d, mask, item, ks_, kvh, j, nchunk);
-        const unsigned mk = mask & seq_cols(A, ks_);   // the item's sequence: its columns only
-        const int p_base = j * ATT_CHUNK;
-        const int nsb = min(ATT_CHUNK / ATT_PAGE, (d.seq_pmax[ks_] - p_base) / ATT_PAGE + 1);
-        const bool one_tile = !tile_in_use(mk, 1, group), tile_used = tile_in_use(mk, mt, group);
-        // per-warp online softmax state: rows (lane/4) and (lane/4)+8 of query tile mt
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int group = c.group, nseq = A.nseq;
+    auto words = [&](int col, int h, int chunk) { return A.attn_tag + (((size_t)col * c.nq + h) * c.n_chunks + chunk) * TS; };
+    uint32_t known = r.w;
+    AttnWalk walk(A, d, mask);
+    AttnItem it;
+#pragma unroll 1
+    while (walk.next(A, d, mask, it)) {
+        const bool one_tile = it.tiles != 3u;
+        const int mt = one_tile ? (int)(it.tiles >> 1) : warp >> 2, qr = warp & 3;
+        const uint32_t k_stage = r.w, v_stage = r.w + it.nsb;
+        r.w += 2 * it.nsb;
+        // last position that rows lane / 4 and lane / 4 + 8 of the tile see (-1: no token)
         int lim[2];
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {
-            const int qcol = mt * 16 + (lane >> 2) + rh * 8, cc = div_group(qcol, group);
-            lim[rh] = (cc < MAX_COLS && ((mk >> cc) & 1u)) ? d.pos[cc] : -1;
+            const int slot = div_group(mt * 16 + (lane >> 2) + rh * 8, group);
+            lim[rh] = slot < 8 && ((it.slots >> slot) & 1u) ? d.pos[slot * nseq + it.k] : -1;
         }
-        // ---- the kv head's query fragments: one round trip to L2, then shared memory
-        {
-            const uint4 *src = reinterpret_cast<const uint4 *>(A.qfrag) + (size_t)kvh * (2 * KSQ * 64);
-            uint4 v[QV];
-#pragma unroll
-            for (int u = 0; u < QV; ++u) v[u] = __ldcg(src + tid + u * CONS_THREADS);
-#pragma unroll
-            for (int u = 0; u < QV; ++u) reinterpret_cast<uint4 *>(&as->qfrag[0][0][0][0])[tid + u * CONS_THREADS] = v[u];
-        }
-        bar_consumers();
+        mbar_wait(S, &sm->x_full[r.xs], r.xp);
         if (tid == 0) trace(S, EV_ATT, 2);   // queries ready
-        float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-        float o[NT][4];
+        const unsigned char *qs = sm->x[r.xs] + (one_tile ? 0 : mt) * (HD * 64) + lane * 32;
+        float s[2][2][4], m[2] = {-INFINITY, -INFINITY};   // scores [slice][n-tile][fragment], row maxima
+        const int sb0 = one_tile ? warp >> 2 : 0, n_sl = one_tile ? (sb0 < it.nsb ? 1 : 0) : it.nsb;
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) o[nt][i] = 0.f;
-        for (int sb = 0; sb < nsb; ++sb) {
-            const int p0 = p_base + sb * ATT_PAGE;
-            float s[2][4];
-            {   // ---- K block
-                const uint32_t slot = r.xs;
-                mbar_wait(S, &sm->x_full[slot], r.xp);
-                if (tid == 0) trace(S, EV_ATT, 3 + 16 * sb);   // K block landed
-                const unsigned char *kb = sm->x[slot];
-                float sh[2][4], sl[2][4];
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { sh[nt][i] = 0.f; sl[nt][i] = 0.f; }
-                const int id = lane >> 3;
-                const int pl = 16 * qr + (lane & 7) + 8 * (id >> 1);
-                const unsigned char *krow = kb + pl * (HD * 2);
-                if (tile_used)
-#pragma unroll
-                for (int k0 = 0; k0 < KSQ; k0 += 4) {   // four k-steps of loads in flight, then their multiply-adds
-                    uint4 qh[4], ql[4];
-                    uint32_t kf[4][4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int ks = k0 + u;
-                        qh[u] = *reinterpret_cast<const uint4 *>(&as->qfrag[mt][ks][lane][0]);
-                        ql[u] = *reinterpret_cast<const uint4 *>(&as->qfrag[mt][ks][lane][4]);
-                        ldmatrix_x4(kf[u], krow + ((((2 * ks) | (id & 1)) ^ (pl & 7)) << 4));
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const uint32_t ah[4] = {qh[u].x, qh[u].y, qh[u].z, qh[u].w}, al[4] = {ql[u].x, ql[u].y, ql[u].z, ql[u].w};
-                        mma16816(sh[0], ah, kf[u][0], kf[u][1]);
-                        mma16816(sh[1], ah, kf[u][2], kf[u][3]);
-                        mma16816(sl[0], al, kf[u][0], kf[u][1]);
-                        mma16816(sl[1], al, kf[u][2], kf[u][3]);
-                    }
-                }
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int pos = p0 + 16 * qr + 8 * nt + 2 * (lane & 3) + (i & 1);
-                        s[nt][i] = pos <= lim[i >> 1] ? sh[nt][i] + sl[nt][i] : -INFINITY;
-                    }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                r.next_x();
-            }
-            // ---- online softmax over this warp's 16 positions
-            uint32_t ph[4], plo[4];
-#pragma unroll
-            for (int rh = 0; rh < 2; ++rh) {
-                float mx = fmaxf(fmaxf(s[0][2 * rh], s[0][2 * rh + 1]), fmaxf(s[1][2 * rh], s[1][2 * rh + 1]));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                const float mn = fmaxf(m_run[rh], mx);
-                float corr = 1.f, p[4] = {0.f, 0.f, 0.f, 0.f};
-                if (mn != -INFINITY) {
-                    corr = __expf(m_run[rh] - mn);
-                    p[0] = __expf(s[0][2 * rh] - mn); p[1] = __expf(s[0][2 * rh + 1] - mn);
-                    p[2] = __expf(s[1][2 * rh] - mn); p[3] = __expf(s[1][2 * rh + 1] - mn);
-                }
-                m_run[rh] = mn;
-                l_run[rh] = l_run[rh] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) { o[nt][2 * rh] *= corr; o[nt][2 * rh + 1] *= corr; }
-                // A fragment of P: a0/a1 = n-tile 0 (rows r / r+8), a2/a3 = n-tile 1
-                const __nv_bfloat162 h0 = __floats2bfloat162_rn(p[0], p[1]), h1 = __floats2bfloat162_rn(p[2], p[3]);
-                ph[rh] = *reinterpret_cast<const uint32_t *>(&h0);
-                ph[2 + rh] = *reinterpret_cast<const uint32_t *>(&h1);
-                plo[rh] = pack_bf16(p[0] - __low2float(h0), p[1] - __high2float(h0));
-                plo[2 + rh] = pack_bf16(p[2] - __low2float(h1), p[3] - __high2float(h1));
-            }
-            {   // ---- V block
-                const uint32_t slot = r.xs;
-                mbar_wait(S, &sm->x_full[slot], r.xp);
-                if (tid == 0) trace(S, EV_ATT, 4 + 16 * sb);   // V block landed
-                const unsigned char *vb = sm->x[slot];
-                const int id = lane >> 3;
-                const int pl = 16 * qr + (lane & 7) + 8 * (id & 1);
-                const unsigned char *vrow = vb + pl * (HD * 2);
-                if (tile_used)
-#pragma unroll
-                for (int n0 = 0; n0 < NT / 2; n0 += 4) {
-                    uint32_t vf[4][4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) ldmatrix_x4_trans(vf[u], vrow + ((((2 * (n0 + u)) | (id >> 1)) ^ (pl & 7)) << 4));
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int np = n0 + u;
-                        mma16816(o[2 * np], ph, vf[u][0], vf[u][1]);
-                        mma16816(o[2 * np + 1], ph, vf[u][2], vf[u][3]);
-                        mma16816(o[2 * np], plo, vf[u][0], vf[u][1]);
-                        mma16816(o[2 * np + 1], plo, vf[u][2], vf[u][3]);
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                r.next_x();
-            }
-        }
-        // ---- row sums over the quad, then merge the four position quarters of each query tile:
-        //      (q0 + q1) and (q2 + q3), then the two halves
-#pragma unroll
-        for (int rh = 0; rh < 2; ++rh) {
-            l_run[rh] += __shfl_xor_sync(0xffffffffu, l_run[rh], 1);
-            l_run[rh] += __shfl_xor_sync(0xffffffffu, l_run[rh], 2);
-        }
-        if (tid == 0) trace(S, EV_ATT, 5);   // sub-blocks done
-        bar_consumers();   // every warp is done with the query fragments, whose space the merge reuses
-        auto words = [&](int cc, int h, int chunk) { return A.attn_tag + (((size_t)cc * c.nq + h) * A.tag_chunks + chunk) * TS; };
-        if (one_tile) {
-            if (mt == 0) attn_merge_to<NT, HD>(o, m_run, l_run, as->oq[qr], as->mlq[qr], lane);
-            bar_consumers();
-            // two features per thread and pass: (quarter 0 + quarter 1) + (quarter 2 + quarter 3), like the warps below
-            for (int idx = tid; idx < 16 * (HD / 2); idx += CONS_THREADS) {
-                const int row = idx / (HD / 2), dim = (idx % (HD / 2)) * 2, cc = div_group(row, group), g = row - cc * group;
-                if (cc >= MAX_COLS || !((mk >> cc) & 1u) || d.pos[cc] < p_base) continue;
-                float m[4], l[4];
-                float2 v[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    m[q] = as->mlq[q][0][row];
-                    l[q] = as->mlq[q][1][row];
-                    v[q] = *reinterpret_cast<const float2 *>(&as->oq[q][row][(dim + 8 * (row & 7)) & (HD - 1)]);
-                }
-                float a, b;
-#pragma unroll
-                for (int q = 0; q < 4; q += 2) {
-                    merge_weights(m[q], l[q], m[q + 1], l[q + 1], a, b);
-                    v[q].x = merge_value(v[q].x, a, v[q + 1].x, b);
-                    v[q].y = merge_value(v[q].y, a, v[q + 1].y, b);
-                }
-                merge_weights(m[0], l[0], m[2], l[2], a, b);
-                unsigned long long *out = words(cc, kvh * group + g, j);
-                st_tagged2(out + dim, merge_value(v[0].x, a, v[2].x, b), merge_value(v[0].y, a, v[2].y, b), tag);
-                if (dim == 0) st_tagged2(out + HD, m[0], l[0], tag);
-            }
-        } else {
-            // merge the four position quarters of each query tile: (q0 + q1) and (q2 + q3), then the two halves
-            // (a query tile without a query in use skips the merge: its warps only keep the barriers)
-            if ((qr & 1) && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
-            bar_consumers();
-            if (!(qr & 1) && tile_used) attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
-            bar_consumers();
-            if (qr == 2 && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
-            bar_consumers();
-            if (qr == 0 && tile_used) {
-                attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
-                // ---- chunk partial (unnormalised output, max, sum) of every valid (column, q head)
-#pragma unroll
-                for (int rh = 0; rh < 2; ++rh) {
-                    const int qcol = mt * 16 + (lane >> 2) + 8 * rh, cc = div_group(qcol, group), g = qcol - cc * group;
-                    if (cc < MAX_COLS && ((mk >> cc) & 1u) && d.pos[cc] >= p_base) {
-                        unsigned long long *out = words(cc, kvh * group + g, j);
-#pragma unroll
-                        for (int nt = 0; nt < NT; ++nt) st_tagged2(out + nt * 8 + 2 * (lane & 3), o[nt][2 * rh], o[nt][2 * rh + 1], tag);
-                        if ((lane & 3) == 0) st_tagged2(out + HD, m_run[rh], l_run[rh], tag);
-                    }
-                }
-            }
-        }
-        if (tid == 0) trace(S, EV_ITEM, item);
-        // ---- this CTA's share of the head's outputs: two features of one (column, q head) per thread and pass; the chunk
-        // partials are folded in ascending order, eight at a time with all their loads in flight, by the running-max rule
-        const int units = __popc(mk) * group * (HD / 2), u1 = units * (j + 1) / nchunk;
-        for (int u = units * j / nchunk + tid; u < u1; u += CONS_THREADS) {
-            const int row = u / (HD / 2), dim = (u % (HD / 2)) * 2, nth = div_group(row, group), g = row - nth * group;
-            int cc = 0;   // the nth active column
-#pragma unroll
-            for (int q = 0; q < MAX_COLS; ++q)
-                if (((mk >> q) & 1u) && __popc(mk & ((1u << q) - 1u)) == nth) cc = q;
-            const int h = kvh * group + g, nch = d.pos[cc] / ATT_CHUNK + 1;
-            const unsigned long long *part = words(cc, h, 0);
-            float Mx = -INFINITY, den = 0.f, ax = 0.f, ay = 0.f;
-            for (int k0 = 0; k0 < nch; k0 += 8) {
-                float ml[8], ll[8], ox[8], oy[8];
-                unsigned long long t0 = 0;
-                for (uint32_t it = 0;; ++it) {
-                    bool ok = true;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        ml[q] = -INFINITY; ll[q] = 0.f; ox[q] = 0.f; oy[q] = 0.f;
-                        if (k0 + q < nch) {
-                            const bool a = ld_tagged2(part + (size_t)(k0 + q) * TS + HD, ml[q], ll[q], tag);
-                            const bool b = ld_tagged2(part + (size_t)(k0 + q) * TS + dim, ox[q], oy[q], tag);
-                            ok = ok && a && b;
-                        }
-                    }
-                    if (ok) break;
-                    if ((it & 15u) == 15u || S.wait_ns < SHORT_LIMIT_NS) {   // bounded like every other wait on another CTA
-                        if (aborted(S)) break;
-                        if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; break; }
-                        const unsigned long long t = gtime();
-                        if (t0 == 0) t0 = t;
-                        else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_GRID); break; }
-                    }
-                }
-                float Mn = Mx;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) Mn = fmaxf(Mn, ml[q]);
-                if (Mn == -INFINITY) continue;
-                const float sc = Mx == -INFINITY ? 0.f : __expf(Mx - Mn);
-                den = __fmul_rn(den, sc); ax = __fmul_rn(ax, sc); ay = __fmul_rn(ay, sc);
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (ml[q] != -INFINITY) {
-                        const float w = __expf(ml[q] - Mn);
-                        den = __fmaf_rn(ll[q], w, den);
-                        ax = __fmaf_rn(ox[q], w, ax);
-                        ay = __fmaf_rn(oy[q], w, ay);
-                    }
-                Mx = Mn;
-            }
-            xfrag_store2(A.XO, h * HD + dim, cc, ax / den, ay / den);
-        }
-        if (tid == 0) trace(S, EV_COMBINE, kvh);
-    }
-}
-
-template <int HD>
-__device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, Rings &r) {
-    const Ctx &c = A.c;
-    Smem *sm = S.sm;
-    AttnSmem<HD> *as = reinterpret_cast<AttnSmem<HD> *>(sm->scratch);
-    constexpr int KSQ = HD / 16, NT = HD / 8;
-    constexpr int ATT_STRIDE = HD + 4;                     // floats per chunk partial: output, max, sum, padding (16-byte rows)
-    constexpr int QV = KSQ * 64 / (CONS_THREADS / 2);      // 16-byte pieces of one query tile's fragments per thread of a warp group
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x, G = gridDim.x;
-    const int group = c.group;
-    const int n_items = attn_items(A, d, mask);
-    const int mt = warp >> 2, qr = warp & 3;
-    (void)layer;
-    // Merge of the chunk partials of one kv head into the O-projection's input (by a whole CTA).
-    auto merge_chunks = [&](int kvh, unsigned mk) {   // mk: the active columns of the work item's sequence
-        // Four features of one (column, q head) per thread and pass; the chunk partials are folded in
-        // ascending order, eight at a time with all their loads in flight, by the usual running-max rule.
-        const int nqc = MAX_COLS * group;
-        for (int idx = tid; idx < nqc * (HD / 4); idx += CONS_THREADS) {
-            const int qcol = idx / (HD / 4), dim = (idx - qcol * (HD / 4)) * 4, cc = div_group(qcol, group), g = qcol - cc * group;
-            if (!((mk >> cc) & 1u)) continue;
-            const int h = kvh * group + g;
-            const int nch = d.pos[cc] / ATT_CHUNK + 1;
-            const float *part = A.attn_part + (((size_t)cc * c.nq + h) * c.n_chunks) * ATT_STRIDE;
-            float Mx = -INFINITY, den = 0.f;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int k0 = 0; k0 < nch; k0 += 8) {
-                float2 ml[8];
-                float4 ov[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const bool ok = k0 + u < nch;
-                    const float *pk = part + (size_t)(k0 + u) * ATT_STRIDE;
-                    ml[u] = ok ? __ldcg(reinterpret_cast<const float2 *>(pk + HD)) : make_float2(-INFINITY, 0.f);
-                    ov[u] = ok ? __ldcg(reinterpret_cast<const float4 *>(pk + dim)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                float Mn = Mx;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) Mn = fmaxf(Mn, ml[u].x);
-                if (Mn == -INFINITY) continue;
-                const float sc = Mx == -INFINITY ? 0.f : __expf(Mx - Mn);
-                den = __fmul_rn(den, sc); acc.x = __fmul_rn(acc.x, sc); acc.y = __fmul_rn(acc.y, sc); acc.z = __fmul_rn(acc.z, sc); acc.w = __fmul_rn(acc.w, sc);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (ml[u].x != -INFINITY) {
-                        const float w = __expf(ml[u].x - Mn);
-                        den = __fmaf_rn(ml[u].y, w, den);
-                        acc.x = __fmaf_rn(ov[u].x, w, acc.x); acc.y = __fmaf_rn(ov[u].y, w, acc.y); acc.z = __fmaf_rn(ov[u].z, w, acc.z); acc.w = __fmaf_rn(ov[u].w, w, acc.w);
-                    }
-                }
-                Mx = Mn;
-            }
-            xfrag_store(A.XO, h * HD + dim, cc, acc.x / den);
-            xfrag_store(A.XO, h * HD + dim + 1, cc, acc.y / den);
-            xfrag_store(A.XO, h * HD + dim + 2, cc, acc.z / den);
-            xfrag_store(A.XO, h * HD + dim + 3, cc, acc.w / den);
-        }
-    };
-    // With at most one work item per CTA the CTA that completes a head last merges it at once; with more,
-    // designated CTAs do (see below).  Who merges does not change what is computed.
-    const bool last_arriver_merges = n_items <= G;
-    // Rounds: one item whose two query tiles go to the two warp groups, or (every sequence's queries in one tile) two
-    // items, one per group.  Every warp walks the ring stages of the whole round in order and releases each of them;
-    // it multiplies only those of its own group's item.
-    const bool dual = attn_dual(A, mask);
-    const int per_round = dual ? 2 : 1;
-    for (int it0 = cta; it0 < n_items; it0 += G * per_round) {
-        AttnItem itg[2];
-        itg[0] = attn_item_of(A, d, mask, it0, n_items, dual, 0);
-        itg[1] = attn_item_of(A, d, mask, dual ? it0 + G : it0, n_items, dual, 1);
-        const AttnItem me = itg[mt];
-        const int kvh = me.kvh, j = me.j, p_base = me.p_base, qt = me.qt;
-        const unsigned mk = me.mk;   // the item's sequence: its columns only
-        // ---- query tile qt of the item's kv head, by this warp group: one round trip to L2, then shared memory
-        {
-            const uint4 *src = reinterpret_cast<const uint4 *>(A.qfrag) + (size_t)kvh * (2 * KSQ * 64) + (size_t)qt * (KSQ * 64);
-            const int gt = tid & (CONS_THREADS / 2 - 1);
-            uint4 v[QV];
-#pragma unroll
-            for (int u = 0; u < QV; ++u) v[u] = me.have ? __ldcg(src + gt + u * (CONS_THREADS / 2)) : make_uint4(0u, 0u, 0u, 0u);
-            bar_consumers();   // the previous round is done with the shared buffers
-#pragma unroll
-            for (int u = 0; u < QV; ++u) reinterpret_cast<uint4 *>(&as->qfrag[mt][0][0][0])[gt + u * (CONS_THREADS / 2)] = v[u];
-        }
-        bar_consumers();
-        if (tid == 0) trace(S, EV_ATT, 2);   // queries ready
-        // ---- per-warp online softmax state: rows (lane/4) and (lane/4)+8 of query tile qt
-        int lim[2];
-#pragma unroll
-        for (int rh = 0; rh < 2; ++rh) {
-            const int qcol = qt * 16 + (lane >> 2) + rh * 8, cc = div_group(qcol, group);
-            lim[rh] = (me.have && cc < MAX_COLS && ((mk >> cc) & 1u)) ? d.pos[cc] : -1;
-        }
-        // a query tile none of whose 16 (column, q head) pairs is in use does no arithmetic (uniform per warp)
-        bool tile_used = false;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int cc = div_group(qt * 16 + q, group);
-            tile_used = tile_used || (cc < MAX_COLS && ((mk >> cc) & 1u));
-        }
-        tile_used = tile_used && me.have;
-        float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-        float o[NT][4];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) o[nt][i] = 0.f;
-        const int nsb = max(itg[0].nsb, dual ? itg[1].nsb : 0);
-        for (int sb = 0; sb < nsb; ++sb) {
-            const int p0 = p_base + sb * ATT_PAGE;
-            const bool act = me.have && sb < me.nsb;   // this warp's item has this sub-block
-            float s[2][4];
+        for (int u = 0; u < 2; ++u) {
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) s[nt][i] = -INFINITY;
-#pragma unroll 1
-            for (int g = 0; g < per_round; ++g) {   // ---- K block(s)
-                if (!itg[g].have || sb >= itg[g].nsb) continue;
-                const uint32_t slot = r.xs;
-                mbar_wait(S, &sm->x_full[slot], r.xp);
-                if (tid == 0) trace(S, EV_ATT, 3 + 16 * sb);   // K block landed
-                if (!dual || g == mt) {
-                    const unsigned char *kb = sm->x[slot];
-                    float sh[2][4], sl[2][4];
+                for (int i = 0; i < 4; ++i) s[u][nt][i] = -INFINITY;
+            if (u >= n_sl) continue;
+            w_wait(S, k_stage + sb0 + u, known);
+            float sh[2][4], sl[2][4];
 #pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
+            for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) { sh[nt][i] = 0.f; sl[nt][i] = 0.f; }
-                    const int id = lane >> 3;
-                    const int pl = 16 * qr + (lane & 7) + 8 * (id >> 1);
-                    const unsigned char *krow = kb + pl * (HD * 2);
-                    if (tile_used)
+                for (int i = 0; i < 4; ++i) { sh[nt][i] = 0.f; sl[nt][i] = 0.f; }
+            const int id = lane >> 3, pl = 16 * qr + (lane & 7) + 8 * (id >> 1);
+            const unsigned char *krow = sm->w[(k_stage + sb0 + u) % NW] + pl * (HD * 2);
 #pragma unroll
-                    for (int k0 = 0; k0 < KSQ; k0 += 4) {   // four k-steps of loads in flight, then their multiply-adds
-                        uint4 qh[4], ql[4];
-                        uint32_t kf[4][4];
+            for (int k0 = 0; k0 < KSQ; k0 += 4) {   // four k-steps of loads in flight, then their multiply-adds
+                uint4 qh[4], ql[4];
+                uint32_t kf[4][4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int ks = k0 + u;
-                            qh[u] = *reinterpret_cast<const uint4 *>(&as->qfrag[mt][ks][lane][0]);
-                            ql[u] = *reinterpret_cast<const uint4 *>(&as->qfrag[mt][ks][lane][4]);
-                            ldmatrix_x4(kf[u], krow + ((((2 * ks) | (id & 1)) ^ (pl & 7)) << 4));
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const uint32_t ah[4] = {qh[u].x, qh[u].y, qh[u].z, qh[u].w}, al[4] = {ql[u].x, ql[u].y, ql[u].z, ql[u].w};
-                            mma16816(sh[0], ah, kf[u][0], kf[u][1]);
-                            mma16816(sh[1], ah, kf[u][2], kf[u][3]);
-                            mma16816(sl[0], al, kf[u][0], kf[u][1]);
-                            mma16816(sl[1], al, kf[u][2], kf[u][3]);
-                        }
-                    }
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int pos = p0 + 16 * qr + 8 * nt + 2 * (lane & 3) + (i & 1);
-                            s[nt][i] = pos <= lim[i >> 1] ? sh[nt][i] + sl[nt][i] : -INFINITY;
-                        }
+                for (int q = 0; q < 4; ++q) {
+                    const int ks = k0 + q;
+                    qh[q] = *reinterpret_cast<const uint4 *>(qs + ks * 1024);
+                    ql[q] = *reinterpret_cast<const uint4 *>(qs + ks * 1024 + 16);
+                    ldmatrix_x4(kf[q], krow + ((((2 * ks) | (id & 1)) ^ (pl & 7)) << 4));
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                r.next_x();
-            }
-            // ---- online softmax over this warp's 16 positions
-            uint32_t ph[4] = {0u, 0u, 0u, 0u}, plo[4] = {0u, 0u, 0u, 0u};
-            if (act) {
 #pragma unroll
-                for (int rh = 0; rh < 2; ++rh) {
-                    float mx = fmaxf(fmaxf(s[0][2 * rh], s[0][2 * rh + 1]), fmaxf(s[1][2 * rh], s[1][2 * rh + 1]));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                    const float mn = fmaxf(m_run[rh], mx);
-                    float corr = 1.f, p[4] = {0.f, 0.f, 0.f, 0.f};
-                    if (mn != -INFINITY) {
-                        corr = __expf(m_run[rh] - mn);
-                        p[0] = __expf(s[0][2 * rh] - mn); p[1] = __expf(s[0][2 * rh + 1] - mn);
-                        p[2] = __expf(s[1][2 * rh] - mn); p[3] = __expf(s[1][2 * rh + 1] - mn);
-                    }
-                    m_run[rh] = mn;
-                    l_run[rh] = l_run[rh] * corr + ((p[0] + p[1]) + (p[2] + p[3]));
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) { o[nt][2 * rh] *= corr; o[nt][2 * rh + 1] *= corr; }
-                    // A fragment of P: a0/a1 = n-tile 0 (rows r / r+8), a2/a3 = n-tile 1
-                    const __nv_bfloat162 h0 = __floats2bfloat162_rn(p[0], p[1]), h1 = __floats2bfloat162_rn(p[2], p[3]);
-                    ph[rh] = *reinterpret_cast<const uint32_t *>(&h0);
-                    ph[2 + rh] = *reinterpret_cast<const uint32_t *>(&h1);
-                    plo[rh] = pack_bf16(p[0] - __low2float(h0), p[1] - __high2float(h0));
-                    plo[2 + rh] = pack_bf16(p[2] - __low2float(h1), p[3] - __high2float(h1));
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t ah[4] = {qh[q].x, qh[q].y, qh[q].z, qh[q].w}, al[4] = {ql[q].x, ql[q].y, ql[q].z, ql[q].w};
+                    mma16816(sh[0], ah, kf[q][0], kf[q][1]);
+                    mma16816(sh[1], ah, kf[q][2], kf[q][3]);
+                    mma16816(sl[0], al, kf[q][0], kf[q][1]);
+                    mma16816(sl[1], al, kf[q][2], kf[q][3]);
                 }
             }
-#pragma unroll 1
-            for (int g = 0; g < per_round; ++g) {   // ---- V block(s)
-                if (!itg[g].have || sb >= itg[g].nsb) continue;
-                const uint32_t slot = r.xs;
-                mbar_wait(S, &sm->x_full[slot], r.xp);
-                if (tid == 0) trace(S, EV_ATT, 4 + 16 * sb);   // V block landed
-                if (!dual || g == mt) {
-                    const unsigned char *vb = sm->x[slot];
-                    const int id = lane >> 3;
-                    const int pl = 16 * qr + (lane & 7) + 8 * (id & 1);
-                    const unsigned char *vrow = vb + pl * (HD * 2);
-                    if (tile_used)
+            const int p0 = it.p_base + (sb0 + u) * ATT_PAGE + 16 * qr + 2 * (lane & 3);
 #pragma unroll
-                    for (int n0 = 0; n0 < NT / 2; n0 += 4) {
-                        uint32_t vf[4][4];
+            for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) ldmatrix_x4_trans(vf[u], vrow + ((((2 * (n0 + u)) | (id >> 1)) ^ (pl & 7)) << 4));
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int np = n0 + u;
-                            mma16816(o[2 * np], ph, vf[u][0], vf[u][1]);
-                            mma16816(o[2 * np + 1], ph, vf[u][2], vf[u][3]);
-                            mma16816(o[2 * np], plo, vf[u][0], vf[u][1]);
-                            mma16816(o[2 * np + 1], plo, vf[u][2], vf[u][3]);
-                        }
-                    }
+                for (int i = 0; i < 4; ++i) {
+                    s[u][nt][i] = p0 + 8 * nt + (i & 1) <= lim[i >> 1] ? sh[nt][i] + sl[nt][i] : -INFINITY;
+                    m[i >> 1] = fmaxf(m[i >> 1], s[u][nt][i]);
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sm->x_empty[slot]);
-                r.next_x();
-            }
         }
-        // ---- row sums over the quad, then merge the four position quarters of each warp group:
-        //      (q0 + q1) and (q2 + q3), then the two halves
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
+        r.next_x();
+        // ---- the chunk's row maxima
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {
-            l_run[rh] += __shfl_xor_sync(0xffffffffu, l_run[rh], 1);
-            l_run[rh] += __shfl_xor_sync(0xffffffffu, l_run[rh], 2);
+            m[rh] = fmaxf(m[rh], __shfl_xor_sync(0xffffffffu, m[rh], 1));
+            m[rh] = fmaxf(m[rh], __shfl_xor_sync(0xffffffffu, m[rh], 2));
+            if ((lane & 3) == 0) as->mx[warp][(lane >> 2) + 8 * rh] = m[rh];
         }
-        if (tid == 0) trace(S, EV_ATT, 5);   // sub-blocks done
-        bar_consumers();   // every warp is done with the query fragments, whose space the merge reuses
-        // (a query tile without a query in use skips the merge: its warps only keep the barriers)
-        if ((qr & 1) && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
-        bar_consumers();
-        if (!(qr & 1) && tile_used) attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][qr >> 1], as->ml[mt][qr >> 1], lane);
-        bar_consumers();
-        if (qr == 2 && tile_used) attn_merge_to<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
-        bar_consumers();
-        if (qr == 0) {
-            if (tile_used) attn_merge_from<NT, HD>(o, m_run, l_run, as->o[mt][0], as->ml[mt][0], lane);
-            // ---- chunk partial (unnormalised output, max, sum) of every valid (column, q head)
+        bar_consumers();   // (A) scores done: maxima in place, K blocks free; and everybody has left the item before
+        if (warp == 0 && lane < it.nsb) mbar_arrive(&sm->w_empty[(k_stage + lane) % NW]);
+        float l[2] = {0.f, 0.f};
+        uint32_t ph[2][4], plo[2][4];   // weights of the two slices as A fragments, high and low parts
 #pragma unroll
-            for (int rh = 0; rh < 2; ++rh) {
-                const int qcol = qt * 16 + (lane >> 2) + 8 * rh, cc = div_group(qcol, group), g = qcol - cc * group;
-                if (me.have && cc < MAX_COLS && ((mk >> cc) & 1u) && d.pos[cc] >= p_base) {
-                    float *out = A.attn_part + (((size_t)cc * c.nq + kvh * group + g) * c.n_chunks + j) * ATT_STRIDE;
+        for (int rh = 0; rh < 2; ++rh) {
+            const int row = (lane >> 2) + 8 * rh;
+            float mm = -INFINITY;
+            if (one_tile) {
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt)
-                        *reinterpret_cast<float2 *>(out + nt * 8 + 2 * (lane & 3)) = make_float2(o[nt][2 * rh], o[nt][2 * rh + 1]);
-                    if ((lane & 3) == 0) *reinterpret_cast<float2 *>(out + HD) = make_float2(m_run[rh], l_run[rh]);
+                for (int w = 0; w < CONS_WARPS; ++w) mm = fmaxf(mm, as->mx[w][row]);
+            } else {
+#pragma unroll
+                for (int w = 0; w < 4; ++w) mm = fmaxf(mm, as->mx[4 * mt + w][row]);
+            }
+            m[rh] = mm;
+            float ls[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                float p[4] = {0.f, 0.f, 0.f, 0.f};
+                if (u < n_sl && mm != -INFINITY) {
+                    p[0] = __expf(s[u][0][2 * rh] - mm); p[1] = __expf(s[u][0][2 * rh + 1] - mm);
+                    p[2] = __expf(s[u][1][2 * rh] - mm); p[3] = __expf(s[u][1][2 * rh + 1] - mm);
+                }
+                ls[u] = (p[0] + p[1]) + (p[2] + p[3]);
+                ls[u] += __shfl_xor_sync(0xffffffffu, ls[u], 1);
+                ls[u] += __shfl_xor_sync(0xffffffffu, ls[u], 2);
+                // A fragment of P: a0/a1 = n-tile 0 (rows r / r+8), a2/a3 = n-tile 1
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(p[0], p[1]), h1 = __floats2bfloat162_rn(p[2], p[3]);
+                ph[u][rh] = *reinterpret_cast<const uint32_t *>(&h0);
+                ph[u][2 + rh] = *reinterpret_cast<const uint32_t *>(&h1);
+                plo[u][rh] = pack_bf16(p[0] - __low2float(h0), p[1] - __high2float(h0));
+                plo[u][2 + rh] = pack_bf16(p[2] - __low2float(h1), p[3] - __high2float(h1));
+            }
+            l[rh] = one_tile ? ls[0] : ls[0] + ls[1];
+        }
+        // ---- outputs of this warp's slice(s)
+        float o[NT][4];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o[nt][i] = 0.f;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (u >= n_sl) continue;
+            w_wait(S, v_stage + sb0 + u, known);
+            const int id = lane >> 3, pl = 16 * qr + (lane & 7) + 8 * (id & 1);
+            const unsigned char *vrow = sm->w[(v_stage + sb0 + u) % NW] + pl * (HD * 2);
+#pragma unroll
+            for (int n0 = 0; n0 < NT / 2; n0 += 4) {
+                uint32_t vf[4][4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) ldmatrix_x4_trans(vf[q], vrow + ((((2 * (n0 + q)) | (id >> 1)) ^ (pl & 7)) << 4));
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int np = n0 + q;
+                    float a[2][4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) a[0][i] = a[1][i] = 0.f;
+                    mma16816(a[0], ph[u], vf[q][0], vf[q][1]);
+                    mma16816(a[1], ph[u], vf[q][2], vf[q][3]);
+                    mma16816(a[0], plo[u], vf[q][0], vf[q][1]);
+                    mma16816(a[1], plo[u], vf[q][2], vf[q][3]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { o[2 * np][i] += a[0][i]; o[2 * np + 1][i] += a[1][i]; }
                 }
             }
         }
-        // ---- the round's partials are complete: count its items (a release that returns nothing, so nobody waits for it)
-        if (tid == 0) trace(S, EV_ITEM, it0);
-        bar_consumers();
-        if (last_arriver_merges) {   // at most one item per CTA: the round holds item it0 alone
-            const int cnt = itg[0].k * c.nkv + itg[0].kvh;
-            if (tid == 0) {   // release this block's partials and acquire the others' in one step
-                unsigned old;
-                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(A.attn_cnt + cnt) : "memory");
-                sm->bcast[2] = (int)old;
-            }
-            bar_consumers();
-            if (sm->bcast[2] == itg[0].nchunk - 1) {
-                merge_chunks(itg[0].kvh, itg[0].mk);
-                if (tid == 0) { A.attn_cnt[cnt] = 0u; trace(S, EV_COMBINE, itg[0].kvh); }
-            }
-        } else if (tid == 0 || (dual && tid == CONS_THREADS / 2)) {
-            const AttnItem &mine = itg[tid == 0 ? 0 : 1];
-            if (mine.have) {
-                __threadfence();
-                red_release_add(A.attn_cnt + mine.k * c.nkv + mine.kvh, 1u);
+        if (tid == 0) trace(S, EV_ATT, 5);   // products done
+        // ---- slices added, eight rows of the tile(s) at a time, and published
+        if ((lane & 3) == 0) {
+            as->l[warp][lane >> 2] = l[0];
+            as->l[warp][(lane >> 2) + 8] = l[1];
+            if (warp == (one_tile ? 0 : 4 * mt)) {   // the maximum's word (the next item's maxima may already be on their way when the sums are read)
+#pragma unroll
+                for (int rh = 0; rh < 2; ++rh)
+                    if (lim[rh] >= it.p_base) {
+                        const int row = 16 * mt + (lane >> 2) + 8 * rh, slot = div_group(row, group);
+                        st_tagged(words(slot * nseq + it.k, it.kvh * group + row - slot * group, it.j) + HD, m[rh], tag);
+                    }
             }
         }
-    }
-    if (last_arriver_merges) return;
-    // ---- The chunk partials of kv head h are merged by one designated CTA, G - 1 - h (the high CTAs
-    // have the fewest work items), once all nchunk items of the head have been counted.  (Letting
-    // whichever CTA arrives last do it looks cheaper but piles up at long contexts: the CTA that
-    // merges one head is late for its next item, so it is last again for the next head, and ends up
-    // merging every head in turn while the rest of the grid waits.)
-    for (int hk = G - 1 - cta; hk < A.nseq * c.nkv; hk += G) {   // (sequence of the launch, kv head) pairs of this CTA
-        const int ks_ = hk / c.nkv, kvh = hk - ks_ * c.nkv, nchunk = seq_chunks(A, d, mask, ks_);
-        if (nchunk == 0) continue;
-        if (tid == 0) grid_wait(S, A.attn_cnt + hk, (unsigned)nchunk);
-        bar_consumers();
-        {
-            merge_chunks(kvh, mask & seq_cols(A, ks_));
-            if (tid == 0) { A.attn_cnt[hk] = 0u; trace(S, EV_COMBINE, kvh); }
+        bool freed = false;
+#pragma unroll
+        for (int rh = 0; rh < 2; ++rh) {
+            // a half of the rows without a token (in any tile in use) is skipped, by all warps alike
+            unsigned rows = 0;   // bit t: half rh of tile t holds a token
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int lo = div_group(16 * t + 8 * rh, group), hi = div_group(16 * t + 8 * rh + 7, group);
+                rows |= ((it.slots & ((2u << min(hi, 30)) - (1u << min(lo, 30)))) != 0 ? 1u : 0u) << t;
+            }
+            rows &= it.tiles;
+            if (rows == 0) continue;
+            if (freed) bar_consumers();   // everybody has read the half before
+            {
+                float *dst = as->o[warp][lane >> 2];
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt)
+                    *reinterpret_cast<float2 *>(dst + ((nt * 8 + 2 * (lane & 3) + 8 * (lane >> 2)) & (HD - 1))) = make_float2(o[nt][2 * rh], o[nt][2 * rh + 1]);
+            }
+            bar_consumers();   // (B) outputs in place
+            if (!freed) {      // V blocks free
+                if (warp == 0 && lane < it.nsb) mbar_arrive(&sm->w_empty[(v_stage + lane) % NW]);
+                freed = true;
+            }
+            const int n_el = (one_tile ? 1 : 2) * 8 * (HD / 2);
+#pragma unroll 1
+            for (int e = tid; e < n_el; e += CONS_THREADS) {
+                const int dim = (e & (HD / 2 - 1)) * 2, rr = (e / (HD / 2)) & 7, t = one_tile ? mt : e / (HD / 2) >> 3;
+                const int row = 16 * t + 8 * rh + rr, slot = div_group(row, group);
+                if (slot >= 8 || !((it.slots >> slot) & 1u)) continue;
+                const int col = slot * nseq + it.k;
+                if (d.pos[col] < it.p_base) continue;
+                const int w0 = one_tile ? 0 : 4 * t, at = (dim + 8 * rr) & (HD - 1);
+                float2 q[4];
+                float ql[4];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    q[w] = *reinterpret_cast<const float2 *>(&as->o[w0 + w][rr][at]);
+                    ql[w] = as->l[w0 + w][8 * rh + rr];
+                    if (one_tile) {
+                        const float2 b = *reinterpret_cast<const float2 *>(&as->o[w + 4][rr][at]);
+                        q[w].x += b.x; q[w].y += b.y;
+                        ql[w] += as->l[w + 4][8 * rh + rr];
+                    }
+                }
+                unsigned long long *out = words(col, it.kvh * group + row - slot * group, it.j);
+                st_tagged2(out + dim, (q[0].x + q[1].x) + (q[2].x + q[3].x), (q[0].y + q[1].y) + (q[2].y + q[3].y), tag);
+                if (dim == 0) st_tagged(out + HD + 1, (ql[0] + ql[1]) + (ql[2] + ql[3]), tag);
+            }
         }
-        bar_consumers();   // the next head's wait must not start before every thread is done with this one
+        if (tid == 0) trace(S, EV_ITEM, it.j);
     }
+    // ---- this CTA's share of the merging: two features of one (column, q head) per thread and pass; the chunk
+    // partials are folded in ascending order, eight at a time with all their loads in flight, by the running-max rule
+    const unsigned total = (unsigned)(__popc(mask) * c.nq * (HD / 2));
+    const int u1 = (int)(total * (blockIdx.x + 1) / gridDim.x);
+#pragma unroll 1
+    for (int u = (int)(total * blockIdx.x / gridDim.x) + tid; u < u1; u += CONS_THREADS) {
+        const int row = u / (HD / 2), dim = (u % (HD / 2)) * 2, h = row % c.nq;
+        int nth = row / c.nq, col = 0;   // the nth active column
+        for (unsigned mm = mask; mm; mm &= mm - 1)
+            if (nth-- == 0) { col = __ffs(mm) - 1; break; }
+        const int nch = d.pos[col] / ATT_CHUNK + 1;
+        const unsigned long long *part = words(col, h, 0);
+        float Mx = -INFINITY, den = 0.f, ax = 0.f, ay = 0.f;
+#pragma unroll 1
+        for (int k0 = 0; k0 < nch; k0 += 8) {
+            float ml[8], ll[8], ox[8], oy[8];
+            unsigned long long t0 = 0;
+            for (uint32_t n = 0;; ++n) {
+                bool ok = true;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    ml[q] = -INFINITY; ll[q] = 0.f; ox[q] = 0.f; oy[q] = 0.f;
+                    if (k0 + q < nch) {
+                        const bool a = ld_tagged2(part + (size_t)(k0 + q) * TS + HD, ml[q], ll[q], tag);
+                        const bool b = ld_tagged2(part + (size_t)(k0 + q) * TS + dim, ox[q], oy[q], tag);
+                        ok = ok && a && b;
+                    }
+                }
+                if (ok) break;
+                if ((n & 15u) == 15u || S.wait_ns < SHORT_LIMIT_NS) {   // bounded like every other wait on another CTA
+                    if (aborted(S)) break;
+                    if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; break; }
+                    const unsigned long long t = gtime();
+                    if (t0 == 0) t0 = t;
+                    else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_GRID); break; }
+                }
+                __nanosleep(32);
+            }
+            float Mn = Mx;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) Mn = fmaxf(Mn, ml[q]);
+            if (Mn == -INFINITY) continue;
+            const float sc = Mx == -INFINITY ? 0.f : __expf(Mx - Mn);
+            den *= sc; ax *= sc; ay *= sc;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (ml[q] != -INFINITY) {
+                    const float w = __expf(ml[q] - Mn);
+                    den = __fmaf_rn(ll[q], w, den);
+                    ax = __fmaf_rn(ox[q], w, ax);
+                    ay = __fmaf_rn(oy[q], w, ay);
+                }
+            Mx = Mn;
+        }
+        xfrag_store2(A.XO, h * HD + dim, col, ax / den, ay / den);
+    }
+    if (tid == 0) trace(S, EV_COMBINE, 0);
 }
 
 // ---------------------------------------------------------------- the walker
@@ -1815,7 +1421,7 @@ template <int HD> struct Epilogue {
     bool next_in, final_in;  // down product: prepares the next layer's input, a head's input
 
     static constexpr int HALF = HD / 2, KSQ = HD / 16;
-    __device__ __forceinline__ int seq_of(int col) const { return A.seq0 + (A.nseq == 1 ? 0 : col / A.c.slots); }
+    __device__ __forceinline__ int seq_of(int col) const { return A.seq0 + (A.nseq == 1 ? 0 : col % A.nseq); }
 
     // operands fetched while the weights stream
     __device__ __forceinline__ void pre(int ps, int tile, int row, int col) const {
@@ -1872,12 +1478,13 @@ template <int HD> struct Epilogue {
                 const int dim = ((n0 & (HD - 1)) >> 1) + (row & 7) + (row >> 3) * HALF;   // rows r and r + 8 hold features j and j + hd/2
                 const float y = a0 * co + (row < 8 ? -other : other) * si;
                 if (n0 < qd) {
-                    const int h = n0 / HD, kvh = div_group(h, c.group), qcol = col * c.group + (h - kvh * c.group);
+                    const int h = n0 / HD, kvh = div_group(h, c.group), k = A.nseq == 1 ? 0 : col % A.nseq, slot = A.nseq == 1 ? col : col / A.nseq;
+                    const int qcol = slot * c.group + (h - kvh * c.group);   // row of the sequence's (token, q head) pairs
                     const int qrow = qcol & 15, m = qcol >> 4, ks = dim >> 4, kk = dim & 15;
                     const int ln = (qrow & 7) * 4 + ((kk & 7) >> 1), reg = (qrow >> 3) + 2 * (kk >> 3);
                     const float yq = y * rsqrtf((float)HD);
                     const __nv_bfloat16 hi = __float2bfloat16_rn(yq);
-                    __nv_bfloat16 *f = reinterpret_cast<__nv_bfloat16 *>(A.qfrag) + ((((size_t)kvh * 2 + m) * KSQ + ks) * 32 + ln) * 16 + reg * 2 + (kk & 1);
+                    __nv_bfloat16 *f = reinterpret_cast<__nv_bfloat16 *>(A.qfrag) + (((((size_t)k * c.nkv + kvh) * 2 + m) * KSQ + ks) * 32 + ln) * 16 + reg * 2 + (kk & 1);
                     f[0] = hi;
                     f[8] = __float2bfloat16_rn(yq - __bfloat162float(hi));
                 } else {
@@ -2016,16 +1623,12 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
             const unsigned mask = active_mask(d, final_head ? L - 1 : inter ? l - 1 : l);
             const unsigned cmask = inter ? (unsigned)d.head_mask & mask : mask;
             if (ph == PH_ATTN) {
-                // work items that hold no row of this pass are fetched before the QKV phase has ended
-                const bool single = attn_items(A, d, mask) <= A.one_item_max;
-                if (ROLE == 1) {
-                    if (single) attn_produce_single(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
-                    else attn_produce(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
-                }
+                if (ROLE == 0) attn_produce_kv(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
+                if (ROLE == 1) attn_produce_q(A, S, d, mask, bar_no * (unsigned)G, r, pol);
                 if (ROLE == 2) {
-                    consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
-                    if (single) attn_consume_single<HD>(A, S, d, l, mask, bar_no + 1, r);
-                    else attn_consume<HD>(A, S, d, l, mask, r);
+                    // (a CTA without an item must not report the phase before the one in front of it is complete)
+                    if (AttnWalk(A, d, mask).n <= (int)blockIdx.x) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
+                    attn_consume<HD>(A, S, d, mask, bar_no + 1, r);
                 }
             } else {
                 // ---- a product.  QKV is finished in its epilogue: q rotated, scaled and stored as tensor-core fragments for the

@@ -541,9 +541,9 @@ struct NoHook {
 };
 
 // The 32 k-steps of one weight stage: fragment loads run four steps ahead of the multiply-adds that use them.
-// K-step j accumulates into chain j % 4: acc[j % 4] (high parts) and acc[4 + j % 4] (low parts).  A chain's multiply-adds wait
-// for one another; with two chains a stage was sixteen of them in a row (0.4 us).
-__device__ __forceinline__ void stage_full(float (&acc)[8][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+// Even k-steps accumulate into acc[0] (high parts) and acc[2] (low parts), odd ones into acc[1] and acc[3].  (A stage of one warp
+// is bound by the shared-memory reads of all eight, 200 cycles of the SM for 16 KB, not by the length of these chains.)
+__device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
     constexpr int PF = 4;
     uint32_t a[PF][4];
     uint4 b[PF];
@@ -555,8 +555,8 @@ __device__ __forceinline__ void stage_full(float (&acc)[8][4], const unsigned ch
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
         const int cur = j % PF;
-        mma16816(acc[j & 3], a[cur], b[cur].x, b[cur].y);
-        mma16816(acc[(j & 3) + 4], a[cur], b[cur].z, b[cur].w);
+        mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
+        mma16816(acc[(j & 1) + 2], a[cur], b[cur].z, b[cur].w);
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
             ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
@@ -566,7 +566,7 @@ __device__ __forceinline__ void stage_full(float (&acc)[8][4], const unsigned ch
 }
 // The same for up to four columns: their high parts are token columns 0..3 of one multiply-add, their low parts 4..7.
 // Half the multiply-adds and half the shared-memory reads; every sum has the order it has above.
-__device__ __forceinline__ void stage_packed(float (&acc)[8][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+__device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
     constexpr int PF = 4;
     uint32_t a[PF][4];
     uint2 b[PF];
@@ -578,7 +578,7 @@ __device__ __forceinline__ void stage_packed(float (&acc)[8][4], const unsigned 
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
         const int cur = j % PF;
-        mma16816(acc[j & 3], a[cur], b[cur].x, b[cur].y);
+        mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
             ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
@@ -646,19 +646,19 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             my_cols |= (act ? (unsigned)__ffs(m) - 1u : 15u) << (4 * ps);
             if (act) epi.pre(ps, g.g0 + slot, row, __ffs(m) - 1);
         }
-        float acc0[8][4], acc1[8][4];   // [hi/lo x chain][fragment] of the one or two matrices
+        float acc0[4][4], acc1[4][4];   // [even/odd step x hi/lo][fragment] of the one or two matrices
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc0[q][i] = acc1[q][i] = 0.f;
         // fold the partial accumulators in a fixed order: the chains of the high parts, those of the low parts, both.
         // Four columns or fewer: the result of column pair cp0 + j stands in the lanes with lane % 4 = j, else of pair j.
         float d0[4], d1[4];
-        auto fold = [&](float (&d)[4], float (&acc)[8][4]) {
+        auto fold = [&](float (&d)[4], float (&acc)[4][4]) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float hi = (acc[0][i] + acc[1][i]) + (acc[2][i] + acc[3][i]);
-                d[i] = hi + (packed ? __shfl_xor_sync(0xffffffffu, hi, 2) : (acc[4][i] + acc[5][i]) + (acc[6][i] + acc[7][i]));
+                const float hi = acc[0][i] + acc[1][i];
+                d[i] = hi + (packed ? __shfl_xor_sync(0xffffffffu, hi, 2) : acc[2][i] + acc[3][i]);
             }
         };
 #pragma unroll 1
@@ -709,7 +709,7 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                     st_relaxed_u64(pb + i * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d0[i]));
                     if (pair == 2) st_relaxed_u64(pb + (4 + i) * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d1[i]));
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) acc0[q][i] = acc1[q][i] = 0.f;
+                    for (int q = 0; q < 4; ++q) acc0[q][i] = acc1[q][i] = 0.f;
                 }
             }
         }
