@@ -1102,6 +1102,8 @@ __device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &
 //
 // An item's 128 positions are eight slices of sixteen.  Where its queries fit one tile of sixteen rows (plain decoding, few tokens
 // in flight) each warp takes a slice; where they span two, warp (tile, quarter) takes slices quarter and quarter + 4 of that tile.
+// Where a CTA has several items of one tile each, two groups of four warps work on different ones, a warp on slices quarter and
+// quarter + 4: an item is a chain of latencies (5 us for 1 us of work), and two chains run side by side.
 // Either way a row's numbers are formed alike: the maximum over the chunk first (exchanged through shared memory), weights
 // exp(score - maximum), one product per slice, slices s and s + 4 added, then (0 + 1) + (2 + 3).  So a token's attention does not
 // depend on which other tokens ride along.  (Running maxima per warp over two sub-blocks left half of the warps idle in the
@@ -1112,6 +1114,11 @@ __device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &
 // the launch's (token, q head, feature pair)s each), in one round trip per eight chunks.  Who merges does not change what is computed.
 template <int HD>
 __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S, const StepDesc &d, unsigned mask, unsigned tag, Rings &r) {
+    // consumers' barrier of the warps that share an item
+    auto meet = [](bool dual, int grp) {
+        if (dual) asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+        else bar_consumers();
+    };
     const Ctx &c = A.c;
     Smem *sm = S.sm;
     AttnSmem<HD> *as = reinterpret_cast<AttnSmem<HD> *>(sm->scratch);
@@ -1123,12 +1130,34 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
     uint32_t known = r.w;
     AttnWalk walk(A, d, mask);
     AttnItem it;
+    // Two items at a time: this CTA has more than one, and every sequence's queries fit one tile.  8B shape at 3000 positions (192
+    // items) 16.0 -> 14.8 us a layer, 13B with four sequences (640) 30.7 -> 27.7.  With 64 features a head an item is half the work
+    // and two one after the other are faster (1B, eight sequences, 128 to 192 items: 10.1 against 11.1 us).
+    const int grp = warp >> 2;
+    bool dual = walk.n > (int)(blockIdx.x + (HD == 64 ? 2 : 1) * gridDim.x);
+    for (int k = 0; k < nseq; ++k) {
+        const unsigned sl = seq_slots(A, mask, k);
+        if (sl) dual = dual && ((__ffs(sl) - 1) * group >= 16 || (32 - __clz(sl)) * group <= 16);
+    }
+    int turn = 0;   // group whose item it is
 #pragma unroll 1
     while (walk.next(A, d, mask, it)) {
-        const bool one_tile = it.tiles != 3u;
-        const int mt = one_tile ? (int)(it.tiles >> 1) : warp >> 2, qr = warp & 3;
+        const bool one_tile = it.tiles != 3u, solo = one_tile && !dual;   // solo: eight warps on one tile
+        const int mt = one_tile ? (int)(it.tiles >> 1) : grp, qr = warp & 3;
+        const int w0 = solo ? 0 : 4 * grp;                                // the first of the warps whose slices make up this warp's tile
+        const bool lead = warp == (dual ? 4 * grp : 0);                   // releases the item's K and V blocks
         const uint32_t k_stage = r.w, v_stage = r.w + it.nsb;
         r.w += 2 * it.nsb;
+        if (dual) {
+            const bool other = turn != grp;
+            turn ^= 1;
+            if (other) {   // the other group's item; activation stages are waited for and released by every warp
+                mbar_wait(S, &sm->x_full[r.xs], r.xp);
+                if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
+                r.next_x();
+                continue;
+            }
+        }
         // last position that rows lane / 4 and lane / 4 + 8 of the tile see (-1: no token)
         int lim[2];
 #pragma unroll
@@ -1140,7 +1169,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
         if (tid == 0) trace(S, EV_ATT, 2);   // queries ready
         const unsigned char *qs = sm->x[r.xs] + (one_tile ? 0 : mt) * (HD * 64) + lane * 32;
         float s[2][2][4], m[2] = {-INFINITY, -INFINITY};   // scores [slice][n-tile][fragment], row maxima
-        const int sb0 = one_tile ? warp >> 2 : 0, n_sl = one_tile ? (sb0 < it.nsb ? 1 : 0) : it.nsb;
+        const int sb0 = solo ? grp : 0, n_sl = solo ? (sb0 < it.nsb ? 1 : 0) : it.nsb;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
 #pragma unroll
@@ -1195,20 +1224,19 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
             m[rh] = fmaxf(m[rh], __shfl_xor_sync(0xffffffffu, m[rh], 2));
             if ((lane & 3) == 0) as->mx[warp][(lane >> 2) + 8 * rh] = m[rh];
         }
-        bar_consumers();   // (A) scores done: maxima in place, K blocks free; and everybody has left the item before
-        if (warp == 0 && lane < it.nsb) mbar_arrive(&sm->w_empty[(k_stage + lane) % NW]);
+        meet(dual, grp);   // (A) scores done: maxima in place, K blocks free; and everybody has left the item before
+        if (lead && lane < it.nsb) mbar_arrive(&sm->w_empty[(k_stage + lane) % NW]);
         float l[2] = {0.f, 0.f};
         uint32_t ph[2][4], plo[2][4];   // weights of the two slices as A fragments, high and low parts
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {
             const int row = (lane >> 2) + 8 * rh;
             float mm = -INFINITY;
-            if (one_tile) {
 #pragma unroll
-                for (int w = 0; w < CONS_WARPS; ++w) mm = fmaxf(mm, as->mx[w][row]);
-            } else {
+            for (int w = 0; w < 4; ++w) mm = fmaxf(mm, as->mx[w0 + w][row]);
+            if (solo) {
 #pragma unroll
-                for (int w = 0; w < 4; ++w) mm = fmaxf(mm, as->mx[4 * mt + w][row]);
+                for (int w = 4; w < CONS_WARPS; ++w) mm = fmaxf(mm, as->mx[w][row]);
             }
             m[rh] = mm;
             float ls[2];
@@ -1229,7 +1257,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
                 plo[u][rh] = pack_bf16(p[0] - __low2float(h0), p[1] - __high2float(h0));
                 plo[u][2 + rh] = pack_bf16(p[2] - __low2float(h1), p[3] - __high2float(h1));
             }
-            l[rh] = one_tile ? ls[0] : ls[0] + ls[1];
+            l[rh] = solo ? ls[0] : ls[0] + ls[1];
         }
         // ---- outputs of this warp's slice(s)
         float o[NT][4];
@@ -1268,7 +1296,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
         if ((lane & 3) == 0) {
             as->l[warp][lane >> 2] = l[0];
             as->l[warp][(lane >> 2) + 8] = l[1];
-            if (warp == (one_tile ? 0 : 4 * mt)) {   // the maximum's word (the next item's maxima may already be on their way when the sums are read)
+            if (warp == w0) {   // the maximum's word (the next item's maxima may already be on their way when the sums are read)
 #pragma unroll
                 for (int rh = 0; rh < 2; ++rh)
                     if (lim[rh] >= it.p_base) {
@@ -1289,34 +1317,34 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
             }
             rows &= it.tiles;
             if (rows == 0) continue;
-            if (freed) bar_consumers();   // everybody has read the half before
+            if (freed) meet(dual, grp);   // everybody has read the half before
             {
                 float *dst = as->o[warp][lane >> 2];
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt)
                     *reinterpret_cast<float2 *>(dst + ((nt * 8 + 2 * (lane & 3) + 8 * (lane >> 2)) & (HD - 1))) = make_float2(o[nt][2 * rh], o[nt][2 * rh + 1]);
             }
-            bar_consumers();   // (B) outputs in place
+            meet(dual, grp);   // (B) outputs in place
             if (!freed) {      // V blocks free
-                if (warp == 0 && lane < it.nsb) mbar_arrive(&sm->w_empty[(v_stage + lane) % NW]);
+                if (lead && lane < it.nsb) mbar_arrive(&sm->w_empty[(v_stage + lane) % NW]);
                 freed = true;
             }
             const int n_el = (one_tile ? 1 : 2) * 8 * (HD / 2);
 #pragma unroll 1
-            for (int e = tid; e < n_el; e += CONS_THREADS) {
+            for (int e = dual ? tid & 127 : tid; e < n_el; e += dual ? 128 : CONS_THREADS) {
                 const int dim = (e & (HD / 2 - 1)) * 2, rr = (e / (HD / 2)) & 7, t = one_tile ? mt : e / (HD / 2) >> 3;
                 const int row = 16 * t + 8 * rh + rr, slot = div_group(row, group);
                 if (slot >= 8 || !((it.slots >> slot) & 1u)) continue;
                 const int col = slot * nseq + it.k;
                 if (d.pos[col] < it.p_base) continue;
-                const int w0 = one_tile ? 0 : 4 * t, at = (dim + 8 * rr) & (HD - 1);
+                const int wq = solo ? 0 : dual ? w0 : 4 * t, at = (dim + 8 * rr) & (HD - 1);
                 float2 q[4];
                 float ql[4];
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
-                    q[w] = *reinterpret_cast<const float2 *>(&as->o[w0 + w][rr][at]);
-                    ql[w] = as->l[w0 + w][8 * rh + rr];
-                    if (one_tile) {
+                    q[w] = *reinterpret_cast<const float2 *>(&as->o[wq + w][rr][at]);
+                    ql[w] = as->l[wq + w][8 * rh + rr];
+                    if (solo) {
                         const float2 b = *reinterpret_cast<const float2 *>(&as->o[w + 4][rr][at]);
                         q[w].x += b.x; q[w].y += b.y;
                         ql[w] += as->l[w + 4][8 * rh + rr];
