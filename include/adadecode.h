@@ -76,7 +76,8 @@ typedef struct {
     double decode_ms;        /* device time of the decode calls (CUDA events on the session stream) */
     int64_t emitted[ADA_MAX_BATCH]; /* tokens returned per sequence (fewer than asked for only after an end-of-sequence token) */
     int64_t finished;        /* sequences that ended on a verified end-of-sequence token during these calls */
-    int64_t path;            /* decode path of the last call: 1 = persistent kernel, 0 = one kernel per operation */
+    int64_t path;            /* decode path of the last call: 1 = persistent kernel (bf16), 0 = the others: small fp32 models in one
+                              * launch per call, else one kernel per operation */
 } ada_stats;
 
 const char *ada_strerror(int code);
@@ -212,9 +213,11 @@ int ada_debug_profile_read(ada_session *s, double *ms_out, int64_t *launches_out
  * Algorithm 1; bf16 models, at most 8 tokens per pass, 64-token KV pages, head_dim 64
  * or 128, at most 4 q heads per kv head, d_model / n_q_heads*head_dim / d_ff multiples of 64); it is
  * the default wherever a session qualifies; a session that qualifies but cannot be set up fails in
- * ada_session_create instead of taking the other path).  0 = one kernel per operation on CUDA cores
- * (any dtype, any batch; sequences of a batch share every layer pass).  On path 1 the sequences of a batch share
- * a launch, and its weight stream, as far as eight token columns go (max_early + 1 each).  ADA_EUNSUPPORTED if path 1 is asked of a
+ * ada_session_create instead of taking the other path).  0 = CUDA cores
+ * (any dtype, any batch; sequences of a batch share every layer pass): one kernel per operation, or, for fp32 sessions of at
+ * most 16 rows a sequence whose rows fit the shared memory, one launch per call.  On path 1 the sequences of a batch share
+ * a launch, and its weight stream, as far as its token columns go (max_early + 1 each; eight, or 24 where eight would take
+ * three launches or more, or hold one sequence only).  ADA_EUNSUPPORTED if path 1 is asked of a
  * session that does not qualify.
  * ada_stats.path reports the path a decode call ran on. */
 int ada_debug_set_path(ada_session *s, int32_t path);

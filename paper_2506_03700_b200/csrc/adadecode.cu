@@ -14,6 +14,14 @@
 #include "mega.cuh"
 #include "resident.cuh"
 #include "dense.cuh"
+// the persistent kernel once more, for 24 token columns
+#undef ADA_TILES
+#undef ADA_ST
+#undef ADA_MG
+#define ADA_TILES 3
+#define ADA_ST st3
+#define ADA_MG mg3
+#include "mega.cuh"
 
 using namespace ada;
 
@@ -139,7 +147,7 @@ struct ada_session {
     // persistent-kernel path (bf16, one sequence, up to eight token columns)
     bool mega = false;
     int grid = 0;
-    mg::MegaArgs margs;
+    MegaArgs margs;
     CUtensorMap *maps_dev = nullptr;      // [6 L + 2]: wqkv, wo, wgu, wup, wdown per layer, lm_head, then T per 1-based layer
     bool sampling = false;   // the call in progress draws its tokens (ada_sampling_decode)
     float inv_temp = 1.0f;
@@ -204,7 +212,7 @@ constexpr int kPartMaxGrid = 256;
 // Chunk partials of the decode attention: as floats for the per-operation kernels, as tagged words (see attn_consume) for the
 // persistent kernel, in the same memory (a session uses one path at a time, and the words are cleared before each launch).
 size_t attn_tag_bytes(const ada_config &g, int n_chunks) {
-    return model_fits_persistent(g) ? sizeof(unsigned long long) * st::MAX_COLS * g.n_q_heads * (size_t)n_chunks * (g.head_dim + 2) : 0;
+    return model_fits_persistent(g) ? sizeof(unsigned long long) * st3::MAX_COLS * g.n_q_heads * (size_t)n_chunks * (g.head_dim + 2) : 0;
 }
 
 // Whether an fp32 model's calls can run in one launch (resident.cuh): most rows of its passes, or 0.  The bounds are those of the
@@ -267,25 +275,26 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
     // persistent-kernel buffers (bf16 models)
     if (g.dtype == ADA_DTYPE_BF16) {
         L.maps = take(sizeof(CUtensorMap) * (6 * (size_t)g.n_layers + 2));
-        L.xa = take(st::xfrag_bytes(g.d_model));
-        L.xb = take(st::xfrag_bytes(g.d_model));
-        L.xf = take(st::xfrag_bytes(g.d_model));
-        L.xt = take(st::xfrag_bytes(g.d_model));
-        L.xo = take(st::xfrag_bytes(qd));
-        L.xh = take(st::xfrag_bytes(g.d_ff));
-        L.ssq_a = take(sizeof(float) * (size_t)((g.d_model + 15) / 16) * st::MAX_COLS);
-        L.ssq_b = take(sizeof(float) * (size_t)((g.d_model + 15) / 16) * st::MAX_COLS);
-        L.qfrag = take((size_t)st::MAX_COLS * g.n_kv_heads * 2 * (g.head_dim / 16) * 1024);   // two tiles per (sequence of a launch, kv head)
+        // products' inputs, for the kernel of eight token columns and behind them for the one of 24 (their padding stays zero)
+        L.xa = take(st::xfrag_bytes(g.d_model) + st3::xfrag_bytes(g.d_model));
+        L.xb = take(st::xfrag_bytes(g.d_model) + st3::xfrag_bytes(g.d_model));
+        L.xf = take(st::xfrag_bytes(g.d_model) + st3::xfrag_bytes(g.d_model));
+        L.xt = take(st::xfrag_bytes(g.d_model) + st3::xfrag_bytes(g.d_model));
+        L.xo = take(st::xfrag_bytes(qd) + st3::xfrag_bytes(qd));
+        L.xh = take(st::xfrag_bytes(g.d_ff) + st3::xfrag_bytes(g.d_ff));
+        L.ssq_a = take(sizeof(float) * (size_t)((g.d_model + 15) / 16) * st3::MAX_COLS);
+        L.ssq_b = take(sizeof(float) * (size_t)((g.d_model + 15) / 16) * st3::MAX_COLS);
+        L.qfrag = take((size_t)st::MAX_SEQS * g.n_kv_heads * 2 * (g.head_dim / 16) * 1024);   // two tiles per (sequence of a launch, kv head)
         L.rope_freq = take(sizeof(double) * (g.head_dim / 2));
-        L.part = take(kPartBytesPerCta * kPartMaxGrid);
+        L.part = take(st3::TILES * kPartBytesPerCta * kPartMaxGrid);
         L.grid_ctr = take(256);
-        L.pub = take(sizeof(mg::Pub) * 2);
+        L.pub = take(sizeof(mg3::Pub) * 2);
         L.err = take(256);
         // sampled decoding: the logits and normalisers of the intermediate head that drew each token in flight, and the
         // random numbers of every sequence position
-        L.q_stage = take(sizeof(float) * (size_t)batch * st::MAX_COLS * g.vocab);
-        L.qinfo = take(sizeof(float4) * (size_t)batch * st::MAX_COLS);
-        L.uniforms = take(sizeof(float) * (size_t)batch * max_seq * mg::SAMPLE_NU);
+        L.q_stage = take(sizeof(float) * (size_t)batch * DRAFT_SLOTS * g.vocab);
+        L.qinfo = take(sizeof(float4) * (size_t)batch * DRAFT_SLOTS);
+        L.uniforms = take(sizeof(float) * (size_t)batch * max_seq * SAMPLE_NU);
     }
     L.total = o;
     return L;
@@ -754,8 +763,10 @@ void add_stats(ada_session *S, const DevStats &d, ada_stats *out, float ms, int6
 
 // ---- persistent-kernel path --------------------------------------------------------------------
 
-template <int HD> const void *persistent_kernel() { return (const void *)mg::k_decode_persistent<HD>; }
-const void *persistent_kernel_for(int hd) { return hd == 64 ? persistent_kernel<64>() : persistent_kernel<128>(); }
+const void *persistent_kernel_for(int hd, bool wide) {
+    if (wide) return hd == 64 ? (const void *)mg3::k_decode_persistent<64> : (const void *)mg3::k_decode_persistent<128>;
+    return hd == 64 ? (const void *)mg::k_decode_persistent<64> : (const void *)mg::k_decode_persistent<128>;
+}
 
 // Whether a model's shape and dtype are ones the persistent kernel is built for (the session adds its
 // own conditions: at most eight token columns per sequence, 64-token pages).
@@ -778,35 +789,38 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     S->mega = false;
     S->path = 0;
     const int qd = g.n_q_heads * g.head_dim;
-    if (!model_fits_persistent(g) || S->slots > st::MAX_COLS || S->page_tokens != mg::ATT_PAGE) return ADA_OK;
+    if (!model_fits_persistent(g) || S->slots > st::MAX_COLS || S->page_tokens != ATT_PAGE) return ADA_OK;
     int dev = 0, sms = 0, coop = 0, nb = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-    const void *kern = persistent_kernel_for(g.head_dim);
     if (!coop || sms < 1) {
         g_cuda_err = "the device does not support cooperative launches, which the persistent decode kernel needs";
         return ADA_EUNSUPPORTED;
     }
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES));
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, mg::MEGA_THREADS, st::SMEM_BYTES));
-    cudaFuncAttributes fa;
-    CK(cudaFuncGetAttributes(&fa, kern));
-    if (nb < 1 || fa.numRegs * mg::MEGA_THREADS < mg::MEGA_REGS) {   // (a warp group waits for registers that the block was not launched with)
-        g_cuda_err = "the persistent decode kernel does not fit on one multiprocessor of this device";
-        return ADA_EUNSUPPORTED;
+    for (const bool wide : {false, true}) {
+        const void *kern = persistent_kernel_for(g.head_dim, wide);
+        const size_t smem = wide ? st3::SMEM_BYTES : st::SMEM_BYTES;
+        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, mg::MEGA_THREADS, smem));
+        cudaFuncAttributes fa;
+        CK(cudaFuncGetAttributes(&fa, kern));
+        if (nb < 1 || fa.numRegs * mg::MEGA_THREADS < mg::MEGA_REGS) {   // (a warp group waits for registers that the block was not launched with)
+            g_cuda_err = "the persistent decode kernel does not fit on one multiprocessor of this device";
+            return ADA_EUNSUPPORTED;
+        }
     }
     S->grid = std::min(sms, S->head_blocks);
     const int L = g.n_layers;
     char *b = (char *)S->scratch;
     S->maps_dev = (CUtensorMap *)(b + lay.maps);
-    S->maps_host.assign((mg::MAPS_PER_LAYER + 1) * (size_t)L + 2, CUtensorMap());
-    mg::MegaModel &M = S->margs.m;
+    S->maps_host.assign((MAPS_PER_LAYER + 1) * (size_t)L + 2, CUtensorMap());
+    MegaModel &M = S->margs.m;
     memset(&M, 0, sizeof(M));
     int rc;
     for (int l = 0; l < L; ++l) {
         const LayerW &w = m->layers[l];
-        CUtensorMap *wm = &S->maps_host[mg::MAPS_PER_LAYER * (size_t)l];
+        CUtensorMap *wm = &S->maps_host[MAPS_PER_LAYER * (size_t)l];
         const bool gu_fused = (const __nv_bfloat16 *)w.w_up == (const __nv_bfloat16 *)w.w_gate + (size_t)g.d_ff * g.d_model;
         if (!w.wqkv_perm) return ADA_ESTATE;
         if ((rc = make_weight_map(wm + 0, w.wqkv_perm, S->c.qkv_rows, g.d_model))) return rc;
@@ -818,7 +832,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
         M.attn_norm[l] = (const __nv_bfloat16 *)w.attn_norm;
         M.ffn_norm[l] = (const __nv_bfloat16 *)w.ffn_norm;
     }
-    if ((rc = make_weight_map(&S->maps_host[mg::MAPS_PER_LAYER * (size_t)L], m->lm_head, g.vocab, g.d_model))) return rc;
+    if ((rc = make_weight_map(&S->maps_host[MAPS_PER_LAYER * (size_t)L], m->lm_head, g.vocab, g.d_model))) return rc;
     M.maps = S->maps_dev;
     M.tok_embed = (const __nv_bfloat16 *)m->tok_embed;
     M.final_norm = (const __nv_bfloat16 *)m->final_norm;
@@ -827,7 +841,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     for (int i = 0; i < g.head_dim / 2; ++i) freq[i] = pow((double)g.rope_base, -2.0 * i / g.head_dim);
     CK(cudaMemcpyAsync(b + lay.rope_freq, freq.data(), sizeof(double) * freq.size(), cudaMemcpyHostToDevice, S->stream));
     CK(cudaStreamSynchronize(S->stream));
-    mg::MegaArgs &a = S->margs;
+    MegaArgs &a = S->margs;
     a.c = S->c;
     a.XA = (__nv_bfloat16 *)(b + lay.xa); a.XB = (__nv_bfloat16 *)(b + lay.xb); a.XO = (__nv_bfloat16 *)(b + lay.xo);
     a.XH = (__nv_bfloat16 *)(b + lay.xh); a.XF = (__nv_bfloat16 *)(b + lay.xf); a.XT = (__nv_bfloat16 *)(b + lay.xt);
@@ -838,7 +852,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     a.rope_freq = (const double *)(b + lay.rope_freq);
     a.part = S->grid <= kPartMaxGrid ? (unsigned long long *)(b + lay.part) : nullptr;
     a.grid_ctr = (unsigned *)(b + lay.grid_ctr);
-    a.pub = (mg::Pub *)(b + lay.pub);
+    a.pub = b + lay.pub;
     a.err = (int *)(b + lay.err);
     a.step_budget = S->steps_per_launch;
     a.seq0 = 0;
@@ -850,7 +864,7 @@ int setup_persistent(ada_session *S, const Layout &lay) {
     a.uniforms = (const float *)(b + lay.uniforms);
     a.q_stage = (float *)(b + lay.q_stage);
     a.qinfo = (float4 *)(b + lay.qinfo);
-    a.trace = st::Trace{nullptr, nullptr, 0};
+    a.trace = Trace{nullptr, nullptr, 0};
     a.trace_step0 = a.trace_step1 = 0;
     S->mega = true;
     S->path = 1;
@@ -964,15 +978,18 @@ int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layer
 }
 
 // Run the persistent kernel until the call's token targets are met.
-// The kernel holds eight token columns.  A sequence needs max_early + 1 of them, so a launch decodes
-// min(8 / (max_early + 1), batch) sequences together (one weight stream for all of them, lock-step: every step runs
-// up to the highest layer any of them reaches); the sequences seq_begin .. seq_end - 1 go in such groups, one group
-// after another.  `together` false: one sequence per launch (prompt passes, which use all eight columns).
+// The kernel holds eight token columns, or 24.  A sequence needs max_early + 1 of them, so a launch decodes as many sequences
+// together (one weight stream for all of them, lock-step: every step runs up to the highest layer any of them reaches); the
+// sequences seq_begin .. seq_end - 1 go in such groups, one group after another.  `together` false: one sequence per launch (prompt
+// passes, which use all eight columns).
+//
+// Which kernel: 24 columns where eight hold one sequence only (max_early > 3) and there are two or more, or where eight would take
+// three launches or more.
 int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool plain, int seq_begin, int seq_end, bool together) {
     const ada_model *m = S->m;
     const ada_config &g = m->cfg;
     const int L = g.n_layers;
-    mg::MegaModel &M = S->margs.m;
+    MegaModel &M = S->margs.m;
     memset(M.exit_at, 0, sizeof(M.exit_at));
     if (!plain) {
         for (int i = 0; i < n_exit; ++i) {
@@ -981,7 +998,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             M.head_scale[e] = m->head_scale[e];
             M.has_T[e] = m->head_T[e] != nullptr;
             if (m->head_T[e]) {
-                const size_t at = mg::MAPS_PER_LAYER * (size_t)L + 1 + e;
+                const size_t at = MAPS_PER_LAYER * (size_t)L + 1 + e;
                 CUtensorMap &tm = S->maps_host[at];
                 int rc = make_weight_map(&tm, m->head_T[e], g.d_model, g.d_model);
                 if (rc) return rc;
@@ -991,11 +1008,21 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
     }
     // a call that ended on a device-side error has left the error word set
     CK(cudaMemsetAsync(S->margs.err, 0, sizeof(int), S->stream));
-    const void *kern = persistent_kernel_for(g.head_dim);
-    const int per_launch = together ? std::max(1, st::MAX_COLS / S->slots) : 1;
+    const int narrow = std::max(1, st::MAX_COLS / S->slots), n_seq = seq_end - seq_begin;
+    const bool wide = together && (narrow == 1 ? n_seq > 1 : (n_seq + narrow - 1) / narrow > 2);
+    const int per_launch = !together ? 1 : wide ? std::min((int)st3::MAX_SEQS, st3::MAX_COLS / S->slots) : narrow;
+    const void *kern = persistent_kernel_for(g.head_dim, wide);
+    const size_t part_bytes = kPartBytesPerCta * (size_t)S->grid * (wide ? st3::TILES : 1);
+    const size_t tag_bytes = attn_tag_bytes(g, S->n_chunks) / st3::MAX_COLS * (wide ? st3::MAX_COLS : st::MAX_COLS);
     for (int sq = seq_begin; sq < seq_end; sq += per_launch) {
-        mg::MegaArgs a = S->margs;
+        MegaArgs a = S->margs;
         a.c = S->c;   // capture pointers may have changed
+        if (wide) {
+            const auto behind = [](__nv_bfloat16 *&p, int K) { p = (__nv_bfloat16 *)((char *)p + st::xfrag_bytes(K)); };
+            for (__nv_bfloat16 **p : {&a.XA, &a.XB, &a.XF, &a.XT}) behind(*p, g.d_model);
+            behind(a.XO, g.n_q_heads * g.head_dim);
+            behind(a.XH, g.d_ff);
+        }
         a.seq0 = sq;
         a.nseq = std::min(per_launch, seq_end - sq);
         a.step_budget = S->steps_per_launch;
@@ -1007,11 +1034,11 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
         for (long long guard = 0;; ++guard) {
             if (guard > (1ll << 24)) return ADA_ETIMEOUT;
             CK(cudaMemsetAsync(a.grid_ctr, 0, sizeof(unsigned), S->stream));
-            CK(cudaMemsetAsync(a.pub, 0, sizeof(mg::Pub) * 2, S->stream));
-            if (a.part) CK(cudaMemsetAsync(a.part, 0, kPartBytesPerCta * (size_t)S->grid, S->stream));
-            CK(cudaMemsetAsync(a.attn_tag, 0, attn_tag_bytes(g, S->n_chunks), S->stream));   // phase numbers start over with every launch
+            CK(cudaMemsetAsync(a.pub, 0, sizeof(mg3::Pub) * 2, S->stream));
+            if (a.part) CK(cudaMemsetAsync(a.part, 0, part_bytes, S->stream));
+            CK(cudaMemsetAsync(a.attn_tag, 0, tag_bytes, S->stream));   // phase numbers start over with every launch
             void *params[] = {(void *)&a};
-            CK(cudaLaunchCooperativeKernel(kern, dim3(S->grid), dim3(mg::MEGA_THREADS), params, st::SMEM_BYTES, S->stream));
+            CK(cudaLaunchCooperativeKernel(kern, dim3(S->grid), dim3(mg::MEGA_THREADS), params, wide ? st3::SMEM_BYTES : st::SMEM_BYTES, S->stream));
             S->launches++;
             CK(cudaMemcpyAsync(S->pinned, &S->c.st->n_climbing, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, S->stream));
             CK(cudaMemcpyAsync(S->pinned + 2, a.err, sizeof(int32_t), cudaMemcpyDeviceToHost, S->stream));
@@ -1019,7 +1046,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             S->syncs++;
             if (S->pinned[2] != 0) {
                 g_cuda_err = "persistent decode kernel: device-side error " + std::to_string(S->pinned[2]);
-                return S->pinned[2] == mg::ERR_BAD_STATE ? ADA_ESTATE : ADA_ETIMEOUT;
+                return S->pinned[2] == ERR_BAD_STATE ? ADA_ESTATE : ADA_ETIMEOUT;
             }
             if (S->pinned[1] >= 1) break;   // the sequences of this launch have reached their targets
         }
@@ -1596,7 +1623,7 @@ int ada_sampling_decode(ada_session *S, int32_t n_tokens, float temperature, flo
                         int32_t n_pos, int32_t *out_host, ada_stats *stats) {
     if (!S || n_exit_layers < 0 || (n_exit_layers > 0 && !exit_layers) || !uniforms_host) return ADA_EINVAL;
     if (!(temperature > 0.0f) || first_pos < 0 || n_pos < 1 || first_pos + (int64_t)n_pos > S->max_seq) return ADA_EINVAL;
-    if (n_exit_layers > mg::SAMPLE_NU - 3) return ADA_ECAPACITY;
+    if (n_exit_layers > SAMPLE_NU - 3) return ADA_ECAPACITY;
     if (!(S->mega && S->path == 1) || S->m->cfg.vocab > mg::DRAW_MAX_VOCAB) return ADA_EUNSUPPORTED;
     // every position the call may draw, test or resample must have its random numbers
     for (int s = 0; s < S->batch; ++s) {
@@ -1606,8 +1633,8 @@ int ada_sampling_decode(ada_session *S, int32_t n_tokens, float temperature, flo
     }
     float *dev = const_cast<float *>(S->margs.uniforms);
     for (int s = 0; s < S->batch; ++s)
-        CK(cudaMemcpyAsync(dev + ((size_t)s * S->max_seq + first_pos) * mg::SAMPLE_NU, uniforms_host + (size_t)s * n_pos * mg::SAMPLE_NU,
-                           sizeof(float) * (size_t)n_pos * mg::SAMPLE_NU, cudaMemcpyHostToDevice, S->stream));
+        CK(cudaMemcpyAsync(dev + ((size_t)s * S->max_seq + first_pos) * SAMPLE_NU, uniforms_host + (size_t)s * n_pos * SAMPLE_NU,
+                           sizeof(float) * (size_t)n_pos * SAMPLE_NU, cudaMemcpyHostToDevice, S->stream));
     S->sampling = true;
     S->inv_temp = 1.0f / temperature;
     const int rc = decode(S, n_tokens, threshold, exit_layers, n_exit_layers, max_early, eos_id, out_host, stats);
@@ -1741,7 +1768,7 @@ int ada_debug_set_launch_steps(ada_session *S, int32_t steps) {
 int ada_debug_trace(ada_session *S, uint64_t *dev_buf, uint32_t *count_dev, uint32_t cap_events, int32_t step0, int32_t step1) {
     if (!S || !S->mega) return ADA_EUNSUPPORTED;
     if (dev_buf && (!count_dev || cap_events < 1 || step0 < 0 || step1 < step0)) return ADA_EINVAL;
-    S->margs.trace = st::Trace{(unsigned long long *)dev_buf, count_dev, dev_buf ? cap_events : 0};
+    S->margs.trace = Trace{(unsigned long long *)dev_buf, count_dev, dev_buf ? cap_events : 0};
     S->margs.trace_step0 = dev_buf ? step0 : 0;
     S->margs.trace_step1 = dev_buf ? step1 : 0;
     return ADA_OK;
@@ -1753,7 +1780,8 @@ int ada_debug_gemm_plan(int32_t N, int32_t K, int32_t mode, int32_t grid, int32_
     st::Gemm g;
     g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0; g.split = split != 0;
     const st::Plan p = st::make_plan(g, cta, grid);
-    const int32_t v[9] = {p.split, p.t0, p.t1, p.n, p.ta, p.tb, p.s0_own_k0, p.s0_pub_k1, p.sl_k1};
+    const int tb = p.t0 + p.n - (p.s0_pub_k1 > 0 ? 0 : 1);
+    const int32_t v[9] = {p.split, p.split ? 0 : p.t0, p.split ? 0 : p.t0 + p.n, p.split ? p.n : 0, p.split ? p.t0 : 0, p.split ? tb : 0, p.s0_own_k0, p.s0_pub_k1, p.sl_k1};
     memcpy(out9, v, sizeof(v));
     return ADA_OK;
 }

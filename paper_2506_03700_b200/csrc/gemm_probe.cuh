@@ -32,7 +32,7 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
     st::Smem *sm = st::smem_base(smem_raw);
     st::smem_init(sm);
     __syncthreads();
-    st::Shared S{sm, err, st::Trace{nullptr, nullptr, 0}, 0, st::WAIT_NS_DEFAULT};
+    st::Shared S{sm, err, Trace{nullptr, nullptr, 0}, 0, st::WAIT_NS_DEFAULT};
     const int warp = threadIdx.x >> 5;
     const int cta = blockIdx.x, G = gridDim.x;
     st::Gemm g;
@@ -44,7 +44,7 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
     st::Rings r;
     if (warp == st::CONS_WARPS) {
         const uint64_t pol = st::policy_evict_first();
-        for (int it = 0; it < repeat; ++it) st::gemm_produce_w(S, pl, W, nullptr, r, pol);
+        for (int it = 0; it < repeat; ++it) st::gemm_produce_w(S, pl, W, nullptr, g.half, r, pol);
     } else if (warp == st::CONS_WARPS + 1) {
         const uint64_t pol = st::policy_evict_last();
         for (int it = 0; it < repeat; ++it) st::gemm_produce_x(S, pl, X, cols_used, r, pol, st::NoHook(), st::NoHook());

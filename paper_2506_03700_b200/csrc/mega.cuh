@@ -17,21 +17,20 @@
 // normalisation partial sums and its layer-(e+1) GEMM input where its last pass left them.
 // Each column's numbers depend only on that column's own inputs (never on which other columns
 // ride along), which is what makes the adaptive output bit-identical to plain greedy decoding.
-#pragma once
-
 #include "kernels.cuh"
-#include "stream.cuh"
+#include "stream.cuh"   // (compiled once per number of column tiles, like this file: see there)
 
 namespace ada {
-namespace mg {
+namespace ADA_MG {
 
-using namespace st;
+using namespace ADA_ST;
 
 constexpr int ACT_CONTINUE = 1, ACT_NEWSTEP = 2, ACT_STOP = 3;
 constexpr int CTRL_START = 0, CTRL_HEAD = 1, CTRL_TOP = 2;
-constexpr int ATT_PAGE = 64;          // cache positions per attention sub-block (= KV page size on this path)
 constexpr int ATT_CHUNK = kAttnChunk; // positions per attention work item (fixed: anchored at position 0)
-constexpr int ERR_BAD_STATE = 3;
+
+constexpr int NO_LAYER = 255;   // above every layer index (ADA_MAX_LAYERS - 1 layers at most)
+static_assert(ADA_MAX_LAYERS <= 256, "layer indexes are kept in a byte");
 
 struct StepDesc {
     int n_cols;                // columns with a token (in flight + newest, over all sequences of the launch)
@@ -40,11 +39,11 @@ struct StepDesc {
     int pmax;                  // highest position of the step
     int fresh;                 // columns whose token enters at layer 1 in this step (their embedding is set up by the control point)
     int run_final;             // the step ends with the final head (0: a prompt pass that is not the last)
-    int first_layer[MAX_COLS]; // 0-based layer at which the column resumes (INT_MAX: no token, or its sequence has left the step)
+    unsigned char first_layer[MAX_COLS];   // 0-based layer at which the column resumes (NO_LAYER: no token, or its sequence has left the step)
     int pos[MAX_COLS];
-    int seq_pmax[MAX_COLS];    // per sequence of the launch: position of its newest token (-1: the sequence is not in this step)
+    int seq_pmax[MAX_SEQS];    // per sequence of the launch: position of its newest token (-1: the sequence is not in this step)
 };
-static_assert(sizeof(StepDesc) <= 32 * sizeof(int), "the step descriptor must fit its shared-memory slot");
+static_assert(sizeof(StepDesc) <= sizeof(Smem::desc[0]), "the step descriptor must fit its shared-memory slot");
 
 struct Pub {                   // what CTA 0 publishes at a control point
     unsigned seq;
@@ -52,51 +51,6 @@ struct Pub {                   // what CTA 0 publishes at a control point
     StepDesc d;
     int cap_keep, cap_at, cap_row0;   // logit capture (test hook): rows to copy, where to, first row of the staging buffer
     int pad[5];
-};
-
-// What the phases need to know of the model.  It travels as a kernel argument: the constant bank answers at once, where a
-// pointer read from global memory was a round trip to L2 in front of the loads that depend on it (the L1 copy does not
-// survive the acquire of a grid barrier).
-struct MegaModel {
-    // per layer: wqkv (the fused q | k | v matrix with the rows of every q and k head reordered for the rotation, see the QKV
-    // phase), wo, wgu (gate stacked over up, or gate alone where gu_two is set), wup, wdown; then the LM head; then T per 1-based layer
-    const CUtensorMap *maps;
-    const __nv_bfloat16 *tok_embed, *final_norm;
-    const __nv_bfloat16 *attn_norm[ADA_MAX_LAYERS], *ffn_norm[ADA_MAX_LAYERS];
-    float head_scale[ADA_MAX_LAYERS + 1];        // by 1-based layer
-    unsigned char exit_at[ADA_MAX_LAYERS + 1];   // 1 + the index of 1-based layer e among the call's exit layers if the call consults its head, else 0
-    unsigned char has_T[ADA_MAX_LAYERS + 1];     // that head has a transformation of its own
-    unsigned char gu_two[ADA_MAX_LAYERS];        // gate and up are separate tensors
-};
-enum { MAPS_PER_LAYER = 5 };
-
-struct MegaArgs {
-    Ctx c;
-    MegaModel m;
-    __nv_bfloat16 *XA, *XB, *XO, *XH, *XF, *XT;   // GEMM inputs in fragment layout (see stream.cuh)
-    float *ssq_a, *ssq_b;      // [d/16][8] partial sums of squares of the residual (per 16-feature tile, per column)
-    uint32_t *qfrag;           // [sequence][nkv][2][hd/16][32][8]: rotated, scaled queries as tensor-core A fragments (bf16 high parts, then low parts)
-    float *head_part;          // [grid][8][4]
-    const double *rope_freq;   // [hd/2]: base^(-2i/hd), computed once on the host
-    unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
-    unsigned long long *attn_tag;   // [8][nq][n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume); zeroed before each launch
-    unsigned *grid_ctr;
-    Pub *pub;                  // [2]
-    int *err;
-    int step_budget;           // steps this launch may start
-    int seq0, nseq;            // the launch decodes sequences seq0 .. seq0 + nseq - 1 of the session together, nseq slots <= 8 (slots = max_early + 1):
-                               // slot j of sequence k of them is token column j nseq + k (neighbouring columns are then of equal age, and a
-                               // pass that carries the newest tokens only fetches few column pairs); they share every weight stream
-    unsigned long long wait_ns;   // a single device-side wait gives up after this long
-    int store_logits;
-    // Sampled decoding (Eq. 1 with a drawn token, Eq. 2 with its acceptance test and the resampling): off = greedy
-    int sampling;
-    float inv_temp;            // 1 / temperature: every head's logits are multiplied by it
-    const float *uniforms;     // [batch][max_seq][SAMPLE_NU]: the random numbers of the token at each sequence position
-    float *q_stage;            // [batch][8][vocab]: logits of the intermediate head that drew the token after position p, slot p % 8
-    float4 *qinfo;             // [batch][8]: (max logit, sum of exp, probability of the drawn token) of that head
-    Trace trace;               // test hook: event trace of the steps [trace_step0, trace_step1) of this launch
-    int trace_step0, trace_step1;
 };
 
 // ---------------------------------------------------------------- small helpers
@@ -116,21 +70,25 @@ __device__ __forceinline__ unsigned active_mask(const StepDesc &d, int layer) {
 // l/8 + 4u in ascending order (32 loads in flight), the four lanes of a column are folded by a
 // butterfly.  The order is fixed, so the factor of a column does not depend on the other columns.
 __device__ __forceinline__ void rstd_produce(Smem *sm, const float *ssq, int ntiles, int d, float eps, unsigned seq) {
-    const int lane = threadIdx.x & 31, col = lane & 7, sub = lane >> 3;
-    float s = 0.f;
-    for (int t0 = 0; t0 < ntiles; t0 += 128) {
-        float v[32];
+    const int lane = threadIdx.x & 31, sub = lane >> 3;
+#pragma unroll 1
+    for (int ct = 0; ct < TILES; ++ct) {
+        const int col = 8 * ct + (lane & 7);
+        float s = 0.f;
+        for (int t0 = 0; t0 < ntiles; t0 += 128) {
+            float v[32];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-            const int t = t0 + sub + 4 * u;
-            v[u] = t < ntiles ? ldcg(ssq + (size_t)t * MAX_COLS + col) : 0.f;
+            for (int u = 0; u < 32; ++u) {
+                const int t = t0 + sub + 4 * u;
+                v[u] = t < ntiles ? ldcg(ssq + (size_t)t * MAX_COLS + col) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 32; ++u) s += v[u];
         }
-#pragma unroll
-        for (int u = 0; u < 32; ++u) s += v[u];
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (lane < 8) sm->vec[col] = 1.0f / sqrtf(s / (float)d + eps);
     }
-    s += __shfl_xor_sync(0xffffffffu, s, 8);
-    s += __shfl_xor_sync(0xffffffffu, s, 16);
-    if (lane < MAX_COLS) sm->vec[lane] = 1.0f / sqrtf(s / (float)d + eps);
     __threadfence_block();
     __syncwarp();
     if (lane == 0) *(volatile unsigned *)&sm->vec_seq = seq;
@@ -188,9 +146,6 @@ __device__ __forceinline__ HeadResult merge_head(const float *head_part, int G, 
 
 // ---------------------------------------------------------------- sampling (CTA 0, consumer warps)
 
-// Random numbers per sequence position: [0] draw at the last layer, [1] acceptance test of Eq. 2, [2] resampling after a
-// rejection, [3 + e] draw at the e-th exit layer of the call.
-constexpr int SAMPLE_NU = 8;
 constexpr int DRAW_CHUNK = 128;                 // vocabulary entries per partial sum
 constexpr int DRAW_OFFSET = 12288;              // the draw's buffers sit in the consumers' scratch behind the control point's copies
 constexpr int DRAW_MAX_CHUNKS = (SCRATCH_BYTES - DRAW_OFFSET - 4 * (CONS_THREADS + DRAW_CHUNK + 8)) / 4;
@@ -509,7 +464,7 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
     if (after_head) {
         for (int col = 0; col < MAX_COLS; ++col) {
             if (!((head_cols >> col) & 1u)) continue;
-            const int s = a.seq0 + (a.nseq == 1 ? 0 : col % a.nseq), pos = dprev->pos[col], slot = s * MAX_COLS + (pos & 7);
+            const int s = a.seq0 + (a.nseq == 1 ? 0 : col % a.nseq), pos = dprev->pos[col], slot = s * DRAFT_SLOTS + (pos & 7);
             float total, wt;
             const int tok = block_draw_head(sm, a.q_stage + (size_t)slot * V, hr_s[col].zmax, a.head_part, col, a.G, V, unif(s, pos + 1, 3 + a.exit_idx), total, wt);
             if (tid == 0) {
@@ -525,7 +480,7 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
             if (nrow < 1 || nrow > cps || dprev->first_layer[(nrow - 1) * a.nseq + k] > a.L - 1) continue;
             bool rejected = false;
             for (int r = 0; r + 1 < nrow && !rejected; ++r) {
-                const int col = r * a.nseq + k, pos_t = bs + r + 1, t = min(max(tok_s[col], 0), V - 1), slot = s * MAX_COLS + ((bs + r) & 7);
+                const int col = r * a.nseq + k, pos_t = bs + r + 1, t = min(max(tok_s[col], 0), V - 1), slot = s * DRAFT_SLOTS + ((bs + r) & 7);
                 const float *zs = a.logit_stage + (size_t)col * V;
                 const float4 qi = a.qinfo[slot];
                 const float ps = __expf(__ldcg(zs + t) - hr_s[col].zmax) / hr_s[col].sumexp;
@@ -567,14 +522,14 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     const MegaModel &M = A.m;
     const int tid = threadIdx.x, G = gridDim.x;
     const int nseq = A.nseq, seq0 = A.seq0, cps = c.slots, L = c.L;   // cps: token columns per sequence
-    Pub *pub = A.pub + (pub_no & 1);
+    Pub *pub = reinterpret_cast<Pub *>(A.pub) + (pub_no & 1);
     // Shared-memory copies for the bookkeeping thread (fetched by many threads at once: a single
     // thread reading them from global memory one after the other spent 30 us here on round trips to L2):
     // the fill levels, the head results, and the tokens the verification compares with.
     int *fill_s = reinterpret_cast<int *>(sm->scratch);                                          // [nseq][L]
     HeadResult *hr_s = reinterpret_cast<HeadResult *>(sm->scratch + 8192);                       // [MAX_COLS]
     int *tok_s = reinterpret_cast<int *>(sm->scratch + 8192 + sizeof(HeadResult) * MAX_COLS);    // [MAX_COLS]: the token after the column's own
-    static_assert(ADA_MAX_LAYERS * MAX_COLS * sizeof(int) <= 8192, "fill levels of a launch's sequences must fit the scratch corner");
+    static_assert(ADA_MAX_LAYERS * MAX_SEQS * sizeof(int) <= 8192, "fill levels of a launch's sequences must fit the scratch corner");
     for (int i = tid; i < nseq * L; i += CONS_THREADS) fill_s[i] = c.fill[(size_t)seq0 * L + i];
     if (tid >= CONS_THREADS - MAX_COLS) {
         const int j = tid - (CONS_THREADS - MAX_COLS), k = j % nseq;
@@ -589,11 +544,12 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     const unsigned head_cols = kind == CTRL_HEAD ? ((unsigned)dprev.head_mask & active_mask(dprev, e - 1))
                                                  : (kind == CTRL_TOP ? active_mask(dprev, L - 1) : 0u);
     if (kind != CTRL_START) {
-        const int w = tid >> 5;
-        if ((head_cols >> w) & 1u) {
-            const HeadResult hr = merge_head(A.head_part, G, w);
-            if ((tid & 31) == 0) { c.head_res[w] = hr; hr_s[w] = hr; }
-        }
+#pragma unroll 1
+        for (int w = tid >> 5; w < MAX_COLS; w += CONS_WARPS)
+            if ((head_cols >> w) & 1u) {
+                const HeadResult hr = merge_head(A.head_part, G, w);
+                if ((tid & 31) == 0) { c.head_res[w] = hr; hr_s[w] = hr; }
+            }
     }
     __threadfence_block();
     bar_consumers();
@@ -614,9 +570,9 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         const float gamma0 = st->gamma;
         const int eos0 = st->eos_id;
         const long long steps0 = __ldcg(&st->st.steps);   // past the L1: the counters are bumped by reductions
-        int len[MAX_COLS], base[MAX_COLS], target[MAX_COLS], done[MAX_COLS];
+        int len[MAX_SEQS], base[MAX_SEQS], target[MAX_SEQS], done[MAX_SEQS];
 #pragma unroll
-        for (int k = 0; k < MAX_COLS; ++k) {
+        for (int k = 0; k < MAX_SEQS; ++k) {
             const bool in = k < nseq;
             len[k] = in ? st->len[seq0 + k] : 0; base[k] = in ? st->base[seq0 + k] : 0;
             target[k] = in ? st->target_len[seq0 + k] : 0; done[k] = in ? st->done[seq0 + k] : 1;
@@ -662,7 +618,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                 bump(&st->st.steps, 1);
                 ++n_steps_seen;
                 for (int j = k; j < MAX_COLS; j += nseq) {   // the sequence sits out the rest of the step
-                    nd.first_layer[j] = INT_MAX;
+                    nd.first_layer[j] = NO_LAYER;
                     nd.head_mask &= ~(1 << j);
                 }
             }
@@ -760,7 +716,8 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         if (action == ACT_NEWSTEP) {
             ++steps_started;
             nd.n_cols = 0; nd.newest_mask = 0; nd.head_mask = 0; nd.pmax = 0; nd.fresh = 0; nd.run_final = 1;
-            for (int j = 0; j < MAX_COLS; ++j) { nd.first_layer[j] = INT_MAX; nd.pos[j] = 0; nd.seq_pmax[j] = -1; }
+            for (int j = 0; j < MAX_COLS; ++j) { nd.first_layer[j] = NO_LAYER; nd.pos[j] = 0; }
+            for (int k = 0; k < MAX_SEQS; ++k) nd.seq_pmax[k] = -1;
             if (pf_end > 0) {   // next pass over the prompt: up to eight positions, all from layer 1
                 const int n = min(MAX_COLS, pf_end - pf_pos);
                 nd.n_cols = n;
@@ -787,7 +744,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                         const int pos = base[k] + j;
                         int fl = 0;
                         for (int l = 0; l < L; ++l) fl += fill_s[k * L + l] > pos;
-                        nd.first_layer[j * nseq + k] = fl;
+                        nd.first_layer[j * nseq + k] = (unsigned char)fl;
                         nd.pos[j * nseq + k] = pos;
                     }
                     const int cn = (nrow - 1) * nseq + k;
@@ -874,7 +831,7 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
                                              int &steps_started) {
     Smem *sm = S.sm;
     ++pub_no;
-    const Pub *pub = A.pub + (pub_no & 1);
+    const Pub *pub = reinterpret_cast<Pub *>(A.pub) + (pub_no & 1);
     int action;
     // the new step descriptor is copied into the role's shared copy `d` by one thread (by every lane of a
     // producer warp: same values), and checked before anything is indexed with it
@@ -887,7 +844,9 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
             for (int i = 0; i < (int)(sizeof(StepDesc) / 4); ++i) dst[i] = src[i];
             bool bad = d.n_cols < 1 || d.n_cols > MAX_COLS || d.pmax < 0 || d.pmax >= A.c.max_seq;
 #pragma unroll
-            for (int i = 0; i < MAX_COLS; ++i) bad = bad || d.pos[i] < 0 || d.pos[i] >= A.c.max_seq || d.seq_pmax[i] >= A.c.max_seq;
+            for (int i = 0; i < MAX_COLS; ++i) bad = bad || d.pos[i] < 0 || d.pos[i] >= A.c.max_seq;
+#pragma unroll
+            for (int i = 0; i < MAX_SEQS; ++i) bad = bad || d.seq_pmax[i] >= A.c.max_seq;
             if (bad) act = ACT_STOP;   // cannot happen unless memory was corrupted; never index with it
         }
         // The two record slots alternate.  A role that fell two control points behind would find its slot
@@ -1451,58 +1410,84 @@ template <int HD> struct Epilogue {
     static constexpr int HALF = HD / 2, KSQ = HD / 16;
     __device__ __forceinline__ int seq_of(int col) const { return A.seq0 + (A.nseq == 1 ? 0 : col % A.nseq); }
 
-    // operands fetched while the weights stream
-    __device__ __forceinline__ void pre(int ps, int tile, int row, int col) const {
+    // Operands fetched while the weights stream: three words per element.
+    //   QKV: rotary factors (cos, sin), cache page; O, down: residual, gain of the next product's input, gain of a head's input
+    __device__ __forceinline__ const void *operand(int w, int tile, int row, int col) const {   // (null: not needed)
         const Ctx &c = A.c;
         const int n0 = tile * 16, n = n0 + row;
+        if (ph == PH_QKV) {
+            if (w == 2) return n0 >= c.nq * HD ? c.page_table + (size_t)seq_of(col) * c.max_pages + (d.pos[col] >> c.page_shift) : nullptr;
+            return n0 < (c.nq + c.nkv) * HD ? c.rope_cs + ((size_t)col * HALF + ((n0 & (HD - 1)) >> 1) + (row & 7)) * 2 + w : nullptr;
+        }
+        if (ph != PH_O && ph != PH_DOWN) return nullptr;
+        if (w == 0) return c.resid + (size_t)col * c.d + n;
+        if (w == 1) return next_in ? (ph == PH_O ? A.m.ffn_norm[l] : A.m.attn_norm[l + 1]) + (n & ~1) : nullptr;
+        return final_in ? A.m.final_norm + (n & ~1) : nullptr;
+    }
+    __device__ __forceinline__ void pre(int ps, int tile, int row, int col) const {
         uint32_t *stash = stash_of(S.sm, ps);
-        if (ph == PH_QKV) {   // rotary factors, cache page
-            const int qd = c.nq * HD, kvd = c.nkv * HD;
-            if (n0 < qd + kvd) {
-                const float *cs = c.rope_cs + ((size_t)col * HALF + ((n0 & (HD - 1)) >> 1) + (row & 7)) * 2;
-                cp_async4(stash, cs);
-                cp_async4(stash + CONS_THREADS, cs + 1);
-            }
-            if (n0 >= qd) cp_async4(stash + 2 * CONS_THREADS, c.page_table + (size_t)seq_of(col) * c.max_pages + (d.pos[col] >> c.page_shift));
-        } else if (ph == PH_O || ph == PH_DOWN) {   // residual and gains
-            cp_async4(stash, c.resid + (size_t)col * c.d + n);
-            if (next_in) cp_async4(stash + CONS_THREADS, (ph == PH_O ? A.m.ffn_norm[l] : A.m.attn_norm[l + 1]) + (n & ~1));
-            if (final_in) cp_async4(stash + 2 * CONS_THREADS, A.m.final_norm + (n & ~1));
+#pragma unroll
+        for (int w = 0; w < 3; ++w) {
+            const void *p = operand(w, tile, row, col);
+            if (p) cp_async4(stash + w * CONS_THREADS, p);
         }
     }
     __device__ __forceinline__ void operator()(int ps, bool act, int tile, int row, int col, float a0, float a1) const {
         const Ctx &c = A.c;
         const int n0 = tile * 16, n = n0 + row;
-        uint32_t *stash = stash_of(S.sm, ps);
         float rs = 1.f;
         if (scaled) { vec_wait(S, vseq); rs = S.sm->vec[col]; }
+        uint32_t ops[3] = {0u, 0u, 0u};
+        if (ph == PH_QKV || ph == PH_O || ph == PH_DOWN) {
+            if (TILES == 1 || ps < STASH_PASSES) {
+                cp_async_wait_all();
+                const uint32_t *stash = stash_of(S.sm, ps);
+#pragma unroll
+                for (int w = 0; w < 3; ++w) ops[w] = stash[w * CONS_THREADS];
+            } else if (act) {
+#pragma unroll
+                for (int w = 0; w < 3; ++w) {
+                    const uint32_t *p = static_cast<const uint32_t *>(operand(w, tile, row, col));
+                    if (p) ops[w] = __ldcg(p);
+                }
+            }
+        }
         a0 *= rs;
         if (ph == PH_GU) {
             a1 *= rs;
             if (act) xfrag_store(A.XH, n, col, a0 / (1.0f + expf(-a0)) * a1);
         } else if (ph == PH_HEAD) {
-            // running (max, sum exp, argmax) of this thread's rows, kept in its stash words; sampled decoding: logits over
-            // the temperature, which are kept, the final head's by column, an intermediate head's by the position of its row
-            // (the verification of the token drawn from them needs them again)
+            // Sampled decoding: logits over the temperature, which are kept, the final head's by column, an intermediate head's by
+            // the position of its row (the verification of the token drawn from them needs them again).
+            // (max, sum exp, argmax) of the tile's sixteen rows by a butterfly, then into the half-warp's running one of this pass.
+            Msa run;
+            run.m = -INFINITY; run.s = 0.f; run.i = INT_MAX;
             if (act && n < c.vocab) {
                 const float z = a0 * scale;
-                if (A.sampling && inter) A.q_stage[((size_t)seq_of(col) * MAX_COLS + (d.pos[col] & 7)) * c.vocab + n] = z;
+                if (A.sampling && inter) A.q_stage[((size_t)seq_of(col) * DRAFT_SLOTS + (d.pos[col] & 7)) * c.vocab + n] = z;
                 else if (A.sampling || A.store_logits) c.logit_stage[(size_t)col * c.vocab + n] = z;
-                Msa run, one;
-                run.m = __uint_as_float(stash[0]); run.s = __uint_as_float(stash[CONS_THREADS]); run.i = (int)stash[2 * CONS_THREADS];
-                one.m = z; one.s = 1.f; one.i = n;
-                run = msa_merge(run, one);
-                stash[0] = __float_as_uint(run.m); stash[CONS_THREADS] = __float_as_uint(run.s); stash[2 * CONS_THREADS] = (uint32_t)run.i;
+                run.m = z; run.s = 1.f; run.i = n;
+            }
+#pragma unroll
+            for (int off = 1; off < 16; off <<= 1) {
+                Msa o;
+                o.m = __shfl_xor_sync(0xffffffffu, run.m, off);
+                o.s = __shfl_xor_sync(0xffffffffu, run.s, off);
+                o.i = __shfl_xor_sync(0xffffffffu, run.i, off);
+                run = msa_merge(run, o);
+            }
+            if (row == 0 && act) {
+                Msa *mine = head_state() + 16 * ps + (threadIdx.x >> 4);
+                *mine = msa_merge(*mine, run);
             }
         } else if (ph == PH_T) {
             if (act) xfrag_store(A.XT, n, col, a0);
         } else if (ph == PH_QKV) {
-            cp_async_wait_all();
             const float other = __shfl_xor_sync(0xffffffffu, a0, 8);   // the partner of a rotation
             const int qd = c.nq * HD, kvd = c.nkv * HD;
             if (!act || n0 >= c.qkv_rows) return;
             if (n0 < qd + kvd) {
-                const float co = __uint_as_float(stash[0]), si = __uint_as_float(stash[CONS_THREADS]);
+                const float co = __uint_as_float(ops[0]), si = __uint_as_float(ops[1]);
                 const int dim = ((n0 & (HD - 1)) >> 1) + (row & 7) + (row >> 3) * HALF;   // rows r and r + 8 hold features j and j + hd/2
                 const float y = a0 * co + (row < 8 ? -other : other) * si;
                 if (n0 < qd) {
@@ -1516,15 +1501,14 @@ template <int HD> struct Epilogue {
                     f[0] = hi;
                     f[8] = __float2bfloat16_rn(yq - __bfloat162float(hi));
                 } else {
-                    cache_row(stash[2 * CONS_THREADS], 0, (n0 - qd) / HD, d.pos[col], dim, y);
+                    cache_row(ops[2], 0, (n0 - qd) / HD, d.pos[col], dim, y);
                 }
             } else {
                 const int nv = n - qd - kvd;
-                cache_row(stash[2 * CONS_THREADS], 1, nv / HD, d.pos[col], nv & (HD - 1), a0);
+                cache_row(ops[2], 1, nv / HD, d.pos[col], nv & (HD - 1), a0);
             }
         } else {   // O and down: residual add, inputs of the products that follow, partial sums of squares
-            cp_async_wait_all();
-            const float v = act ? __uint_as_float(stash[0]) + a0 : 0.f;
+            const float v = act ? __uint_as_float(ops[0]) + a0 : 0.f;
             float sq = v * v;
             sq += __shfl_xor_sync(0xffffffffu, sq, 8);
             sq += __shfl_xor_sync(0xffffffffu, sq, 1);
@@ -1532,8 +1516,8 @@ template <int HD> struct Epilogue {
             sq += __shfl_xor_sync(0xffffffffu, sq, 4);
             if (!act) return;
             c.resid[(size_t)col * c.d + n] = v;
-            if (next_in) xfrag_store(ph == PH_O ? A.XB : A.XA, n, col, v * bf16_of_word(stash[CONS_THREADS], n));
-            if (final_in) xfrag_store(A.XF, n, col, v * bf16_of_word(stash[2 * CONS_THREADS], n));
+            if (next_in) xfrag_store(ph == PH_O ? A.XB : A.XA, n, col, v * bf16_of_word(ops[1], n));
+            if (final_in) xfrag_store(A.XF, n, col, v * bf16_of_word(ops[2], n));
             if (row == 0) (ph == PH_O ? A.ssq_b : A.ssq_a)[(size_t)tile * MAX_COLS + col] = sq;
         }
     }
@@ -1542,46 +1526,22 @@ template <int HD> struct Epilogue {
         const size_t blk = ((((size_t)page * c.L + l) * 2 + which) * c.nkv + kvh) * ((size_t)ATT_PAGE * HD) + (size_t)(pos & (ATT_PAGE - 1)) * HD;
         reinterpret_cast<__nv_bfloat16 *>(c.kv_pool)[blk + ((((dim >> 3) ^ (pos & 7)) << 3) | (dim & 7))] = __float2bfloat16_rn(v);
     }
-    __device__ __forceinline__ void head_begin() const {
-#pragma unroll 1
-        for (int ps = 0; ps < STASH_PASSES; ++ps) {
-            uint32_t *stash = stash_of(S.sm, ps);
-            stash[0] = __float_as_uint(-INFINITY); stash[CONS_THREADS] = 0u; stash[2 * CONS_THREADS] = (uint32_t)INT_MAX;
-        }
+    // running (max, sum exp, argmax) of every half-warp and pass: (tile slot, column) u of gemm_consume is half-warp u % 16 of pass u / 16
+    __device__ __forceinline__ Msa *head_state() const { return reinterpret_cast<Msa *>(S.sm->scratch + RED_BYTES); }
+    __device__ __forceinline__ void head_begin() const {   // (each by the thread that uses it)
+        if ((threadIdx.x & 15) == 0)
+            for (int ps = 0; ps < MAX_COLS / 2; ++ps) {
+                Msa &m = head_state()[16 * ps + (threadIdx.x >> 4)];
+                m.m = -INFINITY; m.s = 0.f; m.i = INT_MAX;
+            }
     }
-    // The CTA's (max, sum exp, argmax) of every column in use: the rows of a half-warp by a butterfly, then the column's
-    // half-warps (tile slots, see gemm_consume) in ascending order.
+    // the CTA's (max, sum exp, argmax) of every column in use: the column's half-warps (tile slots) in ascending order
     __device__ __forceinline__ void head_end(const Plan &pl, unsigned mask) const {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        float *wp = reinterpret_cast<float *>(S.sm->scratch);   // [half-warp of all passes][4]
-        bar_consumers();
-#pragma unroll 1
-        for (int ps = 0; ps < STASH_PASSES; ++ps) {
-            const uint32_t *stash = stash_of(S.sm, ps);
-            Msa run;
-            run.m = __uint_as_float(stash[0]); run.s = __uint_as_float(stash[CONS_THREADS]); run.i = (int)stash[2 * CONS_THREADS];
-#pragma unroll
-            for (int off = 1; off < 16; off <<= 1) {
-                Msa o;
-                o.m = __shfl_xor_sync(0xffffffffu, run.m, off);
-                o.s = __shfl_xor_sync(0xffffffffu, run.s, off);
-                o.i = __shfl_xor_sync(0xffffffffu, run.i, off);
-                run = msa_merge(run, o);
-            }
-            if ((lane & 15) == 0) {
-                float *o = wp + (16 * ps + 2 * warp + (lane >> 4)) * 4;
-                o[0] = run.m; o[1] = run.s; o[2] = __int_as_float(run.i);
-            }
-        }
         bar_consumers();
         if (threadIdx.x < MAX_COLS && ((mask >> threadIdx.x) & 1u)) {
             const int sh = element_shift(Groups(pl).left), ci = __popc(mask & ((1u << threadIdx.x) - 1u));
             Msa a; a.m = -INFINITY; a.s = 0.f; a.i = INT_MAX;
-            for (int w = 0; w < 1 << sh; ++w) {
-                const float *o = wp + ((ci << sh) + w) * 4;
-                Msa x; x.m = o[0]; x.s = o[1]; x.i = __float_as_int(o[2]);
-                a = msa_merge(a, x);
-            }
+            for (int w = 0; w < 1 << sh; ++w) a = msa_merge(a, head_state()[(ci << sh) + w]);
             float *o = A.head_part + ((size_t)blockIdx.x * MAX_COLS + threadIdx.x) * 4;
             o[0] = a.m; o[1] = a.s; o[2] = __int_as_float(a.i);
         }
@@ -1611,7 +1571,9 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
     if (ROLE != 2 || threadIdx.x == 0) {
         d.n_cols = 0; d.newest_mask = 0; d.head_mask = 0; d.pmax = 0; d.fresh = 0; d.run_final = 1;
 #pragma unroll
-        for (int i = 0; i < MAX_COLS; ++i) { d.first_layer[i] = INT_MAX; d.pos[i] = 0; d.seq_pmax[i] = -1; }
+        for (int i = 0; i < MAX_COLS; ++i) { d.first_layer[i] = NO_LAYER; d.pos[i] = 0; }
+#pragma unroll
+        for (int i = 0; i < MAX_SEQS; ++i) d.seq_pmax[i] = -1;
     }
     if (ROLE == 2) bar_consumers(); else __syncwarp();
 
@@ -1673,7 +1635,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 if (ROLE == 0) {
                     const CUtensorMap *W = M.maps + (ph == PH_HEAD ? MAPS_PER_LAYER * L : ph == PH_T ? MAPS_PER_LAYER * L + 1 + l
                                                      : MAPS_PER_LAYER * l + (ph == PH_QKV ? 0 : ph == PH_O ? 1 : ph == PH_GU ? 2 : 4));
-                    gemm_produce_w(S, pl, W, ph == PH_GU && M.gu_two[l] ? W + 1 : nullptr, r, pol);
+                    gemm_produce_w(S, pl, W, ph == PH_GU && M.gu_two[l] ? W + 1 : nullptr, c.dff, r, pol);
                 }
                 if (ROLE == 1) {
                     const __nv_bfloat16 *X = ph == PH_QKV ? A.XA : ph == PH_O ? A.XO : ph == PH_GU ? A.XB : ph == PH_DOWN ? A.XH : ph == PH_HEAD && with_T ? A.XT : A.XF;
@@ -1723,6 +1685,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
     }
 }
 
+#if ADA_TILES == 1
 // Repack on load.  Destination row `prow` of the fused q | k | v matrix: v rows are copied as they are; inside
 // every q and k head the rows are reordered so that the 16-row tile t of the head holds the features
 // [8 t, 8 t + 8) in its rows 0..7 and [hd/2 + 8 t, hd/2 + 8 t + 8) in its rows 8..15.  The two partners
@@ -1760,6 +1723,8 @@ __global__ void k_prefill_arm(Ctx c, int seq, int n_prompt) {
     for (int l = 0; l < c.L; ++l) c.fill[(size_t)seq * c.L + l] = 0;
 }
 
+#endif
+
 // Warps 0-7 consume, warp 8 produces weights, warp 9 activations and K / V blocks; warps 10 and 11 only complete the producers'
 // warp group, which hands registers to the consumers.  (At 168 registers a thread -- three warps on a quarter of the SM --
 // the consumers kept loop variables in local memory, whose L1 lines do not survive the acquires of the grid barrier.)
@@ -1790,5 +1755,5 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
     settle_on_abort(S);
 }
 
-}  // namespace mg
+}  // namespace ADA_MG
 }  // namespace ada

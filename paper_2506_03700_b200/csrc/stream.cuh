@@ -16,15 +16,31 @@
 //     the multiply-adds; the bound stays the memory system.
 //   * all CTAs of the persistent grid meet at a counter-based grid barrier between phases.
 // Every wait is bounded: on expiry an error word is set and all later waits fall through.
-#pragma once
+//
+// This file and mega.cuh are compiled once per number of token columns: ADA_TILES column tiles of eight, in the namespaces
+// ADA_ST and ADA_MG.  One tile (st, mg) is the kernel for up to eight columns; three (st3, mg3) carry several sequences with
+// several tokens each over one weight stream.  A column's numbers are formed alike in both.
+#ifndef ADA_TILES
+#define ADA_TILES 1
+#define ADA_ST st
+#define ADA_MG mg
+#endif
+#if (ADA_TILES == 1 && !defined(ADA_STREAM_1)) || (ADA_TILES == 3 && !defined(ADA_STREAM_3))
+#if ADA_TILES == 1
+#define ADA_STREAM_1
+#else
+#define ADA_STREAM_3
+#endif
 
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "decode_args.cuh"
+
 namespace ada {
-namespace st {
+namespace ADA_ST {
 
 constexpr int KC = 512;                          // k elements per stage
 constexpr int KSTEPS = KC / 16;                  // mma k-steps per stage
@@ -32,19 +48,18 @@ constexpr int TILE_N = 16;                       // weight rows per stage (mma M
 constexpr int KG = KC / 64;                      // 64-element (128-byte) k groups per stage
 constexpr int W_STAGE = TILE_N * KC * 2;         // 16384: [k group][row][128 B, 16-byte chunks xor-swizzled by row%8]
 constexpr int X_STAGE = KSTEPS * 32 * 16;        // 16384: [column pair][k-step][8 slots][b0.hi b1.hi b0.lo b1.lo]
-#ifndef ADA_NW
-#define ADA_NW 9
-#endif
-#ifndef ADA_NX
-#define ADA_NX 3
-#endif
-constexpr int NW = ADA_NW;                       // weight stages in flight per CTA
-constexpr int NX = ADA_NX;                       // activation / KV stages
+constexpr int TILES = ADA_TILES;                 // token column tiles
+// weight / activation stages in flight per CTA.  (One tile: 10 / 2 measured the same.  Three: a chunk's activations alone may
+// take three stages, and the next chunk's must be on their way.)
+constexpr int NW = TILES == 1 ? 9 : 6;
+constexpr int NX = TILES == 1 ? 3 : 6;
 constexpr int CONS_WARPS = 8;
 constexpr int CONS_THREADS = CONS_WARPS * 32;
 constexpr int THREADS = CONS_THREADS + 64;       // + weight producer warp + activation producer warp
-constexpr int MAX_COLS = 8;                      // tokens per pass (mma N)
-constexpr int RED_BYTES = CONS_WARPS * 2 * 128 * 4;  // cross-warp reduction scratch (two tiles per warp)
+constexpr int MAX_COLS = 8 * TILES;              // tokens per pass (one tile: mma N)
+constexpr int MAX_SEQS = 8;                      // sequences per launch
+constexpr int RED_BYTES = CONS_WARPS * 2 * TILES * 128 * 4;  // cross-warp reduction scratch (two matrices per warp)
+constexpr int X_BLOCK = TILES * X_STAGE;         // activations of one chunk in global memory, all columns
 constexpr int SCRATCH_BYTES = 33 * 1024;         // consumers' scratch: GEMM reduction, or the attention phase's buffers
 
 constexpr int ERR_TIMEOUT_MBAR = 1, ERR_TIMEOUT_GRID = 2;
@@ -85,15 +100,14 @@ __host__ __device__ __forceinline__ void cta_tile_range(int T, int cta, int G, i
 // GEMMs with fewer units per CTA than chunks per tile, or more tiles per CTA than consumer warps,
 // keep whole tiles.  The plan is a function of the GEMM's shape and the grid only.
 struct Plan {
-    int pair, half, nch;   // of the GEMM; nch = k chunks
-    int split;       // 0: whole tiles [t0, t1) in groups of CONS_WARPS
-    int t0, t1;
-    // split: one group of n slots; slot s holds tile ta + s, except that
-    int n, ta, tb;
-    int s0_own_k0;   //   slot 0 multiplies its own tile from chunk s0_own_k0 on (0: a whole tile),
-    int s0_pub_k1;   //   and before that the chunks below s0_pub_k1 of tile tb, to publish (0: none);
-    int sl_k1;       //   the last slot (if not slot 0) multiplies chunks below sl_k1 only, to publish (nch: a whole tile)
-    int ksp;         // split with a tail part: k-splits in which the CTA before publishes its head part
+    int t0, n;             // tiles t0 .. t0 + n - 1: whole ones, in groups of CONS_WARPS; or (split) one group of n slots, slot s
+                           // holding tile t0 + s, except that
+    short nch;             // k chunks of the GEMM
+    short s0_own_k0;       //   slot 0 multiplies its own tile from chunk s0_own_k0 on (0: a whole tile),
+    short s0_pub_k1;       //   and before that the chunks below s0_pub_k1 of tile t0 + n, to publish (0: none);
+    short sl_k1;           //   the last slot (if not slot 0) multiplies chunks below sl_k1 only, to publish (nch: a whole tile)
+    short ksp;             // split with a tail part: k-splits in which the CTA before publishes its head part
+    unsigned char pair, split;
 };
 // the k-splits of a group of ng slots
 __host__ __device__ __forceinline__ int group_ks(int ng) {
@@ -103,12 +117,12 @@ __host__ __device__ __forceinline__ int group_ks(int ng) {
 }
 __host__ __device__ inline Plan make_plan(const Gemm &g, int cta, int C, bool with_ksp = true) {
     Plan p;
-    p.pair = g.pair;
-    p.half = g.half;
+    p.pair = (unsigned char)g.pair;
     p.split = 0;
-    p.t0 = p.t1 = p.n = p.ta = p.tb = p.s0_own_k0 = p.s0_pub_k1 = p.ksp = 0;
+    p.t0 = p.n = 0;
+    p.s0_own_k0 = p.s0_pub_k1 = p.ksp = 0;
     const int T = g.tiles(), nch = (g.K + KC - 1) / KC;
-    p.nch = p.sl_k1 = nch;
+    p.nch = p.sl_k1 = (short)nch;
     if (cta < 0 || cta >= C) return p;
     // 32-bit arithmetic throughout (a 64-bit division costs hundreds of cycles); GEMMs whose unit
     // count times the CTA count does not fit keep whole tiles
@@ -116,28 +130,30 @@ __host__ __device__ inline Plan make_plan(const Gemm &g, int cta, int C, bool wi
     const bool fits = (unsigned long long)T * nch * (unsigned)(C + 1) < 0x7fffffffull;
     const unsigned L = (U + C - 1) / C;      // most units of one CTA; a run of L units touches <= (L + nch - 2) / nch + 1 tiles
     if (!g.split || !fits || U / C < (unsigned)nch || (L + nch - 2) / nch + 1 > (unsigned)CONS_WARPS) {
-        cta_tile_range(T, cta, C, p.t0, p.t1);
+        int t1;
+        cta_tile_range(T, cta, C, p.t0, t1);
+        p.n = t1 - p.t0;
         return p;
     }
     p.split = 1;
     const unsigned u0 = U * (unsigned)cta / C, u1 = U * (unsigned)(cta + 1) / C;
-    p.ta = (int)(u0 / nch);
-    p.tb = (int)((u1 - 1) / nch);
-    const int ka = (int)(u0 - p.ta * nch), kb = (int)((u1 - 1) - p.tb * nch) + 1;
+    const int ta = (int)(u0 / nch), tb = (int)((u1 - 1) / nch);
+    const int ka = (int)(u0 - ta * nch), kb = (int)((u1 - 1) - tb * nch) + 1;
     const bool has_tail = ka > 0, has_head = kb < nch;
     const bool shared = has_tail && has_head && kb <= ka;
-    p.s0_own_k0 = ka;
-    p.n = p.tb - p.ta + 1;
-    if (shared) { p.s0_pub_k1 = kb; p.n -= 1; }
-    else if (has_head) p.sl_k1 = kb;
-    if (ka > 0 && with_ksp) p.ksp = group_ks(make_plan(g, cta - 1, C, false).n);
+    p.t0 = ta;
+    p.n = tb - ta + 1;
+    p.s0_own_k0 = (short)ka;
+    if (shared) { p.s0_pub_k1 = (short)kb; p.n -= 1; }
+    else if (has_head) p.sl_k1 = (short)kb;
+    if (ka > 0 && with_ksp) p.ksp = (short)group_ks(make_plan(g, cta - 1, C, false).n);
     return p;
 }
 // the tile slot s of a split plan multiplies at chunk kc (-1: none)
 __host__ __device__ __forceinline__ int plan_tile(const Plan &p, int s, int kc) {
-    if (s == 0) return kc < p.s0_pub_k1 ? p.tb : (kc >= p.s0_own_k0 ? p.ta : -1);
+    if (s == 0) return kc < p.s0_pub_k1 ? p.t0 + p.n : (kc >= p.s0_own_k0 ? p.t0 : -1);
     if (s == p.n - 1 && kc >= p.sl_k1) return -1;
-    return p.ta + s;
+    return p.t0 + s;
 }
 
 struct Smem {                                    // must start on a 1024-byte boundary (swizzle pattern)
@@ -146,7 +162,7 @@ struct Smem {                                    // must start on a 1024-byte bo
     alignas(16) unsigned char scratch[SCRATCH_BYTES];
     alignas(16) float vec[MAX_COLS];                   // per-column scalars (rstd, ...)
     alignas(8) unsigned long long w_full[NW], w_empty[NW], x_full[NX], x_empty[NX];
-    alignas(16) int desc[3][32];                  // per-role copy of the step descriptor (persistent decode kernel)
+    alignas(16) int desc[3][TILES == 1 ? 24 : 44];                  // per-role copy of the step descriptor (persistent decode kernel)
     int abort;
     int bcast[8];
     unsigned trace_n;
@@ -243,15 +259,6 @@ __device__ __forceinline__ void red_release_add(unsigned *p, unsigned v) {
 
 // ---------------------------------------------------------------- bounded waits
 
-// Optional event trace (test hook): records (globaltimer ns, code) pairs while `tr_on` is set.
-// Every CTA writes its own region of the buffer, so that recording costs a shared-memory counter
-// and one store.
-struct Trace {
-    unsigned long long *buf;   // [grid][cap][2], or nullptr
-    unsigned *count;           // [grid]
-    unsigned cap;              // events per CTA
-};
-
 struct Shared {            // what every role needs to wait safely
     Smem *sm;
     int *err;              // global error word (0 = fine)
@@ -305,7 +312,8 @@ __device__ __forceinline__ void mbar_wait(const Shared &S, unsigned long long *b
 // value held in a register across the main loop ties up the register file, and wherever the
 // compiler has to move it the warp first waits for the load.  Each thread reads back only its own
 // words, after cp_async_wait_all().  The exchange of partial sums uses the first 8 KB of the scratch area.
-constexpr int STASH_OFFSET = RED_BYTES, STASH_WORDS = 3, STASH_PASSES = 4;   // passes: 8 tiles x 8 columns of 16 rows by 256 threads
+// (Passes beyond the stash, which only three column tiles have, fetch theirs when they need them.)
+constexpr int STASH_OFFSET = RED_BYTES, STASH_WORDS = 3, STASH_PASSES = TILES == 1 ? 4 : 3;   // one tile: 8 tiles x 8 columns of 16 rows by 256 threads
 static_assert(STASH_OFFSET + STASH_PASSES * STASH_WORDS * CONS_THREADS * 4 <= SCRATCH_BYTES, "stash exceeds the scratch area");
 __device__ __forceinline__ uint32_t *stash_of(Smem *sm, int pass) {
     return reinterpret_cast<uint32_t *>(sm->scratch + STASH_OFFSET) + pass * (STASH_WORDS * CONS_THREADS) + threadIdx.x;
@@ -358,8 +366,8 @@ __device__ __forceinline__ void grid_wait(const Shared &S, const unsigned *ctr, 
 
 // ---------------------------------------------------------------- activation layout
 
-// Activations for a GEMM of depth K live in global memory as ceil(K/KC) blocks of X_STAGE bytes.
-// A block holds four sub-blocks of 4 KB, one per pair of token columns; in sub-block p, k-step s,
+// Activations for a GEMM of depth K live in global memory as ceil(K/KC) blocks of X_BLOCK bytes.
+// A block holds four sub-blocks of 4 KB per column tile, one per pair of token columns; in sub-block p, k-step s,
 // slot j (0..7) holds 16 bytes: the mma B fragment (b0, b1) of the bf16 high parts, then of the
 // bf16 low parts, for token column 2 p + j/4 and k = 16 s + 2 (j%4) + {0,1} (+8 for b1).  Lane l of
 // a warp reads slot l%8 of sub-block l/8.  A pass that carries few tokens fetches only the
@@ -369,7 +377,7 @@ __device__ __forceinline__ void grid_wait(const Shared &S, const unsigned *ctr, 
 __device__ __forceinline__ size_t xfrag_index(int k, int col) {   // index in 2-byte units of the high part
     const int chunk = k / KC, ks = (k % KC) >> 4, kk = k & 15;
     const int slot = (col & 1) * 4 + ((kk & 7) >> 1);
-    return (((((size_t)chunk * 4 + (col >> 1)) * KSTEPS + ks) * 8 + slot) << 3) + ((kk >> 3) << 1) + (kk & 1);
+    return (((((size_t)chunk * (4 * TILES) + (col >> 1)) * KSTEPS + ks) * 8 + slot) << 3) + ((kk >> 3) << 1) + (kk & 1);
 }
 __device__ __forceinline__ void xfrag_store(__nv_bfloat16 *X, int k, int col, float v) {
     const __nv_bfloat16 hi = __float2bfloat16_rn(v);
@@ -385,7 +393,7 @@ __device__ __forceinline__ void xfrag_store2(__nv_bfloat16 *X, int k, int col, f
     *reinterpret_cast<__nv_bfloat162 *>(X + i) = h;
     *reinterpret_cast<__nv_bfloat162 *>(X + i + 4) = __floats2bfloat162_rn(a - __low2float(h), b - __high2float(h));
 }
-__host__ __device__ inline size_t xfrag_bytes(int K) { return (size_t)((K + KC - 1) / KC) * X_STAGE; }
+__host__ __device__ inline size_t xfrag_bytes(int K) { return (size_t)((K + KC - 1) / KC) * X_BLOCK; }
 
 // ---------------------------------------------------------------- GEMM phase
 
@@ -400,6 +408,8 @@ struct Cols {
     // ring holds three stages; with one chunk per stage a CTA that owns two weight tiles would wait
     // for an activation copy every 96 KB of weights.)
     __device__ __forceinline__ int chunks() const { return ncp == 1 ? 4 : ncp == 2 ? 2 : 1; }   // a power of two
+    // column tiles of four pairs, counted from the first pair fetched; each is an activation stage of its own where there are several
+    __device__ __forceinline__ int tiles() const { return TILES == 1 ? 1 : (ncp + 3) >> 2; }
     // Up to four columns: one multiply-add takes their high parts as token columns 0..3 and their low parts as 4..7.
     __device__ __forceinline__ bool packed() const { return ncp <= 2; }
 };
@@ -412,7 +422,7 @@ struct Rings {   // position of one role in the two rings: number of the next we
 // A plan as a sequence of groups of at most CONS_WARPS slots: a split plan is one group.
 struct Groups {
     int g0, left;
-    __device__ __forceinline__ explicit Groups(const Plan &p) : g0(p.split ? p.ta : p.t0), left(p.split ? p.n : p.t1 - p.t0) {}
+    __device__ __forceinline__ explicit Groups(const Plan &p) : g0(p.t0), left(p.n) {}
     __device__ __forceinline__ int slots() const { return min(left, CONS_WARPS); }
     __device__ __forceinline__ void next() { g0 += CONS_WARPS; left -= CONS_WARPS; }
 };
@@ -466,8 +476,8 @@ __device__ __forceinline__ void w_wait(const Shared &S, uint32_t i, uint32_t &kn
 }
 
 // Weight producer warp: streams this CTA's tiles of the GEMM through the weight ring.  W2: map of the second matrix of a
-// pair where the two are separate tensors (null: stacked in W).
-__device__ __forceinline__ void gemm_produce_w(const Shared &S, const Plan &pl, const CUtensorMap *W, const CUtensorMap *W2, Rings &r, uint64_t pol) {
+// pair where the two are separate tensors (null: stacked in W, `half` rows on).
+__device__ __forceinline__ void gemm_produce_w(const Shared &S, const Plan &pl, const CUtensorMap *W, const CUtensorMap *W2, int half, Rings &r, uint64_t pol) {
     Smem *sm = S.sm;
     const int lane = threadIdx.x & 31;
     const int nch = pl.nch, pair = pl.pair;
@@ -489,7 +499,7 @@ __device__ __forceinline__ void gemm_produce_w(const Shared &S, const Plan &pl, 
                     if (lane == 0) {
                         if (!aborted(S)) {
                             mbar_expect_tx(&sm->w_full[ws], (uint32_t)W_STAGE);
-                            tma_load_3d(sm->w[ws], (p && W2) ? W2 : W, 0, tile * TILE_N + ((p && !W2) ? pl.half : 0), kc * KG, &sm->w_full[ws], pol);
+                            tma_load_3d(sm->w[ws], (p && W2) ? W2 : W, 0, tile * TILE_N + ((p && !W2) ? half : 0), kc * KG, &sm->w_full[ws], pol);
                         }
                         w_issued_set(sm, r.w);
                     }
@@ -509,7 +519,6 @@ __device__ __forceinline__ void gemm_produce_x(const Shared &S, const Plan &pl, 
     Smem *sm = S.sm;
     const int lane = threadIdx.x & 31;
     const int nch = pl.nch, XC = cols.chunks();
-    const uint32_t bytes = (uint32_t)cols.ncp * 4096u;
     const unsigned char *src = reinterpret_cast<const unsigned char *>(X) + cols.cp0 * 4096;
     // as many rounds as the plan has groups; a CTA without any still passes `ready` and the hook
     Groups g(pl);
@@ -523,12 +532,17 @@ __device__ __forceinline__ void gemm_produce_x(const Shared &S, const Plan &pl, 
             if (first) ready();
             if (some) {
                 const int nc = min(XC, nch - kc);
-                if (lane == 0 && !aborted(S)) {
-                    mbar_expect_tx(&sm->x_full[r.xs], bytes * nc);
-                    for (int q = 0; q < nc; ++q)   // chunk kc+q: column pairs cp0.. at [q][pair - cp0] of the stage
-                        bulk_g2s(sm->x[r.xs] + q * bytes, src + (size_t)(kc + q) * X_STAGE, bytes, &sm->x_full[r.xs], pol);
+#pragma unroll 1
+                for (int t = 0; t < cols.tiles(); ++t) {
+                    const uint32_t bytes = (uint32_t)min(cols.ncp - 4 * t, 4) * 4096u;
+                    if (t > 0) mbar_wait(S, &sm->x_empty[r.xs], r.xp ^ 1);
+                    if (lane == 0 && !aborted(S)) {
+                        mbar_expect_tx(&sm->x_full[r.xs], bytes * nc);
+                        for (int q = 0; q < nc; ++q)   // chunk kc+q: column pairs cp0 + 4 t .. at [q][pair] of the stage
+                            bulk_g2s(sm->x[r.xs] + q * bytes, src + (size_t)(kc + q) * X_BLOCK + t * 16384, bytes, &sm->x_full[r.xs], pol);
+                    }
+                    r.next_x();
                 }
-                r.next_x();
             }
             if (first) { after_first(); first = false; }
             if (!some) break;
@@ -543,24 +557,30 @@ struct NoHook {
 // The 32 k-steps of one weight stage: fragment loads run four steps ahead of the multiply-adds that use them.
 // Even k-steps accumulate into acc[0] (high parts) and acc[2] (low parts), odd ones into acc[1] and acc[3].  (A stage of one warp
 // is bound by the shared-memory reads of all eight, 200 cycles of the SM for 16 KB, not by the length of these chains.)
-__device__ __forceinline__ void stage_full(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
-    constexpr int PF = 4;
+template <int T>
+__device__ __forceinline__ void stage_full(float (&acc)[TILES][4][4], const unsigned char *ws, const unsigned char *const (&xs)[TILES], int a_hi, int a_sw) {
+    constexpr int PF = T == 1 ? 4 : 2;
     uint32_t a[PF][4];
-    uint4 b[PF];
+    uint4 b[PF][T];
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
         ldmatrix_x4(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
-        b[j] = *reinterpret_cast<const uint4 *>(xs + j * 128);
+#pragma unroll
+        for (int t = 0; t < T; ++t) b[j][t] = *reinterpret_cast<const uint4 *>(xs[t] + j * 128);
     }
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
         const int cur = j % PF;
-        mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
-        mma16816(acc[(j & 1) + 2], a[cur], b[cur].z, b[cur].w);
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            mma16816(acc[t][j & 1], a[cur], b[cur][t].x, b[cur][t].y);
+            mma16816(acc[t][(j & 1) + 2], a[cur], b[cur][t].z, b[cur][t].w);
+        }
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
             ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
-            b[cur] = *reinterpret_cast<const uint4 *>(xs + ks * 128);
+#pragma unroll
+            for (int t = 0; t < T; ++t) b[cur][t] = *reinterpret_cast<const uint4 *>(xs[t] + ks * 128);
         }
     }
 }
@@ -614,9 +634,15 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
     // ldmatrix source of this lane inside a stage: row (lane%8) + 8 ((lane/8)%2), 16-byte chunk lane/16 of the k-step
     const int a_row = (lane & 7) + ((lane >> 3) & 1) * 8;
     const int a_off = a_row * 128, a_hi = lane >> 4, a_sw = a_row & 7;
-    // this lane's column pair, if it was fetched (else any fetched pair: its column is not in use), and its 16 (8) bytes
-    const int xpair = packed ? min((lane >> 3) & 1, cols.ncp - 1) : min(max((lane >> 3) - cols.cp0, 0), cols.ncp - 1);
-    const int x_off = xpair * 4096 + (lane & 7) * 16 + (packed ? (lane >> 4) * 8 : 0);
+    const int nt = cols.tiles();
+    // this lane's column pair of every tile, counted from the first fetched (past the last: any, its columns are not in use), and
+    // its 16 (8) bytes
+    int x_off[TILES];
+#pragma unroll
+    for (int t = 0; t < TILES; ++t) {
+        const int xpair = min(packed ? (lane >> 3) & 1 : lane >> 3, max(cols.ncp - 1 - 4 * t, 0));
+        x_off[t] = xpair * 4096 + (lane & 7) * 16 + (packed ? (lane >> 4) * 8 : 0);
+    }
     const int nact = __popc(mask), row = lane & 15;
     uint32_t known = r.w;
     bool first = true;
@@ -634,8 +660,8 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
         const int my_own_k0 = (!mine || pub_only) ? nch : slot_id == 0 ? s0_own_k0 : 0;
         const int own_tile = (mine && !pub_only) ? g.g0 + slot_id : -1;
         const bool tail = own_tile >= 0 && my_own_k0 > 0;   // the head part of this tile comes from CTA cta - 1
-        // this thread's elements: columns by pass, four bits each
-        unsigned my_cols = 0;
+        // this thread's elements: columns by pass, five bits each
+        unsigned long long my_cols = 0;
 #pragma unroll 1
         for (int ps = 0; ps < n_pass; ++ps) {
             const int u = 16 * ps + 2 * warp + (lane >> 4), slot = u & (eslots - 1);
@@ -643,27 +669,48 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             unsigned m = mask;
             for (; ci > 0 && m; --ci) m &= m - 1;
             const bool act = m != 0 && slot < ng && !(slot > 0 && slot == ng - 1 && sl_k1 < nch);
-            my_cols |= (act ? (unsigned)__ffs(m) - 1u : 15u) << (4 * ps);
-            if (act) epi.pre(ps, g.g0 + slot, row, __ffs(m) - 1);
+            my_cols |= (unsigned long long)(act ? __ffs(m) - 1 : 31) << (5 * ps);
+            if (act && ps < STASH_PASSES) epi.pre(ps, g.g0 + slot, row, __ffs(m) - 1);
         }
-        float acc0[4][4], acc1[4][4];   // [even/odd step x hi/lo][fragment] of the one or two matrices
+        float acc0[TILES][4][4], acc1[TILES][4][4];   // [column tile][even/odd step x hi/lo][fragment] of the one or two matrices
+        auto clear = [&]() {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+            for (int t = 0; t < TILES; ++t)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc0[q][i] = acc1[q][i] = 0.f;
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc0[t][q][i] = acc1[t][q][i] = 0.f;
+        };
+        clear();
         // fold the partial accumulators in a fixed order: the chains of the high parts, those of the low parts, both.
-        // Four columns or fewer: the result of column pair cp0 + j stands in the lanes with lane % 4 = j, else of pair j.
-        float d0[4], d1[4];
-        auto fold = [&](float (&d)[4], float (&acc)[4][4]) {
+        // The result of column pair cp0 + 4 t + j stands in tile t, lanes with lane % 4 = j.
+        float d0[TILES][4], d1[TILES][4];
+        auto fold = [&](float (&d)[TILES][4], float (&acc)[TILES][4][4]) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float hi = acc[0][i] + acc[1][i];
-                d[i] = hi + (packed ? __shfl_xor_sync(0xffffffffu, hi, 2) : acc[2][i] + acc[3][i]);
-            }
+            for (int t = 0; t < TILES; ++t)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float hi = acc[t][0][i] + acc[t][1][i];
+                    d[t][i] = hi + (packed ? __shfl_xor_sync(0xffffffffu, hi, 2) : acc[t][2][i] + acc[t][3][i]);
+                }
         };
 #pragma unroll 1
         for (int kc = 0; kc < nch; ++kc) {
-            if ((kc & (XC - 1)) == 0) mbar_wait(S, &sm->x_full[r.xs], r.xp);
+            const unsigned char *xt[TILES];   // the chunk's activations, by column tile
+            if (TILES == 1) {
+                if ((kc & (XC - 1)) == 0) mbar_wait(S, &sm->x_full[r.xs], r.xp);
+                xt[0] = sm->x[r.xs] + (kc & (XC - 1)) * cols.ncp * 4096 + x_off[0];
+            } else {
+                uint32_t xs = r.xs, xp = r.xp;
+#pragma unroll
+                for (int t = 0; t < TILES; ++t) {
+                    xt[t] = sm->x[xs] + (t == 0 ? (kc & (XC - 1)) * cols.ncp * 4096 : 0) + x_off[t];
+                    if (t < nt) {
+                        if ((kc & (XC - 1)) == 0) mbar_wait(S, &sm->x_full[xs], xp);
+                        if (++xs == NX) { xs = 0; xp ^= 1; }
+                    }
+                }
+            }
             if (threadIdx.x == 0 && first) trace(S, EV_X0, 0);
             first = false;
             // the k-splits of a slot take whole stages in turn, counted from the first chunk of the part
@@ -673,7 +720,6 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             const bool here = kc < my_pub_k1 || kc >= my_own_k0;   // this slot has a stage at chunk kc
             const int kbase = kc < my_pub_k1 ? 0 : my_own_k0;
             if (here && ((kc - kbase) & (KS - 1)) == ks_id) {
-                const unsigned char *xs = sm->x[r.xs] + (kc & (XC - 1)) * cols.ncp * 4096 + x_off;
                 const bool gap0 = slot_id > 0 && kc >= s0_pub_k1 && kc < s0_own_k0;   // slot 0 has none here
                 uint32_t i = r.w + (uint32_t)((stages_before(pl, ng, kc) + slot_id - gap0) * pair);
 #pragma unroll 1
@@ -682,11 +728,17 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                     const uint32_t wslot = i % NW;
                     const unsigned char *ws = sm->w[wslot] + a_off;
                     if (packed) {
-                        if (p == 0) stage_packed(acc0, ws, xs, a_hi, a_sw);
-                        else stage_packed(acc1, ws, xs, a_hi, a_sw);
-                    } else {
-                        if (p == 0) stage_full(acc0, ws, xs, a_hi, a_sw);
-                        else stage_full(acc1, ws, xs, a_hi, a_sw);
+                        if (p == 0) stage_packed(acc0[0], ws, xt[0], a_hi, a_sw);
+                        else stage_packed(acc1[0], ws, xt[0], a_hi, a_sw);
+                    } else if (nt == 1) {
+                        if (p == 0) stage_full<1>(acc0, ws, xt, a_hi, a_sw);
+                        else stage_full<1>(acc1, ws, xt, a_hi, a_sw);
+                    } else if (TILES > 1 && nt == 2) {
+                        if (p == 0) stage_full<TILES < 2 ? TILES : 2>(acc0, ws, xt, a_hi, a_sw);
+                        else stage_full<TILES < 2 ? TILES : 2>(acc1, ws, xt, a_hi, a_sw);
+                    } else if (TILES > 1) {
+                        if (p == 0) stage_full<TILES>(acc0, ws, xt, a_hi, a_sw);
+                        else stage_full<TILES>(acc1, ws, xt, a_hi, a_sw);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
@@ -694,23 +746,29 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             }
             if ((kc & (XC - 1)) == XC - 1 || kc == nch - 1) {   // activation stages are shared: every warp waits for and releases each of them
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
-                r.next_x();
+#pragma unroll 1
+                for (int t = 0; t < nt; ++t) {
+                    if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
+                    r.next_x();
+                }
             }
             if (kc + 1 == my_pub_k1) {
                 // The head part of a split tile is complete: every k-split warp publishes its own sums
                 // (no meeting inside the CTA in the middle of the stream) and starts over for the tail
                 // part that may follow in this slot.
-                unsigned long long *pb = part + (size_t)(cta * CONS_WARPS + ks_id) * 256;
                 fold(d0, acc0);
                 if (pair == 2) fold(d1, acc1);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    st_relaxed_u64(pb + i * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d0[i]));
-                    if (pair == 2) st_relaxed_u64(pb + (4 + i) * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d1[i]));
+                for (int t = 0; t < TILES; ++t) {
+                    if (t >= nt) break;
+                    unsigned long long *pb = part + (size_t)((cta * CONS_WARPS + ks_id) * TILES + t) * 256;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) acc0[q][i] = acc1[q][i] = 0.f;
+                    for (int i = 0; i < 4; ++i) {
+                        st_relaxed_u64(pb + i * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d0[t][i]));
+                        if (pair == 2) st_relaxed_u64(pb + (4 + i) * 32 + lane, ((unsigned long long)phase_id << 32) | __float_as_uint(d1[t][i]));
+                    }
                 }
+                clear();
             }
         }
         r.w += (uint32_t)(stages_before(pl, ng, nch) * pair);
@@ -724,27 +782,35 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             unsigned long long t0 = 0;
             for (uint32_t it = 0;; ++it) {
                 bool ok = true;
-                float add[2][4];
+                float add[2][TILES][4];
 #pragma unroll
                 for (int p = 0; p < 2; ++p)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) add[p][i] = 0.f;
+                    for (int t = 0; t < TILES; ++t)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) add[p][t][i] = 0.f;
                 for (int q = ks_id; q < pl.ksp; q += KS) {
-                    const unsigned long long *pb = part + (size_t)((cta - 1) * CONS_WARPS + q) * 256;
 #pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        if (p >= pair) break;
+                    for (int t = 0; t < TILES; ++t) {
+                        if (t >= nt) break;
+                        const unsigned long long *pb = part + (size_t)(((cta - 1) * CONS_WARPS + q) * TILES + t) * 256;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const unsigned long long v = ld_relaxed_u64(pb + (p * 4 + i) * 32 + lane);
-                            ok = ok && (unsigned)(v >> 32) == phase_id;
-                            add[p][i] += __uint_as_float((unsigned)v);
+                        for (int p = 0; p < 2; ++p) {
+                            if (p >= pair) break;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const unsigned long long v = ld_relaxed_u64(pb + (p * 4 + i) * 32 + lane);
+                                ok = ok && (unsigned)(v >> 32) == phase_id;
+                                add[p][t][i] += __uint_as_float((unsigned)v);
+                            }
                         }
                     }
                 }
                 if (__all_sync(0xffffffffu, ok)) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) { d0[i] += add[0][i]; d1[i] += add[1][i]; }
+                    for (int t = 0; t < TILES; ++t)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) { d0[t][i] += add[0][t][i]; d1[t][i] += add[1][t][i]; }
                     break;
                 }
                 if ((it & 15u) == 15u || S.wait_ns < SHORT_LIMIT_NS) {   // bounded like every other wait on another CTA
@@ -757,25 +823,30 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 __nanosleep(64);
             }
         }
-        float *red = reinterpret_cast<float *>(sm->scratch);   // [matrix][warp][fragment element][lane]
+        float *red = reinterpret_cast<float *>(sm->scratch);   // [matrix][warp][column tile][fragment element][lane]
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            red[(warp * 4 + i) * 32 + lane] = d0[i];
-            if (pair == 2) red[((CONS_WARPS + warp) * 4 + i) * 32 + lane] = d1[i];
+        for (int t = 0; t < TILES; ++t) {
+            if (t >= nt) break;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                red[((warp * TILES + t) * 4 + i) * 32 + lane] = d0[t][i];
+                if (pair == 2) red[(((CONS_WARPS + warp) * TILES + t) * 4 + i) * 32 + lane] = d1[t][i];
+            }
         }
         bar_consumers();
 #pragma unroll 1
         for (int ps = 0; ps < n_pass; ++ps) {
-            const int slot = (16 * ps + 2 * warp + (lane >> 4)) & (eslots - 1), cn = (my_cols >> (4 * ps)) & 15;
+            const int slot = (16 * ps + 2 * warp + (lane >> 4)) & (eslots - 1), cn = (int)(my_cols >> (5 * ps)) & 31;
             const bool act = cn < MAX_COLS;
             const int col = act ? cn : 0;
-            // element (row, column) of a warp's sums: fragment element 2 (row / 8) + column % 2 of lane 4 (row % 8) + column pair
-            const float *o = red + (((slot & (TS - 1)) * 4 + 2 * (row >> 3) + (col & 1)) * 32 + ((row & 7) << 2) + ((col >> 1) - (packed && act ? cols.cp0 : 0)));
+            // element (row, column) of a warp's sums: fragment element 2 (row / 8) + column % 2 of lane 4 (row % 8) + column pair % 4, tile pair / 4
+            const int pr = act ? (col >> 1) - cols.cp0 : 0;
+            const float *o = red + ((((slot & (TS - 1)) * TILES + (pr >> 2)) * 4 + 2 * (row >> 3) + (col & 1)) * 32 + ((row & 7) << 2) + (pr & 3));
             float v0[CONS_WARPS], v1[CONS_WARPS];
 #pragma unroll
             for (int q = 0; q < CONS_WARPS; ++q) {
-                v0[q] = q < KS ? o[(q << lts) * 128] : 0.f;
-                v1[q] = q < KS && pair == 2 ? o[(CONS_WARPS + (q << lts)) * 128] : 0.f;
+                v0[q] = q < KS ? o[(q << lts) * (TILES * 128)] : 0.f;
+                v1[q] = q < KS && pair == 2 ? o[(CONS_WARPS + (q << lts)) * (TILES * 128)] : 0.f;
             }
             float e0 = v0[0], e1 = v1[0];
 #pragma unroll
@@ -819,5 +890,7 @@ __device__ __forceinline__ void settle_on_abort(const Shared &S) {
     while (gtime() - t0 < 200000ull) __nanosleep(1000);
 }
 
-}  // namespace st
+}  // namespace ADA_ST
 }  // namespace ada
+
+#endif
