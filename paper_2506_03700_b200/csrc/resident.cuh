@@ -240,56 +240,71 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             if (layer == 0) plain = A.tok_embed + (size_t)s.st->tok[seq_of(r)][s.st->pos[r] & (TOK_RING - 1)] * d;
             else if (layer > 0 && s.st->fl[r] == layer) plain = A.c.resid + (size_t)r * d;
             float ss = 0.f;
-            float *xr = s.xs + (size_t)r * d;
+            float *xr = s.xs + (size_t)r * d, *ur = s.us + (size_t)r * A.ku;
+            float2 v[8], g[8];   // up to 512 elements of the row and of the gain stay in registers
+#pragma unroll 1
             for (int k0 = 0; k0 < d; k0 += 64 * 8) {
-                float a[8], b[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int k = k0 + 64 * q + 2 * lane();
+                    g[q] = k < d ? __ldg(reinterpret_cast<const float2 *>(gain + k)) : make_float2(0.f, 0.f);
+                }
                 until(A, s.st, [&]() {
                     bool ok = true;
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         const int k = k0 + 64 * q + 2 * lane();
-                        a[q] = b[q] = 0.f;
+                        v[q] = make_float2(0.f, 0.f);
                         if (k >= d) continue;
-                        if (plain) { const float2 v = __ldcg(reinterpret_cast<const float2 *>(plain + k)); a[q] = v.x; b[q] = v.y; }
-                        else ok = get2(X + (size_t)r * d + k, a[q], b[q], want) && ok;
+                        if (plain) v[q] = __ldcg(reinterpret_cast<const float2 *>(plain + k));
+                        else ok = get2(X + (size_t)r * d + k, v[q].x, v[q].y, want) && ok;
                     }
                     return ok;
                 });
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int k = k0 + 64 * q + 2 * lane();
-                    if (k < d) *reinterpret_cast<float2 *>(xr + k) = make_float2(a[q], b[q]);
-                    ss = fmaf(a[q], a[q], ss);
-                    ss = fmaf(b[q], b[q], ss);
+                    if (k < d) *reinterpret_cast<float2 *>(xr + k) = v[q];
+                    ss = fmaf(v[q].x, v[q].x, ss);
+                    ss = fmaf(v[q].y, v[q].y, ss);
                 }
             }
             const float rstd = 1.0f / sqrtf(warp_sum(ss) / d + A.c.eps);
-            for (int k = 2 * lane(); k < d; k += 64) {   // each lane its own elements
-                const float2 v = *reinterpret_cast<const float2 *>(xr + k), g = __ldg(reinterpret_cast<const float2 *>(gain + k));
-                *reinterpret_cast<float2 *>(s.us + (size_t)r * A.ku + k) = make_float2(v.x * rstd * g.x, v.y * rstd * g.y);
+            if (d <= 64 * 8) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int k = 64 * q + 2 * lane();
+                    if (k < d) *reinterpret_cast<float2 *>(ur + k) = make_float2(v[q].x * rstd * g[q].x, v[q].y * rstd * g[q].y);
+                }
+            } else {
+                for (int k = 2 * lane(); k < d; k += 64) {   // each lane its own elements
+                    const float2 x = *reinterpret_cast<const float2 *>(xr + k), gn = __ldg(reinterpret_cast<const float2 *>(gain + k));
+                    *reinterpret_cast<float2 *>(ur + k) = make_float2(x.x * rstd * gn.x, x.y * rstd * gn.y);
+                }
             }
         }
     }
-    // rows of exchanged words as they are
+    // rows of exchanged words as they are, 256 elements of a row per warp at a time
     __device__ __forceinline__ void load_words(u64 mask, const u64 *X, unsigned want, int K) const {
+        const int parts = (K + 255) >> 8;
         int i = 0;
-        for (u64 m = mask; m; m &= m - 1, ++i) {
-            if (i % WARPS != warp()) continue;
+        for (u64 m = mask; m; m &= m - 1) {
             const int r = __ffsll((long long)m) - 1;
-            for (int k0 = 0; k0 < K; k0 += 64 * 8) {
-                float a[8], b[8];
+            for (int pt = 0; pt < parts; ++pt, ++i) {
+                if (i % WARPS != warp()) continue;
+                float a[4], b[4];
                 until(A, s.st, [&]() {
                     bool ok = true;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int k = k0 + 64 * q + 2 * lane();
+                    for (int q = 0; q < 4; ++q) {
+                        const int k = 256 * pt + 64 * q + 2 * lane();
                         if (k < K) ok = get2(X + (size_t)r * K + k, a[q], b[q], want) && ok;
                     }
                     return ok;
                 });
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int k = k0 + 64 * q + 2 * lane();
+                for (int q = 0; q < 4; ++q) {
+                    const int k = 256 * pt + 64 * q + 2 * lane();
                     if (k < K) *reinterpret_cast<float2 *>(s.us + (size_t)r * A.ku + k) = make_float2(a[q], b[q]);
                 }
             }
@@ -463,11 +478,12 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
     // chunk partials of every head, merged in ascending order, as the O product's input
     __device__ __forceinline__ void load_attention(u64 mask, unsigned want) const {
         const Ctx &c = A.c;
-        int i = 0;
-        for (u64 m = mask; m; m &= m - 1, ++i) {
-            if (i % WARPS != warp()) continue;
+        int i = 0;   // 64 features of a row per warp at a time
+        for (u64 m = mask; m; m &= m - 1) {
             const int r = __ffsll((long long)m) - 1, nch = s.st->pos[r] / kAttnChunk + 1;
-            for (int k = 2 * lane(); k < c.nq * HD; k += 64) {
+            for (int k0 = 0; k0 < c.nq * HD; k0 += 64, ++i) {
+                const int k = k0 + 2 * lane();
+                if (i % WARPS != warp() || k >= c.nq * HD) continue;
                 const int h = k / HD, dim = k - h * HD;
                 const u64 *part = A.PT + ((size_t)r * c.nq + h) * c.n_chunks * (HD + 2);
                 float M = -INFINITY, den = 0.f, ox = 0.f, oy = 0.f;
@@ -621,12 +637,12 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             const int r = __ffsll((long long)m) - 1, G = gridDim.x;
             Msa a;
             a.m = -INFINITY; a.s = 0.f; a.i = INT_MAX;
-            for (int b0 = 0; b0 < G; b0 += 32 * 4) {
-                float pm[4], ps[4], pi[4];
+            for (int b0 = 0; b0 < G; b0 += 32 * 5) {
+                float pm[5], ps[5], pi[5];
                 until(A, s.st, [&]() {
                     bool ok = true;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
+                    for (int q = 0; q < 5; ++q) {
                         const int b = b0 + 32 * q + lane();
                         if (b >= G) continue;
                         const u64 *o = A.HP + ((size_t)b * A.R + r) * 4;
@@ -636,7 +652,7 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
                     return ok;
                 });
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < 5; ++q) {
                     const int b = b0 + 32 * q + lane();
                     if (b >= G) continue;
                     Msa x;
