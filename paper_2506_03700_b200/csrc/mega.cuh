@@ -1382,16 +1382,20 @@ enum { PH_QKV = 0, PH_O, PH_GU, PH_DOWN, PH_T, PH_HEAD, PH_PRODUCTS, PH_ATTN = P
 __device__ __forceinline__ int prof_class(int ph) {   // class of ada_debug_profile that the phase's time is booked to
     return ph == PH_QKV ? 2 : ph == PH_ATTN ? 4 : ph == PH_O ? 5 : ph == PH_GU ? 6 : ph == PH_DOWN ? 8 : ph == PH_T ? 10 : 9;
 }
-// The one product of the layer where the unit-balanced split pays is gate / up (measured: it shortens it by 1.4 us, but
-// lengthens down, QKV and O, whose tile groups are k-split among the warps).
-__device__ __forceinline__ Gemm phase_gemm(const MegaArgs &A, int ph) {
+// Whole tiles or units of (tile, chunk): cutting tiles costs an exchange of partial sums at the end of the phase (some 0.7 us)
+// and saves the stages by which the CTA with most whole tiles exceeds its share, 0.36 us each: taken from four stages on.
+// Measured, whole -> cut: 13B O (8 stages fewer) 13.6 -> 12.1 us, down (22) 30.0 -> 25.4, QKV (5) 28.1 -> 26.9; 8B down (7)
+// 21.2 -> 20.5, QKV (3) 11.7 -> 11.7, O (2) 9.0 -> 9.3; 1B QKV (2) 6.2 -> 6.7.
+constexpr int CUT_STAGES = 4;
+__host__ __device__ __forceinline__ Gemm phase_gemm(const MegaArgs &A, int ph, int G) {
     const Ctx &c = A.c;
     Gemm g;
     g.N = ph == PH_QKV ? c.qkv_rows : ph == PH_GU ? 2 * c.dff : ph == PH_HEAD ? c.vocab : c.d;
     g.K = ph == PH_O ? c.nq * c.hd : ph == PH_DOWN ? c.dff : c.d;
     g.pair = ph == PH_GU ? 2 : 1;
     g.half = ph == PH_GU ? c.dff : 0;
-    g.split = ph == PH_GU && A.part != nullptr;
+    const int T = g.tiles(), nch = (g.K + KC - 1) / KC, most = (T + G - 1) / G * nch, share = (T * nch + G - 1) / G;
+    g.split = A.part != nullptr && ph != PH_HEAD && (most - share) * g.pair >= CUT_STAGES;
     return g;
 }
 
@@ -1739,7 +1743,7 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
     smem_init(sm);
     if (threadIdx.x >= 32 && threadIdx.x < 32 + PH_PRODUCTS) {
         const int ph = threadIdx.x - 32;
-        sm->plan[ph] = make_plan(phase_gemm(A, ph), blockIdx.x, gridDim.x);
+        sm->plan[ph] = make_plan(phase_gemm(A, ph, gridDim.x), blockIdx.x, gridDim.x);
     }
     __syncthreads();
     Shared S{sm, A.err, A.trace, 0, A.wait_ns};
