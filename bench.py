@@ -338,7 +338,7 @@ def run_ours(args):
     # = algorithmic bytes of the calls (layer passes x layer bytes + head evaluations x LM-head bytes + KV reads)
     # over the device time of the calls (the library's CUDA events on the session stream around its launches).
     n_dec_launches = max(1, int(a_st.kernel_launches) - K) if path == 1 else int(a_st.kernel_launches)
-    dom = "k_decode_persistent" if path == 1 else "k_gemv (one kernel per operation; the whole call is reported)"
+    dom = "k_decode_persistent" if path == 1 else "k_decode_resident, or k_gemv (one kernel per operation); the whole call is reported"
     dom_gbs = a_bytes / (a_st.decode_ms * 1e-3) / 1e9
     ratio = DRAM_TRAFFIC_RATIO["adaptive"] if path == 1 else None
     prompt_desc = (f"{cfg.prompt_len}-token uniform-random prompt" if cfg.batch == 1 else
