@@ -1,18 +1,19 @@
 // The persistent decode kernel: Algorithm 1 of the paper, one cooperative launch for many steps.
 //
-// One CTA per SM, ten warps: a weight producer, an activation / KV producer and eight consumers.
+// One CTA per SM: a warp that produces weights and K / V blocks, one that produces activations and queries, eight consumers.
 // Every CTA walks the same program
 //     control | for each layer: QKV | attention | O | gate-up | down | [head, control] ... | final head | control
-// with a grid barrier between phases.  The weight producer is not held by those barriers: it
-// keeps the TMA ring full with the tiles of the coming phases, so HBM keeps streaming while the
-// consumers meet.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
+// with a grid barrier between phases.  The weight producer is not held by those barriers (but for cache rows
+// of the pass itself): it keeps the TMA ring full with the tiles of the coming phases, so HBM keeps streaming while the
+// grid meets.  Measured, one layer in a plain step (1B / 8B shape): QKV 6.2 / 11.7 us, attention 7.2 / 9.9 (60 / 1040 positions),
+// O 5.4 / 9.0, gate-up 13.5 / 38.1, down 9.1 / 20.5, of which the bytes alone take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
 // residuals, counters) lives in device memory; the control points run in CTA 0, which publishes
 // each decision (continue the climb, start the next token, stop) to the other CTAs through a
 // sequence-numbered record.  The host launches, waits, and launches again until the call is done.
 //
-// Token columns: the up-to-eight tokens of a pass (the newest token and the early-predicted
-// tokens still in flight, Algorithm 1's P[l] (+) t_i) are the eight columns of the tensor-core
-// tile; column = position - base, fixed for the life of a token.  Per-column buffers therefore
+// Token columns: the tokens of a pass (per sequence the newest token and the early-predicted
+// tokens still in flight, Algorithm 1's P[l] (+) t_i) are the columns of one or three tensor-core
+// tiles; column = (position - base) x sequences of the launch + sequence, fixed for the life of a token.  Per-column buffers therefore
 // persist across steps: a token that left the climb at layer e finds its residual, its
 // normalisation partial sums and its layer-(e+1) GEMM input where its last pass left them.
 // Each column's numbers depend only on that column's own inputs (never on which other columns
@@ -521,7 +522,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     DevState *st = c.st;
     const MegaModel &M = A.m;
     const int tid = threadIdx.x, G = gridDim.x;
-    const int nseq = A.nseq, seq0 = A.seq0, cps = c.slots, L = c.L;   // cps: token columns per sequence
+    const int nseq = A.nseq, seq0 = A.seq0, cps = c.slots, L = c.L;   // cps: token columns per sequence (slots)
     Pub *pub = reinterpret_cast<Pub *>(A.pub) + (pub_no & 1);
     // Shared-memory copies for the bookkeeping thread (fetched by many threads at once: a single
     // thread reading them from global memory one after the other spent 30 us here on round trips to L2):

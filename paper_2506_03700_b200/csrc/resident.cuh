@@ -16,6 +16,9 @@
 // head partials that ends every step: a fence before, a fence after.
 //
 // Invariance rule as in kernels.cuh: a row's numbers depend on that row's inputs and the launch geometry only.
+//
+// Measured, four layers of width 256 (16 + 128 tokens, up to five early ones): 11.1 ms, 20.2 with a launch per operation.  Plain
+// decoding takes 115 us a token: some 4 to 7 us a phase, an exchange through L2 with the latency of its loads before and after.
 #pragma once
 
 #include "kernels.cuh"

@@ -1,7 +1,7 @@
 // Weight-streaming primitives of the persistent decode kernel (sm_100a).
 //
 // The decode step is bound by HBM bandwidth: every weight byte is read once per pass and used
-// for at most eight tokens.  The pieces here keep the memory pipe full:
+// for a few tokens (eight columns, or 24).  The pieces here keep the memory pipe full:
 //   * weights reach shared memory through TMA tensor copies (cp.async.bulk.tensor, one 16 KB box
 //     of 16 rows x 512 k per instruction, 128-byte swizzled) issued by a dedicated producer warp
 //     into a ring of stages guarded by mbarriers; the producer runs ahead of the consumers across
@@ -11,8 +11,8 @@
 //   * activations arrive through a second, small ring in the register layout the tensor-core
 //     instruction wants, already split into a bf16 high part and a bf16 low part, so that
 //     fp32 activations lose nothing: W.x = W.hi(x) + W.lo(x) with fp32 accumulation;
-//   * eight consumer warps multiply with mma.sync m16n8k16 (weights are the 16-row operand, the
-//     up-to-eight tokens are the 8 columns).  The tensor cores are used as a cheap way to issue
+//   * eight consumer warps multiply with mma.sync m16n8k16 (weights are the 16-row operand, eight
+//     tokens are the columns of a tile).  The tensor cores are used as a cheap way to issue
 //     the multiply-adds; the bound stays the memory system.
 //   * all CTAs of the persistent grid meet at a counter-based grid barrier between phases.
 // Every wait is bounded: on expiry an error word is set and all later waits fall through.
