@@ -17,8 +17,8 @@
 //
 // Invariance rule as in kernels.cuh: a row's numbers depend on that row's inputs and the launch geometry only.
 //
-// Measured, four layers of width 256 (16 + 128 tokens, up to five early ones): 11.1 ms, 20.2 with a launch per operation.  Plain
-// decoding takes 115 us a token: some 4 to 7 us a phase, an exchange through L2 with the latency of its loads before and after.
+// Measured, four layers of width 256 (16 + 128 tokens, up to five early ones): 10.3 ms, 20.2 with a launch per operation.  Plain
+// decoding takes 105 us a token: some 3 to 7 us a phase, an exchange through L2 with the latency of its loads before and after.
 #pragma once
 
 #include "kernels.cuh"
@@ -73,9 +73,10 @@ struct Shm {   // carved from dynamic shared memory
     State *st;
     double *freq;                        // rotary frequencies [hd / 2]
 };
+__host__ __device__ constexpr size_t walker_bytes(size_t n) { return (n + 15) / 16 * 16; }
 __host__ __device__ inline size_t shm_bytes(int R, int d, int ku, int hd, int n_cs, int batch, int L) {
     return sizeof(float) * ((size_t)R * d + (size_t)R * ku + (size_t)n_cs * hd + (size_t)WARPS * (hd + 2)) + sizeof(Msa) * WARPS * (size_t)R +
-           sizeof(int) * (size_t)batch * L + sizeof(State) + sizeof(double) * (hd / 2) + 64;
+           sizeof(int) * (size_t)batch * L + sizeof(State) + sizeof(double) * (hd / 2) + walker_bytes(sizeof(Args) + sizeof(Shm) + sizeof(u64)) + 64;
 }
 
 __device__ __forceinline__ int popc64(u64 m) { return __popcll(m); }
@@ -197,13 +198,15 @@ template <int NW, class Ptr> struct Product {
 // ---------------------------------------------------------------- the walker
 
 // The phases are functions of their own: inlined into one body, their addresses and prefetched weights together spilled
-// thousands of bytes; a call costs little beside a phase.
+// thousands of bytes; a call costs little beside a phase.  The object they work on, the arguments with it, lives in shared
+// memory (a copy per thread in local memory, and arguments read through a pointer to the parameters, were loads from L2 in front
+// of every phase: their L1 lines do not survive the fences of a step).
+// `tag`: number of the phase whose output is being written; `tag_x`: of the last layer output.
 template <int EPL> struct Walker {   // EPL = head_dim / 32
     static constexpr int HD = 32 * EPL, HALF = HD / 2;
-    const Args &A;
+    Args A;
     Shm s;
-    unsigned tag = 0, tag_x = 0;   // number of the phase whose output is being written; of the last layer output
-    u64 t_last = 0;
+    u64 t_last;   // thread 0 of CTA 0
 
     __device__ __forceinline__ int lane() const { return threadIdx.x & 31; }
     __device__ __forceinline__ int warp() const { return threadIdx.x >> 5; }
@@ -316,7 +319,7 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
 
     // ---- q, k, v: rotated (q, k), exchanged, and k, v to their cache rows.  A unit is a rotation's pair of features (i, i + hd/2) of a
     // q or k head, or two neighbouring features of v.
-    __device__ __noinline__ void qkv(int l, u64 mask) {
+    __device__ __noinline__ void qkv(int l, u64 mask, unsigned tag_x, unsigned tag) {
         const Ctx &c = A.c;
         const LayerPtrs &w = A.layer[l];
         const int nqk = (c.nq + c.nkv) * HALF, units = nqk + c.nkv * HALF;
@@ -327,7 +330,6 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             }
             return w.wv + (size_t)(2 * (u - nqk) + i) * c.d;
         };
-        ++tag;
         Product<2, decltype(wptr)> p(wptr, c.d, units, mask);
         load_norm(mask, A.XA, tag_x, l, w.attn_norm);
         __syncthreads();
@@ -372,10 +374,9 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
 
     // ---- attention: one (row, q head, 128-position chunk) per CTA at a time, sixteen positions per warp.  Positions of this pass
     // come from the exchanged words, earlier ones from the cache (requested before the queries have arrived).
-    __device__ __noinline__ void attention(int l, u64 mask) {
+    __device__ __noinline__ void attention(int l, u64 mask, unsigned tag) {
         const Ctx &c = A.c;
-        const unsigned want = tag;
-        ++tag;
+        const unsigned want = tag - 1;
         const float *pool = reinterpret_cast<const float *>(c.kv_pool);
         const float scale = rsqrtf((float)HD);
         int total = 0;
@@ -521,13 +522,12 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
     }
 
     // O and down: residual + product, exchanged; the layer's output is also kept (a row may wait at an exit layer)
-    __device__ __noinline__ void o_product(int l, u64 mask) {
+    __device__ __noinline__ void o_product(int l, u64 mask, unsigned tag) {
         const Ctx &c = A.c;
         const float *W = A.layer[l].wo;
         const int K = c.nq * HD;
         auto wptr = [&](int u, int) { return W + (size_t)u * K; };
-        const unsigned want = tag;
-        ++tag;
+        const unsigned want = tag - 1;
         Product<1, decltype(wptr)> p(wptr, K, c.d, mask);
         load_attention(mask, want);
         __syncthreads();
@@ -537,12 +537,11 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         __syncthreads();
         book(5);
     }
-    __device__ __noinline__ void gate_up(int l, u64 mask) {
+    __device__ __noinline__ void gate_up(int l, u64 mask, unsigned tag) {
         const Ctx &c = A.c;
         const LayerPtrs &w = A.layer[l];
         auto wptr = [&](int u, int i) { return (i ? w.wu : w.wg) + (size_t)u * c.d; };
-        const unsigned want = tag;
-        ++tag;
+        const unsigned want = tag - 1;
         Product<2, decltype(wptr)> p(wptr, c.d, c.dff, mask);
         // the rotary factors of the token that this step may emit, by warps that are waiting (their entry's position is complete)
         if (l == 0 && A.pf_n == 0)
@@ -556,12 +555,11 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         __syncthreads();
         book(6);
     }
-    __device__ __noinline__ void down(int l, u64 mask) {
+    __device__ __noinline__ void down(int l, u64 mask, unsigned tag) {
         const Ctx &c = A.c;
         const float *W = A.layer[l].wd;
         auto wptr = [&](int u, int) { return W + (size_t)u * c.dff; };
-        const unsigned want = tag;
-        tag_x = ++tag;
+        const unsigned want = tag - 1;
         Product<1, decltype(wptr)> p(wptr, c.dff, c.d, mask);
         load_words(mask, A.HT, want, c.dff);
         __syncthreads();
@@ -577,7 +575,7 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
 
     // ---- head over the rows of `mask` (layer1: 1-based layer, 0 = final): every CTA's (max, sum exp, argmax) of its vocabulary
     // entries, exchanged, and merged by every CTA alike into st->hr.
-    __device__ __noinline__ void head(int layer1, u64 mask) {
+    __device__ __noinline__ void head(int layer1, u64 mask, unsigned tag_x, unsigned tag) {
         const Ctx &c = A.c;
         const float *T = layer1 > 0 ? A.head_T[layer1] : nullptr;
         const float scale = layer1 > 0 ? A.head_scale[layer1] : 1.0f;
@@ -585,21 +583,18 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         auto wptr = [&](int u, int i) -> const float * { return 2 * u + i < c.vocab ? A.lm_head + (size_t)(2 * u + i) * c.d : nullptr; };
         if (T) {
             auto tptr = [&](int u, int) { return T + (size_t)u * c.d; };
-            ++tag;
             Product<1, decltype(tptr)> p(tptr, c.d, c.d, mask);
             load_norm(mask, A.XA, tag_x, -1, A.final_norm);
             __syncthreads();
             p.run(s.us, A.ku, mask, [&](int n, int r, float (&a)[1]) {
-                if (lane() == 0) put(A.TT + (size_t)r * c.d + n, a[0], tag);
+                if (lane() == 0) put(A.TT + (size_t)r * c.d + n, a[0], tag - 1);
             });
             __syncthreads();
             book(10);
         }
-        const unsigned want = tag;   // of T's output
-        ++tag;
         for (int r = lane(); r < A.R; r += 32) { Msa &m = s.red[warp() * A.R + r]; m.m = -INFINITY; m.s = 0.f; m.i = INT_MAX; }
         Product<2, decltype(wptr)> p(wptr, c.d, n_units, mask);
-        if (T) load_words(mask, A.TT, want, c.d);
+        if (T) load_words(mask, A.TT, tag - 1, c.d);
         else load_norm(mask, A.XA, tag_x, -1, A.final_norm);
         __threadfence();   // what this thread stored plainly in the step is ordered before the partials below
         __syncthreads();
@@ -629,11 +624,11 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             put(o + 1, a.s, tag);
             put(o + 2, __int_as_float(a.i), tag);
         }
-        meet(mask);
+        meet(mask, tag);
         book(9);
     }
     // the partials of all CTAs: one warp per row, lane l merges CTAs l, l + 32, ..., then the lanes by a butterfly
-    __device__ __forceinline__ void meet(u64 mask) {
+    __device__ __forceinline__ void meet(u64 mask, unsigned tag) {
         int i = 0;
         for (u64 m = mask; m; m &= m - 1, ++i) {
             if (i % WARPS != warp()) continue;
@@ -822,12 +817,14 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         st->n_done = ndone;
     }
 
-    __device__ __forceinline__ void layers(int l, u64 mask) {
-        qkv(l, mask);
-        attention(l, mask);
-        o_product(l, mask);
-        gate_up(l, mask);
-        down(l, mask);
+    // the phases tag + 1 .. tag + 5; `tag` becomes the last of them, the layer's output
+    __device__ __forceinline__ void layers(int l, u64 mask, unsigned tag_x, unsigned &tag) {
+        qkv(l, mask, tag_x, tag + 1);
+        attention(l, mask, tag + 2);
+        o_product(l, mask, tag + 3);
+        gate_up(l, mask, tag + 4);
+        down(l, mask, tag + 5);
+        tag += 5;
     }
     __device__ __forceinline__ bool aborted() const { return *(volatile int *)&s.st->abort != 0; }
 
@@ -852,6 +849,7 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             if (pos < st->len[q]) rotary(q * A.cs_ring + (pos & (A.cs_ring - 1)), pos);
         }
         __syncthreads();
+        unsigned tag = 0, tag_x = 0;
         for (long long step = 0; st->n_done < batch; ++step) {
             if (step >= A.max_steps) {   // every step emits or verifies a token
                 if (tid == 0 && blockIdx.x == 0) atomicCAS(A.err, 0, ERR_STEPS);
@@ -873,7 +871,8 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             book(0);
             bool up = true;
             for (int l = 0; l < c.L && up; ++l) {
-                layers(l, active_rows(st, rows, l));
+                layers(l, active_rows(st, rows, l), tag_x, tag);
+                tag_x = tag;
                 if (l + 1 < c.L && A.exit_at[l + 1]) {
                     u64 sel = 0;   // newest rows that may leave early
                     for (int q = 0; q < batch; ++q) {
@@ -881,7 +880,8 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
                         if (st->climbing[q] && slot < A.max_early && st->len[q] < st->target[q]) sel |= 1ull << (q * c.slots + slot);
                     }
                     if (sel) {
-                        head(l + 1, sel);
+                        tag += 2;   // (the first: T's output)
+                        head(l + 1, sel, tag_x, tag);
                         if (tid == 0) exit_control(l + 1);
                         __syncthreads();
                         book(0);
@@ -890,7 +890,8 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
                 }
             }
             if (up) {
-                head(0, active_rows(st, rows, c.L - 1));
+                tag += 2;
+                head(0, active_rows(st, rows, c.L - 1), tag_x, tag);
                 if (tid == 0) verify();
                 __syncthreads();
                 capture();
@@ -913,6 +914,7 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         DevState *g = c.st;
         const int tid = threadIdx.x, sq = A.pf_seq;
         if (tid == 0) st->cap_n = g->capture_n;
+        unsigned tag = 0, tag_x = 0;
         for (int p0 = 0; p0 < A.pf_n; p0 += A.pf_rows) {
             const int n = min(A.pf_rows, A.pf_n - p0);
             const bool last = p0 + n == A.pf_n;
@@ -921,15 +923,19 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             for (int r = tid; r < n; r += THREADS) st->tok[sq][(p0 + r) & (TOK_RING - 1)] = c.tokens[(size_t)sq * c.max_seq + p0 + r];
             for (int r = warp(); r < n; r += WARPS) rotary(r, p0 + r);
             __syncthreads();
-            for (int l = 0; l < c.L; ++l) layers(l, active_rows(st, n, l));
+            for (int l = 0; l < c.L; ++l) {
+                layers(l, active_rows(st, n, l), tag_x, tag);
+                tag_x = tag;
+            }
             if (last) {
-                head(0, 1ull << (n - 1));
+                tag += 2;
+                head(0, 1ull << (n - 1), tag_x, tag);
             } else {   // the next pass reads this one's cache rows
                 __threadfence();
                 __syncthreads();
                 ++tag;
                 if (tid == 0) { u64 *o = A.HP + (size_t)blockIdx.x * A.R * 4; put(o, -INFINITY, tag); put(o + 1, 0.f, tag); put(o + 2, 0.f, tag); }
-                meet(1ull);
+                meet(1ull, tag);
             }
             if (aborted()) break;
         }
@@ -951,25 +957,32 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
     }
 };
 
-template <int EPL> __global__ void __launch_bounds__(THREADS, 1) k_decode_resident(const __grid_constant__ Args A) {
+template <int EPL> __global__ void __launch_bounds__(THREADS, 1) k_decode_resident(const __grid_constant__ Args args) {
     extern __shared__ __align__(16) unsigned char raw[];
-    const Ctx &c = A.c;
-    Walker<EPL> w{A};
-    w.s.freq = reinterpret_cast<double *>(raw);
-    float *f = reinterpret_cast<float *>(raw + sizeof(double) * (c.hd / 2));
-    const int batch = A.batch, n_cs = max(A.R, batch * A.cs_ring);
-    w.s.xs = f; f += (size_t)A.R * c.d;
-    w.s.us = f; f += (size_t)A.R * A.ku;
-    w.s.cs = f; f += (size_t)n_cs * c.hd;
-    w.s.ao = f; f += (size_t)WARPS * (c.hd + 2);
-    w.s.red = reinterpret_cast<Msa *>(f); f += 3 * (size_t)WARPS * A.R;
-    w.s.fill = reinterpret_cast<int *>(f); f += (size_t)batch * c.L;
-    w.s.st = reinterpret_cast<State *>(f);
-    for (int j = threadIdx.x; j < c.hd / 2; j += THREADS) w.s.freq[j] = pow((double)A.rope_base, -2.0 * j / c.hd);
-    if (threadIdx.x == 0) { w.s.st->abort = 0; w.s.st->keep = w.s.st->keep_row = 0; }
+    Walker<EPL> &w = *reinterpret_cast<Walker<EPL> *>(raw);
+    static_assert(sizeof(Args) % 4 == 0, "the arguments are copied by words");
+    for (int i = threadIdx.x; i < (int)(sizeof(Args) / 4); i += THREADS) reinterpret_cast<int *>(&w.A)[i] = reinterpret_cast<const int *>(&args)[i];
+    const Ctx &c = args.c;
+    if (threadIdx.x == 0) {
+        unsigned char *at = raw + walker_bytes(sizeof(Walker<EPL>));
+        w.s.freq = reinterpret_cast<double *>(at);
+        float *f = reinterpret_cast<float *>(at + sizeof(double) * (c.hd / 2));
+        const int batch = args.batch, n_cs = max(args.R, batch * args.cs_ring);
+        w.s.xs = f; f += (size_t)args.R * c.d;
+        w.s.us = f; f += (size_t)args.R * args.ku;
+        w.s.cs = f; f += (size_t)n_cs * c.hd;
+        w.s.ao = f; f += (size_t)WARPS * (c.hd + 2);
+        w.s.red = reinterpret_cast<Msa *>(f); f += 3 * (size_t)WARPS * args.R;
+        w.s.fill = reinterpret_cast<int *>(f); f += (size_t)batch * c.L;
+        w.s.st = reinterpret_cast<State *>(f);
+        w.s.st->abort = 0;
+        w.s.st->keep = w.s.st->keep_row = 0;
+        w.t_last = now();
+    }
     __syncthreads();
-    w.t_last = now();
-    if (A.pf_n > 0) w.prefill();
+    for (int j = threadIdx.x; j < c.hd / 2; j += THREADS) w.s.freq[j] = pow((double)args.rope_base, -2.0 * j / c.hd);
+    __syncthreads();
+    if (args.pf_n > 0) w.prefill();
     else w.decode();
 }
 
