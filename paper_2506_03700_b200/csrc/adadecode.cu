@@ -222,11 +222,10 @@ int resident_rows(const ada_config &g, int batch, int max_early) {
     const int R = rows_alloc_for(g, batch, max_early);
     return max_early + 1 <= rs::MAX_SLOTS && R <= rs::MAX_R ? R : 0;
 }
-constexpr int kResidentMaxGrid = 256;
 // exchanged words: layer input, FFN input, T output, q | k | v, attention partials, FFN activations, head partials
 size_t resident_words(const ada_config &g, int R, int n_chunks) {
     const size_t qkv = (size_t)(g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim, part = (size_t)g.n_q_heads * n_chunks * (g.head_dim + 2);
-    return (size_t)R * (3 * (size_t)g.d_model + qkv + part + g.d_ff) + 4 * (size_t)R * kResidentMaxGrid;
+    return (size_t)R * (3 * (size_t)g.d_model + qkv + part + g.d_ff) + 4 * (size_t)R * rs::MAX_GRID;
 }
 
 Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, int head_blocks) {
@@ -907,7 +906,7 @@ int setup_resident(ada_session *S, const Layout &lay) {
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, rs::THREADS, S->res_smem));
     if (nb < 1) return ADA_OK;
-    S->res_grid = std::min(sms, kResidentMaxGrid);
+    S->res_grid = rs::grid_for(sms, g.d_model);
     rs::Args &a = S->rargs;
     memset(&a, 0, sizeof(a));
     a.tok_embed = (const float *)m->tok_embed;
@@ -933,7 +932,7 @@ int setup_resident(ada_session *S, const Layout &lay) {
     a.QT = take((size_t)R * S->c.qkv_rows);
     a.PT = take((size_t)R * g.n_q_heads * S->n_chunks * (g.head_dim + 2));
     a.HT = take((size_t)R * g.d_ff);
-    a.HP = take(4 * (size_t)R * kResidentMaxGrid);
+    a.HP = take(4 * (size_t)R * rs::MAX_GRID);
     a.err = (int *)((char *)S->scratch + lay.res_err);
     S->resident = true;
     return ADA_OK;
@@ -1785,6 +1784,17 @@ int ada_debug_gemm_plan(int32_t N, int32_t K, int32_t mode, int32_t grid, int32_
     const int tb = p.t0 + p.n - (p.s0_pub_k1 > 0 ? 0 : 1);
     const int32_t v[9] = {p.split, p.split ? 0 : p.t0, p.split ? 0 : p.t0 + p.n, p.split ? p.n : 0, p.split ? p.t0 : 0, p.split ? tb : 0, p.s0_own_k0, p.s0_pub_k1, p.sl_k1};
     memcpy(out9, v, sizeof(v));
+    return ADA_OK;
+}
+
+int ada_debug_resident_plan(const ada_config *cfg, int32_t sms, int32_t cta, int32_t *out5) {
+    if (!cfg || !out5 || sms < 1 || cta < 0) return ADA_EINVAL;
+    const int rc = check_cfg(*cfg);
+    if (rc) return rc;
+    const ada_config &g = *cfg;
+    const int grid = rs::grid_for(sms, g.d_model), units[4] = {(g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim / 2, g.d_model, g.d_ff, g.d_model};
+    out5[0] = grid;
+    for (int i = 0; i < 4; ++i) out5[1 + i] = cta < grid ? rs::units_of(units[i], cta, grid) : 0;
     return ADA_OK;
 }
 

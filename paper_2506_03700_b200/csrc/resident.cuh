@@ -10,10 +10,14 @@
 //     numbers in the same order; CTA 0 also writes them back.  Nobody waits for a decision to be published;
 //   * the weights of a warp's first outputs are in registers before the input they multiply has arrived.
 // Phases of a layer: RMSNorm + q, k, v with rotation | attention partials (row, head, 128-position chunk) | their merge + O +
-// residual | RMSNorm + gate, up, SwiGLU | down + residual.  Every phase's output depends on all CTAs' previous outputs that it
-// reads, so a buffer is written again only after everybody has read it (a layer later).  What has to last longer than a phase
-// (cache rows, the residual of rows that wait at an exit layer, staged logits) is stored plainly and ordered by the exchange of
-// head partials that ends every step: a fence before, a fence after.
+// residual | RMSNorm + gate, up, SwiGLU | down + residual.  A buffer is written again a layer later, and a reader that comes late
+// would not find its phase number any more.  What holds the writers back is the reader's own next output, which they wait for: so
+// every CTA must own an output between each of its reads and the next writing of what it read.  The grid has no more CTAs than the
+// model has features (grid_for): each then owns one of O and one of down in every layer, and one of the two lies in every such
+// interval (XA: read by q, k, v, written by down; XB: gate / up, O; HT: down, gate / up; PT: O, attention; head partials and
+// staged logits: a head, the next one).  What has to last longer than a phase (cache rows, the residual of rows that wait at an
+// exit layer, staged logits) is stored plainly and ordered by the exchange of head partials that ends every step: a fence
+// before, a fence after.
 //
 // Invariance rule as in kernels.cuh: a row's numbers depend on that row's inputs and the launch geometry only.
 //
@@ -78,6 +82,12 @@ __host__ __device__ inline size_t shm_bytes(int R, int d, int ku, int hd, int n_
     return sizeof(float) * ((size_t)R * d + (size_t)R * ku + (size_t)n_cs * hd + (size_t)WARPS * (hd + 2)) + sizeof(Msa) * WARPS * (size_t)R +
            sizeof(int) * (size_t)batch * L + sizeof(State) + sizeof(double) * (hd / 2) + walker_bytes(sizeof(Args) + sizeof(Shm) + sizeof(u64)) + 64;
 }
+
+// CTAs of a launch on a device of `sms` SMs (see above why no more than d), and the units of a product of `units` that CTA `cta` of
+// them works on: unit u is warp u / grid's of CTA u mod grid (Product).
+constexpr int MAX_GRID = 256;
+__host__ __device__ constexpr int grid_for(int sms, int d) { return sms < MAX_GRID ? (sms < d ? sms : d) : (MAX_GRID < d ? MAX_GRID : d); }
+__host__ __device__ constexpr int units_of(int units, int cta, int grid) { return units > cta ? (units - cta + grid - 1) / grid : 0; }
 
 __device__ __forceinline__ int popc64(u64 m) { return __popcll(m); }
 __device__ __forceinline__ u64 now() { u64 t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }

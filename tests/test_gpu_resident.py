@@ -24,8 +24,10 @@ def decode(gm, cfg, prompts, n, early, max_early, mode):
 
 
 # (q heads, kv heads, head_dim, width, d_ff, vocabulary): one and several 16-byte pieces per lane, ragged ones, rows of 768
-# elements and more (the weights of a row in several pieces; prompt passes of fewer rows), an odd vocabulary
-SHAPES = [(4, 4, 64, 256, 688, 2048), (6, 2, 32, 192, 328, 1001), (2, 1, 128, 256, 800, 515), (4, 1, 32, 1032, 136, 300)]
+# elements and more (the weights of a row in several pieces; prompt passes of fewer rows), an odd vocabulary; narrower than the
+# GPU has SMs
+SHAPES = [(4, 4, 64, 256, 688, 2048), (6, 2, 32, 192, 328, 1001), (2, 1, 128, 256, 800, 515), (4, 1, 32, 1032, 136, 300),
+          (4, 2, 32, 128, 344, 1024), (2, 2, 32, 64, 128, 600), (1, 1, 32, 24, 40, 256)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
