@@ -615,7 +615,7 @@ __global__ void k_head_final(Ctx c, int n_blocks, int sel) {
         a = msa_merge(a, x);
     }
     if (lane == 0) {
-        HeadResult hr; hr.token = a.i; hr.zmax = a.m; hr.sumexp = a.s; hr.p = 1.0f / a.s;
+        HeadResult hr; hr.token = min(a.i, c.vocab - 1); hr.zmax = a.m; hr.sumexp = a.s; hr.p = 1.0f / a.s;   // (no logit is a number: no argmax)
         c.head_res[r] = hr;
     }
 }

@@ -679,7 +679,8 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             }
             if (lane() == 0) {
                 HeadResult hr;
-                hr.token = a.i; hr.zmax = a.m; hr.sumexp = a.s; hr.p = 1.0f / a.s;
+                hr.token = min(a.i, A.c.vocab - 1);   // (no logit is a number: no argmax)
+                hr.zmax = a.m; hr.sumexp = a.s; hr.p = 1.0f / a.s;
                 s.st->hr[r] = hr;
                 if (blockIdx.x == 0) A.c.head_res[r] = hr;
             }
@@ -951,9 +952,9 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         }
         if (tid == 0) {
             const int n_last = (A.pf_n - 1) % A.pf_rows;
+            set_token(sq, A.pf_n, st->hr[n_last].token);
             if (blockIdx.x == 0) {
                 for (int l = 0; l < c.L; ++l) c.fill[sq * c.L + l] = A.pf_n;
-                c.tokens[(size_t)sq * c.max_seq + A.pf_n] = st->hr[n_last].token;
                 g->base[sq] = A.pf_n;
                 g->len[sq] = A.pf_n + 1;
                 g->n_prompt[sq] = A.pf_n;

@@ -58,3 +58,23 @@ def test_one_launch_equals_the_per_operation_path(shape, lens, early, mode):
     assert np.array_equal(out[0][:stop], ref[0][:stop])
     for s in range(1, len(lens)):   # the other sequences' logits are not kept: their tokens
         assert np.array_equal(out[s], ref[s])
+
+
+# fp32 in one launch; fp32 and bf16 in one launch per operation (room for sixteen early tokens; 96 features a head); the bf16 kernel
+@pytest.mark.parametrize("dtype,hd,max_early", [("fp32", 64, 5), ("fp32", 64, 16), ("bf16", 96, 5), ("bf16", 64, 5)])
+def test_tokens_stay_in_the_vocabulary_where_no_logit_is_a_number(dtype, hd, max_early):
+    """The argmax of logits that are all NaN is none; what is emitted, and read back as an embedding row, is a token all the same,
+    the one after the prompt included."""
+    cfg = synth.small_config(dtype=dtype, n_layers=3, d_model=256, n_q_heads=2, n_kv_heads=1, head_dim=hd, d_ff=320, vocab=500,
+                             exit_layers=(1, 2))
+    w = synth.make_weights(cfg, device="cuda", tied=False)
+    w["lm_head"].fill_(float("nan"))
+    gm = binding.Model(cfg, w)
+    for l in cfg.exit_layers:
+        gm.set_exit_head(l, None, 4.0)
+    S = binding.Session(gm, 2, 64, 64, max_early)
+    for mode in ("plain", "adaptive"):
+        for i, n in enumerate((5, 12)):
+            S.prefill(synth.make_prompt(cfg, n=n, seq=i).numpy(), seq=i)
+        out = S.plain_decode(6) if mode == "plain" else S.adaptive_decode(6, 0.1, cfg.exit_layers, 5)
+        assert out.min() >= 0 and out.max() < cfg.vocab
