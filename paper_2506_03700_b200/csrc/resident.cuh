@@ -148,23 +148,26 @@ template <int NW, class Ptr> __device__ __forceinline__ void load_w(Wreg<NW> &r,
     }
 }
 // A product of `units` units (NW weight rows each) over the rows in `mask`: units are dealt to the warps of the grid, groups of
-// eight rows apart where there are more.  Before the input has arrived: the constructor loads the first unit's weights.  Then
-// run(): out(unit, row, sums) by the whole warp.
+// eight rows apart where there are more.  `same_warp`: a unit belongs to the same warp in every group.  (The head needs it: a warp
+// folds its units' exponentials before they meet the others', and a row's group depends on how many rows are in front of it.)
+// Before the input has arrived: the constructor loads the first unit's weights.  Then run(): out(unit, row, sums) by the whole warp.
 template <int NW, class Ptr> struct Product {
     const Ptr &wptr;
-    int K, units, groups, first, stride;
+    int K, units, groups, first, stride, pitch;   // item unit + pitch * group is item / stride's of warp item % stride
     Wreg<NW> r;
-    __device__ __forceinline__ Product(const Ptr &p, int K_, int units_, u64 mask)
+    __device__ __forceinline__ Product(const Ptr &p, int K_, int units_, u64 mask, bool same_warp = false)
         : wptr(p), K(K_), units(units_), groups((popc64(mask) + 7) >> 3), first((int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x), stride(WARPS * (int)gridDim.x) {
-        if (first < units * groups) load_w<NW>(r, wptr, first % units, K, 0);
+        pitch = same_warp ? (units + stride - 1) / stride * stride : units;
+        if (first < pitch * groups && first % pitch < units) load_w<NW>(r, wptr, first % pitch, K, 0);
     }
     // Two rows at a time; a weight row of up to 128 U elements is loaded once for all rows of the group.
     template <class Out> __device__ __forceinline__ void run(const float *us, int ldu, u64 mask, Out &&out) {
         const int lane = threadIdx.x & 31, nch = K / 4;
         int at = 0;   // piece of the unit's weights in registers
 #pragma unroll 1
-        for (int wk = first; wk < units * groups; wk += stride) {
-            const int unit = wk % units, grp = wk / units;
+        for (int wk = first; wk < pitch * groups; wk += stride) {
+            const int unit = wk % pitch, grp = wk / pitch;
+            if (unit >= units) continue;
             u64 m = mask;
             for (int i = 0; i < 8 * grp; ++i) m &= m - 1;
             if (wk != first) at = -1;
@@ -603,7 +606,7 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
             book(10);
         }
         for (int r = lane(); r < A.R; r += 32) { Msa &m = s.red[warp() * A.R + r]; m.m = -INFINITY; m.s = 0.f; m.i = INT_MAX; }
-        Product<2, decltype(wptr)> p(wptr, c.d, n_units, mask);
+        Product<2, decltype(wptr)> p(wptr, c.d, n_units, mask, true);
         if (T) load_words(mask, A.TT, tag - 1, c.d);
         else load_norm(mask, A.XA, tag_x, -1, A.final_norm);
         __threadfence();   // what this thread stored plainly in the step is ordered before the partials below

@@ -78,3 +78,30 @@ def test_tokens_stay_in_the_vocabulary_where_no_logit_is_a_number(dtype, hd, max
             S.prefill(synth.make_prompt(cfg, n=n, seq=i).numpy(), seq=i)
         out = S.plain_decode(6) if mode == "plain" else S.adaptive_decode(6, 0.1, cfg.exit_layers, 5)
         assert out.min() >= 0 and out.max() < cfg.vocab
+
+
+@pytest.mark.parametrize("batch,max_early", [(16, 2), (9, 4)])
+def test_heads_over_more_than_eight_rows_give_each_sequence_its_own_bits(batch, max_early):
+    """More than eight newest tokens at an intermediate head: a row's probability does not depend on its company.  (Without early
+    exits every step evaluates every sequence at every exit layer; the log holds them in that order.)"""
+    cfg = synth.small_config(n_layers=4, d_model=256, n_q_heads=4, n_kv_heads=4, head_dim=64, d_ff=688, vocab=2048, sigma=0.08,
+                             resid_scale=0.5, exit_layers=(1, 3))
+    gm = binding.Model(cfg, synth.make_weights(cfg, device="cuda", norm_gain_jitter=0.2))
+    for l in cfg.exit_layers:
+        gm.set_exit_head(l, None, 4.0)
+    prompts = [synth.make_prompt(cfg, n=5 + i, seq=i).numpy() for i in range(batch)]
+
+    def run(ps):
+        S = binding.Session(gm, len(ps), 64, 16, max_early)
+        S.capture_heads()
+        for i, p in enumerate(ps):
+            S.prefill(p, seq=i)
+        out = S.adaptive_decode(20, 2.0, cfg.exit_layers, max_early)
+        return out, S.captured_heads()[:, 2:].reshape(-1, len(ps), 2).copy()   # (token, p) by step and layer, sequence
+
+    out, log = run(prompts)
+    assert len(log) >= 30
+    for i, p in enumerate(prompts):
+        o, l = run([p])
+        assert np.array_equal(o[0], out[i])
+        assert np.array_equal(l[:, 0], log[:, i]), i
