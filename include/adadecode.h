@@ -256,10 +256,12 @@ int ada_debug_trace(ada_session *s, uint64_t *dev_buf, uint32_t *count_dev, uint
  * A k chunk is 512 wide.  No GPU is touched.  ADA_EINVAL on bad arguments. */
 int ada_debug_gemm_plan(int32_t N, int32_t K, int32_t mode, int32_t grid, int32_t cta, int32_t split, int32_t *out9);
 
-/* Host-only: the grid that the one-launch path of fp32 models takes for a model on a device of `sms` multiprocessors, and what CTA
- * `cta` of it works on in every layer.  out5 (host) receives {CTAs of the grid, units of q | k | v (two features each), of the
- * O product, of gate / up and of down (one)}; the units are 0 for a cta outside the grid.  No GPU is touched.  ADA_EINVAL on bad arguments. */
-int ada_debug_resident_plan(const ada_config *cfg, int32_t sms, int32_t cta, int32_t *out5);
+/* Host-only: whether the calls of a session of this model, batch and max_early run in one launch (fp32 models; shape and measured
+ * speed decide), the grid that launch takes on a device of `sms` multiprocessors, and what CTA `cta` of it works on in every layer.
+ * out7 (host) receives {most rows of a pass (0: one kernel per operation), whether prompts take it too, CTAs of the grid, units of
+ * q | k | v (two features each), of the O product, of gate / up and of down (one)}; the units are 0 for a cta outside the grid.  No
+ * GPU is touched.  ADA_EINVAL on bad arguments. */
+int ada_debug_resident_plan(const ada_config *cfg, int32_t batch, int32_t max_early, int32_t sms, int32_t cta, int32_t *out7);
 
 /* Run the weight-streaming skinny GEMM of the decode kernel by itself (the kernel behind the QKV,
  * O, gate/up, down and LM-head products of a layer pass, Algorithm 1 "process all tokens in P[l]

@@ -130,7 +130,7 @@ def load() -> C.CDLL:
         L.ada_gemm_noalloc.argtypes = [vp, i32, i32, i32, vp, i32, vp, i32, vp]
         L.ada_debug_profile.argtypes = [vp, i32]
         L.ada_debug_profile_read.argtypes = [vp, vp, vp, vp]
-        L.ada_debug_resident_plan.argtypes = [C.POINTER(Config), i32, i32, C.POINTER(i32)]
+        L.ada_debug_resident_plan.argtypes = [C.POINTER(Config), i32, i32, i32, i32, C.POINTER(i32)]
         L.ada_debug_gemm_plan.argtypes = [i32, i32, i32, i32, i32, i32, C.POINTER(i32)]
         L.ada_debug_gemm_work_bytes.restype = sz
         L.ada_debug_gemm_work_bytes.argtypes = [i32]
@@ -152,12 +152,14 @@ def debug_gemm_plan(N: int, K: int, mode: int, grid: int, cta: int, split: bool 
     return dict(zip(keys, list(out)))
 
 
-def debug_resident_plan(cfg, sms: int, cta: int) -> dict:
-    """ada_debug_resident_plan: grid of the fp32 one-launch path and the units of CTA `cta` in every layer (host only, no GPU)."""
-    c = Config(cfg.n_layers, cfg.d_model, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.d_ff, cfg.vocab, 0, 1, cfg.rope_base, cfg.rms_eps)
-    out = (C.c_int32 * 5)()
-    _ck(load().ada_debug_resident_plan(C.byref(c), sms, cta, out), "ada_debug_resident_plan")
-    return dict(zip(("grid", "qkv", "o", "gate_up", "down"), list(out)))
+def debug_resident_plan(cfg, batch: int = 1, max_early: int = 5, sms: int = 148, cta: int = 0) -> dict:
+    """ada_debug_resident_plan: rows of a pass of the fp32 one-launch path (0: not taken), whether prompts take it, its grid and the
+    units of CTA `cta` in every layer (host only, no GPU)."""
+    c = Config(cfg.n_layers, cfg.d_model, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.d_ff, cfg.vocab, 1 if cfg.dtype == "bf16" else 0, 1,
+               cfg.rope_base, cfg.rms_eps)
+    out = (C.c_int32 * 7)()
+    _ck(load().ada_debug_resident_plan(C.byref(c), batch, max_early, sms, cta, out), "ada_debug_resident_plan")
+    return dict(zip(("rows", "prompts", "grid", "qkv", "o", "gate_up", "down"), list(out)))
 
 
 def debug_dense_plan(rows: int, N: int, per_tile: int, K: int, pairs: int, pair: int):

@@ -152,7 +152,7 @@ struct ada_session {
     bool sampling = false;   // the call in progress draws its tokens (ada_sampling_decode)
     float inv_temp = 1.0f;
     // fp32 models whose rows fit: whole calls in one launch (resident.cuh)
-    bool resident = false;
+    bool resident = false, res_prompts = false;   // decode calls; prompts
     size_t res_smem = 0, res_words = 0;      // shared memory of a CTA; bytes of the exchanged words
     int res_grid = 0;
     rs::Args rargs;
@@ -215,12 +215,44 @@ size_t attn_tag_bytes(const ada_config &g, int n_chunks) {
     return model_fits_persistent(g) ? sizeof(unsigned long long) * st3::MAX_COLS * g.n_q_heads * (size_t)n_chunks * (g.head_dim + 2) : 0;
 }
 
-// Whether an fp32 model's calls can run in one launch (resident.cuh): most rows of its passes, or 0.  The bounds are those of the
-// kernel's tables; that the rows fit the shared memory is asked of the device when the session is created.
-int resident_rows(const ada_config &g, int batch, int max_early) {
-    if (g.dtype != ADA_DTYPE_FP32 || g.n_layers >= rs::MAX_L || (g.head_dim != 32 && g.head_dim != 64 && g.head_dim != 128)) return 0;
-    const int R = rows_alloc_for(g, batch, max_early);
-    return max_early + 1 <= rs::MAX_SLOTS && R <= rs::MAX_R ? R : 0;
+// How the calls of an fp32 session run in one launch (resident.cuh).
+struct ResidentFit {
+    int rows = 0;            // most rows of a pass (0: one kernel per operation)
+    bool prompts = false;    // prompts too
+    int ku = 0, ring = 0;    // widest product input; rotary factors kept per sequence
+    size_t smem = 0;         // shared memory of a CTA
+};
+constexpr size_t kSharedMax = 232448;   // 227 KB: most shared memory of a block on sm_100
+// A phase of the one-launch kernel costs an exchange through L2 where the per-operation kernels cost a launch; its products read
+// their inputs from shared memory, two rows at a time, and its head's entries come one pair per warp after the other, where theirs
+// hold eight rows in registers and four entries in flight.  So it is taken where the layers' latency outweighs both; measured
+// against one kernel per operation, times of decode calls (plain, and adaptive with everything and little accepted):
+//   rows of a step, by the widest input: any number up to 896 (d_model 64 .. 320: 0.49 .. 0.94; sixteen sequences of width 256
+//     0.94), three up to 1024 (width 384: 0.67 .. 0.89; eight 0.98 .. 1.10), two up to 2048 (width 512: 0.62 .. 0.94, 768: 0.92 .. 1.00;
+//     three 0.88 .. 1.05), one up to 3584 (width 1024: 0.71 .. 0.91, 1408: 0.93 .. 0.96; two 0.73 .. 1.05);
+//   weights of the head per layer: 2^21 (width 256, four layers: vocabulary 32000 0.69, 64000 1.02; width 512 8192 0.88, 32000 1.06),
+//     from four sequences on 2^19 (width 256, eight sequences: 8192 0.90, 16384 0.95, 32000 1.07).
+// Prompts go 32 rows a pass in both, and the longer the prompt the more its products count: widths up to 768 with small heads only
+// (width 64 .. 192 0.71 .. 0.99; width 256: one token 0.82, eight 1.06, sixteen 1.00, 64 0.89, 500 0.91; a d_ff of 2816 1.15, width 512 1.3).
+ResidentFit resident_fit(const ada_config &g, int batch, int max_early) {
+    ResidentFit f;
+    if (g.dtype != ADA_DTYPE_FP32 || g.n_layers >= rs::MAX_L || (g.head_dim != 32 && g.head_dim != 64 && g.head_dim != 128)) return f;
+    if (max_early + 1 > rs::MAX_SLOTS || batch * (max_early + 1) > rs::MAX_R) return f;
+    f.ku = std::max({g.d_model, g.n_q_heads * g.head_dim, g.d_ff});
+    const long long head = (long long)g.vocab * g.d_model / g.n_layers;
+    const int most = f.ku <= 896 ? rs::MAX_R : f.ku <= 1024 ? 3 : f.ku <= 2048 ? 2 : f.ku <= 3584 ? 1 : 0;
+    if (batch > most || head > (batch > 3 ? 1 << 19 : 1 << 21)) return f;
+    f.prompts = f.ku <= 768 && head <= 1 << 18;
+    f.ring = 2;
+    while (f.ring < max_early + 2) f.ring *= 2;
+    // a prompt pass takes fewer rows where that is what fits (a row is d_model + ku floats of shared memory)
+    const int need = std::max(batch * (max_early + 1), 8);
+    for (int R = f.prompts ? rows_alloc_for(g, batch, max_early) : need;; R -= 8) {
+        R = std::max(R, need);
+        f.smem = rs::shm_bytes(R, g.d_model, f.ku, g.head_dim, std::max(R, batch * f.ring), batch, g.n_layers);
+        if (f.smem <= kSharedMax) f.rows = R;
+        if (f.rows || R == need) return f;
+    }
 }
 // exchanged words: layer input, FFN input, T output, q | k | v, attention partials, FFN activations, head partials
 size_t resident_words(const ada_config &g, int R, int n_chunks) {
@@ -267,8 +299,8 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.pf_err = take(256);
         L.pf_flag = take(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS);
     }
-    if (resident_rows(g, batch, max_early) > 0) {
-        L.res = take(resident_words(g, R, n_chunks) * sizeof(rs::u64));
+    if (const int rows = resident_fit(g, batch, max_early).rows) {
+        L.res = take(resident_words(g, rows, n_chunks) * sizeof(rs::u64));
         L.res_err = take(256);
     }
     // persistent-kernel buffers (bf16 models)
@@ -878,29 +910,21 @@ int setup_resident(ada_session *S, const Layout &lay) {
     const ada_model *m = S->m;
     const ada_config &g = m->cfg;
     S->resident = false;
-    int R = resident_rows(g, S->batch, S->max_early);
+    const ResidentFit fit = resident_fit(g, S->batch, S->max_early);
+    const int R = fit.rows;
     if (R == 0) return ADA_OK;
     // embeddings and gains are read eight bytes at a time, weight rows sixteen (as the per-operation kernels do)
     auto aligned = [](const void *p, size_t a) { return (uintptr_t)p % a == 0; };
     bool ok = aligned(m->tok_embed, 8) && aligned(m->final_norm, 8);
     for (const LayerW &w : m->layers) ok = ok && aligned(w.attn_norm, 8) && aligned(w.ffn_norm, 8);
     if (!ok) return ADA_OK;
-    const int qd = g.n_q_heads * g.head_dim, ku = std::max(std::max(g.d_model, qd), g.d_ff);
-    int ring = 2;
-    while (ring < S->slots + 1) ring *= 2;
     int dev = 0, sms = 0, coop = 0, smem = 0, nb = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     CK(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    // a prompt pass takes fewer rows where that is what fits (a row is d_model + ku floats of shared memory)
-    const int need = std::max(S->batch * S->slots, 8);
-    for (;; R -= 8) {
-        if (R < need) R = need;
-        S->res_smem = rs::shm_bytes(R, g.d_model, ku, g.head_dim, std::max(R, S->batch * ring), S->batch, g.n_layers);
-        if (S->res_smem <= (size_t)smem) break;
-        if (R == need) return ADA_OK;
-    }
+    S->res_smem = fit.smem;
+    if (fit.smem > (size_t)smem) return ADA_OK;
     if (!coop) return ADA_OK;
     const void *kern = resident_kernel(g.head_dim);
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -920,8 +944,8 @@ int setup_resident(ada_session *S, const Layout &lay) {
     a.rope_base = g.rope_base;
     a.batch = S->batch;
     a.R = R;
-    a.ku = ku;
-    a.cs_ring = ring;
+    a.ku = fit.ku;
+    a.cs_ring = fit.ring;
     a.pf_rows = std::min(R, rs::TOK_RING);
     S->res_words = resident_words(g, R, S->n_chunks) * sizeof(rs::u64);
     rs::u64 *w = (rs::u64 *)((char *)S->scratch + lay.res);
@@ -935,6 +959,7 @@ int setup_resident(ada_session *S, const Layout &lay) {
     a.HP = take(4 * (size_t)R * rs::MAX_GRID);
     a.err = (int *)((char *)S->scratch + lay.res_err);
     S->resident = true;
+    S->res_prompts = fit.prompts;
     return ADA_OK;
 }
 
@@ -1100,7 +1125,9 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
     if (S->mega && S->path == 1) {
         if ((rc = run_persistent(S, exit_layers, n_exit, plain, 0, S->batch, true))) return rc;
     } else if (S->resident) {
-        if ((rc = run_resident(S, 0, 0, exit_layers, plain ? 0 : n_exit, gamma, max_early, eos_id, tape_n, n_tokens))) return rc;
+        // (the token after a prompt is there already: a call for it alone has no step to run)
+        if (max_steps_plain > 0 && (rc = run_resident(S, 0, 0, exit_layers, plain ? 0 : n_exit, gamma, max_early, eos_id, tape_n, n_tokens)))
+            return rc;
     } else if (plain) {
         // every step is one token through all layers; the step count is known, no read-back needed
         for (int it = 0; it < max_steps_plain; ++it) {
@@ -1577,7 +1604,7 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         S->h_reported[seq] = 0;
         return ADA_OK;
     }
-    if (S->resident) {
+    if (S->resident && S->res_prompts) {
         if ((rc = run_resident(S, seq, n_prompt, nullptr, 0, 2.0f, 0, -1, 0, 0))) return rc;
         S->prefilled[seq] = 1;
         S->h_prompt[seq] = n_prompt;
@@ -1787,14 +1814,17 @@ int ada_debug_gemm_plan(int32_t N, int32_t K, int32_t mode, int32_t grid, int32_
     return ADA_OK;
 }
 
-int ada_debug_resident_plan(const ada_config *cfg, int32_t sms, int32_t cta, int32_t *out5) {
-    if (!cfg || !out5 || sms < 1 || cta < 0) return ADA_EINVAL;
+int ada_debug_resident_plan(const ada_config *cfg, int32_t batch, int32_t max_early, int32_t sms, int32_t cta, int32_t *out7) {
+    if (!cfg || !out7 || batch < 1 || max_early < 0 || sms < 1 || cta < 0) return ADA_EINVAL;
     const int rc = check_cfg(*cfg);
     if (rc) return rc;
     const ada_config &g = *cfg;
     const int grid = rs::grid_for(sms, g.d_model), units[4] = {(g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim / 2, g.d_model, g.d_ff, g.d_model};
-    out5[0] = grid;
-    for (int i = 0; i < 4; ++i) out5[1 + i] = cta < grid ? rs::units_of(units[i], cta, grid) : 0;
+    const ResidentFit fit = resident_fit(g, batch, max_early);
+    out7[0] = fit.rows;
+    out7[1] = fit.rows > 0 && fit.prompts;
+    out7[2] = grid;
+    for (int i = 0; i < 4; ++i) out7[3 + i] = cta < grid ? rs::units_of(units[i], cta, grid) : 0;
     return ADA_OK;
 }
 
