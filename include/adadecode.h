@@ -238,6 +238,9 @@ int ada_debug_set_launch_steps(ada_session *s, int32_t steps);
  * usable again.  A limit shorter than a grid-wide wait normally lasts (a few microseconds) makes the
  * next decode call time out: that is how the give-up path is tested. */
 int ada_debug_set_wait_limit(ada_session *s, uint64_t ns);
+
+/* Bytes of attention chunk partials that the session's last prompt or decode call cleared before its launches (host counter). */
+int ada_debug_cleared_bytes(ada_session *s, int64_t *bytes_out);
 /* Event trace of the persistent kernel: while the kernel runs the steps [step0, step1) of a launch
  * (counted from 0 in every launch), every CTA appends (nanosecond timestamp, code) pairs of
  * uint64 to its own region of dev_buf [SMs][cap_events][2]; code = CTA << 32 | argument << 8 | event (1 phase begin, 2

@@ -34,7 +34,7 @@ EXPORTS = [
     "ada_model_arena_bytes", "ada_model_set_arena", "ada_debug_set_wait_limit", "ada_debug_set_prefill",
     "ada_debug_dense_gemm", "ada_debug_dense_gemm_work_bytes", "ada_sampling_decode",
     "ada_debug_dense_plan", "ada_debug_dense_product", "ada_debug_dense_product_work_bytes",
-    "ada_debug_resident_plan",
+    "ada_debug_resident_plan", "ada_debug_cleared_bytes",
 ]
 
 
@@ -95,6 +95,7 @@ def load() -> C.CDLL:
         L.ada_model_arena_bytes.argtypes = [vp]
         L.ada_model_set_arena.argtypes = [vp, vp, sz]
         L.ada_debug_set_wait_limit.argtypes = [vp, C.c_uint64]
+        L.ada_debug_cleared_bytes.argtypes = [vp, C.POINTER(C.c_int64)]
         L.ada_debug_set_prefill.argtypes = [vp, i32]
         L.ada_debug_dense_gemm_work_bytes.restype = sz
         L.ada_debug_dense_gemm_work_bytes.argtypes = [i32]
@@ -426,6 +427,11 @@ class Session:
 
     def set_wait_limit(self, ns: int):
         _ck(load().ada_debug_set_wait_limit(self.h, ns), "ada_debug_set_wait_limit")
+
+    def cleared_bytes(self) -> int:
+        n = C.c_int64(0)
+        _ck(load().ada_debug_cleared_bytes(self.h, C.byref(n)), "ada_debug_cleared_bytes")
+        return n.value
 
     def trace(self, cap_events: int, step0: int, step1: int):
         """Record the persistent kernel's events of steps [step0, step1) of every following launch

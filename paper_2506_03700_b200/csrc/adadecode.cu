@@ -171,6 +171,7 @@ struct ada_session {
     int pf_kv_box = 0;                         // positions one copy of it covers
     bool prefill_dense = true;                 // ada_debug_set_prefill
     int64_t launches = 0, syncs = 0, layer_passes = 0;
+    int64_t cleared = 0;                       // bytes of attention partials that the last prompt or decode call cleared
     // per-class profiling
     bool prof = false;
     std::vector<cudaEvent_t> prof_ev;
@@ -208,6 +209,8 @@ constexpr int kDenseMin = 9;        // prompt tokens from which the dense pass i
 // exchange area of weight tiles split between two CTAs: 8 k-splits x 256 tagged words per CTA
 constexpr size_t kPartBytesPerCta = (size_t)st::CONS_WARPS * 256 * sizeof(unsigned long long);
 constexpr int kPartMaxGrid = 256;
+
+int chunks_of(int positions) { return (positions + kAttnChunk - 1) / kAttnChunk; }
 
 // Chunk partials of the decode attention: as floats for the per-operation kernels, as tagged words (see attn_consume) for the
 // persistent kernel, in the same memory (a session uses one path at a time, and the words are cleared before each launch).
@@ -264,7 +267,7 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
     Layout L{};
     const int R = rows_alloc_for(g, batch, max_early);
     const int qd = g.n_q_heads * g.head_dim, qkv_rows = (g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim;
-    const int n_chunks = (max_seq + kAttnChunk - 1) / kAttnChunk;
+    const int n_chunks = chunks_of(max_seq);
     const int max_pages = (max_seq + 15) / 16;  // upper bound for any page size >= 16
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
@@ -1011,7 +1014,10 @@ int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layer
 // three launches or more: one stream of the weights for what took as many streams as launches (13B, four sequences with five early
 // tokens, 16 tokens each: 319 -> 188 ms with their prompts).  Two launches of several sequences each stay with eight columns, whose
 // rings are deeper.
-int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool plain, int seq_begin, int seq_end, bool together) {
+//
+// `reach`: positions of the longest sequence at the end of the call.  The attention's chunk partials are laid out, and cleared, for as
+// many (laid out for the session's length, a call of a few tokens in an 8B session of 131072 positions cleared 273 MB: 50 us).
+int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool plain, int seq_begin, int seq_end, bool together, int reach) {
     const ada_model *m = S->m;
     const ada_config &g = m->cfg;
     const int L = g.n_layers;
@@ -1039,10 +1045,12 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
     const int per_launch = !together ? 1 : wide ? std::min((int)st3::MAX_SEQS, st3::MAX_COLS / S->slots) : narrow;
     const void *kern = persistent_kernel_for(g.head_dim, wide);
     const size_t part_bytes = kPartBytesPerCta * (size_t)S->grid * (wide ? st3::TILES : 1);
-    const size_t tag_bytes = attn_tag_bytes(g, S->n_chunks) / st3::MAX_COLS * (wide ? st3::MAX_COLS : st::MAX_COLS);
+    const int chunks = chunks_of(reach);
+    const size_t tag_bytes = attn_tag_bytes(g, chunks) / st3::MAX_COLS * (wide ? st3::MAX_COLS : st::MAX_COLS);
     for (int sq = seq_begin; sq < seq_end; sq += per_launch) {
         MegaArgs a = S->margs;
         a.c = S->c;   // capture pointers may have changed
+        a.c.n_chunks = chunks;
         if (wide) {
             const auto behind = [](__nv_bfloat16 *&p, int K) { p = (__nv_bfloat16 *)((char *)p + st::xfrag_bytes(K)); };
             for (__nv_bfloat16 **p : {&a.XA, &a.XB, &a.XF, &a.XT}) behind(*p, g.d_model);
@@ -1063,6 +1071,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             CK(cudaMemsetAsync(a.pub, 0, sizeof(mg3::Pub) * 2, S->stream));
             if (a.part) CK(cudaMemsetAsync(a.part, 0, part_bytes, S->stream));
             CK(cudaMemsetAsync(a.attn_tag, 0, tag_bytes, S->stream));   // phase numbers start over with every launch
+            S->cleared += (int64_t)tag_bytes;
             void *params[] = {(void *)&a};
             CK(cudaLaunchCooperativeKernel(kern, dim3(S->grid), dim3(mg::MEGA_THREADS), params, wide ? st3::SMEM_BYTES : st::SMEM_BYTES, S->stream));
             S->launches++;
@@ -1100,7 +1109,8 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
     }
     CallTargets tg;
     memset(&tg, 0, sizeof(tg));
-    int max_steps_plain = 0;
+    int max_steps_plain = 0, reach = 0;
+    S->cleared = 0;
     for (int s = 0; s < S->batch; ++s) {
         int target = S->h_prompt[s] + S->h_reported[s] + (S->finished[s] ? 0 : n_tokens);
         if (target + 1 > S->max_seq) return ADA_ECAPACITY;
@@ -1108,6 +1118,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
         if (rc) return rc;
         tg.target_len[s] = target;
         max_steps_plain = std::max(max_steps_plain, target - S->h_len[s]);
+        reach = std::max(reach, target);
     }
     const int64_t l0 = S->launches, s0 = S->syncs, p0 = S->layer_passes;
     const int rows = S->batch * S->slots;
@@ -1123,7 +1134,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
 
     const bool plain = (n_exit == 0 || max_early == 0);
     if (S->mega && S->path == 1) {
-        if ((rc = run_persistent(S, exit_layers, n_exit, plain, 0, S->batch, true))) return rc;
+        if ((rc = run_persistent(S, exit_layers, n_exit, plain, 0, S->batch, true, reach))) return rc;
     } else if (S->resident) {
         // (the token after a prompt is there already: a call for it alone has no step to run)
         if (max_steps_plain > 0 && (rc = run_resident(S, 0, 0, exit_layers, plain ? 0 : n_exit, gamma, max_early, eos_id, tape_n, n_tokens)))
@@ -1436,7 +1447,7 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
     S->rows_alloc = rows_alloc_for(g, batch, max_early);
     S->n_pages = n_pages;
     S->max_pages = (max_seq_len + 15) / 16;
-    S->n_chunks = (max_seq_len + kAttnChunk - 1) / kAttnChunk;
+    S->n_chunks = chunks_of(max_seq_len);
     S->head_blocks = kHeadBlocks;
     S->stream = (cudaStream_t)cuda_stream;
     S->scratch = scratch_dev;
@@ -1573,6 +1584,7 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
     for (int i = 0; i < n_prompt; ++i) if (prompt_host[i] < 0 || prompt_host[i] >= g.vocab) return ADA_EINVAL;
     int rc = ada_session_reset(S, seq);
     if (rc) return rc;
+    S->cleared = 0;
     if ((rc = ensure_pages(S, seq, n_prompt + 1))) return rc;
     CK(cudaMemcpyAsync(S->c.tokens + (size_t)seq * S->max_seq, prompt_host, sizeof(int32_t) * n_prompt,
                        cudaMemcpyHostToDevice, S->stream));
@@ -1589,7 +1601,7 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         // prompt passes of eight positions through the persistent kernel
         mg::k_prefill_arm<<<1, 32, 0, S->stream>>>(S->c, seq, n_prompt);
         CK(cudaGetLastError());
-        if ((rc = run_persistent(S, nullptr, 0, true, seq, seq + 1, false))) return rc;
+        if ((rc = run_persistent(S, nullptr, 0, true, seq, seq + 1, false, n_prompt))) return rc;
         S->prefilled[seq] = 1;
         S->h_prompt[seq] = n_prompt;
         S->h_len[seq] = n_prompt + 1;
@@ -1673,6 +1685,12 @@ int ada_sampling_decode(ada_session *S, int32_t n_tokens, float temperature, flo
 int ada_debug_set_wait_limit(ada_session *S, uint64_t ns) {
     if (!S || ns < 1) return ADA_EINVAL;
     S->wait_ns = ns;
+    return ADA_OK;
+}
+
+int ada_debug_cleared_bytes(ada_session *S, int64_t *bytes_out) {
+    if (!S || !bytes_out) return ADA_EINVAL;
+    *bytes_out = S->cleared;
     return ADA_OK;
 }
 

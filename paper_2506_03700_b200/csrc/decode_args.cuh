@@ -48,7 +48,8 @@ struct MegaArgs {
     float *head_part;          // [grid][8][4]
     const double *rope_freq;   // [hd/2]: base^(-2i/hd), computed once on the host
     unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
-    unsigned long long *attn_tag;   // [8][nq][n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume); zeroed before each launch
+    unsigned long long *attn_tag;   // [columns][nq][c.n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume), for the chunks that
+                               // the call can reach; zeroed before each launch
     unsigned *grid_ctr;
     void *pub;                 // Pub[2] of the kernel launched
     int *err;

@@ -83,3 +83,32 @@ def test_decode_attention_against_a_plain_softmax(head_dim, nq, nkv):
             ref = W["tok_embed"] @ (rms(x) * W["final_norm"])
             # the cache is given, so only the splits into two bf16 parts (2^-17 of a value) and fp32 sums remain; six products deep
             assert np.linalg.norm(logits[i] - ref) <= 6e-5 * np.linalg.norm(ref), (n_prompt, i)
+
+
+@pytest.mark.parametrize("dtype", ["bf16"])
+@pytest.mark.parametrize("batch,max_early", [(1, 5), (3, 5)])
+def test_calls_pay_for_the_positions_they_reach_not_for_the_sessions_length(dtype, batch, max_early):
+    """Short calls whose context grows over chunk boundaries (the layout of the chunk partials changes with it), in a session of
+    512 positions and in one of 32768: the same bits, and the same bytes cleared."""
+    cfg = synth.small_config(dtype=dtype, n_layers=3, d_model=256, n_q_heads=8, n_kv_heads=4, head_dim=64, d_ff=704, vocab=1024,
+                             sigma=0.08, resid_scale=0.8, exit_layers=(1, 2))
+    gm = binding.Model(cfg, synth.make_weights(cfg, device="cuda"))
+    for l in cfg.exit_layers:
+        gm.set_exit_head(l, None, 4.0)
+    got = []
+    for max_seq in (512, 32768):
+        S = binding.Session(gm, batch, max_seq, 64, max_early, kv_pages=8 * batch)
+        S.capture_logits(64)
+        seen, cleared = [], []
+        for first in (5, 120):   # (a prompt of the decode kernel's passes, one of the dense pass where there is one)
+            for i in range(batch):
+                S.prefill(synth.make_prompt(cfg, n=first + 3 * i, seq=i).numpy(), seq=i)
+                cleared.append(S.cleared_bytes())
+            for n in (1, 7, 3, 20):
+                seen.append(S.adaptive_decode(n, 0.2, cfg.exit_layers, max_early))
+                cleared.append(S.cleared_bytes())
+            seen.append(S.captured_logits().cpu().numpy().copy())
+        got.append((seen, cleared))
+    assert all(np.array_equal(a, b) for a, b in zip(got[0][0], got[1][0]))
+    assert got[0][1] == got[1][1]
+    assert got[0][1][-1] > got[0][1][-4] > 0   # (the last call reaches a second chunk)
