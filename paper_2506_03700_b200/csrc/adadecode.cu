@@ -153,7 +153,7 @@ struct ada_session {
     float inv_temp = 1.0f;
     // fp32 models whose rows fit: whole calls in one launch (resident.cuh)
     bool resident = false, res_prompts = false;   // decode calls; prompts
-    size_t res_smem = 0, res_words = 0;      // shared memory of a CTA; bytes of the exchanged words
+    size_t res_smem = 0;                     // shared memory of a CTA
     int res_grid = 0;
     rs::Args rargs;
     int steps_per_launch = 256;
@@ -257,11 +257,12 @@ ResidentFit resident_fit(const ada_config &g, int batch, int max_early) {
         if (f.rows || R == need) return f;
     }
 }
-// exchanged words: layer input, FFN input, T output, q | k | v, attention partials, FFN activations, head partials
-size_t resident_words(const ada_config &g, int R, int n_chunks) {
-    const size_t qkv = (size_t)(g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim, part = (size_t)g.n_q_heads * n_chunks * (g.head_dim + 2);
-    return (size_t)R * (3 * (size_t)g.d_model + qkv + part + g.d_ff) + 4 * (size_t)R * rs::MAX_GRID;
+// exchanged words: layer input, FFN input, T output, q | k | v, FFN activations, head partials; behind them the attention partials
+size_t resident_words(const ada_config &g, int R) {
+    const size_t qkv = (size_t)(g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim;
+    return (size_t)R * (3 * (size_t)g.d_model + qkv + g.d_ff) + 4 * (size_t)R * rs::MAX_GRID;
 }
+size_t resident_part_words(const ada_config &g, int R, int n_chunks) { return (size_t)R * g.n_q_heads * n_chunks * (g.head_dim + 2); }
 
 Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, int head_blocks) {
     Layout L{};
@@ -303,7 +304,7 @@ Layout make_layout(const ada_config &g, int batch, int max_seq, int max_early, i
         L.pf_flag = take(sizeof(unsigned) * 2 * dg::MAX_PAIRS * dg::GEPI_WARPS);
     }
     if (const int rows = resident_fit(g, batch, max_early).rows) {
-        L.res = take(resident_words(g, rows, n_chunks) * sizeof(rs::u64));
+        L.res = take((resident_words(g, rows) + resident_part_words(g, rows, n_chunks)) * sizeof(rs::u64));
         L.res_err = take(256);
     }
     // persistent-kernel buffers (bf16 models)
@@ -950,24 +951,24 @@ int setup_resident(ada_session *S, const Layout &lay) {
     a.ku = fit.ku;
     a.cs_ring = fit.ring;
     a.pf_rows = std::min(R, rs::TOK_RING);
-    S->res_words = resident_words(g, R, S->n_chunks) * sizeof(rs::u64);
     rs::u64 *w = (rs::u64 *)((char *)S->scratch + lay.res);
     auto take = [&](size_t n) { rs::u64 *at = w; w += n; return at; };
     a.XA = take((size_t)R * g.d_model);
     a.XB = take((size_t)R * g.d_model);
     a.TT = take((size_t)R * g.d_model);
     a.QT = take((size_t)R * S->c.qkv_rows);
-    a.PT = take((size_t)R * g.n_q_heads * S->n_chunks * (g.head_dim + 2));
     a.HT = take((size_t)R * g.d_ff);
     a.HP = take(4 * (size_t)R * rs::MAX_GRID);
+    a.PT = w;
     a.err = (int *)((char *)S->scratch + lay.res_err);
     S->resident = true;
     S->res_prompts = fit.prompts;
     return ADA_OK;
 }
 
-// One launch: the prompt of sequence pf_seq (pf_n tokens), or, with pf_n = 0, a whole decode call.
-int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layers, int n_exit, float gamma, int max_early, int eos_id, int tape_n, int n_tokens) {
+// One launch: the prompt of sequence pf_seq (pf_n tokens), or, with pf_n = 0, a whole decode call.  `reach` as for run_persistent.
+int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layers, int n_exit, float gamma, int max_early, int eos_id, int tape_n, int n_tokens,
+                 int reach) {
     const ada_model *m = S->m;
     rs::Args &a = S->rargs;
     a.c = S->c;   // capture pointers may have changed
@@ -989,7 +990,10 @@ int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layer
     a.pf_n = pf_n;
     a.max_steps = (long long)(n_tokens + 2) * (max_early + 2) * 4 + 16;
     a.wait_ns = S->wait_ns;
-    CK(cudaMemsetAsync(a.XA, 0, S->res_words, S->stream));   // phase numbers start over with every launch
+    a.c.n_chunks = chunks_of(reach);
+    const size_t part_bytes = resident_part_words(m->cfg, a.R, a.c.n_chunks) * sizeof(rs::u64);
+    CK(cudaMemsetAsync(a.XA, 0, (size_t)((char *)a.PT - (char *)a.XA) + part_bytes, S->stream));   // phase numbers start over with every launch
+    S->cleared += (int64_t)part_bytes;
     CK(cudaMemsetAsync(a.err, 0, sizeof(int), S->stream));
     void *params[] = {(void *)&a};
     CK(cudaLaunchCooperativeKernel(resident_kernel(m->cfg.head_dim), dim3(S->res_grid), dim3(rs::THREADS), params, S->res_smem, S->stream));
@@ -1137,7 +1141,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
         if ((rc = run_persistent(S, exit_layers, n_exit, plain, 0, S->batch, true, reach))) return rc;
     } else if (S->resident) {
         // (the token after a prompt is there already: a call for it alone has no step to run)
-        if (max_steps_plain > 0 && (rc = run_resident(S, 0, 0, exit_layers, plain ? 0 : n_exit, gamma, max_early, eos_id, tape_n, n_tokens)))
+        if (max_steps_plain > 0 && (rc = run_resident(S, 0, 0, exit_layers, plain ? 0 : n_exit, gamma, max_early, eos_id, tape_n, n_tokens, reach)))
             return rc;
     } else if (plain) {
         // every step is one token through all layers; the step count is known, no read-back needed
@@ -1617,7 +1621,7 @@ int ada_prefill(ada_session *S, int32_t seq, const int32_t *prompt_host, int32_t
         return ADA_OK;
     }
     if (S->resident && S->res_prompts) {
-        if ((rc = run_resident(S, seq, n_prompt, nullptr, 0, 2.0f, 0, -1, 0, 0))) return rc;
+        if ((rc = run_resident(S, seq, n_prompt, nullptr, 0, 2.0f, 0, -1, 0, 0, n_prompt))) return rc;
         S->prefilled[seq] = 1;
         S->h_prompt[seq] = n_prompt;
         S->h_len[seq] = n_prompt + 1;

@@ -51,7 +51,8 @@ struct Args {
     float rope_base, gamma;
     int batch, max_early, eos_id, tape_n, capture_cap;
     long long max_steps;                 // more steps than any call takes
-    u64 *XA, *XB, *QT, *PT, *HT, *TT, *HP;   // exchanged words: layer input, FFN input, q | k | v, attention partials, FFN activations, T output, head partials
+    u64 *XA, *XB, *QT, *PT, *HT, *TT, *HP;   // exchanged words: layer input, FFN input, q | k | v, attention partials [row][q head][c.n_chunks: as
+                                         // many as the call can reach][hd + 2], FFN activations, T output, head partials
     int R;                               // rows of the buffers
     int ku;                              // widest product input: max(d_model, q width, d_ff)
     int cs_ring;                         // rotary factors kept per sequence (a power of two above the rows in flight)
