@@ -188,3 +188,36 @@ def test_same_numbers_same_decisions_for_every_sequence_of_a_batch():
     for f in ("head_evals", "early_exits", "accepted", "rejected", "discarded"):
         assert getattr(st, f) == sum(getattr(o, f) for o in sts), f
     assert st.early_exits > 0 and st.accepted > 0
+
+
+# the kernel of 24 token columns: several sequences with four or five early tokens, eight with two; two launches (five sequences of
+# six columns); vocabularies that tiles of sixteen and draws of 128 entries do not divide
+@pytest.mark.parametrize("batch,max_early", [(2, 5), (4, 5), (5, 5), (4, 4), (8, 2)])
+@pytest.mark.parametrize("mk,resid_scale,vocab", [(gqa, 0.1, 1024), (gqa, 0.25, 1001), (hd128, 0.2, 2050)])
+def test_many_columns_draw_as_each_sequence_alone(mk, resid_scale, vocab, batch, max_early):
+    """Sampled decoding of several sequences over one weight stream with 24 columns: each equals its own run by the kernel of eight
+    with the same random numbers, in tokens, counters and (the first) logits."""
+    cfg = mk(logit_scale=2.0, resid_scale=resid_scale, vocab=vocab)
+    gm = Pair(cfg).gm
+    prompts = [synth.make_prompt(cfg, n=m, seq=i).numpy() for i, m in enumerate((9, 31, 14, 5, 22, 12, 17, 8)[:batch])]
+    n, max_seq = 24, 80
+    u = np.random.default_rng(5).random((batch, max_seq, NU), dtype=np.float32)
+    names = ("head_evals", "early_exits", "accepted", "rejected", "discarded", "steps", "verify_steps")
+
+    def run(ps, us):
+        S = binding.Session(gm, len(ps), max_seq, 64, max_early)
+        assert S.get_path() == 1
+        S.capture_logits(n + 8)
+        for i, p in enumerate(ps):
+            S.prefill(p, seq=i)
+        st = binding.Stats()
+        out = S.sampling_decode(n, 0.6, 0.1, cfg.exit_layers, max_early, us, 0, st)
+        return out, np.array([getattr(st, f) for f in names]), S.captured_logits().cpu().numpy().copy()
+
+    out, counts, lg = run(prompts, u)
+    alone = [run([p], u[i:i + 1]) for i, p in enumerate(prompts)]
+    for i, (o, _, _) in enumerate(alone):
+        assert np.array_equal(out[i], o[0]), i
+    assert np.array_equal(lg, alone[0][2])
+    assert np.array_equal(counts, sum(c for _, c, _ in alone))
+    assert counts[1] > 0 and counts[2] > 0 and counts[3] > 0   # early, accepted, rejected
