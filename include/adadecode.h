@@ -231,8 +231,8 @@ int ada_debug_set_prefill(ada_session *s, int32_t dense);
 /* Steps of Algorithm 1 one launch of the persistent kernel may start before it returns to the host
  * (default 256; the host relaunches until the call is complete). */
 int ada_debug_set_launch_steps(ada_session *s, int32_t steps);
-/* Every wait inside the persistent kernel and the dense prompt pass (on a shared-memory barrier, on the grid-wide counter,
- * on another CTA's partial sums) gives up after `ns` nanoseconds (default 2 s): the kernel then sets an
+/* Every wait inside the persistent kernel, the fp32 one-launch kernel and the dense prompt pass (on a shared-memory barrier, on the
+ * grid-wide counter, on another CTA's words) gives up after `ns` nanoseconds (default 2 s): the kernel then sets an
  * error word, lets every other wait fall through, ends, and the decode or prefill call returns ADA_ETIMEOUT.
  * The sequence state is undefined after that; ada_session_reset + ada_prefill make the session
  * usable again.  A limit shorter than a grid-wide wait normally lasts (a few microseconds) makes the

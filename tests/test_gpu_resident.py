@@ -3,6 +3,7 @@ qualify for it: here one with room for sixteen early tokens."""
 
 import numpy as np
 import pytest
+import torch
 
 from paper_2506_03700_b200 import binding, synth
 
@@ -105,3 +106,44 @@ def test_heads_over_more_than_eight_rows_give_each_sequence_its_own_bits(batch, 
         o, l = run([p])
         assert np.array_equal(o[0], out[i])
         assert np.array_equal(l[:, 0], log[:, i]), i
+
+
+@pytest.mark.parametrize("during", ["prompt", "decode"])
+def test_a_wait_that_runs_out_ends_the_call_with_a_timeout_and_the_session_recovers(during):
+    """Values pass between the CTAs as words that the readers wait for, with a limit.  Set far below the time that a word takes, the
+    first wait that is not satisfied at once gives up, the others follow, and the call returns ADA_ETIMEOUT.  After a reset and
+    a prompt the session gives what a fresh one gives."""
+    cfg = synth.small_config(n_layers=4, d_model=256, n_q_heads=4, n_kv_heads=4, head_dim=64, d_ff=688, vocab=2048, sigma=0.08,
+                             resid_scale=0.5, exit_layers=(1, 3))
+    plan = binding.debug_resident_plan(cfg, 2, 5)
+    assert plan["rows"] > 0 and plan["prompts"]
+    gm = binding.Model(cfg, synth.make_weights(cfg, device="cuda", norm_gain_jitter=0.2))
+    gm.set_exit_head(1, synth.make_head_transform(cfg, 1, device="cuda", noise=0.1), 4.0)
+    gm.set_exit_head(3, None, 4.0)
+    prompts = [synth.make_prompt(cfg, n=k, seq=i).numpy() for i, k in enumerate((40, 12))]
+    n = 16
+
+    def whole(S):
+        for i, p in enumerate(prompts):
+            S.prefill(p, seq=i)
+        return S.adaptive_decode(n, 0.3, cfg.exit_layers, 5), S.captured_logits().cpu().numpy().copy()
+
+    def session():
+        S = binding.Session(gm, 2, 96, 16, 5)
+        S.capture_logits(n)
+        return S
+
+    ref, lr = whole(session())
+    S = session()
+    if during == "decode":
+        for i, p in enumerate(prompts):
+            S.prefill(p, seq=i)
+    S.set_wait_limit(20)                  # nanoseconds
+    with pytest.raises(binding.AdaError) as e:
+        S.prefill(prompts[0], seq=0) if during == "prompt" else S.adaptive_decode(n, 0.3, cfg.exit_layers, 5)
+    assert e.value.code == -5
+    torch.cuda.synchronize()              # the context is intact
+    S.set_wait_limit(2_000_000_000)
+    S.reset()
+    out, lg = whole(S)
+    assert np.array_equal(out, ref) and np.array_equal(lg, lr)
