@@ -1031,7 +1031,10 @@ __device__ __forceinline__ void attn_produce_kv(const MegaArgs &A, const Shared 
     }
 }
 // The items' query fragments come through the activation ring, one stage per item: the tiles in use, 64 hd bytes each.
-__device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &S, const StepDesc &d, unsigned mask, unsigned bar_target, Rings &r, uint64_t pol) {
+// `after_first` as for gemm_produce_x.
+template <class Hook>
+__device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &S, const StepDesc &d, unsigned mask, unsigned bar_target, Rings &r, uint64_t pol,
+                                               Hook &&after_first) {
     const Ctx &c = A.c;
     Smem *sm = S.sm;
     const uint32_t tile_bytes = (uint32_t)c.hd * 64;
@@ -1041,7 +1044,8 @@ __device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &
 #pragma unroll 1
     while (w.next(A, d, mask, it)) {
         mbar_wait(S, &sm->x_empty[r.xs], r.xp ^ 1);
-        if (!synced) {
+        const bool first = !synced;
+        if (first) {
             grid_wait(S, A.grid_ctr, bar_target);
             fence_proxy_async();
             synced = true;
@@ -1052,6 +1056,7 @@ __device__ __forceinline__ void attn_produce_q(const MegaArgs &A, const Shared &
             mbar_expect_tx(&sm->x_full[r.xs], bytes);
             bulk_g2s(sm->x[r.xs], src, bytes, &sm->x_full[r.xs], pol);
         }
+        if (first) after_first();
         r.next_x();
     }
 }
@@ -1582,14 +1587,18 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
     }
     if (ROLE == 2) bar_consumers(); else __syncwarp();
 
-    unsigned long long t_last = gtime();
-    auto book = [&](int cls) {   // CTA 0 books the time since the last event to a class
-        if (ROLE == 2 && blockIdx.x == 0 && threadIdx.x == 0) {
+    // Phase times: a phase ends when the whole grid has reported it.  The activation producer of CTA 0 sees that first (it waits for
+    // it before it fetches the next input, and books after that).  The consumers do not wait for it, and a CTA without a tile of a
+    // product passes it in no time: booked by them, the 1B shape's down product took 2 us of its 9.
+    if (ROLE == 1) sm->t_booked = gtime();
+    int behind = -1;   // class of the phase whose end has not been booked yet
+    auto book = [&](int cls) {
+        if (ROLE == 1 && blockIdx.x == 0 && (threadIdx.x & 31) == 0 && cls >= 0) {
             const unsigned long long t = gtime();
-            // reductions, not read-modify-write: thread 0 of CTA 0 must not wait for a load from L2 at every phase
-            atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_ns[cls]), t - t_last);
+            // reductions, not read-modify-write: nobody waits for a load from L2 at every phase
+            atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_ns[cls]), t - sm->t_booked);
             atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.phase_count[cls]), 1ull);
-            t_last = t;
+            sm->t_booked = t;
         }
     };
 
@@ -1598,6 +1607,11 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
 #pragma unroll 1
     for (;;) {
         if (ROLE == 2 && blockIdx.x == 0) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);   // CTA 0 reads every CTA's head partials
+        if (ROLE == 1 && blockIdx.x == 0) {
+            grid_wait(S, A.grid_ctr, bar_no * (unsigned)G);
+            book(behind);
+            behind = -1;
+        }
         const int action = control_point<ROLE>(A, S, ctl, e, pub_no, d, steps_started);
         book(0);
         if (action == ACT_NEWSTEP) {
@@ -1619,7 +1633,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
             const unsigned cmask = inter ? (unsigned)d.head_mask & mask : mask;
             if (ph == PH_ATTN) {
                 if (ROLE == 0) attn_produce_kv(A, S, d, l, mask, bar_no * (unsigned)G, r, pol);
-                if (ROLE == 1) attn_produce_q(A, S, d, mask, bar_no * (unsigned)G, r, pol);
+                if (ROLE == 1) attn_produce_q(A, S, d, mask, bar_no * (unsigned)G, r, pol, [&]() { book(behind); });
                 if (ROLE == 2) {
                     // (a CTA without an item must not report the phase before the one in front of it is complete)
                     if (AttnWalk(A, d, mask).n <= (int)blockIdx.x) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
@@ -1645,7 +1659,10 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 if (ROLE == 1) {
                     const __nv_bfloat16 *X = ph == PH_QKV ? A.XA : ph == PH_O ? A.XO : ph == PH_GU ? A.XB : ph == PH_DOWN ? A.XH : ph == PH_HEAD && with_T ? A.XT : A.XF;
                     gemm_produce_x(S, pl, reinterpret_cast<const uint4 *>(X), Cols(cmask), r, pol,
-                                   [&]() { if (scaled) rstd_produce(sm, ph == PH_GU ? A.ssq_b : A.ssq_a, ntd, d_model, c.eps, vseq); },
+                                   [&]() {
+                                       book(behind);
+                                       if (scaled) rstd_produce(sm, ph == PH_GU ? A.ssq_b : A.ssq_a, ntd, d_model, c.eps, vseq);
+                                   },
                                    [&]() {   // the input must not be fetched before the phase that wrote it is complete
                                        grid_wait(S, A.grid_ctr, bar_no * (unsigned)G);
                                        fence_proxy_async();
@@ -1663,10 +1680,8 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                     if (ph == PH_HEAD) epi.head_end(pl, cmask);
                 }
             }
-            if (ROLE == 2) {
-                consumers_arrive(S, A.grid_ctr, prof_class(ph));
-                book(prof_class(ph));
-            }
+            if (ROLE == 2) consumers_arrive(S, A.grid_ctr, prof_class(ph));
+            behind = prof_class(ph);
             ++bar_no;
             // ---- what comes next
             if (ph == PH_HEAD) {

@@ -168,6 +168,7 @@ struct Smem {                                    // must start on a 1024-byte bo
     unsigned trace_n;
     unsigned vec_seq;                             // phase for which vec[] holds the normalisation factors (see vec_wait)
     unsigned w_issued;                            // weight stages issued so far (see w_wait)
+    unsigned long long t_booked;                  // CTA 0's activation producer: time up to which phases have been booked
     Plan plan[6];                                 // this CTA's share of every product of the program
 };
 

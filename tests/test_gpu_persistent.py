@@ -505,3 +505,40 @@ def test_both_attention_arrangements_agree_with_more_items_than_ctas():
         assert np.array_equal(A.adaptive_decode(n, 0.5, cfg.exit_layers, 5, st)[0], out)
         assert torch.equal(A.captured_logits()[:n], lg)
         assert st.early_exits >= 5
+
+
+def test_phase_times_are_the_grids_not_one_ctas():
+    """Products with fewer tiles than the GPU has SMs leave CTA 0, whose clock the phase timers use, without a tile.  Their time is that
+    of the grid all the same: no product of the 1B shape streams its weights faster than HBM delivers them (8 TB/s nominal; eight
+    layers, so that no weight survives in L2 until the next step), and the phases add up to the call."""
+    cfg = synth.small_config(dtype="bf16", n_layers=8, d_model=2048, n_q_heads=32, n_kv_heads=8, head_dim=64, d_ff=8192, vocab=32000,
+                             resid_scale=0.2, exit_layers=(4,))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    nrm = lambda *s: torch.empty(*s, dtype=torch.bfloat16, device="cuda").normal_(0, 0.02, generator=gen)
+    one = torch.ones(cfg.d_model, dtype=torch.bfloat16, device="cuda")
+    w = {"tok_embed": nrm(cfg.vocab, cfg.d_model), "final_norm": one}
+    for l in range(cfg.n_layers):
+        p = "layers.%d." % l
+        w[p + "attn_norm"] = w[p + "ffn_norm"] = one
+        w[p + "wqkv"], w[p + "wo"] = nrm(cfg.qkv_rows, cfg.d_model), nrm(cfg.d_model, cfg.d_model)
+        w[p + "w_gate_up"], w[p + "w_down"] = nrm(2 * cfg.d_ff, cfg.d_model), nrm(cfg.d_model, cfg.d_ff)
+    gm = binding.Model(cfg, w)
+    gm.set_exit_head(4, None, 1.0)
+    S = binding.Session(gm, 1, 256, 64, 5)
+    prompt = synth.make_prompt(cfg, n=33).numpy()
+    S.prefill(prompt)
+    S.plain_decode(4)
+    S.prefill(prompt)
+    S.profile(True)
+    st = binding.Stats()
+    S.adaptive_decode(40, 2.0, cfg.exit_layers, 5, st)
+    prof = S.profile_read()
+    S.profile(False)
+    size = dict(qkv_gemm=cfg.qkv_rows * 2048, o_gemm=2048 * 2048, gate_up_gemm=2 * 8192 * 2048, down_gemm=2048 * 8192, lm_head=32000 * 2048)
+    for name, n in size.items():
+        p = prof[name]
+        assert p["launches"] == (39 * 8 if name != "lm_head" else 39 * 2), name
+        assert p["ms"] * 1e-3 / p["launches"] >= 2 * n / 8.0e12, (name, p)
+    assert prof["attention"]["launches"] == 39 * 8
+    total = sum(p["ms"] for p in prof.values())
+    assert 0.9 * st.decode_ms <= total <= 1.02 * st.decode_ms, (total, st.decode_ms)
