@@ -28,7 +28,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    extra = os.environ.get("ADA_NVCC_EXTRA", "").split()      # e.g. "-DADA_NW=8 -DADA_NX=4" (ring depths, see stream.cuh)
+    extra = os.environ.get("ADA_NVCC_EXTRA", "").split()      # further nvcc flags
     cmd = [nvcc] + NVCC_FLAGS + extra + (["-Xptxas", "-v"] if verbose else []) + ["-shared", "-o", LIB] + \
           [os.path.join(CSRC, s) for s in SOURCES]
     subprocess.check_call(cmd)

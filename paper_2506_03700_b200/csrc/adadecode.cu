@@ -144,7 +144,7 @@ struct ada_session {
     int32_t *pinned = nullptr; // small read-back area
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     int path = 0;
-    // persistent-kernel path (bf16, one sequence, up to eight token columns)
+    // persistent-kernel path (bf16, up to eight sequences in eight or 24 token columns)
     bool mega = false;
     int grid = 0;
     MegaArgs margs;
@@ -230,12 +230,13 @@ constexpr size_t kSharedMax = 232448;   // 227 KB: most shared memory of a block
 // their inputs from shared memory, two rows at a time, and its head's entries come one pair per warp after the other, where theirs
 // hold eight rows in registers and four entries in flight.  So it is taken where the layers' latency outweighs both; measured
 // against one kernel per operation, times of decode calls (plain, and adaptive with everything and little accepted):
-//   rows of a step, by the widest input: any number up to 896 (d_model 64 .. 320: 0.49 .. 0.94; sixteen sequences of width 256
-//     0.94), three up to 1024 (width 384: 0.67 .. 0.89; eight 0.98 .. 1.10), two up to 2048 (width 512: 0.62 .. 0.94, 768: 0.92 .. 1.00;
-//     three 0.88 .. 1.05), one up to 3584 (width 1024: 0.71 .. 0.91, 1408: 0.93 .. 0.96; two 0.73 .. 1.05);
+//   sequences, by the widest input: any number up to 896 (d_model 64 .. 320: 0.49 .. 0.94; sixteen sequences of width 256
+//     0.94), three up to 1024 (width 384: 0.67 .. 0.89; eight 0.98 .. 1.10), two up to 2048 (width 512: 0.64 .. 0.76, 768: 0.75 .. 0.85;
+//     three 0.88 .. 1.05), one up to 3584 (width 1024: 0.70 .. 0.77, 1408: 0.93 .. 0.96; two 0.73 .. 1.05)
+//     (what is not taken was measured with shared memory laid out for prompts too: up to 20 % slower than without);
 //   weights of the head per layer: 2^21 (width 256, four layers: vocabulary 32000 0.69, 64000 1.02; width 512 8192 0.88, 32000 1.06),
 //     from four sequences on 2^19 (width 256, eight sequences: 8192 0.90, 16384 0.95, 32000 1.07).
-// Prompts go 32 rows a pass in both, and the longer the prompt the more its products count: widths up to 768 with small heads only
+// Prompts go up to 32 rows a pass in both, and the longer the prompt the more its products count: widths up to 768 with small heads only
 // (width 64 .. 192 0.71 .. 0.99; width 256: one token 0.82, eight 1.06, sixteen 1.00, 64 0.89, 500 0.91; a d_ff of 2816 1.15, width 512 1.3).
 ResidentFit resident_fit(const ada_config &g, int batch, int max_early) {
     ResidentFit f;

@@ -43,11 +43,11 @@ struct MegaArgs {
     Ctx c;
     MegaModel m;
     __nv_bfloat16 *XA, *XB, *XO, *XH, *XF, *XT;   // GEMM inputs in fragment layout (see stream.cuh)
-    float *ssq_a, *ssq_b;      // [d/16][8] partial sums of squares of the residual (per 16-feature tile, per column)
+    float *ssq_a, *ssq_b;      // [d/16][columns] partial sums of squares of the residual (per 16-feature tile, per column)
     uint32_t *qfrag;           // [sequence][nkv][2][hd/16][32][8]: rotated, scaled queries as tensor-core A fragments (bf16 high parts, then low parts)
-    float *head_part;          // [grid][8][4]
+    float *head_part;          // [grid][columns][4]
     const double *rope_freq;   // [hd/2]: base^(-2i/hd), computed once on the host
-    unsigned long long *part;  // [grid][8][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
+    unsigned long long *part;  // [grid][8 k-splits][column tiles][256]: tagged partial sums of weight tiles split between two CTAs (null: none)
     unsigned long long *attn_tag;   // [columns][nq][c.n_chunks][hd + 2]: chunk partials as tagged words (see attn_consume), for the chunks that
                                // the call can reach; zeroed before each launch
     unsigned *grid_ctr;

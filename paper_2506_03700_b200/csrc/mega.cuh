@@ -65,9 +65,8 @@ __device__ __forceinline__ unsigned active_mask(const StepDesc &d, int layer) {
     return m;
 }
 
-// rstd[c] = 1 / sqrt(sum_tiles ssq[tile][c] / d + eps), one warp per column, fixed summation order.
-// RMSNorm factors 1/sqrt(mean square + eps) of the eight columns from the per-tile sums of squares
-// ssq[tile][column], by the activation producer warp: lane l sums column l%8 over the tiles
+// RMSNorm factors 1/sqrt(mean square + eps) of all columns from the per-tile sums of squares
+// ssq[tile][column], by the activation producer warp, eight columns at a time: lane l sums column l%8 over the tiles
 // l/8 + 4u in ascending order (32 loads in flight), the four lanes of a column are folded by a
 // butterfly.  The order is fixed, so the factor of a column does not depend on the other columns.
 __device__ __forceinline__ void rstd_produce(Smem *sm, const float *ssq, int ntiles, int d, float eps, unsigned seq) {
@@ -1558,7 +1557,7 @@ template <int HD> struct Epilogue {
     }
 };
 
-// ROLE 0: weight producer warp, 1: activation / KV producer warp, 2: consumer warps.
+// ROLE 0: producer warp of weights and K / V blocks, 1: of activations and queries, 2: consumer warps.
 //
 // A step is a sequence of phases; every role walks it with one loop whose body holds each piece of code once (one product, one
 // attention, one control point) and takes from the phase number what differs.
@@ -1645,7 +1644,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                 // rows (Algorithm 1: "update KV cache at layer l by processing all tokens in P[l] in parallel").
                 // The rows of every q and k head come reordered so that a 16-row tile holds the features
                 // [8 t, 8 t + 8) and [hd/2 + 8 t, hd/2 + 8 t + 8): the two partners (i, i + hd/2) of a rotation
-                // are then rows r and r + 8 of one tile, which one thread holds for its two columns.
+                // are then rows r and r + 8 of one tile, which two lanes of a warp finish, eight lanes apart.
                 const Plan pl = sm->plan[ph];
                 const bool with_T = inter && M.has_T[l];
                 const unsigned vseq = bar_no + 1;
@@ -1709,7 +1708,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
 // Repack on load.  Destination row `prow` of the fused q | k | v matrix: v rows are copied as they are; inside
 // every q and k head the rows are reordered so that the 16-row tile t of the head holds the features
 // [8 t, 8 t + 8) in its rows 0..7 and [hd/2 + 8 t, hd/2 + 8 t + 8) in its rows 8..15.  The two partners
-// (i, i + hd/2) of a rotation then sit in rows r and r + 8 of one tensor-core tile, i.e. in one thread of the
+// (i, i + hd/2) of a rotation then sit in rows r and r + 8 of one tensor-core tile, i.e. in two lanes of one warp of the
 // QKV epilogue.  d must be a multiple of 8 and every pointer 16-byte aligned.
 __global__ void k_repack_qkv(const __nv_bfloat16 *__restrict__ wq, const __nv_bfloat16 *__restrict__ wk, const __nv_bfloat16 *__restrict__ wv,
                              __nv_bfloat16 *__restrict__ dst, int nq, int nkv, int hd, int d) {
@@ -1745,7 +1744,7 @@ __global__ void k_prefill_arm(Ctx c, int seq, int n_prompt) {
 
 #endif
 
-// Warps 0-7 consume, warp 8 produces weights, warp 9 activations and K / V blocks; warps 10 and 11 only complete the producers'
+// Warps 0-7 consume, warp 8 produces weights and K / V blocks, warp 9 activations and queries; warps 10 and 11 only complete the producers'
 // warp group, which hands registers to the consumers.  (At 168 registers a thread -- three warps on a quarter of the SM --
 // the consumers kept loop variables in local memory, whose L1 lines do not survive the acquires of the grid barrier.)
 constexpr int MEGA_THREADS = CONS_THREADS + 128;

@@ -48,9 +48,8 @@ def test_host_side_argument_checks_need_no_gpu():
 
 
 def test_session_scratch_does_not_pay_for_chunk_partials_that_cannot_occur():
-    """The tagged partials of the one-item attention path are laid out for the chunks that 256 work items can have (32 of 128
-    positions with eight kv heads), whatever the session's length: from there on a position costs its share of the other
-    buffers only (attention partials: 8 columns x 32 heads x 132 floats per 128 positions)."""
+    """The decode kernel's tagged chunk partials (24 columns of 8-byte words) share the memory of the per-operation path's (64 rows of
+    floats): a position costs the larger of the two and its share of the other buffers, not both."""
     lib = binding.load()
     h = ctypes.c_void_p()
     cfg = binding.Config(32, 4096, 32, 8, 128, 14336, 128256, 1, 0, 500000.0, 1e-5)
