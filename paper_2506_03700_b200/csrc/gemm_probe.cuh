@@ -51,7 +51,7 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
     } else {
         const ProbeEpilogue epi{Y, ldy, mode, mode == 0 ? N : g.half};
         for (int it = 0; it < repeat; ++it) {
-            st::gemm_consume(S, pl, cols_used, (1u << cols) - 1u, part, 1u, cta, r, epi);
+            st::gemm_consume<false>(S, pl, cols_used, (1u << cols) - 1u, part, 1u, cta, r, epi);
             st::bar_consumers();   // the exchange area is free for the next product
         }
     }

@@ -5,8 +5,9 @@
 //     control | for each layer: QKV | attention | O | gate-up | down | [head, control] ... | final head | control
 // with a grid barrier between phases.  The weight producer is not held by those barriers (but for cache rows
 // of the pass itself): it keeps the TMA ring full with the tiles of the coming phases, so HBM keeps streaming while the
-// grid meets.  Measured, one layer in a plain step (1B / 8B shape): QKV 6.2 / 11.7 us, attention 7.2 / 9.9 (60 / 1040 positions),
-// O 5.4 / 9.0, gate-up 13.5 / 38.1, down 9.1 / 20.5, of which the bytes alone take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
+// grid meets, and the consumers move what has landed on to tensor memory (park_stage in stream.cuh).  Measured, one layer in a plain
+// step (1B / 8B shape): QKV 5.9 / 10.8 us, attention 7.2 / 9.9 (60 / 1040 positions),
+// O 5.2 / 7.7, gate-up 11.4 / 35.8, down 7.7 / 19.2, of which the bytes alone take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
 // residuals, counters) lives in device memory; the control points run in CTA 0, which publishes
 // each decision (continue the climb, start the next token, stop) to the other CTAs through a
 // sequence-numbered record.  The host launches, waits, and launches again until the call is done.
@@ -1675,7 +1676,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                     // (an idle CTA must not report a phase before the one in front of it is complete: the counter would run ahead)
                     if (Groups(pl).left <= 0) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
                     if (ph == PH_HEAD) epi.head_begin();
-                    gemm_consume(S, pl, Cols(cmask), cmask, A.part, vseq, blockIdx.x, r, epi);
+                    gemm_consume<TILES == 1>(S, pl, Cols(cmask), cmask, A.part, vseq, blockIdx.x, r, epi);
                     if (ph == PH_HEAD) epi.head_end(pl, cmask);
                 }
             }
@@ -1760,9 +1761,15 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
         const int ph = threadIdx.x - 32;
         sm->plan[ph] = make_plan(phase_gemm(A, ph, gridDim.x), blockIdx.x, gridDim.x);
     }
-    __syncthreads();
-    Shared S{sm, A.err, A.trace, 0, A.wait_ns};
     const int warp = threadIdx.x >> 5;
+    if (TILES == 1 && warp == CONS_WARPS + 2) {   // tensor memory for parked weight stages; all of it, there is one CTA per SM
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&sm->tmem)), "r"(PARK_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tc_fence_before();
+    }
+    __syncthreads();
+    if (TILES == 1) tc_fence_after();
+    Shared S{sm, A.err, A.trace, 0, A.wait_ns};
     if (warp < CONS_WARPS) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_CONSUME));
         run<2, HD>(A, S);
@@ -1771,7 +1778,12 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
         if (warp == CONS_WARPS) run<0, HD>(A, S);
         else if (warp == CONS_WARPS + 1) run<1, HD>(A, S);
     }
-    settle_on_abort(S);
+    if (TILES == 1) tc_fence_before();
+    settle_on_abort(S);   // (meets the whole block)
+    if (TILES == 1 && warp == CONS_WARPS + 2) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm->tmem), "r"(PARK_COLS) : "memory");
+    }
 }
 
 }  // namespace ADA_MG

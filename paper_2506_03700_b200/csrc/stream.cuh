@@ -38,6 +38,7 @@
 #include <stdint.h>
 
 #include "decode_args.cuh"
+#include "tmem.cuh"
 
 namespace ada {
 namespace ADA_ST {
@@ -168,6 +169,7 @@ struct Smem {                                    // must start on a 1024-byte bo
     unsigned trace_n;
     unsigned vec_seq;                             // phase for which vec[] holds the normalisation factors (see vec_wait)
     unsigned w_issued;                            // weight stages issued so far (see w_wait)
+    uint32_t tmem;                                // base of this CTA's tensor memory (kernels that park weight stages there)
     unsigned long long t_booked;                  // CTA 0's activation producer: time up to which phases have been booked
     Plan plan[6];                                 // this CTA's share of every product of the program
 };
@@ -190,6 +192,17 @@ __device__ __forceinline__ bool mbar_try(unsigned long long *bar, uint32_t parit
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(s32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_test(unsigned long long *bar, uint32_t parity) {   // (does not wait)
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(s32(bar)), "r"(parity)
@@ -608,6 +621,64 @@ __device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned 
     }
 }
 
+// A parked stage (see park_stage): the fragments come back from tensor memory, eight k-steps at a time, the next eight on their way
+// while these are multiplied.  The same multiply-adds in the same order as above.
+template <bool PACKED>
+__device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, const unsigned char *xs) {
+    uint32_t a[2][32];
+    tmem_ld32_start(a[0], tm);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        uint4 b[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const unsigned char *p = xs + (8 * h + j) * 128;
+            if (PACKED) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(p);
+                b[j] = make_uint4(v.x, v.y, 0, 0);
+            } else {
+                b[j] = *reinterpret_cast<const uint4 *>(p);
+            }
+        }
+        uint32_t(&cur)[32] = a[h & 1];
+        tmem_ld_wait(cur);
+        if (h < 3) tmem_ld32_start(a[(h + 1) & 1], tm + 32 * (h + 1));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t f[4] = {cur[4 * j], cur[4 * j + 1], cur[4 * j + 2], cur[4 * j + 3]};
+            mma16816(acc[j & 1], f, b[j].x, b[j].y);
+            if (!PACKED) mma16816(acc[(j & 1) + 2], f, b[j].z, b[j].w);
+        }
+    }
+}
+
+// Weight stages parked in tensor memory.  Between a phase's end and the arrival of the next one's activations (3 to 4 us: report,
+// last CTA's report seen, copy) the consumers have nothing to multiply, and the nine stages of the ring cover 3 us of the
+// stream only: HBM idled for the rest.  So the warps use the wait to move the stages they own from the ring to tensor memory, up to
+// two each, as the fragments that the multiply-add wants; the ring's slots go back to the producer at once.  That makes 25
+// stages (400 KB) per CTA, and the parked ones do not pass through shared memory again when the activations are there.
+// Warp w can address the lanes of quadrant w % 4 only; it holds its stages there in columns 256 (w / 4) on, 128 a stage.
+// A layer of the 8B shape (1B), us, without and with: QKV 11.7 -> 10.8 (6.2 -> 5.9), O 9.0 -> 7.7 (5.3 -> 5.2), gate-up 38.6 -> 35.8
+// (13.4 -> 11.4), down 20.6 -> 19.2 (9.0 -> 7.7); short requests of the 1B shape 37.6 -> 34.7 ms.  (The kernel of
+// one column tile only: with 24 columns the products are bound by their activations.)
+constexpr int PARK_MAX = 2, PARK_COLS = 512;
+__device__ __forceinline__ void park_stage(const unsigned char *ws, int a_hi, int a_sw, uint32_t tm) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        uint32_t v[32];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int ks = 8 * h + j;
+            uint32_t a[4];
+            ldmatrix_x4(a, ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[4 * j + i] = a[i];
+        }
+        tmem_st32(tm + 32 * h, v);
+    }
+    tmem_st_wait();
+}
+
 // Consumer warps.  Within a group of up to eight tiles the warps are arranged as TS tile slots x
 // KS k-splits (TS * KS = 8, TS the smallest power of two holding the group); a warp multiplies
 // the stages of its slot whose k chunk is ks_id (mod KS).  The arrangement depends only on the tile partition, never on which
@@ -623,8 +694,9 @@ __device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned 
 // One body for every product of a program (the caller loops over its phases and branches on the phase in `pre` and `epi`): with
 // a copy of it per product and role the persistent kernel was 790 KB of code, more than the instruction caches hold, and every
 // phase began and ended with instruction fetches from L2 on its critical path.
+// PARK: the kernel has tensor memory for parked stages (sm->tmem).
 // k steps past K multiply zeros (the tensor map fills weights with them, the activation blocks are padded with them).
-template <class Epi>
+template <bool PARK, class Epi>
 __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, const Cols &cols, unsigned mask, unsigned long long *part, unsigned phase_id, int cta,
                                              Rings &r, const Epi &epi) {
     Smem *sm = S.sm;
@@ -673,6 +745,45 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             my_cols |= (unsigned long long)(act ? __ffs(m) - 1 : 31) << (5 * ps);
             if (act && ps < STASH_PASSES) epi.pre(ps, g.g0 + slot, row, __ffs(m) - 1);
         }
+        // This warp's chunks in order: n_pub of the part it publishes, then those of its own tile; every KS-th one from the first of
+        // the part.  (A warp then multiplies all 32 k-steps of a stage, which amortises the per-stage waiting and set-up: splitting
+        // every stage among the warps streamed 20-30 % slower.)
+        const int lks = 3 - lts, n_pub = max(0, my_pub_k1 - ks_id + KS - 1) >> lks, n_all = n_pub + (max(0, nch - my_own_k0 - ks_id + KS - 1) >> lks);
+        auto chunk_of = [&](int j) { return j < n_pub ? ks_id + (j << lks) : my_own_k0 + ks_id + ((j - n_pub) << lks); };
+        auto stage_of = [&](int kc) {   // number of its (first) weight stage at chunk kc
+            const bool gap0 = slot_id > 0 && kc >= s0_pub_k1 && kc < s0_own_k0;   // slot 0 has none here
+            return r.w + (uint32_t)((stages_before(pl, ng, kc) + slot_id - gap0) * pair);
+        };
+        // stages parked while the activations are on their way: those that land before they do, at most PARK_MAX
+        int n_parked = 0, n_used = 0;
+        const uint32_t tm = PARK ? sm->tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (128 * PARK_MAX) : 0u;
+        if (PARK && first) {
+            unsigned long long t0 = 0;
+            const int most = min(n_all * pair, PARK_MAX);
+#pragma unroll 1
+            while (n_parked < most) {
+                const uint32_t i = stage_of(chunk_of(pair == 2 ? n_parked >> 1 : n_parked)) + (pair == 2 ? n_parked & 1 : 0), wslot = i % NW;
+                bool go = true;
+#pragma unroll 1
+                for (uint32_t it = 0;; ++it) {
+                    if (__any_sync(0xffffffffu, mbar_test(&sm->x_full[r.xs], r.xp))) { go = false; break; }
+                    if ((int)(known - i) <= 0) known = w_issued_get(sm);
+                    if (__all_sync(0xffffffffu, (int)(known - i) > 0 && mbar_test(&sm->w_full[wslot], (i / NW) & 1))) break;
+                    if ((it & 127u) == 127u || S.wait_ns < SHORT_LIMIT_NS) {   // the wait for the activations below reports what is wrong
+                        bool stop = aborted(S) || *(volatile int *)S.err != 0;
+                        const unsigned long long t = gtime();
+                        if (t0 == 0) t0 = t;
+                        else if (t - t0 > S.wait_ns) stop = true;
+                        if (__any_sync(0xffffffffu, stop)) { go = false; break; }
+                    }
+                }
+                if (!go) break;
+                park_stage(sm->w[wslot] + a_off, a_hi, a_sw, tm + 128 * n_parked);
+                ++n_parked;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
+            }
+        }
         float acc0[TILES][4][4], acc1[TILES][4][4];   // [column tile][even/odd step x hi/lo][fragment] of the one or two matrices
         auto clear = [&]() {
 #pragma unroll
@@ -695,65 +806,36 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                     d[t][i] = hi + (packed ? __shfl_xor_sync(0xffffffffu, hi, 2) : acc[t][2][i] + acc[t][3][i]);
                 }
         };
-#pragma unroll 1
-        for (int kc = 0; kc < nch; ++kc) {
-            const unsigned char *xt[TILES];   // the chunk's activations, by column tile
-            if (TILES == 1) {
-                if ((kc & (XC - 1)) == 0) mbar_wait(S, &sm->x_full[r.xs], r.xp);
-                xt[0] = sm->x[r.xs] + (kc & (XC - 1)) * cols.ncp * 4096 + x_off[0];
-            } else {
-                uint32_t xs = r.xs, xp = r.xp;
+        // Activation stages are shared: every warp waits for and releases each of them.  A warp goes from one of its own chunks to the
+        // next; looking at every chunk cost 400 cycles for each that is not its own, which parked stages would not have hidden.
+        int x0 = 0;                       // first chunk of the activation stage(s) at hand
+        const unsigned char *xt[TILES];   // this lane's bytes of them, by column tile
+        auto x_wait = [&]() {
+            uint32_t xs = r.xs, xp = r.xp;
 #pragma unroll
-                for (int t = 0; t < TILES; ++t) {
-                    xt[t] = sm->x[xs] + (t == 0 ? (kc & (XC - 1)) * cols.ncp * 4096 : 0) + x_off[t];
-                    if (t < nt) {
-                        if ((kc & (XC - 1)) == 0) mbar_wait(S, &sm->x_full[xs], xp);
-                        if (++xs == NX) { xs = 0; xp ^= 1; }
-                    }
+            for (int t = 0; t < TILES; ++t) {
+                xt[t] = sm->x[xs] + x_off[t];
+                if (t < nt) {
+                    mbar_wait(S, &sm->x_full[xs], xp);
+                    if (TILES > 1 && ++xs == NX) { xs = 0; xp ^= 1; }
                 }
             }
-            if (threadIdx.x == 0 && first) trace(S, EV_X0, 0);
-            first = false;
-            // the k-splits of a slot take whole stages in turn, counted from the first chunk of the part
-            // (chunk kc belongs to split (kc - first) mod KS): a warp then multiplies all 32 k-steps of
-            // a stage, which amortises the per-stage waiting and set-up (splitting every stage among
-            // the warps streamed 20-30 % slower)
-            const bool here = kc < my_pub_k1 || kc >= my_own_k0;   // this slot has a stage at chunk kc
-            const int kbase = kc < my_pub_k1 ? 0 : my_own_k0;
-            if (here && ((kc - kbase) & (KS - 1)) == ks_id) {
-                const bool gap0 = slot_id > 0 && kc >= s0_pub_k1 && kc < s0_own_k0;   // slot 0 has none here
-                uint32_t i = r.w + (uint32_t)((stages_before(pl, ng, kc) + slot_id - gap0) * pair);
+        };
+        auto x_release = [&]() {
+            __syncwarp();
 #pragma unroll 1
-                for (int p = 0; p < pair; ++p, ++i) {
-                    w_wait(S, i, known);
-                    const uint32_t wslot = i % NW;
-                    const unsigned char *ws = sm->w[wslot] + a_off;
-                    if (packed) {
-                        if (p == 0) stage_packed(acc0[0], ws, xt[0], a_hi, a_sw);
-                        else stage_packed(acc1[0], ws, xt[0], a_hi, a_sw);
-                    } else if (nt == 1) {
-                        if (p == 0) stage_full<1>(acc0, ws, xt, a_hi, a_sw);
-                        else stage_full<1>(acc1, ws, xt, a_hi, a_sw);
-                    } else if (TILES > 1 && nt == 2) {
-                        if (p == 0) stage_full<TILES < 2 ? TILES : 2>(acc0, ws, xt, a_hi, a_sw);
-                        else stage_full<TILES < 2 ? TILES : 2>(acc1, ws, xt, a_hi, a_sw);
-                    } else if (TILES > 1) {
-                        if (p == 0) stage_full<TILES>(acc0, ws, xt, a_hi, a_sw);
-                        else stage_full<TILES>(acc1, ws, xt, a_hi, a_sw);
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
-                }
+            for (int t = 0; t < nt; ++t) {
+                if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
+                r.next_x();
             }
-            if ((kc & (XC - 1)) == XC - 1 || kc == nch - 1) {   // activation stages are shared: every warp waits for and releases each of them
-                __syncwarp();
+            x0 += XC;
+        };
+        x_wait();
+        if (threadIdx.x == 0 && first) trace(S, EV_X0, 0);
+        first = false;
 #pragma unroll 1
-                for (int t = 0; t < nt; ++t) {
-                    if (lane == 0) mbar_arrive(&sm->x_empty[r.xs]);
-                    r.next_x();
-                }
-            }
-            if (kc + 1 == my_pub_k1) {
+        for (int j = 0;; ++j) {
+            if (j == n_pub && my_pub_k1 > 0) {
                 // The head part of a split tile is complete: every k-split warp publishes its own sums
                 // (no meeting inside the CTA in the middle of the stream) and starts over for the tail
                 // part that may follow in this slot.
@@ -771,7 +853,47 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 }
                 clear();
             }
+            if (j >= n_all) break;
+            const int kc = chunk_of(j);
+            while (kc >= x0 + XC) { x_release(); x_wait(); }
+            const unsigned char *xc[TILES];
+#pragma unroll
+            for (int t = 0; t < TILES; ++t) xc[t] = xt[t] + (t == 0 ? (kc - x0) * cols.ncp * 4096 : 0);
+            uint32_t i = stage_of(kc);
+#pragma unroll 1
+            for (int p = 0; p < pair; ++p, ++i) {
+                if (PARK && n_used < n_parked) {
+                    const uint32_t at = tm + 128 * n_used++;
+                    if (packed) {
+                        if (p == 0) stage_parked<true>(acc0[0], at, xc[0]);
+                        else stage_parked<true>(acc1[0], at, xc[0]);
+                    } else {
+                        if (p == 0) stage_parked<false>(acc0[0], at, xc[0]);
+                        else stage_parked<false>(acc1[0], at, xc[0]);
+                    }
+                    continue;
+                }
+                w_wait(S, i, known);
+                const uint32_t wslot = i % NW;
+                const unsigned char *ws = sm->w[wslot] + a_off;
+                if (packed) {
+                    if (p == 0) stage_packed(acc0[0], ws, xc[0], a_hi, a_sw);
+                    else stage_packed(acc1[0], ws, xc[0], a_hi, a_sw);
+                } else if (nt == 1) {
+                    if (p == 0) stage_full<1>(acc0, ws, xc, a_hi, a_sw);
+                    else stage_full<1>(acc1, ws, xc, a_hi, a_sw);
+                } else if (TILES > 1 && nt == 2) {
+                    if (p == 0) stage_full<TILES < 2 ? TILES : 2>(acc0, ws, xc, a_hi, a_sw);
+                    else stage_full<TILES < 2 ? TILES : 2>(acc1, ws, xc, a_hi, a_sw);
+                } else if (TILES > 1) {
+                    if (p == 0) stage_full<TILES>(acc0, ws, xc, a_hi, a_sw);
+                    else stage_full<TILES>(acc1, ws, xc, a_hi, a_sw);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
+            }
         }
+        for (x_release(); x0 < nch; x_release()) x_wait();
         r.w += (uint32_t)(stages_before(pl, ng, nch) * pair);
         if (threadIdx.x == 0 && g.left <= CONS_WARPS) trace(S, EV_MAIN_END, 0);
         fold(d0, acc0);
@@ -844,10 +966,11 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             const int pr = act ? (col >> 1) - cols.cp0 : 0;
             const float *o = red + ((((slot & (TS - 1)) * TILES + (pr >> 2)) * 4 + 2 * (row >> 3) + (col & 1)) * 32 + ((row & 7) << 2) + (pr & 3));
             float v0[CONS_WARPS], v1[CONS_WARPS];
+            const int step = (TILES * 128) << lts;   // floats from one k-split to the next
 #pragma unroll
             for (int q = 0; q < CONS_WARPS; ++q) {
-                v0[q] = q < KS ? o[(q << lts) * (TILES * 128)] : 0.f;
-                v1[q] = q < KS && pair == 2 ? o[(CONS_WARPS + (q << lts)) * (TILES * 128)] : 0.f;
+                v0[q] = q < KS ? o[q * step] : 0.f;
+                v1[q] = q < KS && pair == 2 ? o[CONS_WARPS * (TILES * 128) + q * step] : 0.f;
             }
             float e0 = v0[0], e1 = v1[0];
 #pragma unroll
