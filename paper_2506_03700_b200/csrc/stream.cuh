@@ -249,6 +249,19 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t (&a)[4], const void *p) {
                  : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
                  : "r"(s32(p)));
 }
+__device__ __forceinline__ void ldmatrix_x4_at(uint32_t (&a)[4], uint32_t p) {   // (shared-memory address)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(p));
+}
+__device__ __forceinline__ uint4 lds128(uint32_t p) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t p) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(p));
+    return v;
+}
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&a)[4], const void *p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
@@ -572,15 +585,15 @@ struct NoHook {
 // Even k-steps accumulate into acc[0] (high parts) and acc[2] (low parts), odd ones into acc[1] and acc[3].  (A stage of one warp
 // is bound by the shared-memory reads of all eight, 200 cycles of the SM for 16 KB, not by the length of these chains.)
 template <int T>
-__device__ __forceinline__ void stage_full(float (&acc)[TILES][4][4], const unsigned char *ws, const unsigned char *const (&xs)[TILES], int a_hi, int a_sw) {
+__device__ __forceinline__ void stage_full(float (&acc)[TILES][4][4], uint32_t ws, const uint32_t (&xs)[TILES], int a_hi, int a_sw) {
     constexpr int PF = T == 1 ? 4 : 2;
     uint32_t a[PF][4];
     uint4 b[PF][T];
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
-        ldmatrix_x4(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
+        ldmatrix_x4_at(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
 #pragma unroll
-        for (int t = 0; t < T; ++t) b[j][t] = *reinterpret_cast<const uint4 *>(xs[t] + j * 128);
+        for (int t = 0; t < T; ++t) b[j][t] = lds128(xs[t] + j * 128);
     }
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
@@ -592,22 +605,22 @@ __device__ __forceinline__ void stage_full(float (&acc)[TILES][4][4], const unsi
         }
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
-            ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
+            ldmatrix_x4_at(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
 #pragma unroll
-            for (int t = 0; t < T; ++t) b[cur][t] = *reinterpret_cast<const uint4 *>(xs[t] + ks * 128);
+            for (int t = 0; t < T; ++t) b[cur][t] = lds128(xs[t] + ks * 128);
         }
     }
 }
 // The same for up to four columns: their high parts are token columns 0..3 of one multiply-add, their low parts 4..7.
 // Half the multiply-adds and half the shared-memory reads; every sum has the order it has above.
-__device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned char *ws, const unsigned char *xs, int a_hi, int a_sw) {
+__device__ __forceinline__ void stage_packed(float (&acc)[4][4], uint32_t ws, uint32_t xs, int a_hi, int a_sw) {
     constexpr int PF = 4;
     uint32_t a[PF][4];
     uint2 b[PF];
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
-        ldmatrix_x4(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
-        b[j] = *reinterpret_cast<const uint2 *>(xs + j * 128);
+        ldmatrix_x4_at(a[j], ws + (j >> 2) * 2048 + (((((j & 3) << 1) | a_hi) ^ a_sw) << 4));
+        b[j] = lds64(xs + j * 128);
     }
 #pragma unroll
     for (int j = 0; j < KSTEPS; ++j) {
@@ -615,8 +628,8 @@ __device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned 
         mma16816(acc[j & 1], a[cur], b[cur].x, b[cur].y);
         if (j + PF < KSTEPS) {
             const int ks = j + PF;
-            ldmatrix_x4(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
-            b[cur] = *reinterpret_cast<const uint2 *>(xs + ks * 128);
+            ldmatrix_x4_at(a[cur], ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
+            b[cur] = lds64(xs + ks * 128);
         }
     }
 }
@@ -624,7 +637,7 @@ __device__ __forceinline__ void stage_packed(float (&acc)[4][4], const unsigned 
 // A parked stage (see park_stage): the fragments come back from tensor memory, eight k-steps at a time, the next eight on their way
 // while these are multiplied.  The same multiply-adds in the same order as above.
 template <bool PACKED>
-__device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, const unsigned char *xs) {
+__device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, uint32_t xs) {
     uint32_t a[2][32];
     tmem_ld32_start(a[0], tm);
 #pragma unroll
@@ -632,12 +645,12 @@ __device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, co
         uint4 b[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const unsigned char *p = xs + (8 * h + j) * 128;
+            const uint32_t p = xs + (8 * h + j) * 128;
             if (PACKED) {
-                const uint2 v = *reinterpret_cast<const uint2 *>(p);
+                const uint2 v = lds64(p);
                 b[j] = make_uint4(v.x, v.y, 0, 0);
             } else {
-                b[j] = *reinterpret_cast<const uint4 *>(p);
+                b[j] = lds128(p);
             }
         }
         uint32_t(&cur)[32] = a[h & 1];
@@ -662,7 +675,7 @@ __device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, co
 // (13.4 -> 11.4), down 20.6 -> 19.2 (9.0 -> 7.7); short requests of the 1B shape 37.6 -> 34.7 ms.  (The kernel of
 // one column tile only: with 24 columns the products are bound by their activations.)
 constexpr int PARK_MAX = 2, PARK_COLS = 512;
-__device__ __forceinline__ void park_stage(const unsigned char *ws, int a_hi, int a_sw, uint32_t tm) {
+__device__ __forceinline__ void park_stage(uint32_t ws, int a_hi, int a_sw, uint32_t tm) {
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
         uint32_t v[32];
@@ -670,7 +683,7 @@ __device__ __forceinline__ void park_stage(const unsigned char *ws, int a_hi, in
         for (int j = 0; j < 8; ++j) {
             const int ks = 8 * h + j;
             uint32_t a[4];
-            ldmatrix_x4(a, ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
+            ldmatrix_x4_at(a, ws + (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4));
 #pragma unroll
             for (int i = 0; i < 4; ++i) v[4 * j + i] = a[i];
         }
@@ -778,7 +791,7 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                     }
                 }
                 if (!go) break;
-                park_stage(sm->w[wslot] + a_off, a_hi, a_sw, tm + 128 * n_parked);
+                park_stage(s32(sm->w[wslot]) + a_off, a_hi, a_sw, tm + 128 * n_parked);
                 ++n_parked;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
@@ -809,12 +822,12 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
         // Activation stages are shared: every warp waits for and releases each of them.  A warp goes from one of its own chunks to the
         // next; looking at every chunk cost 400 cycles for each that is not its own, which parked stages would not have hidden.
         int x0 = 0;                       // first chunk of the activation stage(s) at hand
-        const unsigned char *xt[TILES];   // this lane's bytes of them, by column tile
+        uint32_t xt[TILES];               // this lane's bytes of them, by column tile
         auto x_wait = [&]() {
             uint32_t xs = r.xs, xp = r.xp;
 #pragma unroll
             for (int t = 0; t < TILES; ++t) {
-                xt[t] = sm->x[xs] + x_off[t];
+                xt[t] = s32(sm->x[xs]) + x_off[t];
                 if (t < nt) {
                     mbar_wait(S, &sm->x_full[xs], xp);
                     if (TILES > 1 && ++xs == NX) { xs = 0; xp ^= 1; }
@@ -856,7 +869,7 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
             if (j >= n_all) break;
             const int kc = chunk_of(j);
             while (kc >= x0 + XC) { x_release(); x_wait(); }
-            const unsigned char *xc[TILES];
+            uint32_t xc[TILES];
 #pragma unroll
             for (int t = 0; t < TILES; ++t) xc[t] = xt[t] + (t == 0 ? (kc - x0) * cols.ncp * 4096 : 0);
             uint32_t i = stage_of(kc);
@@ -875,7 +888,7 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 }
                 w_wait(S, i, known);
                 const uint32_t wslot = i % NW;
-                const unsigned char *ws = sm->w[wslot] + a_off;
+                const uint32_t ws = s32(sm->w[wslot]) + a_off;
                 if (packed) {
                     if (p == 0) stage_packed(acc0[0], ws, xc[0], a_hi, a_sw);
                     else stage_packed(acc1[0], ws, xc[0], a_hi, a_sw);
