@@ -1757,10 +1757,10 @@ __global__ void k_prefill_arm(Ctx c, int seq, int n_prompt) {
 // Warps 0-7 consume, warp 8 produces weights and K / V blocks, warp 9 activations and queries; warps 10 and 11 only complete the producers'
 // warp group, which hands registers to the consumers.  (At 168 registers a thread -- three warps on a quarter of the SM --
 // the consumers kept loop variables in local memory, whose L1 lines do not survive the acquires of the grid barrier: a round trip to
-// L2 for each on the critical path of a phase.  One column tile: at 200 / 104 nothing is spilled; 216 / 72 spilled 64 bytes in the
-// producers and cost 0.5 to 2 % of a request.  Three tiles: 216 / 72 spills 132 bytes, 208 / 88 40, 200 / 104 148, no difference measured.)
+// L2 for each on the critical path of a phase.  At 200 / 104 one column tile spills nothing; 216 / 72 spilled 64 bytes in the
+// producers and cost 0.5 to 2 % of a request.  Three tiles: 120 bytes at 216 / 72, 40 at 200 / 104, no difference measured.)
 constexpr int MEGA_THREADS = CONS_THREADS + 128;
-constexpr int REGS_CONSUME = TILES == 1 ? 200 : 208, REGS_PRODUCE = TILES == 1 ? 104 : 88;
+constexpr int REGS_CONSUME = 200, REGS_PRODUCE = 104;
 constexpr int MEGA_REGS = CONS_THREADS * REGS_CONSUME + 128 * REGS_PRODUCE;   // the block must have been launched with as many
 
 template <int HD>
