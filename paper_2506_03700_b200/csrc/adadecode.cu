@@ -928,8 +928,10 @@ int setup_resident(ada_session *S, const Layout &lay) {
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     CK(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    S->res_smem = fit.smem;
     if (fit.smem > (size_t)smem) return ADA_OK;
+    const size_t page_words = (size_t)S->batch * S->max_pages, page_bytes = page_words * sizeof(int32_t);
+    const bool pages = page_bytes <= 4096 && fit.smem + page_bytes <= std::min((size_t)smem, kSharedMax);   // the page table too, where there is room
+    S->res_smem = fit.smem + (pages ? page_bytes : 0);
     if (!coop) return ADA_OK;
     const void *kern = resident_kernel(g.head_dim);
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -951,6 +953,7 @@ int setup_resident(ada_session *S, const Layout &lay) {
     a.R = R;
     a.ku = fit.ku;
     a.cs_ring = fit.ring;
+    a.page_words = pages ? (int)page_words : 0;
     a.pf_rows = std::min(R, rs::TOK_RING);
     rs::u64 *w = (rs::u64 *)((char *)S->scratch + lay.res);
     auto take = [&](size_t n) { rs::u64 *at = w; w += n; return at; };

@@ -56,6 +56,7 @@ struct Args {
     int R;                               // rows of the buffers
     int ku;                              // widest product input: max(d_model, q width, d_ff)
     int cs_ring;                         // rotary factors kept per sequence (a power of two above the rows in flight)
+    int page_words;                      // entries of the page table that are kept in shared memory: all, or none
     int store_logits, prof;
     int pf_seq, pf_n;                    // prompt passes of this sequence (pf_n tokens), or pf_n = 0: decode
     int pf_rows;                         // prompt positions per pass
@@ -159,7 +160,8 @@ template <int NW, class Ptr> struct Product {
     __device__ __forceinline__ Product(const Ptr &p, int K_, int units_, u64 mask, bool same_warp = false)
         : wptr(p), K(K_), units(units_), groups((popc64(mask) + 7) >> 3), first((int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x), stride(WARPS * (int)gridDim.x) {
         pitch = same_warp ? (units + stride - 1) / stride * stride : units;
-        if (first < pitch * groups && first % pitch < units) load_w<NW>(r, wptr, first % pitch, K, 0);
+        const int unit = groups == 1 ? first : first % pitch;   // (up to eight rows: no division in front of the first load)
+        if (first < pitch * groups && unit < units) load_w<NW>(r, wptr, unit, K, 0);
     }
     // Two rows at a time; a weight row of up to 128 U elements is loaded once for all rows of the group.
     template <class Out> __device__ __forceinline__ void run(const float *us, int ldu, u64 mask, Out &&out) {
@@ -167,7 +169,7 @@ template <int NW, class Ptr> struct Product {
         int at = 0;   // piece of the unit's weights in registers
 #pragma unroll 1
         for (int wk = first; wk < pitch * groups; wk += stride) {
-            const int unit = wk % pitch, grp = wk / pitch;
+            const int grp = groups == 1 ? 0 : wk / pitch, unit = wk - grp * pitch;
             if (unit >= units) continue;
             u64 m = mask;
             for (int i = 0; i < 8 * grp; ++i) m &= m - 1;
@@ -386,6 +388,18 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         return ok;
     }
 
+    // EPL elements of a cache row, or zeros
+    __device__ __forceinline__ static void cached(float (&v)[EPL], const float *p, bool there) {
+        if constexpr (EPL == 1) v[0] = there ? __ldcg(p) : 0.f;
+        else {
+#pragma unroll
+            for (int e = 0; e < EPL; e += 2) {
+                const float2 x = there ? __ldcg(reinterpret_cast<const float2 *>(p + e)) : make_float2(0.f, 0.f);
+                v[e] = x.x;
+                v[e + 1] = x.y;
+            }
+        }
+    }
     // ---- attention: one (row, q head, 128-position chunk) per CTA at a time, sixteen positions per warp.  Positions of this pass
     // come from the exchanged words, earlier ones from the cache (requested before the queries have arrived).
     __device__ __noinline__ void attention(int l, u64 mask, unsigned tag) {
@@ -414,11 +428,8 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
 #pragma unroll
             for (int u = 0; u < 16; ++u) {
                 const bool old = t0 + u <= pos && t0 + u < lo;
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) {
-                    kk[u][e] = old ? __ldcg(kp + u * HD + e) : 0.f;
-                    vv[u][e] = old ? __ldcg(vp + u * HD + e) : 0.f;
-                }
+                cached(kk[u], kp + u * HD, old);
+                cached(vv[u], vp + u * HD, old);
             }
             until(A, s.st, [&]() {
                 bool ok = words(A.QT + (size_t)r * c.qkv_rows + h * HD + lane() * EPL, q, want);
@@ -595,6 +606,9 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         const float scale = layer1 > 0 ? A.head_scale[layer1] : 1.0f;
         const int n_units = (c.vocab + 1) / 2;
         auto wptr = [&](int u, int i) -> const float * { return 2 * u + i < c.vocab ? A.lm_head + (size_t)(2 * u + i) * c.d : nullptr; };
+        // What this thread stored plainly in the step (cache rows, residuals) is ordered before the partials below; here, where it waits
+        // for the layer's output anyway.
+        __threadfence();
         if (T) {
             auto tptr = [&](int u, int) { return T + (size_t)u * c.d; };
             Product<1, decltype(tptr)> p(tptr, c.d, c.d, mask);
@@ -610,7 +624,6 @@ template <int EPL> struct Walker {   // EPL = head_dim / 32
         Product<2, decltype(wptr)> p(wptr, c.d, n_units, mask, true);
         if (T) load_words(mask, A.TT, tag - 1, c.d);
         else load_norm(mask, A.XA, tag_x, -1, A.final_norm);
-        __threadfence();   // what this thread stored plainly in the step is ordered before the partials below
         __syncthreads();
         p.run(s.us, A.ku, mask, [&](int u, int r, float (&a)[2]) {
             if (lane() != 0) return;
@@ -995,6 +1008,11 @@ template <int EPL> __global__ void __launch_bounds__(THREADS, 1) k_decode_reside
         w.t_last = now();
     }
     __syncthreads();
+    if (args.page_words > 0) {   // the page table, behind the rest: an entry is looked up for every cache row that is written or read, each a load from L2
+        int32_t *table = reinterpret_cast<int32_t *>(w.s.st + 1);
+        for (int i = threadIdx.x; i < args.page_words; i += THREADS) table[i] = c.page_table[i];
+        if (threadIdx.x == 0) w.A.c.page_table = table;
+    }
     for (int j = threadIdx.x; j < c.hd / 2; j += THREADS) w.s.freq[j] = pow((double)args.rope_base, -2.0 * j / c.hd);
     __syncthreads();
     if (args.pf_n > 0) w.prefill();
