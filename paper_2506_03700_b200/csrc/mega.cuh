@@ -516,6 +516,23 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
 // Applies the outcome of the step that just ended (Eq. 1 after a head; verification and rollback,
 // Eq. 2 at temperature zero, after the final head), then sets up the next step: its columns, the
 // embedding of its newest token, that token's rotary table; finally publishes the action.
+// What the bookkeeping works on, in the consumers' scratch.  (The next step's descriptor and the sequences' lengths as arrays of the
+// bookkeeping thread were local memory, a load from L2 for each first touch behind the barrier's acquire: 13 us with eight sequences.)
+struct Ctl {
+    StepDesc nd;
+    int len[MAX_SEQS], base[MAX_SEQS], target[MAX_SEQS], done[MAX_SEQS];
+    int newest[MAX_SEQS];      // the newest token
+};
+constexpr int CTL_OFFSET = 8192 + ((int)sizeof(HeadResult) + 4) * MAX_COLS;
+static_assert(CTL_OFFSET % 16 == 0 && CTL_OFFSET + (int)sizeof(Ctl) <= DRAW_OFFSET, "the control point's copies overlap the draw's buffers");
+
+// eight neighbouring bf16 elements; `aligned`: their address is a multiple of 16
+__device__ __forceinline__ uint4 load_bf16x8(const __nv_bfloat16 *p, bool aligned) {
+    if (aligned) return __ldg(reinterpret_cast<const uint4 *>(p));
+    const unsigned short *h = reinterpret_cast<const unsigned short *>(p);
+    return make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16, h[6] | (uint32_t)h[7] << 16);
+}
+
 __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int kind, int e, unsigned pub_no, const StepDesc &dprev,
                                           int &steps_started) {
     const Ctx &c = A.c;
@@ -531,7 +548,20 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     HeadResult *hr_s = reinterpret_cast<HeadResult *>(sm->scratch + 8192);                       // [MAX_COLS]
     int *tok_s = reinterpret_cast<int *>(sm->scratch + 8192 + sizeof(HeadResult) * MAX_COLS);    // [MAX_COLS]: the token after the column's own
     static_assert(ADA_MAX_LAYERS * MAX_SEQS * sizeof(int) <= 8192, "fill levels of a launch's sequences must fit the scratch corner");
+    Ctl &ctl = *reinterpret_cast<Ctl *>(sm->scratch + CTL_OFFSET);
+    StepDesc &nd = ctl.nd;
     for (int i = tid; i < nseq * L; i += CONS_THREADS) fill_s[i] = c.fill[(size_t)seq0 * L + i];
+    if (tid < (int)(sizeof(StepDesc) / 4)) reinterpret_cast<int *>(&nd)[tid] = reinterpret_cast<const int *>(&dprev)[tid];
+    if (tid >= 64 && tid < 64 + MAX_SEQS) {
+        const int k = tid - 64, s = seq0 + k;
+        const bool in = k < nseq;
+        const int ln = in ? st->len[s] : 0;
+        ctl.len[k] = ln;
+        ctl.base[k] = in ? st->base[s] : 0;
+        ctl.target[k] = in ? st->target_len[s] : 0;
+        ctl.done[k] = in ? st->done[s] : 1;
+        ctl.newest[k] = in && ln > 0 && ln <= c.max_seq ? c.tokens[(size_t)s * c.max_seq + ln - 1] : 0;
+    }
     if (tid >= CONS_THREADS - MAX_COLS) {
         const int j = tid - (CONS_THREADS - MAX_COLS), k = j % nseq;
         int v = -1;
@@ -560,34 +590,40 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                       kind == CTRL_HEAD ? (int)M.exit_at[e] - 1 : 0, A.head_part, G};
         sample_stage(sa, sm, kind == CTRL_HEAD, &dprev, head_cols);
     }
-    // (b) bookkeeping, one thread.  Every scalar it may need is read up front (the loads overlap);
-    // counters are bumped by reductions, which do not wait for memory.
-    if (tid == 0) {
-        auto bump = [](long long *p, long long v) { atomicAdd(reinterpret_cast<unsigned long long *>(p), (unsigned long long)v); };
+    // (b) bookkeeping, one warp: every lane follows the same decisions, lane 0 writes them down, loops over the layers are shared out.
+    // Every scalar it may need is read up front (the loads overlap); counters are bumped by reductions, which do not wait for memory.
+    if (tid < 32) {
+        const int lane = tid;
+        const bool w0 = lane == 0;
+        auto bump = [&](long long *p, long long v) { if (w0) atomicAdd(reinterpret_cast<unsigned long long *>(p), (unsigned long long)v); };
+        // fill levels of sequence k at layers below n become `to`; the sum of (from - old level)
+        auto refill = [&](int k, int n, int from, int to) {
+            int rl = 0;
+            for (int l = lane; l < n; l += 32) {
+                rl += from - fill_s[k * L + l];
+                fill_s[k * L + l] = to;
+                c.fill[(size_t)(seq0 + k) * L + l] = to;
+            }
+            return (long long)__reduce_add_sync(0xffffffffu, rl);
+        };
         const int err0 = *(volatile int *)A.err;
         const int pf_end0 = st->pf_end, pf_pos0 = st->pf_pos, max_early0 = st->max_early;
         const int tape_n0 = st->tape_n, hl_n0 = st->head_log_n;
-        int tape_i = st->tape_i, hl_n = hl_n0;
+        const int tape_i0 = st->tape_i;
+        int tape_i = tape_i0, hl_n = hl_n0;
         const float gamma0 = st->gamma;
         const int eos0 = st->eos_id;
         const long long steps0 = __ldcg(&st->st.steps);   // past the L1: the counters are bumped by reductions
-        int len[MAX_SEQS], base[MAX_SEQS], target[MAX_SEQS], done[MAX_SEQS];
-#pragma unroll
-        for (int k = 0; k < MAX_SEQS; ++k) {
-            const bool in = k < nseq;
-            len[k] = in ? st->len[seq0 + k] : 0; base[k] = in ? st->base[seq0 + k] : 0;
-            target[k] = in ? st->target_len[seq0 + k] : 0; done[k] = in ? st->done[seq0 + k] : 1;
-        }
         int action = ACT_NEWSTEP, verified = 0;
+        int keep_rows = 0, keep_row0 = 0;
         int pf_end = pf_end0, pf_pos = pf_pos0;
-        StepDesc nd = dprev;
         if (err0 != 0) action = ACT_STOP;
         // ---- Eq. 1 after an intermediate head: every sequence whose newest token consulted it decides for itself
         if (action != ACT_STOP && kind == CTRL_HEAD) {
             unsigned still = 0;   // sequences that go on climbing in this step
             int n_steps_seen = 0;
             for (int k = 0; k < nseq; ++k) {
-                const int s = seq0 + k, col = (len[k] - 1 - base[k]) * nseq + k;
+                const int s = seq0 + k, len = ctl.len[k], col = (len - 1 - ctl.base[k]) * nseq + k;
                 if (col < 0 || col >= MAX_COLS || dprev.first_layer[col] > e - 1) continue;   // not in this step any more
                 if (!((head_cols >> col) & 1u)) { still |= 1u << k; continue; }                // climbing, but may not exit early
                 const HeadResult hr = hr_s[col];
@@ -600,31 +636,29 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                 bump(&st->st.head_evals, 1);
                 if (s == 0 && c.head_log && hl_n < kHeadLogCap) {
                     float *hl = c.head_log + 4 * (size_t)hl_n;
-                    hl[0] = (float)(steps0 + n_steps_seen); hl[1] = (float)e; hl[2] = (float)hr.token; hl[3] = hr.p;
+                    if (w0) { hl[0] = (float)(steps0 + n_steps_seen); hl[1] = (float)e; hl[2] = (float)hr.token; hl[3] = hr.p; }
                     ++hl_n;
                 }
                 if (!decide) { still |= 1u << k; continue; }
-                long long rl = 0;
-                for (int l = 0; l < e; ++l) {
-                    rl += len[k] - fill_s[k * L + l];
-                    fill_s[k * L + l] = len[k];
-                    c.fill[(size_t)s * L + l] = len[k];
+                bump(&st->st.row_layers, refill(k, e, len, len));
+                const int token = min(max(hr.token, 0), c.vocab - 1);
+                if (w0) {
+                    c.tokens[(size_t)s * c.max_seq + len] = token;
+                    ctl.newest[k] = token;
+                    ctl.len[k] = len + 1;
+                    st->len[s] = len + 1;
+                    for (int j = k; j < MAX_COLS; j += nseq) {   // the sequence sits out the rest of the step
+                        nd.first_layer[j] = NO_LAYER;
+                        nd.head_mask &= ~(1 << j);
+                    }
                 }
-                bump(&st->st.row_layers, rl);
-                c.tokens[(size_t)s * c.max_seq + len[k]] = min(max(hr.token, 0), c.vocab - 1);
-                len[k] += 1;
-                st->len[s] = len[k];
                 bump(&st->st.early_exits, 1);
                 bump(&st->st.exits_at_layer[e], 1);
                 bump(&st->st.steps, 1);
                 ++n_steps_seen;
-                for (int j = k; j < MAX_COLS; j += nseq) {   // the sequence sits out the rest of the step
-                    nd.first_layer[j] = NO_LAYER;
-                    nd.head_mask &= ~(1 << j);
-                }
             }
-            if (tape_i != st->tape_i) st->tape_i = tape_i;
-            if (hl_n != hl_n0) st->head_log_n = hl_n;
+            if (w0 && tape_i != tape_i0) st->tape_i = tape_i;
+            if (w0 && hl_n != hl_n0) st->head_log_n = hl_n;
             if (still) action = ACT_CONTINUE;
             else bump(&st->st.layer_passes, e);   // the weights of layers 1..e were streamed once, for all the sequences
         }
@@ -632,57 +666,60 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         if (action != ACT_STOP && kind == CTRL_TOP && prefilling) {
             // a pass over prompt positions [pf_pos, pf_pos + n) of the launch's one sequence is complete at every layer
             const int s = seq0, n = dprev.n_cols, end = pf_pos + n;
-            for (int l = 0; l < L; ++l) { fill_s[l] = end; c.fill[(size_t)s * L + l] = end; }
+            refill(0, L, 0, end);
             pf_pos = end;
-            st->pf_pos = end;
+            if (w0) st->pf_pos = end;
             if (end >= pf_end) {   // KV cache <- LM(x) done: the full-depth argmax at the last prompt token is the first generated token
-                const int np = pf_end;
-                c.tokens[(size_t)s * c.max_seq + np] = min(max(hr_s[n - 1].token, 0), c.vocab - 1);
-                len[0] = np + 1; base[0] = np; done[0] = 1; pf_end = 0;
-                st->len[s] = np + 1;
-                st->base[s] = np;
-                st->n_prompt[s] = np;
-                st->done[s] = 1;
-                st->pf_end = 0;
-                st->keep_rows = 1;
-                st->keep_row0 = n - 1;
+                const int np = pf_end, token = min(max(hr_s[n - 1].token, 0), c.vocab - 1);
+                pf_end = 0;
+                keep_rows = 1;
+                keep_row0 = n - 1;
                 verified = s == 0;
+                if (w0) {
+                    c.tokens[(size_t)s * c.max_seq + np] = token;
+                    ctl.newest[0] = token;
+                    ctl.len[0] = np + 1; ctl.base[0] = np; ctl.done[0] = 1;
+                    st->len[s] = np + 1;
+                    st->base[s] = np;
+                    st->n_prompt[s] = np;
+                    st->done[s] = 1;
+                    st->pf_end = 0;
+                    st->keep_rows = 1;
+                    st->keep_row0 = n - 1;
+                }
             }
         }
         // ---- verification (Eq. 2 at temperature zero) of every sequence whose newest token reached the last layer
         if (action != ACT_STOP && kind == CTRL_TOP && !prefilling) {
             for (int k = 0; k < nseq; ++k) {
-                const int s = seq0 + k, nrow = len[k] - base[k];
+                const int s = seq0 + k, len = ctl.len[k], base = ctl.base[k], nrow = len - base;
                 if (nrow < 1 || nrow > cps || dprev.first_layer[(nrow - 1) * nseq + k] > L - 1) continue;   // left the step at an exit layer, or idle
                 int32_t *tok = c.tokens + (size_t)s * c.max_seq;
-                long long rl = 0;
-                for (int l = 0; l < L; ++l) rl += len[k] - fill_s[k * L + l];
-                bump(&st->st.row_layers, rl);
                 int bad = -1;
                 for (int j = 0; j + 1 < nrow; ++j)
                     if (hr_s[j * nseq + k].token != tok_s[j * nseq + k]) { bad = j; break; }
                 int new_base, keep;
+                const int token = min(max(hr_s[(bad < 0 ? nrow - 1 : bad) * nseq + k].token, 0), c.vocab - 1);
                 if (bad < 0) {
                     bump(&st->st.accepted, nrow - 1);
-                    tok[len[k]] = min(max(hr_s[(nrow - 1) * nseq + k].token, 0), c.vocab - 1);
-                    new_base = len[k];
+                    new_base = len;
                     keep = nrow;
                 } else {
                     bump(&st->st.accepted, bad);
                     bump(&st->st.rejected, 1);
                     bump(&st->st.discarded, nrow - 2 - bad);
-                    new_base = base[k] + bad + 1;
-                    tok[new_base] = min(max(hr_s[bad * nseq + k].token, 0), c.vocab - 1);
+                    new_base = base + bad + 1;
                     keep = bad + 1;
                 }
+                if (w0) tok[new_base] = token;
                 // Algorithm 1 runs "while t_i != [EOS]": the verified tokens of this step (positions base + 1 .. new_base,
                 // each equal to the full-depth argmax of the row before it) end the sequence at the first end-of-sequence
                 // token among them.  An early-predicted end-of-sequence token stops nothing until it is verified here.
-                int tgt = target[k];
+                int tgt = ctl.target[k];
                 if (eos0 >= 0) {
                     for (int j = 0; j < keep; ++j)
                         if (min(max(hr_s[j * nseq + k].token, 0), c.vocab - 1) == eos0) {
-                            if (base[k] + j + 2 <= tgt) { tgt = base[k] + j + 2; st->eos_hit[s] = 1; }
+                            if (base + j + 2 <= tgt) { tgt = base + j + 2; if (w0) st->eos_hit[s] = 1; }
                             break;
                         }
                 }
@@ -692,138 +729,153 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
                     new_len = tgt;
                     new_base = new_len - 1;
                 }
-                keep = new_len - 1 - base[k];   // verified tokens that stay: their logit rows are the ones a capture keeps
-                for (int l = 0; l < L; ++l) { fill_s[k * L + l] = new_base; c.fill[(size_t)s * L + l] = new_base; }
-                len[k] = new_len; base[k] = new_base;
-                st->len[s] = new_len;
-                st->base[s] = new_base;
+                keep = new_len - 1 - base;   // verified tokens that stay: their logit rows are the ones a capture keeps
+                bump(&st->st.row_layers, refill(k, L, len, new_base));
+                if (w0) {
+                    ctl.newest[k] = token;   // (a sequence that was cut short is done, and embeds nothing)
+                    ctl.len[k] = new_len; ctl.base[k] = new_base;
+                    st->len[s] = new_len;
+                    st->base[s] = new_base;
+                    if (new_len >= tgt) { ctl.done[k] = 1; st->done[s] = 1; }
+                }
                 bump(&st->st.verify_steps, 1);
                 bump(&st->st.steps, 1);
-                if (new_len >= tgt) { done[k] = 1; st->done[s] = 1; }
                 if (s == 0) {
-                    st->keep_rows = keep;
-                    st->keep_row0 = 0;
+                    keep_rows = keep;
+                    keep_row0 = 0;
+                    if (w0) { st->keep_rows = keep; st->keep_row0 = 0; }
                     verified = 1;
                 }
             }
         }
+        __syncwarp();
         if (action != ACT_STOP && kind == CTRL_TOP && !prefilling) bump(&st->st.layer_passes, L);
         if (action == ACT_NEWSTEP) {
             bool all_done = true;
-            for (int k = 0; k < nseq; ++k) all_done = all_done && done[k];
-            if (all_done) { action = ACT_STOP; st->n_done = 1; }
+            for (int k = 0; k < nseq; ++k) all_done = all_done && ctl.done[k];
+            if (all_done) { action = ACT_STOP; if (w0) st->n_done = 1; }
             else if (steps_started >= A.step_budget) action = ACT_STOP;
         }
         if (action == ACT_NEWSTEP) {
             ++steps_started;
-            nd.n_cols = 0; nd.newest_mask = 0; nd.head_mask = 0; nd.pmax = 0; nd.fresh = 0; nd.run_final = 1;
-            for (int j = 0; j < MAX_COLS; ++j) { nd.first_layer[j] = NO_LAYER; nd.pos[j] = 0; }
-            for (int k = 0; k < MAX_SEQS; ++k) nd.seq_pmax[k] = -1;
+            int n_cols = 0, newest_mask = 0, head_mask = 0, pmax = 0, fresh = 0, run_final = 1;
+            if (lane < MAX_COLS) { nd.first_layer[lane] = NO_LAYER; nd.pos[lane] = 0; }
+            if (lane < MAX_SEQS) nd.seq_pmax[lane] = -1;
+            __syncwarp();
             if (pf_end > 0) {   // next pass over the prompt: up to eight positions, all from layer 1
                 const int n = min(MAX_COLS, pf_end - pf_pos);
-                nd.n_cols = n;
-                nd.newest_mask = 1 << (n - 1);
-                nd.pmax = pf_pos + n - 1;
-                nd.seq_pmax[0] = nd.pmax;
-                nd.fresh = (1 << n) - 1;
-                nd.run_final = pf_pos + n >= pf_end;
-                if (n < 1 || nd.pmax >= c.max_seq) {
-                    atomicCAS(A.err, 0, ERR_BAD_STATE);
+                n_cols = n;
+                newest_mask = 1 << (n - 1);
+                pmax = pf_pos + n - 1;
+                fresh = (1 << n) - 1;
+                run_final = pf_pos + n >= pf_end;
+                if (n < 1 || pmax >= c.max_seq) {
+                    if (w0) atomicCAS(A.err, 0, ERR_BAD_STATE);
                     action = ACT_STOP;
                 }
-                for (int j = 0; j < n; ++j) { nd.first_layer[j] = 0; nd.pos[j] = pf_pos + j; }
+                if (lane < n) { nd.first_layer[lane] = 0; nd.pos[lane] = pf_pos + lane; }
+                if (w0) nd.seq_pmax[0] = pmax;
             } else {
                 for (int k = 0; k < nseq; ++k) {
-                    if (done[k]) continue;   // a sequence that has reached its target idles while the others go on
-                    const int nrow = len[k] - base[k];
-                    if (nrow < 1 || nrow > cps || nrow * nseq > MAX_COLS || len[k] > c.max_seq || base[k] < 0) {
-                        atomicCAS(A.err, 0, ERR_BAD_STATE);
+                    if (ctl.done[k]) continue;   // a sequence that has reached its target idles while the others go on
+                    const int len = ctl.len[k], base = ctl.base[k], nrow = len - base;
+                    if (nrow < 1 || nrow > cps || nrow * nseq > MAX_COLS || len > c.max_seq || base < 0) {
+                        if (w0) atomicCAS(A.err, 0, ERR_BAD_STATE);
                         action = ACT_STOP;
                         break;
                     }
                     for (int j = 0; j < nrow; ++j) {
-                        const int pos = base[k] + j;
+                        const int pos = base + j;
                         int fl = 0;
-                        for (int l = 0; l < L; ++l) fl += fill_s[k * L + l] > pos;
-                        nd.first_layer[j * nseq + k] = (unsigned char)fl;
-                        nd.pos[j * nseq + k] = pos;
+                        for (int l = lane; l < L; l += 32) fl += fill_s[k * L + l] > pos;
+                        fl = __reduce_add_sync(0xffffffffu, fl);
+                        if (w0) { nd.first_layer[j * nseq + k] = (unsigned char)fl; nd.pos[j * nseq + k] = pos; }
                     }
                     const int cn = (nrow - 1) * nseq + k;
-                    nd.n_cols += nrow;
-                    nd.newest_mask |= 1 << cn;
-                    nd.fresh |= 1 << cn;
-                    if (nrow - 1 < max_early0 && len[k] < target[k]) nd.head_mask |= 1 << cn;
-                    nd.seq_pmax[k] = len[k] - 1;
-                    nd.pmax = max(nd.pmax, len[k] - 1);
+                    n_cols += nrow;
+                    newest_mask |= 1 << cn;
+                    fresh |= 1 << cn;
+                    if (nrow - 1 < max_early0 && len < ctl.target[k]) head_mask |= 1 << cn;
+                    if (w0) nd.seq_pmax[k] = len - 1;
+                    pmax = max(pmax, len - 1);
                 }
             }
+            if (w0) { nd.n_cols = n_cols; nd.newest_mask = newest_mask; nd.head_mask = head_mask; nd.pmax = pmax; nd.fresh = fresh; nd.run_final = run_final; }
         }
-        if (action == ACT_NEWSTEP || action == ACT_CONTINUE) pub->d = nd;
-        pub->action = action;
-        pub->cap_keep = 0;
-        if (kind == CTRL_TOP && c.capture && verified) {
-            const int at = st->capture_n, keep = min(st->keep_rows, st->capture_cap - at);
-            pub->cap_keep = max(keep, 0);
-            pub->cap_at = at;
-            pub->cap_row0 = st->keep_row0;
-            if (keep > 0) st->capture_n = at + keep;
+        __syncwarp();
+        if (action == ACT_NEWSTEP || action == ACT_CONTINUE)
+            for (int i = lane; i < (int)(sizeof(StepDesc) / 4); i += 32) reinterpret_cast<int *>(&pub->d)[i] = reinterpret_cast<const int *>(&nd)[i];
+        if (w0) {
+            pub->action = action;
+            pub->cap_keep = 0;
+            if (kind == CTRL_TOP && c.capture && verified) {
+                const int at = st->capture_n, keep = min(keep_rows, st->capture_cap - at);
+                pub->cap_keep = max(keep, 0);
+                pub->cap_at = at;
+                pub->cap_row0 = keep_row0;
+                if (keep > 0) st->capture_n = at + keep;
+            }
+            sm->bcast[0] = action;
         }
-        sm->bcast[0] = action;
     }
     bar_consumers();
     const int action = sm->bcast[0];
-    // (c) the embedding of the next newest token
+    // (c) the embeddings of the tokens that enter, and their rotary factors
     if (action == ACT_NEWSTEP) {
-        const StepDesc &nd = pub->d;
         const __nv_bfloat16 *g0 = M.attn_norm[0];
-        const int half = c.hd / 2;
-        for (int col = 0; col < MAX_COLS; ++col) {
-            if (!((nd.fresh >> col) & 1)) continue;
-            const int pos = nd.pos[col];
-            const int tokid = min(max(c.tokens[(size_t)(seq0 + (nseq == 1 ? 0 : col % nseq)) * c.max_seq + pos], 0), c.vocab - 1);
-            const __nv_bfloat16 *erow = M.tok_embed + (size_t)tokid * c.d;
-            for (int n0 = 0; n0 < c.d; n0 += 8 * CONS_THREADS) {   // eight loads of the embedding row and of the gain in flight per thread
-                float v[8], gn[8];
+        const int half = c.hd / 2, nf = __popc(nd.fresh);
+        for (int i = tid; i < nf * half; i += CONS_THREADS) {
+            const int w = i % half;
+            unsigned m = (unsigned)nd.fresh;
+            for (int q = i / half; q > 0; --q) m &= m - 1;
+            const int col = __ffs(m) - 1, pos = nd.pos[col];
+            // angle = pos * freq in double, reduced to [-pi, pi] in double, then single-precision sin / cos
+            // (double-precision transcendentals with large arguments are slow on this GPU)
+            const double a = (double)pos * A.rope_freq[w];
+            const double r = a - 6.283185307179586476925 * rint(a * 0.15915494309189533577);
+            float sn, cs;
+            sincosf((float)r, &sn, &cs);
+            c.rope_cs[((size_t)col * half + w) * 2 + 0] = cs;
+            c.rope_cs[((size_t)col * half + w) * 2 + 1] = sn;
+        }
+        // 8 / 4 / 2 / 1 warps a column, eight elements a lane and turn, the next turn's loads in flight
+        const int ws = nf == 1 ? 3 : nf == 2 ? 2 : nf <= 4 ? 1 : 0, at = 8 * (tid & ((32 << ws) - 1)), step = 256 << ws;
+#pragma unroll 1
+        for (int f = tid >> (5 + ws); f < nf; f += CONS_WARPS >> ws) {
+            unsigned m = (unsigned)nd.fresh;
+            for (int q = f; q > 0; --q) m &= m - 1;
+            const int col = __ffs(m) - 1, k = nseq == 1 ? 0 : col % nseq;
+            const int token = st->pf_end > 0 ? c.tokens[(size_t)(seq0 + k) * c.max_seq + nd.pos[col]] : ctl.newest[k];
+            const __nv_bfloat16 *erow = M.tok_embed + (size_t)min(max(token, 0), c.vocab - 1) * c.d;
+            const bool al = ((reinterpret_cast<uintptr_t>(erow) | reinterpret_cast<uintptr_t>(g0)) & 15) == 0;
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            uint4 ev = at < c.d ? load_bf16x8(erow + at, al) : zero, gv = at < c.d ? load_bf16x8(g0 + at, al) : zero;
+#pragma unroll 1
+            for (int n0 = 0; n0 < c.d; n0 += step) {
+                const int n = n0 + at, nn = n + step;
+                const uint32_t e[4] = {ev.x, ev.y, ev.z, ev.w}, g[4] = {gv.x, gv.y, gv.z, gv.w};
+                ev = nn < c.d ? load_bf16x8(erow + nn, al) : zero;
+                gv = nn < c.d ? load_bf16x8(g0 + nn, al) : zero;
+                float v[8], q[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int n = n0 + u * CONS_THREADS + tid;
-                    v[u] = n < c.d ? __bfloat162float(erow[n]) : 0.f;
-                    gn[u] = n < c.d ? __bfloat162float(g0[n]) : 0.f;
-                }
+                for (int i = 0; i < 8; ++i) { v[i] = bf16_of_word(e[i >> 1], i); q[i] = __fmul_rn(v[i], v[i]); }
+                // sum of the squares of sixteen neighbours, as a tree
+                float sq = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
+                sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+                if (n < c.d) {
+                    float4 *o = reinterpret_cast<float4 *>(c.resid + (size_t)col * c.d + n);
+                    o[0] = make_float4(v[0], v[1], v[2], v[3]);
+                    o[1] = make_float4(v[4], v[5], v[6], v[7]);
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int n = n0 + u * CONS_THREADS + tid;
-                    if (n < c.d) {
-                        c.resid[(size_t)col * c.d + n] = v[u];
-                        xfrag_store(A.XA, n, col, v[u] * gn[u]);
-                    }
-                    float q = v[u] * v[u];
-                    q += __shfl_xor_sync(0xffffffffu, q, 1);
-                    q += __shfl_xor_sync(0xffffffffu, q, 2);
-                    q += __shfl_xor_sync(0xffffffffu, q, 4);
-                    q += __shfl_xor_sync(0xffffffffu, q, 8);
-                    if ((tid & 15) == 0 && n < c.d) A.ssq_a[(size_t)(n >> 4) * MAX_COLS + col] = q;
+                    for (int i = 0; i < 8; i += 2) xfrag_store2(A.XA, n + i, col, v[i] * bf16_of_word(g[i >> 1], i), v[i + 1] * bf16_of_word(g[i >> 1], i + 1));
+                    if ((tid & 1) == 0) A.ssq_a[(size_t)(n >> 4) * MAX_COLS + col] = sq;
                 }
-            }
-            for (int i = tid; i < half; i += CONS_THREADS) {
-                // angle = pos * freq in double, reduced to [-pi, pi] in double, then single-precision sin / cos
-                // (double-precision transcendentals with large arguments are slow on this GPU)
-                const double a = (double)pos * A.rope_freq[i];
-                const double r = a - 6.283185307179586476925 * rint(a * 0.15915494309189533577);
-                float sn, cs;
-                sincosf((float)r, &sn, &cs);
-                c.rope_cs[((size_t)col * half + i) * 2 + 0] = cs;
-                c.rope_cs[((size_t)col * half + i) * 2 + 1] = sn;
             }
         }
     }
-    __threadfence();
-    fence_proxy_async();
+    // the release orders what all threads wrote (through the barrier); readers of bulk copies pass a proxy fence of their own
     bar_consumers();
-    if (tid == 0) {
-        __threadfence();
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&pub->seq), "r"(pub_no) : "memory");
-    }
+    if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&pub->seq), "r"(pub_no) : "memory");
 }
 
 // Every role of every CTA passes here; returns the action and (for a new step) the descriptor.
