@@ -611,6 +611,36 @@ __device__ __forceinline__ void stage_full(float (&acc)[TILES][4][4], uint32_t w
         }
     }
 }
+// The gate and up stages of a chunk together: a k-step's activations are read once for both.  Three column tiles: 20 instead of 32
+// shared-memory cycles a k-step and warp.
+template <int T>
+__device__ __forceinline__ void stage_full2(float (&acc0)[TILES][4][4], float (&acc1)[TILES][4][4], uint32_t ws0, uint32_t ws1, const uint32_t (&xs)[TILES], int a_hi,
+                                            int a_sw) {
+    constexpr int PF = 2;
+    uint32_t a0[PF][4], a1[PF][4];
+    uint4 b[PF][T];
+    auto load = [&](int cur, int ks) {
+        const uint32_t at = (ks >> 2) * 2048 + (((((ks & 3) << 1) | a_hi) ^ a_sw) << 4);
+        ldmatrix_x4_at(a0[cur], ws0 + at);
+        ldmatrix_x4_at(a1[cur], ws1 + at);
+#pragma unroll
+        for (int t = 0; t < T; ++t) b[cur][t] = lds128(xs[t] + ks * 128);
+    };
+#pragma unroll
+    for (int j = 0; j < PF; ++j) load(j, j);
+#pragma unroll
+    for (int j = 0; j < KSTEPS; ++j) {
+        const int cur = j % PF;
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            mma16816(acc0[t][j & 1], a0[cur], b[cur][t].x, b[cur][t].y);
+            mma16816(acc1[t][j & 1], a1[cur], b[cur][t].x, b[cur][t].y);
+            mma16816(acc0[t][(j & 1) + 2], a0[cur], b[cur][t].z, b[cur][t].w);
+            mma16816(acc1[t][(j & 1) + 2], a1[cur], b[cur][t].z, b[cur][t].w);
+        }
+        if (j + PF < KSTEPS) load(cur, j + PF);
+    }
+}
 // The same for up to four columns: their high parts are token columns 0..3 of one multiply-add, their low parts 4..7.
 // Half the multiply-adds and half the shared-memory reads; every sum has the order it has above.
 __device__ __forceinline__ void stage_packed(float (&acc)[4][4], uint32_t ws, uint32_t xs, int a_hi, int a_sw) {
@@ -873,6 +903,20 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
 #pragma unroll
             for (int t = 0; t < TILES; ++t) xc[t] = xt[t] + (t == 0 ? (kc - x0) * cols.ncp * 4096 : 0);
             uint32_t i = stage_of(kc);
+            if (TILES > 1 && pair == 2 && !packed) {
+                w_wait(S, i, known);
+                w_wait(S, i + 1, known);
+                const uint32_t ws0 = s32(sm->w[i % NW]) + a_off, ws1 = s32(sm->w[(i + 1) % NW]) + a_off;
+                if (nt == 1) stage_full2<1>(acc0, acc1, ws0, ws1, xc, a_hi, a_sw);
+                else if (nt == 2) stage_full2<TILES < 2 ? 1 : 2>(acc0, acc1, ws0, ws1, xc, a_hi, a_sw);
+                else stage_full2<TILES>(acc0, acc1, ws0, ws1, xc, a_hi, a_sw);
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&sm->w_empty[i % NW]);
+                    mbar_arrive(&sm->w_empty[(i + 1) % NW]);
+                }
+                continue;
+            }
 #pragma unroll 1
             for (int p = 0; p < pair; ++p, ++i) {
                 if (PARK && n_used < n_parked) {
@@ -893,14 +937,12 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                     if (p == 0) stage_packed(acc0[0], ws, xc[0], a_hi, a_sw);
                     else stage_packed(acc1[0], ws, xc[0], a_hi, a_sw);
                 } else if (nt == 1) {
-                    if (p == 0) stage_full<1>(acc0, ws, xc, a_hi, a_sw);
+                    if (p == 0 || TILES > 1) stage_full<1>(acc0, ws, xc, a_hi, a_sw);
                     else stage_full<1>(acc1, ws, xc, a_hi, a_sw);
                 } else if (TILES > 1 && nt == 2) {
-                    if (p == 0) stage_full<TILES < 2 ? TILES : 2>(acc0, ws, xc, a_hi, a_sw);
-                    else stage_full<TILES < 2 ? TILES : 2>(acc1, ws, xc, a_hi, a_sw);
+                    stage_full<TILES < 2 ? TILES : 2>(acc0, ws, xc, a_hi, a_sw);
                 } else if (TILES > 1) {
-                    if (p == 0) stage_full<TILES>(acc0, ws, xc, a_hi, a_sw);
-                    else stage_full<TILES>(acc1, ws, xc, a_hi, a_sw);
+                    stage_full<TILES>(acc0, ws, xc, a_hi, a_sw);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
