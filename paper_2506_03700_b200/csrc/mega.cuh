@@ -526,13 +526,6 @@ struct Ctl {
 constexpr int CTL_OFFSET = 8192 + ((int)sizeof(HeadResult) + 4) * MAX_COLS;
 static_assert(CTL_OFFSET % 16 == 0 && CTL_OFFSET + (int)sizeof(Ctl) <= DRAW_OFFSET, "the control point's copies overlap the draw's buffers");
 
-// eight neighbouring bf16 elements; `aligned`: their address is a multiple of 16
-__device__ __forceinline__ uint4 load_bf16x8(const __nv_bfloat16 *p, bool aligned) {
-    if (aligned) return __ldg(reinterpret_cast<const uint4 *>(p));
-    const unsigned short *h = reinterpret_cast<const unsigned short *>(p);
-    return make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16, h[6] | (uint32_t)h[7] << 16);
-}
-
 __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int kind, int e, unsigned pub_no, const StepDesc &dprev,
                                           int &steps_started) {
     const Ctx &c = A.c;
@@ -847,15 +840,16 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
             const int col = __ffs(m) - 1, k = nseq == 1 ? 0 : col % nseq;
             const int token = st->pf_end > 0 ? c.tokens[(size_t)(seq0 + k) * c.max_seq + nd.pos[col]] : ctl.newest[k];
             const __nv_bfloat16 *erow = M.tok_embed + (size_t)min(max(token, 0), c.vocab - 1) * c.d;
-            const bool al = ((reinterpret_cast<uintptr_t>(erow) | reinterpret_cast<uintptr_t>(g0)) & 15) == 0;
+            // (tensors start on 16-byte boundaries, ada_model_set_tensor, and a row is a multiple of 64 elements)
+            auto load = [&](const __nv_bfloat16 *p, int n) { return __ldg(reinterpret_cast<const uint4 *>(p + n)); };
             const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-            uint4 ev = at < c.d ? load_bf16x8(erow + at, al) : zero, gv = at < c.d ? load_bf16x8(g0 + at, al) : zero;
+            uint4 ev = at < c.d ? load(erow, at) : zero, gv = at < c.d ? load(g0, at) : zero;
 #pragma unroll 1
             for (int n0 = 0; n0 < c.d; n0 += step) {
                 const int n = n0 + at, nn = n + step;
                 const uint32_t e[4] = {ev.x, ev.y, ev.z, ev.w}, g[4] = {gv.x, gv.y, gv.z, gv.w};
-                ev = nn < c.d ? load_bf16x8(erow + nn, al) : zero;
-                gv = nn < c.d ? load_bf16x8(g0 + nn, al) : zero;
+                ev = nn < c.d ? load(erow, nn) : zero;
+                gv = nn < c.d ? load(g0, nn) : zero;
                 float v[8], q[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) { v[i] = bf16_of_word(e[i >> 1], i); q[i] = __fmul_rn(v[i], v[i]); }
@@ -1809,10 +1803,11 @@ __global__ void k_prefill_arm(Ctx c, int seq, int n_prompt) {
 // Warps 0-7 consume, warp 8 produces weights and K / V blocks, warp 9 activations and queries; warps 10 and 11 only complete the producers'
 // warp group, which hands registers to the consumers.  (At 168 registers a thread -- three warps on a quarter of the SM --
 // the consumers kept loop variables in local memory, whose L1 lines do not survive the acquires of the grid barrier: a round trip to
-// L2 for each on the critical path of a phase.  At 200 / 104 one column tile spills nothing; 216 / 72 spilled 64 bytes in the
-// producers and cost 0.5 to 2 % of a request.  Three tiles: 120 bytes at 216 / 72, 40 at 200 / 104, no difference measured.)
+// L2 for each on the critical path of a phase.  One column tile: at 200 / 104 nothing is spilled; 216 / 72 spilled 64 bytes in the
+// producers and cost 0.5 to 2 % of a request.  Three tiles: the consumers' sums need more; 216 / 72 (which spills 200 bytes in the
+// producers) 58 us a gate / up product of the 13B shape, 200 / 104 67; requests 183.3 ms, 208 / 88 185, 200 / 104 187.5.)
 constexpr int MEGA_THREADS = CONS_THREADS + 128;
-constexpr int REGS_CONSUME = 200, REGS_PRODUCE = 104;
+constexpr int REGS_CONSUME = TILES == 1 ? 200 : 216, REGS_PRODUCE = TILES == 1 ? 104 : 72;
 constexpr int MEGA_REGS = CONS_THREADS * REGS_CONSUME + 128 * REGS_PRODUCE;   // the block must have been launched with as many
 
 template <int HD>
