@@ -6,8 +6,8 @@
 // with a grid barrier between phases.  The weight producer is not held by those barriers (but for cache rows
 // of the pass itself): it keeps the TMA ring full with the tiles of the coming phases, so HBM keeps streaming while the
 // grid meets, and the consumers move what has landed on to tensor memory (park_stage in stream.cuh).  Measured, one layer in a plain
-// step (1B / 8B shape): QKV 5.9 / 10.8 us, attention 7.2 / 9.9 (60 / 1040 positions),
-// O 5.2 / 7.7, gate-up 11.4 / 35.8, down 7.7 / 19.2, of which the bytes alone take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
+// step (1B / 8B shape): QKV 5.7 / 10.9 us, attention 6.6 / 10.3 (60 / 1040 positions),
+// O 5.1 / 7.6, gate-up 10.6 / 36.8, down 7.8 / 18.6, of which the bytes alone take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
 // residuals, counters) lives in device memory; the control points run in CTA 0, which publishes
 // each decision (continue the climb, start the next token, stop) to the other CTAs through a
 // sequence-numbered record.  The host launches, waits, and launches again until the call is done.
@@ -1150,7 +1150,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
         const unsigned sl = seq_slots(A, mask, k);
         if (sl) dual = dual && ((__ffs(sl) - 1) * group >= 16 || (32 - __clz(sl)) * group <= 16);
     }
-    // Every row of the step has a single chunk: its item finishes it, there is nothing to merge (1B shape at 60 positions 7.4 -> 6.5 us a layer).
+    // Every row of the step has a single chunk: its item finishes it, there is nothing to merge (1B shape at 60 positions 7.4 -> 6.6 us a layer).
     const bool one_chunk = d.pmax < ATT_CHUNK;
     int turn = 0;   // group whose item it is
 #pragma unroll 1

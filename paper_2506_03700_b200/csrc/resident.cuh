@@ -21,8 +21,8 @@
 //
 // Invariance rule as in kernels.cuh: a row's numbers depend on that row's inputs and the launch geometry only.
 //
-// Measured, four layers of width 256 (16 + 128 tokens, up to five early ones): 10.3 ms, 20.2 with a launch per operation.  Plain
-// decoding takes 105 us a token: some 3 to 7 us a phase, an exchange through L2 with the latency of its loads before and after.
+// Measured, four layers of width 256 (16 + 128 tokens, up to five early ones): 10.1 ms, 20.2 with a launch per operation.  Plain
+// decoding takes 102 us a token: some 3 to 7 us a phase, an exchange through L2 with the latency of its loads before and after.
 #pragma once
 
 #include "kernels.cuh"
