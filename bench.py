@@ -33,7 +33,7 @@ UNIT = "tokens/s"
 # from the ncu captures summarised in profiles/ (1B-shaped launches; traffic grows in proportion to the
 # bytes streamed, so a ratio carries over to the larger shapes), keyed by decoding mode.  None = not
 # captured for the kernel as it stands.
-DRAM_TRAFFIC_RATIO = {"plain": 1.0027, "adaptive": 1.0020}   # profiles/k_decode_persistent_1b_dram_traffic_ncu.md
+DRAM_TRAFFIC_RATIO = {"plain": 1.0027, "adaptive": 1.0021}   # profiles/k_decode_persistent_1b_dram_traffic_ncu.md
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 
