@@ -867,7 +867,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
             }
         }
     }
-    // the release orders what all threads wrote (through the barrier); readers of bulk copies pass a proxy fence of their own
+    // the release orders what all threads wrote (through the barrier); the producers pass a proxy fence behind their acquire of it
     bar_consumers();
     if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&pub->seq), "r"(pub_no) : "memory");
 }
@@ -947,6 +947,9 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
     } else {
         grid_wait(S, &pub->seq, pub_no);
         action = fetch();
+        // What the grid wrote before this control point -- cache rows of the steps before, the next step's input -- is ordered before the
+        // bulk copies of the steps after it: those of cache blocks without rows of their own pass wait for no barrier.
+        fence_proxy_async();
         __syncwarp();
     }
     return action;
@@ -1040,7 +1043,8 @@ struct AttnWalk {
 // and the O product's weights: per item K of its sub-blocks, then V.  Nine blocks are in flight per CTA instead of the three that
 // the activation ring held, and O's weights follow without a gap.
 // The rows of the tokens of this pass are written by the QKV epilogues of other CTAs: an item that holds one is fetched once the
-// grid has passed the barrier that ends the QKV phase (`bar_target`), every other as soon as the ring has room.
+// grid has passed the barrier that ends the QKV phase (`bar_target`), every other as soon as the ring has room: its rows were written in
+// earlier steps, in front of the control point behind which this producer fenced its copies (control_point).
 __device__ __forceinline__ void attn_produce_kv(const MegaArgs &A, const Shared &S, const StepDesc &d, int layer, unsigned mask, unsigned bar_target,
                                                 Rings &r, uint64_t pol) {
     const Ctx &c = A.c;

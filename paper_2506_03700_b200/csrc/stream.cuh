@@ -372,8 +372,8 @@ __device__ __forceinline__ void vec_wait(const Shared &S, unsigned seq) {
 __device__ __forceinline__ void grid_arrive(unsigned *ctr) {
     // the release of the reduction orders this thread's earlier writes, and through the block-level
     // barrier before it those of the whole CTA; a separate fence before it only adds its latency.  What bulk copies read of
-    // them is ordered by the proxy fence that every reader passes between its acquire and its first copy (one here as well
-    // cost 0.2 us a phase).
+    // them is ordered by the proxy fence that a producer passes between its acquire -- of this counter, or of the record of a later
+    // control point -- and its first copy (one here as well cost 0.2 us a phase).
     red_release_add(ctr, 1u);
 }
 __device__ __forceinline__ void grid_wait(const Shared &S, const unsigned *ctr, unsigned target) {

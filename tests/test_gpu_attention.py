@@ -112,3 +112,32 @@ def test_calls_pay_for_the_positions_they_reach_not_for_the_sessions_length(dtyp
     assert all(np.array_equal(a, b) for a, b in zip(got[0][0], got[1][0]))
     assert got[0][1] == got[1][1]
     assert got[0][1][-1] > got[0][1][batch + 1] > 0   # (the last call reaches a second chunk, the first of several tokens does not)
+
+
+@pytest.mark.parametrize("head_dim,nq,nkv,batch", [(64, 8, 2, 1), (128, 4, 4, 1), (64, 8, 8, 3)])
+def test_rows_written_in_a_launch_reach_the_chunks_of_its_later_steps(head_dim, nq, nkv, batch):
+    """A chunk that the context has just left is read by bulk copies that wait for no barrier of their own step.  Its rows were written
+    in earlier steps, by other CTAs: in the same launch here, in launches of their own (one step each) for what is compared, so that
+    the end of a kernel orders them.  The same bits: prompts through the decode path, plain and adaptive decoding, across several chunks."""
+    cfg = synth.small_config(dtype="bf16", n_layers=3, d_model=512, n_q_heads=nq, n_kv_heads=nkv, head_dim=head_dim, d_ff=704,
+                             vocab=1024, sigma=0.08, resid_scale=0.8, exit_layers=(1, 2))
+    gm = binding.Model(cfg, synth.make_weights(cfg, device="cuda"))
+    for l in cfg.exit_layers:
+        gm.set_exit_head(l, None, cfg.logit_scale)
+    n = 20
+    for n_prompt in (120, 247, 377):
+        prompts = [synth.make_prompt(cfg, n=n_prompt - 3 * s, seq=s).numpy() for s in range(batch)]
+        for early in (0, 1):
+            got = []
+            for steps in (256, 1):
+                S = binding.Session(gm, batch, 512, 64, early)
+                S.set_prefill(False)
+                S.set_launch_steps(steps)
+                S.capture_logits(n + 4)
+                for s, p in enumerate(prompts):
+                    S.prefill(p, seq=s)
+                st = binding.Stats()
+                out = S.adaptive_decode(n, 0.2, cfg.exit_layers, early, st) if early else S.plain_decode(n, st)
+                got.append((out, S.captured_logits()[:n].cpu().numpy()))
+                assert (st.kernel_launches >= n // 2) == (steps == 1)
+            assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1]), (n_prompt, early)
