@@ -950,6 +950,8 @@ __device__ __forceinline__ int control_point(const MegaArgs &A, const Shared &S,
         // What the grid wrote before this control point -- cache rows of the steps before, the next step's input -- is ordered before the
         // bulk copies of the steps after it: those of cache blocks without rows of their own pass wait for no barrier.
         fence_proxy_async();
+        // the lanes stop together: one may have seen an error that another has not
+        if (__any_sync(0xffffffffu, action == ACT_STOP)) action = ACT_STOP;
         __syncwarp();
     }
     return action;
@@ -1843,6 +1845,7 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
     if (TILES == 1) tc_fence_before();
     settle_on_abort(S);   // (meets the whole block)
     if (TILES == 1 && warp == CONS_WARPS + 2) {
+        __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm->tmem), "r"(PARK_COLS) : "memory");
     }

@@ -319,19 +319,22 @@ __device__ __noinline__ void raise_error(const Shared &S, int code) {
 // Wait for an mbarrier phase.  Once an error is raised (here or anywhere in the grid) every wait
 // falls through at once: the roles then run to the end of their loops on whatever data is there,
 // so that no warp is left behind at a block-level barrier, and the kernel ends.
+// Called by whole warps.  The lanes poll for themselves and may leave at different turns, on a satisfied wait or on an error; what
+// follows (fragment and tensor-memory loads, multiply-adds, votes) wants them together, so that is where the wait ends.
 __device__ __forceinline__ void mbar_wait(const Shared &S, unsigned long long *bar, uint32_t parity) {
-    if (mbar_try(bar, parity)) return;
-    unsigned long long t0 = 0;
-    for (uint32_t it = 0;; ++it) {
-        if (mbar_try(bar, parity)) return;
-        if ((it & 127u) == 0 || S.wait_ns < SHORT_LIMIT_NS) {
-            if (aborted(S)) return;
-            if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; return; }
-            unsigned long long t = gtime();
-            if (t0 == 0) t0 = t;
-            else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_MBAR); return; }
+    if (!mbar_try(bar, parity)) {
+        unsigned long long t0 = 0;
+        for (uint32_t it = 0; !mbar_try(bar, parity); ++it) {
+            if ((it & 127u) == 0 || S.wait_ns < SHORT_LIMIT_NS) {
+                if (aborted(S)) break;
+                if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; break; }
+                unsigned long long t = gtime();
+                if (t0 == 0) t0 = t;
+                else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_MBAR); break; }
+            }
         }
     }
+    __syncwarp();
 }
 
 // Epilogue operands are fetched while the weights stream, by 4-byte asynchronous copies into words of
@@ -483,7 +486,8 @@ __device__ __forceinline__ uint32_t w_issued_get(Smem *sm) {
     asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(n) : "r"(s32(&sm->w_issued)) : "memory");
     return n;
 }
-// Wait until stage i has landed; `known`: stages this warp knows to be issued.
+// Wait until stage i has landed; `known`: stages this warp knows to be issued.  (A stage that was not issued when the wait for that ended
+// on an error lets the second wait fall through as well.)
 __device__ __forceinline__ void w_wait(const Shared &S, uint32_t i, uint32_t &known) {
     if ((int)(known - i) <= 0) {
         unsigned long long t0 = 0;
@@ -491,11 +495,11 @@ __device__ __forceinline__ void w_wait(const Shared &S, uint32_t i, uint32_t &kn
             known = w_issued_get(S.sm);
             if ((int)(known - i) > 0) break;
             if ((it & 127u) == 127u || S.wait_ns < SHORT_LIMIT_NS) {
-                if (aborted(S)) return;
-                if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; return; }
+                if (aborted(S)) break;
+                if (*(volatile int *)S.err != 0) { *(volatile int *)&S.sm->abort = 1; break; }
                 const unsigned long long t = gtime();
                 if (t0 == 0) t0 = t;
-                else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_MBAR); return; }
+                else if (t - t0 > S.wait_ns) { raise_error(S, ERR_TIMEOUT_MBAR); break; }
             }
         }
     }

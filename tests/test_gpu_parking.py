@@ -60,3 +60,35 @@ def test_columns_of_several_sequences(batch, early):
     together = decode(prompts)
     for s, p in enumerate(prompts):
         assert np.array_equal(together[s], decode([p])[0]), s
+
+
+@pytest.mark.parametrize("batch,early", [(1, 5), (3, 1), (2, 5)])   # one sequence; six columns of one tile; 24 columns
+def test_waits_that_run_out_anywhere(batch, early):
+    """Limits from far below what a wait lasts to about as long as a phase: which wait gives up first, in which lane, with stages
+    parked or not and at a control point or not, differs from run to run.  Every call ends with a time-out or with the right tokens,
+    and the session decodes correctly afterwards."""
+    cfg = config(576, 4224, 8, 2, 64, 2400)
+    pair = Pair(cfg)
+    n = 9
+    prompts = [synth.make_prompt(cfg, n=118 + 5 * s, seq=s).numpy() for s in range(batch)]
+    S = binding.Session(pair.gm, batch, 256, 64, early)
+
+    def decode(limit):
+        S.set_wait_limit(2_000_000_000)
+        S.reset()
+        for s, p in enumerate(prompts):
+            S.prefill(p, seq=s)
+        S.set_wait_limit(limit)
+        return S.adaptive_decode(n, 0.2, cfg.exit_layers, early)
+
+    ref = decode(2_000_000_000)
+    ran_out = 0
+    for limit in (50, 400, 1500, 3000, 6000, 12000, 40000):
+        try:
+            assert np.array_equal(decode(limit), ref), limit
+        except binding.AdaError as e:
+            assert e.code == -5, limit
+            ran_out += 1
+            torch.cuda.synchronize()      # the context is intact
+        assert np.array_equal(decode(2_000_000_000), ref), limit
+    assert ran_out > 0
