@@ -585,6 +585,8 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     }
     // (b) bookkeeping, one warp: every lane follows the same decisions, lane 0 writes them down, loops over the layers are shared out.
     // Every scalar it may need is read up front (the loads overlap); counters are bumped by reductions, which do not wait for memory.
+    // The lanes have to agree on all of it, or they would part ways at the sums over the warp: the error word, which any CTA may set at
+    // any time, is settled by a vote, and lane 0 writes nothing before every lane has read.
     if (tid < 32) {
         const int lane = tid;
         const bool w0 = lane == 0;
@@ -599,7 +601,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
             }
             return (long long)__reduce_add_sync(0xffffffffu, rl);
         };
-        const int err0 = *(volatile int *)A.err;
+        const bool stop0 = __any_sync(0xffffffffu, *(volatile int *)A.err != 0);
         const int pf_end0 = st->pf_end, pf_pos0 = st->pf_pos, max_early0 = st->max_early;
         const int tape_n0 = st->tape_n, hl_n0 = st->head_log_n;
         const int tape_i0 = st->tape_i;
@@ -610,7 +612,8 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
         int action = ACT_NEWSTEP, verified = 0;
         int keep_rows = 0, keep_row0 = 0;
         int pf_end = pf_end0, pf_pos = pf_pos0;
-        if (err0 != 0) action = ACT_STOP;
+        __syncwarp();
+        if (stop0) action = ACT_STOP;
         // ---- Eq. 1 after an intermediate head: every sequence whose newest token consulted it decides for itself
         if (action != ACT_STOP && kind == CTRL_HEAD) {
             unsigned still = 0;   // sequences that go on climbing in this step
