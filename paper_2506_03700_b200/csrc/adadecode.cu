@@ -141,6 +141,7 @@ struct ada_session {
     std::vector<int> h_len, h_prompt, h_reported;
     std::vector<char> prefilled, finished;   // finished: the sequence ended on an end-of-sequence token (eos_tok)
     std::vector<int> eos_tok;
+    std::vector<char> dirty;   // a call that a device-side error ended may have left anything in the sequence's cache pages
     int32_t *pinned = nullptr; // small read-back area
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     int path = 0;
@@ -755,6 +756,7 @@ int prefill_dense(ada_session *S, int seq, int n_prompt) {
     CK(cudaStreamSynchronize(S->stream));
     if (S->pinned[0] != 0) {
         g_cuda_err = "dense prompt pass: a bounded device-side wait expired";
+        S->dirty.assign(S->batch, 1);
         return ADA_ETIMEOUT;
     }
     return ADA_OK;
@@ -1007,6 +1009,7 @@ int run_resident(ada_session *S, int pf_seq, int pf_n, const int32_t *exit_layer
     S->syncs++;
     if (S->pinned[0] != 0) {
         g_cuda_err = "fp32 decode kernel: device-side error " + std::to_string(S->pinned[0]);
+        S->dirty.assign(S->batch, 1);
         return ADA_ETIMEOUT;
     }
     return ADA_OK;
@@ -1089,6 +1092,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
             S->syncs++;
             if (S->pinned[2] != 0) {
                 g_cuda_err = "persistent decode kernel: device-side error " + std::to_string(S->pinned[2]);
+                S->dirty.assign(S->batch, 1);
                 return S->pinned[2] == ERR_BAD_STATE ? ADA_ESTATE : ADA_ETIMEOUT;
             }
             if (S->pinned[1] >= 1) break;   // the sequences of this launch have reached their targets
@@ -1558,6 +1562,7 @@ int ada_session_create(const ada_model *m, int32_t batch, int32_t max_seq_len, i
     S->prefilled.assign(batch, 0);
     S->finished.assign(batch, 0);
     S->eos_tok.assign(batch, -1);
+    S->dirty.assign(batch, 0);
     *out = S;
     return ADA_OK;
 }
@@ -1575,6 +1580,11 @@ int ada_session_reset(ada_session *S, int32_t seq) {
     if (!S || seq >= S->batch) return ADA_EINVAL;
     for (int s = 0; s < S->batch; ++s) {
         if (seq >= 0 && s != seq) continue;
+        if (S->dirty[s]) {   // masked cache rows must hold finite numbers, whoever gets the pages next
+            const size_t bytes = ada_kv_page_bytes(S->m, S->page_tokens);
+            for (int p : S->seq_pages[s]) CK(cudaMemsetAsync((char *)S->c.kv_pool + p * bytes, 0, bytes, S->stream));
+            S->dirty[s] = 0;
+        }
         for (int p : S->seq_pages[s]) S->free_pages.push_back(p);
         S->seq_pages[s].clear();
         S->prefilled[s] = 0;

@@ -337,6 +337,29 @@ def test_a_wait_that_runs_out_ends_the_call_with_a_timeout_and_the_session_recov
     assert np.array_equal(S.adaptive_decode(n, 0.3, cfg.exit_layers, 5, st)[0], ref) and st.early_exits > 0
 
 
+@pytest.mark.parametrize("dense", [True, False])
+def test_a_call_that_ran_out_leaves_nothing_in_the_cache(dense):
+    """Numbers that are not finite in cache rows behind the context would spoil the rows in front of them (a masked weight is a zero,
+    which a product with NaN does not hide).  A call that gave up may have written any: here every row of the session's pages."""
+    cfg = hd128()
+    pair = Pair(cfg)
+    prompt = synth.make_prompt(cfg, n=125).numpy()
+    n = 12
+    S = session(pair, max_seq=192, kv_pages=3)
+    S.set_prefill(dense)
+    S.prefill(prompt)
+    ref = S.plain_decode(n)[0]
+    S.prefill(prompt)
+    S.set_wait_limit(20)
+    with pytest.raises(binding.AdaError) as e:
+        S.plain_decode(n)
+    assert e.value.code == -5
+    S.set_wait_limit(2_000_000_000)
+    S.kv_pool.fill_(0xff)                 # NaN
+    S.prefill(prompt)
+    assert np.array_equal(S.plain_decode(n)[0], ref)
+
+
 @pytest.mark.parametrize("mk,n_prompt", [(gqa, 200), (hd128, 131), (mha, 77)])
 def test_dense_prompt_pass_matches_the_pass_through_the_decode_path_and_the_oracle(mk, n_prompt):
     """KV cache <- LM(x): prompts of 9 tokens or more run in blocks of up to 2048 positions through the tcgen05
