@@ -239,6 +239,12 @@ int ada_debug_set_launch_steps(ada_session *s, int32_t steps);
  * next decode call time out: that is how the give-up path is tested. */
 int ada_debug_set_wait_limit(ada_session *s, uint64_t ns);
 
+/* While the grid meets, the warps of the persistent kernel (eight token columns) move weight stages that have landed into tensor memory:
+ * at most `most` each, 0 to 2 (the default).  The bits of a result do not depend on it.  ada_debug_parked: stages that the session's
+ * last decode call moved, all CTAs together (which ones land in time differs from run to run). */
+int ada_debug_set_parking(ada_session *s, int32_t most);
+int ada_debug_parked(ada_session *s, int64_t *stages_out);
+
 /* Bytes of attention chunk partials that the session's last prompt or decode call cleared before its launches (host counter). */
 int ada_debug_cleared_bytes(ada_session *s, int64_t *bytes_out);
 /* Event trace of the persistent kernel: while the kernel runs the steps [step0, step1) of a launch
@@ -281,6 +287,12 @@ size_t ada_debug_gemm_work_bytes(int32_t K);
 int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const float *X_dev, int32_t cols,
                    void *work_dev, size_t work_bytes, float *Y_dev, int32_t ldy, int32_t repeat, void *cuda_stream,
                    float *ms_out);
+/* One such product whose activations are fetched hold_ns nanoseconds late (at most 10 ms), so that the consumer warps park as many
+ * weight stages as they may, `most` each (0 to 2); a single wait gives up after wait_ns (a limit below hold_ns: ADA_ETIMEOUT, stages
+ * parked).  *parked_out (nullable, host): stages parked, all CTAs together. */
+int ada_debug_gemm_parked(const void *W_dev, int32_t N, int32_t K, int32_t mode, const float *X_dev, int32_t cols,
+                          void *work_dev, size_t work_bytes, float *Y_dev, int32_t ldy, int32_t most, uint64_t hold_ns,
+                          uint64_t wait_ns, void *cuda_stream, int32_t *parked_out);
 
 /* Run the dense GEMM of the prompt pass by itself (Algorithm 1, first line: all prompt tokens go through the
  * model at once): Y[m][n] = (or +=, if `accumulate`) sum_k X[m][k] W[n][k] for up to 128 rows m, on tcgen05

@@ -34,7 +34,7 @@ EXPORTS = [
     "ada_model_arena_bytes", "ada_model_set_arena", "ada_debug_set_wait_limit", "ada_debug_set_prefill",
     "ada_debug_dense_gemm", "ada_debug_dense_gemm_work_bytes", "ada_sampling_decode",
     "ada_debug_dense_plan", "ada_debug_dense_product", "ada_debug_dense_product_work_bytes",
-    "ada_debug_resident_plan", "ada_debug_cleared_bytes",
+    "ada_debug_resident_plan", "ada_debug_cleared_bytes", "ada_debug_set_parking", "ada_debug_parked", "ada_debug_gemm_parked",
 ]
 
 
@@ -96,6 +96,9 @@ def load() -> C.CDLL:
         L.ada_model_set_arena.argtypes = [vp, vp, sz]
         L.ada_debug_set_wait_limit.argtypes = [vp, C.c_uint64]
         L.ada_debug_cleared_bytes.argtypes = [vp, C.POINTER(C.c_int64)]
+        L.ada_debug_set_parking.argtypes = [vp, i32]
+        L.ada_debug_parked.argtypes = [vp, C.POINTER(C.c_int64)]
+        L.ada_debug_gemm_parked.argtypes = [vp, i32, i32, i32, vp, i32, vp, sz, vp, i32, i32, C.c_uint64, C.c_uint64, vp, C.POINTER(i32)]
         L.ada_debug_set_prefill.argtypes = [vp, i32]
         L.ada_debug_dense_gemm_work_bytes.restype = sz
         L.ada_debug_dense_gemm_work_bytes.argtypes = [i32]
@@ -189,6 +192,24 @@ def debug_gemm(W, X, mode: int = 0, repeat: int = 1):
     _ck(lib.ada_debug_gemm(W.data_ptr(), N, K, mode, X.data_ptr(), cols, work.data_ptr() + off, wb, Y.data_ptr(), n_out,
                            repeat, torch.cuda.current_stream().cuda_stream, C.byref(ms)), "ada_debug_gemm")
     return Y, ms.value
+
+
+def debug_gemm_parked(W, X, mode: int = 0, most: int = 2, hold_ns: int = 0, wait_ns: int = 2_000_000_000):
+    """ada_debug_gemm_parked: (Y fp32 [cols, N or N/2], weight stages parked in tensor memory)."""
+    import torch
+    lib = load()
+    (N, K), cols = W.shape, X.shape[0]
+    assert W.is_cuda and W.dtype == torch.bfloat16 and W.is_contiguous()
+    assert X.is_cuda and X.dtype == torch.float32 and X.is_contiguous() and X.shape[1] == K
+    n_out = N // 2 if mode == 1 else N
+    wb = lib.ada_debug_gemm_work_bytes(K)
+    work = torch.empty(wb + 256, dtype=torch.uint8, device="cuda")
+    off = (-work.data_ptr()) % 256
+    Y = torch.zeros(cols, n_out, dtype=torch.float32, device="cuda")
+    parked = C.c_int32(0)
+    _ck(lib.ada_debug_gemm_parked(W.data_ptr(), N, K, mode, X.data_ptr(), cols, work.data_ptr() + off, wb, Y.data_ptr(), n_out, most, hold_ns,
+                                  wait_ns, torch.cuda.current_stream().cuda_stream, C.byref(parked)), "ada_debug_gemm_parked")
+    return Y, parked.value
 
 
 def debug_dense_gemm(W, X, Y=None):
@@ -427,6 +448,14 @@ class Session:
 
     def set_wait_limit(self, ns: int):
         _ck(load().ada_debug_set_wait_limit(self.h, ns), "ada_debug_set_wait_limit")
+
+    def set_parking(self, most: int):
+        _ck(load().ada_debug_set_parking(self.h, most), "ada_debug_set_parking")
+
+    def parked(self) -> int:
+        n = C.c_int64(0)
+        _ck(load().ada_debug_parked(self.h, C.byref(n)), "ada_debug_parked")
+        return n.value
 
     def cleared_bytes(self) -> int:
         n = C.c_int64(0)

@@ -173,6 +173,8 @@ struct ada_session {
     bool prefill_dense = true;                 // ada_debug_set_prefill
     int64_t launches = 0, syncs = 0, layer_passes = 0;
     int64_t cleared = 0;                       // bytes of attention partials that the last prompt or decode call cleared
+    int64_t parked = 0;                        // weight stages that the last decode call parked in tensor memory
+    int park = st::PARK_MAX;                   // how many of them a warp may park at a time
     // per-class profiling
     bool prof = false;
     std::vector<cudaEvent_t> prof_ev;
@@ -1072,6 +1074,7 @@ int run_persistent(ada_session *S, const int32_t *exit_layers, int n_exit, bool 
         a.nseq = std::min(per_launch, seq_end - sq);
         a.step_budget = S->steps_per_launch;
         a.wait_ns = S->wait_ns;
+        a.park = S->park;
         a.store_logits = (S->capture_dev && sq == 0) ? 1 : 0;
         a.sampling = S->sampling ? 1 : 0;
         a.inv_temp = S->sampling ? S->inv_temp : 1.0f;
@@ -1273,6 +1276,7 @@ int decode(ada_session *S, int n_tokens, float gamma, const int32_t *exit_layers
             S->prof_bytes[i] += wbytes[i] * (double)ds.phase_count[i];
         }
     }
+    S->parked = ds.parked;
     add_stats(S, ds, stats, ms, l0, s0, p0);
     return ADA_OK;
 }
@@ -1706,6 +1710,18 @@ int ada_debug_set_wait_limit(ada_session *S, uint64_t ns) {
     return ADA_OK;
 }
 
+int ada_debug_set_parking(ada_session *S, int32_t most) {
+    if (!S || most < 0 || most > st::PARK_MAX) return ADA_EINVAL;
+    S->park = most;
+    return ADA_OK;
+}
+
+int ada_debug_parked(ada_session *S, int64_t *stages_out) {
+    if (!S || !stages_out) return ADA_EINVAL;
+    *stages_out = S->parked;
+    return ADA_OK;
+}
+
 int ada_debug_cleared_bytes(ada_session *S, int64_t *bytes_out) {
     if (!S || !bytes_out) return ADA_EINVAL;
     *bytes_out = S->cleared;
@@ -1869,8 +1885,10 @@ size_t ada_debug_gemm_work_bytes(int32_t K) {
     return st::xfrag_bytes(K) + 512 + kPartBytesPerCta * kPartMaxGrid + 256;
 }
 
-int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const float *X_dev, int32_t cols, void *work_dev,
-                   size_t work_bytes, float *Y_dev, int32_t ldy, int32_t repeat, void *cuda_stream, float *ms_out) {
+namespace {
+// The streaming GEMM by itself (ada_debug_gemm, ada_debug_gemm_parked).
+int run_gemm_probe(const void *W_dev, int32_t N, int32_t K, int32_t mode, const float *X_dev, int32_t cols, void *work_dev, size_t work_bytes, float *Y_dev,
+                   int32_t ldy, int32_t repeat, const ProbeParking &parking, unsigned long long wait_ns, void *cuda_stream, float *ms_out, int32_t *parked_out) {
     if (!W_dev || !X_dev || !work_dev || !Y_dev || N < 1 || K < 64 || K % 64 || cols < 1 || cols > st::MAX_COLS) return ADA_EINVAL;
     if (mode < 0 || mode > 1 || repeat < 1) return ADA_EINVAL;
     if (mode == 1 && (N % 2 || (N / 2) % 16)) return ADA_EINVAL;
@@ -1880,13 +1898,13 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    CK(cudaFuncSetAttribute(k_gemm_probe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES));
-    int *err = (int *)((char *)work_dev + st::xfrag_bytes(K));
+    CK(cudaFuncSetAttribute(k_gemm_probe<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES));
+    int *err = (int *)((char *)work_dev + st::xfrag_bytes(K));   // the error word and the count of parked stages
     CUtensorMap *dmap = (CUtensorMap *)((char *)work_dev + st::xfrag_bytes(K) + 256);
     CUtensorMap hmap;
     int rc = make_weight_map(&hmap, W_dev, N, K);
     if (rc) return rc;
-    CK(cudaMemsetAsync(err, 0, sizeof(int), stream));
+    CK(cudaMemsetAsync(err, 0, 2 * sizeof(int), stream));
     CK(cudaMemcpyAsync(dmap, &hmap, sizeof(hmap), cudaMemcpyHostToDevice, stream));
     CK(cudaStreamSynchronize(stream));   // hmap lives on this stack frame
     k_xfrag_pack<<<(K + st::KC - 1) / st::KC * 2, st::KC / 2, 0, stream>>>(X_dev, K, cols, (__nv_bfloat16 *)work_dev);
@@ -1898,11 +1916,11 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     unsigned long long *part = (unsigned long long *)((char *)work_dev + st::xfrag_bytes(K) + 512);
     if (sms > kPartMaxGrid || repeat != 1) part = nullptr;
     else CK(cudaMemsetAsync(part, 0, kPartBytesPerCta * (size_t)sms, stream));
-    k_gemm_probe<<<sms, st::THREADS, st::SMEM_BYTES, stream>>>(dmap, N, K, mode, (const uint4 *)work_dev, Y_dev, ldy, cols, repeat, err, part);
+    k_gemm_probe<true><<<sms, st::THREADS, st::SMEM_BYTES, stream>>>(dmap, N, K, mode, (const uint4 *)work_dev, Y_dev, ldy, cols, repeat, err, part, parking, wait_ns);
     cudaError_t le = cudaGetLastError();
     cudaEventRecord(e1, stream);
-    int herr = 0;
-    cudaError_t ce = le == cudaSuccess ? cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream) : le;
+    int herr[2] = {0, 0};
+    cudaError_t ce = le == cudaSuccess ? cudaMemcpyAsync(herr, err, sizeof(herr), cudaMemcpyDeviceToHost, stream) : le;
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(stream);
     float ms = 0.f;
     if (ce == cudaSuccess) ce = cudaEventElapsedTime(&ms, e0, e1);
@@ -1910,7 +1928,21 @@ int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const 
     cudaEventDestroy(e1);
     CK(ce);
     if (ms_out) *ms_out = ms;
-    return herr ? ADA_ETIMEOUT : ADA_OK;
+    if (parked_out) *parked_out = herr[1];
+    return herr[0] ? ADA_ETIMEOUT : ADA_OK;
+}
+}  // namespace
+
+int ada_debug_gemm(const void *W_dev, int32_t N, int32_t K, int32_t mode, const float *X_dev, int32_t cols, void *work_dev,
+                   size_t work_bytes, float *Y_dev, int32_t ldy, int32_t repeat, void *cuda_stream, float *ms_out) {
+    return run_gemm_probe(W_dev, N, K, mode, X_dev, cols, work_dev, work_bytes, Y_dev, ldy, repeat, ProbeParking{st::PARK_MAX, 0}, st::WAIT_NS_DEFAULT,
+                          cuda_stream, ms_out, nullptr);
+}
+
+int ada_debug_gemm_parked(const void *W_dev, int32_t N, int32_t K, int32_t mode, const float *X_dev, int32_t cols, void *work_dev, size_t work_bytes,
+                          float *Y_dev, int32_t ldy, int32_t most, uint64_t hold_ns, uint64_t wait_ns, void *cuda_stream, int32_t *parked_out) {
+    if (most < 0 || most > st::PARK_MAX || hold_ns > 10000000 || wait_ns < 1) return ADA_EINVAL;
+    return run_gemm_probe(W_dev, N, K, mode, X_dev, cols, work_dev, work_bytes, Y_dev, ldy, 1, ProbeParking{most, hold_ns}, wait_ns, cuda_stream, nullptr, parked_out);
 }
 
 int ada_debug_dense_plan(int32_t rows, int32_t N, int32_t per_tile, int32_t K, int32_t pairs, int32_t pair, int32_t *plan7,
@@ -2046,7 +2078,7 @@ int ada_gemm_noalloc(const void *W_dev, int32_t N, int32_t K, int32_t mode, cons
         unsigned char *ptr = nullptr;
         CK(cudaGetSymbolAddress((void **)&ptr, g_noalloc_scratch));
         CK(cudaDeviceGetAttribute(&sms_of_device[dev], cudaDevAttrMultiProcessorCount, dev));
-        CK(cudaFuncSetAttribute(k_gemm_probe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES));
+        CK(cudaFuncSetAttribute(k_gemm_probe<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES));
         scratch_of_device[dev] = ptr;
     }
     unsigned char *base = scratch_of_device[dev];
@@ -2062,7 +2094,8 @@ int ada_gemm_noalloc(const void *W_dev, int32_t N, int32_t K, int32_t mode, cons
     CK(cudaStreamSynchronize(stream));   // hmap lives on this stack frame
     k_xfrag_pack<<<(K + st::KC - 1) / st::KC * 2, st::KC / 2, 0, stream>>>(X_dev, K, cols, (__nv_bfloat16 *)base);
     CK(cudaGetLastError());
-    k_gemm_probe<<<sms_of_device[dev], st::THREADS, st::SMEM_BYTES, stream>>>(dmap, N, K, mode, (const uint4 *)base, Y_dev, ldy, cols, 1, err, nullptr);
+    k_gemm_probe<false><<<sms_of_device[dev], st::THREADS, st::SMEM_BYTES, stream>>>(dmap, N, K, mode, (const uint4 *)base, Y_dev, ldy, cols, 1, err, nullptr,
+                                                                                      ProbeParking{0, 0}, st::WAIT_NS_DEFAULT);
     CK(cudaGetLastError());
     int herr = 0;
     CK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream));

@@ -29,6 +29,7 @@ struct DevStats {
     long long layer_passes;              // counted on the device by the persistent kernel
     long long phase_ns[ADA_PROF_CLASSES];    // device time per phase class (persistent kernel, measured in CTA 0)
     long long phase_count[ADA_PROF_CLASSES];
+    long long parked;                    // weight stages that passed through tensor memory
 };
 
 // Device-resident decoding state of a session.

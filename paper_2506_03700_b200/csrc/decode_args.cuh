@@ -58,6 +58,7 @@ struct MegaArgs {
                                // slot j of sequence k of them is token column j nseq + k (neighbouring columns are then of equal age, and a
                                // pass that carries the newest tokens only fetches few column pairs); they share every weight stream
     unsigned long long wait_ns;   // a single device-side wait gives up after this long
+    int park;                  // weight stages that a warp parks in tensor memory at a time, at most
     int store_logits;
     // Sampled decoding (Eq. 1 with a drawn token, Eq. 2 with its acceptance test and the resampling): off = greedy
     int sampling;

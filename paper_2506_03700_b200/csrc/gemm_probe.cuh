@@ -23,17 +23,30 @@ struct ProbeEpilogue {
     }
 };
 
+// How a launch parks weight stages: at most `most` per warp; the activations are fetched `hold_ns` nanoseconds late, so that as many land before them.
+struct ProbeParking {
+    int most;
+    unsigned long long hold_ns;
+};
+
 // mode 0: Y[col][n] = sum_k W[n][k] X[col][k]                       (N rows)
 // mode 1: Y[col][n] = silu(g) * u, g = W[n].X, u = W[half + n].X     (half = N/2 rows of each)
+// PARK: as the decode kernel of one column tile, with tensor memory for parked stages; err[1] counts them.
+template <bool PARK>
 __global__ void __launch_bounds__(st::THREADS, 1)
 k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const uint4 *__restrict__ X, float *__restrict__ Y,
-             int ldy, int cols, int repeat, int *err, unsigned long long *part) {
+             int ldy, int cols, int repeat, int *err, unsigned long long *part, ProbeParking parking, unsigned long long wait_ns) {
     extern __shared__ unsigned char smem_raw[];
     st::Smem *sm = st::smem_base(smem_raw);
-    st::smem_init(sm);
-    __syncthreads();
-    st::Shared S{sm, err, Trace{nullptr, nullptr, 0}, 0, st::WAIT_NS_DEFAULT};
     const int warp = threadIdx.x >> 5;
+    st::smem_init(sm);
+    if (PARK && warp == st::CONS_WARPS) {
+        st::park_alloc(sm);
+        tc_fence_before();
+    }
+    __syncthreads();
+    if (PARK) tc_fence_after();
+    st::Shared S{sm, err, Trace{nullptr, nullptr, 0}, 0, wait_ns};
     const int cta = blockIdx.x, G = gridDim.x;
     st::Gemm g;
     g.N = N; g.K = K; g.pair = mode == 1 ? 2 : 1; g.half = mode == 1 ? N / 2 : 0;
@@ -47,15 +60,28 @@ k_gemm_probe(const CUtensorMap *__restrict__ W, int N, int K, int mode, const ui
         for (int it = 0; it < repeat; ++it) st::gemm_produce_w(S, pl, W, nullptr, g.half, r, pol);
     } else if (warp == st::CONS_WARPS + 1) {
         const uint64_t pol = st::policy_evict_last();
-        for (int it = 0; it < repeat; ++it) st::gemm_produce_x(S, pl, X, cols_used, r, pol, st::NoHook(), st::NoHook());
+        const auto hold = [&]() {
+            if (parking.hold_ns == 0) return;
+            const unsigned long long t0 = st::gtime();
+            while (st::gtime() - t0 < parking.hold_ns) __nanosleep(100);
+            __syncwarp();
+        };
+        for (int it = 0; it < repeat; ++it) st::gemm_produce_x(S, pl, X, cols_used, r, pol, st::NoHook(), hold);
     } else {
         const ProbeEpilogue epi{Y, ldy, mode, mode == 0 ? N : g.half};
         for (int it = 0; it < repeat; ++it) {
-            st::gemm_consume<false>(S, pl, cols_used, (1u << cols) - 1u, part, 1u, cta, r, epi);
+            st::gemm_consume<PARK>(S, pl, cols_used, (1u << cols) - 1u, part, 1u, cta, r, epi, parking.most);
             st::bar_consumers();   // the exchange area is free for the next product
         }
+        if (PARK && (threadIdx.x & 31) == 0 && r.parked) atomicAdd(err + 1, r.parked);
     }
+    if (PARK) tc_fence_before();
     st::settle_on_abort(S);
+    if (PARK && warp == st::CONS_WARPS) {
+        __syncwarp();
+        tc_fence_after();
+        st::park_free(sm);
+    }
 }
 
 }  // namespace ada

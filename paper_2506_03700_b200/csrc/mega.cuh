@@ -1685,6 +1685,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
         } else if (action == ACT_CONTINUE) {
             l = e;   // exit layers are below the last one
         } else {
+            if (ROLE == 2 && TILES == 1 && (threadIdx.x & 31) == 0) atomicAdd(reinterpret_cast<unsigned long long *>(&c.st->st.parked), (unsigned long long)r.parked);
             return;
         }
         ph = PH_QKV;
@@ -1740,7 +1741,7 @@ __device__ __forceinline__ void run(const MegaArgs &A, Shared &S) {
                     // (an idle CTA must not report a phase before the one in front of it is complete: the counter would run ahead)
                     if (Groups(pl).left <= 0) consumers_meet(S, A.grid_ctr, bar_no * (unsigned)G);
                     if (ph == PH_HEAD) epi.head_begin();
-                    gemm_consume<TILES == 1>(S, pl, Cols(cmask), cmask, A.part, vseq, blockIdx.x, r, epi);
+                    gemm_consume<TILES == 1>(S, pl, Cols(cmask), cmask, A.part, vseq, blockIdx.x, r, epi, A.park);
                     if (ph == PH_HEAD) epi.head_end(pl, cmask);
                 }
             }
@@ -1829,9 +1830,8 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
         sm->plan[ph] = make_plan(phase_gemm(A, ph, gridDim.x), blockIdx.x, gridDim.x);
     }
     const int warp = threadIdx.x >> 5;
-    if (TILES == 1 && warp == CONS_WARPS + 2) {   // tensor memory for parked weight stages; all of it, there is one CTA per SM
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&sm->tmem)), "r"(PARK_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (TILES == 1 && warp == CONS_WARPS + 2) {   // tensor memory for parked weight stages
+        park_alloc(sm);
         tc_fence_before();
     }
     __syncthreads();
@@ -1850,7 +1850,7 @@ __global__ void __launch_bounds__(MEGA_THREADS, 1) k_decode_persistent(const __g
     if (TILES == 1 && warp == CONS_WARPS + 2) {
         __syncwarp();
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm->tmem), "r"(PARK_COLS) : "memory");
+        park_free(sm);
     }
 }
 

@@ -446,6 +446,7 @@ struct Cols {
 
 struct Rings {   // position of one role in the two rings: number of the next weight stage; slot and parity of the next activation stage
     uint32_t w = 0, xs = 0, xp = 0;
+    int parked = 0;   // weight stages that this (consumer) warp has parked so far
     __device__ __forceinline__ void next_x() { if (++xs == NX) { xs = 0; xp ^= 1; } }
 };
 
@@ -709,6 +710,14 @@ __device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, ui
 // (13.4 -> 11.4), down 20.6 -> 19.2 (9.0 -> 7.7); short requests of the 1B shape 37.6 -> 34.7 ms.  (The kernel of
 // one column tile only: with 24 columns the products are bound by their activations.)
 constexpr int PARK_MAX = 2, PARK_COLS = 512;
+// The CTA's tensor memory, all of it (there is one CTA per SM); both by the same whole warp.
+__device__ __forceinline__ void park_alloc(Smem *sm) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&sm->tmem)), "r"(PARK_COLS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void park_free(Smem *sm) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm->tmem), "r"(PARK_COLS) : "memory");
+}
 __device__ __forceinline__ void park_stage(uint32_t ws, int a_hi, int a_sw, uint32_t tm) {
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
@@ -741,11 +750,12 @@ __device__ __forceinline__ void park_stage(uint32_t ws, int a_hi, int a_sw, uint
 // One body for every product of a program (the caller loops over its phases and branches on the phase in `pre` and `epi`): with
 // a copy of it per product and role the persistent kernel was 790 KB of code, more than the instruction caches hold, and every
 // phase began and ended with instruction fetches from L2 on its critical path.
-// PARK: the kernel has tensor memory for parked stages (sm->tmem).
+// PARK: the kernel has tensor memory for parked stages (sm->tmem), of which a warp parks at most `park` (up to PARK_MAX).  (As a
+// member of `S`, which lives in local memory, the limit cost 0.4 % of a short request.)
 // k steps past K multiply zeros (the tensor map fills weights with them, the activation blocks are padded with them).
 template <bool PARK, class Epi>
 __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, const Cols &cols, unsigned mask, unsigned long long *part, unsigned phase_id, int cta,
-                                             Rings &r, const Epi &epi) {
+                                             Rings &r, const Epi &epi, int park) {
     Smem *sm = S.sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nch = pl.nch, pair = pl.pair, XC = cols.chunks();
@@ -806,7 +816,7 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
         const uint32_t tm = PARK ? sm->tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (128 * PARK_MAX) : 0u;
         if (PARK && first) {
             unsigned long long t0 = 0;
-            const int most = min(n_all * pair, PARK_MAX);
+            const int most = min(n_all * pair, park);
 #pragma unroll 1
             while (n_parked < most) {
                 const uint32_t i = stage_of(chunk_of(pair == 2 ? n_parked >> 1 : n_parked)) + (pair == 2 ? n_parked & 1 : 0), wslot = i % NW;
@@ -830,6 +840,7 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&sm->w_empty[wslot]);
             }
+            r.parked += n_parked;
         }
         float acc0[TILES][4][4], acc1[TILES][4][4];   // [column tile][even/odd step x hi/lo][fragment] of the one or two matrices
         auto clear = [&]() {

@@ -92,3 +92,72 @@ def test_waits_that_run_out_anywhere(batch, early):
             torch.cuda.synchronize()      # the context is intact
         assert np.array_equal(decode(2_000_000_000), ref), limit
     assert ran_out > 0
+
+
+@pytest.mark.parametrize("d,ff,nq,nkv,hd,vocab,n_prompt,n", SHAPES)
+def test_parked_stages_leave_the_bits(d, ff, nq, nkv, hd, vocab, n_prompt, n):
+    """Stages are parked, and a call without parking gives the same logits, bit for bit: one column and up to six."""
+    cfg = config(d, ff, nq, nkv, hd, vocab)
+    gm = binding.Model(cfg, synth.make_weights(cfg, device="cuda"))
+    for l in cfg.exit_layers:
+        gm.set_exit_head(l, None, cfg.logit_scale)
+    prompt = synth.make_prompt(cfg, n=n_prompt).numpy()
+    for early in (0, 5):
+        got = []
+        for most in (2, 1, 0):
+            S = binding.Session(gm, 1, n_prompt + n + 8, 64, 5)
+            S.set_parking(most)
+            S.capture_logits(n + 8)
+            S.prefill(prompt)
+            out = S.adaptive_decode(n, 0.0, cfg.exit_layers, early) if early else S.plain_decode(n)
+            got.append((out[0], S.captured_logits()[:n].clone()))
+            assert (S.parked() > 0) == (most > 0), (early, most)
+        for out, logits in got[1:]:
+            assert np.array_equal(out, got[0][0]) and torch.equal(logits, got[0][1]), early
+
+
+def parkable(N, K, mode, most):
+    """(most stages that the warps of all CTAs can park, whether all of them are sure to land): host arithmetic from the plans."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nch, pair, total = (K + 511) // 512, 2 if mode else 1, 0
+    sure = most >= pair   # (a second matrix' stage that is not parked keeps its place in the ring)
+    for cta in range(sms):
+        p = binding.debug_gemm_plan(N, K, mode, sms, cta)
+        ng = p["n"] if p["split"] else min(p["t1"] - p["t0"], 8)
+        ts = 1 << max(ng - 1, 0).bit_length()
+        ks = 8 // ts
+        for slot in range(ng):
+            chunks = list(range(nch))
+            if p["split"] and slot == 0:
+                chunks = [k for k in chunks if k < p["s0_pub_k1"] or k >= p["s0_own_k0"]]
+            elif p["split"] and slot == ng - 1:
+                chunks = chunks[:p["sl_k1"]]
+            sure = sure and len(chunks) == nch   # a slot with a gap may find the ring full of other warps' third stages
+            published = p["s0_pub_k1"] if p["split"] and slot == 0 else 0
+            parts = [chunks[:published], chunks[published:]]
+            for k in range(ks):
+                total += min(sum(len(c[k::ks]) for c in parts) * pair, most)
+    return total, sure
+
+
+# one stage for one warp of a CTA; one for each; more than two for each; a pair of matrices, one chunk and many; several slots, some of them
+# idle; tiles cut between CTAs, their first parts published; two groups of tiles
+@pytest.mark.parametrize("N,K,mode", [(148 * 16, 512, 0), (148 * 16, 4096, 0), (148 * 16, 14336, 0), (2 * 148 * 16, 512, 1), (2 * 148 * 16, 4096, 1),
+                                      (148 * 16 * 5, 1216, 0), (6144, 4096, 0), (2 * 5504, 2048, 1), (24000, 576, 0), (1000, 192, 0)])
+@pytest.mark.parametrize("cols", [1, 4, 5, 8])
+def test_products_from_parked_stages(N, K, mode, cols):
+    W = synth.normal_tensor(5, 11, (N, K), 0.05, torch.bfloat16, "cuda")
+    X = synth.normal_tensor(5, 12, (cols, K), 1.0, torch.float32, "cuda")
+    ref, none = binding.debug_gemm_parked(W, X, mode, most=0, hold_ns=200_000)
+    assert none == 0
+    for most in (1, 2):
+        Y, parked = binding.debug_gemm_parked(W, X, mode, most=most, hold_ns=200_000)   # (a stage lands within 2 us)
+        total, sure = parkable(N, K, mode, most)
+        assert 0 < parked <= total and (parked == total or not sure), (most, parked, total)
+        assert torch.equal(Y, ref), most
+    assert torch.equal(binding.debug_gemm(W, X, mode)[0], ref)
+    # the activations come after the consumers have given up: parked stages are multiplied with whatever is there, and the call says so
+    with pytest.raises(binding.AdaError) as e:
+        binding.debug_gemm_parked(W, X, mode, hold_ns=400_000, wait_ns=100_000)
+    assert e.value.code == -5
+    assert torch.equal(binding.debug_gemm_parked(W, X, mode)[0], ref)
