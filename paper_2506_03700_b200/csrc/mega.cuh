@@ -1318,7 +1318,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
         if ((lane & 3) == 0) {
             as->l[warp][lane >> 2] = l[0];
             as->l[warp][(lane >> 2) + 8] = l[1];
-            if (warp == w0) {   // the maximum's word (the next item's maxima may already be on their way when the sums are read)
+            if (warp == w0 && !one_chunk) {   // the maximum's word (the next item's maxima may already be on their way when the sums are read)
 #pragma unroll
                 for (int rh = 0; rh < 2; ++rh)
                     if (lim[rh] >= it.p_base) {
