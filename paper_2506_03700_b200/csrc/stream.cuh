@@ -951,12 +951,14 @@ __device__ __forceinline__ void gemm_consume(const Shared &S, const Plan &pl, co
                 if (packed) {
                     if (p == 0) stage_packed(acc0[0], ws, xc[0], a_hi, a_sw);
                     else stage_packed(acc1[0], ws, xc[0], a_hi, a_sw);
-                } else if (nt == 1) {
-                    if (p == 0 || TILES > 1) stage_full<1>(acc0, ws, xc, a_hi, a_sw);
+                } else if (TILES == 1) {
+                    if (p == 0) stage_full<1>(acc0, ws, xc, a_hi, a_sw);
                     else stage_full<1>(acc1, ws, xc, a_hi, a_sw);
-                } else if (TILES > 1 && nt == 2) {
+                } else if (nt == 1) {   // (several tiles: the two matrices of a pair were multiplied together above, this is a single one)
+                    stage_full<1>(acc0, ws, xc, a_hi, a_sw);
+                } else if (nt == 2) {
                     stage_full<TILES < 2 ? TILES : 2>(acc0, ws, xc, a_hi, a_sw);
-                } else if (TILES > 1) {
+                } else {
                     stage_full<TILES>(acc0, ws, xc, a_hi, a_sw);
                 }
                 __syncwarp();
