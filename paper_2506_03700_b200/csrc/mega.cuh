@@ -6,8 +6,10 @@
 // with a grid barrier between phases.  The weight producer is not held by those barriers (but for cache rows
 // of the pass itself): it keeps the TMA ring full with the tiles of the coming phases, so HBM keeps streaming while the
 // grid meets, and the consumers move what has landed on to tensor memory (park_stage in stream.cuh).  Measured, one layer in a plain
-// step (1B / 8B shape): QKV 5.7 / 10.9 us, attention 6.6 / 10.3 (60 / 1040 positions),
-// O 5.1 / 7.6, gate-up 10.6 / 36.8, down 7.8 / 18.6, of which the bytes alone take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
+// step (1B / 8B shape): QKV 5.7 / 10.9 us, attention 6.6 / 10.2 (60 / 1040 positions), O 4.9 / 7.5, gate-up 10.7 / 36.7, down 8.0 / 18.6,
+// of which a phase's own bytes take 1.9 / 7.8, - / 0.7, 1.3 / 5.2, 10.3 / 36, 5.1 / 18.  (Not a floor of the phase: up to 25 stages a
+// CTA, 9 us of the stream, have been fetched in earlier phases, and as many of the next ones' are fetched in it.  Boxes differ by up to
+// 0.6 us a phase.)  All decoding state (sequence, per-layer fill levels, in-flight tokens, row
 // residuals, counters) lives in device memory; the control points run in CTA 0, which publishes
 // each decision (continue the climb, start the next token, stop) to the other CTAs through a
 // sequence-numbered record.  The host launches, waits, and launches again until the call is done.
@@ -513,11 +515,8 @@ __device__ __noinline__ void sample_stage(SampleArgs a, Smem *sm, bool after_hea
 
 // ---------------------------------------------------------------- control point (CTA 0, consumer warps)
 
-// Applies the outcome of the step that just ended (Eq. 1 after a head; verification and rollback,
-// Eq. 2 at temperature zero, after the final head), then sets up the next step: its columns, the
-// embedding of its newest token, that token's rotary table; finally publishes the action.
 // What the bookkeeping works on, in the consumers' scratch.  (The next step's descriptor and the sequences' lengths as arrays of the
-// bookkeeping thread were local memory, a load from L2 for each first touch behind the barrier's acquire: 13 us with eight sequences.)
+// bookkeeping warp were local memory, a load from L2 for each first touch behind the barrier's acquire: 13 us with eight sequences.)
 struct Ctl {
     StepDesc nd;
     int len[MAX_SEQS], base[MAX_SEQS], target[MAX_SEQS], done[MAX_SEQS];
@@ -526,6 +525,9 @@ struct Ctl {
 constexpr int CTL_OFFSET = 8192 + ((int)sizeof(HeadResult) + 4) * MAX_COLS;
 static_assert(CTL_OFFSET % 16 == 0 && CTL_OFFSET + (int)sizeof(Ctl) <= DRAW_OFFSET, "the control point's copies overlap the draw's buffers");
 
+// Applies the outcome of the step that just ended (Eq. 1 after a head; verification and rollback,
+// Eq. 2 at temperature zero, after the final head), then sets up the next step: its columns, the
+// embeddings of its newest tokens, their rotary factors; finally publishes the action.
 __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int kind, int e, unsigned pub_no, const StepDesc &dprev,
                                           int &steps_started) {
     const Ctx &c = A.c;
@@ -534,7 +536,7 @@ __device__ __forceinline__ void control_cta0(const MegaArgs &A, Smem *sm, int ki
     const int tid = threadIdx.x, G = gridDim.x;
     const int nseq = A.nseq, seq0 = A.seq0, cps = c.slots, L = c.L;   // cps: token columns per sequence (slots)
     Pub *pub = reinterpret_cast<Pub *>(A.pub) + (pub_no & 1);
-    // Shared-memory copies for the bookkeeping thread (fetched by many threads at once: a single
+    // Shared-memory copies for the bookkeeping warp (fetched by many threads at once: a single
     // thread reading them from global memory one after the other spent 30 us here on round trips to L2):
     // the fill levels, the head results, and the tokens the verification compares with.
     int *fill_s = reinterpret_cast<int *>(sm->scratch);                                          // [nseq][L]
@@ -1159,7 +1161,7 @@ __device__ __forceinline__ void attn_consume(const MegaArgs &A, const Shared &S,
         const unsigned sl = seq_slots(A, mask, k);
         if (sl) dual = dual && ((__ffs(sl) - 1) * group >= 16 || (32 - __clz(sl)) * group <= 16);
     }
-    // Every row of the step has a single chunk: its item finishes it, there is nothing to merge (1B shape at 60 positions 7.4 -> 6.6 us a layer).
+    // Every row of the step has a single chunk: its item finishes it, there is nothing to merge (1B shape at 60 positions 7.2 -> 6.6 us a layer).
     const bool one_chunk = d.pmax < ATT_CHUNK;
     int turn = 0;   // group whose item it is
 #pragma unroll 1
@@ -1453,9 +1455,10 @@ __device__ __forceinline__ int prof_class(int ph) {   // class of ada_debug_prof
     return ph == PH_QKV ? 2 : ph == PH_ATTN ? 4 : ph == PH_O ? 5 : ph == PH_GU ? 6 : ph == PH_DOWN ? 8 : ph == PH_T ? 10 : 9;
 }
 // Whole tiles or units of (tile, chunk): cutting tiles costs an exchange of partial sums at the end of the phase (some 0.7 us)
-// and saves the stages by which the CTA with most whole tiles exceeds its share, 0.36 us each: taken from four stages on.
-// Measured, whole -> cut: 13B O (8 stages fewer) 13.6 -> 12.1 us, down (22) 30.0 -> 25.4, QKV (5) 28.1 -> 26.9; 8B down (7)
-// 21.2 -> 20.5, QKV (3) 11.7 -> 11.7, O (2) 9.0 -> 9.3; 1B QKV (2) 6.2 -> 6.7.
+// and saves the stages by which the CTA with most whole tiles exceeds its share, 0.36 us each (less where they are parked): taken from
+// four stages on.  Measured, whole -> cut: 13B, four columns, O (8 stages fewer) 12.8 -> 10.4 us, down (22) 28.1 -> 22.9, QKV (5)
+// 27.1 -> 26.1; 8B gate-up (14) 40.2 -> 36.9, down (7) 19.5 -> 18.8, QKV (3) 10.8 -> 11.0, O (2) 7.6 -> 7.7; 1B gate-up (4)
+// 12.7 -> 11.3, QKV (2) 5.6 -> 6.3.  (13B gate-up, 2 stages, gains all the same: 44.7 -> 43.9.)
 constexpr int CUT_STAGES = 4;
 __host__ __device__ __forceinline__ Gemm phase_gemm(const MegaArgs &A, int ph, int G) {
     const Ctx &c = A.c;
@@ -1813,9 +1816,9 @@ __global__ void k_prefill_arm(Ctx c, int seq, int n_prompt) {
 // Warps 0-7 consume, warp 8 produces weights and K / V blocks, warp 9 activations and queries; warps 10 and 11 only complete the producers'
 // warp group, which hands registers to the consumers.  (At 168 registers a thread -- three warps on a quarter of the SM --
 // the consumers kept loop variables in local memory, whose L1 lines do not survive the acquires of the grid barrier: a round trip to
-// L2 for each on the critical path of a phase.  One column tile: at 200 / 104 nothing is spilled; 216 / 72 spilled 64 bytes in the
-// producers and cost 0.5 to 2 % of a request.  Three tiles: the consumers' sums need more; 216 / 72 (which spills 200 bytes in the
-// producers) 58 us a gate / up product of the 13B shape, 200 / 104 67; requests 183.3 ms, 208 / 88 185, 200 / 104 187.5.)
+// L2 for each on the critical path of a phase.  One column tile: at 200 / 104 nothing is spilled; 216 / 72 spills 24 bytes in the
+// producers (8B down 18.5 -> 18.9 us, the other phases alike; 64 bytes, when it was 64, cost 0.5 to 2 % of a request).  Three tiles: the
+// consumers' sums need more; 216 / 72 (which spills 200 bytes in the producers) 58 us a gate / up product of the 13B shape, 200 / 104 67; requests 183.3 ms, 208 / 88 185, 200 / 104 187.5.)
 constexpr int MEGA_THREADS = CONS_THREADS + 128;
 constexpr int REGS_CONSUME = TILES == 1 ? 200 : 216, REGS_PRODUCE = TILES == 1 ? 104 : 72;
 constexpr int MEGA_REGS = CONS_THREADS * REGS_CONSUME + 128 * REGS_PRODUCE;   // the block must have been launched with as many

@@ -706,9 +706,11 @@ __device__ __forceinline__ void stage_parked(float (&acc)[4][4], uint32_t tm, ui
 // two each, as the fragments that the multiply-add wants; the ring's slots go back to the producer at once.  That makes 25
 // stages (400 KB) per CTA, and the parked ones do not pass through shared memory again when the activations are there.
 // Warp w can address the lanes of quadrant w % 4 only; it holds its stages there in columns 256 (w / 4) on, 128 a stage.
-// A layer of the 8B shape (1B), us, without and with: QKV 11.7 -> 10.8 (6.2 -> 5.9), O 9.0 -> 7.7 (5.3 -> 5.2), gate-up 38.6 -> 35.8
-// (13.4 -> 11.4), down 20.6 -> 19.2 (9.0 -> 7.7); short requests of the 1B shape 37.6 -> 34.7 ms.  (The kernel of
-// one column tile only: with 24 columns the products are bound by their activations.)
+// A layer of the 8B shape (1B), us, with no, one and two stages a warp: QKV 12.3, 11.2, 10.9 (6.4, 5.8, 5.7), O 9.3, 7.5, 7.5 (5.4,
+// 4.8, 4.9), gate-up 39.0, 39.2, 36.7 (13.5, 13.2, 10.7), down 20.9, 19.2, 18.6 (9.3, 7.7, 8.0); attention, whose K and V blocks have
+// less time to arrive, 10.0, 10.2, 10.2 (6.6 each).  (The kernel of one column tile only.  With more than four columns in use the
+// products of the other one are bound by their activations; its steps of up to four would gain too, but three tiles' sums leave no
+// registers for it: some 200 bytes are spilled as it is.)
 constexpr int PARK_MAX = 2, PARK_COLS = 512;
 // The CTA's tensor memory, all of it (there is one CTA per SM); both by the same whole warp.
 __device__ __forceinline__ void park_alloc(Smem *sm) {
